@@ -1,40 +1,80 @@
-"""Builds libpf.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libpf.so (the C-ABI CUDA library, nvcc for sm_100a) and _pf_native.so (its Python marshalling
+module, g++ against torch's headers) in-tree."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
+from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
+OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpf.so")
+NATIVE = os.path.join(PKG, "_pf_native.so")
 SOURCES = ["pf_api.cu", "pf_simt.cu", "pf_pack.cu", "pf_tc.cu", "pf_tc_chain.cu", "pf_tc_chain_multi.cu", "pf_tc_chain_act.cu", "pf_tc_pair.cu", "pf_static.cu"]
-NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-              "-Xcompiler", "-fPIC", "-shared"]
+NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
 
 
-def sources():
-    return [os.path.join(CSRC, s) for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
+def _mtime(path: str) -> float:
+    return os.path.getmtime(path) if os.path.exists(path) else 0.0
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "pf.h")]
-    return any(os.path.getmtime(d) > t for d in deps)
+def _newest(paths) -> float:
+    return max(os.path.getmtime(p) for p in paths)
+
+
+def _headers():
+    return [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))] + [os.path.join(ROOT, "include", "pf.h")]
+
+
+def _build_lib(force: bool, verbose: bool) -> None:
+    sources = [os.path.join(CSRC, s) for s in SOURCES]
+    if not force and _mtime(LIB) > _newest(sources + _headers()):
+        return
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    os.makedirs(OBJ, exist_ok=True)
+    headers = _newest(_headers())
+
+    def compile_one(src: str) -> str:
+        obj = os.path.join(OBJ, os.path.basename(src)[:-3] + ".o")
+        if force or _mtime(obj) <= max(headers, os.path.getmtime(src)):
+            tmp = obj + f".tmp{os.getpid()}.o"
+            subprocess.check_call([nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
+                                  ["-I", os.path.join(ROOT, "include"), "-I", CSRC, "-c", "-o", tmp, src])
+            os.replace(tmp, obj)
+        return obj
+
+    with ThreadPoolExecutor(max_workers=min(len(sources), os.cpu_count() or 1)) as pool:
+        objects = list(pool.map(compile_one, sources))
+    tmp = LIB + f".tmp{os.getpid()}"
+    subprocess.check_call([nvcc] + NVCC_FLAGS + ["-shared", "-o", tmp] + objects)
+    os.replace(tmp, LIB)
+
+
+def _build_native(force: bool) -> None:
+    src = os.path.join(CSRC, "pf_python.cpp")
+    if not force and _mtime(NATIVE) > _newest([src, os.path.join(ROOT, "include", "pf.h")]):
+        return
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    includes = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+                os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    subprocess.check_call(
+        [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=1", "-o", tmp, src] +
+        [a for d in includes for a in ("-isystem", d)] +
+        ["-I", os.path.join(ROOT, "include"), "-L", os.path.join(torch_dir, "lib"), "-L", PKG, "-l:libpf.so", "-ltorch_python", "-ltorch_cuda",
+         "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, NATIVE)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale():
-        return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    tmp = LIB + f".tmp{os.getpid()}"
-    cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + \
-        ["-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", tmp] + sources()
-    subprocess.check_call(cmd)
-    os.replace(tmp, LIB)
+    _build_lib(force, verbose)
+    _build_native(force)
     return LIB
 
 
