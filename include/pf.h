@@ -224,8 +224,9 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
  * matrices themselves are as in the ungrouped calls.  sx = 0 means ONE input x shared by all groups
  * (the gates of an LSTM all read the same x_t); factors and outputs are always per group.
  * With bf16 and 16-byte aligned pointers, pitches and strides the whole call is two launches
- * (all x_g U_g, then all T_g V_g^T), whatever `groups`; other layouts, and fp32, run group by group
- * through the ungrouped kernels (same results, more launches).
+ * (all x_g U_g, then all T_g V_g^T), whatever `groups`; ragged widths (not a multiple of 8) add one launch
+ * that copies those operands to 16-byte pitches; other layouts, and fp32, run group by group through the
+ * ungrouped kernels (same results, more launches).
  *
  * Backward, for dY_g [m, n] (stride sdy):
  *   dU_g = x_g^T (dY_g V_g),  dV_g = dY_g^T (x_g U_g)                       (strides sdu, sdv)
@@ -233,7 +234,7 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
  *   dX   = sum over g of (dY_g V_g) U_g^T, ONE m x k matrix (sdx ignored)   when x is shared (sx = 0),
  *          since a shared input collects the gradient of every group that reads it.
  *   NULL dX = not wanted.  T_stash (stride st): the forward's stash, or NULL to recompute.
- * Two launches (three when T is recomputed) on the fast path.
+ * Two launches (three when T is recomputed) on the fast path, one more for ragged widths.
  * ------------------------------------------------------------------------------- */
 size_t pf_lowrank_linear_grouped_workspace(int groups, int64_t m, int64_t k, int64_t n, int64_t r,
                                            int dtype, int is_bwd);

@@ -112,13 +112,16 @@ cudaError_t act_bwd(const void* y, int64_t ldy, void* dY, int64_t lddy, void* db
 cudaError_t bias_act_inplace(void* y, int64_t ld, int64_t rows, int64_t cols, const void* bias, int act, int dtype,
                              cudaStream_t stream);
 
-// Several such copies in one launch (row counts and widths below 2^31).
+// Copies to 16-byte aligned rows whose pitch is a multiple of 8 elements (the tail of a row's last 8 elements
+// is zeroed), up to six in one launch.  A job covers `groups` matrices gs_src elements apart (0 is one matrix),
+// which land one after the other.
 struct RepackJob {
     const void* src;
     int64_t ld_src;
     void* dst;
     int64_t ld_dst;
-    int64_t rows, cols, cols_padded;
+    int64_t rows, cols;
+    int64_t groups = 1, gs_src = 0;
 };
 cudaError_t repack_rows_bf16_multi(const RepackJob* jobs, int count, cudaStream_t stream);
 

@@ -191,37 +191,63 @@ repack_rows_kernel(const unsigned short* __restrict__ src, int64_t ld_src,
 
 // Several re-pitch copies in one launch.  A work item is one 16-byte piece (8 elements) of a
 // destination row: the destination is 16-byte aligned with a pitch that is a multiple of 8
-// elements, the source may start anywhere, so it is read element by element.
+// elements, the source may start at any element.  Pure streaming (4 bytes per element), so both sides move
+// 16 bytes per access: a whole piece is assembled from the two aligned source vectors that cover it with a
+// funnel shift (each of them holds at least one byte of the piece), only a row's last piece reads elements.
+// A job may cover several matrices (groups) a fixed stride apart, which land one after the other.
+// Launched with programmatic dependent launch: its start hides behind the previous kernel's tail, and the
+// product that reads the copies starts its own prologue meanwhile.
 constexpr int kRepackJobs = 6;
 struct RepackBatchArgs {
     const unsigned short* src[kRepackJobs];
     unsigned short* dst[kRepackJobs];
-    long long ld_src[kRepackJobs], ld_dst[kRepackJobs];
-    int cols[kRepackJobs], pieces_per_row[kRepackJobs];
-    long long item_end[kRepackJobs];   // running total of items up to and including job j
+    long long ld_src[kRepackJobs], ld_dst[kRepackJobs], gs_src[kRepackJobs];
+    int cols[kRepackJobs], pieces_per_row[kRepackJobs], rows[kRepackJobs];   // rows of one group
+    unsigned int item_end[kRepackJobs];   // running total of items up to and including job j
     int count;
 };
+__device__ __forceinline__ uint4 shifted_vector(const uint4 lo, const uint4 hi, unsigned q, unsigned bit) {
+    unsigned w0, w1, w2, w3, w4;
+    switch (q) {
+        case 0: w0 = lo.x; w1 = lo.y; w2 = lo.z; w3 = lo.w; w4 = hi.x; break;
+        case 1: w0 = lo.y; w1 = lo.z; w2 = lo.w; w3 = hi.x; w4 = hi.y; break;
+        case 2: w0 = lo.z; w1 = lo.w; w2 = hi.x; w3 = hi.y; w4 = hi.z; break;
+        default: w0 = lo.w; w1 = hi.x; w2 = hi.y; w3 = hi.z; w4 = hi.w; break;
+    }
+    return make_uint4(__funnelshift_r(w0, w1, bit), __funnelshift_r(w1, w2, bit), __funnelshift_r(w2, w3, bit),
+                      __funnelshift_r(w3, w4, bit));
+}
 __global__ void __launch_bounds__(256)
-repack_multi_kernel(const RepackBatchArgs a) {
-    const long long total = a.item_end[a.count - 1];
-    for (long long it = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; it < total;
-         it += static_cast<long long>(gridDim.x) * blockDim.x) {
+repack_multi_kernel(const __grid_constant__ RepackBatchArgs a) {
+    const unsigned int total = a.item_end[a.count - 1];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (unsigned int it = blockIdx.x * blockDim.x + threadIdx.x; it < total; it += gridDim.x * blockDim.x) {
         int j = 0;
         while (j + 1 < a.count && it >= a.item_end[j]) ++j;
-        const long long local = it - (j > 0 ? a.item_end[j - 1] : 0);
-        const int ppr = a.pieces_per_row[j];
-        const long long row = local / ppr;
+        const unsigned int local = it - (j > 0 ? a.item_end[j - 1] : 0u);
+        const unsigned int ppr = static_cast<unsigned int>(a.pieces_per_row[j]);
+        const unsigned int row = local / ppr;
         const int c0 = static_cast<int>(local - row * ppr) * 8;
-        const unsigned short* sp = a.src[j] + row * a.ld_src[j] + c0;
+        const unsigned int g = a.gs_src[j] ? row / static_cast<unsigned int>(a.rows[j]) : 0u;
+        const unsigned short* sp = a.src[j] + g * a.gs_src[j] + (row - g * static_cast<unsigned int>(a.rows[j])) * a.ld_src[j] + c0;
         const int left = a.cols[j] - c0;
-        unsigned short v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = e < left ? sp[e] : static_cast<unsigned short>(0);
         uint4 o;
-        o.x = v[0] | (static_cast<unsigned int>(v[1]) << 16);
-        o.y = v[2] | (static_cast<unsigned int>(v[3]) << 16);
-        o.z = v[4] | (static_cast<unsigned int>(v[5]) << 16);
-        o.w = v[6] | (static_cast<unsigned int>(v[7]) << 16);
+        if (left >= 8) {
+            const unsigned int sh = static_cast<unsigned int>(reinterpret_cast<uintptr_t>(sp)) & 15u;
+            const uint4* v = reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(sp) - sh);
+            const uint4 lo = __ldg(v);
+            o = lo;
+            if (sh) o = shifted_vector(lo, __ldg(v + 1), sh >> 2, (sh & 3u) * 8u);
+        } else {
+            unsigned short e[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) e[i] = i < left ? sp[i] : static_cast<unsigned short>(0);
+            o.x = e[0] | (static_cast<unsigned int>(e[1]) << 16);
+            o.y = e[2] | (static_cast<unsigned int>(e[3]) << 16);
+            o.z = e[4] | (static_cast<unsigned int>(e[5]) << 16);
+            o.w = e[6] | (static_cast<unsigned int>(e[7]) << 16);
+        }
         *reinterpret_cast<uint4*>(a.dst[j] + row * a.ld_dst[j] + c0) = o;
     }
 }
@@ -495,45 +521,37 @@ cudaError_t repack_rows_bf16(const void* src, int64_t ld_src, void* dst, int64_t
 }
 
 cudaError_t repack_rows_bf16_multi(const RepackJob* jobs, int count, cudaStream_t stream) {
-    while (count > 0) {
-        RepackBatchArgs a;
-        a.count = 0;
-        long long total = 0;
-        const int n = count < kRepackJobs ? count : kRepackJobs;
-        for (int i = 0; i < n; ++i) {
-            const RepackJob& j = jobs[i];
-            if (j.rows <= 0 || j.cols <= 0) continue;
-            const bool fast = (reinterpret_cast<uintptr_t>(j.dst) & 15) == 0 && j.ld_dst % 8 == 0 &&
-                              j.cols_padded == (j.cols + 7) / 8 * 8 && j.cols_padded <= j.ld_dst;
-            if (!fast) {   // arbitrary destination: the element-wise copy
-                cudaError_t e = repack_rows_bf16(j.src, j.ld_src, j.dst, j.ld_dst, j.rows, j.cols, j.cols_padded, stream);
-                if (e != cudaSuccess) return e;
-                continue;
-            }
-            const int k = a.count++;
-            a.src[k] = static_cast<const unsigned short*>(j.src);
-            a.dst[k] = static_cast<unsigned short*>(j.dst);
-            a.ld_src[k] = j.ld_src; a.ld_dst[k] = j.ld_dst;
-            a.cols[k] = static_cast<int>(j.cols);
-            a.pieces_per_row[k] = static_cast<int>(j.cols_padded / 8);
-            total += j.rows * (j.cols_padded / 8);
-            a.item_end[k] = total;
-        }
-        if (a.count > 0) {
-            for (int k = a.count; k < kRepackJobs; ++k) {
-                a.src[k] = a.src[0]; a.dst[k] = a.dst[0]; a.ld_src[k] = 0; a.ld_dst[k] = 0; a.cols[k] = 0;
-                a.pieces_per_row[k] = 1; a.item_end[k] = total;
-            }
-            const long long blocks = ceil_div(total, 256) < 8 * num_sms() ? ceil_div(total, 256) : 8 * num_sms();
-            repack_multi_kernel<<<static_cast<int>(blocks), 256, 0, stream>>>(a);
-            count_launch();
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-        }
-        jobs += n;
-        count -= n;
+    if (count > kRepackJobs) return cudaErrorInvalidValue;
+    RepackBatchArgs a = {};
+    long long total = 0;
+    for (int i = 0; i < count; ++i) {
+        const RepackJob& j = jobs[i];
+        const long long rows = j.rows * j.groups, pieces = (j.cols + 7) / 8;
+        if (rows <= 0 || j.cols <= 0) continue;
+        if (total + rows * pieces > 0x7fffffffLL) return cudaErrorInvalidValue;
+        const int k = a.count++;
+        a.src[k] = static_cast<const unsigned short*>(j.src);
+        a.dst[k] = static_cast<unsigned short*>(j.dst);
+        a.ld_src[k] = j.ld_src; a.ld_dst[k] = j.ld_dst;
+        a.gs_src[k] = j.groups > 1 && j.gs_src != j.rows * j.ld_src ? j.gs_src : 0;   // 0: one run of rows
+        a.cols[k] = static_cast<int>(j.cols);
+        a.rows[k] = static_cast<int>(j.rows);
+        a.pieces_per_row[k] = static_cast<int>(pieces);
+        total += rows * pieces;
+        a.item_end[k] = static_cast<unsigned int>(total);
     }
-    return cudaSuccess;
+    if (a.count == 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(ceil_div(total, 256) < 16 * num_sms() ? ceil_div(total, 256) : 16 * num_sms()));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, repack_multi_kernel, a);
+    if (e == cudaSuccess) count_launch();
+    return e;
 }
 
 }  // namespace pf

@@ -54,8 +54,8 @@ struct GemmParams {
     int tiles_x;             // row tiles of this product (tile id = column tile * tiles_x + row tile)
     void* C;                 // bf16 [M, ldc]
     long long ldc;
-    void* C2;                // optional second copy of the result at another pitch (split contractions only)
-    long long ldc2;
+    void* C2;                // optional second copy of the result at another pitch, groups c2_gstride elements apart
+    long long ldc2, c2_gstride;
     float* partial;          // splits > 1: fp32 slices, one 128 x BN block per (tile, slice)
     unsigned int* counters;  // splits > 1: two counters per tile
     unsigned int* status;
@@ -380,6 +380,25 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                             }
                             dst += row_step;
                         }
+                        if (p.C2) {          // the second copy, at a pitch that takes element pairs at best
+                            __nv_bfloat16* C2b = reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride;
+                            const bool pair2 = (p.ldc2 % 2) == 0 && (reinterpret_cast<uintptr_t>(C2b) & 3) == 0;
+                            const int c2 = n0 + c * 64 + 2 * lane;
+                            for (int j = 0; j < 32; ++j) {
+                                const int rowj = m0 + q * 32 + j;
+                                if (rowj >= p.M || q * 32 + j >= p.rows_tile) break;
+                                uint32_t w;
+                                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(panel + static_cast<uint32_t>(j) * 128u +
+                                             ((static_cast<uint32_t>(lane >> 2) ^ static_cast<uint32_t>(j & 7)) << 4) + static_cast<uint32_t>(lane & 3) * 4u));
+                                __nv_bfloat16* d2 = C2b + static_cast<size_t>(rowj) * p.ldc2 + c2;
+                                if (pair2 && c2 + 1 < p.N) {
+                                    *reinterpret_cast<uint32_t*>(d2) = w;
+                                } else {
+                                    if (c2 < p.N) d2[0] = __ushort_as_bfloat16(static_cast<unsigned short>(w & 0xffffu));
+                                    if (c2 + 1 < p.N) d2[1] = __ushort_as_bfloat16(static_cast<unsigned short>(w >> 16));
+                                }
+                            }
+                        }
                         __syncwarp();
                     }
                 } else
@@ -463,7 +482,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     __syncthreads();
     if (ctl->fix_ok) {
         __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
-        __nv_bfloat16* C2b = reinterpret_cast<__nv_bfloat16*>(p.C2);
+        __nv_bfloat16* C2b = p.C2 ? reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride : nullptr;
         const uint32_t base = smem_u32(tiles);
         const bool vec8 = (p.ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 7) == 0;
         // consecutive threads take consecutive 16-byte pieces of one row
@@ -770,7 +789,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
     p.a_mn = A.mn_major; p.b_mn = B.mn_major;
     p.C = C; p.ldc = ldc; p.partial = partial;
-    p.C2 = nullptr; p.ldc2 = 0;
+    p.C2 = nullptr; p.ldc2 = 0; p.c2_gstride = 0;
     p.conv_mode = 0; p.cv_blks = 1; p.cv_kw = 1; p.cv_pad = 0; p.cv_C = 1; p.cv_box_h = 1; p.cv_tpi = 1;
     if (cv) {
         p.conv_mode = cv->mode; p.cv_kw = cv->kw; p.cv_pad = cv->pad; p.cv_C = cv->Cw;
@@ -830,7 +849,7 @@ int launch_prepared(const GemmLaunch& g, cudaStream_t stream) {
 }
 
 // `copy2` (optional): asks for a second copy of C at pitch ldc2; *copy2_done tells whether the launch
-// wrote it (only a split contraction can), else the caller copies C itself.
+// wrote it (the CTA-pair kernel cannot), else the caller copies C itself.
 int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
          int splits, float* partial, cudaStream_t stream, const ConvA* cv = nullptr, void* copy2 = nullptr,
          int64_t ldc2 = 0, bool* copy2_done = nullptr) {
@@ -847,7 +866,7 @@ int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, vo
     if (st == PF_ERR_UNSUPPORTED && splits > 1) st = gemm_prepare(A, B, M, N, K, C, ldc, 1, nullptr, cv, &g);
     if (st != PF_OK) return st;
     if (copy2_done) *copy2_done = false;
-    if (copy2 && g.p.splits > 1) {
+    if (copy2) {
         g.p.C2 = copy2; g.p.ldc2 = ldc2;
         if (copy2_done) *copy2_done = true;
     }
@@ -944,7 +963,7 @@ int stage_operand(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& 
     if (tma_ok(p, ld)) { out->p = p; out->ld = ld; return 0; }
     if (cols % 8 == 0) return 1;   // the workspace query reserves repack room only for ragged widths
     const int64_t ldp = pad8(cols);
-    list->jobs[list->count++] = RepackJob{p, ld, scratch, ldp, rows, cols, ldp};
+    list->jobs[list->count++] = RepackJob{p, ld, scratch, ldp, rows, cols};
     out->p = scratch; out->ld = ldp;
     scratch += align_up(static_cast<size_t>(rows) * ldp * 2, 256);
     return 0;
@@ -1080,7 +1099,7 @@ int linear_bwd(const LinearArgs& a, int* handled) {
         if (tma_ok(a.T, a.ldt)) { T.p = a.T; T.ld = a.ldt; }
         else if (a.r % 8 == 0) return PF_OK;   // odd pitch on an even width: FMA path
         else {
-            repacks.jobs[repacks.count++] = RepackJob{a.T, a.ldt, Tbuf, pad8(a.r), a.m, a.r, pad8(a.r)};
+            repacks.jobs[repacks.count++] = RepackJob{a.T, a.ldt, Tbuf, pad8(a.r), a.m, a.r};
             T.p = Tbuf; T.ld = pad8(a.r);
         }
     }
@@ -1234,33 +1253,69 @@ GroupedPlan grouped_plan(int groups, int64_t m, int64_t k, int64_t n, int64_t r)
     return g;
 }
 bool grouped_ok(const void* p, int64_t ld, int64_t gs) { return tma_ok(p, ld) && gs % 8 == 0; }
+
+// A grouped operand that TMA must read: as it is, or (ragged widths) all its groups copied to `scratch` at a
+// padded pitch.  A shared operand is one matrix.
+struct StagedGroups {
+    const void* p;
+    int64_t ld, gs;
+};
+int stage_groups(const void* p, int64_t ld, int64_t gs, int groups, bool shared, int64_t rows, int64_t cols, char*& scratch,
+                 StagedGroups* out, RepackList* list) {
+    *out = StagedGroups{p, ld, gs};
+    if (grouped_ok(p, ld, gs)) return 0;
+    if (cols % 8 == 0) return 1;          // the workspace query reserves repack room only for ragged widths
+    const int64_t ldp = pad8(cols), n = shared ? 1 : groups;
+    list->jobs[list->count++] = RepackJob{p, ld, scratch, ldp, rows, cols, n, gs};
+    *out = StagedGroups{scratch, ldp, shared ? 0 : rows * ldp};
+    scratch += align_up(static_cast<size_t>(n) * rows * ldp * 2, 256);
+    return 0;
+}
+size_t groups_room(int groups, int64_t rows, int64_t cols) {
+    return cols % 8 == 0 ? 0 : align_up(static_cast<size_t>(groups) * rows * pad8(cols) * 2, 256);
+}
 }  // namespace
 
 size_t grouped_workspace(int groups, int64_t m, int64_t k, int64_t n, int64_t r, bool bwd) {
     const GroupedPlan g = grouped_plan(groups, m, k, n, r);
-    return g.t_bytes + g.p1_bytes + (bwd ? g.t_bytes + g.pu_bytes + g.pv_bytes : 0);
+    size_t b = g.t_bytes + g.p1_bytes + (bwd ? g.t_bytes + g.pu_bytes + g.pv_bytes : 0);
+    b += groups_room(groups, m, k) + groups_room(groups, k, r) + groups_room(groups, n, r);      // x, U, V
+    if (bwd) b += groups_room(groups, m, n) + groups_room(groups, m, r);                          // dY, T
+    return b;
 }
 
 int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     *handled = 0;
     if (encode_fn() == nullptr || a.groups > 1024 || a.k > (1 << 22) || a.n > (1 << 22) || a.r > (1 << 22)) return PF_OK;
-    if (!grouped_ok(a.x, a.ldx, a.sx) || !grouped_ok(a.U, a.ldu, a.su) || !grouped_ok(a.V, a.ldv, a.sv)) return PF_OK;
     const GroupedPlan gp = grouped_plan(a.groups, a.m, a.k, a.n, a.r);
-    // T: the stash itself when TMA can read it back, else scratch at a padded pitch (copied out afterwards)
+    const bool shared_x = a.sx == 0 && a.groups > 1;
+    char* ws = a.ws;
+    char* Tbuf = ws; ws += gp.t_bytes;
+    float* p1 = reinterpret_cast<float*>(ws); ws += gp.p1_bytes;
+    StagedGroups x, U, V;
+    RepackList repacks;
+    if (stage_groups(a.x, a.ldx, a.sx, a.groups, shared_x, a.m, a.k, ws, &x, &repacks) ||
+        stage_groups(a.U, a.ldu, a.su, a.groups, false, a.k, a.r, ws, &U, &repacks) ||
+        stage_groups(a.V, a.ldv, a.sv, a.groups, false, a.n, a.r, ws, &V, &repacks))
+        return PF_OK;
+    // T: the stash itself when TMA can read it back, else scratch at a padded pitch; the first product then
+    // writes the stash beside it
     const bool stash_direct = a.T && grouped_ok(a.T, a.ldt, a.st);
-    if (a.T && !stash_direct) return PF_OK;
-    void* T = stash_direct ? a.T : static_cast<void*>(a.ws);
+    void* T = stash_direct ? a.T : static_cast<void*>(Tbuf);
     const int64_t ldT = stash_direct ? a.ldt : pad8(a.r), sT = stash_direct ? a.st : a.m * pad8(a.r);
-    float* p1 = reinterpret_cast<float*>(a.ws + gp.t_bytes);
     GemmLaunch g1, g2;
     const Grouping gt{a.groups, sT, false}, gy{a.groups, a.sy, false};
-    int st = gemm_prepare({a.x, a.ldx, false, a.sx}, {a.U, a.ldu, true, a.su}, a.m, a.r, a.k, T, ldT, gp.s1, p1, nullptr, &g1, &gt);
+    int st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, T, ldT, gp.s1, p1, nullptr, &g1, &gt);
     if (st == PF_OK)
-        st = gemm_prepare({T, ldT, false, sT}, {a.V, a.ldv, false, a.sv}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, nullptr, &g2, &gy);
+        st = gemm_prepare({T, ldT, false, sT}, {V.p, V.ld, false, V.gs}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, nullptr, &g2, &gy);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
+    if (a.T && !stash_direct) {
+        g1.p.C2 = a.T; g1.p.ldc2 = a.ldt; g1.p.c2_gstride = a.st;
+    }
     *handled = 1;
-    st = launch_prepared(g1, a.stream);
+    st = repacks.flush(a.stream);
+    if (st == PF_OK) st = launch_prepared(g1, a.stream);
     if (st != PF_OK) return st;
     return launch_prepared(g2, a.stream);
 }
@@ -1268,34 +1323,39 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
 int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     *handled = 0;
     if (encode_fn() == nullptr || a.groups > 1024 || a.k > (1 << 22) || a.n > (1 << 22) || a.r > (1 << 22)) return PF_OK;
-    if (!grouped_ok(a.x, a.ldx, a.sx) || !grouped_ok(a.U, a.ldu, a.su) || !grouped_ok(a.V, a.ldv, a.sv) ||
-        !grouped_ok(a.dY, a.lddy, a.sdy) || (a.T && !grouped_ok(a.T, a.ldt, a.st)))
-        return PF_OK;
     const GroupedPlan gp = grouped_plan(a.groups, a.m, a.k, a.n, a.r);
+    const bool shared_x = a.sx == 0 && a.groups > 1;
     char* ws = a.ws;
     void* Tbuf = ws; ws += gp.t_bytes;
     float* p1 = reinterpret_cast<float*>(ws); ws += gp.p1_bytes;
     void* Gbuf = ws; ws += gp.t_bytes;
     float* pu = reinterpret_cast<float*>(ws); ws += gp.pu_bytes;
-    float* pv = reinterpret_cast<float*>(ws);
+    float* pv = reinterpret_cast<float*>(ws); ws += gp.pv_bytes;
     const int64_t ldW = pad8(a.r), sW = a.m * pad8(a.r);
-    const void* T = a.T ? a.T : Tbuf;
-    const int64_t ldT = a.T ? a.ldt : ldW, sT = a.T ? a.st : sW;
-    const bool shared_x = a.sx == 0 && a.groups > 1;
+    StagedGroups x, U, V, dY, T{Tbuf, ldW, sW};
+    RepackList repacks;
+    if (stage_groups(a.x, a.ldx, a.sx, a.groups, shared_x, a.m, a.k, ws, &x, &repacks) ||
+        stage_groups(a.U, a.ldu, a.su, a.groups, false, a.k, a.r, ws, &U, &repacks) ||
+        stage_groups(a.V, a.ldv, a.sv, a.groups, false, a.n, a.r, ws, &V, &repacks) ||
+        stage_groups(a.dY, a.lddy, a.sdy, a.groups, false, a.m, a.n, ws, &dY, &repacks) ||
+        (a.T && stage_groups(a.T, a.ldt, a.st, a.groups, false, a.m, a.r, ws, &T, &repacks)))
+        return PF_OK;
     GemmLaunch gT, gG, gV, gU, gX;
     const Grouping gw{a.groups, sW, false}, gdv{a.groups, a.sdv, false}, gdu{a.groups, a.sdu, false};
     const Grouping gdx{a.groups, shared_x ? 0 : a.sdx, shared_x};
     int st = PF_OK;
-    if (!a.T) st = gemm_prepare({a.x, a.ldx, false, a.sx}, {a.U, a.ldu, true, a.su}, a.m, a.r, a.k, Tbuf, ldW, gp.s1, p1, nullptr, &gT, &gw);
+    if (!a.T) st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, Tbuf, ldW, gp.s1, p1, nullptr, &gT, &gw);
     // the recomputed T and G share the slice buffer p1: they are separate launches, one after the other
-    if (st == PF_OK) st = gemm_prepare({a.dY, a.lddy, false, a.sdy}, {a.V, a.ldv, true, a.sv}, a.m, a.r, a.n, Gbuf, ldW, gp.sg, p1, nullptr, &gG, &gw);
-    if (st == PF_OK) st = gemm_prepare({a.dY, a.lddy, true, a.sdy}, {T, ldT, true, sT}, a.n, a.r, a.m, a.dV, a.lddv, gp.sv, pv, nullptr, &gV, &gdv);
-    if (st == PF_OK) st = gemm_prepare({a.x, a.ldx, true, a.sx}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, gp.su, pu, nullptr, &gU, &gdu);
+    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, false, dY.gs}, {V.p, V.ld, true, V.gs}, a.m, a.r, a.n, Gbuf, ldW, gp.sg, p1, nullptr, &gG, &gw);
+    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, true, dY.gs}, {T.p, T.ld, true, T.gs}, a.n, a.r, a.m, a.dV, a.lddv, gp.sv, pv, nullptr, &gV, &gdv);
+    if (st == PF_OK) st = gemm_prepare({x.p, x.ld, true, x.gs}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, gp.su, pu, nullptr, &gU, &gdu);
     if (st == PF_OK && a.dX)
-        st = gemm_prepare({Gbuf, ldW, false, sW}, {a.U, a.ldu, false, a.su}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gX, &gdx);
+        st = gemm_prepare({Gbuf, ldW, false, sW}, {U.p, U.ld, false, U.gs}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gX, &gdx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
     *handled = 1;
+    st = repacks.flush(a.stream);
+    if (st != PF_OK) return st;
     if (!a.T) {
         st = launch_prepared(gT, a.stream);
         if (st != PF_OK) return st;
