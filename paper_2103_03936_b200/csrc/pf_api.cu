@@ -633,7 +633,7 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         int nj = 0;
         if (su_info.splits > 1)
             jobs[nj++] = SliceSums{su_info.partial, user_dU, R, static_cast<int>(Keff), R, su_info.splits, su_info.bn,
-                                   su_info.tiles_x, su_info.tiles_y, g_f32, g_acc};
+                                   su_info.tiles_x, su_info.tiles_y, g_f32, g_acc, su_info.conv_c};
         else
             PF_CUDA(grad_combine(user_dU, R, gdtype, dU, R, dtype, Keff, R, g_acc, stream));
         if (sv_info.splits > 1)

@@ -101,6 +101,7 @@ struct SliceSums {
     long long ld;
     int M, N, splits, bn, tiles_x, tiles_y;
     bool out_f32, accumulate;
+    int conv_c = 0;     // > 0: rows are pairs of 64-channel blocks of a [taps][conv_c] index
 };
 cudaError_t slices_to_gradients(const SliceSums* jobs, int count, cudaStream_t stream);
 // Backward of y = act(z + bias): dY becomes dZ in place, db (optional) its column sums.  `part` holds

@@ -1,13 +1,5 @@
-// Tensor-core path (bf16 storage) for sm_100a: tcgen05 MMAs with accumulators in tensor memory,
-// operands staged in shared memory by TMA through an mbarrier pipeline.
-//
-// Kernel in this file:
-//   tc_gemm_kernel<BN>  C[M,N] = A * B for every operand orientation the factorized layers need
-//                       (row-major operands read either along or across the contraction index,
-//                       i.e. K-major or MN-major shared-memory descriptors), with an optional
-//                       reduction split whose fp32 partials are summed in a fixed order.
-// Warp roles: warp 0 = TMA producer of operand A, warp 1 = TMEM allocation + MMA issue, warps 2..5 =
-// epilogue (each owns the 32 TMEM lanes of its warp-id quadrant), warp 6 = TMA producer of operand B.
+// Tensor-core path (bf16 storage) for sm_100a: host planning of every product (tensor maps, tiles, slices of split
+// contractions, which products share a launch) and the plain product kernels of pf_tc_gemm_kernel.cuh.
 #include "pf_tc.h"
 
 #include <cuda.h>
@@ -16,552 +8,19 @@
 #include <atomic>
 #include <mutex>
 
+#include "pf_tc_gemm_kernel.cuh"
 #include "pf_tc_host.h"
-#include "pf_tc_prims.cuh"
 
 namespace pf {
 namespace tc {
 namespace {
 
-constexpr int kBM = 128;       // rows of the output tile = TMEM lanes
-constexpr int kBK = 64;        // contraction elements per pipeline stage (128 bytes of bf16)
-constexpr int kMaxStages = 6;
-constexpr int kGemmThreads = 224;   // A producer, MMA issue, 4 epilogue warps, B producer
 constexpr int kFixSlots = 32;  // counter sets handed out round-robin to launches that split a contraction
 constexpr int kFixTiles = 160; // output tiles of one split product (tiles * slices never exceeds the SM count)
 
 // Arrival / departure counters of the in-kernel slice sum, two per output tile.  They are zero
 // between launches: the last CTA to leave a tile clears its pair.
 __device__ unsigned int g_fix_counters[kFixSlots][kFixTiles * 2];
-
-struct GemmCtl {
-    uint64_t full[kMaxStages];
-    uint64_t empty[kMaxStages];
-    uint64_t tmem_full;
-    uint64_t fix_full;       // the slices this CTA sums have been copied into shared memory
-    uint32_t tmem_base;
-    uint32_t abort;
-    uint32_t fix_ok;
-};
-
-struct GemmParams {
-    int M, N, K;
-    int a_mn, b_mn;          // 1 = operand stored with the M/N index contiguous
-    int kb_per_split;        // k-blocks handled by one z-slice
-    int splits;
-    int num_stages;
-    int bn;                  // columns of an output tile (the kernel's template value; 64 or 128 in a shared launch)
-    int tiles_x;             // row tiles of this product (tile id = column tile * tiles_x + row tile)
-    void* C;                 // bf16 [M, ldc]
-    long long ldc;
-    void* C2;                // optional second copy of the result at another pitch, groups c2_gstride elements apart
-    long long ldc2, c2_gstride;
-    float* partial;          // splits > 1: fp32 slices, one 128 x BN block per (tile, slice)
-    unsigned int* counters;  // splits > 1: two counters per tile
-    unsigned int* status;
-    // Implicit-GEMM convolution operand A (tmA is then a 4-D NHWC map):
-    //   conv_mode 1 (dX): A K-major; row tile = cv_box_h full-width image rows of dT; k-block =
-    //                     (tap, 64-rank block), tap offsets flipped; B rows are offset by tap * cv_C.
-    //   conv_mode 2 (dU): A MN-major; row tile = (tap, 128-channel block) of the unrolled factor;
-    //                     k-block = 64 pixels (cv_box_h full-width rows) of the image x.
-    int conv_mode, cv_blks, cv_kw, cv_pad, cv_C, cv_box_h, cv_tpi;
-    int rows_tile;           // output rows per CTA: 128, or cv_box_h * W pixels for conv_mode 1
-    int kpix;                // conv_mode 2: pixels per k-block (cv_box_h * W <= 64), else 64
-    int nkb_total;           // k-blocks of the whole contraction
-    int independent;         // 1: reads nothing the preceding kernel of the stream writes (see gemm_tile)
-    // Grouped products (several problems of one shape in a launch): tmA / tmB are 3-D maps whose outermost
-    // coordinate is the group (a shared operand has one group only), outputs of group g start g * c_gstride
-    // elements after C.  kb_per_group > 0 instead makes the group part of the CONTRACTION: k-block kb reads
-    // group kb / kb_per_group, 64-element block kb % kb_per_group of both operands (the sum over groups of
-    // A_g B_g^T, i.e. dX of several factor pairs that share one input).
-    int groups, a_shared, b_shared, kb_per_group, tiles_y;
-    long long c_gstride;
-};
-
-__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
-        : "memory");
-}
-
-// One output tile (128 rows x BN columns) of C = A * B, or one slice of its contraction.
-//
-// Epilogue.  Unsplit: each epilogue warp turns its 32 accumulator rows into bf16, transposes them
-// through a padded shared-memory panel and writes whole 128-byte row segments (any pitch, any
-// alignment, clipped at the matrix edge).  Split: the fp32 slice goes to the workspace in the
-// order [32-column chunk][4-column group][row][4], which makes every store instruction of a warp
-// one contiguous 512-byte run; then the CTAs of a tile meet at a counter and each sums, in slice
-// order, its share of the rows over all slices and writes bf16 (bit-reproducible, no second launch).
-template <int BN>
-__device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p,
-                                          const int bx, const int by, const int bz, const int bg) {
-    constexpr uint32_t kABytes = kBM * kBK * 2;          // 16 KB
-    constexpr uint32_t kBBytes = BN * kBK * 2;
-    constexpr uint32_t kStageBytes = kABytes + kBBytes;
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t raw_addr = smem_u32(smem_raw);
-    uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
-    GemmCtl* ctl = reinterpret_cast<GemmCtl*>(smem);
-    uint8_t* tiles = smem + 1024;
-    volatile uint32_t* abort_flag = &ctl->abort;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = bx * p.rows_tile, n0 = by * BN;
-    const int nkb_total = p.nkb_total;
-    const int kb_beg = bz * p.kb_per_split;
-    const int kb_end = min(nkb_total, kb_beg + p.kb_per_split);
-    const int nkb = kb_end - kb_beg;
-    const uint32_t NS = static_cast<uint32_t>(p.num_stages);
-    const int tile = (bg * p.tiles_y + by) * p.tiles_x + bx;
-    const bool grouped = p.groups > 1 || p.kb_per_group > 0;
-
-    if (threadIdx.x == 0) {
-        for (uint32_t s = 0; s < NS; ++s) {
-            mbar_init(smem_u32(&ctl->full[s]), 2);     // one expect_tx arrival per producer thread
-            mbar_init(smem_u32(&ctl->empty[s]), 1);
-        }
-        mbar_init(smem_u32(&ctl->tmem_full), 1);
-        mbar_init(smem_u32(&ctl->fix_full), 1);
-        ctl->abort = 0;
-        ctl->fix_ok = 0;
-        fence_barrier_init();
-        fence_proxy_async_smem();
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
-    }
-    if (p.conv_mode == 2 && p.kpix < 64) {
-        // k-blocks hold fewer than 64 pixels: the unused contraction rows of every A stage must be
-        // zero (TMA never writes them), so that they add nothing to the sum
-        for (int i = threadIdx.x; i < static_cast<int>(NS) * static_cast<int>(kABytes / 16); i += blockDim.x) {
-            const int st = i / static_cast<int>(kABytes / 16), off = i - st * static_cast<int>(kABytes / 16);
-            *reinterpret_cast<uint4*>(tiles + st * kStageBytes + off * 16) = make_uint4(0, 0, 0, 0);
-        }
-        fence_proxy_async_smem();
-    }
-    if (warp == 1) tmem_alloc(smem_u32(&ctl->tmem_base), BN);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    // A product marked independent reads nothing that the kernel launched just before it writes, so
-    // it does not wait for that kernel: its blocks run beside it on SMs that kernel leaves free.  (Every
-    // kernel of this library lets its successor start only after its own wait has returned, i.e. once
-    // everything older in the stream is complete, so older results are safe to read.)
-    if (!p.independent) pdl_wait();     // everything above overlapped the previous kernel's tail
-    pdl_launch_dependents();
-    const uint32_t tmem_base = ctl->tmem_base;
-
-    // Producers and MMA issuer are each one thread chosen with elect.sync that runs its whole role
-    // (a thread singled out by a lane-id test issues TMA / tcgen05 instructions several times slower).
-    // Two producers, one per operand: a producer thread needs about 130 ns per stage for its loop,
-    // barrier wait and expect_tx plus 40 ns per TMA instruction, which with four tile loads per
-    // stage paced the whole pipeline when one thread issued both operands.
-    if (warp == 0 || warp == 6) {
-        if (elect_one()) {
-            const bool do_a = warp == 0;
-            const uint32_t my_bytes = !do_a ? kBBytes
-                                      : p.conv_mode == 1 ? static_cast<uint32_t>(p.rows_tile) * 128u
-                                      : p.conv_mode == 2 ? static_cast<uint32_t>(p.kpix) * 256u
-                                                         : kABytes;
-            uint32_t s = 0, ph = 0;
-            // convolution operands: tap / block / image positions advance as counters (an integer
-            // division per k-block would sit on the producer's critical path)
-            int c1_rb = 0, c1_ta = 0, c1_tb = 0, c1_img = 0, c1_h0 = 0;     // conv_mode 1
-            int c2_c0 = 0, c2_x = 0, c2_y = 0, c2_img = 0, c2_t = 0;          // conv_mode 2
-            if (p.conv_mode == 1) {
-                const int tap = kb_beg / p.cv_blks;
-                c1_rb = kb_beg - tap * p.cv_blks;
-                c1_ta = tap / p.cv_kw;
-                c1_tb = tap - c1_ta * p.cv_kw;
-                c1_img = bx / p.cv_tpi;
-                c1_h0 = (bx - c1_img * p.cv_tpi) * p.cv_box_h + p.cv_pad;
-            } else if (p.conv_mode == 2) {
-                const int tap = m0 / p.cv_C;
-                c2_c0 = m0 - tap * p.cv_C;
-                const int ta = tap / p.cv_kw;
-                c2_x = tap - ta * p.cv_kw - p.cv_pad;
-                c2_y = ta - p.cv_pad;
-                c2_img = kb_beg / p.cv_tpi;
-                c2_t = kb_beg - c2_img * p.cv_tpi;
-            }
-            for (int i = 0; i < nkb; ++i) {
-                if (!mbar_wait(smem_u32(&ctl->empty[s]), ph ^ 1u, abort_flag, p.status)) break;
-                const uint32_t full = smem_u32(&ctl->full[s]);
-                const uint32_t a_dst = smem_u32(tiles + s * kStageBytes);
-                const uint32_t b_dst = a_dst + kABytes;
-                mbar_expect_tx(full, my_bytes);
-                const int k0 = (kb_beg + i) * kBK;
-                if (p.conv_mode == 1) {
-                    if (do_a) tma_load_4d(a_dst, &tmA, full, c1_rb * 64, p.cv_pad - c1_tb, c1_h0 - c1_ta, c1_img);
-                    else tma_load_2d(b_dst, &tmB, full, c1_rb * 64, (c1_ta * p.cv_kw + c1_tb) * p.cv_C + n0);
-                    if (++c1_rb == p.cv_blks) {
-                        c1_rb = 0;
-                        if (++c1_tb == p.cv_kw) { c1_tb = 0; ++c1_ta; }
-                    }
-                    if (++s == NS) { s = 0; ph ^= 1u; }
-                    continue;
-                }
-                if (p.conv_mode == 2) {
-                    const int hy = c2_t * p.cv_box_h + c2_y;
-                    if (do_a) {
-                        tma_load_4d(a_dst, &tmA, full, c2_c0, c2_x, hy, c2_img);
-                        tma_load_4d(a_dst + 8192, &tmA, full, c2_c0 + 64, c2_x, hy, c2_img);
-                    } else {
-#pragma unroll
-                        for (int h = 0; h < BN / 64; ++h)
-                            tma_load_2d(b_dst + h * 8192, &tmB, full, n0 + 64 * h, (kb_beg + i) * p.kpix);
-                    }
-                    if (++c2_t == p.cv_tpi) { c2_t = 0; ++c2_img; }
-                    if (++s == NS) { s = 0; ph ^= 1u; }
-                    continue;
-                } else if (grouped) {
-                    int g = bg, kk0 = k0;
-                    if (p.kb_per_group > 0) {
-                        g = (kb_beg + i) / p.kb_per_group;
-                        kk0 = ((kb_beg + i) - g * p.kb_per_group) * kBK;
-                    }
-                    if (do_a) {
-                        const int ga = p.a_shared ? 0 : g;
-                        if (p.a_mn) {
-                            tma_load_3d(a_dst, &tmA, full, m0, kk0, ga);
-                            tma_load_3d(a_dst + 8192, &tmA, full, m0 + 64, kk0, ga);
-                        } else {
-                            tma_load_3d(a_dst, &tmA, full, kk0, m0, ga);
-                        }
-                    } else {
-                        const int gb = p.b_shared ? 0 : g;
-                        if (p.b_mn) {
-#pragma unroll
-                            for (int h = 0; h < BN / 64; ++h) tma_load_3d(b_dst + h * 8192, &tmB, full, n0 + 64 * h, kk0, gb);
-                        } else {
-                            tma_load_3d(b_dst, &tmB, full, kk0, n0, gb);
-                        }
-                    }
-                } else if (do_a) {
-                    if (p.a_mn) {
-                        tma_load_2d(a_dst, &tmA, full, m0, k0);
-                        tma_load_2d(a_dst + 8192, &tmA, full, m0 + 64, k0);
-                    } else {
-                        tma_load_2d(a_dst, &tmA, full, k0, m0);
-                    }
-                } else if (p.b_mn) {
-#pragma unroll
-                    for (int h = 0; h < BN / 64; ++h) tma_load_2d(b_dst + h * 8192, &tmB, full, n0 + 64 * h, k0);
-                } else {
-                    tma_load_2d(b_dst, &tmB, full, k0, n0);
-                }
-                if (++s == NS) { s = 0; ph ^= 1u; }
-            }
-        }
-    } else if (warp == 1) {
-        if (elect_one()) {
-            const uint32_t idesc = make_idesc_bf16(kBM, BN, p.a_mn, p.b_mn);
-            // K-major: 8-row groups 1024 B apart, 16 contraction elements = 32 B along the row.
-            // MN-major: 64-element M/N panels 8192 B apart (LBO), 8 contraction rows per
-            // 1024 B group (SBO), 16 contraction rows = 2048 B.
-            const uint32_t a_step = p.a_mn ? 128u : 2u, b_step = p.b_mn ? 128u : 2u;   // in 16-byte units
-            uint32_t s = 0, ph = 0;
-            bool ok = true;
-            for (int i = 0; i < nkb; ++i) {
-                ok = mbar_wait(smem_u32(&ctl->full[s]), ph, abort_flag, p.status);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a_addr = smem_u32(tiles + s * kStageBytes);
-                const uint32_t b_addr = a_addr + kABytes;
-                const uint64_t a_desc = p.a_mn ? make_smem_desc(a_addr, 8192, 1024) : make_smem_desc(a_addr, 16, 1024);
-                const uint64_t b_desc = p.b_mn ? make_smem_desc(b_addr, 8192, 1024) : make_smem_desc(b_addr, 16, 1024);
-                tc_mma_bf16(tmem_base, a_desc, b_desc, idesc, i > 0 ? 1u : 0u);
-                tc_mma_bf16(tmem_base, a_desc + a_step, b_desc + b_step, idesc, 1u);
-                tc_mma_bf16(tmem_base, a_desc + 2 * a_step, b_desc + 2 * b_step, idesc, 1u);
-                tc_mma_bf16(tmem_base, a_desc + 3 * a_step, b_desc + 3 * b_step, idesc, 1u);
-                tc_commit(smem_u32(&ctl->empty[s]));   // frees the stage once these MMAs have read it
-                if (++s == NS) { s = 0; ph ^= 1u; }
-            }
-            if (ok) tc_commit(smem_u32(&ctl->tmem_full));
-        }
-    } else if (warp < 6) {
-        const int q = warp & 3;                          // TMEM lane quadrant this warp may access
-        const bool ok = mbar_wait_warp(smem_u32(&ctl->tmem_full), 0, abort_flag, p.status);
-        tc_fence_after();
-        if (ok) {
-            const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-            if (p.splits > 1) {
-                // fp32 slice: this warp's 32 rows go to shared memory as rows of BN floats (the 16-byte
-                // pieces of a row XOR-permuted by the row, which keeps the writes and the later reads
-                // free of bank conflicts), leave as ONE bulk copy of 32 x BN x 4 bytes to the
-                // workspace (the workspace keeps the permuted order; only the sum below reads it),
-                // and the warp reports its arrival once the copy has completed
-                constexpr uint32_t kRowBytes = BN * 4, kPieces = BN / 4;
-                const uint32_t wbase = smem_u32(tiles) + static_cast<uint32_t>(q * 32) * kRowBytes;
-                const uint32_t rbase = wbase + static_cast<uint32_t>(lane) * kRowBytes;
-                const uint32_t rsw = static_cast<uint32_t>(q * 32 + lane) & (kPieces - 1);
-#pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
-                    uint32_t v[32];
-                    tmem_ld32(lane_base + c * 32, v);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int g = 0; g < 8; ++g)
-                        st_shared_v4(rbase + (((static_cast<uint32_t>(c * 8 + g)) ^ rsw) << 4),
-                                     make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]));
-                }
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    uint8_t* dst = reinterpret_cast<uint8_t*>(p.partial) +
-                                   (static_cast<size_t>(tile) * p.splits + bz) * (static_cast<size_t>(kBM) * kRowBytes) +
-                                   static_cast<size_t>(q * 32) * kRowBytes;
-                    bulk_store(dst, wbase, 32u * kRowBytes);
-                    tma_store_commit();
-                    tma_store_wait_all();          // the rows are in the workspace
-                    fence_proxy_async_all();
-                    __threadfence();
-                    atomicAdd(p.counters + 2 * tile, 1u);
-                }
-            } else {
-                // every MMA has completed, so the pipeline stages are free: 32 x 33-word panel per warp
-                uint32_t* stg = reinterpret_cast<uint32_t*>(tiles) + (warp - 2) * (32 * 33);
-                __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
-                const bool pair_ok = (p.ldc % 2) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 3) == 0;
-                const bool vec_ok = (p.ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0;
-                if (vec_ok) {
-                    // 16-byte aligned rows: stage 32 rows x 64 columns (128 bytes per row, 16-byte pieces
-                    // XOR-swizzled by the row so that both passes are free of bank conflicts), then
-                    // store four whole 128-byte row segments per instruction
-                    const uint32_t panel = smem_u32(tiles) + static_cast<uint32_t>(warp - 2) * 4096u;
-                    const uint32_t own = panel + static_cast<uint32_t>(lane) * 128u, sw = static_cast<uint32_t>(lane & 7);
-                    const int sub = lane >> 3, piece = lane & 7;
-                    const size_t row_step = static_cast<size_t>(4) * p.ldc;
-#pragma unroll 1
-                    for (int c = 0; c < BN / 64; ++c) {
-                        uint32_t v0[32], v1[32];
-                        tmem_ld32(lane_base + c * 64, v0);
-                        tmem_ld32(lane_base + c * 64 + 32, v1);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            uint4 o;
-                            o.x = pack_bf16x2(__uint_as_float(v0[8 * t + 0]), __uint_as_float(v0[8 * t + 1]));
-                            o.y = pack_bf16x2(__uint_as_float(v0[8 * t + 2]), __uint_as_float(v0[8 * t + 3]));
-                            o.z = pack_bf16x2(__uint_as_float(v0[8 * t + 4]), __uint_as_float(v0[8 * t + 5]));
-                            o.w = pack_bf16x2(__uint_as_float(v0[8 * t + 6]), __uint_as_float(v0[8 * t + 7]));
-                            st_shared_v4(own + ((static_cast<uint32_t>(t) ^ sw) << 4), o);
-                            o.x = pack_bf16x2(__uint_as_float(v1[8 * t + 0]), __uint_as_float(v1[8 * t + 1]));
-                            o.y = pack_bf16x2(__uint_as_float(v1[8 * t + 2]), __uint_as_float(v1[8 * t + 3]));
-                            o.z = pack_bf16x2(__uint_as_float(v1[8 * t + 4]), __uint_as_float(v1[8 * t + 5]));
-                            o.w = pack_bf16x2(__uint_as_float(v1[8 * t + 6]), __uint_as_float(v1[8 * t + 7]));
-                            st_shared_v4(own + ((static_cast<uint32_t>(4 + t) ^ sw) << 4), o);
-                        }
-                        __syncwarp();
-                        const int col = n0 + c * 64 + piece * 8;
-                        const int rin0 = q * 32 + sub;
-                        __nv_bfloat16* dst = Cb + static_cast<size_t>(m0 + rin0) * p.ldc + col;
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int rr = i * 4 + sub, rin_i = rin0 + i * 4;
-                            const uint4 w = ld_shared_v4(panel + static_cast<uint32_t>(rr) * 128u +
-                                                         ((static_cast<uint32_t>(piece) ^ static_cast<uint32_t>(rr & 7)) << 4));
-                            if (m0 + rin_i < p.M && rin_i < p.rows_tile) {
-                                if (col + 8 <= p.N) {
-                                    *reinterpret_cast<uint4*>(dst) = w;
-                                } else {
-                                    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e)
-                                        if (col + e < p.N)
-                                            dst[e] = __ushort_as_bfloat16(static_cast<unsigned short>((ws[e >> 1] >> ((e & 1) * 16)) & 0xffffu));
-                                }
-                            }
-                            dst += row_step;
-                        }
-                        if (p.C2) {          // the second copy, at a pitch that takes element pairs at best
-                            __nv_bfloat16* C2b = reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride;
-                            const bool pair2 = (p.ldc2 % 2) == 0 && (reinterpret_cast<uintptr_t>(C2b) & 3) == 0;
-                            const int c2 = n0 + c * 64 + 2 * lane;
-                            for (int j = 0; j < 32; ++j) {
-                                const int rowj = m0 + q * 32 + j;
-                                if (rowj >= p.M || q * 32 + j >= p.rows_tile) break;
-                                uint32_t w;
-                                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(panel + static_cast<uint32_t>(j) * 128u +
-                                             ((static_cast<uint32_t>(lane >> 2) ^ static_cast<uint32_t>(j & 7)) << 4) + static_cast<uint32_t>(lane & 3) * 4u));
-                                __nv_bfloat16* d2 = C2b + static_cast<size_t>(rowj) * p.ldc2 + c2;
-                                if (pair2 && c2 + 1 < p.N) {
-                                    *reinterpret_cast<uint32_t*>(d2) = w;
-                                } else {
-                                    if (c2 < p.N) d2[0] = __ushort_as_bfloat16(static_cast<unsigned short>(w & 0xffffu));
-                                    if (c2 + 1 < p.N) d2[1] = __ushort_as_bfloat16(static_cast<unsigned short>(w >> 16));
-                                }
-                            }
-                        }
-                        __syncwarp();
-                    }
-                } else
-#pragma unroll 1
-                for (int c = 0; c < BN / 64; ++c) {
-                    uint32_t v0[32], v1[32];
-                    tmem_ld32(lane_base + c * 64, v0);
-                    tmem_ld32(lane_base + c * 64 + 32, v1);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int w = 0; w < 16; ++w) {
-                        stg[lane * 33 + w] = pack_bf16x2(__uint_as_float(v0[2 * w]), __uint_as_float(v0[2 * w + 1]));
-                        stg[lane * 33 + 16 + w] = pack_bf16x2(__uint_as_float(v1[2 * w]), __uint_as_float(v1[2 * w + 1]));
-                    }
-                    __syncwarp();
-                    const int col = n0 + c * 64 + 2 * lane;
-#pragma unroll 4
-                    for (int j = 0; j < 32; ++j) {
-                        const int rj = q * 32 + j, rowj = m0 + rj;
-                        if (rowj < p.M && rj < p.rows_tile) {
-                            const uint32_t w = stg[j * 33 + lane];
-                            __nv_bfloat16* dst = Cb + static_cast<size_t>(rowj) * p.ldc + col;
-                            if (pair_ok && col + 1 < p.N) {
-                                *reinterpret_cast<uint32_t*>(dst) = w;
-                            } else {
-                                if (col < p.N) dst[0] = __ushort_as_bfloat16(static_cast<unsigned short>(w & 0xffffu));
-                                if (col + 1 < p.N) dst[1] = __ushort_as_bfloat16(static_cast<unsigned short>(w >> 16));
-                            }
-                        }
-                    }
-                    __syncwarp();
-                }
-            }
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, BN);
-    if (p.splits <= 1) return;
-
-    // ---- slice sum: wait until every slice of this tile is in the workspace (four warps of every slice
-    // report), then sum a share of it.  A share is a run of whole rows, contiguous in every slice, so
-    // one bulk copy per slice brings it into the idle pipeline stages: a single trip to L2 for the
-    // whole sum.  The slices are added in slice order (bit-reproducible) and each summed row leaves as
-    // whole 8-byte pieces, a warp writing 256 contiguous bytes per instruction.
-    unsigned int* cnt = p.counters + 2 * tile;
-    const int S = p.splits;
-    constexpr uint32_t kRowBytes = BN * 4, kPieces = BN / 4;
-    const int rper = (kBM + S - 1) / S;
-    const int r_beg = bz * rper;
-    const int nr = max(0, min(kBM, r_beg + rper) - r_beg);
-    const uint32_t share = static_cast<uint32_t>(nr) * kRowBytes;
-    if (threadIdx.x == 0) {
-        uint32_t good = (*abort_flag == 0u) ? 1u : 0u;
-        if (good) {
-            const unsigned int want = 4u * static_cast<unsigned int>(S);
-            const long long t0 = clock64();
-            while (ld_acquire_gpu(cnt) < want) {
-                if (clock64() - t0 > kWaitCycleLimit) {
-                    good = 0u;
-                    if (p.status) atomicExch(p.status, kStatusTimeout);
-                    break;
-                }
-            }
-            __threadfence();
-            fence_proxy_async_all();
-            if (good && nr > 0) {
-                const uint32_t bar = smem_u32(&ctl->fix_full);
-                const uint8_t* src = reinterpret_cast<const uint8_t*>(p.partial) +
-                                     (static_cast<size_t>(tile) * S) * (static_cast<size_t>(kBM) * kRowBytes) +
-                                     static_cast<size_t>(r_beg) * kRowBytes;
-                mbar_expect_tx(bar, share * static_cast<uint32_t>(S));
-                for (int s = 0; s < S; ++s)
-                    bulk_load(smem_u32(tiles) + static_cast<uint32_t>(s) * share,
-                              src + static_cast<size_t>(s) * (static_cast<size_t>(kBM) * kRowBytes), share, bar);
-                good = mbar_wait(bar, 0, abort_flag, p.status) ? 1u : 0u;
-            }
-        }
-        ctl->fix_ok = good;
-    }
-    __syncthreads();
-    if (ctl->fix_ok) {
-        __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
-        __nv_bfloat16* C2b = p.C2 ? reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride : nullptr;
-        const uint32_t base = smem_u32(tiles);
-        const bool vec8 = (p.ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 7) == 0;
-        // consecutive threads take consecutive 16-byte pieces of one row
-        for (int id = threadIdx.x; id < nr * static_cast<int>(kPieces); id += kGemmThreads) {
-            const int rl = id / static_cast<int>(kPieces), pc = id % static_cast<int>(kPieces);
-            const int rr = r_beg + rl;
-            const uint32_t off = static_cast<uint32_t>(rl) * kRowBytes +
-                                 ((static_cast<uint32_t>(pc) ^ (static_cast<uint32_t>(rr) & (kPieces - 1))) << 4);
-            uint4 w = ld_shared_v4(base + off);
-            float4 acc = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
-#pragma unroll 4
-            for (int s = 1; s < S; ++s) {
-                w = ld_shared_v4(base + static_cast<uint32_t>(s) * share + off);
-                acc.x += __uint_as_float(w.x); acc.y += __uint_as_float(w.y);
-                acc.z += __uint_as_float(w.z); acc.w += __uint_as_float(w.w);
-            }
-            const int row = m0 + rr, col = n0 + pc * 4;
-            if (row < p.M) {
-                __nv_bfloat16* dst = Cb + static_cast<size_t>(row) * p.ldc + col;
-                if (vec8 && col + 3 < p.N) {
-                    *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
-                } else {
-                    if (col < p.N) dst[0] = __float2bfloat16_rn(acc.x);
-                    if (col + 1 < p.N) dst[1] = __float2bfloat16_rn(acc.y);
-                    if (col + 2 < p.N) dst[2] = __float2bfloat16_rn(acc.z);
-                    if (col + 3 < p.N) dst[3] = __float2bfloat16_rn(acc.w);
-                }
-                if (C2b) {   // the same sums once more, for a destination whose pitch the first cannot have
-                    __nv_bfloat16* d2 = C2b + static_cast<size_t>(row) * p.ldc2 + col;
-                    if (col < p.N) d2[0] = __float2bfloat16_rn(acc.x);
-                    if (col + 1 < p.N) d2[1] = __float2bfloat16_rn(acc.y);
-                    if (col + 2 < p.N) d2[2] = __float2bfloat16_rn(acc.z);
-                    if (col + 3 < p.N) d2[3] = __float2bfloat16_rn(acc.w);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && ctl->fix_ok) {
-        const unsigned int left = atomicAdd(cnt + 1, 1u);
-        if (left + 1u == static_cast<unsigned int>(S)) {   // every slice has read what it needs
-            cnt[0] = 0u;
-            cnt[1] = 0u;
-            __threadfence();
-        }
-    }
-}
-
-template <int BN>
-__global__ void __launch_bounds__(kGemmThreads, BN <= 128 ? 2 : 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const GemmParams p) {
-    const int sl = p.splits < 1 ? 1 : p.splits;
-    gemm_tile<BN>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
-}
-
-// Up to three independent products in one launch (dU = x^T G, dV = dY^T T and, where it is a plain
-// product, dX of one layer): CTAs [0, end0) work on product 0, [end0, end1) on product 1, the rest on
-// product 2; each decodes (row tile, column tile, slice) from its linear index.  One launch pays the
-// start-up latency once and packs the short CTAs of one product beside the long ones of another.
-// Tiles may be 64 or 128 columns wide per product.
-__device__ __forceinline__ void gemm_any(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, int idx,
-                                         const int2 t) {
-    const int sl = p.splits < 1 ? 1 : p.splits;
-    const int bx = idx % t.x, by = (idx / t.x) % t.y, zz = idx / (t.x * t.y);
-    if (p.bn == 64) gemm_tile<64>(tmA, tmB, p, bx, by, zz % sl, zz / sl);
-    else gemm_tile<128>(tmA, tmB, p, bx, by, zz % sl, zz / sl);
-}
-__global__ void __launch_bounds__(kGemmThreads, 2)
-tc_gemm3_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
-                const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
-                const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
-                const GemmParams p0, const GemmParams p1, const GemmParams p2, const int end0, const int end1,
-                const int2 tiles0, const int2 tiles1, const int2 tiles2) {
-    const int idx = blockIdx.x;
-    if (idx < end0) gemm_any(tmA0, tmB0, p0, idx, tiles0);
-    else if (idx < end1) gemm_any(tmA1, tmB1, p1, idx - end0, tiles1);
-    else gemm_any(tmA2, tmB2, p2, idx - end1, tiles2);
-}
 
 // ------------------------------------------------------------------------------ host side
 // One operand of C = A * B.  `mn_major == false`: stored [MN, K] row-major (contraction index
@@ -638,17 +97,14 @@ int pick_stages(int bn, int64_t ctas) {
 template <int BN>
 cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p, dim3 grid,
                         cudaStream_t stream) {
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(std::min(gemm_smem(BN, kMaxStages), static_cast<size_t>(227 * 1024))));
-        if (e != cudaSuccess) return e;
-        configured[dev] = true;
+    cudaError_t e;
+    if (p.conv_mode != 0) {
+        e = launch_gemm_conv(BN, grid, gemm_smem(BN, p.num_stages), stream, ta, tb, p);
+    } else {
+        e = allow_smem(tc_gemm_kernel<BN, 0>, std::min(gemm_smem(BN, kMaxStages), static_cast<size_t>(227 * 1024)));
+        if (e == cudaSuccess)
+            e = launch_overlapped(tc_gemm_kernel<BN, 0>, grid, dim3(kGemmThreads), gemm_smem(BN, p.num_stages), stream, ta, tb, p);
     }
-    cudaError_t e = launch_overlapped(tc_gemm_kernel<BN>, grid, dim3(kGemmThreads), gemm_smem(BN, p.num_stages), stream,
-                                      ta, tb, p);
     if (e == cudaSuccess) count_launch();
     return e;
 }
@@ -695,22 +151,21 @@ bool pair_worthwhile(int64_t M, int64_t N, int64_t K) {
     return N >= 256 && (tiles >= num_sms() || (tiles >= 48 && K >= 2048));
 }
 
-// Slice counts for two products that share one launch (dU: Mu x N, dV: Mv x N, both contracting
-// over K): all CTAs should fit one wave and finish together, so the longest CTA (in k-blocks) is
+// Slice counts for two products that share one launch (dU: Mu x N over nkb_u k-blocks, dV: Mv x N over nkb_v):
+// all CTAs should fit one wave and finish together, so the longest CTA (in k-blocks) is
 // minimised subject to tiles_u * su + tiles_v * sv <= SM count.
-void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t K, int kblock, int* su, int* sv) {
+void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t nkb_u, int64_t nkb_v, int* su, int* sv) {
     const int bn = pick_bn(N);
     const int64_t tu = ceil_div(Mu, kBM) * ceil_div(N, bn), tv = ceil_div(Mv, kBM) * ceil_div(N, bn);
-    const int64_t nkb = ceil_div(K, kblock);
     *su = 1; *sv = 1;
-    if (tu < 1 || tv < 1 || nkb < 1 || tu + tv > num_sms()) return;
-    int64_t best = nkb + 1;
-    for (int64_t a = 1; a <= 64 && a <= nkb && tu * a + tv <= num_sms(); ++a) {
+    if (tu < 1 || tv < 1 || nkb_u < 1 || nkb_v < 1 || tu + tv > num_sms()) return;
+    int64_t best = std::max(nkb_u, nkb_v) + 1;
+    for (int64_t a = 1; a <= 64 && a <= nkb_u && tu * a + tv <= num_sms(); ++a) {
         int64_t b = (num_sms() - tu * a) / tv;
         if (b > 64) b = 64;
-        if (b > nkb) b = nkb;
+        if (b > nkb_v) b = nkb_v;
         if (b < 1) continue;
-        const int64_t longest = std::max(ceil_div(nkb, a), ceil_div(nkb, b));
+        const int64_t longest = std::max(ceil_div(nkb_u, a), ceil_div(nkb_v, b));
         if (longest < best) { best = longest; *su = static_cast<int>(a); *sv = static_cast<int>(b); }
     }
 }
@@ -725,7 +180,7 @@ void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t K, int kblock, 
 // 20 SMs the split fused kernel leaves idle are free, loses more through the long dV blocks than the
 // overlap gains.)
 void bwd_split_plan(int64_t m, int64_t k, int64_t n, int64_t r, bool fused_dx, int* su, int* sv, bool* beside) {
-    pick_pair_splits(k, n, r, m, kBK, su, sv);
+    pick_pair_splits(k, n, r, ceil_div(m, kBK), ceil_div(m, kBK), su, sv);
     *beside = false;
     if (!fused_dx || n < 2 * k) return;
     const int bn = pick_bn(r);
@@ -743,12 +198,17 @@ void bwd_split_plan(int64_t m, int64_t k, int64_t n, int64_t r, bool fused_dx, i
     *beside = true;
 }
 
-// C[M,N] (bf16, ldc) = A * B.  `partial` must hold splits*M*N floats when splits > 1.
 struct ConvA {
     int mode;                   // 1: dX (A = dT image), 2: dU (A = x image)
-    int N, H, W, Cimg;          // the NHWC tensor A is read from (Cimg channels)
-    int kw, pad, Cw;            // kernel width, padding, channels of the layer input (rows per tap of U)
+    int N, H, W, C, R, Ho, Wo, kh, kw, pad, stride;     // the layer
 };
+// Blocks of output pixels that the contraction of dU runs over, and of the pixels of one class that dX covers.
+ConvTiling conv_k_tiling(const ConvA& c) { return conv_tiling(c.N, c.Ho, c.Wo, kBK); }
+ConvTiling conv_dx_tiling(const ConvA& c) {
+    return conv_tiling(c.N, static_cast<int>(ceil_div(c.H, c.stride)), static_cast<int>(ceil_div(c.W, c.stride)), kBM);
+}
+// Row tiles of dU: pairs of 64-channel blocks of the unrolled factor.
+int64_t conv_du_tiles(int kh, int kw, int C) { return ceil_div(static_cast<int64_t>(kh) * kw * ceil_div(C, 64), 2); }
 
 struct GemmLaunch {
     CUtensorMap ta, tb;
@@ -770,12 +230,15 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     CUtensorMap& ta = out->ta;
     CUtensorMap& tb = out->tb;
     bool oka, okb;
-    if (cv && cv->mode == 1) {          // B = U as a (taps * Cw) x R matrix, K-major
-        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->H, cv->W, cv->Cimg, cv->W, conv_box_h(cv->H, cv->W, 128));
-        okb = cached_map_2d(&tb, B.p, static_cast<int64_t>(K / cv->Cimg) * cv->Cw, cv->Cimg, B.ld, bn);
+    ConvTiling ct;
+    if (cv && cv->mode == 1) {
+        ct = conv_dx_tiling(*cv);
+        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->Ho, cv->Wo, cv->R, static_cast<int>(ceil_div(cv->W, cv->stride)), ct.bh, ct.nb, 1);
+        okb = cached_map_2d(&tb, B.p, static_cast<int64_t>(cv->kh) * cv->kw * cv->C, cv->R, B.ld, bn);   // rows past a tap's C: columns past N
     } else if (cv && cv->mode == 2) {
-        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->H, cv->W, cv->Cimg, cv->W, conv_box_h(cv->H, cv->W, 64));
-        okb = cached_map_2d(&tb, B.p, K, N, B.ld, 64);
+        ct = conv_k_tiling(*cv);
+        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->H, cv->W, cv->C, cv->Wo, ct.bh, ct.nb, cv->stride);
+        okb = cached_map_nhwc(&tb, B.p, cv->N, cv->Ho, cv->Wo, cv->R, cv->Wo, ct.bh, ct.nb, 1);
     } else if (gr) {
         const int64_t ga = A.gs == 0 ? 1 : groups, gb = B.gs == 0 ? 1 : groups;
         oka = A.mn_major ? cached_map_3d(&ta, A.p, ga, K, M, A.ld, A.gs, 64) : cached_map_3d(&ta, A.p, ga, M, K, A.ld, A.gs, kBM);
@@ -790,20 +253,36 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.a_mn = A.mn_major; p.b_mn = B.mn_major;
     p.C = C; p.ldc = ldc; p.partial = partial;
     p.C2 = nullptr; p.ldc2 = 0; p.c2_gstride = 0;
-    p.conv_mode = 0; p.cv_blks = 1; p.cv_kw = 1; p.cv_pad = 0; p.cv_C = 1; p.cv_box_h = 1; p.cv_tpi = 1;
+    p.conv_mode = 0; p.cv_blks = 1; p.cv_kw = 1; p.cv_kh = 1; p.cv_pad = 0; p.cv_stride = 1; p.cv_C = 1; p.cv_bh = 1; p.cv_nb = 1;
+    p.cv_tpi = 1; p.cv_N = p.cv_H = p.cv_W = p.cv_bw = p.cv_inv_bw = p.cv_inv_bh = p.cv_tiles_class = 1; p.cv_blocks = 0;
+    p.rows_tile = kBM; p.kpix = kBK; p.ksteps = kBK / 16;
+    int64_t row_tiles = ceil_div(M, kBM);
     if (cv) {
-        p.conv_mode = cv->mode; p.cv_kw = cv->kw; p.cv_pad = cv->pad; p.cv_C = cv->Cw;
-        p.cv_blks = cv->Cimg / 64;
-        p.cv_box_h = conv_box_h(cv->H, cv->W, cv->mode == 1 ? 128 : 64);
-        p.cv_tpi = cv->H / p.cv_box_h;
+        p.conv_mode = cv->mode; p.cv_kw = cv->kw; p.cv_kh = cv->kh; p.cv_pad = cv->pad; p.cv_stride = cv->stride; p.cv_C = cv->C;
+        p.cv_bh = ct.bh; p.cv_nb = ct.nb; p.cv_tpi = ct.tpi; p.cv_N = cv->N; p.cv_H = cv->H; p.cv_W = cv->W;
+        if (cv->mode == 1) {
+            p.cv_blks = static_cast<int>(ceil_div(cv->R, 64));
+            p.cv_bw = static_cast<int>(ceil_div(cv->W, cv->stride));
+            p.cv_inv_bw = 65535 / p.cv_bw + 1;
+            p.cv_inv_bh = 65535 / p.cv_bh + 1;
+            p.cv_tiles_class = static_cast<int>(ct.blocks);
+            p.rows_tile = ct.pixels;
+            if (cv->R < kBK) p.ksteps = static_cast<int>(ceil_div(cv->R, 16));
+            row_tiles = ct.blocks * cv->stride * cv->stride;
+        } else {
+            p.cv_blks = static_cast<int>(ceil_div(cv->C, 64));
+            p.cv_blocks = cv->kh * cv->kw * p.cv_blks;
+            p.kpix = ct.pixels;
+            p.ksteps = static_cast<int>(ceil_div(ct.pixels, 16));
+            row_tiles = conv_du_tiles(cv->kh, cv->kw, cv->C);
+        }
     }
-    p.rows_tile = (cv && cv->mode == 1) ? p.cv_box_h * cv->W : kBM;
-    p.kpix = (cv && cv->mode == 2) ? p.cv_box_h * cv->W : kBK;
     p.groups = gr ? groups : 1;
     p.a_shared = gr && A.gs == 0; p.b_shared = gr && B.gs == 0;
     p.c_gstride = gr ? gr->c_gs : 0;
     p.kb_per_group = 0;
-    int64_t nkb = ceil_div(K, p.kpix);
+    int64_t nkb = ceil_div(K, kBK);
+    if (cv) nkb = cv->mode == 2 ? ct.blocks : static_cast<int64_t>(cv->kh) * cv->kw * p.cv_blks;   // (dX: at most, the kernel counts per class)
     if (sum_groups) {                       // the groups are part of the contraction: one output
         p.kb_per_group = static_cast<int>(nkb);
         nkb *= groups;
@@ -814,7 +293,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.kb_per_split = static_cast<int>(ceil_div(nkb, splits < 1 ? 1 : splits));
     p.splits = static_cast<int>(ceil_div(nkb, p.kb_per_split));   // every slice gets >= 1 k-block
     p.status = device_status_ptr();
-    dim3 grid(static_cast<unsigned>(ceil_div(M, p.rows_tile)), static_cast<unsigned>(ceil_div(N, bn)),
+    dim3 grid(static_cast<unsigned>(row_tiles), static_cast<unsigned>(ceil_div(N, bn)),
               static_cast<unsigned>(p.splits * out_groups));
     if (grid.y > 65535 || grid.z > 65535) return PF_ERR_UNSUPPORTED;
     p.tiles_x = static_cast<int>(grid.x);
@@ -917,23 +396,24 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
                 return PF_ERR_UNSUPPORTED;
         }
     }
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {
-        if (cudaFuncSetAttribute(tc_gemm3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(gemm_smem(128, kMaxStages))) != cudaSuccess)
-            return PF_ERR_CUDA;
-        configured[dev] = true;
+    Gemm3Args k;
+    bool conv = false;
+    for (int i = 0; i < 3; ++i) {
+        const GemmLaunch* src = g[i < count ? i : 0];
+        k.ta[i] = src->ta; k.tb[i] = src->tb; k.p[i] = prm[i];
+        k.tiles[i] = make_int2(src->grid.x, src->grid.y);
+        conv = conv || src->p.conv_mode != 0;
     }
-    const GemmLaunch* a = g[0];
-    const GemmLaunch* b = g[count > 1 ? 1 : 0];
-    const GemmLaunch* c = g[count > 2 ? 2 : 0];
-    const int end0 = ctas[0], end1 = ctas[0] + ctas[1];
-    const cudaError_t e = launch_overlapped(
-        tc_gemm3_kernel, dim3(static_cast<unsigned>(total)), dim3(kGemmThreads), smem, stream, a->ta, a->tb, b->ta, b->tb,
-        c->ta, c->tb, prm[0], prm[1], prm[2], end0, end1, make_int2(a->grid.x, a->grid.y), make_int2(b->grid.x, b->grid.y),
-        make_int2(c->grid.x, c->grid.y));
+    k.end0 = ctas[0]; k.end1 = ctas[0] + ctas[1];
+    cudaError_t e;
+    if (conv) {
+        e = launch_gemm3_conv(total, smem, stream, k);
+    } else {
+        e = allow_smem(tc_gemm3_kernel<false>, gemm_smem(128, kMaxStages));
+        if (e == cudaSuccess)
+            e = launch_overlapped(tc_gemm3_kernel<false>, dim3(static_cast<unsigned>(total)), dim3(kGemmThreads), smem, stream, k.ta[0], k.tb[0],
+                                  k.ta[1], k.tb[1], k.ta[2], k.tb[2], k.p[0], k.p[1], k.p[2], k.end0, k.end1, k.tiles[0], k.tiles[1], k.tiles[2]);
+    }
     if (e != cudaSuccess) return PF_ERR_CUDA;
     count_launch();
     return PF_OK;
@@ -1381,28 +861,36 @@ void reset_fix_counters() {
     if (cudaGetSymbolAddress(&ptr, g_fix_counters) == cudaSuccess) cudaMemset(ptr, 0, sizeof(unsigned int) * kFixSlots * kFixTiles * 2);
 }
 
-// Tensor-core envelope of the factorized convolution: stride 1, "same" padding, channel counts
-// that tile evenly, image rows that pack into 128-pixel (forward, dX) and 64-pixel (dU) tiles.
-// (The forward also takes stride 2: its image tiles are fetched with a step of two pixels, and only the
-// output row has to fit a tile.  The backward of a strided convolution runs on the FMA kernels.)
-static bool conv_tc_ok(const ConvArgs& a, bool fwd = false) {
-    if ((a.stride != 1 && !(fwd && a.stride == 2)) || a.kh != a.kw || 2 * a.pad != a.kh - 1) return false;
-    if (a.C % 128 != 0 || a.R % 64 != 0 || a.O % 8 != 0 || a.R > 384) return false;
-    if (fwd ? a.Wo > 128 : a.W > 64) return false;    // backward: one image row must fit a 64-pixel k-block of dU
-    if (static_cast<int64_t>(a.N) * a.H * a.W > 0x7fffffff) return false;
+// Tensor-core envelope of the factorized convolution: channel counts that are multiples of 8 (TMA pitches; a
+// ragged 64-channel block is zero-filled), output rows that fit the tiles (128 pixels forward and dX, 64 for
+// the contraction of dU), and for a strided backward at least one tap per pixel class (kernel >= stride).
+static bool conv_tc_ok(const ConvArgs& a, bool fwd) {
+    if (a.kh != a.kw || a.C % 8 != 0 || a.R % 8 != 0 || a.O % 8 != 0 || a.R > 384) return false;
+    if (a.stride > 4 || a.Wo > (fwd ? 128 : 64) || a.stride * a.Wo > 256) return false;
+    if (!fwd && (a.kh < a.stride || ceil_div(a.W, a.stride) > 128)) return false;
+    if (static_cast<int64_t>(a.N) * a.H * a.W > 0x7fffffff || static_cast<int64_t>(a.kh) * a.kw * a.C > 0x7fffffff) return false;
     return encode_fn() != nullptr;
 }
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+namespace {
+// Slices of dU and dV of a convolution: both reductions share one launch.
+void conv_splits(const ConvA& c, int O, int* su, int* sv) {
+    pick_pair_splits(conv_du_tiles(c.kh, c.kw, c.C) * kBM, O, c.R, conv_k_tiling(c).blocks,
+                     ceil_div(static_cast<int64_t>(c.N) * c.Ho * c.Wo, kBK), su, sv);
+}
+size_t conv_du_partials(const ConvA& c, int su) { return align_up(partial_bytes(conv_du_tiles(c.kh, c.kw, c.C) * kBM, c.R, su), 256); }
+}  // namespace
+
 size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad,
                             bool bwd) {
-    if (!bwd) return 0;
+    const int Ho = (H + 2 * pad - kh) / stride + 1, Wo = (W + 2 * pad - kw) / stride + 1;
+    if (!bwd || N < 1 || Ho < 1 || Wo < 1) return 0;
     // split partials of dU ((kh*kw*C) x R) and dV (O x R)
-    const int64_t P = static_cast<int64_t>(N) * H * W, Keff = static_cast<int64_t>(kh) * kw * C;
+    const ConvA c{2, N, H, W, C, R, Ho, Wo, kh, kw, pad, stride};
     int su, sv;
-    pick_pair_splits(Keff, O, R, P, conv_box_h(H, W, 64) * W, &su, &sv);
-    (void)stride; (void)pad;
-    return align_up(partial_bytes(Keff, R, su), 256) + align_up(partial_bytes(O, R, sv), 256);
+    conv_splits(c, O, &su, &sv);
+    return conv_du_partials(c, su) + align_up(partial_bytes(O, R, sv), 256);
 }
 
 int conv_fwd(const ConvArgs& a, int* handled) {
@@ -1410,36 +898,33 @@ int conv_fwd(const ConvArgs& a, int* handled) {
     if (!conv_tc_ok(a, true) || !aligned16(a.x) || !aligned16(a.U) || !aligned16(a.V) || !aligned16(a.y) ||
         (a.T && !aligned16(a.T)))
         return PF_OK;
-    const int64_t M = static_cast<int64_t>(a.N) * a.Ho * a.Wo, Keff = static_cast<int64_t>(a.kh) * a.kw * a.C;
-    if (M < 1 || a.stride * a.Wo > 256) return PF_OK;
-    ChainPlan plan;
-    if (!chain_plan(M, Keff, a.O, a.R, true, &plan, conv_box_h(a.Ho, a.Wo, 128) * a.Wo)) return PF_OK;
-    *handled = 1;
     const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
-    return chain(a.x, a.C, M, Keff, a.U, a.R, a.R, a.V, a.R, a.O, a.y, a.O, a.T, a.R, a.stream, &cv);
+    const int st = chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, a.y, a.O, a.T, a.R, a.stream, &cv);
+    if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
+    *handled = 1;
+    return st;
 }
 
 int conv_bwd(const ConvArgs& a, int* handled) {
     *handled = 0;
-    if (!conv_tc_ok(a) || !aligned16(a.x) || !aligned16(a.U) || !aligned16(a.V) || !aligned16(a.dY) ||
+    if (!conv_tc_ok(a, false) || !aligned16(a.x) || !aligned16(a.U) || !aligned16(a.V) || !aligned16(a.dY) ||
         (a.T && !aligned16(a.T)) || (a.dX && !aligned16(a.dX)))
         return PF_OK;
-    const int64_t M = static_cast<int64_t>(a.N) * a.H * a.W, Keff = static_cast<int64_t>(a.kh) * a.kw * a.C;
-    ChainPlan plan;
-    if (!a.T && !chain_plan(M, Keff, a.O, a.R, false, &plan)) return PF_OK;
+    const int64_t P = static_cast<int64_t>(a.N) * a.Ho * a.Wo, Keff = static_cast<int64_t>(a.kh) * a.kw * a.C;
     int st;
     const void* T = a.T ? a.T : a.ws_T;
     void* dT = a.ws_G;
-    int su, sv;
-    pick_pair_splits(Keff, a.O, a.R, M, conv_box_h(a.H, a.W, 64) * a.W, &su, &sv);
-    float* pu = reinterpret_cast<float*>(a.ws);
-    float* pv = reinterpret_cast<float*>(a.ws + align_up(partial_bytes(Keff, a.R, su), 256));
     // Every product is prepared (tensor maps, geometry; nothing launched) before the call is
     // accepted, so a shape that one of them cannot take still reaches the FMA kernels.
-    // dU[tap] = shifted x^T dT ; dV = dY^T T   (reductions over all pixels, split across CTAs)
-    // dX = sum over taps of shifted dT times U[tap]^T  (implicit GEMM, contraction kh*kw*R)
-    const ConvA cu{2, a.N, a.H, a.W, a.C, a.kw, a.pad, a.C};
-    const ConvA cx{1, a.N, a.H, a.W, a.R, a.kw, a.pad, a.C};
+    // dU[tap] = shifted x^T dT ; dV = dY^T T   (reductions over all output pixels, split across CTAs)
+    // dX = sum over taps of shifted dT times U[tap]^T  (implicit GEMM over (tap, rank))
+    const ConvA cu{2, a.N, a.H, a.W, a.C, a.R, a.Ho, a.Wo, a.kh, a.kw, a.pad, a.stride};
+    ConvA cx = cu;
+    cx.mode = 1;
+    int su, sv;
+    conv_splits(cu, a.O, &su, &sv);
+    float* pu = reinterpret_cast<float*>(a.ws);
+    float* pv = reinterpret_cast<float*>(a.ws + conv_du_partials(cu, su));
     GemmLaunch gt, gu, gv, gx;
     auto prepare = [](const Operand& A, const Operand& B, int64_t Mm, int64_t Nn, int64_t Kk, void* C, int64_t ldc,
                       int splits, float* partial, const ConvA* cv, GemmLaunch* out) {
@@ -1447,14 +932,20 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         if (r == PF_ERR_UNSUPPORTED && splits > 1) r = gemm_prepare(A, B, Mm, Nn, Kk, C, ldc, 1, nullptr, cv, out);
         return r;
     };
-    st = prepare({a.dY, a.O, false}, {a.V, a.R, true}, M, a.R, a.O, dT, a.R, 1, nullptr, nullptr, &gt);
-    if (st == PF_OK) st = prepare({a.x, a.C, true}, {dT, a.R, true}, Keff, a.R, M, a.dU, a.R, su, pu, &cu, &gu);
-    if (st == PF_OK) st = prepare({a.dY, a.O, true}, {T, a.R, true}, a.O, a.R, M, a.dV, a.R, sv, pv, nullptr, &gv);
+    st = prepare({a.dY, a.O, false}, {a.V, a.R, true}, P, a.R, a.O, dT, a.R, 1, nullptr, nullptr, &gt);
+    if (st == PF_OK) st = prepare({a.x, a.C, true}, {dT, a.R, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
+    if (st == PF_OK) st = prepare({a.dY, a.O, true}, {T, a.R, true}, a.O, a.R, P, a.dV, a.R, sv, pv, nullptr, &gv);
     if (st == PF_OK && a.dX)
-        st = prepare({dT, a.R, false}, {a.U, a.R, false}, M, a.C, static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1,
-                     nullptr, &cx, &gx);
+        st = prepare({dT, a.R, false}, {a.U, a.R, false}, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
+                     static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1, nullptr, &cx, &gx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     if (st != PF_OK) return st;
+    if (!a.T) {   // recompute the thin convolution (phase 1 of the forward only)
+        const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
+        st = chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
+        if (st == PF_ERR_UNSUPPORTED) return PF_OK;
+        if (st != PF_OK) return st;
+    }
     *handled = 1;
     {   // both reductions are launched exactly as prepared (together or one by one)
         const GemmLaunch* gs[2] = {&gu, &gv};
@@ -1465,13 +956,9 @@ int conv_bwd(const ConvArgs& a, int* handled) {
             if (gs[i]->p.splits > 1) {
                 outs[i]->partial = gs[i]->p.partial; outs[i]->splits = gs[i]->p.splits; outs[i]->bn = gs[i]->bn;
                 outs[i]->tiles_x = static_cast<int>(gs[i]->grid.x); outs[i]->tiles_y = static_cast<int>(gs[i]->grid.y);
+                outs[i]->conv_c = i == 0 ? a.C : 0;
             }
         }
-    }
-    if (!a.T) {   // recompute the thin convolution (phase 1 of the forward only)
-        const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad};
-        st = chain(a.x, a.C, M, Keff, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
-        if (st != PF_OK) return st;
     }
     // dT = dY V  (per pixel)
     st = launch_prepared(gt, a.stream);

@@ -27,6 +27,7 @@ struct LinearArgs {
     struct Slices {
         const float* partial = nullptr;
         int splits = 0, bn = 0, tiles_x = 0, tiles_y = 0;
+        int conv_c = 0;     // > 0: tiles are pairs of 64-channel blocks of a [taps][conv_c] row index
     };
     Slices* du_slices = nullptr;
     Slices* dv_slices = nullptr;
@@ -50,14 +51,18 @@ struct ChainPlan {
 // `max_split` caps the number of column ranges the output is split into (0 = no cap).
 bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, ChainPlan* plan, int rows_tile = 128,
                 int max_split = 0);
-int conv_box_h(int H, int W, int limit);
-// When `conv` is given, A is an NHWC image and phase 1 is the implicit GEMM of a kh x kw, stride-1,
-// "same"-padded convolution: M = N*H*W pixels, K1 = kh*kw*C, B1 = U as a (kh*kw*C) x r matrix.
-// stride (1 or 2) applies to the k x k convolution: M = N*Ho*Wo output pixels, and the image tile of a tap
-// is fetched with that step between pixels (a tensor map with element strides).
+// Blocks of output pixels of a convolution (see conv_tiling): bh full-width rows of nb images, tpi blocks per
+// image (nb > 1 only with whole images).
+struct ConvTiling {
+    int nb = 1, bh = 1, tpi = 1, pixels = 0;
+    int64_t blocks = 0;
+};
+ConvTiling conv_tiling(int N, int Ho, int Wo, int limit);
+// When `conv` is given, A is an NHWC image and phase 1 is the implicit GEMM of a kh x kw convolution: B1 = U
+// as [kh*kw][C][r] (M and K1 are derived from it).  stride applies to the k x k convolution: the image tile of
+// a tap is fetched with that step between pixels (a tensor map with element strides).
 struct ChainConv {
-    int N, H, W, C, kh, kw, pad;
-    int stride = 1;
+    int N, H, W, C, kh, kw, pad, stride;
 };
 int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t r,
           const void* B2, int64_t ldb2, int64_t N2, void* out, int64_t ldo, void* T, int64_t ldt,

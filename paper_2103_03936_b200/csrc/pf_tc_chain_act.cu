@@ -13,20 +13,9 @@ namespace tc {
 int chain_launch_act(bool persistent, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta,
                      const CUtensorMap& tb1, const CUtensorMap& tb2, const CUtensorMap& to, const CUtensorMap& tt,
                      const ChainParams& p) {
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {
-        if (cudaFuncSetAttribute(tc_chain_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
-                cudaSuccess ||
-            cudaFuncSetAttribute(tc_chain_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
-                cudaSuccess)
-            return PF_ERR_CUDA;
-        configured[dev] = true;
-    }
-    const cudaError_t e =
-        persistent ? launch_overlapped(tc_chain_kernel<true, true>, grid, dim3(kChainThreads), smem, stream, ta, tb1, tb2, to, tt, p)
-                   : launch_overlapped(tc_chain_kernel<false, true>, grid, dim3(kChainThreads), smem, stream, ta, tb1, tb2, to, tt, p);
+    auto* kernel = persistent ? tc_chain_kernel<true, true, 0> : tc_chain_kernel<false, true, 0>;
+    cudaError_t e = allow_smem(kernel, 227 * 1024);
+    if (e == cudaSuccess) e = launch_overlapped(kernel, grid, dim3(kChainThreads), smem, stream, ta, tb1, tb2, to, tt, p);
     if (e != cudaSuccess) return PF_ERR_CUDA;
     count_launch();
     return PF_OK;

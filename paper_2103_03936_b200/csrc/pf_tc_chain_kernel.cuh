@@ -23,9 +23,9 @@
 // accumulators then live beside T's in tensor memory (128 + 3 x 128 columns) instead of on top of it.
 // Shared memory: control block | T (r_pad x 256 B) | ring of stages (16 KB A or B2 tile + r_pad x
 // 128 B B1 tile).  In phase 2 the B1 part of every stage is idle and serves as store staging.
-// This header holds the kernel (a template, instantiated once per translation unit: the single-tile
-// form in pf_tc_chain.cu, the persistent form in pf_tc_chain_multi.cu, so that each lives in a module
-// of its own) and the parameter block the host fills.
+// This header holds the kernel (a template, instantiated in several translation units: the single-tile
+// form in pf_tc_chain.cu, the forms with a bias / activation epilogue in pf_tc_chain_act.cu, the convolution in
+// pf_tc_chain_conv.cu, so that each lives in a module of its own) and the parameter block the host fills.
 #ifndef PF_TC_CHAIN_KERNEL_CUH_
 #define PF_TC_CHAIN_KERNEL_CUH_
 
@@ -45,10 +45,12 @@ struct ChainParams {
     int store_T;
     int boxes_per_stage;    // phase 2: B2 boxes (16 KB each) loaded per ring stage
     int staging_off;        // byte offset (from the 1 KB-aligned base) of dedicated store staging, 0 = none
-    // Implicit-GEMM convolution as phase 1 (conv_cblks > 0): tmA is a 4-D NHWC map, a row tile is
-    // box_h full-width image rows (box_h * W = 128 pixels) and k-block kb = (tap, 64-channel block).
-    int conv_cblks, conv_kw, conv_pad, conv_box_h, conv_tiles_per_img;
-    int rows_tile;          // rows of A in one tile: 128, or box_h * W pixels (<= 128) for the convolution
+    // Implicit-GEMM convolution as phase 1 (conv_cblks > 0): tmA is a 4-D NHWC map, tmB1 the factor as
+    // (taps * C) x r; a row tile is conv_bh full-width output rows of conv_nb images (conv_nb > 1 only with whole
+    // images) and a k-block is (tap, 64-channel block).  The last tile of an image, and the last group of
+    // images, starts early enough to be full: it recomputes rows of the tile before it, to the same values.
+    int conv_cblks, conv_kw, conv_pad, conv_stride, conv_bh, conv_nb, conv_tpi, conv_Ho, conv_N;
+    int rows_tile;          // rows of A in one tile: 128, or the output pixels of a convolution's tile (<= 128)
     int row_tiles;          // tiles along M; a CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...
     int acc_base, acc_bufs; // TMEM column of the first phase-2 accumulator and their number (4 on top of T's
                             // columns, or 3 behind them when tiles overlap)
@@ -94,6 +96,20 @@ __device__ __forceinline__ uint32_t relu_bf16x2(uint32_t w) {
     return r;
 }
 
+// First image and first output row of a convolution's row tile; image * Ho + row is its position in the
+// output (and stash) maps, which count whole output rows.
+struct ConvOrigin {
+    int img, row;
+};
+__device__ __forceinline__ ConvOrigin conv_origin(const ChainParams& p, int tile) {
+    const int g = tile / p.conv_tpi;
+    return ConvOrigin{min(g * p.conv_nb, p.conv_N - p.conv_nb), min((tile - g * p.conv_tpi) * p.conv_bh, p.conv_Ho - p.conv_bh)};
+}
+__device__ __forceinline__ int conv_out_row(const ChainParams& p, int tile) {
+    const ConvOrigin o = conv_origin(p, tile);
+    return o.img * p.conv_Ho + o.row;
+}
+
 // Position in the cycle of phase-2 accumulators: buffer index and its phase bit.
 struct AccPos {
     uint32_t b = 0, ph = 0;
@@ -113,7 +129,9 @@ struct RingPos {
 // kMulti: a CTA may own several row tiles (persistent grid); otherwise exactly the tile blockIdx.x, and
 // the loops over tiles below fold away at compile time.
 // kEpi: the output epilogue adds a bias row and applies the activation (see ChainParams).
-template <bool kMulti, bool kEpi = false>
+// kConv: 0 = plain, 1 = convolution, 2 = convolution whose C is not a multiple of 64: tmB1 is then 3-D, [taps][C][r],
+// zero-filled past a tap's channels (the 3-D map costs 10 % of the pace, so the others stay 2-D).
+template <bool kMulti, bool kEpi, int kConv>
 __global__ void __launch_bounds__(kChainThreads, 1)
 tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB1,
                 const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmOut,
@@ -131,7 +149,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int nt_total = (p.N2 + 127) / 128;
     const int t_beg = blockIdx.y * p.tiles_per_split;
     const int ntile = max(0, min(nt_total, t_beg + p.tiles_per_split) - t_beg);
-    const int nkb1 = (p.K1 + 63) / 64;
+    const int nkb1 = (p.K1 + 63) / 64;              // a convolution's K1 counts whole 64-channel blocks
     const int nkb2 = p.r_pad / 64;
     const uint32_t NS = static_cast<uint32_t>(p.num_stages);
     const uint32_t S = static_cast<uint32_t>(p.stage_bytes);
@@ -165,7 +183,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     // While the previous kernel of the stream finishes, ask L2 for this block's first tiles.  A prefetch
     // only moves lines into L2, the point of coherence, so it is harmless even if that kernel is
     // still writing the tensor; the loads that consume the data are issued after the wait below.
-    if (p.conv_cblks == 0) {
+    if (kConv == 0) {
         if (warp == 0 && elect_one()) {
             for (int kb = 0; kb < kEarlyTiles && kb < nkb1; ++kb) tma_prefetch_l2_2d(&tmA, kb * 64, tile0 * p.rows_tile);
         } else if (warp == 10 && elect_one()) {
@@ -194,25 +212,32 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int m0 = tile * p.rows_tile;
                 // convolution: (tap row, tap column, channel block) advance as counters; integer divisions
                 // in the loop over k-blocks would sit on the producer's critical path
-                const int cv_img = p.conv_cblks > 0 ? tile / p.conv_tiles_per_img : 0;
-                const int cv_h0 = (tile - cv_img * p.conv_tiles_per_img) * p.conv_box_h - p.conv_pad;
-                int cv_cb = 0, cv_ta = 0, cv_tb = 0;
-                for (int kb = 0; kb < nkb1; ++kb) {
-                    ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
-                    if (!ok) break;
-                    const uint32_t full = full0 + 8 * rp.s;
-                    const uint32_t dst = ring + rp.off;
-                    mbar_expect_tx(full, txa);
-                    if (p.conv_cblks > 0) {
-                        tma_load_4d(dst, &tmA, full, cv_cb * 64, cv_tb - p.conv_pad, cv_h0 + cv_ta, cv_img);
-                        if (++cv_cb == p.conv_cblks) {
-                            cv_cb = 0;
-                            if (++cv_tb == p.conv_kw) { cv_tb = 0; ++cv_ta; }
+                const ConvOrigin cv = kConv ? conv_origin(p, tile) : ConvOrigin{0, 0};
+                const int cv_img = cv.img, cv_h0 = cv.row * p.conv_stride - p.conv_pad;
+                if constexpr (kConv != 0) {
+                    const int cblks = p.conv_cblks, kw = p.conv_kw, x0 = -p.conv_pad, x1 = kw - p.conv_pad;
+                    int cb = 0, x = x0, y = cv_h0;
+                    for (int kb = 0; kb < nkb1; ++kb) {
+                        ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
+                        if (!ok) break;
+                        const uint32_t full = full0 + 8 * rp.s;
+                        mbar_expect_tx(full, txa);
+                        tma_load_4d(ring + rp.off, &tmA, full, cb * 64, x, y, cv_img);
+                        if (++cb == cblks) {
+                            cb = 0;
+                            if (++x == x1) { x = x0; ++y; }
                         }
-                    } else {
-                        tma_load_2d(dst, &tmA, full, kb * 64, m0);
+                        rp.advance(NS, S);
                     }
-                    rp.advance(NS, S);
+                } else {
+                    for (int kb = 0; kb < nkb1; ++kb) {
+                        ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
+                        if (!ok) break;
+                        const uint32_t full = full0 + 8 * rp.s;
+                        mbar_expect_tx(full, txa);
+                        tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0);
+                        rp.advance(NS, S);
+                    }
                 }
                 // the B producer fills the tile's phase-2 stages alone; this thread still takes each of
                 // them in turn (waits, loads nothing), so that it never runs more than one lap ahead
@@ -243,13 +268,20 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const uint32_t txb = static_cast<uint32_t>(p.r_pad) * 128u;
             int tile = tile0;
             do {
+                const int cblks = p.conv_cblks;
+                int cb = 0, tap = 0;
                 for (int kb = 0; kb < nkb1; ++kb) {
                     ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
                     if (!ok) break;
                     const uint32_t full = full0 + 8 * rp.s;
                     const uint32_t dst = ring + rp.off + kTileBytes;
                     mbar_expect_tx(full, txb);
-                    for (int q = 0; q < nkb2; ++q) tma_load_2d(dst + q * 8192, &tmB1, full, q * 64, kb * 64);
+                    if constexpr (kConv == 2) {
+                        for (int q = 0; q < nkb2; ++q) tma_load_3d(dst + q * 8192, &tmB1, full, q * 64, cb * 64, tap);
+                        if (++cb == cblks) { cb = 0; ++tap; }
+                    } else {
+                        for (int q = 0; q < nkb2; ++q) tma_load_2d(dst + q * 8192, &tmB1, full, q * 64, kb * 64);
+                    }
                     rp.advance(NS, S);
                 }
                 for (int j = 0; j < ntile && ok; ++j) {
@@ -318,8 +350,9 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 if (!ok) break;
                 tc_fence_after();
                 if (p.store_T && blockIdx.y == 0) {
+                    const int crow = kConv ? conv_out_row(p, tile) : 0;
                     for (int q = 0; q < nkb2; ++q) {
-                        if (p.conv_cblks > 0) tma_store_3d(&tmT, t_smem + q * kTileBytes, q * 64, 0, tile);
+                        if constexpr (kConv != 0) tma_store_3d(&tmT, t_smem + q * kTileBytes, q * 64, 0, crow);
                         else tma_store_2d(&tmT, t_smem + q * kTileBytes, q * 64, tile * p.rows_tile);
                     }
                     tma_store_commit();
@@ -399,6 +432,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (lane == 0) mbar_arrive(smem_u32(&ctl->t_ready));
 
             const int r0 = tile * p.rows_tile + q * 32;
+            const int crow = kConv ? conv_out_row(p, tile) : 0;
             for (int j = 0; j < ntile; ++j) {
                 // kEpi: the bias of this warp's 64 columns, as 32 bf16 pairs per thread (every lane loads the
                 // same addresses: one broadcast transaction per load), fetched before the accumulator arrives
@@ -459,7 +493,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 if (lane == 0) {
                     const int n0 = (t_beg + j) * 128 + hcol * 64;
                     if (r0 < p.M && q * 32 < p.rows_tile && n0 < p.N2) {
-                        if (p.conv_cblks > 0) tma_store_3d(&tmOut, stg, n0, q * 32, tile);
+                        if constexpr (kConv != 0) tma_store_3d(&tmOut, stg, n0, q * 32, crow);
                         else tma_store_2d(&tmOut, stg, n0, r0);
                         tma_store_commit();
                         stored = true;
@@ -489,9 +523,9 @@ int chain_launch_act(bool persistent, dim3 grid, size_t smem, cudaStream_t strea
 // Launch of the software-pipelined persistent form (pf_tc_chain_pipe.cuh, compiled in pf_tc_chain_multi.cu).
 int chain_launch_pipe(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1,
                       const CUtensorMap& tb2, const CUtensorMap& to, const CUtensorMap& tt, const ChainParams& p);
-// Launch of the persistent form (pf_tc_chain_multi.cu); same arguments as the kernel.
-int chain_launch_multi(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1,
-                       const CUtensorMap& tb2, const CUtensorMap& to, const CUtensorMap& tt, const ChainParams& p);
+// Launch of the forms with a convolution as first product (pf_tc_chain_conv.cu); pipe = software-pipelined persistent.
+int chain_launch_conv(bool pipe, bool ragged, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1,
+                      const CUtensorMap& tb2, const CUtensorMap& to, const CUtensorMap& tt, const ChainParams& p);
 
 }  // namespace tc
 }  // namespace pf

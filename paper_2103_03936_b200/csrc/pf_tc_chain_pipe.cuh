@@ -31,6 +31,7 @@ struct PipeCtl {
     uint32_t abort;
 };
 
+template <int kConv>
 __global__ void __launch_bounds__(kChainThreads, 1)
 tc_chain_pipe_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB1,
                      const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmOut,
@@ -96,24 +97,32 @@ tc_chain_pipe_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                 if (t < nt) {
                     const int tile = tile0 + t * tile_step;
                     const int m0 = tile * p.rows_tile;
-                    const int cv_img = p.conv_cblks > 0 ? tile / p.conv_tiles_per_img : 0;
-                    const int cv_h0 = (tile - cv_img * p.conv_tiles_per_img) * p.conv_box_h - p.conv_pad;
-                    int cv_cb = 0, cv_ta = 0, cv_tb = 0;
-                    for (int kb = 0; kb < nkb1; ++kb) {
-                        ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
-                        if (!ok) break;
-                        const uint32_t full = full0 + 8 * rp.s;
-                        mbar_expect_tx(full, txa);
-                        if (p.conv_cblks > 0) {
-                            tma_load_4d(ring + rp.off, &tmA, full, cv_cb * 64, cv_tb - p.conv_pad, cv_h0 + cv_ta, cv_img);
-                            if (++cv_cb == p.conv_cblks) {
-                                cv_cb = 0;
-                                if (++cv_tb == p.conv_kw) { cv_tb = 0; ++cv_ta; }
+                    const ConvOrigin cv = kConv ? conv_origin(p, tile) : ConvOrigin{0, 0};
+                    const int cv_img = cv.img, cv_h0 = cv.row * p.conv_stride - p.conv_pad;
+                    if constexpr (kConv != 0) {
+                        const int cblks = p.conv_cblks, kw = p.conv_kw, x0 = -p.conv_pad, x1 = kw - p.conv_pad;
+                        int cb = 0, x = x0, y = cv_h0;
+                        for (int kb = 0; kb < nkb1; ++kb) {
+                            ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
+                            if (!ok) break;
+                            const uint32_t full = full0 + 8 * rp.s;
+                            mbar_expect_tx(full, txa);
+                            tma_load_4d(ring + rp.off, &tmA, full, cb * 64, x, y, cv_img);
+                            if (++cb == cblks) {
+                                cb = 0;
+                                if (++x == x1) { x = x0; ++y; }
                             }
-                        } else {
-                            tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0);
+                            rp.advance(NS, S);
                         }
-                        rp.advance(NS, S);
+                    } else {
+                        for (int kb = 0; kb < nkb1; ++kb) {
+                            ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
+                            if (!ok) break;
+                            const uint32_t full = full0 + 8 * rp.s;
+                            mbar_expect_tx(full, txa);
+                            tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0);
+                            rp.advance(NS, S);
+                        }
                     }
                 }
                 if (t >= 1) {
@@ -132,13 +141,20 @@ tc_chain_pipe_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             const uint32_t txb = static_cast<uint32_t>(p.r_pad) * 128u;
             for (int t = 0; t <= nt && ok; ++t) {
                 if (t < nt) {
+                    const int cblks = p.conv_cblks;
+                    int cb = 0, tap = 0;
                     for (int kb = 0; kb < nkb1; ++kb) {
                         ok = mbar_wait(empty0 + 8 * rp.s, rp.ph ^ 1u, abort_flag, p.status);
                         if (!ok) break;
                         const uint32_t full = full0 + 8 * rp.s;
                         const uint32_t dst = ring + rp.off + kTileBytes;
                         mbar_expect_tx(full, txb);
-                        for (int q = 0; q < nkb2; ++q) tma_load_2d(dst + q * 8192, &tmB1, full, q * 64, kb * 64);
+                        if constexpr (kConv == 2) {
+                            for (int q = 0; q < nkb2; ++q) tma_load_3d(dst + q * 8192, &tmB1, full, q * 64, cb * 64, tap);
+                            if (++cb == cblks) { cb = 0; ++tap; }
+                        } else {
+                            for (int q = 0; q < nkb2; ++q) tma_load_2d(dst + q * 8192, &tmB1, full, q * 64, kb * 64);
+                        }
                         rp.advance(NS, S);
                     }
                 }
@@ -198,8 +214,9 @@ tc_chain_pipe_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     const uint32_t t_smem = t_smem0 + static_cast<uint32_t>(u & 1) * t_bytes;
                     const int tile = tile0 + u * tile_step;
                     if (p.store_T) {
+                        const int crow = kConv ? conv_out_row(p, tile) : 0;
                         for (int q = 0; q < nkb2; ++q) {
-                            if (p.conv_cblks > 0) tma_store_3d(&tmT, t_smem + q * kTileBytes, q * 64, 0, tile);
+                            if constexpr (kConv != 0) tma_store_3d(&tmT, t_smem + q * kTileBytes, q * 64, 0, crow);
                             else tma_store_2d(&tmT, t_smem + q * kTileBytes, q * 64, tile * p.rows_tile);
                         }
                         tma_store_commit();
@@ -267,6 +284,7 @@ tc_chain_pipe_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             if (t >= 1) {
                 const int tile = tile0 + (t - 1) * tile_step;
                 const int r0 = tile * p.rows_tile + q * 32;
+                const int crow = kConv ? conv_out_row(p, tile) : 0;
                 for (int j = 0; j < ntile; ++j) {
                     ok = mbar_wait_warp(smem_u32(&ctl->acc_full[ap.b]), ap.ph, abort_flag, p.status);
                     tc_fence_after();
@@ -291,7 +309,7 @@ tc_chain_pipe_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     if (lane == 0) {
                         const int n0 = j * 128 + hcol * 64;
                         if (r0 < p.M && q * 32 < p.rows_tile && n0 < p.N2) {
-                            if (p.conv_cblks > 0) tma_store_3d(&tmOut, stg, n0, q * 32, tile);
+                            if constexpr (kConv != 0) tma_store_3d(&tmOut, stg, n0, q * 32, crow);
                             else tma_store_2d(&tmOut, stg, n0, r0);
                             tma_store_commit();
                             stored = true;

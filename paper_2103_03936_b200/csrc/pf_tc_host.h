@@ -72,66 +72,93 @@ inline bool cached_map_2d(CUtensorMap* map, const void* p, int64_t rows, int64_t
     return true;
 }
 
-// 4-D bf16 tensor map over an NHWC image [N, H, W, C]: boxes are 64 channels x box_w x box_h pixels
-// of one image (box_w * box_h rows of 128 bytes in shared memory, pixel-major); coordinates may
-// start outside the image (zero padding of the convolution), out-of-range pixels read as zero.
-inline bool cached_map_nhwc(CUtensorMap* map, const void* p, int64_t N, int64_t H, int64_t W, int64_t C,
-                            int box_w, int box_h) {
-    constexpr int kSlots = 64;
-    struct Slot { MapKey key; CUtensorMap map; bool used; };
+// The maps below are described by eight numbers; they share one cache.
+struct WideKey {
+    const void* p;
+    int64_t v[8];
+    bool operator==(const WideKey& o) const {
+        if (p != o.p) return false;
+        for (int i = 0; i < 8; ++i)
+            if (v[i] != o.v[i]) return false;
+        return true;
+    }
+};
+template <typename Make>
+inline bool cached_map_wide(CUtensorMap* map, const WideKey& key, Make make) {
+    constexpr int kSlots = 256;
+    struct Slot { WideKey key; CUtensorMap map; bool used; };
     static Slot slots[kSlots];
     static std::mutex mu;
-    const MapKey key{p, N * 100003 + H, C, W, -(box_h * 1024 + box_w)};
-    const uint64_t h = reinterpret_cast<uintptr_t>(p) * 0x9E3779B97F4A7C15ull + static_cast<uint64_t>(key.rows) * 31 +
-                       static_cast<uint64_t>(C) * 131 + static_cast<uint64_t>(W) * 1031 + static_cast<uint64_t>(-key.box_rows);
-    Slot& s = slots[(h >> 20) % kSlots];
+    uint64_t h = reinterpret_cast<uintptr_t>(key.p) * 0x9E3779B97F4A7C15ull;
+    for (int i = 0; i < 8; ++i) h = (h ^ static_cast<uint64_t>(key.v[i])) * 0xC2B2AE3D27D4EB4Full;
+    Slot& s = slots[(h >> 24) % kSlots];
     std::lock_guard<std::mutex> lock(mu);
     if (s.used && s.key == key) { *map = s.map; return true; }
     EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W), static_cast<cuuint64_t>(H),
-                                static_cast<cuuint64_t>(N)};
-    const cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 2, static_cast<cuuint64_t>(W) * C * 2,
-                                   static_cast<cuuint64_t>(H) * W * C * 2};
-    const cuuint32_t box[4] = {64u, static_cast<cuuint32_t>(box_w), static_cast<cuuint32_t>(box_h), 1u};
-    const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-    if (fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p), dims, strides, box, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
+    if (!fn || !make(fn)) return false;
     s.key = key; s.map = *map; s.used = true;
     return true;
 }
+inline bool encode_bf16(EncodeTiledFn fn, CUtensorMap* map, const void* p, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                        const cuuint32_t* box, const cuuint32_t* estr) {
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, static_cast<cuuint32_t>(rank), const_cast<void*>(p), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
-// 3-D view of a contiguous row-major [tiles * rows_tile, cols] matrix as [tiles][rows_tile][cols]:
-// a store box of box_rows rows that starts inside a tile is clipped at the end of that tile, which
-// is how partially filled 128-row MMA tiles (image rows that do not pack into 128 pixels) are
-// written without touching the next tile's pixels.
-inline bool cached_map_tiled_rows(CUtensorMap* map, const void* p, int64_t tiles, int rows_tile, int64_t cols,
-                                  int box_rows) {
-    constexpr int kSlots = 64;
-    struct Slot { MapKey key; CUtensorMap map; bool used; };
-    static Slot slots[kSlots];
+// 4-D bf16 tensor map over an NHWC image [N, H, W, C]: boxes are 64 channels x box_w x box_h pixels of box_n
+// images (box_w * box_h * box_n rows of 128 bytes in shared memory, pixel-major), taking every stride-th
+// pixel along W and H; coordinates may start outside the image (zero padding of the convolution),
+// out-of-range pixels, channels and images read as zero.
+inline bool cached_map_nhwc(CUtensorMap* map, const void* p, int64_t N, int64_t H, int64_t W, int64_t C, int box_w, int box_h,
+                            int box_n, int stride) {
+    return cached_map_wide(map, WideKey{p, {N, H, W, C, box_w, box_h, box_n, stride}}, [&](EncodeTiledFn fn) {
+        const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W), static_cast<cuuint64_t>(H),
+                                    static_cast<cuuint64_t>(N)};
+        const cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 2, static_cast<cuuint64_t>(W) * C * 2,
+                                       static_cast<cuuint64_t>(H) * W * C * 2};
+        // box extents are given in traversed elements, i.e. times the stride
+        const cuuint32_t box[4] = {64u, static_cast<cuuint32_t>(box_w * stride), static_cast<cuuint32_t>(box_h * stride),
+                                   static_cast<cuuint32_t>(box_n)};
+        const cuuint32_t estr[4] = {1u, static_cast<cuuint32_t>(stride), static_cast<cuuint32_t>(stride), 1u};
+        return encode_bf16(fn, map, p, 4, dims, strides, box, estr);
+    });
+}
+
+// 3-D view of a contiguous [planes][rows][cols] tensor with boxes of 64 columns x box_rows rows of one plane:
+// a box that reaches past the rows of its plane reads zeros (or is clipped) instead of running into the
+// next.  plane_step, in rows, is the distance between planes: `rows` for the factor of a convolution
+// (planes = taps), less for overlapping windows (the output tiles of a convolution, one window per
+// image row, so that a tile may start at any row and is clipped at its own end).
+inline bool cached_map_planes(CUtensorMap* map, const void* p, int64_t planes, int64_t rows, int64_t cols, int64_t plane_step,
+                              int box_rows) {
+    return cached_map_wide(map, WideKey{p, {planes, rows, cols, plane_step, box_rows, -1, -1, -1}}, [&](EncodeTiledFn fn) {
+        const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(planes)};
+        const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 2, static_cast<cuuint64_t>(plane_step) * cols * 2};
+        const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u};
+        const cuuint32_t estr[3] = {1u, 1u, 1u};
+        return encode_bf16(fn, map, p, 3, dims, strides, box, estr);
+    });
+}
+
+// Raises a kernel's dynamic shared memory limit, once per kernel and device.
+template <typename... KArgs>
+inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
+    struct Done { void (*k)(KArgs...); bool dev[64]; };
+    constexpr int kKernels = 16;
+    static Done done[kKernels];
     static std::mutex mu;
-    const MapKey key{p, tiles, cols, rows_tile, -(1 << 24) - box_rows};
-    const uint64_t h = reinterpret_cast<uintptr_t>(p) * 0x9E3779B97F4A7C15ull + static_cast<uint64_t>(tiles) * 31 +
-                       static_cast<uint64_t>(cols) * 131 + static_cast<uint64_t>(rows_tile) * 1031 + box_rows;
-    Slot& s = slots[(h >> 20) % kSlots];
+    int dev = 0;
+    cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lock(mu);
-    if (s.used && s.key == key) { *map = s.map; return true; }
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows_tile),
-                                static_cast<cuuint64_t>(tiles)};
-    const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 2, static_cast<cuuint64_t>(rows_tile) * cols * 2};
-    const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    if (fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(p), dims, strides, box, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
-    s.key = key; s.map = *map; s.used = true;
-    return true;
+    for (Done& d : done) {
+        if (d.k != nullptr && d.k != kernel) continue;
+        if (d.k == kernel && dev >= 0 && dev < 64 && d.dev[dev]) return cudaSuccess;
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+        if (e == cudaSuccess && dev >= 0 && dev < 64) { d.k = kernel; d.dev[dev] = true; }
+        return e;
+    }
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
 }
 
 // Launch with programmatic stream serialization: the kernel's prologue (barrier set-up, TMEM

@@ -208,3 +208,28 @@ def test_stride2_forward_on_tensor_cores(N, H, W, C, R, O):
     gT.check()
     assert pf.pf_last_device_status() == 0
     run_conv(c)          # and the whole forward + backward against the oracle
+
+
+@pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad", [
+    (5, 5, 5, 64, 16, 64, 3, 1, 1),      # several whole images per tile (a ragged last group), one 64-channel block per tap
+    (3, 7, 7, 96, 24, 40, 3, 1, 1),      # ragged channel block, 49-pixel reduction blocks (zero-filled tail)
+    (2, 13, 11, 72, 8, 16, 3, 1, 1),     # image rows that do not divide into tiles
+    (4, 9, 9, 160, 40, 80, 3, 2, 1),     # stride 2, odd image: four pixel classes of unequal size
+    (7, 4, 6, 128, 80, 256, 3, 2, 1),    # stride 2, several images per tile, ranks past one 64-block
+    (2, 12, 12, 64, 16, 72, 5, 3, 2),    # stride 3, 5 x 5 taps
+    (3, 6, 6, 32, 16, 24, 3, 1, 0),      # no padding: fewer output than input pixels
+    (2, 16, 16, 24, 8, 16, 2, 2, 0),     # one tap per class
+    (150, 4, 4, 64, 16, 64, 3, 1, 1),
+])
+def test_tensor_core_tilings(N, H, W, C, R, O, k, stride, pad):
+    """Edges of the implicit-GEMM tilings: tiles of several images, rows that do not divide, ragged channel
+    blocks and strided backward passes, with and without stash / dX; fp32 gradients from the slices."""
+    c = wl.ConvCase("til", N, H, W, C, R, O, wl.BF16, 91, kh=k, kw=k, stride=stride, pad=pad)
+    run_conv(c)
+    run_conv(c, stash=False, need_dX=False)
+    d = c.generate()
+    x, U, V, dY = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V", "dY"))
+    _, dU0, dV0 = pf.pf_lowrank_conv_bwd(x, U, V, dY, stride=stride, pad=pad)
+    _, dU1, dV1 = pf.pf_lowrank_conv_bwd(x, U, V, dY, stride=stride, pad=pad, grads_f32=True)
+    torch.cuda.synchronize()
+    assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
