@@ -63,7 +63,8 @@ typedef enum {
 } pf_status;
 
 typedef enum {
-    PF_F32 = 0, /* fp32 storage, fp32 FMA arithmetic */
+    PF_F32 = 0, /* fp32 storage and accuracy: tensor-core products of exactly split operands (three bf16 parts, fp32
+                   accumulation), fp32 FMA arithmetic where a layout does not allow them */
     PF_BF16 = 1 /* bf16 storage, tensor-core products with fp32 accumulation */
 } pf_dtype;
 

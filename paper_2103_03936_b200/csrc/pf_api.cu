@@ -80,7 +80,7 @@ LinearWs linear_ws(int64_t m, int64_t k, int64_t n, int64_t r, int dtype, bool b
         w.off_gtmp = off; off += align_up(static_cast<size_t>(k) * r * s, 256) + align_up(static_cast<size_t>(n) * r * s, 256);
     }
     w.off_tc = off;
-    if (dtype == PF_BF16) off += align_up(tc::linear_extra_workspace(m, k, n, r, bwd), 256);
+    off += align_up(dtype == PF_BF16 ? tc::linear_extra_workspace(m, k, n, r, bwd) : tc::f32_linear_workspace(m, k, n, r, bwd), 256);
     w.total = off;
     return w;
 }
@@ -184,7 +184,11 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     size_t need = w.total;
     if (exact_need) {
         bool tc_handles = false;
-        const size_t tc_need = dtype == PF_BF16 ? tc::linear_fwd_need(a, &tc_handles) : 0;
+        size_t tc_need = dtype == PF_BF16 ? tc::linear_fwd_need(a, &tc_handles) : 0;
+        if (dtype == PF_F32) {        // (taken only when it fits; the FMA kernels need less)
+            tc_need = tc::f32_linear_workspace(m, k, n, r, false);
+            tc_handles = w.off_tc + tc_need <= workspace_bytes;
+        }
         if (tc_handles) need = tc_need ? w.off_tc + tc_need : 0;
         else need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * dtype_size(dtype);   // FMA kernels: x U only
     }
@@ -195,6 +199,10 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     if (dtype == PF_BF16) {
         int handled = 0;
         st = tc::linear_fwd(a, &handled);
+        if (st != PF_OK || handled) return st;
+    } else if (workspace_bytes > w.off_tc) {
+        int handled = 0;
+        st = tc::f32_linear_fwd(a, &handled, workspace_bytes - w.off_tc);
         if (st != PF_OK || handled) return st;
     }
     void* T = T_stash ? T_stash : static_cast<void*>(ws + w.off_T);
@@ -292,13 +300,13 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
     const int64_t user_lddu = lddu, user_lddv = lddv;
     bool indirect = false;
 
+    tc::LinearArgs a;
+    a.x = x; a.ldx = ldx; a.U = U; a.ldu = ldu; a.V = V; a.ldv = ldv;
+    a.dY = dY; a.lddy = lddy; a.T = const_cast<void*>(T_stash); a.ldt = ldt;
+    a.dX = dX; a.lddx = lddx; a.dU = dU; a.lddu = lddu; a.dV = dV; a.lddv = lddv;
+    a.m = m; a.k = k; a.n = n; a.r = r;
+    a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.ws_G = ws + w.off_G; a.stream = stream;
     if (dtype == PF_BF16) {
-        tc::LinearArgs a;
-        a.x = x; a.ldx = ldx; a.U = U; a.ldu = ldu; a.V = V; a.ldv = ldv;
-        a.dY = dY; a.lddy = lddy; a.T = const_cast<void*>(T_stash); a.ldt = ldt;
-        a.dX = dX; a.lddx = lddx; a.dU = dU; a.lddu = lddu; a.dV = dV; a.lddv = lddv;
-        a.m = m; a.k = k; a.n = n; a.r = r;
-        a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.ws_G = ws + w.off_G; a.stream = stream;
         tc::LinearArgs::Slices su_info, sv_info;
         if (flags) {
             // plain gradients go to the workspace; where a reduction was split, its fp32 slices are still
@@ -329,10 +337,23 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
             return PF_OK;
         }
         if (handled) return PF_OK;
-    } else if (flags) {
-        indirect = true;
-        dU = ws + w.off_gtmp; lddu = r;
-        dV = ws + w.off_gtmp + align_up(static_cast<size_t>(k) * r * s, 256); lddv = r;
+    } else {
+        if (g_acc) {
+            indirect = true;
+            dU = ws + w.off_gtmp; lddu = r;
+            dV = ws + w.off_gtmp + align_up(static_cast<size_t>(k) * r * s, 256); lddv = r;
+            a.dU = dU; a.lddu = lddu; a.dV = dV; a.lddv = lddv;
+        }
+        int handled = 0;
+        st = tc::f32_linear_bwd(a, &handled);
+        if (st != PF_OK) return st;
+        if (handled) {
+            if (indirect) {
+                PF_CUDA(grad_combine(user_dU, user_lddu, gdtype, dU, lddu, dtype, k, r, g_acc, stream));
+                PF_CUDA(grad_combine(user_dV, user_lddv, gdtype, dV, lddv, dtype, n, r, g_acc, stream));
+            }
+            return PF_OK;
+        }
     }
     const void* T = T_stash;
     int64_t ldT = ldt;
@@ -513,7 +534,14 @@ ConvWs conv_ws(int N, int H, int W, int C, int R, int O, int kh, int kw, int str
         w.off_gtmp = off; off += align_up(static_cast<size_t>(Keff) * R * s, 256) + align_up(static_cast<size_t>(O) * R * s, 256);
     }
     w.off_tc = off;
-    if (dtype == PF_BF16) off += align_up(tc::conv_extra_workspace(N, H, W, C, R, O, kh, kw, stride, pad, bwd), 256);
+    if (dtype == PF_BF16) {
+        off += align_up(tc::conv_extra_workspace(N, H, W, C, R, O, kh, kw, stride, pad, bwd), 256);
+    } else {
+        tc::ConvArgs a;
+        std::memset(&a, 0, sizeof(a));
+        a.N = N; a.H = H; a.W = W; a.C = C; a.R = R; a.O = O; a.kh = kh; a.kw = kw; a.stride = stride; a.pad = pad; a.Ho = w.Ho; a.Wo = w.Wo;
+        off += align_up(tc::f32_conv_workspace(a, bwd), 256);
+    }
     w.total = off;
     return w;
 }
@@ -560,7 +588,7 @@ int pf_lowrank_conv_fwd(const void* x, const void* U, const void* V, void* y, vo
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     char* ws = static_cast<char*>(workspace);
 
-    if (dtype == PF_BF16) {
+    {
         tc::ConvArgs a;
         std::memset(&a, 0, sizeof(a));
         a.x = x; a.U = U; a.V = V; a.y = y; a.T = T_stash;
@@ -568,7 +596,7 @@ int pf_lowrank_conv_fwd(const void* x, const void* U, const void* V, void* y, vo
         a.stride = stride; a.pad = pad; a.Ho = w.Ho; a.Wo = w.Wo;
         a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.stream = stream;
         int handled = 0;
-        st = tc::conv_fwd(a, &handled);
+        st = dtype == PF_BF16 ? tc::conv_fwd(a, &handled) : tc::f32_conv_fwd(a, &handled);
         if (st != PF_OK || handled) return st;
     }
     void* T = T_stash ? T_stash : static_cast<void*>(ws + w.off_T);
@@ -645,7 +673,7 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         return PF_OK;
     };
 
-    if (dtype == PF_BF16) {
+    {
         tc::ConvArgs a;
         std::memset(&a, 0, sizeof(a));
         a.x = x; a.U = U; a.V = V; a.dY = dY; a.T = const_cast<void*>(T_stash);
@@ -655,7 +683,7 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.ws_G = ws + w.off_dT; a.stream = stream;
         a.du_slices = &su_info; a.dv_slices = &sv_info;
         int handled = 0;
-        st = tc::conv_bwd(a, &handled);
+        st = dtype == PF_BF16 ? tc::conv_bwd(a, &handled) : tc::f32_conv_bwd(a, &handled);
         if (st != PF_OK) return st;
         if (handled) return finish();
         su_info = tc::LinearArgs::Slices();

@@ -32,7 +32,7 @@ inline size_t dtype_size(int dtype) { return dtype == PF_BF16 ? 2 : 4; }
 
 // ---------------------------------------------------------------------------------------
 // Generic strided / implicit matrix views consumed by the FMA (SIMT) GEMM.  The FMA path
-// serves fp32 storage and every bf16 shape outside the tensor-core envelope.
+// serves every shape and layout outside the tensor-core envelopes.
 // ---------------------------------------------------------------------------------------
 enum AKind : int {
     A_PLAIN = 0,     // A(i,l) = p[i*s_row + l*s_col]

@@ -1,7 +1,7 @@
 // FMA (CUDA-core) GEMM with implicit-matrix views.
 //
-// Serves the fp32 storage path (single-pass TF32 cannot reach 1e-4 after two chained
-// products) and every bf16 shape outside the tensor-core envelope.  One kernel, templated on
+// Serves every shape and layout outside the tensor-core envelopes (odd row pitches on even widths,
+// channel counts that are not multiples of 8 in bf16 or 4 in fp32).  One kernel, templated on
 // how operand A is addressed: plain strided, im2col of an NHWC image (convolution forward
 // and dU), or the gather form of the transposed convolution (dX).  Products accumulate in
 // fp32; a reduction split over K writes fp32 partials that a second kernel sums in a fixed

@@ -109,21 +109,6 @@ cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const Gemm
     return e;
 }
 
-// Device address of the counter set a launch may use (sets rotate, so that launches in flight on
-// different streams do not share counters unless more than kFixSlots of them overlap).
-unsigned int* next_fix_counters() {
-    static unsigned int* base[64] = {};
-    static std::atomic<unsigned int> next{0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (!base[dev]) {
-        void* ptr = nullptr;
-        if (cudaGetSymbolAddress(&ptr, g_fix_counters) != cudaSuccess) return nullptr;
-        base[dev] = static_cast<unsigned int*>(ptr);
-    }
-    return base[dev] + static_cast<size_t>(next.fetch_add(1) % kFixSlots) * (kFixTiles * 2);
-}
-
 // Workspace floats of a split product: one 128 x bn block per (tile, slice).
 size_t partial_bytes(int64_t M, int64_t N, int splits) {
     if (splits <= 1) return 0;
@@ -311,7 +296,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
         const int64_t rper = ceil_div(kBM, p.splits);
         const int64_t room = static_cast<int64_t>(p.num_stages) * (kBM * kBK * 2 + bn * kBK * 2);
         if (rper * p.splits * (bn * 4) > room || static_cast<int64_t>(kBM) * bn * 4 > room) return PF_ERR_UNSUPPORTED;
-        p.counters = next_fix_counters();
+        p.counters = split_counters();
         if (!p.counters) return PF_ERR_CUDA;
     }
     out->grid = grid;
@@ -469,6 +454,21 @@ void bwd_partial_bytes(int64_t m, int64_t k, int64_t n, int64_t r, size_t* bytes
 }
 
 }  // namespace
+
+// Device address of the counter set a launch may use (sets rotate, so that launches in flight on
+// different streams do not share counters unless more than kFixSlots of them overlap).
+unsigned int* split_counters() {
+    static unsigned int* base[64] = {};
+    static std::atomic<unsigned int> next{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (!base[dev]) {
+        void* ptr = nullptr;
+        if (cudaGetSymbolAddress(&ptr, g_fix_counters) != cudaSuccess) return nullptr;
+        base[dev] = static_cast<unsigned int*>(ptr);
+    }
+    return base[dev] + static_cast<size_t>(next.fetch_add(1) % kFixSlots) * (kFixTiles * 2);
+}
 
 // Extra workspace of the tensor-core linear path: repack buffers for operands whose width is not a
 // multiple of 8 elements (TMA needs 16-byte row pitches), the two m x r intermediates at a padded

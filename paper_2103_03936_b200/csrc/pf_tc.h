@@ -99,6 +99,16 @@ void reset_fix_counters();  // clears the slice-sum counters (after PF_ERR_TIMEO
 size_t linear_fwd_need(const LinearArgs& a, bool* handles);   // bytes of a.ws the forward really touches
 int linear_fwd(const LinearArgs& a, int* handled);
 int linear_bwd(const LinearArgs& a, int* handled);
+
+// fp32 storage (pf_tc_f32.cu).  `room`: bytes available at a.ws (a call that does not fit is declined).
+size_t f32_linear_workspace(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd);
+int f32_linear_fwd(const LinearArgs& a, int* handled, size_t room);
+int f32_linear_bwd(const LinearArgs& a, int* handled);
+size_t f32_conv_workspace(const ConvArgs& a, bool bwd);      // a: sizes only
+int f32_conv_fwd(const ConvArgs& a, int* handled);
+int f32_conv_bwd(const ConvArgs& a, int* handled);
+// Device counters for one product whose contraction is split (null on error).
+unsigned int* split_counters();
 int conv_fwd(const ConvArgs& a, int* handled);
 int conv_bwd(const ConvArgs& a, int* handled);
 

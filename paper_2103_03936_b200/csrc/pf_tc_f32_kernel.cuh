@@ -1,0 +1,664 @@
+// fp32 products on the tensor cores (sm_100a): every fp32 operand value is split exactly into three bf16 values
+//   x = x1 + x2 + x3,  x1 = bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2
+// (8 + 8 + 8 significand bits), and a product a b is the sum of the six partial products that reach fp32
+// precision: a1 b1 | a1 b2 + a2 b1 + a2 b2 + a1 b3 + a3 b1 (the three left out are below 2^-24 of it).
+//
+// Accumulation.  A tcgen05.mma truncates when it adds to its fp32 accumulator (measured: -0.5 ulp per MMA on
+// sums of one sign), so long sums must not stay in tensor memory: the main products a1 b1 accumulate over 64
+// elements of the contraction in one of two accumulators, which the worker warps then add, with
+// round-to-nearest, to fp32 sums in their registers; the five correction products, 2^-8 of the sum, have an
+// accumulator of their own, added once at the end.  The result is as accurate as an fp32 FMA kernel.
+//
+// One CTA computes a 128 x BN tile of C = A * B or one slice of its contraction.  Warps: 0 = TMA producer of
+// A, 1 = tensor memory + MMA issue, 2..17 = workers (split the operands, drain the accumulators, epilogue),
+// 18 = TMA producer of B.  A k-block is 32 elements: the fp32 tiles (128-byte-swizzled boxes of 32 floats)
+// arrive in a ring and the workers split them into one of two half buffers of planes, which 12 MMAs read.  The
+// workers are two groups of eight warps that take alternate k-blocks (and half buffers): one k-block is a chain
+// of waits and shared-memory round trips of about 1 us for a warp whatever it computes.
+// Splitting on chip rather than in a pass of its own: no workspace, no extra launch, 32 KB of loads per
+// k-block instead of 48 KB.
+// What bounds it is shared-memory bandwidth: an MMA that takes both operands from shared memory reads 128
+// bytes per clock, all there is, while TMA writes and the workers read and write the tiles.  So the planes of
+// A go to TENSOR memory (a thread splits 16 contraction elements of its row, whatever the operand's
+// orientation) and only B's planes, shared by all rows, to shared memory: 136 KB instead of 208 KB through
+// shared memory per k-block of a 128 x 128 tile, 0.95 -> 0.6 us.
+#ifndef PF_TC_F32_KERNEL_CUH_
+#define PF_TC_F32_KERNEL_CUH_
+
+#include <cuda.h>
+
+#include "pf_tc_prims.cuh"
+
+namespace pf {
+namespace tc {
+
+struct F32Params {
+    int M, N;
+    int a_mn, b_mn;          // 1 = operand stored with the M/N index contiguous
+    int bn;                  // columns of a tile: 64 or 128
+    int nkb, kb_per_split, splits;     // 32-element k-blocks
+    int num_stages;
+    int mode;                // 0 = plain, 1 / 2 / 3 = the convolution products below
+    int tiles_x, tiles_y;
+    float* C;
+    long long ldc;
+    float* C2;               // optional second copy at another pitch
+    long long ldc2;
+    const float* bias;       // optional epilogue of an unsplit product: C = act(A B + bias)
+    int act;
+    float* partial;          // splits > 1: slices, [tile][slice][column quarter][128 rows][bn / 4], pieces XOR-permuted by the row
+    unsigned int* counters;
+    unsigned int* status;
+    // Convolution (kMode 1 = dX, 2 = dU, 3 = the thin convolution forward); names as in pf_tc_gemm_kernel.cuh, with 32-channel
+    // blocks.  Tiles of modes 1 and 3 are blocks of pixels of an image of out_h x out_w output pixels, `step` pixels apart.
+    int cv_blks, cv_kw, cv_kh, cv_pad, cv_stride, cv_C, cv_bh, cv_nb, cv_tpi, cv_N, cv_bw, cv_inv_bw, cv_inv_bh, cv_tiles_class;
+    int out_h, out_w, step;
+    int cv_blocks;           // dU: 32-channel blocks of the unrolled factor
+    int cv_wblk;             // dU: blocks of cv_bw pixels per image row
+    int rows_tile, kpix;
+    int ragged;              // mode 3: C is not a multiple of 32, tmB is [taps][C][R]
+};
+
+struct F32Launch {
+    CUtensorMap ta[3], tb[3];
+    F32Params p[3];
+    int end[3];              // running total of blocks
+};
+// Launch of the instantiation with the convolution's modes (pf_tc_f32_conv.cu).
+cudaError_t launch_f32_conv(int blocks, size_t smem, cudaStream_t stream, const F32Launch& a);
+
+namespace {
+
+constexpr int kF32Threads = 608;
+constexpr int kF32MaxStages = 8;
+constexpr int kChunk = 2;                    // k-blocks per main accumulator: 64 elements of the contraction
+static_assert(kChunk == 2, "one k-block per worker group and chunk");
+constexpr uint32_t kF32TileA = 16384;        // 128 x 32 floats
+constexpr uint32_t kColsA = 16;              // tensor-memory columns of one plane of A's k-block (32 bf16 per row)
+
+struct F32Ctl {
+    uint64_t full[kF32MaxStages];
+    uint64_t empty[kF32MaxStages];
+    uint64_t split_full[2];      // a half buffer of planes is complete (8 worker warps)
+    uint64_t split_empty[2];     // the MMAs have read it
+    uint64_t main_full[2];       // a main accumulator holds its chunk
+    uint64_t main_empty[2];      // the workers have drained it (16 warps)
+    uint64_t corr_full;
+    uint64_t fix_full;
+    uint32_t tmem_base;
+    uint32_t abort;
+    uint32_t fix_ok;
+};
+
+__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// The three bf16 planes of a pair of floats.
+__device__ __forceinline__ void split_pair(float lo, float hi, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
+    p1 = cvt_bf16x2(lo, hi);
+    lo -= __uint_as_float(p1 << 16);
+    hi -= __uint_as_float(p1 & 0xffff0000u);
+    p2 = cvt_bf16x2(lo, hi);
+    lo -= __uint_as_float(p2 << 16);
+    hi -= __uint_as_float(p2 & 0xffff0000u);
+    p3 = __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);      // what is left has at most 8 bits: no rounding
+}
+__device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_acquire(const unsigned int* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// A: the thread owns row q * 32 + lane of the tile and 16 of the k-block's elements (half kh), whose planes it writes to
+// tensor memory.  K-major tile: four 16-byte chunks of the row; MN-major: box q holds the rows' 32 columns, one
+// word per contraction row (both free of bank conflicts).
+__device__ __forceinline__ void split_a(uint32_t src, uint32_t taddr, bool mn, int q, int kh, int lane) {
+    float x[16];
+    if (mn) {
+        const uint32_t box = src + static_cast<uint32_t>(q) * 4096u + static_cast<uint32_t>(kh) * 2048u + static_cast<uint32_t>(lane & 3) * 4u;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            x[k] = __uint_as_float(ld_shared_u32(box + static_cast<uint32_t>(k) * 128u + (static_cast<uint32_t>((lane >> 2) ^ (k & 7)) << 4)));
+    } else {
+        const uint32_t row = src + static_cast<uint32_t>(q * 32 + lane) * 128u;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint4 v = ld_shared_v4(row + (static_cast<uint32_t>((kh * 4 + c) ^ (lane & 7)) << 4));
+            x[4 * c] = __uint_as_float(v.x); x[4 * c + 1] = __uint_as_float(v.y);
+            x[4 * c + 2] = __uint_as_float(v.z); x[4 * c + 3] = __uint_as_float(v.w);
+        }
+    }
+    uint32_t p1[8], p2[8], p3[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) split_pair(x[2 * c], x[2 * c + 1], p1[c], p2[c], p3[c]);
+    tmem_st8(taddr, p1);
+    tmem_st8(taddr + kColsA, p2);
+    tmem_st8(taddr + 2 * kColsA, p3);
+}
+
+// B: each warp splits kRows / 8 rows of 32 floats (row = 128 bytes, 16-byte chunks XOR-swizzled by the row, as TMA
+// wrote them) into the planes.  K-major: row r is row r of a plane, its 64 bytes go to half h of the 128-byte
+// row.  MN-major: the rows are [box of 32 columns][contraction row], a panel of 64 columns is two boxes and
+// the contraction row lies in half h of the panel.  Eight lanes read one row's eight chunks (no conflicts);
+// the rows of a half warp differ by 4, so that their 64-byte runs fall into different banks.  All loads
+// come before the first store (asm statements keep their order).
+template <int kRows>
+__device__ __forceinline__ void split_b(uint32_t src, uint32_t dst, uint32_t plane, bool mn, uint32_t h, int w, int lane) {
+    const int q = lane >> 3, j = lane & 7;
+    uint4 v[kRows / 32];
+    auto row_of = [&](int it) { return w * (kRows / 8) + (it >> 1) * 8 + (it & 1) * 2 + (q & 1) * 4 + (q >> 1); };
+#pragma unroll
+    for (int it = 0; it < kRows / 32; ++it) {
+        const int r = row_of(it);
+        v[it] = ld_shared_v4(src + static_cast<uint32_t>(r) * 128u + (static_cast<uint32_t>(j ^ (r & 7)) << 4));
+    }
+#pragma unroll
+    for (int it = 0; it < kRows / 32; ++it) {
+        const int r = row_of(it);
+        const uint32_t hi = mn ? static_cast<uint32_t>(r >> 5) & 1u : h;
+        const uint32_t row = mn ? (static_cast<uint32_t>(r >> 6) << 6) + 32u * h + static_cast<uint32_t>(r & 31) : static_cast<uint32_t>(r);
+        const uint32_t at = dst + row * 128u + ((((hi << 2) + static_cast<uint32_t>(j >> 1)) ^ static_cast<uint32_t>(r & 7)) << 4) +
+                            static_cast<uint32_t>(j & 1) * 8u;
+        uint32_t a1, a2, a3, b1, b2, b3;
+        split_pair(__uint_as_float(v[it].x), __uint_as_float(v[it].y), a1, a2, a3);
+        split_pair(__uint_as_float(v[it].z), __uint_as_float(v[it].w), b1, b2, b3);
+        st_shared_v2(at, a1, b1);
+        st_shared_v2(at + plane, a2, b2);
+        st_shared_v2(at + 2 * plane, a3, b3);
+    }
+}
+
+struct F32Origin {
+    int img, row, ph, pw, na, nb, a0, b0;
+};
+template <int kMode>
+__device__ __forceinline__ F32Origin f32_origin(const F32Params& p, int bx) {
+    F32Origin o = {};
+    if constexpr (kMode == 1 || kMode == 3) {
+        int t = bx;
+        o.na = p.cv_kh;
+        o.nb = p.cv_kw;
+        if (kMode == 1 && p.cv_stride > 1) {
+            const int s = p.cv_stride, cls = bx / p.cv_tiles_class;
+            t = bx - cls * p.cv_tiles_class;
+            o.ph = cls / s;
+            o.pw = cls - o.ph * s;
+            o.a0 = (o.ph + p.cv_pad) % s;
+            o.b0 = (o.pw + p.cv_pad) % s;
+            o.na = (p.cv_kh - o.a0 + s - 1) / s;
+            o.nb = (p.cv_kw - o.b0 + s - 1) / s;
+        }
+        const int g = p.cv_tpi > 1 ? t / p.cv_tpi : t;
+        o.img = g * p.cv_nb;
+        o.row = (t - g * p.cv_tpi) * p.cv_bh;
+    }
+    return o;
+}
+// Row of the output matrix that row r of tile bx holds, -1 if none.
+template <int kMode>
+__device__ __forceinline__ int f32_row(const F32Params& p, const F32Origin& o, int bx, int r) {
+    if constexpr (kMode == 0) {
+        const int row = bx * 128 + r;
+        return row < p.M ? row : -1;
+    } else if constexpr (kMode == 2) {
+        const int blk = bx * 4 + (r >> 5), tap = blk / p.cv_blks, c = (blk - tap * p.cv_blks) * 32 + (r & 31);
+        return (blk < p.cv_blocks && c < p.cv_C) ? tap * p.cv_C + c : -1;
+    } else {
+        const int line = (r * p.cv_inv_bw) >> 16, w = (r - line * p.cv_bw) * p.step + o.pw;
+        const int i = (line * p.cv_inv_bh) >> 16, img = o.img + i, h = (o.row + line - i * p.cv_bh) * p.step + o.ph;
+        return (r < p.rows_tile && img < p.cv_N && h < p.out_h && w < p.out_w) ? (img * p.out_h + h) * p.out_w + w : -1;
+    }
+}
+
+template <int BN, int kMode>
+__device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorMap& tmB, const F32Params& p, const int bx, const int by,
+                                         const int bz) {
+    constexpr uint32_t kTileB = BN * 128;                 // BN x 32 floats
+    constexpr uint32_t kStage = kF32TileA + kTileB;
+    constexpr uint32_t kPlaneB = BN * 128;                // BN x 64 bf16
+    constexpr int kCols = BN / 4;                         // columns of a worker warp
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    uint8_t* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);
+    F32Ctl* ctl = reinterpret_cast<F32Ctl*>(smem);
+    const uint32_t planes_b = smem_u32(smem + 1024);      // three planes of B (A's are in tensor memory)
+    constexpr uint32_t kTmemA = 3 * BN;                   // after two main accumulators and the correction's: two half buffers
+    const uint32_t ring = planes_b + 3 * kPlaneB;
+    volatile uint32_t* abort_flag = &ctl->abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n0 = by * BN;
+    const F32Origin org = f32_origin<kMode>(p, bx);
+    const int nkb_total = kMode == 1 ? org.na * org.nb * p.cv_blks : p.nkb;
+    const int kb_beg = bz * p.kb_per_split;
+    const int nkb = min(nkb_total, kb_beg + p.kb_per_split) - kb_beg;
+    const uint32_t NS = static_cast<uint32_t>(p.num_stages);
+    const int tile = by * p.tiles_x + bx;
+
+    if (threadIdx.x == 0) {
+        for (uint32_t s = 0; s < NS; ++s) {
+            mbar_init(smem_u32(&ctl->full[s]), 2);
+            mbar_init(smem_u32(&ctl->empty[s]), 8);
+        }
+        for (int h = 0; h < 2; ++h) {
+            mbar_init(smem_u32(&ctl->split_full[h]), 8);
+            mbar_init(smem_u32(&ctl->split_empty[h]), 1);
+            mbar_init(smem_u32(&ctl->main_full[h]), 1);
+            mbar_init(smem_u32(&ctl->main_empty[h]), 16);
+        }
+        mbar_init(smem_u32(&ctl->corr_full), 1);
+        mbar_init(smem_u32(&ctl->fix_full), 1);
+        ctl->abort = 0;
+        ctl->fix_ok = 0;
+        fence_barrier_init();
+        fence_proxy_async_smem();
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
+    if (kMode == 2 && p.kpix < 32) {
+        // contraction rows that TMA never writes must read as zero in every 32-row box of every stage
+        const int pieces = (32 - p.kpix) * 8, boxes = static_cast<int>(kStage / 4096) * static_cast<int>(NS);
+        for (int i = threadIdx.x; i < boxes * pieces; i += blockDim.x) {
+            const int box = i / pieces;
+            st_shared_v4(ring + box * 4096 + p.kpix * 128 + (i - box * pieces) * 16, make_uint4(0, 0, 0, 0));
+        }
+        fence_proxy_async_smem();
+    }
+    if (warp == 1) tmem_alloc(smem_u32(&ctl->tmem_base), 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    pdl_wait();                 // everything above overlapped the previous kernel's tail
+    pdl_launch_dependents();
+    const uint32_t tmem = ctl->tmem_base;
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+
+    if (warp == 0 || warp == 18) {
+        if (elect_one()) {
+            const bool do_a = warp == 0;
+            const uint32_t base = ring + (do_a ? 0u : kF32TileA);
+            uint32_t bytes = do_a ? kF32TileA : kTileB;
+            int boxes = 4;                                 // dU: 32-channel blocks of A that exist
+            if constexpr (kMode == 2) {
+                boxes = min(4, p.cv_blocks - bx * 4);
+                bytes = static_cast<uint32_t>(p.kpix) * 128u * static_cast<uint32_t>(do_a ? boxes : BN / 32);
+            } else if constexpr (kMode != 0) {
+                if (do_a) bytes = static_cast<uint32_t>(p.rows_tile) * 128u;
+            }
+            auto produce = [&](auto&& issue) {
+                uint32_t s = 0, ph = 1, dst = base;
+                for (int i = 0; i < nkb; ++i) {
+                    if (!mbar_wait(empty0 + 8 * s, ph, abort_flag, p.status)) break;
+                    const uint32_t full = full0 + 8 * s;
+                    mbar_expect_tx(full, bytes);
+                    issue(dst, full);
+                    dst += kStage;
+                    if (++s == NS) { s = 0; dst = base; ph ^= 1u; }
+                }
+            };
+            int k0 = kb_beg * 32;
+            if constexpr (kMode == 0) {
+                const int mn0 = do_a ? bx * 128 : n0, width = do_a ? 4 : BN / 32;
+                const CUtensorMap* map = do_a ? &tmA : &tmB;
+                if (do_a ? p.a_mn : p.b_mn) {
+                    produce([&](uint32_t dst, uint32_t full) {
+                        for (int b = 0; b < width; ++b) tma_load_2d(dst + b * 4096, map, full, mn0 + b * 32, k0);
+                        k0 += 32;
+                    });
+                } else {
+                    produce([&](uint32_t dst, uint32_t full) { tma_load_2d(dst, map, full, k0, mn0); k0 += 32; });
+                }
+            } else if constexpr (kMode == 2) {
+                const int bh = p.cv_bh, bw = p.cv_bw, nwb = p.cv_wblk, tpi = p.cv_tpi;
+                int wb = kb_beg % nwb, t = kb_beg / nwb, img = t / tpi;
+                t -= img * tpi;
+                img *= p.cv_nb;
+                auto advance = [&] {
+                    if (++wb == nwb) { wb = 0; if (++t == tpi) { t = 0; img += p.cv_nb; } }
+                };
+                if (do_a) {
+                    int c[4], x[4], y[4];
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const int blk = bx * 4 + b, tap = blk / p.cv_blks, ta = tap / p.cv_kw;
+                        c[b] = (blk - tap * p.cv_blks) * 32;
+                        x[b] = tap - ta * p.cv_kw - p.cv_pad;
+                        y[b] = ta - p.cv_pad;
+                    }
+                    const int s = p.cv_stride;
+                    produce([&](uint32_t dst, uint32_t full) {
+                        const int x0 = wb * bw * s, y0 = t * bh * s;
+#pragma unroll
+                        for (int b = 0; b < 4; ++b)
+                            if (b < boxes) tma_load_4d(dst + b * 4096, &tmA, full, c[b], x0 + x[b], y0 + y[b], img);
+                        advance();
+                    });
+                } else {
+                    produce([&](uint32_t dst, uint32_t full) {
+#pragma unroll
+                        for (int b = 0; b < BN / 32; ++b) tma_load_4d(dst + b * 4096, &tmB, full, n0 + 32 * b, wb * bw, t * bh, img);
+                        advance();
+                    });
+                }
+            } else {
+                const int blks = p.cv_blks, ntb = org.nb;
+                int cb = kb_beg % blks, tb = kb_beg / blks, ta = tb / ntb;
+                tb -= ta * ntb;
+                auto advance = [&] {
+                    if (++cb == blks) { cb = 0; if (++tb == ntb) { tb = 0; ++ta; } }
+                };
+                if (do_a) {
+                    const int s = p.cv_stride, sign = kMode == 1 ? -1 : 1;
+                    const int y0 = kMode == 1 ? org.row + (org.ph + p.cv_pad - org.a0) / s : org.row * s - p.cv_pad;
+                    const int x0 = kMode == 1 ? (org.pw + p.cv_pad - org.b0) / s : -p.cv_pad;
+                    produce([&](uint32_t dst, uint32_t full) {
+                        tma_load_4d(dst, &tmA, full, cb * 32, x0 + sign * tb, y0 + sign * ta, org.img);
+                        advance();
+                    });
+                } else if constexpr (kMode == 1) {
+                    const int s = p.cv_stride;
+                    produce([&](uint32_t dst, uint32_t full) {
+                        tma_load_2d(dst, &tmB, full, cb * 32, ((org.a0 + ta * s) * p.cv_kw + org.b0 + tb * s) * p.cv_C + n0);
+                        advance();
+                    });
+                } else if (p.ragged) {
+                    produce([&](uint32_t dst, uint32_t full) {
+                        for (int b = 0; b < BN / 32; ++b) tma_load_3d(dst + b * 4096, &tmB, full, n0 + 32 * b, cb * 32, ta * ntb + tb);
+                        advance();
+                    });
+                } else {
+                    produce([&](uint32_t dst, uint32_t full) {
+                        for (int b = 0; b < BN / 32; ++b) tma_load_2d(dst + b * 4096, &tmB, full, n0 + 32 * b, k0);
+                        k0 += 32;
+                    });
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (elect_one()) {
+            const uint32_t idesc = make_idesc_bf16(128, BN, 0, p.b_mn);
+            const uint64_t b_desc0 = p.b_mn ? make_smem_desc(planes_b, 8192, 1024) : make_smem_desc(planes_b, 16, 1024);
+            const uint32_t b_half = p.b_mn ? 256u : 4u;      // 16-byte units to half 1
+            const uint32_t b_step = p.b_mn ? 128u : 2u;      // ... to the next 16 elements
+            constexpr uint32_t pb = kPlaneB >> 4;
+            const uint32_t corr = tmem + 2 * BN;
+            bool ok = true;
+            int in_chunk = 0;
+            uint32_t buf = 0, bufph = 1;                  // phase of main_empty[buf]: the first use of each finds it free
+            for (int i = 0; i < nkb; ++i) {
+                const uint32_t h = static_cast<uint32_t>(i) & 1u;
+                if (in_chunk == 0) {
+                    ok = mbar_wait(smem_u32(&ctl->main_empty[buf]), bufph, abort_flag, p.status);
+                    if (!ok) break;
+                }
+                ok = mbar_wait(smem_u32(&ctl->split_full[h]), static_cast<uint32_t>(i >> 1) & 1u, abort_flag, p.status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t b0 = b_desc0 + h * b_half;
+                const uint32_t a0 = tmem + kTmemA + h * (3 * kColsA), d = tmem + buf * BN;
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                    const uint64_t b = b0 + ks * b_step;
+                    const uint32_t a = a0 + ks * 8u;
+                    tc_mma_bf16_ta(corr, a + 2 * kColsA, b, idesc, (i > 0 || ks > 0) ? 1u : 0u);
+                    tc_mma_bf16_ta(corr, a, b + 2 * pb, idesc, 1u);
+                    tc_mma_bf16_ta(corr, a + kColsA, b + pb, idesc, 1u);
+                    tc_mma_bf16_ta(corr, a + kColsA, b, idesc, 1u);
+                    tc_mma_bf16_ta(corr, a, b + pb, idesc, 1u);
+                    tc_mma_bf16_ta(d, a, b, idesc, (in_chunk > 0 || ks > 0) ? 1u : 0u);
+                }
+                tc_commit(smem_u32(&ctl->split_empty[h]));
+                if (++in_chunk == kChunk || i + 1 == nkb) {
+                    tc_commit(smem_u32(&ctl->main_full[buf]));
+                    in_chunk = 0;
+                    buf ^= 1u;
+                    if (buf == 0) bufph ^= 1u;
+                }
+            }
+            if (ok) tc_commit(smem_u32(&ctl->corr_full));
+        }
+    } else {
+        const int w = (warp - 2) & 7, grp = (warp - 2) >> 3, q = warp & 3, kh = w >> 2, colq = grp * 2 + kh;
+        const uint32_t rows_base = tmem + (static_cast<uint32_t>(q * 32) << 16);
+        const uint32_t lane_base = rows_base + static_cast<uint32_t>(colq * kCols);
+        const bool a_mn = p.a_mn, b_mn = p.b_mn;
+        const uint32_t h = static_cast<uint32_t>(grp);
+        const uint32_t a_dst = rows_base + kTmemA + h * (3 * kColsA) + static_cast<uint32_t>(kh * 8);
+        const int chunks = (nkb + kChunk - 1) / kChunk;
+        float acc[kCols];
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
+        auto add_from = [&](uint32_t taddr) {
+            uint32_t v[kCols];
+            if constexpr (kCols == 32) tmem_ld32(taddr, v);
+            else tmem_ld16(taddr, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < kCols; ++e) acc[e] += __uint_as_float(v[e]);
+        };
+        bool ok = true;
+        auto drain = [&](int c) {
+            const uint32_t b = static_cast<uint32_t>(c) & 1u;
+            ok = mbar_wait_warp(smem_u32(&ctl->main_full[b]), static_cast<uint32_t>(c >> 1) & 1u, abort_flag, p.status);
+            tc_fence_after();
+            if (!ok) return;
+            add_from(lane_base + b * BN);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&ctl->main_empty[b]));
+        };
+        uint32_t s = static_cast<uint32_t>(grp), sph = 0;          // ring position of this group's next k-block
+        for (int c = 0; c < chunks && ok; ++c) {
+            const int i = c * kChunk + grp;
+            if (i < nkb) {
+                ok = mbar_wait_warp(smem_u32(&ctl->split_empty[h]), (static_cast<uint32_t>(c) & 1u) ^ 1u, abort_flag, p.status);
+                if (!ok) break;
+                ok = mbar_wait_warp(full0 + 8 * s, sph, abort_flag, p.status);
+                if (!ok) break;
+                __syncwarp();                 // orders every lane's reads of the tile after lane 0's wait
+                tc_fence_after();             // the MMAs of two k-blocks ago have read this half buffer
+                const uint32_t stage = ring + s * kStage;
+                split_a(stage, a_dst, a_mn, q, kh, lane);
+                split_b<BN>(stage + kF32TileA, planes_b, kPlaneB, b_mn, h, w, lane);
+                tmem_st_wait();
+                tc_fence_before();
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(smem_u32(&ctl->split_full[h]));
+                    mbar_arrive(empty0 + 8 * s);
+                }
+                s += 2;
+                if (s >= NS) { s -= NS; sph ^= 1u; }
+            }
+            if (c > 0) drain(c - 1);
+        }
+        if (ok) drain(chunks - 1);
+        if (ok) {
+            ok = mbar_wait_warp(smem_u32(&ctl->corr_full), 0, abort_flag, p.status);
+            tc_fence_after();
+        }
+        if (ok) {
+            add_from(lane_base + 2 * BN);
+            // 32 rows of kCols floats go through shared memory (the ring is idle: every warp has split its last k-block once
+            // corr_full fired), 16-byte pieces XOR-permuted by the row against bank conflicts
+            constexpr uint32_t kPieces = kCols / 4, kRowBytes = kCols * 4;
+            const uint32_t panel = ring + static_cast<uint32_t>(colq * 128 + q * 32) * kRowBytes;
+            const uint32_t own = panel + static_cast<uint32_t>(lane) * kRowBytes;
+#pragma unroll
+            for (uint32_t g = 0; g < kPieces; ++g)
+                st_shared_v4(own + ((g ^ (static_cast<uint32_t>(lane) & (kPieces - 1))) << 4),
+                             make_uint4(__float_as_uint(acc[4 * g]), __float_as_uint(acc[4 * g + 1]), __float_as_uint(acc[4 * g + 2]),
+                                        __float_as_uint(acc[4 * g + 3])));
+            if (p.splits > 1) {
+                // slice: they leave as one bulk copy; then the warp reports
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    uint8_t* dst = reinterpret_cast<uint8_t*>(p.partial) + (static_cast<size_t>(tile) * p.splits + bz) * (128u * BN * 4u) +
+                                   static_cast<size_t>(colq * 128 + q * 32) * kRowBytes;
+                    bulk_store(dst, panel, 32u * kRowBytes);
+                    tma_store_commit();
+                    tma_store_wait_all();
+                    fence_proxy_async_all();
+                    __threadfence();
+                    atomicAdd(p.counters + 2 * tile, 1u);
+                }
+            } else {
+                // stored as whole row segments, 32 / kPieces rows per instruction
+                __syncwarp();
+                constexpr int kRowsPer = 32 / static_cast<int>(kPieces);
+                const int sub = lane / static_cast<int>(kPieces), piece = lane % static_cast<int>(kPieces);
+                const bool vec = (p.ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(p.C) & 15) == 0;
+                const int col = n0 + colq * kCols + piece * 4;
+                float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (p.bias) {
+                    if (col < p.N) b.x = __ldg(p.bias + col);
+                    if (col + 1 < p.N) b.y = __ldg(p.bias + col + 1);
+                    if (col + 2 < p.N) b.z = __ldg(p.bias + col + 2);
+                    if (col + 3 < p.N) b.w = __ldg(p.bias + col + 3);
+                }
+#pragma unroll 4
+                for (int i = 0; i < 32 / kRowsPer; ++i) {
+                    const int rr = i * kRowsPer + sub;
+                    const uint4 u = ld_shared_v4(panel + static_cast<uint32_t>(rr) * kRowBytes +
+                                                 ((static_cast<uint32_t>(piece) ^ (static_cast<uint32_t>(rr) & (kPieces - 1))) << 4));
+                    float4 v = make_float4(__uint_as_float(u.x) + b.x, __uint_as_float(u.y) + b.y, __uint_as_float(u.z) + b.z,
+                                           __uint_as_float(u.w) + b.w);
+                    if (p.act == 1) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+                    const int row = f32_row<kMode>(p, org, bx, q * 32 + rr);
+                    if (row < 0) continue;
+                    float* dst = p.C + static_cast<size_t>(row) * p.ldc + col;
+                    if (vec && col + 3 < p.N) {
+                        *reinterpret_cast<float4*>(dst) = v;
+                    } else {
+                        if (col < p.N) dst[0] = v.x;
+                        if (col + 1 < p.N) dst[1] = v.y;
+                        if (col + 2 < p.N) dst[2] = v.z;
+                        if (col + 3 < p.N) dst[3] = v.w;
+                    }
+                    if (p.C2) {
+                        float* d2 = p.C2 + static_cast<size_t>(row) * p.ldc2 + col;
+                        if (col < p.N) d2[0] = v.x;
+                        if (col + 1 < p.N) d2[1] = v.y;
+                        if (col + 2 < p.N) d2[2] = v.z;
+                        if (col + 3 < p.N) d2[3] = v.w;
+                    }
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem, 512);
+    if (p.splits <= 1) return;
+
+    // ---- slice sum (as in pf_tc_gemm_kernel.cuh): once all slices of the tile are in the workspace, each CTA gathers its
+    // share of the rows from every slice, adds them in slice order and stores them
+    constexpr uint32_t kPieces = kCols / 4, kRowBytes = kCols * 4;
+    unsigned int* cnt = p.counters + 2 * tile;
+    const int S = p.splits;
+    const int rper = (128 + S - 1) / S, r_beg = bz * rper;
+    const int nr = max(0, min(128, r_beg + rper) - r_beg);
+    const uint32_t share = static_cast<uint32_t>(nr) * kRowBytes;       // bytes of one column quarter of one slice
+    if (warp == 0) {
+        uint32_t good = (*abort_flag == 0u) ? 1u : 0u;
+        if (good && lane == 0) {
+            const unsigned int want = 16u * static_cast<unsigned int>(S);
+            const long long t0 = clock64();
+            while (ld_acquire(cnt) < want) {
+                if (clock64() - t0 > kWaitCycleLimit) {
+                    good = 0u;
+                    if (p.status) atomicExch(p.status, kStatusTimeout);
+                    break;
+                }
+            }
+            __threadfence();
+            if (good && nr > 0) mbar_expect_tx(smem_u32(&ctl->fix_full), 4u * share * static_cast<uint32_t>(S));
+        }
+        good = __shfl_sync(0xffffffffu, good, 0);
+        __syncwarp();                        // lane 0's acquire orders the copies of all lanes
+        fence_proxy_async_all();
+        if (good && nr > 0) {
+            const uint32_t bar = smem_u32(&ctl->fix_full);
+            const uint8_t* src = reinterpret_cast<const uint8_t*>(p.partial) + static_cast<size_t>(tile) * S * (128u * BN * 4u) +
+                                 static_cast<size_t>(r_beg) * kRowBytes;
+            for (int e = lane; e < 4 * S; e += 32)          // (slice, column quarter) pairs, one copy each
+                bulk_load(ring + static_cast<uint32_t>(e) * share,
+                          src + static_cast<size_t>(e >> 2) * (128u * BN * 4u) + static_cast<size_t>(e & 3) * 128u * kRowBytes, share, bar);
+            good = mbar_wait_warp(bar, 0, abort_flag, p.status) ? 1u : 0u;
+        }
+        if (lane == 0) ctl->fix_ok = good;
+    }
+    __syncthreads();
+    if (ctl->fix_ok) {
+        const bool vec = (p.ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(p.C) & 15) == 0;
+        for (int id = threadIdx.x; id < nr * static_cast<int>(4 * kPieces); id += kF32Threads) {
+            const int rl = id / static_cast<int>(4 * kPieces), pc = id % static_cast<int>(4 * kPieces);
+            const int cq = pc / static_cast<int>(kPieces), pp = pc % static_cast<int>(kPieces), rr = r_beg + rl;
+            const uint32_t o = static_cast<uint32_t>(cq) * share + static_cast<uint32_t>(rl) * kRowBytes +
+                               ((static_cast<uint32_t>(pp) ^ (static_cast<uint32_t>(rr) & (kPieces - 1))) << 4);
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+            for (int sl = 0; sl < S; ++sl) {
+                const uint4 v = ld_shared_v4(ring + static_cast<uint32_t>(4 * sl) * share + o);
+                a.x += __uint_as_float(v.x); a.y += __uint_as_float(v.y);
+                a.z += __uint_as_float(v.z); a.w += __uint_as_float(v.w);
+            }
+            const int row = f32_row<kMode>(p, org, bx, rr), col = n0 + cq * kCols + pp * 4;
+            if (row < 0) continue;
+            const float v[4] = {a.x, a.y, a.z, a.w};
+            float* dst = p.C + static_cast<size_t>(row) * p.ldc + col;
+            if (vec && col + 3 < p.N) *reinterpret_cast<float4*>(dst) = a;
+            else
+                for (int e = 0; e < 4; ++e)
+                    if (col + e < p.N) dst[e] = v[e];
+            if (p.C2)
+                for (int e = 0; e < 4; ++e)
+                    if (col + e < p.N) p.C2[static_cast<size_t>(row) * p.ldc2 + col + e] = v[e];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && ctl->fix_ok) {
+        const unsigned int left = atomicAdd(cnt + 1, 1u);
+        if (left + 1u == static_cast<unsigned int>(S)) {   // every slice has read what it needs
+            cnt[0] = 0u;
+            cnt[1] = 0u;
+            __threadfence();
+        }
+    }
+}
+
+// Up to three independent products in one launch, blocks [end[i - 1], end[i]) working on product i; kConv compiles the
+// convolution's addressing modes in (a translation unit of its own, as for the bf16 kernels).
+template <int kMode>
+__device__ __forceinline__ void f32_any(const CUtensorMap& ta, const CUtensorMap& tb, const F32Params& p, int idx) {
+    const int bx = idx % p.tiles_x, by = (idx / p.tiles_x) % p.tiles_y, bz = idx / (p.tiles_x * p.tiles_y);
+    if (p.bn == 64) f32_tile<64, kMode>(ta, tb, p, bx, by, bz);
+    else f32_tile<128, kMode>(ta, tb, p, bx, by, bz);
+}
+template <bool kConv>
+__device__ __forceinline__ void f32_product(const CUtensorMap& ta, const CUtensorMap& tb, const F32Params& p, int idx) {
+    if constexpr (kConv) {
+        if (p.mode == 1) return f32_any<1>(ta, tb, p, idx);
+        if (p.mode == 2) return f32_any<2>(ta, tb, p, idx);
+        if (p.mode == 3) return f32_any<3>(ta, tb, p, idx);
+    }
+    f32_any<0>(ta, tb, p, idx);
+}
+template <bool kConv>
+__global__ void __launch_bounds__(kF32Threads, 1)
+tc_f32_kernel(const __grid_constant__ F32Launch a) {
+    const int idx = blockIdx.x;
+    const int i = idx < a.end[0] ? 0 : idx < a.end[1] ? 1 : 2;
+    f32_product<kConv>(a.ta[i], a.tb[i], a.p[i], idx - (i > 0 ? a.end[i - 1] : 0));
+}
+
+}  // namespace
+}  // namespace tc
+}  // namespace pf
+#endif

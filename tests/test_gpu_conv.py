@@ -233,3 +233,13 @@ def test_tensor_core_tilings(N, H, W, C, R, O, k, stride, pad):
     _, dU1, dV1 = pf.pf_lowrank_conv_bwd(x, U, V, dY, stride=stride, pad=pad, grads_f32=True)
     torch.cuda.synchronize()
     assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
+
+
+@pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad", [(2, 9, 40, 36, 20, 24, 3, 1, 1), (5, 5, 5, 64, 16, 64, 3, 1, 1), (3, 11, 13, 100, 12, 40, 3, 2, 1),
+                                                      (1, 6, 6, 32, 132, 64, 3, 1, 0), (2, 12, 12, 64, 32, 72, 5, 3, 2)])
+def test_fp32_tensor_core_tilings(N, H, W, C, R, O, k, stride, pad):
+    """fp32 convolutions through the split-operand kernel: image rows longer than a reduction block, several images per
+    tile, ragged channel blocks, strided backward; held to fp32 accuracy."""
+    errs = run_conv(wl.ConvCase("f32tc", N, H, W, C, R, O, wl.F32, 93, kh=k, kw=k, stride=stride, pad=pad))
+    assert max(errs.values()) <= 1e-5, errs
+    run_conv(wl.ConvCase("f32tc", N, H, W, C, R, O, wl.F32, 94, kh=k, kw=k, stride=stride, pad=pad), stash=False, need_dX=False)

@@ -248,3 +248,15 @@ def test_invalid_arguments_raise_not_launch():
     with pytest.raises(pf.PfError) as e:
         pf.pf_lowrank_linear_fwd(x, U, V, workspace=torch.empty(8, dtype=torch.uint8, device="cuda"))
     assert e.value.status == 3
+
+
+@pytest.mark.parametrize("m,k,n,r", [(128, 32, 64, 64), (129, 36, 132, 68), (1, 4, 4, 4), (257, 100, 260, 33), (64, 1000, 72, 129),
+                                     (2500, 64, 200, 24), (300, 2052, 1028, 260)])
+def test_fp32_products_on_tensor_cores(m, k, n, r):
+    """fp32 storage through the split-operand kernel: edges of the 128-row, 64- and 128-column tiles and of the
+    32-element k-blocks, whole and sliced contractions, ragged pitches; held to fp32 accuracy, ten times
+    tighter than the fp32 tolerance asks."""
+    c = wl.LinearCase("f32tc", m, k, n, r, wl.F32, 23)
+    errs = run_case(c)
+    assert max(errs.values()) <= 1e-5, errs
+    run_case(wl.LinearCase("f32tc", m, k, n, r, wl.F32, 24), stash=False, need_dX=False)
