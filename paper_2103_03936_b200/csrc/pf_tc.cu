@@ -6,7 +6,6 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "pf_tc_gemm_kernel.cuh"
 #include "pf_tc_host.h"
@@ -45,38 +44,15 @@ struct Grouping {
 // box_rows rows of one group; out-of-range elements read as zero).  Cached like the 2-D maps.
 bool cached_map_3d(CUtensorMap* map, const void* p, int64_t groups, int64_t rows, int64_t cols, int64_t ld, int64_t gs,
                    int box_rows) {
-    constexpr int kSlots = 128;
-    struct Key { const void* p; int64_t groups, rows, cols, ld, gs; int box_rows; };
-    struct Slot { Key key; CUtensorMap map; bool used; };
-    static Slot slots[kSlots];
-    static std::mutex mu;
     if (groups < 1) return false;
     if (groups == 1) gs = rows * ld;                       // a single group: any valid stride
     if ((gs * 2) % 16 != 0 || gs * 2 >= (1LL << 40)) return false;
-    uint64_t h = reinterpret_cast<uintptr_t>(p) * 0x9E3779B97F4A7C15ull;
-    h ^= static_cast<uint64_t>(rows) * 0xC2B2AE3D27D4EB4Full + static_cast<uint64_t>(cols) * 0x165667B19E3779F9ull +
-         static_cast<uint64_t>(ld) * 31 + static_cast<uint64_t>(box_rows) + static_cast<uint64_t>(gs) * 131 + static_cast<uint64_t>(groups) * 7;
-    Slot& sl = slots[(h >> 20) % kSlots];
-    std::lock_guard<std::mutex> lock(mu);
-    const Key& k = sl.key;
-    if (sl.used && k.p == p && k.groups == groups && k.rows == rows && k.cols == cols && k.ld == ld && k.gs == gs &&
-        k.box_rows == box_rows) {
-        *map = sl.map;
-        return true;
-    }
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(groups)};
-    const cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * 2, static_cast<cuuint64_t>(gs) * 2};
-    const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    if (fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(p), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
-    sl.key = Key{p, groups, rows, cols, ld, gs, box_rows};
-    sl.map = *map;
-    sl.used = true;
-    return true;
+    return cached_map(map, MapKey{p, {groups, rows, cols, ld, gs, box_rows, -7, 0}}, [&](EncodeTiledFn fn) {
+        const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(groups)};
+        const cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * 2, static_cast<cuuint64_t>(gs) * 2};
+        const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u}, estr[3] = {1u, 1u, 1u};
+        return encode_bf16(fn, map, p, 3, dims, strides, box, estr);
+    });
 }
 
 size_t gemm_smem(int bn, int stages) {

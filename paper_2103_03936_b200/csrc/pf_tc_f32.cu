@@ -26,7 +26,7 @@ bool f32_encode(EncodeTiledFn fn, CUtensorMap* map, const void* p, int rank, con
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 bool f32_map_2d(CUtensorMap* map, const void* p, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-    return cached_map_wide(map, WideKey{p, {rows, cols, ld, box_rows, -2, -4, -4, -4}}, [&](EncodeTiledFn fn) {
+    return cached_map(map, MapKey{p, {rows, cols, ld, box_rows, -2, -4, -4, -4}}, [&](EncodeTiledFn fn) {
         const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
         const cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld) * 4};
         const cuuint32_t box[2] = {32u, static_cast<cuuint32_t>(box_rows)}, estr[2] = {1u, 1u};
@@ -34,7 +34,7 @@ bool f32_map_2d(CUtensorMap* map, const void* p, int64_t rows, int64_t cols, int
     });
 }
 bool f32_map_planes(CUtensorMap* map, const void* p, int64_t planes, int64_t rows, int64_t cols, int box_rows) {
-    return cached_map_wide(map, WideKey{p, {planes, rows, cols, box_rows, -3, -4, -4, -4}}, [&](EncodeTiledFn fn) {
+    return cached_map(map, MapKey{p, {planes, rows, cols, box_rows, -3, -4, -4, -4}}, [&](EncodeTiledFn fn) {
         const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(planes)};
         const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 4, static_cast<cuuint64_t>(rows) * cols * 4};
         const cuuint32_t box[3] = {32u, static_cast<cuuint32_t>(box_rows), 1u}, estr[3] = {1u, 1u, 1u};
@@ -42,7 +42,7 @@ bool f32_map_planes(CUtensorMap* map, const void* p, int64_t planes, int64_t row
     });
 }
 bool f32_map_nhwc(CUtensorMap* map, const void* p, int64_t N, int64_t H, int64_t W, int64_t C, int box_w, int box_h, int box_n, int stride) {
-    return cached_map_wide(map, WideKey{p, {N, H * 4096 + W, C, box_w, box_h, box_n, stride, -5}}, [&](EncodeTiledFn fn) {
+    return cached_map(map, MapKey{p, {N, H * 4096 + W, C, box_w, box_h, box_n, stride, -5}}, [&](EncodeTiledFn fn) {
         const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W), static_cast<cuuint64_t>(H), static_cast<cuuint64_t>(N)};
         const cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 4, static_cast<cuuint64_t>(W) * C * 4, static_cast<cuuint64_t>(H) * W * C * 4};
         const cuuint32_t box[4] = {32u, static_cast<cuuint32_t>(box_w * stride), static_cast<cuuint32_t>(box_h * stride),

@@ -30,72 +30,36 @@ inline EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// 2-D bf16 tensor map over a row-major [rows, cols] matrix with row pitch ld (elements); boxes are
-// 64 columns (128 bytes, the swizzle span) by box_rows rows; out-of-range elements read as zero.
-inline bool make_map_2d(CUtensorMap* map, const void* p, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld) * 2};
-    const cuuint32_t box[2] = {64u, static_cast<cuuint32_t>(box_rows)};
-    const cuuint32_t estr[2] = {1u, 1u};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(p), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Encoding a tensor map costs a driver call of about a microsecond, and a training step issues the
-// same few maps over and over, so encoded maps are kept in a small direct-mapped cache keyed by
-// everything the encoding depends on (the map holds no data, only addresses and shapes).
+// Encoding a tensor map costs a driver call of one to two microseconds, and a training step issues the
+// same maps over and over, so encoded maps are kept in a small cache keyed by everything the encoding depends
+// on (the map holds no data, only addresses and shapes).  Four ways per set: a step uses some dozens of maps,
+// and with a direct-mapped cache a colliding pair was encoded anew on every call.
 struct MapKey {
     const void* p;
-    int64_t rows, cols, ld;
-    int box_rows;
-    bool operator==(const MapKey& o) const {
-        return p == o.p && rows == o.rows && cols == o.cols && ld == o.ld && box_rows == o.box_rows;
-    }
-};
-inline bool cached_map_2d(CUtensorMap* map, const void* p, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-    constexpr int kSlots = 512;
-    struct Slot { MapKey key; CUtensorMap map; bool used; };
-    static Slot slots[kSlots];
-    static std::mutex mu;
-    const MapKey key{p, rows, cols, ld, box_rows};
-    uint64_t h = reinterpret_cast<uintptr_t>(p) * 0x9E3779B97F4A7C15ull;
-    h ^= static_cast<uint64_t>(rows) * 0xC2B2AE3D27D4EB4Full + static_cast<uint64_t>(cols) * 0x165667B19E3779F9ull +
-         static_cast<uint64_t>(ld) * 31 + static_cast<uint64_t>(box_rows);
-    Slot& s = slots[(h >> 20) % kSlots];
-    std::lock_guard<std::mutex> lock(mu);
-    if (s.used && s.key == key) { *map = s.map; return true; }
-    if (!make_map_2d(map, p, rows, cols, ld, box_rows)) return false;
-    s.key = key; s.map = *map; s.used = true;
-    return true;
-}
-
-// The maps below are described by eight numbers; they share one cache.
-struct WideKey {
-    const void* p;
     int64_t v[8];
-    bool operator==(const WideKey& o) const {
-        if (p != o.p) return false;
-        for (int i = 0; i < 8; ++i)
-            if (v[i] != o.v[i]) return false;
-        return true;
+    bool operator==(const MapKey& o) const {
+        bool same = p == o.p;
+        for (int i = 0; i < 8; ++i) same = same && v[i] == o.v[i];
+        return same;
     }
 };
 template <typename Make>
-inline bool cached_map_wide(CUtensorMap* map, const WideKey& key, Make make) {
-    constexpr int kSlots = 256;
-    struct Slot { WideKey key; CUtensorMap map; bool used; };
-    static Slot slots[kSlots];
+inline bool cached_map(CUtensorMap* map, const MapKey& key, Make make) {
+    constexpr int kSets = 256, kWays = 4;
+    struct Slot { MapKey key; CUtensorMap map; bool used; };
+    struct Set { Slot way[kWays]; int next; };
+    static Set sets[kSets];
     static std::mutex mu;
     uint64_t h = reinterpret_cast<uintptr_t>(key.p) * 0x9E3779B97F4A7C15ull;
     for (int i = 0; i < 8; ++i) h = (h ^ static_cast<uint64_t>(key.v[i])) * 0xC2B2AE3D27D4EB4Full;
-    Slot& s = slots[(h >> 24) % kSlots];
+    Set& set = sets[(h >> 40) % kSets];
     std::lock_guard<std::mutex> lock(mu);
-    if (s.used && s.key == key) { *map = s.map; return true; }
+    for (Slot& s : set.way)
+        if (s.used && s.key == key) { *map = s.map; return true; }
     EncodeTiledFn fn = encode_fn();
     if (!fn || !make(fn)) return false;
+    Slot& s = set.way[set.next];
+    set.next = (set.next + 1) % kWays;
     s.key = key; s.map = *map; s.used = true;
     return true;
 }
@@ -106,13 +70,24 @@ inline bool encode_bf16(EncodeTiledFn fn, CUtensorMap* map, const void* p, int r
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 2-D bf16 tensor map over a row-major [rows, cols] matrix with row pitch ld (elements); boxes are
+// 64 columns (128 bytes, the swizzle span) by box_rows rows; out-of-range elements read as zero.
+inline bool cached_map_2d(CUtensorMap* map, const void* p, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+    return cached_map(map, MapKey{p, {rows, cols, ld, box_rows, -6, 0, 0, 0}}, [&](EncodeTiledFn fn) {
+        const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
+        const cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld) * 2};
+        const cuuint32_t box[2] = {64u, static_cast<cuuint32_t>(box_rows)}, estr[2] = {1u, 1u};
+        return encode_bf16(fn, map, p, 2, dims, strides, box, estr);
+    });
+}
+
 // 4-D bf16 tensor map over an NHWC image [N, H, W, C]: boxes are 64 channels x box_w x box_h pixels of box_n
 // images (box_w * box_h * box_n rows of 128 bytes in shared memory, pixel-major), taking every stride-th
 // pixel along W and H; coordinates may start outside the image (zero padding of the convolution),
 // out-of-range pixels, channels and images read as zero.
 inline bool cached_map_nhwc(CUtensorMap* map, const void* p, int64_t N, int64_t H, int64_t W, int64_t C, int box_w, int box_h,
                             int box_n, int stride) {
-    return cached_map_wide(map, WideKey{p, {N, H, W, C, box_w, box_h, box_n, stride}}, [&](EncodeTiledFn fn) {
+    return cached_map(map, MapKey{p, {N, H, W, C, box_w, box_h, box_n, stride}}, [&](EncodeTiledFn fn) {
         const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W), static_cast<cuuint64_t>(H),
                                     static_cast<cuuint64_t>(N)};
         const cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 2, static_cast<cuuint64_t>(W) * C * 2,
@@ -132,7 +107,7 @@ inline bool cached_map_nhwc(CUtensorMap* map, const void* p, int64_t N, int64_t 
 // image row, so that a tile may start at any row and is clipped at its own end).
 inline bool cached_map_planes(CUtensorMap* map, const void* p, int64_t planes, int64_t rows, int64_t cols, int64_t plane_step,
                               int box_rows) {
-    return cached_map_wide(map, WideKey{p, {planes, rows, cols, plane_step, box_rows, -1, -1, -1}}, [&](EncodeTiledFn fn) {
+    return cached_map(map, MapKey{p, {planes, rows, cols, plane_step, box_rows, -1, -1, -1}}, [&](EncodeTiledFn fn) {
         const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(planes)};
         const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 2, static_cast<cuuint64_t>(plane_step) * cols * 2};
         const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u};
