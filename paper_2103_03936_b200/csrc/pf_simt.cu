@@ -403,62 +403,129 @@ cudaError_t slices_to_gradients(const SliceSums* jobs, int count, cudaStream_t s
 // Backward of y = act(z + bias): dZ = dY where y > 0 (act = max(0, .)) or everywhere (identity), written
 // over dY; partial column sums of dZ per chunk of rows go to `part` [chunks, cols] (fp32), summed in chunk
 // order by the second kernel into db (deterministic).
-template <typename T>
+// Bound by memory: a lane reads kVec consecutive columns (16 bytes where pitch and pointers allow) of every eighth
+// row of the chunk, four rows in flight.
+template <typename T, int kVec>
+struct alignas(sizeof(T) * kVec) Pack {
+    T v[kVec];
+};
+template <typename T, int kVec>
 __global__ void __launch_bounds__(256) act_bwd_kernel(const T* y, int64_t ldy, T* dY, int64_t lddy, int64_t rows,
                                                       int64_t cols, int act, float* part, int rows_per_chunk) {
-    const int64_t col = static_cast<int64_t>(blockIdx.x) * 32 + (threadIdx.x & 31);
+    using P = Pack<T, kVec>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t col = (static_cast<int64_t>(blockIdx.x) * 32 + lane) * kVec;
     const int64_t r_beg = static_cast<int64_t>(blockIdx.y) * rows_per_chunk;
     const int64_t r_end = r_beg + rows_per_chunk < rows ? r_beg + rows_per_chunk : rows;
-    float sum = 0.f;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    float sum[kVec];
+#pragma unroll
+    for (int e = 0; e < kVec; ++e) sum[e] = 0.f;
     if (col < cols) {
-        for (int64_t r = r_beg + (threadIdx.x >> 5); r < r_end; r += 8) {
-            float g = static_cast<float>(dY[r * lddy + col]);
-            if (act == 1 && !(static_cast<float>(y[r * ldy + col]) > 0.f)) {
-                g = 0.f;
-                dY[r * lddy + col] = static_cast<T>(0.f);
+        auto one = [&](int64_t r, P g, const P& yv) {
+            if (act == 1) {
+                bool cut = false;
+#pragma unroll
+                for (int e = 0; e < kVec; ++e)
+                    if (!(static_cast<float>(yv.v[e]) > 0.f)) { g.v[e] = static_cast<T>(0.f); cut = true; }
+                if (cut) *reinterpret_cast<P*>(dY + r * lddy + col) = g;
             }
-            sum += g;
+#pragma unroll
+            for (int e = 0; e < kVec; ++e) sum[e] += static_cast<float>(g.v[e]);
+        };
+        int64_t r = r_beg + warp;
+        for (; r + 24 < r_end; r += 32) {
+            P g[4], yv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) g[u] = *reinterpret_cast<const P*>(dY + (r + 8 * u) * lddy + col);
+            if (act == 1)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) yv[u] = *reinterpret_cast<const P*>(y + (r + 8 * u) * ldy + col);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) one(r + 8 * u, g[u], act == 1 ? yv[u] : g[u]);
+        }
+        for (; r < r_end; r += 8) {
+            const P g = *reinterpret_cast<const P*>(dY + r * lddy + col);
+            one(r, g, act == 1 ? *reinterpret_cast<const P*>(y + r * ldy + col) : g);
         }
     }
-    __shared__ float red[8][33];
-    red[threadIdx.x >> 5][threadIdx.x & 31] = sum;
+    if (!part) return;
+    __shared__ float red[8][32 * kVec + 1];
+#pragma unroll
+    for (int e = 0; e < kVec; ++e) red[warp][lane * kVec + e] = sum[e];
     __syncthreads();
-    if (threadIdx.x < 32 && col < cols && part) {
+    for (int c = threadIdx.x; c < 32 * kVec; c += 256) {
+        const int64_t cc = static_cast<int64_t>(blockIdx.x) * 32 * kVec + c;
+        if (cc >= cols) break;
         float s = 0.f;
-        for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
-        part[static_cast<int64_t>(blockIdx.y) * cols + col] = s;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += red[w][c];
+        part[static_cast<int64_t>(blockIdx.y) * cols + cc] = s;
     }
 }
+// Eight warps per 32 columns: warp w adds chunks w, w + 8, ..., then the eight sums are added in warp order.
 template <typename T>
-__global__ void act_bwd_bias_kernel(const float* part, int chunks, int64_t cols, T* db) {
-    const int64_t col = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (col >= cols) return;
+__global__ void __launch_bounds__(256) act_bwd_bias_kernel(const float* part, int chunks, int64_t cols, T* db) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t col = static_cast<int64_t>(blockIdx.x) * 32 + lane;
     float s = 0.f;
-    for (int c = 0; c < chunks; ++c) s += part[static_cast<int64_t>(c) * cols + col];
-    db[col] = static_cast<T>(s);
+    if (col < cols)
+#pragma unroll 8
+        for (int c = warp; c < chunks; c += 8) s += part[static_cast<int64_t>(c) * cols + col];
+    __shared__ float red[8][32];
+    red[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && col < cols) {
+        for (int w = 1; w < 8; ++w) s += red[w][lane];
+        db[col] = static_cast<T>(s);
+    }
 }
 int act_bwd_chunks(int64_t rows) {
-    const int64_t c = ceil_div(rows, 256);
+    const int64_t c = ceil_div(rows, 128);
     return static_cast<int>(c < 1 ? 1 : (c > 64 ? 64 : c));
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(256); cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    if (e == cudaSuccess) count_launch();
+    return e;
+}
+template <typename T>
+static cudaError_t act_bwd_typed(const T* y, int64_t ldy, T* dY, int64_t lddy, T* db, int64_t rows, int64_t cols, int act, float* part,
+                                 cudaStream_t stream) {
+    const int chunks = act_bwd_chunks(rows);
+    const int rpc = static_cast<int>(ceil_div(rows, chunks));
+    float* pp = db ? part : nullptr;
+    // the widest access that keeps every row aligned and whole
+    constexpr int64_t kSize = sizeof(T);
+    int64_t unit = static_cast<int64_t>(reinterpret_cast<uintptr_t>(dY)) | (lddy * kSize) | (cols * kSize) | 16;
+    if (act == 1) unit |= static_cast<int64_t>(reinterpret_cast<uintptr_t>(y)) | (ldy * kSize);
+    const int vec = static_cast<int>((unit & -unit) / kSize);
+    auto grid = [&](int v) { return dim3(static_cast<unsigned>(ceil_div(cols, 32 * v)), static_cast<unsigned>(chunks)); };
+    cudaError_t e;
+    if (vec >= 8) e = launch_pdl(act_bwd_kernel<T, static_cast<int>(16 / kSize)>, grid(8), stream, y, ldy, dY, lddy, rows, cols, act, pp, rpc);
+    else if (vec >= 4) e = launch_pdl(act_bwd_kernel<T, 4>, grid(4), stream, y, ldy, dY, lddy, rows, cols, act, pp, rpc);
+    else if (vec >= 2) e = launch_pdl(act_bwd_kernel<T, 2>, grid(2), stream, y, ldy, dY, lddy, rows, cols, act, pp, rpc);
+    else e = launch_pdl(act_bwd_kernel<T, 1>, grid(1), stream, y, ldy, dY, lddy, rows, cols, act, pp, rpc);
+    if (e != cudaSuccess || !db) return e;
+    return launch_pdl(act_bwd_bias_kernel<T>, dim3(static_cast<unsigned>(ceil_div(cols, 32))), stream, part, chunks, cols, db);
 }
 cudaError_t act_bwd(const void* y, int64_t ldy, void* dY, int64_t lddy, void* db, int64_t rows, int64_t cols, int act,
                     int dtype, float* part, cudaStream_t stream) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
-    const int chunks = act_bwd_chunks(rows);
-    const int rpc = static_cast<int>(ceil_div(rows, chunks));
-    const dim3 grid(static_cast<unsigned>(ceil_div(cols, 32)), static_cast<unsigned>(chunks));
-    float* pp = db ? part : nullptr;
-    if (dtype == PF_BF16) {
-        act_bwd_kernel<<<grid, 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(y), ldy, static_cast<__nv_bfloat16*>(dY), lddy,
-                                                 rows, cols, act, pp, rpc);
-        if (db) act_bwd_bias_kernel<<<static_cast<unsigned>(ceil_div(cols, 256)), 256, 0, stream>>>(part, chunks, cols, static_cast<__nv_bfloat16*>(db));
-    } else {
-        act_bwd_kernel<<<grid, 256, 0, stream>>>(static_cast<const float*>(y), ldy, static_cast<float*>(dY), lddy, rows, cols,
-                                                 act, pp, rpc);
-        if (db) act_bwd_bias_kernel<<<static_cast<unsigned>(ceil_div(cols, 256)), 256, 0, stream>>>(part, chunks, cols, static_cast<float*>(db));
-    }
-    count_launch(db ? 2 : 1);
-    return cudaGetLastError();
+    if (dtype == PF_BF16)
+        return act_bwd_typed(static_cast<const __nv_bfloat16*>(y), ldy, static_cast<__nv_bfloat16*>(dY), lddy, static_cast<__nv_bfloat16*>(db),
+                             rows, cols, act, part, stream);
+    return act_bwd_typed(static_cast<const float*>(y), ldy, static_cast<float*>(dY), lddy, static_cast<float*>(db), rows, cols, act, part, stream);
 }
 
 // y = act(y + bias) in place (the paths that do not fuse the epilogue into the producing kernel).
