@@ -109,10 +109,9 @@ int pf_lowrank_linear_fwd(const void* x, int64_t ldx, const void* U, int64_t ldu
  * factorized layer followed by its bias (the second half of the FFN, the LSTM gate pre-activations
  * of Section 2.3).
  *   bias [n] in `dtype`, contiguous; NULL = no bias.     act: PF_ACT_NONE or PF_ACT_RELU.
- * bias and activation are applied to the fp32 result before the single rounding to `dtype` in the
- * fused kernel (m >= 2048 rows at r <= 192, PF_BF16).  On the other paths y is first stored in
- * `dtype` and a second pass adds the bias and applies the activation in place (two roundings for
- * PF_BF16; one extra launch).  T_stash is x U as in pf_lowrank_linear_fwd (bias does not enter it).
+ * bias and activation are applied to the fp32 result before the single rounding to `dtype` (PF_BF16 layouts
+ * that only the FMA kernels take: y is stored first and a second pass applies them in place, two roundings).
+ * T_stash is x U as in pf_lowrank_linear_fwd (bias does not enter it).
  * Same workspace, pitches and error behaviour as pf_lowrank_linear_fwd; an act outside the enum is
  * PF_ERR_INVALID_ARG.  The backward of the activation (dY masked by y > 0) and the bias gradient
  * (column sums of dY) are the caller's: pf_lowrank_linear_bwd takes the gradient of (x U) V^T. */

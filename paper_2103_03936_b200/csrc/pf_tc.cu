@@ -214,6 +214,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.a_mn = A.mn_major; p.b_mn = B.mn_major;
     p.C = C; p.ldc = ldc; p.partial = partial;
     p.C2 = nullptr; p.ldc2 = 0; p.c2_gstride = 0;
+    p.bias = nullptr; p.act = 0;
     p.conv_mode = 0; p.cv_blks = 1; p.cv_kw = 1; p.cv_kh = 1; p.cv_pad = 0; p.cv_stride = 1; p.cv_C = 1; p.cv_bh = 1; p.cv_nb = 1;
     p.cv_tpi = 1; p.cv_N = p.cv_H = p.cv_W = p.cv_bw = p.cv_inv_bw = p.cv_inv_bh = p.cv_tiles_class = 1; p.cv_blocks = 0;
     p.rows_tile = kBM; p.kpix = kBK; p.ksteps = kBK / 16;
@@ -292,10 +293,10 @@ int launch_prepared(const GemmLaunch& g, cudaStream_t stream) {
 // wrote it (the CTA-pair kernel cannot), else the caller copies C itself.
 int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
          int splits, float* partial, cudaStream_t stream, const ConvA* cv = nullptr, void* copy2 = nullptr,
-         int64_t ldc2 = 0, bool* copy2_done = nullptr) {
+         int64_t ldc2 = 0, bool* copy2_done = nullptr, const void* bias = nullptr, int act = 0) {
     // wide, many-tile (tensor-bound) products run on CTA pairs, which halve the operand traffic per SM
     if (!cv && splits <= 1 && pair_worthwhile(M, N, K)) {
-        const int st2 = gemm_pair_2sm(A.p, A.ld, A.mn_major, B.p, B.ld, B.mn_major, M, N, K, C, ldc, stream);
+        const int st2 = gemm_pair_2sm(A.p, A.ld, A.mn_major, B.p, B.ld, B.mn_major, M, N, K, C, ldc, stream, bias, act);
         if (st2 != PF_ERR_UNSUPPORTED) {
             if (copy2_done) *copy2_done = false;
             return st2;
@@ -310,6 +311,7 @@ int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, vo
         g.p.C2 = copy2; g.p.ldc2 = ldc2;
         if (copy2_done) *copy2_done = true;
     }
+    g.p.bias = bias; g.p.act = act;               // (given for unsplit products only)
     const GemmParams& p = g.p;
     cudaError_t e = g.bn == 64    ? launch_gemm<64>(g.ta, g.tb, p, g.grid, stream)
                     : g.bn == 128 ? launch_gemm<128>(g.ta, g.tb, p, g.grid, stream)
@@ -523,11 +525,8 @@ int linear_fwd(const LinearArgs& a, int* handled) {
                   pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream, nullptr,
                   (a.T && !stash_direct) ? a.T : nullptr, a.ldt, &stash_written);
         if (st != PF_OK) return st;
-        st = gemm({T, ldT, false}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, a.stream);
-        // unfused products: bias and activation in a pass of their own over y
-        if (st == PF_OK && (a.bias || a.act) &&
-            bias_act_inplace(a.y, a.ldy, a.m, a.n, a.bias, a.act, PF_BF16, a.stream) != cudaSuccess)
-            return PF_ERR_CUDA;
+        st = gemm({T, ldT, false}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, a.stream, nullptr, nullptr, 0, nullptr,
+                  a.bias, a.act);
     }
     if (st != PF_OK) return st;
     if (a.T && !stash_direct && !stash_written &&

@@ -72,7 +72,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
 // Plain product on CTA pairs (pf_tc_pair.cu); PF_ERR_UNSUPPORTED when the output is not 16-byte aligned
 // with a pitch that is a multiple of 8 elements.
 int gemm_pair_2sm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb, bool b_mn, int64_t M, int64_t N,
-                  int64_t K, void* C, int64_t ldc, cudaStream_t stream);
+                  int64_t K, void* C, int64_t ldc, cudaStream_t stream, const void* bias = nullptr, int act = 0);
 
 // Grouped factorized linear layer: `groups` problems of one shape (several factor pairs applied to the
 // same or to different inputs) in two launches forward and two backward, whatever the group count.

@@ -29,6 +29,8 @@ struct GemmParams {
     long long ldc;
     void* C2;                // optional second copy of the result at another pitch, groups c2_gstride elements apart
     long long ldc2, c2_gstride;
+    const void* bias;        // unsplit plain products: C = act(A B + bias), bias [N] in bf16 or null
+    int act;
     float* partial;          // splits > 1: fp32 slices, one 128 x BN block per (tile, slice)
     unsigned int* counters;  // splits > 1: two counters per tile
     unsigned int* status;
@@ -432,6 +434,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                         tmem_ld32(lane_base + c * 64, v0);
                         tmem_ld32(lane_base + c * 64 + 32, v1);
                         tmem_ld_wait();
+                        if (kMode == 0 && (p.bias || p.act)) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
 #pragma unroll
                         for (int t = 0; t < 4; ++t) {
                             uint4 o;
@@ -494,6 +497,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                     tmem_ld32(lane_base + c * 64, v0);
                     tmem_ld32(lane_base + c * 64 + 32, v1);
                     tmem_ld_wait();
+                    if (kMode == 0 && (p.bias || p.act)) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
 #pragma unroll
                     for (int w = 0; w < 16; ++w) {
                         stg[lane * 33 + w] = pack_bf16x2(__uint_as_float(v0[2 * w]), __uint_as_float(v0[2 * w + 1]));

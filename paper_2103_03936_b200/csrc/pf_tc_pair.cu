@@ -56,6 +56,8 @@ struct PairParams {
     int a_mn, b_mn;          // 1 = operand stored with the M/N index contiguous
     void* C;                 // bf16 [M, ldc], 16-byte aligned, ldc a multiple of 8
     long long ldc;
+    const void* bias;        // C = act(A B + bias), bias [N] in bf16 or null
+    int act;
     int tiles_m, tiles;      // 256-row tile rows, and all 256 x 256 tiles (tile t = (t % tiles_m, t / tiles_m))
     unsigned int* status;
 };
@@ -291,6 +293,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(acc_empty_leader0 + 8 * buf);
                 }
+                if (p.bias || p.act) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     uint4 o;
@@ -345,7 +348,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 // C[M,N] (bf16, 16-byte aligned, ldc % 8 == 0) = A * B on CTA pairs.  Returns PF_ERR_UNSUPPORTED when
 // the operands do not fit (the caller then uses the single-CTA kernel).
 int gemm_pair_2sm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb, bool b_mn, int64_t M, int64_t N,
-                  int64_t K, void* C, int64_t ldc, cudaStream_t stream) {
+                  int64_t K, void* C, int64_t ldc, cudaStream_t stream, const void* bias, int act) {
     if (M < 1 || N < 1 || K < 1 || M > 0x7fffffff || N > 0x7fffffff || K > 0x7fffffff) return PF_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(C) & 15) != 0 || ldc % 8 != 0) return PF_ERR_UNSUPPORTED;
     const int64_t tiles_m = ceil_div(M, 256), tiles_n = ceil_div(N, 256);
@@ -357,7 +360,7 @@ int gemm_pair_2sm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t 
     if (!oka || !okb) return PF_ERR_CUDA;
     PairParams p;
     p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
-    p.a_mn = a_mn; p.b_mn = b_mn; p.C = C; p.ldc = ldc; p.status = device_status_ptr();
+    p.a_mn = a_mn; p.b_mn = b_mn; p.C = C; p.ldc = ldc; p.bias = bias; p.act = act; p.status = device_status_ptr();
     p.tiles_m = static_cast<int>(tiles_m); p.tiles = static_cast<int>(tiles_m * tiles_n);
     const size_t smem = 1024 + 1024 + kPairStaging + static_cast<size_t>(kPairStages) * kPairStageBytes;
     static bool configured[64] = {};

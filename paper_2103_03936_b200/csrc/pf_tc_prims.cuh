@@ -273,6 +273,28 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// Bias and activation (1 = max(0, .)) on 64 accumulator columns col .. col + 63 of a row, before the rounding: every
+// lane fetches two of the columns' values (bf16), the columns take them from the lanes.
+__device__ __forceinline__ void bias_act64(uint32_t (&v0)[32], uint32_t (&v1)[32], const void* bias, int act, int col, int n, int lane) {
+    if (bias) {
+        const unsigned short* b = reinterpret_cast<const unsigned short*>(bias);
+        const float b0 = col + lane < n ? __uint_as_float(static_cast<uint32_t>(b[col + lane]) << 16) : 0.f;
+        const float b1 = col + 32 + lane < n ? __uint_as_float(static_cast<uint32_t>(b[col + 32 + lane]) << 16) : 0.f;
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+            v0[e] = __float_as_uint(__uint_as_float(v0[e]) + __shfl_sync(0xffffffffu, b0, e));
+            v1[e] = __float_as_uint(__uint_as_float(v1[e]) + __shfl_sync(0xffffffffu, b1, e));
+        }
+    }
+    if (act == 1) {
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+            v0[e] = __float_as_uint(fmaxf(__uint_as_float(v0[e]), 0.f));
+            v1[e] = __float_as_uint(fmaxf(__uint_as_float(v1[e]), 0.f));
+        }
+    }
+}
+
 }  // namespace tc
 }  // namespace pf
 #endif
