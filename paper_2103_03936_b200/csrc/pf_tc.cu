@@ -741,6 +741,7 @@ size_t grouped_workspace(int groups, int64_t m, int64_t k, int64_t n, int64_t r,
 
 int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     *handled = 0;
+    if (a.groups == 1) return PF_OK;      // one group is the ungrouped layer, whose kernels take 2-D maps
     if (encode_fn() == nullptr || a.groups > 1024 || a.k > (1 << 22) || a.n > (1 << 22) || a.r > (1 << 22)) return PF_OK;
     const GroupedPlan gp = grouped_plan(a.groups, a.m, a.k, a.n, a.r);
     const bool shared_x = a.sx == 0 && a.groups > 1;
@@ -777,6 +778,7 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
 
 int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     *handled = 0;
+    if (a.groups == 1) return PF_OK;      // one group is the ungrouped layer, whose kernels take 2-D maps
     if (encode_fn() == nullptr || a.groups > 1024 || a.k > (1 << 22) || a.n > (1 << 22) || a.r > (1 << 22)) return PF_OK;
     const GroupedPlan gp = grouped_plan(a.groups, a.m, a.k, a.n, a.r);
     const bool shared_x = a.sx == 0 && a.groups > 1;

@@ -119,6 +119,12 @@ def test_attention_projection_shape(shared_x):
     assert (lf, lb) == (2, 2)
 
 
+@pytest.mark.parametrize("m,k,n,r", [(300, 136, 264, 40), (130, 100, 60, 33)])
+def test_one_group_is_the_ungrouped_layer(m, k, n, r):
+    run_grouped(1, m, k, n, r, wl.BF16, 245, False)
+    run_grouped(1, m, k, n, r, wl.BF16, 246, False, stash=False, need_dX=False)
+
+
 def test_grouped_backward_is_bit_reproducible():
     G, m, k, n, r = 4, 4096, 256, 320, 64
     x_h, U_h, V_h, dY_h = make(G, m, k, n, r, wl.BF16, 240, False)
