@@ -182,7 +182,10 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.stream = stream;
     a.bias = bias; a.act = act;
     size_t need = w.total;
-    if (exact_need) {
+    const bool small_rows = dtype == PF_BF16 && small::linear_fwd_fits(m, k, n, r);
+    if (exact_need && small_rows) {
+        need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * 2;
+    } else if (exact_need) {
         bool tc_handles = false;
         size_t tc_need = dtype == PF_BF16 ? tc::linear_fwd_need(a, &tc_handles) : 0;
         if (dtype == PF_F32) {        // (taken only when it fits; the FMA kernels need less)
@@ -196,6 +199,7 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     if (st != PF_OK) return st;
     if (m == 0) return PF_OK;
 
+    if (small_rows) return small::linear_fwd(a, T_stash ? T_stash : static_cast<void*>(ws + w.off_T), T_stash ? ldt : r);
     if (dtype == PF_BF16) {
         int handled = 0;
         st = tc::linear_fwd(a, &handled);

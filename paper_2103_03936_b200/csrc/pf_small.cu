@@ -1,0 +1,323 @@
+// Layers with few rows (a time step of a recurrent layer, generation, the smallest batches): forward on any
+// layout, without re-pitch copies.
+//
+// With a few dozen rows the factors are the work: every element of U and V is read once and used m times, so the
+// layer is bound by getting them through the SMs, and in practice by latencies: a tcgen05 tile of 128 rows pays
+// its set-up, TMA round trips and slice sums (three launches, 18 us for 20 x 1500 -> 6000 at r 375) for rows
+// that do not exist.  Here the factor takes the 128-row side of nothing: warps multiply 16 x 16 blocks of it by
+// all m rows of the batch with mma.sync (m16n8k16, fp32 accumulation), which needs no descriptors, takes any
+// alignment and starts as soon as its operands are in registers.
+//   small_reduce_kernel   T[m, r] = A[m, K] B[K, r]     (A, B) = (x, U): long contraction, few outputs; a CTA owns 16
+//                         columns of r and a cluster of CTAs shares the contraction (sum through distributed
+//                         shared memory, in rank order).
+//   small_out_kernel      y[m, n] = act(T[m, r] V[n, r]^T + bias): a CTA owns 32 rows of V, which it stages BEFORE
+//                         waiting for the kernel that produces T (that kernel does not write V).
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "pf_tc.h"
+#include "pf_tc_host.h"
+
+namespace pf {
+namespace small {
+namespace {
+
+constexpr int kThreads = 512;
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pair(unsigned short lo, unsigned short hi) { return lo | (static_cast<uint32_t>(hi) << 16); }
+
+struct ReduceParams {
+    const unsigned short *A, *B;     // bf16
+    unsigned short* C;
+    long long lda, ldb, ldc;
+    int m, K, r;
+    int k_per_rank;                  // multiple of 16
+};
+
+// kTiles: blocks of 8 batch rows.  kPairs: rows of A are 4-byte aligned and K is even.
+template <int kTiles, bool kPairs>
+__global__ void __launch_bounds__(kThreads) small_reduce_kernel(const ReduceParams p) {
+    constexpr int kWarps = kThreads / 32;
+    __shared__ float part[kWarps][16][kTiles * 8 + 1];
+    __shared__ float sums[16][kTiles * 8 + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int r0 = blockIdx.x * 16;
+    const int k_beg = blockIdx.y * p.k_per_rank, k_end = min(p.K, k_beg + p.k_per_rank);
+    const int k_pair = p.K - 2;
+    pdl_wait();
+    pdl_launch_dependents();
+    float acc[kTiles][4];
+#pragma unroll
+    for (int j = 0; j < kTiles; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+    // loads are unconditional (addresses clamped, values masked afterwards)
+    const unsigned short* bcol0 = p.B + min(r0 + g, p.r - 1);
+    const unsigned short* bcol1 = p.B + min(r0 + g + 8, p.r - 1);
+    const unsigned short* xrow[kTiles];
+#pragma unroll
+    for (int j = 0; j < kTiles; ++j) xrow[j] = p.A + static_cast<long long>(min(j * 8 + g, p.m - 1)) * p.lda;
+#pragma unroll 1
+    for (int k0 = k_beg + warp * 16; k0 < k_end; k0 += kWarps * 16) {
+        uint32_t a[4], b[kTiles][2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = k0 + 2 * t + 8 * h;
+            const int ka = min(k, k_end - 1), kb = min(k + 1, k_end - 1);
+            // a0: (r g, k 2t, 2t+1), a1: (r g + 8, same k), a2 / a3: k + 8
+            const unsigned short u0 = bcol0[ka * p.ldb], u1 = bcol0[kb * p.ldb], v0 = bcol1[ka * p.ldb], v1 = bcol1[kb * p.ldb];
+#pragma unroll
+            for (int j = 0; j < kTiles; ++j) {
+                if constexpr (kPairs) b[j][h] = *reinterpret_cast<const uint32_t*>(xrow[j] + min(k, k_pair));
+                else b[j][h] = pair(xrow[j][ka], xrow[j][kb]);
+            }
+            a[2 * h] = pair(u0, u1);
+            a[2 * h + 1] = pair(v0, v1);
+            // contraction past the end: zero on both sides (0 * Inf would not be zero)
+            const uint32_t keep = (k < k_end ? 0xffffu : 0u) | (k + 1 < k_end ? 0xffff0000u : 0u);
+            a[2 * h] &= keep;
+            a[2 * h + 1] &= keep;
+#pragma unroll
+            for (int j = 0; j < kTiles; ++j) b[j][h] &= keep;
+        }
+#pragma unroll
+        for (int j = 0; j < kTiles; ++j) mma16816(acc[j], a, b[j][0], b[j][1]);
+    }
+    // c0, c1: (r g, rows 2t, 2t + 1); c2, c3: r g + 8
+#pragma unroll
+    for (int j = 0; j < kTiles; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part[warp][g + 8 * (e >> 1)][j * 8 + 2 * t + (e & 1)] = acc[j][e];
+    __syncthreads();
+    constexpr int kOut = 16 * kTiles * 8;
+    for (int i = threadIdx.x; i < kOut; i += kThreads) {
+        const int c = i & 15, row = i >> 4;
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) s += part[w][c][row];
+        sums[c][row] = s;
+    }
+    const int ranks = gridDim.y;
+    if (ranks > 1) {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    } else {
+        __syncthreads();
+    }
+    // each rank stores a share of the outputs: the sums of all ranks, added in rank order
+    const int rank = blockIdx.y;
+    for (int i = rank * kThreads + threadIdx.x; i < kOut; i += ranks * kThreads) {
+        const int c = i & 15, row = i >> 4;
+        float s = 0.f;
+        if (ranks > 1) {
+            const uint32_t local = static_cast<uint32_t>(__cvta_generic_to_shared(&sums[c][row]));
+            for (int q = 0; q < ranks; ++q) {
+                uint32_t addr;
+                float v;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(local), "r"(q));
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+                s += v;
+            }
+        } else {
+            s = sums[c][row];
+        }
+        if (row < p.m && r0 + c < p.r) p.C[row * p.ldc + r0 + c] = __bfloat16_as_ushort(__float2bfloat16_rn(s));
+    }
+    if (ranks > 1) {        // nobody leaves while its sums may still be read
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    }
+}
+
+// Copies `rows` rows of `cols` bf16 (any element alignment and pitch) into shared memory rows of `pitch` bytes (a
+// multiple of 16), zero-filled to whole 16-byte pieces up to `pieces` per row.  Both sides move 16 bytes: a piece is
+// assembled from the two aligned source vectors that cover it (each holds at least one of its bytes).
+// Four pieces per thread at a time, loads before uses; one copy of the code for both operands (these kernels run for
+// two or three microseconds, of which cold instructions are a part).
+__device__ __noinline__ void stage_rows(uint8_t* dst, uint32_t pitch, int pieces, const unsigned short* src, long long ld, int rows, int cols) {
+    constexpr int kBatch = 4;
+    const int total = rows * pieces;
+    for (int base = threadIdx.x; base < total; base += kBatch * kThreads) {
+        uint4 lo[kBatch], hi[kBatch];
+        uint32_t at[kBatch], sh[kBatch];
+        int left_[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int i = min(base + u * kThreads, total - 1);          // (a clamped piece is written twice, alike)
+            const int row = i / pieces, pc = i - row * pieces, left = cols - pc * 8;
+            const unsigned short* sp = src + row * ld + pc * 8;
+            at[u] = static_cast<uint32_t>(row) * pitch + static_cast<uint32_t>(pc) * 16u;
+            sh[u] = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(sp)) & 15u;
+            lo[u] = hi[u] = make_uint4(0, 0, 0, 0);
+            // aligned vectors that hold at least one byte of the piece (of what the row has of it)
+            const uint4* v = reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(sp) - sh[u]);
+            left_[u] = min(left, 8);
+            if (left > 0) lo[u] = v[0];
+            if (left > 0 && static_cast<int>(sh[u]) + 2 * left_[u] > 16) hi[u] = v[1];
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const uint32_t q = sh[u] >> 2, bit = (sh[u] & 3u) * 8u;
+            const uint4 o = lo[u], h = hi[u];
+            const bool q1 = q & 1, q2 = q & 2;
+            // words q .. q + 4 of the window lo:hi
+            const uint32_t x0 = q2 ? o.z : o.x, x1 = q2 ? o.w : o.y, x2 = q2 ? h.x : o.z, x3 = q2 ? h.y : o.w, x4 = q2 ? h.z : h.x, x5 = q2 ? h.w : h.y;
+            const uint32_t w0 = q1 ? x1 : x0, w1 = q1 ? x2 : x1, w2 = q1 ? x3 : x2, w3 = q1 ? x4 : x3, w4 = q1 ? x5 : x4;
+            uint4 r = make_uint4(__funnelshift_r(w0, w1, bit), __funnelshift_r(w1, w2, bit), __funnelshift_r(w2, w3, bit), __funnelshift_r(w3, w4, bit));
+            if (left_[u] < 8) {            // zeros behind the row's end
+                auto keep = [&](int e) { return (e < left_[u] ? 0xffffu : 0u) | (e + 1 < left_[u] ? 0xffff0000u : 0u); };
+                r.x &= keep(0); r.y &= keep(2); r.z &= keep(4); r.w &= keep(6);
+            }
+            *reinterpret_cast<uint4*>(dst + at[u]) = r;
+        }
+    }
+}
+
+struct OutParams {
+    const unsigned short *T, *V, *bias;
+    unsigned short* y;
+    long long ldt, ldv, ldy;
+    int m, n, r, act;
+    int steps;                       // 16-element steps of the contraction
+    uint32_t pitch;                  // bytes of a staged row: 16 modulo 128, so that fragment loads do not conflict
+};
+
+// Sixteen warps: two blocks of 16 rows of V times eight parts of the contraction.
+template <int kTiles>
+__global__ void __launch_bounds__(kThreads) small_out_kernel(const OutParams p) {
+    extern __shared__ uint4 smem4[];
+    uint8_t* sV = reinterpret_cast<uint8_t*>(smem4);
+    uint8_t* sT = sV + 32 * p.pitch;
+    __shared__ float part[8][32][kTiles * 8 + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int n0 = blockIdx.x * 32, rows = min(32, p.n - n0);
+    stage_rows(sV, p.pitch, p.steps * 2, p.V + n0 * p.ldv, p.ldv, rows, p.r);
+    for (int i = threadIdx.x; i < (32 - rows) * p.steps * 2; i += kThreads)
+        *reinterpret_cast<uint4*>(sV + (rows + i / (p.steps * 2)) * p.pitch + (i % (p.steps * 2)) * 16) = make_uint4(0, 0, 0, 0);
+    pdl_wait();
+    pdl_launch_dependents();
+    stage_rows(sT, p.pitch, p.steps * 2, p.T, p.ldt, p.m, p.r);
+    for (int i = threadIdx.x; i < (kTiles * 8 - p.m) * p.steps * 2; i += kThreads)
+        *reinterpret_cast<uint4*>(sT + (p.m + i / (p.steps * 2)) * p.pitch + (i % (p.steps * 2)) * 16) = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    const int block = warp & 1, part_k = warp >> 1;
+    float acc[kTiles][4];
+#pragma unroll
+    for (int j = 0; j < kTiles; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+    const uint8_t* va = sV + (block * 16 + g) * p.pitch + t * 4;
+    const uint8_t* tb = sT + g * p.pitch + t * 4;
+#pragma unroll 1
+    for (int s = part_k; s < p.steps; s += 8) {
+        uint32_t a[4];
+        a[0] = *reinterpret_cast<const uint32_t*>(va + s * 32);
+        a[1] = *reinterpret_cast<const uint32_t*>(va + 8 * p.pitch + s * 32);
+        a[2] = *reinterpret_cast<const uint32_t*>(va + s * 32 + 16);
+        a[3] = *reinterpret_cast<const uint32_t*>(va + 8 * p.pitch + s * 32 + 16);
+#pragma unroll
+        for (int j = 0; j < kTiles; ++j) {
+            const uint8_t* tj = tb + j * 8 * p.pitch + s * 32;
+            mma16816(acc[j], a, *reinterpret_cast<const uint32_t*>(tj), *reinterpret_cast<const uint32_t*>(tj + 16));
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kTiles; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part[part_k][block * 16 + g + 8 * (e >> 1)][j * 8 + 2 * t + (e & 1)] = acc[j][e];
+    __syncthreads();
+    const int c = lane;
+    const bool in = n0 + c < p.n;
+    const float b = p.bias && in ? __uint_as_float(static_cast<uint32_t>(p.bias[n0 + c]) << 16) : 0.f;
+    for (int row = warp; row < p.m; row += kThreads / 32) {
+        float v = part[0][c][row];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) v += part[q][c][row];
+        v += b;
+        if (p.act == PF_ACT_RELU) v = fmaxf(v, 0.f);
+        if (in) p.y[row * p.ldy + n0 + c] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+    }
+}
+
+cudaError_t launch_reduce(void (*kernel)(const ReduceParams), dim3 grid, cudaStream_t stream, const ReduceParams& p) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = grid.y; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
+    if (e == cudaSuccess) count_launch();
+    return e;
+}
+
+// Blocks of 8 batch rows that the kernels are compiled for.
+int tiles_of(int64_t m) {
+    const int t = static_cast<int>(ceil_div(m, 8));
+    return t;
+}
+size_t out_smem(int64_t m, int64_t r) {
+    const size_t row = static_cast<size_t>(ceil_div(r, 16)) * 32;
+    return (32 + static_cast<size_t>(tiles_of(m)) * 8) * ((row + 111) / 128 * 128 + 16);
+}
+
+template <int kTiles>
+int forward(const tc::LinearArgs& a, void* T, int64_t ldt) {
+    ReduceParams q;
+    q.A = static_cast<const unsigned short*>(a.x); q.B = static_cast<const unsigned short*>(a.U); q.C = static_cast<unsigned short*>(T);
+    q.lda = a.ldx; q.ldb = a.ldu; q.ldc = ldt;
+    q.m = static_cast<int>(a.m); q.K = static_cast<int>(a.k); q.r = static_cast<int>(a.r);
+    const bool pairs = (reinterpret_cast<uintptr_t>(a.x) & 3) == 0 && a.ldx % 2 == 0 && a.k % 2 == 0;
+    // as many ranks as keep at least one 16-element step per warp, while the grid fits the machine
+    const int64_t blocks = ceil_div(a.r, 16);
+    int ranks = 1;
+    while (ranks < 8 && blocks * ranks * 2 <= num_sms() && a.k > 16 * (kThreads / 32) * ranks) ranks *= 2;
+    q.k_per_rank = static_cast<int>(ceil_div(ceil_div(a.k, ranks), 16) * 16);
+    if (launch_reduce(pairs ? small_reduce_kernel<kTiles, true> : small_reduce_kernel<kTiles, false>, dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(ranks)), a.stream, q) != cudaSuccess) return PF_ERR_CUDA;
+    OutParams o;
+    o.T = static_cast<const unsigned short*>(T); o.V = static_cast<const unsigned short*>(a.V); o.bias = static_cast<const unsigned short*>(a.bias);
+    o.y = static_cast<unsigned short*>(a.y);
+    o.ldt = ldt; o.ldv = a.ldv; o.ldy = a.ldy;
+    o.m = q.m; o.n = static_cast<int>(a.n); o.r = q.r; o.act = a.act;
+    o.steps = static_cast<int>(ceil_div(a.r, 16));
+    o.pitch = static_cast<uint32_t>((o.steps * 32 + 111) / 128 * 128 + 16);
+    const size_t smem = out_smem(a.m, a.r);
+    if (tc::allow_smem(small_out_kernel<kTiles>, 190 * 1024) != cudaSuccess ||
+        tc::launch_overlapped(small_out_kernel<kTiles>, dim3(static_cast<unsigned>(ceil_div(a.n, 32))), dim3(kThreads), smem, a.stream, o) != cudaSuccess)
+        return PF_ERR_CUDA;
+    count_launch();
+    return PF_OK;
+}
+}  // namespace
+
+bool linear_fwd_fits(int64_t m, int64_t k, int64_t n, int64_t r) {
+    // beyond about 2^26 multiplications the 128-row tiles win (4096 x 4096, r 256: 11.2 against 13.0 us at 20 rows, 15.0
+    // against 13.1 at 32), beyond 2^27 where they need re-pitch copies; up to 8 rows never
+    const int64_t most = (k % 8 || r % 8) ? 1LL << 27 : 1LL << 26;
+    return m >= 1 && m <= 32 && k <= (1 << 24) && n <= (1 << 24) && r <= (1 << 16) && out_smem(m, r) <= 190 * 1024 &&
+           (m <= 8 || m * (k + n) * r < most);
+}
+
+// T [m, r]: the stash or scratch.
+int linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt) {
+    switch (tiles_of(a.m)) {
+        case 1: return forward<1>(a, T, ldt);
+        case 2: return forward<2>(a, T, ldt);
+        case 3: return forward<3>(a, T, ldt);
+        default: return forward<4>(a, T, ldt);
+    }
+}
+
+}  // namespace small
+}  // namespace pf

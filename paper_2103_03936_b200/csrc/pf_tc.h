@@ -113,5 +113,11 @@ int conv_fwd(const ConvArgs& a, int* handled);
 int conv_bwd(const ConvArgs& a, int* handled);
 
 }  // namespace tc
+
+// Few rows (pf_small.cu), bf16, any layout.
+namespace small {
+bool linear_fwd_fits(int64_t m, int64_t k, int64_t n, int64_t r);
+int linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt);
+}  // namespace small
 }  // namespace pf
 #endif

@@ -260,3 +260,28 @@ def test_fp32_products_on_tensor_cores(m, k, n, r):
     errs = run_case(c)
     assert max(errs.values()) <= 1e-5, errs
     run_case(wl.LinearCase("f32tc", m, k, n, r, wl.F32, 24), stash=False, need_dX=False)
+
+
+@pytest.mark.parametrize("m,k,n,r", [(1, 1, 1, 1), (1, 17, 33, 15), (8, 256, 64, 16), (9, 300, 100, 17), (16, 1000, 31, 40), (20, 1500, 600, 375),
+                                     (25, 2049, 65, 33), (32, 513, 257, 129), (32, 64, 96, 1000)])
+def test_few_rows_forward(m, k, n, r):
+    """Up to 32 rows: the kernels without re-pitch copies; edges of the 8-row, 16-column and 32-row blocks, contractions
+    shared by clusters, odd pitches, bias and activation."""
+    c = wl.LinearCase("few", m, k, n, r, wl.BF16, 27)
+    for pad in (0, 3):
+        d = c.generate()
+        def up(a, cols):
+            buf = torch.zeros((a.shape[0], cols + pad), dtype=torch.bfloat16, device="cuda")
+            buf[:, :cols] = dev(a, c.dtype)
+            return buf[:, :cols]
+        gy, gT = Guarded((m, n), c.dtype, ld=n + pad), Guarded((m, r), c.dtype, ld=r + pad)
+        b = wl.round_to(wl.normal(28, 7, (n,), 0.5), c.dtype)
+        pf.pf_lowrank_linear_fwd_act(up(d["x"], k), up(d["U"], r), up(d["V"], r), bias=dev(b, c.dtype), act=pf.PF_ACT_RELU, y=gy.t, T_stash=gT.t)
+        torch.cuda.synchronize()
+        y_ref, T_ref = oracle.linear_fwd_act(d["x"], d["U"], d["V"], b, relu=True)
+        assert_close(gT.t, T_ref, c.dtype, "few rows T")
+        if np.linalg.norm(y_ref) > 0:
+            assert_close(gy.t, y_ref, c.dtype, "few rows y")
+        gy.check()
+        gT.check()
+    assert pf.pf_last_device_status() == 0
