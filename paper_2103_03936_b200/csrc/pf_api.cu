@@ -182,9 +182,9 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.stream = stream;
     a.bias = bias; a.act = act;
     size_t need = w.total;
-    const bool small_rows = dtype == PF_BF16 && small::linear_fwd_fits(m, k, n, r);
-    if (exact_need && small_rows) {
-        need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * 2;
+    const bool is_small = dtype == PF_BF16 ? small::linear_fwd_fits(m, k, n, r) : small::f32_fits(m, k, n, r, false);
+    if (exact_need && is_small) {
+        need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * dtype_size(dtype);
     } else if (exact_need) {
         bool tc_handles = false;
         size_t tc_need = dtype == PF_BF16 ? tc::linear_fwd_need(a, &tc_handles) : 0;
@@ -199,7 +199,11 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     if (st != PF_OK) return st;
     if (m == 0) return PF_OK;
 
-    if (small_rows) return small::linear_fwd(a, T_stash ? T_stash : static_cast<void*>(ws + w.off_T), T_stash ? ldt : r);
+    if (is_small) {
+        void* Ts = T_stash ? T_stash : static_cast<void*>(ws + w.off_T);
+        const int64_t ldTs = T_stash ? ldt : r;
+        return dtype == PF_BF16 ? small::linear_fwd(a, Ts, ldTs) : small::f32_linear_fwd(a, Ts, ldTs);
+    }
     if (dtype == PF_BF16) {
         int handled = 0;
         st = tc::linear_fwd(a, &handled);
@@ -348,8 +352,8 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
             dV = ws + w.off_gtmp + align_up(static_cast<size_t>(k) * r * s, 256); lddv = r;
             a.dU = dU; a.lddu = lddu; a.dV = dV; a.lddv = lddv;
         }
-        int handled = 0;
-        st = tc::f32_linear_bwd(a, &handled);
+        int handled = small::f32_fits(m, k, n, r, true) ? 1 : 0;
+        st = handled ? small::f32_linear_bwd(a) : tc::f32_linear_bwd(a, &handled);
         if (st != PF_OK) return st;
         if (handled) {
             if (indirect) {

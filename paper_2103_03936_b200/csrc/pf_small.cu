@@ -319,5 +319,132 @@ int linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt) {
     }
 }
 
+// ------------------------------------------------------------------------------ fp32, small products
+// The smallest fp32 layers (a few million multiplications per product) are all latency: the split-operand tensor-core
+// kernel needs 6 us a launch for them (set-up, ring fill, splitting, drains).  Here a CTA computes a 16 x 32 tile of
+// C with plain FMAs: all loads of 128 elements of the contraction are in flight at once, the next 128 while these
+// are multiplied.  64 x 256 -> 256 at r 32, forward + backward: 25.8 -> 17.1 us.
+namespace {
+
+constexpr int kF32Chunk = 128;
+struct F32Product {
+    const float *A, *B, *bias;
+    float* C;
+    long long a_row, a_l, b_l, b_col, ldc;      // A(i, l) = A[i a_row + l a_l], B(l, j) = B[l b_l + j b_col]
+    int M, N, K, act, tiles_x;
+};
+struct F32Pair {
+    F32Product p[2];
+    int end0;
+};
+
+__global__ void __launch_bounds__(256) small_f32_kernel(const F32Pair both) {
+    __shared__ float sA[16][kF32Chunk + 4];
+    __shared__ float sB[kF32Chunk][34];
+    const bool first = static_cast<int>(blockIdx.x) < both.end0;
+    const F32Product& p = both.p[first ? 0 : 1];
+    const int idx = blockIdx.x - (first ? 0 : both.end0);
+    const int i0 = (idx % p.tiles_x) * 16, j0 = (idx / p.tiles_x) * 32, tid = threadIdx.x;
+    pdl_wait();
+    pdl_launch_dependents();
+    // consecutive threads read consecutive addresses: along the contraction, or along the rows / columns
+    const bool al = p.a_l == 1, bl = p.b_l == 1;
+    const int ai = al ? tid >> 7 : tid & 15, ak = al ? tid & 127 : tid >> 4;
+    const int bj = bl ? tid >> 7 : tid & 31, bk = bl ? tid & 127 : tid >> 5;
+    const int ai_step = al ? 2 : 0, ak_step = al ? 0 : 16, bj_step = bl ? 2 : 0, bk_step = bl ? 0 : 8;
+    float ra[8], rb[16];
+    auto load = [&](int l0) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int i = i0 + ai + q * ai_step, l = l0 + ak + q * ak_step;
+            ra[q] = i < p.M && l < p.K ? __ldg(p.A + i * p.a_row + l * p.a_l) : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const int j = j0 + bj + q * bj_step, l = l0 + bk + q * bk_step;
+            rb[q] = j < p.N && l < p.K ? __ldg(p.B + l * p.b_l + j * p.b_col) : 0.f;
+        }
+    };
+    const int ti = tid >> 4, tj = (tid & 15) * 2;
+    float c0 = 0.f, c1 = 0.f;
+    load(0);
+    for (int l0 = 0; l0 < p.K; l0 += kF32Chunk) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sA[ai + q * ai_step][ak + q * ak_step] = ra[q];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) sB[bk + q * bk_step][bj + q * bj_step] = rb[q];
+        __syncthreads();
+        if (l0 + kF32Chunk < p.K) load(l0 + kF32Chunk);
+        const int left = min(kF32Chunk, p.K - l0);
+#pragma unroll 4
+        for (int l = 0; l < left; l += 4) {           // (zeros behind the end)
+            const float4 a = *reinterpret_cast<const float4*>(&sA[ti][l]);
+            const float2 b0 = *reinterpret_cast<const float2*>(&sB[l][tj]), b1 = *reinterpret_cast<const float2*>(&sB[l + 1][tj]);
+            const float2 b2 = *reinterpret_cast<const float2*>(&sB[l + 2][tj]), b3 = *reinterpret_cast<const float2*>(&sB[l + 3][tj]);
+            c0 = fmaf(a.x, b0.x, c0); c1 = fmaf(a.x, b0.y, c1);
+            c0 = fmaf(a.y, b1.x, c0); c1 = fmaf(a.y, b1.y, c1);
+            c0 = fmaf(a.z, b2.x, c0); c1 = fmaf(a.z, b2.y, c1);
+            c0 = fmaf(a.w, b3.x, c0); c1 = fmaf(a.w, b3.y, c1);
+        }
+        __syncthreads();
+    }
+    const int i = i0 + ti, j = j0 + tj;
+    if (i >= p.M) return;
+    if (p.bias) {
+        if (j < p.N) c0 += __ldg(p.bias + j);
+        if (j + 1 < p.N) c1 += __ldg(p.bias + j + 1);
+    }
+    if (p.act == PF_ACT_RELU) { c0 = fmaxf(c0, 0.f); c1 = fmaxf(c1, 0.f); }
+    float* dst = p.C + i * p.ldc + j;
+    if (j < p.N) dst[0] = c0;
+    if (j + 1 < p.N) dst[1] = c1;
+}
+
+F32Product f32_product(const void* A, int64_t a_row, int64_t a_l, const void* B, int64_t b_l, int64_t b_col, void* C, int64_t ldc, int64_t M,
+                       int64_t N, int64_t K) {
+    F32Product p = {};
+    p.A = static_cast<const float*>(A); p.B = static_cast<const float*>(B); p.C = static_cast<float*>(C);
+    p.a_row = a_row; p.a_l = a_l; p.b_l = b_l; p.b_col = b_col; p.ldc = ldc;
+    p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
+    p.tiles_x = static_cast<int>(ceil_div(M, 16));
+    return p;
+}
+int f32_run(const F32Product& a, const F32Product* b, cudaStream_t stream) {
+    F32Pair both{{a, b ? *b : a}, static_cast<int>(a.tiles_x * ceil_div(a.N, 32))};
+    const unsigned blocks = static_cast<unsigned>(both.end0 + (b ? b->tiles_x * ceil_div(b->N, 32) : 0));
+    if (tc::launch_overlapped(small_f32_kernel, dim3(blocks), dim3(256), 0, stream, both) != cudaSuccess) return PF_ERR_CUDA;
+    count_launch();
+    return PF_OK;
+}
+}  // namespace
+
+// Every product short (its contraction in two loads) and small.  Beyond, the tensor cores are as fast or faster
+// (128 x 512 -> 512, r 64: 13.7 + 15.2 against 13.4 + 15.4 us; 512 x 512 -> 512, r 32: 14.0 against 16.4).
+bool f32_fits(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd) {
+    const int64_t longest = std::max({k, r, bwd ? std::max(n, m) : int64_t{1}});
+    return longest <= 256 && n <= 4096 && m <= 4096 && m * r * std::max(k, n) <= (1 << 21);
+}
+int f32_linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt) {
+    const int st = f32_run(f32_product(a.x, a.ldx, 1, a.U, a.ldu, 1, T, ldt, a.m, a.r, a.k), nullptr, a.stream);
+    if (st != PF_OK) return st;
+    F32Product y = f32_product(T, ldt, 1, a.V, 1, a.ldv, a.y, a.ldy, a.m, a.n, a.r);
+    y.bias = static_cast<const float*>(a.bias);
+    y.act = a.act;
+    return f32_run(y, nullptr, a.stream);
+}
+// T: the stash, or ws_T to have it recomputed there.
+int f32_linear_bwd(const tc::LinearArgs& a) {
+    const void* T = a.T ? a.T : a.ws_T;
+    const int64_t ldt = a.T ? a.ldt : a.r;
+    int st = PF_OK;
+    if (!a.T) st = f32_run(f32_product(a.x, a.ldx, 1, a.U, a.ldu, 1, a.ws_T, a.r, a.m, a.r, a.k), nullptr, a.stream);
+    if (st != PF_OK) return st;
+    const F32Product dv = f32_product(a.dY, 1, a.lddy, T, ldt, 1, a.dV, a.lddv, a.n, a.r, a.m);
+    st = f32_run(f32_product(a.dY, a.lddy, 1, a.V, a.ldv, 1, a.ws_G, a.r, a.m, a.r, a.n), &dv, a.stream);
+    if (st != PF_OK) return st;
+    const F32Product dx = f32_product(a.ws_G, a.r, 1, a.U, 1, a.ldu, a.dX, a.lddx, a.m, a.k, a.r);
+    return f32_run(f32_product(a.x, 1, a.ldx, a.ws_G, a.r, 1, a.dU, a.lddu, a.k, a.r, a.m), a.dX ? &dx : nullptr, a.stream);
+}
+
 }  // namespace small
 }  // namespace pf

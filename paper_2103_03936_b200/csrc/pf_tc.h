@@ -114,10 +114,14 @@ int conv_bwd(const ConvArgs& a, int* handled);
 
 }  // namespace tc
 
-// Few rows (pf_small.cu), bf16, any layout.
+// Few rows, bf16, any layout (pf_small.cu).
 namespace small {
 bool linear_fwd_fits(int64_t m, int64_t k, int64_t n, int64_t r);
 int linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt);
+// fp32, small products, any layout.
+bool f32_fits(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd);
+int f32_linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt);
+int f32_linear_bwd(const tc::LinearArgs& a);
 }  // namespace small
 }  // namespace pf
 #endif
