@@ -40,21 +40,6 @@ struct Grouping {
     bool sum_groups = false;
 };
 
-// 3-D bf16 tensor map over `groups` row-major [rows, cols] matrices gs elements apart (boxes of 64 columns x
-// box_rows rows of one group; out-of-range elements read as zero).  Cached like the 2-D maps.
-bool cached_map_3d(CUtensorMap* map, const void* p, int64_t groups, int64_t rows, int64_t cols, int64_t ld, int64_t gs,
-                   int box_rows) {
-    if (groups < 1) return false;
-    if (groups == 1) gs = rows * ld;                       // a single group: any valid stride
-    if ((gs * 2) % 16 != 0 || gs * 2 >= (1LL << 40)) return false;
-    return cached_map(map, MapKey{p, {groups, rows, cols, ld, gs, box_rows, -7, 0}}, [&](EncodeTiledFn fn) {
-        const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(groups)};
-        const cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * 2, static_cast<cuuint64_t>(gs) * 2};
-        const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u}, estr[3] = {1u, 1u, 1u};
-        return encode_bf16(fn, map, p, 3, dims, strides, box, estr);
-    });
-}
-
 size_t gemm_smem(int bn, int stages) {
     return 1024 + 1024 + static_cast<size_t>(stages) * (kBM * kBK * 2 + bn * kBK * 2);
 }
@@ -296,7 +281,10 @@ int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, vo
          int64_t ldc2 = 0, bool* copy2_done = nullptr, const void* bias = nullptr, int act = 0) {
     // wide, many-tile (tensor-bound) products run on CTA pairs, which halve the operand traffic per SM
     if (!cv && splits <= 1 && pair_worthwhile(M, N, K)) {
-        const int st2 = gemm_pair_2sm(A.p, A.ld, A.mn_major, B.p, B.ld, B.mn_major, M, N, K, C, ldc, stream, bias, act);
+        PairJob j{A.p, A.ld, A.mn_major, 0, B.p, B.ld, B.mn_major, 0, M, N, K, C, ldc};
+        j.bias = bias;
+        j.act = act;
+        const int st2 = gemm_pairs(&j, 1, 1, stream);
         if (st2 != PF_ERR_UNSUPPORTED) {
             if (copy2_done) *copy2_done = false;
             return st2;
@@ -602,6 +590,20 @@ int linear_bwd(const LinearArgs& a, int* handled) {
         st = chain(dY.p, dY.ld, a.m, a.n, V.p, V.ld, a.r, U.p, U.ld, a.k, a.dX, a.lddx, G, ldG, a.stream, nullptr,
                    dv_beside ? 1 : 0);
         if (st != PF_OK) return st;
+    } else if (!a.du_slices && pair_worthwhile(a.m, a.r, a.n) && pair_worthwhile(a.n, a.r, a.m) && pair_worthwhile(a.k, a.r, a.m) &&
+               (!a.dX || pair_worthwhile(a.m, a.k, a.r))) {
+        // Large ranks, tensor-bound: two launches of CTA pairs, G beside dV and dU beside dX, so that the tiles of the
+        // second product fill the pairs that the few long tiles of the first leave free (16384 x 4096 -> 4096 at
+        // r 1024: each product alone left 14 % of the pairs idle).  Calls that want the slices go product by product.
+        const PairJob jg{dY.p, dY.ld, false, 0, V.p, V.ld, true, 0, a.m, a.r, a.n, G, ldG};
+        const PairJob jv{dY.p, dY.ld, true, 0, T.p, T.ld, true, 0, a.n, a.r, a.m, a.dV, a.lddv};
+        const PairJob ju{x.p, x.ld, true, 0, G, ldG, true, 0, a.k, a.r, a.m, a.dU, a.lddu};
+        const PairJob jx{G, ldG, false, 0, U.p, U.ld, false, 0, a.m, a.k, a.r, a.dX, a.lddx};
+        const PairJob first[2] = {a.m >= a.n ? jv : jg, a.m >= a.n ? jg : jv};
+        const PairJob second[2] = {a.m >= a.r || !a.dX ? ju : jx, a.m >= a.r ? jx : ju};
+        st = gemm_pairs(first, 2, 1, a.stream);
+        if (st != PF_OK) return st;
+        return gemm_pairs(second, a.dX ? 2 : 1, 1, a.stream);
     } else {
         // Few rows: G = dY V is a contraction split across blocks, and dV = dY^T T, which needs nothing
         // of it, shares its launch (the second block slot of every SM); dU and dX follow in a second one.
@@ -709,6 +711,60 @@ GroupedPlan grouped_plan(int groups, int64_t m, int64_t k, int64_t n, int64_t r)
 }
 bool grouped_ok(const void* p, int64_t ld, int64_t gs) { return tma_ok(p, ld) && gs % 8 == 0; }
 
+// Expected microseconds of one launch of prepared products on single CTAs, and of the same products on CTA pairs:
+// a single CTA's 128 x 128 tile takes 0.31 us per k-block alone on its SM and 0.55 us beside another (its SM's load
+// path is what it waits for), a pair's 256 x 256 tile 0.28 us (the tensor cores); 3 - 4.5 us of start-up and
+// epilogue, of which a persistent pair overlaps all but the first and last; an output pitch that TMA and 16-byte
+// stores cannot take makes a pair's epilogue 3 us.
+double single_us(const GemmLaunch* const* g, int count) {
+    double ctas = 0, load = 0, longest = 0;
+    bool split = false;
+    for (int i = 0; i < count; ++i) {
+        const double n = static_cast<double>(g[i]->grid.x) * g[i]->grid.y * g[i]->grid.z, kb = g[i]->p.kb_per_split;
+        ctas += n;
+        load += n * (0.55 * kb + 4.5);
+        longest = std::max(longest, kb);
+        split = split || g[i]->p.splits > 1;
+    }
+    if (ctas <= num_sms()) return 0.31 * longest + 3.0 + (split ? 6.5 : 0.0);
+    return std::max(load / (2.0 * num_sms()), 0.55 * longest + 4.5);
+}
+double pairs_us(const PairJob* j, int count) {
+    double load = 0, longest = 0;
+    for (int i = 0; i < count; ++i) {
+        const double tiles = static_cast<double>(ceil_div(j[i].M, 256) * ceil_div(j[i].N, 256)) * (j[i].sum_groups ? 1 : j[i].groups);
+        const double kb = static_cast<double>(ceil_div(j[i].K, 64)) * (j[i].sum_groups ? j[i].groups : 1);
+        const bool vec = j[i].ldc % 8 == 0 && j[i].c_gs % 8 == 0 && (reinterpret_cast<uintptr_t>(j[i].C) & 15) == 0;
+        const double us = std::max(0.28 * kb, vec ? 1.3 : 3.0);
+        load += tiles * us;
+        longest = std::max(longest, us);
+    }
+    const int pairs = num_sms() / 2;
+    double total = load / pairs;
+    if (count == 1) total = longest * static_cast<double>(ceil_div(static_cast<int64_t>(load / longest + 0.5), pairs));
+    return std::max(total, longest) + 4.0;
+}
+// One launch of one or two products, on whichever form is expected to be faster.  The products are independent of
+// each other; jobs[i] describes the same product as *g[i].
+int launch_faster(const GemmLaunch* const* g, const PairJob* jobs, int count, cudaStream_t stream) {
+    if (pairs_us(jobs, count) < 0.9 * single_us(g, count)) {
+        PairJob order[2] = {jobs[0], jobs[count > 1 ? 1 : 0]};
+        auto kb = [](const PairJob& j) { return ceil_div(j.K, 64) * (j.sum_groups ? j.groups : 1); };
+        if (count > 1 && kb(order[1]) > kb(order[0])) std::swap(order[0], order[1]);     // long tiles first
+        const int st = gemm_pairs(order, count, 1, stream);
+        if (st != PF_ERR_UNSUPPORTED) return st;
+    }
+    const GemmLaunch* list[2] = {g[0], g[count > 1 ? 1 : 0]};
+    if (count > 1 && list[0]->p.splits <= 1 && list[1]->p.splits > 1) std::swap(list[0], list[1]);   // split products first
+    int st = count > 1 ? gemm_multi(list, count, stream) : PF_ERR_UNSUPPORTED;
+    for (int i = 0; st == PF_ERR_UNSUPPORTED && i < count; ++i) {
+        const int one = launch_prepared(*g[i], stream);
+        if (one != PF_OK) return one;
+        if (i + 1 == count) return PF_OK;
+    }
+    return st;
+}
+
 // A grouped operand that TMA must read: as it is, or (ragged widths) all its groups copied to `scratch` at a
 // padded pitch.  A shared operand is one matrix.
 struct StagedGroups {
@@ -773,7 +829,9 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     st = repacks.flush(a.stream);
     if (st == PF_OK) st = launch_prepared(g1, a.stream);
     if (st != PF_OK) return st;
-    return launch_prepared(g2, a.stream);
+    PairJob jy{T, ldT, false, sT, V.p, V.ld, false, V.gs, a.m, a.n, a.r, a.y, a.ldy, a.sy, a.groups};
+    const GemmLaunch* const ly[1] = {&g2};
+    return launch_faster(ly, &jy, 1, a.stream);
 }
 
 int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
@@ -818,18 +876,15 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
         if (st != PF_OK) return st;
     }
     // launch A: G = dY V and dV = dY^T T (independent of each other); launch B: dU = x^T G and dX = G U^T
-    auto pair = [&](const GemmLaunch& p0, const GemmLaunch& q0, bool has_q) {
-        const GemmLaunch* list[2] = {&p0, &q0};
-        if (has_q && p0.p.splits <= 1 && q0.p.splits > 1) { list[0] = &q0; list[1] = &p0; }   // split products first
-        int r2 = gemm_multi(list, has_q ? 2 : 1, a.stream);
-        if (r2 != PF_ERR_UNSUPPORTED) return r2;
-        r2 = launch_prepared(p0, a.stream);
-        if (r2 == PF_OK && has_q) r2 = launch_prepared(q0, a.stream);
-        return r2;
-    };
-    st = pair(gG, gV, true);
+    const PairJob ja[2] = {{dY.p, dY.ld, false, dY.gs, V.p, V.ld, true, V.gs, a.m, a.r, a.n, Gbuf, ldW, sW, a.groups},
+                           {dY.p, dY.ld, true, dY.gs, T.p, T.ld, true, T.gs, a.n, a.r, a.m, a.dV, a.lddv, a.sdv, a.groups}};
+    const PairJob jb[2] = {{x.p, x.ld, true, x.gs, Gbuf, ldW, true, sW, a.k, a.r, a.m, a.dU, a.lddu, a.sdu, a.groups},
+                           {Gbuf, ldW, false, sW, U.p, U.ld, false, U.gs, a.m, a.k, a.r, a.dX, a.lddx, shared_x ? 0 : a.sdx, a.groups, shared_x}};
+    const GemmLaunch* const la[2] = {&gG, &gV};
+    const GemmLaunch* const lb[2] = {&gU, &gX};
+    st = launch_faster(la, ja, 2, a.stream);
     if (st != PF_OK) return st;
-    return pair(gU, gX, a.dX != nullptr);
+    return launch_faster(lb, jb, a.dX ? 2 : 1, a.stream);
 }
 
 // After a bounded wait has expired some CTAs may have left their tile counters non-zero.

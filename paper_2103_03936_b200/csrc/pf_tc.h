@@ -69,10 +69,27 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
           cudaStream_t stream, const ChainConv* conv = nullptr, int max_split = 0, const void* bias = nullptr,
           int act = 0);   // bias [N2] (bf16) and act (0 identity, 1 max(0, .)) apply to `out`
 
-// Plain product on CTA pairs (pf_tc_pair.cu); PF_ERR_UNSUPPORTED when the output is not 16-byte aligned
-// with a pitch that is a multiple of 8 elements.
-int gemm_pair_2sm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb, bool b_mn, int64_t M, int64_t N,
-                  int64_t K, void* C, int64_t ldc, cudaStream_t stream, const void* bias = nullptr, int act = 0);
+// Products on CTA pairs (pf_tc_pair.cu): C[M,N] = act(A * B + bias) for `groups` problems of one shape, matrices *_gs
+// elements apart (0 = one operand shared by all groups); sum_groups: the groups are summed into one C.
+struct PairJob {
+    const void* A;
+    int64_t lda;
+    bool a_mn;
+    int64_t a_gs;
+    const void* B;
+    int64_t ldb;
+    bool b_mn;
+    int64_t b_gs;
+    int64_t M, N, K;
+    void* C;
+    int64_t ldc;
+    int64_t c_gs = 0;
+    int groups = 1;
+    bool sum_groups = false;
+    const void* bias = nullptr;
+    int act = 0;
+};
+int gemm_pairs(const PairJob* jobs, int count, int first, cudaStream_t stream);
 
 // Grouped factorized linear layer: `groups` problems of one shape (several factor pairs applied to the
 // same or to different inputs) in two launches forward and two backward, whatever the group count.

@@ -81,6 +81,21 @@ inline bool cached_map_2d(CUtensorMap* map, const void* p, int64_t rows, int64_t
     });
 }
 
+// 3-D bf16 tensor map over `groups` row-major [rows, cols] matrices gs elements apart (boxes of 64 columns x
+// box_rows rows of one group; out-of-range elements read as zero).  Cached like the 2-D maps.
+inline bool cached_map_3d(CUtensorMap* map, const void* p, int64_t groups, int64_t rows, int64_t cols, int64_t ld, int64_t gs,
+                   int box_rows) {
+    if (groups < 1) return false;
+    if (groups == 1) gs = rows * ld;                       // a single group: any valid stride
+    if ((gs * 2) % 16 != 0 || gs * 2 >= (1LL << 40)) return false;
+    return cached_map(map, MapKey{p, {groups, rows, cols, ld, gs, box_rows, -7, 0}}, [&](EncodeTiledFn fn) {
+        const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(groups)};
+        const cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * 2, static_cast<cuuint64_t>(gs) * 2};
+        const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u}, estr[3] = {1u, 1u, 1u};
+        return encode_bf16(fn, map, p, 3, dims, strides, box, estr);
+    });
+}
+
 // 4-D bf16 tensor map over an NHWC image [N, H, W, C]: boxes are 64 channels x box_w x box_h pixels of box_n
 // images (box_w * box_h * box_n rows of 128 bytes in shared memory, pixel-major), taking every stride-th
 // pixel along W and H; coordinates may start outside the image (zero padding of the convolution),

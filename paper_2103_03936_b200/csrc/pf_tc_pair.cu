@@ -51,15 +51,62 @@ struct PairCtl {
     uint32_t abort;
 };
 
-struct PairParams {
-    int M, N, K;
+// One product of a launch.  Grouped products: operands are 3-D maps whose outermost coordinate is the group (a
+// shared operand has one), group g's output starts g * c_gstride elements after C; kb_per_group > 0 instead makes
+// the groups part of the contraction (one output).
+struct PairProduct {
+    int M, N, nkb;
     int a_mn, b_mn;          // 1 = operand stored with the M/N index contiguous
-    void* C;                 // bf16 [M, ldc], 16-byte aligned, ldc a multiple of 8
-    long long ldc;
+    int a_shared, b_shared, kb_per_group;
+    int tiles_m, tiles_mn, tiles;       // 256-row tile rows; tiles of one group; all tiles
+    void* C;                 // bf16 [M, ldc]
+    long long ldc, c_gstride;
     const void* bias;        // C = act(A B + bias), bias [N] in bf16 or null
     int act;
-    int tiles_m, tiles;      // 256-row tile rows, and all 256 x 256 tiles (tile t = (t % tiles_m, t / tiles_m))
+};
+// Up to three products.  Their tiles form two lists, the long ones first: list 0 (products 0 .. first - 1) is dealt
+// to the pairs in turn; list 1 (the rest) is dealt so that the pairs which got one tile of list 0 less start `delay`
+// rounds earlier, i.e. all pairs finish together.
+struct PairLaunch {
+    CUtensorMap ta[3], tb[3];
+    PairProduct p[3];
+    int count, first, total0, total1, early, delay;
     unsigned int* status;
+};
+
+// The tiles of one pair, in order; every role of a CTA walks the same sequence.
+struct PairWalk {
+    int i, pair, pairs;
+    bool second;
+    __device__ __forceinline__ PairWalk(int pair_, int pairs_) : i(0), pair(pair_), pairs(pairs_), second(false) {}
+    // product and its tile; false at the end
+    template <bool kOne>
+    __device__ __forceinline__ bool next(const PairLaunch& L, int& q, int& t) {
+        if constexpr (kOne) {
+            t = pair + i * pairs;
+            q = 0;
+            ++i;
+            return t < L.total0;
+        }
+        if (!second) {
+            t = pair + i * pairs;
+            if (t < L.total0) {
+                ++i;
+                q = 0;
+                if (L.first > 1 && t >= L.p[0].tiles) { t -= L.p[0].tiles; q = 1; }
+                return true;
+            }
+            second = true;
+            i = pairs - 1 - pair < L.early ? 0 : L.delay;
+        }
+        const int e = pairs - 1 - pair;
+        t = i < L.delay ? i * L.early + e : L.delay * L.early + (i - L.delay) * pairs + e;
+        if (t >= L.total1) return false;
+        ++i;
+        q = L.first;
+        if (q + 1 < L.count && t >= L.p[q].tiles) { t -= L.p[q].tiles; ++q; }
+        return true;
+    }
 };
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -128,6 +175,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(cluster_bar), "r"(c0), "r"(c1)
         : "memory");
 }
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int c0, int c1, int c2) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst), "l"(map), "r"(cluster_bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+}
 // D[tmem of both CTAs] (+)= A * B over the CTA pair.
 __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                                  uint32_t accumulate) {
@@ -145,9 +198,12 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
         : "memory");
 }
 
+// kForm 0: one ungrouped product with 16-byte aligned output rows (its parameters stay at fixed places and its
+// epilogue, which paces short contractions, has one form); 1: several; 2: grouped products.
+template <int kForm>
 __global__ void __launch_bounds__(kPairThreads, 1)
-tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const PairParams p) {
+tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
+    constexpr bool kGrouped = kForm == 2;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
@@ -159,7 +215,6 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int pair = static_cast<int>(blockIdx.x) >> 1, npairs = static_cast<int>(gridDim.x) >> 1;
-    const int nkb = (p.K + 63) / 64;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kPairStages; ++s) {
@@ -173,8 +228,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         ctl->abort = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
+        tma_prefetch_desc(&L.ta[0]);
+        tma_prefetch_desc(&L.tb[0]);
     }
     if (warp == 1) tmem_alloc_pair(smem_u32(&ctl->tmem_base), 2 * kPairCols);
     tc_fence_before();
@@ -190,34 +245,56 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             // ------------------------------------------------------------ producers (A: warp 0, B: warp 10)
             const bool do_a = warp == 0;
             const uint32_t full_leader0 = map_to_cta(smem_u32(&ctl->full[0]), 0);
-            uint32_t s = 0, ph = 0;
+            const uint32_t empty0 = smem_u32(&ctl->empty[0]), full0 = smem_u32(&ctl->full[0]);
+            const uint32_t dst0 = smem_u32(tiles) + (do_a ? 0u : kHalfBytes);
+            uint32_t s = 0, ph = 1, dst = dst0;
             bool ok = true;
-            for (int t = pair; t < p.tiles && ok; t += npairs) {
+            PairWalk walk(pair, npairs);
+            int q, t;
+            while (ok && walk.next<kForm == 0>(L, q, t)) {
+                const PairProduct& p = kForm == 0 ? L.p[0] : L.p[q];
+                const CUtensorMap* map = kForm == 0 ? (do_a ? &L.ta[0] : &L.tb[0]) : (do_a ? &L.ta[q] : &L.tb[q]);
+                const int nkb = p.nkb;
+                int g = 0;
+                if constexpr (kGrouped) {
+                    g = t / p.tiles_mn;
+                    t -= g * p.tiles_mn;
+                }
                 const int tn = t / p.tiles_m, tm = t - tn * p.tiles_m;
-                const int m0 = tm * 256 + static_cast<int>(rank) * 128;      // this CTA's rows of A
-                const int nb0 = tn * 256 + static_cast<int>(rank) * 128;     // this CTA's part of B
+                // this CTA's rows of A, or its part of the columns of B
+                const int mn0 = (do_a ? tm : tn) * 256 + static_cast<int>(rank) * 128;
+                const bool mn = do_a ? p.a_mn : p.b_mn;
+                int k0 = 0, left = 0x7fffffff, gc = g;
+                if constexpr (kGrouped) {
+                    if (p.kb_per_group > 0) { left = p.kb_per_group; gc = 0; }
+                }
+                const bool shared = do_a ? p.a_shared : p.b_shared;
                 for (int i = 0; i < nkb; ++i) {
-                    ok = mbar_wait(smem_u32(&ctl->empty[s]), ph ^ 1u, abort_flag, p.status);
+                    ok = mbar_wait(empty0 + 8 * s, ph, abort_flag, L.status);
                     if (!ok) break;
-                    if (rank == 0) mbar_expect_tx(smem_u32(&ctl->full[s]), 2 * kHalfBytes);   // both CTAs' tiles of this operand
+                    if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * kHalfBytes);   // both CTAs' tiles of this operand
                     const uint32_t bar = full_leader0 + 8 * s;
-                    const uint32_t a_dst = smem_u32(tiles + s * kPairStageBytes);
-                    const uint32_t b_dst = a_dst + kHalfBytes;
-                    const int k0 = i * 64;
-                    if (do_a) {
-                        if (p.a_mn) {
-                            tma_load_2d_pair(a_dst, &tmA, bar, m0, k0);
-                            tma_load_2d_pair(a_dst + 8192, &tmA, bar, m0 + 64, k0);
+                    if constexpr (kGrouped) {
+                        const int gg = shared ? 0 : gc;
+                        if (mn) {
+                            tma_load_3d_pair(dst, map, bar, mn0, k0, gg);
+                            tma_load_3d_pair(dst + 8192, map, bar, mn0 + 64, k0, gg);
                         } else {
-                            tma_load_2d_pair(a_dst, &tmA, bar, k0, m0);
+                            tma_load_3d_pair(dst, map, bar, k0, mn0, gg);
                         }
-                    } else if (p.b_mn) {
-                        tma_load_2d_pair(b_dst, &tmB, bar, nb0, k0);
-                        tma_load_2d_pair(b_dst + 8192, &tmB, bar, nb0 + 64, k0);
+                        k0 += 64;
+                        if (--left == 0) { ++gc; k0 = 0; left = p.kb_per_group; }
                     } else {
-                        tma_load_2d_pair(b_dst, &tmB, bar, k0, nb0);
+                        if (mn) {
+                            tma_load_2d_pair(dst, map, bar, mn0, k0);
+                            tma_load_2d_pair(dst + 8192, map, bar, mn0 + 64, k0);
+                        } else {
+                            tma_load_2d_pair(dst, map, bar, k0, mn0);
+                        }
+                        k0 += 64;
                     }
-                    if (++s == kPairStages) { s = 0; ph ^= 1u; }
+                    dst += kPairStageBytes;
+                    if (++s == kPairStages) { s = 0; dst = dst0; ph ^= 1u; }
                 }
             }
         }
@@ -228,35 +305,42 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             // both CTAs must have been given the same tensor-memory columns
             if (ld_cluster_u32(map_to_cta(smem_u32(&ctl->tmem_base), 1)) != tmem_base) {
                 *abort_flag = 1u;
-                if (p.status) atomicExch(p.status, kStatusTimeout);
+                if (L.status) atomicExch(L.status, kStatusTimeout);
                 ok = false;
             }
-            const uint32_t idesc = make_idesc_bf16(256, 256, p.a_mn, p.b_mn);
-            const uint32_t a_step = p.a_mn ? 128u : 2u, b_step = p.b_mn ? 128u : 2u;   // in 16-byte units
-            uint32_t s = 0, ph = 0;
+            const uint32_t tiles0 = smem_u32(tiles);
+            const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+            uint32_t s = 0, ph = 0, off = 0;
             uint32_t j = 0;
-            for (int t = pair; t < p.tiles && ok; t += npairs, ++j) {
+            PairWalk walk(pair, npairs);
+            int q, t;
+            while (ok && walk.next<kForm == 0>(L, q, t)) {
+                const PairProduct& p = kForm == 0 ? L.p[0] : L.p[q];
+                const int nkb = p.nkb;
+                const uint32_t idesc = make_idesc_bf16(256, 256, p.a_mn, p.b_mn);
+                const uint32_t a_step = p.a_mn ? 128u : 2u, b_step = p.b_mn ? 128u : 2u;   // in 16-byte units
+                const uint64_t a_desc0 = p.a_mn ? make_smem_desc(tiles0, 8192, 1024) : make_smem_desc(tiles0, 16, 1024);
+                const uint64_t b_desc0 = p.b_mn ? make_smem_desc(tiles0 + kHalfBytes, 8192, 1024) : make_smem_desc(tiles0 + kHalfBytes, 16, 1024);
                 const uint32_t buf = j & 1u;
-                ok = mbar_wait_cluster(smem_u32(&ctl->acc_empty[buf]), ((j >> 1) & 1u) ^ 1u, abort_flag, p.status);
+                ok = mbar_wait_cluster(smem_u32(&ctl->acc_empty[buf]), ((j >> 1) & 1u) ^ 1u, abort_flag, L.status);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * kPairCols;
                 for (int i = 0; i < nkb; ++i) {
-                    ok = mbar_wait(smem_u32(&ctl->full[s]), ph, abort_flag, p.status);
+                    ok = mbar_wait(full0 + 8 * s, ph, abort_flag, L.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t a_addr = smem_u32(tiles + s * kPairStageBytes);
-                    const uint32_t b_addr = a_addr + kHalfBytes;
-                    const uint64_t a_desc = p.a_mn ? make_smem_desc(a_addr, 8192, 1024) : make_smem_desc(a_addr, 16, 1024);
-                    const uint64_t b_desc = p.b_mn ? make_smem_desc(b_addr, 8192, 1024) : make_smem_desc(b_addr, 16, 1024);
+                    const uint64_t a_desc = a_desc0 + off, b_desc = b_desc0 + off;
                     tc_mma_bf16_pair(d_tmem, a_desc, b_desc, idesc, i > 0 ? 1u : 0u);
                     tc_mma_bf16_pair(d_tmem, a_desc + a_step, b_desc + b_step, idesc, 1u);
                     tc_mma_bf16_pair(d_tmem, a_desc + 2 * a_step, b_desc + 2 * b_step, idesc, 1u);
                     tc_mma_bf16_pair(d_tmem, a_desc + 3 * a_step, b_desc + 3 * b_step, idesc, 1u);
-                    tc_commit_pair(smem_u32(&ctl->empty[s]));
-                    if (++s == kPairStages) { s = 0; ph ^= 1u; }
+                    tc_commit_pair(empty0 + 8 * s);
+                    off += kPairStageBytes >> 4;
+                    if (++s == kPairStages) { s = 0; off = 0; ph ^= 1u; }
                 }
                 if (ok) tc_commit_pair(smem_u32(&ctl->acc_full[buf]));
+                ++j;
             }
         }
     } else if (warp < 10) {
@@ -266,20 +350,29 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const int q = warp & 3;
         const int c_beg = ((warp - 2) >> 2) * 2;
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-        __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C);
         // 32 rows x 64 columns staged per warp (128 bytes per row, 16-byte pieces XOR-swizzled by
         // the row), then four whole 128-byte row segments per store instruction
         const uint32_t panel = smem_u32(staging) + static_cast<uint32_t>(warp - 2) * 4096u;
         const uint32_t own = panel + static_cast<uint32_t>(lane) * 128u, sw = static_cast<uint32_t>(lane & 7);
         const int sub = lane >> 3, piece = lane & 7;
-        const size_t row_step = static_cast<size_t>(4) * p.ldc;
         const uint32_t acc_empty_leader0 = map_to_cta(smem_u32(&ctl->acc_empty[0]), 0);
-        uint32_t j = 0;
-        for (int t = pair; t < p.tiles; t += npairs, ++j) {
+        PairWalk walk(pair, npairs);
+        int pq, t;
+        for (uint32_t j = 0; walk.next<kForm == 0>(L, pq, t); ++j) {
+            const PairProduct& p = kForm == 0 ? L.p[0] : L.p[pq];
             const uint32_t buf = j & 1u;
+            __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C);
+            if constexpr (kGrouped) {
+                const int g = t / p.tiles_mn;
+                t -= g * p.tiles_mn;
+                Cb += static_cast<long long>(g) * p.c_gstride;
+            }
             const int tn = t / p.tiles_m, tm = t - tn * p.tiles_m;
             const int m0 = tm * 256 + static_cast<int>(rank) * 128, n0 = tn * 256;
-            if (!mbar_wait_warp(smem_u32(&ctl->acc_full[buf]), (j >> 1) & 1u, abort_flag, p.status)) break;
+            const size_t row_step = static_cast<size_t>(4) * p.ldc;
+            const bool vec = (p.ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0;
+            const bool even = (p.ldc % 2) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 3) == 0;
+            if (!mbar_wait_warp(smem_u32(&ctl->acc_full[buf]), (j >> 1) & 1u, abort_flag, L.status)) break;
             tc_fence_after();
 #pragma unroll 1
             for (int c = c_beg; c < c_beg + 2; ++c) {
@@ -309,6 +402,29 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     st_shared_v4(own + ((static_cast<uint32_t>(4 + u) ^ sw) << 4), o);
                 }
                 __syncwarp();
+                if (kForm != 0 && !vec) {
+                    // other pitches and alignments: a lane takes one pair of columns of each row
+                    const int col = n0 + c * 64 + 2 * lane, rows = min(32, p.M - m0 - q * 32);
+                    const bool in0 = col < p.N, in1 = col + 1 < p.N;
+                    unsigned short* d = reinterpret_cast<unsigned short*>(Cb) + static_cast<long long>(m0 + q * 32) * p.ldc + col;
+#pragma unroll 8
+                    for (int r = 0; r < 32; ++r) {
+                        const uint32_t w = ld_shared_u32(panel + static_cast<uint32_t>(r) * 128u +
+                                                         ((static_cast<uint32_t>(lane >> 2) ^ static_cast<uint32_t>(r & 7)) << 4) +
+                                                         static_cast<uint32_t>(lane & 3) * 4u);
+                        if (r < rows) {
+                            if (even && in1) {
+                                *reinterpret_cast<uint32_t*>(d) = w;
+                            } else {
+                                if (in0) d[0] = static_cast<unsigned short>(w & 0xffffu);
+                                if (in1) d[1] = static_cast<unsigned short>(w >> 16);
+                            }
+                        }
+                        d += p.ldc;
+                    }
+                    __syncwarp();
+                    continue;
+                }
                 const int col = n0 + c * 64 + piece * 8;
                 const int rin0 = q * 32 + sub;
                 __nv_bfloat16* dst = Cb + static_cast<size_t>(m0 + rin0) * p.ldc + col;
@@ -345,33 +461,53 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
 }  // namespace
 
-// C[M,N] (bf16, 16-byte aligned, ldc % 8 == 0) = A * B on CTA pairs.  Returns PF_ERR_UNSUPPORTED when
-// the operands do not fit (the caller then uses the single-CTA kernel).
-int gemm_pair_2sm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb, bool b_mn, int64_t M, int64_t N,
-                  int64_t K, void* C, int64_t ldc, cudaStream_t stream, const void* bias, int act) {
-    if (M < 1 || N < 1 || K < 1 || M > 0x7fffffff || N > 0x7fffffff || K > 0x7fffffff) return PF_ERR_UNSUPPORTED;
-    if ((reinterpret_cast<uintptr_t>(C) & 15) != 0 || ldc % 8 != 0) return PF_ERR_UNSUPPORTED;
-    const int64_t tiles_m = ceil_div(M, 256), tiles_n = ceil_div(N, 256);
-    if (tiles_m * tiles_n > 0x7fffffff) return PF_ERR_UNSUPPORTED;
-    const int64_t pairs = std::min<int64_t>(tiles_m * tiles_n, num_sms() / 2);   // persistent: one CTA per SM
-    CUtensorMap ta, tb;
-    const bool oka = a_mn ? cached_map_2d(&ta, A, K, M, lda, 64) : cached_map_2d(&ta, A, M, K, lda, 128);
-    const bool okb = b_mn ? cached_map_2d(&tb, B, K, N, ldb, 64) : cached_map_2d(&tb, B, N, K, ldb, 128);
-    if (!oka || !okb) return PF_ERR_CUDA;
-    PairParams p;
-    p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
-    p.a_mn = a_mn; p.b_mn = b_mn; p.C = C; p.ldc = ldc; p.bias = bias; p.act = act; p.status = device_status_ptr();
-    p.tiles_m = static_cast<int>(tiles_m); p.tiles = static_cast<int>(tiles_m * tiles_n);
-    const size_t smem = 1024 + 1024 + kPairStaging + static_cast<size_t>(kPairStages) * kPairStageBytes;
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {
-        if (cudaFuncSetAttribute(tc_gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
-            cudaSuccess)
-            return PF_ERR_CUDA;
-        configured[dev] = true;
+// Launches up to three products together; jobs[0 .. first - 1] are dealt first (the longer tiles, of one cost).
+// PF_ERR_UNSUPPORTED: the sizes do not fit (the caller then uses the single-CTA kernels).
+int gemm_pairs(const PairJob* jobs, int count, int first, cudaStream_t stream) {
+    if (count < 1 || count > 3 || first < 1 || first > count) return PF_ERR_UNSUPPORTED;
+    PairLaunch L;
+    bool grouped = false;
+    for (int i = 0; i < count; ++i) grouped = grouped || jobs[i].groups > 1;
+    int64_t totals[2] = {0, 0};
+    for (int i = 0; i < 3; ++i) {
+        const PairJob& j = jobs[i < count ? i : 0];
+        if (j.M < 1 || j.N < 1 || j.K < 1 || j.M > 0x7fffffff || j.N > 0x7fffffff || j.K > 0x7fffffff) return PF_ERR_UNSUPPORTED;
+        PairProduct& p = L.p[i];
+        const int64_t tiles_m = ceil_div(j.M, 256), tiles_mn = tiles_m * ceil_div(j.N, 256), tiles = j.sum_groups ? tiles_mn : tiles_mn * j.groups;
+        if (tiles > (1 << 24)) return PF_ERR_UNSUPPORTED;
+        p.M = static_cast<int>(j.M); p.N = static_cast<int>(j.N);
+        p.nkb = static_cast<int>(ceil_div(j.K, 64));
+        p.kb_per_group = j.sum_groups ? p.nkb : 0;
+        if (j.sum_groups) p.nkb *= j.groups;
+        p.a_mn = j.a_mn; p.b_mn = j.b_mn;
+        p.a_shared = j.groups > 1 && j.a_gs == 0; p.b_shared = j.groups > 1 && j.b_gs == 0;
+        p.tiles_m = static_cast<int>(tiles_m); p.tiles_mn = static_cast<int>(tiles_mn); p.tiles = static_cast<int>(tiles);
+        p.C = j.C; p.ldc = j.ldc; p.c_gstride = j.c_gs;
+        p.bias = j.bias; p.act = j.act;
+        if (i < count) totals[i < first ? 0 : 1] += tiles;
+        bool ok;
+        if (grouped) {
+            const int ga = p.a_shared ? 1 : j.groups, gb = p.b_shared ? 1 : j.groups;
+            ok = (j.a_mn ? cached_map_3d(&L.ta[i], j.A, ga, j.K, j.M, j.lda, j.a_gs, 64) : cached_map_3d(&L.ta[i], j.A, ga, j.M, j.K, j.lda, j.a_gs, 128)) &&
+                 (j.b_mn ? cached_map_3d(&L.tb[i], j.B, gb, j.K, j.N, j.ldb, j.b_gs, 64) : cached_map_3d(&L.tb[i], j.B, gb, j.N, j.K, j.ldb, j.b_gs, 128));
+        } else {
+            ok = (j.a_mn ? cached_map_2d(&L.ta[i], j.A, j.K, j.M, j.lda, 64) : cached_map_2d(&L.ta[i], j.A, j.M, j.K, j.lda, 128)) &&
+                 (j.b_mn ? cached_map_2d(&L.tb[i], j.B, j.K, j.N, j.ldb, 64) : cached_map_2d(&L.tb[i], j.B, j.N, j.K, j.ldb, 128));
+        }
+        if (!ok) return PF_ERR_CUDA;
     }
+    const int64_t pairs = std::min<int64_t>(totals[0] + totals[1], num_sms() / 2);   // persistent: one CTA per SM
+    L.count = count; L.first = first;
+    L.total0 = static_cast<int>(totals[0]); L.total1 = static_cast<int>(totals[1]);
+    const int64_t extra = totals[0] % pairs;         // pairs with one tile of list 0 more
+    L.early = static_cast<int>(pairs - extra);
+    L.delay = extra == 0 || first == count ? 0 : static_cast<int>((L.p[0].nkb + L.p[first].nkb / 2) / L.p[first].nkb);
+    L.status = device_status_ptr();
+    const bool aligned = (reinterpret_cast<uintptr_t>(jobs[0].C) & 15) == 0 && jobs[0].ldc % 8 == 0;
+    if (count == 1 && !grouped && !aligned) return PF_ERR_UNSUPPORTED;
+    auto* kernel = grouped ? tc_gemm_pair_kernel<2> : count > 1 ? tc_gemm_pair_kernel<1> : tc_gemm_pair_kernel<0>;
+    const size_t smem = 1024 + 1024 + kPairStaging + static_cast<size_t>(kPairStages) * kPairStageBytes;
+    if (allow_smem(kernel, smem) != cudaSuccess) return PF_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(pairs * 2), 1, 1);
     cfg.blockDim = dim3(kPairThreads);
@@ -383,7 +519,7 @@ int gemm_pair_2sm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t 
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, tc_gemm_pair_kernel, ta, tb, p) != cudaSuccess) return PF_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, kernel, L) != cudaSuccess) return PF_ERR_CUDA;
     count_launch();
     return PF_OK;
 }
