@@ -931,7 +931,8 @@ int conv_fwd(const ConvArgs& a, int* handled) {
         (a.T && !aligned16(a.T)))
         return PF_OK;
     const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
-    const int st = chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, a.y, a.O, a.T, a.R, a.stream, &cv);
+    int st = conv_res_fwd(a);
+    if (st == PF_ERR_UNSUPPORTED) st = chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, a.y, a.O, a.T, a.R, a.stream, &cv);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     *handled = 1;
     return st;

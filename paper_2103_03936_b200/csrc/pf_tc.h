@@ -126,6 +126,8 @@ int f32_conv_fwd(const ConvArgs& a, int* handled);
 int f32_conv_bwd(const ConvArgs& a, int* handled);
 // Device counters for one product whose contraction is split (null on error).
 unsigned int* split_counters();
+// 3 x 3, stride-1 convolutions on resident image windows (pf_tc_conv_res.cu); PF_ERR_UNSUPPORTED outside their envelope.
+int conv_res_fwd(const ConvArgs& a);
 int conv_fwd(const ConvArgs& a, int* handled);
 int conv_bwd(const ConvArgs& a, int* handled);
 

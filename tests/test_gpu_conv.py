@@ -243,3 +243,10 @@ def test_fp32_tensor_core_tilings(N, H, W, C, R, O, k, stride, pad):
     errs = run_conv(wl.ConvCase("f32tc", N, H, W, C, R, O, wl.F32, 93, kh=k, kw=k, stride=stride, pad=pad))
     assert max(errs.values()) <= 1e-5, errs
     run_conv(wl.ConvCase("f32tc", N, H, W, C, R, O, wl.F32, 94, kh=k, kw=k, stride=stride, pad=pad), stash=False, need_dX=False)
+
+
+@pytest.mark.parametrize("N,H,W,C,R,O", [(170, 15, 17, 64, 16, 72), (600, 7, 9, 72, 24, 40), (3000, 4, 4, 64, 64, 136), (12, 56, 56, 128, 40, 64), (1300, 6, 5, 64, 64, 256)])
+def test_resident_image_windows(N, H, W, C, R, O):
+    """Many tiles of a 3 x 3, stride-1 convolution: the flat image sequence (a zero column and row between images) whose
+    windows serve all taps; tiles across image borders, boxes of rows and of whole images, ragged channel blocks."""
+    run_conv(wl.ConvCase("res", N, H, W, C, R, O, wl.BF16, 95))
