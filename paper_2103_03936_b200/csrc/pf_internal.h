@@ -94,7 +94,7 @@ cudaError_t round_out_f32(const float* acc, void* dst, int64_t ld_dst, int64_t r
 cudaError_t grad_combine(void* out, int64_t ld_out, int out_dtype, const void* src, int64_t ld_src, int src_dtype,
                          int64_t rows, int64_t cols, bool accumulate, cudaStream_t stream);
 // out = (accumulate ? out : 0) + the sum, in slice order, of the fp32 slices a split tensor-core reduction
-// left at `partial` ([tile][slice][128][bn], see pf_simt.cu); one launch for up to two matrices.
+// left at `partial` (layout: see pf_simt.cu); one launch for up to two matrices.
 struct SliceSums {
     const float* partial;
     void* out;          // fp32 (out_f32) or bf16 matrix, pitch ld in its own elements

@@ -335,8 +335,8 @@ cudaError_t grad_combine(void* out, int64_t ld_out, int out_dtype, const void* s
 
 // The fp32 slices a split tensor-core reduction left in the workspace, summed once more in slice order
 // (the very sums the reduction rounded to bf16) and written unrounded to an fp32 matrix and / or added to
-// the old contents.  Slice layout: [tile][slice][128 rows][bn floats], tile = column tile * tiles_x + row
-// tile, the 16-byte pieces of a row XOR-permuted by the row index.
+// the old contents.  Slice layout: [tile][slice][32-row quadrant][4-column group][row][4 floats], tile = column
+// tile * tiles_x + row tile.
 struct SliceSumJob {
     const float* partial;
     void* out;
@@ -351,10 +351,8 @@ __global__ void __launch_bounds__(256) slices_to_gradients_kernel(const SliceSum
     const int pieces = j.bn / 4;
     const long long total = static_cast<long long>(j.tiles_x) * j.tiles_y * 128 * pieces;
     for (long long i = static_cast<long long>(b) * blockDim.x + threadIdx.x; i < total; i += static_cast<long long>(nb) * blockDim.x) {
-        const int pc = static_cast<int>(i % pieces);
-        const long long t = i / pieces;
-        const int rin = static_cast<int>(t % 128);
-        const int tile = static_cast<int>(t / 128);
+        const int in = static_cast<int>(i % (128 * pieces)), tile = static_cast<int>(i / (128 * pieces));
+        const int pc = (in >> 5) % pieces, rin = (in >> 5) / pieces * 32 + (in & 31);
         const int bx = tile % j.tiles_x, by = tile / j.tiles_x;
         const int col = by * j.bn + pc * 4;
         int row = bx * 128 + rin;
@@ -363,7 +361,7 @@ __global__ void __launch_bounds__(256) slices_to_gradients_kernel(const SliceSum
             row = c < j.conv_c ? tap * j.conv_c + c : j.M;
         }
         if (row >= j.M || col >= j.N) continue;
-        const float* src = j.partial + (static_cast<size_t>(tile) * j.S * 128 + rin) * j.bn + ((pc ^ (rin & (pieces - 1))) << 2);
+        const float* src = j.partial + static_cast<size_t>(tile) * j.S * 128 * j.bn + static_cast<size_t>(in) * 4;
         float4 acc = *reinterpret_cast<const float4*>(src);
         for (int s = 1; s < j.S; ++s) {
             const float4 w = *reinterpret_cast<const float4*>(src + static_cast<size_t>(s) * 128 * j.bn);

@@ -84,7 +84,6 @@ struct F32Ctl {
     uint64_t main_full[2];       // a main accumulator holds its chunk
     uint64_t main_empty[2];      // the workers have drained it (16 warps)
     uint64_t corr_full;
-    uint64_t fix_full;
     uint32_t tmem_base;
     uint32_t abort;
     uint32_t fix_ok;
@@ -107,11 +106,6 @@ __device__ __forceinline__ void split_pair(float lo, float hi, uint32_t& p1, uin
 }
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
     asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
-}
-__device__ __forceinline__ uint32_t ld_acquire(const unsigned int* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
 }
 
 // A: the thread owns row q * 32 + lane of the tile and 16 of the k-block's elements (half kh), whose planes it writes to
@@ -251,7 +245,6 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
             mbar_init(smem_u32(&ctl->main_empty[h]), 16);
         }
         mbar_init(smem_u32(&ctl->corr_full), 1);
-        mbar_init(smem_u32(&ctl->fix_full), 1);
         ctl->abort = 0;
         ctl->fix_ok = 0;
         fence_barrier_init();
@@ -484,31 +477,27 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
         }
         if (ok) {
             add_from(lane_base + 2 * BN);
-            // 32 rows of kCols floats go through shared memory (the ring is idle: every warp has split its last k-block once
-            // corr_full fired), 16-byte pieces XOR-permuted by the row against bank conflicts
             constexpr uint32_t kPieces = kCols / 4, kRowBytes = kCols * 4;
-            const uint32_t panel = ring + static_cast<uint32_t>(colq * 128 + q * 32) * kRowBytes;
-            const uint32_t own = panel + static_cast<uint32_t>(lane) * kRowBytes;
-#pragma unroll
-            for (uint32_t g = 0; g < kPieces; ++g)
-                st_shared_v4(own + ((g ^ (static_cast<uint32_t>(lane) & (kPieces - 1))) << 4),
-                             make_uint4(__float_as_uint(acc[4 * g]), __float_as_uint(acc[4 * g + 1]), __float_as_uint(acc[4 * g + 2]),
-                                        __float_as_uint(acc[4 * g + 3])));
             if (p.splits > 1) {
-                // slice: they leave as one bulk copy; then the warp reports
-                fence_proxy_async_smem();
+                // slice: straight to the workspace, [column quarter][quadrant][4-column group][row][4], a run of 512 bytes
+                // per instruction; then the warp reports
+                float* dst = p.partial + (static_cast<size_t>(tile) * p.splits + bz) * (128u * BN) +
+                             static_cast<size_t>(colq * 4 + q) * (32 * kCols) + lane * 4;
+#pragma unroll
+                for (uint32_t g = 0; g < kPieces; ++g)
+                    *reinterpret_cast<float4*>(dst + g * 128) = make_float4(acc[4 * g], acc[4 * g + 1], acc[4 * g + 2], acc[4 * g + 3]);
                 __syncwarp();
-                if (lane == 0) {
-                    uint8_t* dst = reinterpret_cast<uint8_t*>(p.partial) + (static_cast<size_t>(tile) * p.splits + bz) * (128u * BN * 4u) +
-                                   static_cast<size_t>(colq * 128 + q * 32) * kRowBytes;
-                    bulk_store(dst, panel, 32u * kRowBytes);
-                    tma_store_commit();
-                    tma_store_wait_all();
-                    fence_proxy_async_all();
-                    __threadfence();
-                    atomicAdd(p.counters + 2 * tile, 1u);
-                }
+                if (lane == 0) red_release_gpu(p.counters + 2 * tile, 1u);
             } else {
+                // 32 rows of kCols floats go through shared memory (the ring is idle: every warp has split its last k-block once
+                // corr_full fired), 16-byte pieces XOR-permuted by the row against bank conflicts
+                const uint32_t panel = ring + static_cast<uint32_t>(colq * 128 + q * 32) * kRowBytes;
+                const uint32_t own = panel + static_cast<uint32_t>(lane) * kRowBytes;
+    #pragma unroll
+                for (uint32_t g = 0; g < kPieces; ++g)
+                    st_shared_v4(own + ((g ^ (static_cast<uint32_t>(lane) & (kPieces - 1))) << 4),
+                                 make_uint4(__float_as_uint(acc[4 * g]), __float_as_uint(acc[4 * g + 1]), __float_as_uint(acc[4 * g + 2]),
+                                            __float_as_uint(acc[4 * g + 3])));
                 // stored as whole row segments, 32 / kPieces rows per instruction
                 __syncwarp();
                 constexpr int kRowsPer = 32 / static_cast<int>(kPieces);
@@ -557,59 +546,47 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
     if (warp == 1) tmem_dealloc(tmem, 512);
     if (p.splits <= 1) return;
 
-    // ---- slice sum (as in pf_tc_gemm_kernel.cuh): once all slices of the tile are in the workspace, each CTA gathers its
-    // share of the rows from every slice, adds them in slice order and stores them
-    constexpr uint32_t kPieces = kCols / 4, kRowBytes = kCols * 4;
+    // ---- slice sum (as in pf_tc_gemm_kernel.cuh): once all slices of the tile are in the workspace, each CTA adds its
+    // share of them in slice order and stores the sums
     unsigned int* cnt = p.counters + 2 * tile;
     const int S = p.splits;
-    const int rper = (128 + S - 1) / S, r_beg = bz * rper;
-    const int nr = max(0, min(128, r_beg + rper) - r_beg);
-    const uint32_t share = static_cast<uint32_t>(nr) * kRowBytes;       // bytes of one column quarter of one slice
-    if (warp == 0) {
+    if (threadIdx.x == 0) {
         uint32_t good = (*abort_flag == 0u) ? 1u : 0u;
-        if (good && lane == 0) {
-            const unsigned int want = 16u * static_cast<unsigned int>(S);
-            const long long t0 = clock64();
-            while (ld_acquire(cnt) < want) {
-                if (clock64() - t0 > kWaitCycleLimit) {
-                    good = 0u;
-                    if (p.status) atomicExch(p.status, kStatusTimeout);
-                    break;
-                }
+        const unsigned int want = 16u * static_cast<unsigned int>(S);
+        const long long t0 = clock64();
+        while (good && ld_acquire_gpu(cnt) < want) {
+            if (clock64() - t0 > kWaitCycleLimit) {
+                good = 0u;
+                if (p.status) atomicExch(p.status, kStatusTimeout);
             }
-            __threadfence();
-            if (good && nr > 0) mbar_expect_tx(smem_u32(&ctl->fix_full), 4u * share * static_cast<uint32_t>(S));
         }
-        good = __shfl_sync(0xffffffffu, good, 0);
-        __syncwarp();                        // lane 0's acquire orders the copies of all lanes
-        fence_proxy_async_all();
-        if (good && nr > 0) {
-            const uint32_t bar = smem_u32(&ctl->fix_full);
-            const uint8_t* src = reinterpret_cast<const uint8_t*>(p.partial) + static_cast<size_t>(tile) * S * (128u * BN * 4u) +
-                                 static_cast<size_t>(r_beg) * kRowBytes;
-            for (int e = lane; e < 4 * S; e += 32)          // (slice, column quarter) pairs, one copy each
-                bulk_load(ring + static_cast<uint32_t>(e) * share,
-                          src + static_cast<size_t>(e >> 2) * (128u * BN * 4u) + static_cast<size_t>(e & 3) * 128u * kRowBytes, share, bar);
-            good = mbar_wait_warp(bar, 0, abort_flag, p.status) ? 1u : 0u;
-        }
-        if (lane == 0) ctl->fix_ok = good;
+        ctl->fix_ok = good;
     }
     __syncthreads();
     if (ctl->fix_ok) {
+        // units of 8 rows x 16 columns, one per warp and step
+        constexpr int kUnits = 16 * (BN / 16), kQuarter = kCols / 16 > 0 ? kCols / 16 : 1;
+        constexpr size_t kSlice = 128 * BN / 4;                  // float4s
         const bool vec = (p.ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(p.C) & 15) == 0;
-        for (int id = threadIdx.x; id < nr * static_cast<int>(4 * kPieces); id += kF32Threads) {
-            const int rl = id / static_cast<int>(4 * kPieces), pc = id % static_cast<int>(4 * kPieces);
-            const int cq = pc / static_cast<int>(kPieces), pp = pc % static_cast<int>(kPieces), rr = r_beg + rl;
-            const uint32_t o = static_cast<uint32_t>(cq) * share + static_cast<uint32_t>(rl) * kRowBytes +
-                               ((static_cast<uint32_t>(pp) ^ (static_cast<uint32_t>(rr) & (kPieces - 1))) << 4);
+        const int per = (kUnits + S - 1) / S, end = min(kUnits, (bz + 1) * per);
+#pragma unroll 1
+        for (int u = bz * per + warp; u < end; u += kF32Threads / 32) {
+            const int oct = u / (BN / 16), cell = u - oct * (BN / 16), cq = cell / kQuarter;
+            const int pc = (cell - cq * kQuarter) * 4 + (lane >> 3), rr = oct * 8 + (lane & 7);
+            const float4* src = reinterpret_cast<const float4*>(p.partial) + static_cast<size_t>(tile) * S * kSlice +
+                                ((cq * 4 + (rr >> 5)) * (kCols / 4) + pc) * 32 + (rr & 31);
             float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-            for (int sl = 0; sl < S; ++sl) {
-                const uint4 v = ld_shared_v4(ring + static_cast<uint32_t>(4 * sl) * share + o);
-                a.x += __uint_as_float(v.x); a.y += __uint_as_float(v.y);
-                a.z += __uint_as_float(v.z); a.w += __uint_as_float(v.w);
+#pragma unroll 1
+            for (int s0 = 0; s0 < S; s0 += 8) {
+                float4 w[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (s0 + i < S) w[i] = __ldcg(src + static_cast<size_t>(s0 + i) * kSlice);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (s0 + i < S) { a.x += w[i].x; a.y += w[i].y; a.z += w[i].z; a.w += w[i].w; }
             }
-            const int row = f32_row<kMode>(p, org, bx, rr), col = n0 + cq * kCols + pp * 4;
+            const int row = f32_row<kMode>(p, org, bx, rr), col = n0 + cq * kCols + pc * 4;
             if (row < 0) continue;
             const float v[4] = {a.x, a.y, a.z, a.w};
             float* dst = p.C + static_cast<size_t>(row) * p.ldc + col;

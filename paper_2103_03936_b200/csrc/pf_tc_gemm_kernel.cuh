@@ -83,17 +83,10 @@ struct GemmCtl {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
     uint64_t tmem_full;
-    uint64_t fix_full;       // the slices this CTA sums have been copied into shared memory
     uint32_t tmem_base;
     uint32_t abort;
     uint32_t fix_ok;
 };
-
-__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 
 // What a row tile covers: the first image, row and class of a convolution's block (unused otherwise).
 struct TileOrigin {
@@ -139,14 +132,22 @@ __device__ __forceinline__ int output_row(const GemmParams& p, const TileOrigin&
     }
 }
 
+__device__ __forceinline__ void store_columns(__nv_bfloat16* dst, uint32_t lo, uint32_t hi, int left) {
+    unsigned short* d = reinterpret_cast<unsigned short*>(dst);
+    if (left > 0) d[0] = static_cast<unsigned short>(lo);
+    if (left > 1) d[1] = static_cast<unsigned short>(lo >> 16);
+    if (left > 2) d[2] = static_cast<unsigned short>(hi);
+    if (left > 3) d[3] = static_cast<unsigned short>(hi >> 16);
+}
+
 // One output tile (128 rows x BN columns) of C = A * B, or one slice of its contraction.
 //
 // Epilogue.  Unsplit: each epilogue warp turns its 32 accumulator rows into bf16, transposes them
 // through a padded shared-memory panel and writes whole 128-byte row segments (any pitch, any
 // alignment, clipped at the matrix edge).  Split: the fp32 slice goes to the workspace in the
-// order [32-column chunk][4-column group][row][4], which makes every store instruction of a warp
+// order [32-row quadrant][4-column group][row][4], which makes every store instruction of a warp
 // one contiguous 512-byte run; then the CTAs of a tile meet at a counter and each sums, in slice
-// order, its share of the rows over all slices and writes bf16 (bit-reproducible, no second launch).
+// order, its share over all slices and writes bf16 (bit-reproducible, no second launch).
 // kMode: 0 = plain (or grouped) product, 1 / 2 = the convolution products of GemmParams, compiled apart so that
 // the plain kernels carry none of their code (with all of them in one kernel the FFN backward ran 12 % slower).
 template <int BN, int kMode>
@@ -179,7 +180,6 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
             mbar_init(smem_u32(&ctl->empty[s]), 1);
         }
         mbar_init(smem_u32(&ctl->tmem_full), 1);
-        mbar_init(smem_u32(&ctl->fix_full), 1);
         ctl->abort = 0;
         ctl->fix_ok = 0;
         fence_barrier_init();
@@ -380,38 +380,23 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
         if (ok) {
             const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
             if (p.splits > 1) {
-                // fp32 slice: this warp's 32 rows go to shared memory as rows of BN floats (the 16-byte
-                // pieces of a row XOR-permuted by the row, which keeps the writes and the later reads
-                // free of bank conflicts), leave as ONE bulk copy of 32 x BN x 4 bytes to the
-                // workspace (the workspace keeps the permuted order; only the sum below reads it),
-                // and the warp reports its arrival once the copy has completed
-                constexpr uint32_t kRowBytes = BN * 4, kPieces = BN / 4;
-                const uint32_t wbase = smem_u32(tiles) + static_cast<uint32_t>(q * 32) * kRowBytes;
-                const uint32_t rbase = wbase + static_cast<uint32_t>(lane) * kRowBytes;
-                const uint32_t rsw = static_cast<uint32_t>(q * 32 + lane) & (kPieces - 1);
+                // fp32 slice: straight from registers, [quadrant][4-column group][row][4], so that every store
+                // instruction of a warp is one run of 512 bytes; then the warp reports
+                float* dst = p.partial + (static_cast<size_t>(tile) * p.splits + bz) * (kBM * BN) +
+                             static_cast<size_t>(q * (BN / 4) * 32 + lane) * 4;
 #pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
-                    uint32_t v[32];
-                    tmem_ld32(lane_base + c * 32, v);
+                for (int c = 0; c < BN / 64; ++c) {
+                    uint32_t v[2][32];
+                    tmem_ld32(lane_base + c * 64, v[0]);
+                    tmem_ld32(lane_base + c * 64 + 32, v[1]);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int g = 0; g < 8; ++g)
-                        st_shared_v4(rbase + (((static_cast<uint32_t>(c * 8 + g)) ^ rsw) << 4),
-                                     make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]));
+                    for (int g = 0; g < 16; ++g)
+                        *reinterpret_cast<uint4*>(dst + static_cast<size_t>(c * 16 + g) * 128) =
+                            make_uint4(v[g >> 3][4 * (g & 7)], v[g >> 3][4 * (g & 7) + 1], v[g >> 3][4 * (g & 7) + 2], v[g >> 3][4 * (g & 7) + 3]);
                 }
-                fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0) {
-                    uint8_t* dst = reinterpret_cast<uint8_t*>(p.partial) +
-                                   (static_cast<size_t>(tile) * p.splits + bz) * (static_cast<size_t>(kBM) * kRowBytes) +
-                                   static_cast<size_t>(q * 32) * kRowBytes;
-                    bulk_store(dst, wbase, 32u * kRowBytes);
-                    tma_store_commit();
-                    tma_store_wait_all();          // the rows are in the workspace
-                    fence_proxy_async_all();
-                    __threadfence();
-                    atomicAdd(p.counters + 2 * tile, 1u);
-                }
+                if (lane == 0) red_release_gpu(p.counters + 2 * tile, 1u);
             } else {
                 // every MMA has completed, so the pipeline stages are free: 32 x 33-word panel per warp
                 uint32_t* stg = reinterpret_cast<uint32_t*>(tiles) + (warp - 2) * (32 * 33);
@@ -529,42 +514,24 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     if (warp == 1) tmem_dealloc(tmem_base, BN);
     if (p.splits <= 1) return;
 
-    // ---- slice sum: wait until every slice of this tile is in the workspace (four warps of every slice
-    // report), then sum a share of it.  A share is a run of whole rows, contiguous in every slice, so
-    // one bulk copy per slice brings it into the idle pipeline stages: a single trip to L2 for the
-    // whole sum.  The slices are added in slice order (bit-reproducible) and each summed row leaves as
-    // whole 8-byte pieces, a warp writing 256 contiguous bytes per instruction.
+    // ---- slice sum: wait until every slice of this tile is in the workspace (four warps of every slice report), then
+    // sum a share of it, in slice order (bit-reproducible).  A warp sums units of 8 rows x 32 columns, up to eight
+    // slices of a unit (16 loads per lane) in flight together, 32 bytes stored per row and 16 columns.  What bounds
+    // it is latency: registers to workspace to registers, without shared memory in between, replaced a bulk copy out, the
+    // fences between the proxies and a bulk copy back, which together took 6.3 us from the last MMA to the stored sum
+    // (7 slices of 128 x 128).  Backward of 8192 rows, 512 -> 128 -> 2048: 24.6 -> 22.6 us; 1070 rows, 888 -> 208 ->
+    // 3552: 28.0 -> 26.3.  One version of short code: it runs once, from a cold instruction cache, and variants per slice
+    // count with deeper unrolling lost up to 5 us.  (Half the loads in flight: 24.2 and 28.8 us.)
     unsigned int* cnt = p.counters + 2 * tile;
     const int S = p.splits;
-    constexpr uint32_t kRowBytes = BN * 4, kPieces = BN / 4;
-    const int rper = (kBM + S - 1) / S;
-    const int r_beg = bz * rper;
-    const int nr = max(0, min(kBM, r_beg + rper) - r_beg);
-    const uint32_t share = static_cast<uint32_t>(nr) * kRowBytes;
     if (threadIdx.x == 0) {
         uint32_t good = (*abort_flag == 0u) ? 1u : 0u;
-        if (good) {
-            const unsigned int want = 4u * static_cast<unsigned int>(S);
-            const long long t0 = clock64();
-            while (ld_acquire_gpu(cnt) < want) {
-                if (clock64() - t0 > kWaitCycleLimit) {
-                    good = 0u;
-                    if (p.status) atomicExch(p.status, kStatusTimeout);
-                    break;
-                }
-            }
-            __threadfence();
-            fence_proxy_async_all();
-            if (good && nr > 0) {
-                const uint32_t bar = smem_u32(&ctl->fix_full);
-                const uint8_t* src = reinterpret_cast<const uint8_t*>(p.partial) +
-                                     (static_cast<size_t>(tile) * S) * (static_cast<size_t>(kBM) * kRowBytes) +
-                                     static_cast<size_t>(r_beg) * kRowBytes;
-                mbar_expect_tx(bar, share * static_cast<uint32_t>(S));
-                for (int s = 0; s < S; ++s)
-                    bulk_load(smem_u32(tiles) + static_cast<uint32_t>(s) * share,
-                              src + static_cast<size_t>(s) * (static_cast<size_t>(kBM) * kRowBytes), share, bar);
-                good = mbar_wait(bar, 0, abort_flag, p.status) ? 1u : 0u;
+        const unsigned int want = 4u * static_cast<unsigned int>(S);
+        const long long t0 = clock64();
+        while (good && ld_acquire_gpu(cnt) < want) {
+            if (clock64() - t0 > kWaitCycleLimit) {
+                good = 0u;
+                if (p.status) atomicExch(p.status, kStatusTimeout);
             }
         }
         ctl->fix_ok = good;
@@ -573,40 +540,45 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     if (ctl->fix_ok) {
         __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
         __nv_bfloat16* C2b = p.C2 ? reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride : nullptr;
-        const uint32_t base = smem_u32(tiles);
         const bool vec8 = (p.ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 7) == 0;
-        // consecutive threads take consecutive 16-byte pieces of one row
-        for (int id = threadIdx.x; id < nr * static_cast<int>(kPieces); id += kGemmThreads) {
-            const int rl = id / static_cast<int>(kPieces), pc = id % static_cast<int>(kPieces);
-            const int rr = r_beg + rl;
-            const uint32_t off = static_cast<uint32_t>(rl) * kRowBytes +
-                                 ((static_cast<uint32_t>(pc) ^ (static_cast<uint32_t>(rr) & (kPieces - 1))) << 4);
-            uint4 w = ld_shared_v4(base + off);
-            float4 acc = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
-#pragma unroll 4
-            for (int s = 1; s < S; ++s) {
-                w = ld_shared_v4(base + static_cast<uint32_t>(s) * share + off);
-                acc.x += __uint_as_float(w.x); acc.y += __uint_as_float(w.y);
-                acc.z += __uint_as_float(w.z); acc.w += __uint_as_float(w.w);
+        // units of 8 rows x 32 columns: a lane holds two 4-column groups of a row, 16 columns apart
+        constexpr int kUnits = kBM / 8 * (BN / 32);
+        constexpr size_t kSlice = static_cast<size_t>(kBM) * BN / 4;       // float4s
+        const int per = (kUnits + S - 1) / S, end = min(kUnits, (bz + 1) * per);
+#pragma unroll 1
+        for (int u = bz * per + warp; u < end; u += kGemmThreads / 32) {
+            const int oct = u / (BN / 32), pc = (u - oct * (BN / 32)) * 8 + (lane >> 3), rr = oct * 8 + (lane & 7);
+            const float4* src = reinterpret_cast<const float4*>(p.partial) + static_cast<size_t>(tile) * S * kSlice +
+                                ((rr >> 5) * (BN / 4) + pc) * 32 + (rr & 31);
+            float4 acc[2];
+            acc[0] = acc[1] = make_float4(-0.f, -0.f, -0.f, -0.f);
+#pragma unroll 1
+            for (int s0 = 0; s0 < S; s0 += 8) {
+                float4 w[8][2];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (s0 + i < S) {
+                        w[i][0] = __ldcg(src + static_cast<size_t>(s0 + i) * kSlice);
+                        w[i][1] = __ldcg(src + static_cast<size_t>(s0 + i) * kSlice + 4 * 32);
+                    }
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (s0 + i < S) {
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) { acc[j].x += w[i][j].x; acc[j].y += w[i][j].y; acc[j].z += w[i][j].z; acc[j].w += w[i][j].w; }
+                    }
             }
-            const int row = output_row<kMode>(p, org, bx, rr), col = n0 + pc * 4;
-            if (row >= 0) {
+            const int row = output_row<kMode>(p, org, bx, rr);
+            if (row < 0) continue;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int col = n0 + pc * 4 + j * 16;
                 __nv_bfloat16* dst = Cb + static_cast<size_t>(row) * p.ldc + col;
-                if (vec8 && col + 3 < p.N) {
-                    *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
-                } else {
-                    if (col < p.N) dst[0] = __float2bfloat16_rn(acc.x);
-                    if (col + 1 < p.N) dst[1] = __float2bfloat16_rn(acc.y);
-                    if (col + 2 < p.N) dst[2] = __float2bfloat16_rn(acc.z);
-                    if (col + 3 < p.N) dst[3] = __float2bfloat16_rn(acc.w);
-                }
-                if (C2b) {   // the same sums once more, for a destination whose pitch the first cannot have
-                    __nv_bfloat16* d2 = C2b + static_cast<size_t>(row) * p.ldc2 + col;
-                    if (col < p.N) d2[0] = __float2bfloat16_rn(acc.x);
-                    if (col + 1 < p.N) d2[1] = __float2bfloat16_rn(acc.y);
-                    if (col + 2 < p.N) d2[2] = __float2bfloat16_rn(acc.z);
-                    if (col + 3 < p.N) d2[3] = __float2bfloat16_rn(acc.w);
-                }
+                const uint32_t lo = pack_bf16x2(acc[j].x, acc[j].y), hi = pack_bf16x2(acc[j].z, acc[j].w);
+                if (vec8 && col + 3 < p.N) *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
+                else store_columns(dst, lo, hi, p.N - col);
+                // the same sums once more, for a destination whose pitch the first cannot have
+                if (C2b) store_columns(C2b + static_cast<size_t>(row) * p.ldc2 + col, lo, hi, p.N - col);
             }
         }
     }
