@@ -40,19 +40,30 @@ struct Grouping {
     bool sum_groups = false;
 };
 
-size_t gemm_smem(int bn, int stages) {
-    return 1024 + 1024 + static_cast<size_t>(stages) * (kBM * kBK * 2 + bn * kBK * 2);
+size_t gemm_smem(int bn, int stages, bool dx = false) {
+    return 1024 + 1024 + static_cast<size_t>(stages) * (kBM * kBK * 2 + bn * kBK * 2) + (dx ? 4 * kDxPanel : 0);
 }
 // Pipeline depth: a grid that fits one wave gets every stage shared memory has room for; a
 // larger grid gets stages small enough for two CTAs per SM, so that the prologue and epilogue of
 // one CTA overlap the main loop of the other.
-int pick_stages(int bn, int64_t ctas) {
+int pick_stages(int bn, int64_t ctas, bool dx = false) {
     const size_t stage = static_cast<size_t>(kBM * kBK * 2 + bn * kBK * 2);
-    const size_t room = (ctas > num_sms() && bn <= 128) ? (113 * 1024 - 2048) : (200 * 1024 - 2048);
+    const size_t room = ((ctas > num_sms() && bn <= 128) ? (113 * 1024 - 2048) : (200 * 1024 - 2048)) - (dx ? 4 * kDxPanel : 0);
     int ns = static_cast<int>(room / stage);
     if (ns > kMaxStages) ns = kMaxStages;
     if (ns < 2) ns = 2;
     return ns;
+}
+
+// Blocks that share the tiles of a convolution's dX: runs of about 16 k-blocks hide the start of a block (2 tiles of a
+// stride-1 layer, 8 of a strided one, whose tiles are short), longer ones make the blocks of the launch unequal
+// (32 x 56 x 56, 64 -> 16 -> 64 with 6 tiles per block: 61 us instead of 56); every SM gets a block first.
+// The tiles of a block are that many blocks apart: no multiple of the stride's factors, so that it gets every class.
+unsigned dx_blocks(int64_t tiles, int64_t kblocks_per_tile, int stride) {
+    const int64_t want = std::min<int64_t>(8, std::max<int64_t>(2, ceil_div(16, std::max<int64_t>(1, kblocks_per_tile))));
+    int64_t blocks = ceil_div(tiles, std::min(want, ceil_div(tiles, num_sms())));
+    while (stride > 1 && blocks < tiles && (blocks % 2 == 0 || blocks % stride == 0)) ++blocks;      // (strides up to 4)
+    return static_cast<unsigned>(blocks);
 }
 
 template <int BN>
@@ -60,7 +71,7 @@ cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const Gemm
                         cudaStream_t stream) {
     cudaError_t e;
     if (p.conv_mode != 0) {
-        e = launch_gemm_conv(BN, grid, gemm_smem(BN, p.num_stages), stream, ta, tb, p);
+        e = launch_gemm_conv(BN, grid, gemm_smem(BN, p.num_stages, p.conv_mode == 1), stream, ta, tb, p);
     } else {
         e = allow_smem(tc_gemm_kernel<BN, 0>, std::min(gemm_smem(BN, kMaxStages), static_cast<size_t>(227 * 1024)));
         if (e == cudaSuccess)
@@ -172,7 +183,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     if (gr && (cv || groups < 1 || groups > 1024 || (sum_groups && (A.mn_major || B.mn_major)))) return PF_ERR_UNSUPPORTED;
     // wide outputs that would need more than one wave of 128-column tiles (two CTAs per SM) take
     // 256-column tiles
-    const int bn = (splits <= 1 && N >= 512 && ceil_div(M, kBM) * ceil_div(N, 128) > 2 * num_sms()) ? 256 : pick_bn(N);
+    const int bn = (!(cv && cv->mode == 1) && splits <= 1 && N >= 512 && ceil_div(M, kBM) * ceil_div(N, 128) > 2 * num_sms()) ? 256 : pick_bn(N);
     CUtensorMap& ta = out->ta;
     CUtensorMap& tb = out->tb;
     bool oka, okb;
@@ -246,7 +257,9 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.tiles_x = static_cast<int>(grid.x);
     p.tiles_y = static_cast<int>(grid.y);
     p.bn = bn;
-    p.num_stages = pick_stages(bn, static_cast<int64_t>(grid.x) * grid.y * grid.z);
+    const bool dx = p.conv_mode == 1;
+    if (dx) grid = dim3(dx_blocks(static_cast<int64_t>(p.tiles_x) * p.tiles_y, nkb / (cv->stride * cv->stride), cv->stride));
+    p.num_stages = pick_stages(bn, static_cast<int64_t>(grid.x) * grid.y * grid.z, dx);
     p.counters = nullptr;
     p.independent = 0;
     if (p.splits > 1) {
@@ -254,10 +267,6 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
         if (static_cast<int64_t>(grid.x) * grid.y * out_groups > kFixTiles || static_cast<int64_t>(grid.x) * grid.y * grid.z > num_sms() ||
             bn == 256 || partial == nullptr)
             return PF_ERR_UNSUPPORTED;
-        // the slices of a CTA's share are gathered in the pipeline stages
-        const int64_t rper = ceil_div(kBM, p.splits);
-        const int64_t room = static_cast<int64_t>(p.num_stages) * (kBM * kBK * 2 + bn * kBK * 2);
-        if (rper * p.splits * (bn * 4) > room || static_cast<int64_t>(kBM) * bn * 4 > room) return PF_ERR_UNSUPPORTED;
         p.counters = split_counters();
         if (!p.counters) return PF_ERR_CUDA;
     }
@@ -337,15 +346,10 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
     for (int i = 0; i < 3; ++i) {
         const GemmLaunch* src = g[i < count ? i : 0];
         prm[i] = src->p;
-        const int stages = pick_stages(src->bn, wave);
+        const bool dx = src->p.conv_mode == 1;
+        const int stages = pick_stages(src->bn, wave, dx);
         prm[i].num_stages = stages;
-        if (i < count) {
-            smem = std::max(smem, gemm_smem(src->bn, stages));
-            const int64_t rper = ceil_div(kBM, prm[i].splits);
-            const int64_t room = static_cast<int64_t>(stages) * (kBM * kBK * 2 + src->bn * kBK * 2);
-            if (prm[i].splits > 1 && (rper * prm[i].splits * (src->bn * 4) > room || static_cast<int64_t>(kBM) * src->bn * 4 > room))
-                return PF_ERR_UNSUPPORTED;
-        }
+        if (i < count) smem = std::max(smem, gemm_smem(src->bn, stages, dx));
     }
     Gemm3Args k;
     bool conv = false;

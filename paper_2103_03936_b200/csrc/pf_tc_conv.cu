@@ -18,11 +18,8 @@ cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtens
 
 cudaError_t launch_gemm_conv(int bn, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb,
                              const GemmParams& p) {
-    if (p.conv_mode == 1)
-        return bn == 64    ? launch_one<64, 1>(grid, smem, stream, ta, tb, p)
-               : bn == 128 ? launch_one<128, 1>(grid, smem, stream, ta, tb, p)
-                           : launch_one<256, 1>(grid, smem, stream, ta, tb, p);
-    if (bn > 128) return cudaErrorInvalidValue;        // dU tiles are as wide as the rank
+    if (bn > 128) return cudaErrorInvalidValue;
+    if (p.conv_mode == 1) return bn == 64 ? launch_one<64, 1>(grid, smem, stream, ta, tb, p) : launch_one<128, 1>(grid, smem, stream, ta, tb, p);
     return bn == 64 ? launch_one<64, 2>(grid, smem, stream, ta, tb, p) : launch_one<128, 2>(grid, smem, stream, ta, tb, p);
 }
 

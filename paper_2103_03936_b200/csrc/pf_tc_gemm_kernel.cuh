@@ -77,12 +77,14 @@ namespace {
 constexpr int kBM = 128;       // rows of the output tile = TMEM lanes
 constexpr int kBK = 64;        // contraction elements per pipeline stage (128 bytes of bf16)
 constexpr int kMaxStages = 6;
+constexpr uint32_t kDxPanel = 2048;      // staging of one epilogue warp of dx_tiles, behind the stages
 constexpr int kGemmThreads = 224;   // A producer, MMA issue, 4 epilogue warps, B producer
 
 struct GemmCtl {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
     uint64_t tmem_full;
+    uint64_t acc_full[2], acc_empty[2];      // dx_tiles
     uint32_t tmem_base;
     uint32_t abort;
     uint32_t fix_ok;
@@ -148,8 +150,8 @@ __device__ __forceinline__ void store_columns(__nv_bfloat16* dst, uint32_t lo, u
 // order [32-row quadrant][4-column group][row][4], which makes every store instruction of a warp
 // one contiguous 512-byte run; then the CTAs of a tile meet at a counter and each sums, in slice
 // order, its share over all slices and writes bf16 (bit-reproducible, no second launch).
-// kMode: 0 = plain (or grouped) product, 1 / 2 = the convolution products of GemmParams, compiled apart so that
-// the plain kernels carry none of their code (with all of them in one kernel the FFN backward ran 12 % slower).
+// kMode: 0 = plain (or grouped) product, 2 = dU of a convolution (dX: dx_tiles), compiled apart so that the plain
+// kernels carry none of its code (with all of them in one kernel the FFN backward ran 12 % slower).
 template <int BN, int kMode>
 __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p,
                                           const int bx, const int by, const int bz, const int bg) {
@@ -166,9 +168,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = bx * kBM, n0 = by * BN;
     const TileOrigin org = tile_origin<kMode>(p, bx);
-    const int nkb_total = kMode == 1 ? org.na * org.nb * p.cv_blks : p.nkb_total;
     const int kb_beg = bz * p.kb_per_split;
-    const int kb_end = min(nkb_total, kb_beg + p.kb_per_split);
+    const int kb_end = min(p.nkb_total, kb_beg + p.kb_per_split);
     const int nkb = kb_end - kb_beg;
     const uint32_t NS = static_cast<uint32_t>(p.num_stages);
     const int tile = (bg * p.tiles_y + by) * p.tiles_x + bx;
@@ -220,9 +221,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
             const bool do_a = warp == 0;
             const bool two = kMode != 2 || bx * 2 + 1 < p.cv_blocks;      // the tile's second channel block exists
             const uint32_t my_bytes = kMode == 2 ? static_cast<uint32_t>(p.kpix) * (do_a ? (two ? 256u : 128u) : BN * 2u)
-                                      : !do_a          ? kBBytes
-                                      : kMode == 1   ? static_cast<uint32_t>(p.rows_tile) * 128u
-                                                         : kABytes;
+                                                 : do_a ? kABytes : kBBytes;
             // One loop per addressing mode, its positions carried as counters in registers: whatever the thread
             // does per k-block beyond waiting and issuing paces the pipeline.
             const uint32_t base = smem_u32(tiles) + (do_a ? 0u : kABytes);
@@ -239,29 +238,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                 }
             };
             int k0 = kb_beg * kBK;
-            if constexpr (kMode == 1) {
-                const int blks = p.cv_blks, ntb = org.nb;
-                int rb = 0, tb = 0;
-                if (do_a) {
-                    const int y0 = org.ph + p.cv_pad - org.a0, xx = org.pw + p.cv_pad - org.b0;      // multiples of the stride
-                    int y = org.row + (p.cv_stride > 1 ? y0 / p.cv_stride : y0);
-                    const int x0 = p.cv_stride > 1 ? xx / p.cv_stride : xx, img = org.img;
-                    produce([&](uint32_t dst, uint32_t full) {
-                        tma_load_4d(dst, &tmA, full, rb * 64, x0 - tb, y, img);
-                        if (++rb == blks) { rb = 0; if (++tb == ntb) { tb = 0; --y; } }
-                    });
-                } else {
-                    int line = (org.a0 * p.cv_kw + org.b0) * p.cv_C + n0, at = line;      // row of U
-                    const int step_b = p.cv_stride * p.cv_C, step_a = step_b * p.cv_kw;
-                    produce([&](uint32_t dst, uint32_t full) {
-                        tma_load_2d(dst, &tmB, full, rb * 64, at);
-                        if (++rb == blks) {
-                            rb = 0; at += step_b;
-                            if (++tb == ntb) { tb = 0; line += step_a; at = line; }
-                        }
-                    });
-                }
-            } else if constexpr (kMode == 2) {
+            if constexpr (kMode == 2) {
                 const int bh = p.cv_bh, nimg = p.cv_nb, tpi = p.cv_tpi;
                 const int g = kb_beg / tpi;
                 int t = kb_beg - g * tpi, img = g * nimg;
@@ -593,12 +570,199 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     }
 }
 
+// Row and column tile of tile t of dX.  The classes of a block of pixels follow one another, so that blocks whose tiles are
+// a number apart that shares no factor with the stride take tiles of every class.
+__device__ __forceinline__ int dx_tile(const GemmParams& p, int t, int* by) {
+    *by = t / p.tiles_x;
+    const int bx = t - *by * p.tiles_x;
+    if (p.cv_stride == 1) return bx;
+    const int classes = p.cv_stride * p.cv_stride, block = bx / classes;
+    return (bx - block * classes) * p.cv_tiles_class + block;
+}
+// dX of a convolution (conv_mode 1): output tiles first, first + step, ... of 128 rows x BN columns.  A tile has few
+// k-blocks (taps of its class x 64-rank blocks: 9 at stride 1, 1 to 4 at stride 2), so with one tile per block the
+// start, the first loads and the epilogue cost as much as the products.  Here the producers run on into the next tiles
+// while the epilogue warps store the last one from the other of two accumulators.  What bounds it now is the SM's load
+// path.  Whole backward, one tile per block -> runs: 128 x 32 x 32, 128 -> 64 -> 256, stride 2: 42 -> 34 us; 128 x 16 x 16,
+// 512 -> 128 -> 512: 114 -> 91 (against 256-column tiles); 128 x 32 x 32, 256 -> 64 -> 256: 122 -> 117. 
+template <int BN>
+__device__ __forceinline__ void dx_tiles(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, const int first, const int step) {
+    constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2, kStageBytes = kABytes + kBBytes;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw_addr = smem_u32(smem_raw);
+    uint8_t* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
+    GemmCtl* ctl = reinterpret_cast<GemmCtl*>(smem);
+    const uint32_t tiles = smem_u32(smem) + 1024u;
+    volatile uint32_t* abort_flag = &ctl->abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t NS = static_cast<uint32_t>(p.num_stages);
+    const int ntiles = p.tiles_x * p.tiles_y;
+
+    if (threadIdx.x == 0) {
+        for (uint32_t s = 0; s < NS; ++s) {
+            mbar_init(smem_u32(&ctl->full[s]), 2);
+            mbar_init(smem_u32(&ctl->empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&ctl->acc_full[b]), 1);
+            mbar_init(smem_u32(&ctl->acc_empty[b]), 4);
+        }
+        ctl->abort = 0;
+        fence_barrier_init();
+        fence_proxy_async_smem();
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
+    if (warp == 1) tmem_alloc(smem_u32(&ctl->tmem_base), 2 * BN);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    pdl_wait();
+    pdl_launch_dependents();
+    const uint32_t tmem_base = ctl->tmem_base;
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+
+    if (warp == 0 || warp == 6) {
+        if (elect_one()) {
+            const bool do_a = warp == 0;
+            const uint32_t my_bytes = do_a ? static_cast<uint32_t>(p.rows_tile) * 128u : kBBytes;
+            const uint32_t base = tiles + (do_a ? 0u : kABytes);
+            const int blks = p.cv_blks;
+            uint32_t s = 0, ph = 1, dst = base;
+            bool ok = true;
+            for (int t = first; t < ntiles && ok; t += step) {
+                int by;
+                const TileOrigin org = tile_origin<1>(p, dx_tile(p, t, &by));
+                const int ntb = org.nb, nkb = org.na * ntb * blks;
+                auto produce = [&](auto&& issue) {
+                    for (int i = 0; i < nkb; ++i) {
+                        ok = mbar_wait(empty0 + 8 * s, ph, abort_flag, p.status);
+                        if (!ok) break;
+                        const uint32_t full = full0 + 8 * s;
+                        mbar_expect_tx(full, my_bytes);
+                        issue(dst, full);
+                        dst += kStageBytes;
+                        if (++s == NS) { s = 0; dst = base; ph ^= 1u; }
+                    }
+                };
+                int rb = 0, tb = 0;
+                if (do_a) {
+                    const int y0 = org.ph + p.cv_pad - org.a0, xx = org.pw + p.cv_pad - org.b0;      // multiples of the stride
+                    int y = org.row + (p.cv_stride > 1 ? y0 / p.cv_stride : y0);
+                    const int x0 = p.cv_stride > 1 ? xx / p.cv_stride : xx, img = org.img;
+                    produce([&](uint32_t to, uint32_t full) {
+                        tma_load_4d(to, &tmA, full, rb * 64, x0 - tb, y, img);
+                        if (++rb == blks) { rb = 0; if (++tb == ntb) { tb = 0; --y; } }
+                    });
+                } else {
+                    int line = (org.a0 * p.cv_kw + org.b0) * p.cv_C + by * BN, at = line;      // row of U
+                    const int step_b = p.cv_stride * p.cv_C, step_a = step_b * p.cv_kw;
+                    produce([&](uint32_t to, uint32_t full) {
+                        tma_load_2d(to, &tmB, full, rb * 64, at);
+                        if (++rb == blks) {
+                            rb = 0; at += step_b;
+                            if (++tb == ntb) { tb = 0; line += step_a; at = line; }
+                        }
+                    });
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (elect_one()) {
+            const uint32_t idesc = make_idesc_bf16(kBM, BN, 0, 0);
+            const uint64_t a_desc0 = make_smem_desc(tiles, 16, 1024), b_desc0 = make_smem_desc(tiles + kABytes, 16, 1024);
+            const int ksteps = p.ksteps;
+            uint32_t s = 0, ph = 0, off = 0, buf = 0, bph = 1;
+            bool ok = true;
+            for (int t = first; t < ntiles && ok; t += step) {
+                int by;
+                const TileOrigin org = tile_origin<1>(p, dx_tile(p, t, &by));
+                const int nkb = org.na * org.nb * p.cv_blks;
+                ok = mbar_wait(smem_u32(&ctl->acc_empty[buf]), bph, abort_flag, p.status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t d = tmem_base + buf * BN;
+                for (int i = 0; i < nkb; ++i) {
+                    ok = mbar_wait(full0 + 8 * s, ph, abort_flag, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t a = a_desc0 + off, b = b_desc0 + off;
+                    tc_mma_bf16(d, a, b, idesc, i > 0 ? 1u : 0u);
+#pragma unroll
+                    for (int k = 1; k < 4; ++k)
+                        if (k < ksteps) tc_mma_bf16(d, a + 2 * k, b + 2 * k, idesc, 1u);
+                    tc_commit(empty0 + 8 * s);
+                    off += kStageBytes >> 4;
+                    if (++s == NS) { s = 0; off = 0; ph ^= 1u; }
+                }
+                if (ok) tc_commit(smem_u32(&ctl->acc_full[buf]));
+                buf ^= 1u;
+                if (buf == 0) bph ^= 1u;
+            }
+        }
+    } else if (warp < 6) {
+        const int q = warp & 3, sub = lane >> 2, piece = lane & 3;
+        // 32 rows x 32 columns per warp behind the stages: rows of 64 bytes, their 16-byte pieces XOR-permuted
+        const uint32_t panel = tiles + NS * kStageBytes + static_cast<uint32_t>(q) * kDxPanel;
+        const uint32_t own = panel + static_cast<uint32_t>(lane) * 64u, sw = static_cast<uint32_t>(lane >> 1) & 3u;
+        __nv_bfloat16* C = reinterpret_cast<__nv_bfloat16*>(p.C);
+        uint32_t buf = 0, bph = 0;
+        for (int t = first; t < ntiles; t += step) {
+            int by;
+            const int bx = dx_tile(p, t, &by);
+            const TileOrigin org = tile_origin<1>(p, bx);
+            int orow[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) orow[i] = output_row<1>(p, org, bx, q * 32 + i * 8 + sub);
+            if (!mbar_wait_warp(smem_u32(&ctl->acc_full[buf]), bph, abort_flag, p.status)) break;
+            tc_fence_after();
+            const uint32_t acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN;
+#pragma unroll 1
+            for (int c = 0; c < BN / 32; ++c) {
+                uint32_t v[32];
+                tmem_ld32(acc + c * 32, v);
+                tmem_ld_wait();
+                if (c + 1 == BN / 32) {               // read: hand the accumulator back before storing
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[buf]));
+                }
+#pragma unroll
+                for (int g = 0; g < 4; ++g)
+                    st_shared_v4(own + ((static_cast<uint32_t>(g) ^ sw) << 4),
+                                 make_uint4(pack_bf16x2(__uint_as_float(v[8 * g]), __uint_as_float(v[8 * g + 1])),
+                                            pack_bf16x2(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3])),
+                                            pack_bf16x2(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5])),
+                                            pack_bf16x2(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7]))));
+                __syncwarp();
+                const int col = by * BN + c * 32 + piece * 8;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t rr = static_cast<uint32_t>(i * 8 + sub);
+                    const uint4 w = ld_shared_v4(panel + rr * 64u + ((static_cast<uint32_t>(piece) ^ ((rr >> 1) & 3u)) << 4));
+                    if (orow[i] >= 0 && col < p.N) *reinterpret_cast<uint4*>(C + static_cast<size_t>(orow[i]) * p.ldc + col) = w;   // N, ldc: multiples of 8
+                }
+                __syncwarp();
+            }
+            buf ^= 1u;
+            if (buf == 0) bph ^= 1u;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem_base, 2 * BN);
+}
+
 template <int BN, int kMode>
 __global__ void __launch_bounds__(kGemmThreads, BN <= 128 ? 2 : 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const GemmParams p) {
-    const int sl = p.splits < 1 ? 1 : p.splits;
-    gemm_tile<BN, kMode>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
+    if constexpr (kMode == 1) {
+        dx_tiles<BN>(tmA, tmB, p, blockIdx.x, gridDim.x);
+    } else {
+        const int sl = p.splits < 1 ? 1 : p.splits;
+        gemm_tile<BN, kMode>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
+    }
 }
 
 // Up to three independent products in one launch (dU = x^T G, dV = dY^T T and, where it is a plain
@@ -609,14 +773,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 template <bool kConv>
 __device__ __forceinline__ void gemm_any(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, int idx,
                                          const int2 t) {
+    if constexpr (kConv) {
+        if (p.conv_mode == 1) {             // t.x = the blocks that share the tiles
+            if (p.bn == 64) dx_tiles<64>(tmA, tmB, p, idx, t.x);
+            else dx_tiles<128>(tmA, tmB, p, idx, t.x);
+            return;
+        }
+    }
     const int sl = p.splits < 1 ? 1 : p.splits;
     const int bx = idx % t.x, by = (idx / t.x) % t.y, zz = idx / (t.x * t.y);
     if constexpr (kConv) {
-        if (p.conv_mode == 1) {
-            if (p.bn == 64) gemm_tile<64, 1>(tmA, tmB, p, bx, by, 0, 0);
-            else gemm_tile<128, 1>(tmA, tmB, p, bx, by, 0, 0);
-            return;
-        }
         if (p.conv_mode == 2) {
             if (p.bn == 64) gemm_tile<64, 2>(tmA, tmB, p, bx, by, zz, 0);
             else gemm_tile<128, 2>(tmA, tmB, p, bx, by, zz, 0);

@@ -250,3 +250,15 @@ def test_resident_image_windows(N, H, W, C, R, O):
     """Many tiles of a 3 x 3, stride-1 convolution: the flat image sequence (a zero column and row between images) whose
     windows serve all taps; tiles across image borders, boxes of rows and of whole images, ragged channel blocks."""
     run_conv(wl.ConvCase("res", N, H, W, C, R, O, wl.BF16, 95))
+
+
+@pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad", [
+    (163, 16, 16, 64, 16, 64, 3, 1, 1),      # two dX tiles per block, a last block with one
+    (41, 30, 30, 136, 24, 40, 3, 2, 1),      # eight per block, two column tiles (one ragged), all classes in a block
+    (330, 9, 7, 72, 72, 40, 3, 2, 1),        # classes of unequal size, two rank blocks per tap
+    (150, 14, 14, 64, 8, 24, 5, 3, 2),       # nine classes of one to four taps
+    (300, 13, 13, 64, 16, 64, 4, 4, 0),      # stride 4: one tap per class
+])
+def test_several_dx_tiles_per_block(N, H, W, C, R, O, k, stride, pad):
+    """Enough output tiles of dX for several in a block: accumulators and pipeline stages change hands between tiles."""
+    run_conv(wl.ConvCase("dx", N, H, W, C, R, O, wl.BF16, 96, kh=k, kw=k, stride=stride, pad=pad))
