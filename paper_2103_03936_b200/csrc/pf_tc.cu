@@ -59,7 +59,7 @@ int pick_stages(int bn, int64_t ctas, bool dx = false) {
 // stride-1 layer, 8 of a strided one, whose tiles are short), longer ones make the blocks of the launch unequal
 // (32 x 56 x 56, 64 -> 16 -> 64 with 6 tiles per block: 61 us instead of 56); every SM gets a block first.
 // The tiles of a block are that many blocks apart: no multiple of the stride's factors, so that it gets every class.
-unsigned dx_blocks(int64_t tiles, int64_t kblocks_per_tile, int stride) {
+unsigned run_blocks(int64_t tiles, int64_t kblocks_per_tile, int stride) {
     const int64_t want = std::min<int64_t>(8, std::max<int64_t>(2, ceil_div(16, std::max<int64_t>(1, kblocks_per_tile))));
     int64_t blocks = ceil_div(tiles, std::min(want, ceil_div(tiles, num_sms())));
     while (stride > 1 && blocks < tiles && (blocks % 2 == 0 || blocks % stride == 0)) ++blocks;      // (strides up to 4)
@@ -172,6 +172,7 @@ struct GemmLaunch {
     GemmParams p;
     dim3 grid;
     int bn;
+    bool runs = false;       // several tiles per block (plain product, K-major A and MN-major B)
 };
 
 // Encodes the tensor maps and launch geometry of C[M,N] = A * B without launching.
@@ -258,7 +259,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.tiles_y = static_cast<int>(grid.y);
     p.bn = bn;
     const bool dx = p.conv_mode == 1;
-    if (dx) grid = dim3(dx_blocks(static_cast<int64_t>(p.tiles_x) * p.tiles_y, nkb / (cv->stride * cv->stride), cv->stride));
+    if (dx) grid = dim3(run_blocks(static_cast<int64_t>(p.tiles_x) * p.tiles_y, nkb / (cv->stride * cv->stride), cv->stride));
     p.num_stages = pick_stages(bn, static_cast<int64_t>(grid.x) * grid.y * grid.z, dx);
     p.counters = nullptr;
     p.independent = 0;
@@ -277,6 +278,11 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
 
 // Launches one prepared product on its own.
 int launch_prepared(const GemmLaunch& g, cudaStream_t stream) {
+    if (g.runs) {
+        if (launch_gemm_runs(g.bn, g.grid, gemm_smem(g.bn, g.p.num_stages, true), stream, g.ta, g.tb, g.p) != cudaSuccess) return PF_ERR_CUDA;
+        count_launch();
+        return PF_OK;
+    }
     const cudaError_t e = g.bn == 64    ? launch_gemm<64>(g.ta, g.tb, g.p, g.grid, stream)
                           : g.bn == 128 ? launch_gemm<128>(g.ta, g.tb, g.p, g.grid, stream)
                                         : launch_gemm<256>(g.ta, g.tb, g.p, g.grid, stream);
@@ -977,6 +983,13 @@ int conv_bwd(const ConvArgs& a, int* handled) {
                      static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1, nullptr, &cx, &gx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     if (st != PF_OK) return st;
+    // dT: more tiles than two per SM, of few k-blocks each, go up to four to a block
+    const int64_t gt_tiles = static_cast<int64_t>(gt.grid.x) * gt.grid.y;
+    if (gt.bn <= 128 && gt.p.nkb_total <= 8 && gt_tiles > 2 * num_sms()) {
+        gt.runs = true;
+        gt.grid = dim3(static_cast<unsigned>(ceil_div(gt_tiles, std::min<int64_t>(4, ceil_div(gt_tiles, 2 * num_sms())))));
+        gt.p.num_stages = pick_stages(gt.bn, gt.grid.x, true);
+    }
     if (!a.T) {   // recompute the thin convolution (phase 1 of the forward only)
         const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
         st = chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);

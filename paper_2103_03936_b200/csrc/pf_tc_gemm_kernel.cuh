@@ -62,6 +62,8 @@ struct GemmParams {
 };
 
 // Launches of the convolution instantiations (pf_tc_conv.cu); same arguments as the kernels.
+cudaError_t launch_gemm_runs(int bn, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb,
+                             const GemmParams& p);
 cudaError_t launch_gemm_conv(int bn, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb,
                              const GemmParams& p);
 struct Gemm3Args {
@@ -77,14 +79,14 @@ namespace {
 constexpr int kBM = 128;       // rows of the output tile = TMEM lanes
 constexpr int kBK = 64;        // contraction elements per pipeline stage (128 bytes of bf16)
 constexpr int kMaxStages = 6;
-constexpr uint32_t kDxPanel = 2048;      // staging of one epilogue warp of dx_tiles, behind the stages
+constexpr uint32_t kDxPanel = 2048;      // staging of one epilogue warp of run_tiles, behind the stages
 constexpr int kGemmThreads = 224;   // A producer, MMA issue, 4 epilogue warps, B producer
 
 struct GemmCtl {
     uint64_t full[kMaxStages];
     uint64_t empty[kMaxStages];
     uint64_t tmem_full;
-    uint64_t acc_full[2], acc_empty[2];      // dx_tiles
+    uint64_t acc_full[2], acc_empty[2];      // run_tiles
     uint32_t tmem_base;
     uint32_t abort;
     uint32_t fix_ok;
@@ -150,7 +152,7 @@ __device__ __forceinline__ void store_columns(__nv_bfloat16* dst, uint32_t lo, u
 // order [32-row quadrant][4-column group][row][4], which makes every store instruction of a warp
 // one contiguous 512-byte run; then the CTAs of a tile meet at a counter and each sums, in slice
 // order, its share over all slices and writes bf16 (bit-reproducible, no second launch).
-// kMode: 0 = plain (or grouped) product, 2 = dU of a convolution (dX: dx_tiles), compiled apart so that the plain
+// kMode: 0 = plain (or grouped) product, 2 = dU of a convolution (dX: run_tiles), compiled apart so that the plain
 // kernels carry none of its code (with all of them in one kernel the FFN backward ran 12 % slower).
 template <int BN, int kMode>
 __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p,
@@ -572,10 +574,11 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
 
 // Row and column tile of tile t of dX.  The classes of a block of pixels follow one another, so that blocks whose tiles are
 // a number apart that shares no factor with the stride take tiles of every class.
-__device__ __forceinline__ int dx_tile(const GemmParams& p, int t, int* by) {
+template <int kMode>
+__device__ __forceinline__ int run_tile(const GemmParams& p, int t, int* by) {
     *by = t / p.tiles_x;
     const int bx = t - *by * p.tiles_x;
-    if (p.cv_stride == 1) return bx;
+    if (kMode == 0 || p.cv_stride == 1) return bx;
     const int classes = p.cv_stride * p.cv_stride, block = bx / classes;
     return (bx - block * classes) * p.cv_tiles_class + block;
 }
@@ -585,8 +588,8 @@ __device__ __forceinline__ int dx_tile(const GemmParams& p, int t, int* by) {
 // while the epilogue warps store the last one from the other of two accumulators.  What bounds it now is the SM's load
 // path.  Whole backward, one tile per block -> runs: 128 x 32 x 32, 128 -> 64 -> 256, stride 2: 42 -> 34 us; 128 x 16 x 16,
 // 512 -> 128 -> 512: 114 -> 91 (against 256-column tiles); 128 x 32 x 32, 256 -> 64 -> 256: 122 -> 117. 
-template <int BN>
-__device__ __forceinline__ void dx_tiles(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, const int first, const int step) {
+template <int BN, int kMode>
+__device__ __forceinline__ void run_tiles(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, const int first, const int step) {
     constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2, kStageBytes = kABytes + kBBytes;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -632,8 +635,9 @@ __device__ __forceinline__ void dx_tiles(const CUtensorMap& tmA, const CUtensorM
             bool ok = true;
             for (int t = first; t < ntiles && ok; t += step) {
                 int by;
-                const TileOrigin org = tile_origin<1>(p, dx_tile(p, t, &by));
-                const int ntb = org.nb, nkb = org.na * ntb * blks;
+                const int bx = run_tile<kMode>(p, t, &by);
+                const TileOrigin org = tile_origin<kMode>(p, bx);
+                const int ntb = org.nb, nkb = kMode == 1 ? org.na * ntb * blks : p.nkb_total;
                 auto produce = [&](auto&& issue) {
                     for (int i = 0; i < nkb; ++i) {
                         ok = mbar_wait(empty0 + 8 * s, ph, abort_flag, p.status);
@@ -646,7 +650,17 @@ __device__ __forceinline__ void dx_tiles(const CUtensorMap& tmA, const CUtensorM
                     }
                 };
                 int rb = 0, tb = 0;
-                if (do_a) {
+                if constexpr (kMode == 0) {
+                    if (do_a) {
+                        produce([&](uint32_t to, uint32_t full) { tma_load_2d(to, &tmA, full, rb, bx * kBM); rb += kBK; });
+                    } else {
+                        produce([&](uint32_t to, uint32_t full) {
+#pragma unroll
+                            for (int h = 0; h < BN / 64; ++h) tma_load_2d(to + h * 8192, &tmB, full, by * BN + 64 * h, rb);
+                            rb += kBK;
+                        });
+                    }
+                } else if (do_a) {
                     const int y0 = org.ph + p.cv_pad - org.a0, xx = org.pw + p.cv_pad - org.b0;      // multiples of the stride
                     int y = org.row + (p.cv_stride > 1 ? y0 / p.cv_stride : y0);
                     const int x0 = p.cv_stride > 1 ? xx / p.cv_stride : xx, img = org.img;
@@ -669,15 +683,19 @@ __device__ __forceinline__ void dx_tiles(const CUtensorMap& tmA, const CUtensorM
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            const uint32_t idesc = make_idesc_bf16(kBM, BN, 0, 0);
-            const uint64_t a_desc0 = make_smem_desc(tiles, 16, 1024), b_desc0 = make_smem_desc(tiles + kABytes, 16, 1024);
+            constexpr uint32_t kStepB = kMode == 0 ? 128 : 2;      // (plain: B is MN-major)
+            const uint32_t idesc = make_idesc_bf16(kBM, BN, 0, kMode == 0);
+            const uint64_t a_desc0 = make_smem_desc(tiles, 16, 1024), b_desc0 = make_smem_desc(tiles + kABytes, kMode == 0 ? 8192 : 16, 1024);
             const int ksteps = p.ksteps;
             uint32_t s = 0, ph = 0, off = 0, buf = 0, bph = 1;
             bool ok = true;
             for (int t = first; t < ntiles && ok; t += step) {
-                int by;
-                const TileOrigin org = tile_origin<1>(p, dx_tile(p, t, &by));
-                const int nkb = org.na * org.nb * p.cv_blks;
+                int nkb = p.nkb_total;
+                if constexpr (kMode == 1) {
+                    int by;
+                    const TileOrigin org = tile_origin<1>(p, run_tile<1>(p, t, &by));
+                    nkb = org.na * org.nb * p.cv_blks;
+                }
                 ok = mbar_wait(smem_u32(&ctl->acc_empty[buf]), bph, abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
@@ -690,7 +708,7 @@ __device__ __forceinline__ void dx_tiles(const CUtensorMap& tmA, const CUtensorM
                     tc_mma_bf16(d, a, b, idesc, i > 0 ? 1u : 0u);
 #pragma unroll
                     for (int k = 1; k < 4; ++k)
-                        if (k < ksteps) tc_mma_bf16(d, a + 2 * k, b + 2 * k, idesc, 1u);
+                        if (kMode == 0 || k < ksteps) tc_mma_bf16(d, a + 2 * k, b + kStepB * k, idesc, 1u);
                     tc_commit(empty0 + 8 * s);
                     off += kStageBytes >> 4;
                     if (++s == NS) { s = 0; off = 0; ph ^= 1u; }
@@ -709,11 +727,11 @@ __device__ __forceinline__ void dx_tiles(const CUtensorMap& tmA, const CUtensorM
         uint32_t buf = 0, bph = 0;
         for (int t = first; t < ntiles; t += step) {
             int by;
-            const int bx = dx_tile(p, t, &by);
-            const TileOrigin org = tile_origin<1>(p, bx);
+            const int bx = run_tile<kMode>(p, t, &by);
+            const TileOrigin org = tile_origin<kMode>(p, bx);
             int orow[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) orow[i] = output_row<1>(p, org, bx, q * 32 + i * 8 + sub);
+            for (int i = 0; i < 4; ++i) orow[i] = output_row<kMode>(p, org, bx, q * 32 + i * 8 + sub);
             if (!mbar_wait_warp(smem_u32(&ctl->acc_full[buf]), bph, abort_flag, p.status)) break;
             tc_fence_after();
             const uint32_t acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + buf * BN;
@@ -758,7 +776,9 @@ __global__ void __launch_bounds__(kGemmThreads, BN <= 128 ? 2 : 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const GemmParams p) {
     if constexpr (kMode == 1) {
-        dx_tiles<BN>(tmA, tmB, p, blockIdx.x, gridDim.x);
+        run_tiles<BN, 1>(tmA, tmB, p, blockIdx.x, gridDim.x);
+    } else if constexpr (kMode == 3) {
+        run_tiles<BN, 0>(tmA, tmB, p, blockIdx.x, gridDim.x);
     } else {
         const int sl = p.splits < 1 ? 1 : p.splits;
         gemm_tile<BN, kMode>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
@@ -775,8 +795,8 @@ __device__ __forceinline__ void gemm_any(const CUtensorMap& tmA, const CUtensorM
                                          const int2 t) {
     if constexpr (kConv) {
         if (p.conv_mode == 1) {             // t.x = the blocks that share the tiles
-            if (p.bn == 64) dx_tiles<64>(tmA, tmB, p, idx, t.x);
-            else dx_tiles<128>(tmA, tmB, p, idx, t.x);
+            if (p.bn == 64) run_tiles<64, 1>(tmA, tmB, p, idx, t.x);
+            else run_tiles<128, 1>(tmA, tmB, p, idx, t.x);
             return;
         }
     }

@@ -257,6 +257,7 @@ def test_resident_image_windows(N, H, W, C, R, O):
     (41, 30, 30, 136, 24, 40, 3, 2, 1),      # eight per block, two column tiles (one ragged), all classes in a block
     (330, 9, 7, 72, 72, 40, 3, 2, 1),        # classes of unequal size, two rank blocks per tap
     (150, 14, 14, 64, 8, 24, 5, 3, 2),       # nine classes of one to four taps
+    (310, 8, 8, 64, 136, 200, 3, 1, 1),      # dT as well: ragged k-block, two column tiles
     (300, 13, 13, 64, 16, 64, 4, 4, 0),      # stride 4: one tap per class
 ])
 def test_several_dx_tiles_per_block(N, H, W, C, R, O, k, stride, pad):
