@@ -46,7 +46,7 @@ struct F32Params {
     long long ldc2;
     const float* bias;       // optional epilogue of an unsplit product: C = act(A B + bias)
     int act;
-    float* partial;          // splits > 1: slices, [tile][slice][column quarter][128 rows][bn / 4], pieces XOR-permuted by the row
+    float* partial;          // splits > 1: slices, [tile][slice][column quarter][32-row quadrant][4-column group][row][4]
     unsigned int* counters;
     unsigned int* status;
     // Convolution (kMode 1 = dX, 2 = dU, 3 = the thin convolution forward); names as in pf_tc_gemm_kernel.cuh, with 32-channel

@@ -253,9 +253,6 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_
     d |= static_cast<uint64_t>(2) << 61;
     return d;
 }
-__device__ __forceinline__ uint64_t desc_advance(uint64_t d, uint32_t bytes) {
-    return d + static_cast<uint64_t>(bytes >> 4);   // start-address field only; never carries out
-}
 // Instruction descriptor for kind::f16: bf16 x bf16 -> fp32, M x N tile, operand majors.
 __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N, int a_mn_major, int b_mn_major) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(a_mn_major) << 15) |
