@@ -81,11 +81,19 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
         M = ct.blocks * ct.pixels;                                  // rows of whole tiles
         K1 = static_cast<int64_t>(conv->kh) * conv->kw * ceil_div(conv->C, 64) * 64;
     }
-    const int rows_tile = conv ? ct.pixels : 128;
+    int rows_tile = conv ? ct.pixels : 128;
     if (!chain_plan(M, K1, N2, r, out != nullptr, &plan, rows_tile, max_split)) return PF_ERR_UNSUPPORTED;
+    // Row tiles of 96 rows where they fit one wave: a block's time is that of its own rows through its SM's load and store
+    // path, so SMs that 128-row tiles leave idle take some of them (the idle MMA rows cost nothing).  Not where the output
+    // columns are split (148 instead of 128 blocks of an FFN layer delay the next launch's start: training step 1-3 %
+    // slower), and not where another launch counts on the idle SMs (max_split).  Forward, 12000 rows, 768 -> 96 -> 3072:
+    // 29.2 -> 25.1 us (125 blocks instead of 94).  112 rows would help 16384-row layers by 1-2 % (147 blocks instead of 128),
+    // but need output boxes of 16 rows, which slowed the 128-row tiles as much.
+    if (!conv && out && max_split <= 0 && plan.nsplit == 1 && ceil_div(M, 96) <= num_sms()) rows_tile = 96;
+    if (!conv) plan.row_tiles = static_cast<int>(ceil_div(M, rows_tile));
     CUtensorMap ta, tb1, tb2, to, tt;
     const bool ragged = conv && conv->C % 64 != 0;
-    bool ok = conv ? cached_map_nhwc(&ta, A, conv->N, conv->H, conv->W, conv->C, Wo, ct.bh, ct.nb, cs) : cached_map_2d(&ta, A, M, K1, lda, 128);
+    bool ok = conv ? cached_map_nhwc(&ta, A, conv->N, conv->H, conv->W, conv->C, Wo, ct.bh, ct.nb, cs) : cached_map_2d(&ta, A, M, K1, lda, rows_tile);
     ok = ok && (ragged ? cached_map_planes(&tb1, B1, static_cast<int64_t>(conv->kh) * conv->kw, conv->C, r, conv->C, 64)
                        : cached_map_2d(&tb1, B1, K1, r, ldb1, 64));
     ok = ok && cached_map_2d(&tb2, B2, N2, r, ldb2, 128);
@@ -95,7 +103,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
         ok = ok && (T ? cached_map_planes(&tt, T, starts, rows_tile, r, Wo, rows_tile) : cached_map_2d(&tt, B2, N2, r, ldb2, 128));
     } else {
         ok = ok && (out ? cached_map_2d(&to, out, M, N2, ldo, 32) : cached_map_2d(&to, B2, N2, r, ldb2, 32));
-        ok = ok && (T ? cached_map_2d(&tt, T, M, r, ldt, 128) : cached_map_2d(&tt, B2, N2, r, ldb2, 128));
+        ok = ok && (T ? cached_map_2d(&tt, T, M, r, ldt, rows_tile) : cached_map_2d(&tt, B2, N2, r, ldb2, 128));
     }
     if (!ok) return PF_ERR_CUDA;
     ChainParams p;

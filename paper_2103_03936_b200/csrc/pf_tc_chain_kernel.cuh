@@ -50,7 +50,7 @@ struct ChainParams {
     // images) and a k-block is (tap, 64-channel block).  The last tile of an image, and the last group of
     // images, starts early enough to be full: it recomputes rows of the tile before it, to the same values.
     int conv_cblks, conv_kw, conv_pad, conv_stride, conv_bh, conv_nb, conv_tpi, conv_Ho, conv_N;
-    int rows_tile;          // rows of A in one tile: 128, or the output pixels of a convolution's tile (<= 128)
+    int rows_tile;          // rows of A in one tile: 128 or 96, or the output pixels of a convolution's tile (<= 128)
     int row_tiles;          // tiles along M; a CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...
     int acc_base, acc_bufs; // TMEM column of the first phase-2 accumulator and their number (4 on top of T's
                             // columns, or 3 behind them when tiles overlap)

@@ -285,3 +285,11 @@ def test_few_rows_forward(m, k, n, r):
         gy.check()
         gT.check()
     assert pf.pf_last_device_status() == 0
+
+
+@pytest.mark.parametrize("m,k,n,r", [(14001, 72, 136, 136), (2331, 128, 64, 72), (9600, 64, 64, 16)])
+def test_row_tiles_of_96(m, k, n, r):
+    """Batches whose 128-row tiles would leave SMs idle run the fused kernel on 96-row tiles: guard bands, ragged last
+    tiles, both directions, padded pitches."""
+    run_case(wl.LinearCase("rows", m, k, n, r, wl.BF16, 29))
+    run_case(wl.LinearCase("rows", m, k, n, r, wl.BF16, 30), ld_pad=8)
