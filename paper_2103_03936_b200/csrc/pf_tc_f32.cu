@@ -102,7 +102,8 @@ F32Work f32_work(int64_t M, int64_t N, int64_t K, const F32Conv* cv = nullptr) {
             w.tiles_x = w.ct.blocks * cv->stride * cv->stride;
             w.nkb = static_cast<int64_t>(taps) * ceil_div(cv->R, 32);
         } else {
-            w.ct = conv_tiling(cv->N, cv->Ho, cv->Wo, 128);
+            // (a box spans stride input rows per output row, and TMA boxes are at most 256 high)
+            w.ct = conv_tiling(cv->N, cv->Ho, cv->Wo, std::min(128, 256 / cv->stride * cv->Wo));
             w.tiles_x = w.ct.blocks;
             w.nkb = static_cast<int64_t>(taps) * ceil_div(cv->C, 32);
         }

@@ -236,10 +236,12 @@ def test_tensor_core_tilings(N, H, W, C, R, O, k, stride, pad):
 
 
 @pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad", [(2, 9, 40, 36, 20, 24, 3, 1, 1), (5, 5, 5, 64, 16, 64, 3, 1, 1), (3, 11, 13, 100, 12, 40, 3, 2, 1),
-                                                      (1, 6, 6, 32, 132, 64, 3, 1, 0), (2, 12, 12, 64, 32, 72, 5, 3, 2)])
+                                                      (1, 6, 6, 32, 132, 64, 3, 1, 0), (2, 12, 12, 64, 32, 72, 5, 3, 2),
+                                                      (2, 300, 3, 8, 8, 12, 3, 3, 1), (1, 520, 4, 12, 4, 8, 4, 4, 0)])
 def test_fp32_tensor_core_tilings(N, H, W, C, R, O, k, stride, pad):
     """fp32 convolutions through the split-operand kernel: image rows longer than a reduction block, several images per
-    tile, ragged channel blocks, strided backward; held to fp32 accuracy."""
+    tile, ragged channel blocks, strided backward, strided images one output pixel wide (boxes of input rows are at most
+    256 high); held to fp32 accuracy."""
     errs = run_conv(wl.ConvCase("f32tc", N, H, W, C, R, O, wl.F32, 93, kh=k, kw=k, stride=stride, pad=pad))
     assert max(errs.values()) <= 1e-5, errs
     run_conv(wl.ConvCase("f32tc", N, H, W, C, R, O, wl.F32, 94, kh=k, kw=k, stride=stride, pad=pad), stash=False, need_dX=False)
