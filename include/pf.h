@@ -64,7 +64,9 @@ typedef enum {
 
 typedef enum {
     PF_F32 = 0, /* fp32 storage and accuracy: tensor-core products of exactly split operands (three bf16 parts, fp32
-                   accumulation), fp32 FMA arithmetic where a layout does not allow them */
+                   accumulation), fp32 FMA arithmetic where a layout does not allow them.  Subnormal operands count in
+                   full.  Outputs that an infinity, a NaN, an operand from 2^112 on or a sum from 2^96 on reaches are
+                   computed again with FMAs, with the whole tile around them, and are what FMA arithmetic gives. */
     PF_BF16 = 1 /* bf16 storage, tensor-core products with fp32 accumulation */
 } pf_dtype;
 

@@ -169,6 +169,10 @@ bool f32_prepare(const F32Work& w, const F32Op& A, const F32Op& B, float* C, int
     p->num_stages = f32_stages(w.bn);
     p->mode = c.mode;
     p->tiles_x = static_cast<int>(w.tiles_x); p->tiles_y = static_cast<int>(w.tiles_y);
+    p->A = static_cast<const float*>(A.p); p->B = static_cast<const float*>(B.p);
+    p->lda = A.ld; p->ldb = B.ld;
+    p->K = static_cast<int>(w.K);
+    p->cv_H = c.mode == 1 ? c.Ho : c.H; p->cv_W = c.mode == 1 ? c.Wo : c.W; p->cv_R = c.R;
     p->C = C; p->ldc = ldc;
     p->partial = partial;
     p->counters = w.splits > 1 ? split_counters() : nullptr;

@@ -1,7 +1,13 @@
 // fp32 products on the tensor cores (sm_100a): every fp32 operand value is split exactly into three bf16 values
-//   x = x1 + x2 + x3,  x1 = bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2
+//   2^16 x = x1 + x2 + x3,  x1 = bf16(2^16 x), x2 = bf16(2^16 x - x1), x3 = 2^16 x - x1 - x2
 // (8 + 8 + 8 significand bits), and a product a b is the sum of the six partial products that reach fp32
 // precision: a1 b1 | a1 b2 + a2 b1 + a2 b2 + a1 b3 + a3 b1 (the three left out are below 2^-24 of it).
+//
+// Range.  The last bit of an fp32 number is 2^-149 or more, that of a bf16 number 2^-133 or more: with the factor 2^16 the
+// split is exact down to the last subnormal (without it operands below 2^-110 lose digits).  The sums leave
+// the chip with 2^-32.  At the other end, operands from 2^112 on, infinities and NaN have a part that is
+// not finite, and sums from 2^96 on overflow: where a CTA finds such a sum it computes its outputs once more with
+// fp32 FMAs (f32_repair), which give what such operands give in fp32.
 //
 // Accumulation.  A tcgen05.mma truncates when it adds to its fp32 accumulator (measured: -0.5 ulp per MMA on
 // sums of one sign), so long sums must not stay in tensor memory: the main products a1 b1 accumulate over 64
@@ -40,6 +46,9 @@ struct F32Params {
     int num_stages;
     int mode;                // 0 = plain, 1 / 2 / 3 = the convolution products below
     int tiles_x, tiles_y;
+    const float *A, *B;      // the operands, as f32_repair reads them (the tiles come through the tensor maps)
+    long long lda, ldb;
+    int K, cv_H, cv_W, cv_R;         // cv_H x cv_W: the image that A is
     float* C;
     long long ldc;
     float* C2;               // optional second copy at another pitch
@@ -87,6 +96,7 @@ struct F32Ctl {
     uint32_t tmem_base;
     uint32_t abort;
     uint32_t fix_ok;
+    uint32_t repair;             // a sum is not finite
 };
 
 __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
@@ -94,8 +104,11 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
+constexpr float kScale = 65536.f, kUnscale = 1.f / (65536.f * 65536.f);
 // The three bf16 planes of a pair of floats.
 __device__ __forceinline__ void split_pair(float lo, float hi, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
+    asm("{\n .reg .b64 v, s;\n mov.b64 v, {%0, %1};\n mov.b64 s, {%2, %2};\n mul.rn.f32x2 v, v, s;\n mov.b64 {%0, %1}, v;\n}"
+        : "+f"(lo), "+f"(hi) : "f"(kScale));
     p1 = cvt_bf16x2(lo, hi);
     lo -= __uint_as_float(p1 << 16);
     hi -= __uint_as_float(p1 & 0xffff0000u);
@@ -209,6 +222,80 @@ __device__ __forceinline__ int f32_row(const F32Params& p, const F32Origin& o, i
     }
 }
 
+// Adds `len` products a[i sa] * b[i sb + c sc] to acc[c], c < n, 64 at a time.
+__device__ __forceinline__ void repair_run(const float* a, long long sa, const float* b, long long sb, long long sc, int len, int n, float (&acc)[4]) {
+#pragma unroll 1
+    for (int i0 = 0; i0 < len; i0 += 64) {
+        float part[4] = {0.f, 0.f, 0.f, 0.f};
+        const int end = min(len, i0 + 64);
+#pragma unroll 4
+        for (int i = i0; i < end; ++i) {
+            const float v = __ldcg(a + i * sa);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (c < n) part[c] = fmaf(v, __ldcg(b + i * sb + c * sc), part[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] += part[c];
+    }
+}
+// The outputs of this CTA (its share of the tile's units of 8 rows x 16 columns) from the operands in global memory,
+// by the definition of the product.  Rare and therefore plain: a lane sums one row's four columns.  The test for it
+// and the factor cost 1-2 % (training step of 2048 rows, 512 -> 128 -> 2048, cold L2: 73.2 -> 74.3 us; convolutions up to
+// 4 %: 32 x 28 x 28, 128 -> 32 -> 128, 176 -> 180 us); with a NaN in every row that linear step takes 1.8 ms.
+// (A second pass over the ring by the same roles was slower where nothing is repaired: 83 us.)
+template <int BN, int kMode>
+__device__ __noinline__ void f32_repair(const F32Params& p, int bx, int by, int bz) {
+    constexpr int kUnits = 16 * (BN / 16);
+    const F32Origin org = f32_origin<kMode>(p, bx);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, per = (kUnits + p.splits - 1) / p.splits, end = min(kUnits, (bz + 1) * per);
+    const int s = p.cv_stride;
+    const long long C = p.cv_C, R = p.cv_R;
+#pragma unroll 1
+    for (int u = bz * per + warp; u < end; u += kF32Threads / 32) {
+        const int oct = u / (BN / 16), row = f32_row<kMode>(p, org, bx, oct * 8 + (lane & 7));
+        const int col = by * BN + (u - oct * (BN / 16)) * 16 + (lane >> 3) * 4, n = min(4, p.N - col);
+        if (row < 0 || n <= 0) continue;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        if constexpr (kMode == 0) {
+            repair_run(p.A + (p.a_mn ? row : row * p.lda), p.a_mn ? p.lda : 1, p.B + (p.b_mn ? col : col * p.ldb), p.b_mn ? p.ldb : 1,
+                       p.b_mn ? 1 : p.ldb, p.K, n, acc);
+        } else if constexpr (kMode == 2) {          // rows (tap, channel), contraction over the output pixels
+            const int tap = row / p.cv_C, ta = tap / p.cv_kw, dx = tap - ta * p.cv_kw - p.cv_pad, dy = ta - p.cv_pad;
+            const int w0 = dx >= 0 ? 0 : (s - 1 - dx) / s, w1 = min(p.out_w, (p.cv_W - 1 - dx + s) / s);
+#pragma unroll 1
+            for (int i = 0; i < p.cv_N * p.out_h; ++i) {
+                const int img = i / p.out_h, h = (i - img * p.out_h) * s + dy;
+                if (h < 0 || h >= p.cv_H || w0 >= w1) continue;
+                repair_run(p.A + ((static_cast<long long>(img) * p.cv_H + h) * p.cv_W + w0 * s + dx) * C + (row - tap * p.cv_C), s * C,
+                           p.B + (static_cast<long long>(i) * p.out_w + w0) * R + col, R, 1, w1 - w0, n, acc);
+            }
+        } else {                                    // rows are pixels, contraction over (tap, channel or rank)
+            const int w = row % p.out_w, t = row / p.out_w, img = t / p.out_h, h = t - img * p.out_h;
+#pragma unroll 1
+            for (int tap = 0; tap < p.cv_kh * p.cv_kw; ++tap) {
+                const int ta = tap / p.cv_kw, tb = tap - ta * p.cv_kw;
+                int y = h * s - p.cv_pad + ta, x = w * s - p.cv_pad + tb;
+                if constexpr (kMode == 1) {         // A = dT: the output pixel that this tap takes from the input pixel
+                    y = h + p.cv_pad - ta; x = w + p.cv_pad - tb;
+                    if (y < 0 || x < 0 || y % s != 0 || x % s != 0) continue;
+                    y /= s; x /= s;
+                }
+                if (y < 0 || x < 0 || y >= p.cv_H || x >= p.cv_W) continue;
+                const long long pix = (static_cast<long long>(img) * p.cv_H + y) * p.cv_W + x;
+                if constexpr (kMode == 1) repair_run(p.A + pix * R, 1, p.B + (tap * C + col) * R, 1, R, p.cv_R, n, acc);
+                else repair_run(p.A + pix * C, 1, p.B + tap * C * R + col, R, 1, p.cv_C, n, acc);
+            }
+        }
+        for (int c = 0; c < n; ++c) {
+            float v = acc[c] + (p.bias ? p.bias[col + c] : 0.f);
+            if (p.act == 1) v = fmaxf(v, 0.f);
+            p.C[static_cast<size_t>(row) * p.ldc + col + c] = v;
+            if (p.C2) p.C2[static_cast<size_t>(row) * p.ldc2 + col + c] = v;
+        }
+    }
+}
+
 template <int BN, int kMode>
 __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorMap& tmB, const F32Params& p, const int bx, const int by,
                                          const int bz) {
@@ -223,7 +310,7 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
     const uint32_t planes_b = smem_u32(smem + 1024);      // three planes of B (A's are in tensor memory)
     constexpr uint32_t kTmemA = 3 * BN;                   // after two main accumulators and the correction's: two half buffers
     const uint32_t ring = planes_b + 3 * kPlaneB;
-    volatile uint32_t* abort_flag = &ctl->abort;
+    volatile uint32_t *abort_flag = &ctl->abort, *repair = &ctl->repair;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n0 = by * BN;
     const F32Origin org = f32_origin<kMode>(p, bx);
@@ -247,6 +334,7 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
         mbar_init(smem_u32(&ctl->corr_full), 1);
         ctl->abort = 0;
         ctl->fix_ok = 0;
+        ctl->repair = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
         tma_prefetch_desc(&tmA);
@@ -511,16 +599,18 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
                     if (col + 2 < p.N) b.z = __ldg(p.bias + col + 2);
                     if (col + 3 < p.N) b.w = __ldg(p.bias + col + 3);
                 }
+                float probe = 0.f;        // becomes NaN with a sum that is not finite
 #pragma unroll 4
                 for (int i = 0; i < 32 / kRowsPer; ++i) {
                     const int rr = i * kRowsPer + sub;
                     const uint4 u = ld_shared_v4(panel + static_cast<uint32_t>(rr) * kRowBytes +
                                                  ((static_cast<uint32_t>(piece) ^ (static_cast<uint32_t>(rr) & (kPieces - 1))) << 4));
-                    float4 v = make_float4(__uint_as_float(u.x) + b.x, __uint_as_float(u.y) + b.y, __uint_as_float(u.z) + b.z,
-                                           __uint_as_float(u.w) + b.w);
-                    if (p.act == 1) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+                    float4 v = make_float4(fmaf(__uint_as_float(u.x), kUnscale, b.x), fmaf(__uint_as_float(u.y), kUnscale, b.y),
+                                           fmaf(__uint_as_float(u.z), kUnscale, b.z), fmaf(__uint_as_float(u.w), kUnscale, b.w));
                     const int row = f32_row<kMode>(p, org, bx, q * 32 + rr);
                     if (row < 0) continue;
+                    probe = fmaf(__uint_as_float(u.x), 0.f, fmaf(__uint_as_float(u.y), 0.f, fmaf(__uint_as_float(u.z), 0.f, fmaf(__uint_as_float(u.w), 0.f, probe))));
+                    if (p.act == 1) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
                     float* dst = p.C + static_cast<size_t>(row) * p.ldc + col;
                     if (vec && col + 3 < p.N) {
                         *reinterpret_cast<float4*>(dst) = v;
@@ -538,13 +628,17 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
                         if (col + 3 < p.N) d2[3] = v.w;
                     }
                 }
+                if (probe != 0.f) *repair = 1u;
             }
         }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
-    if (p.splits <= 1) return;
+    if (p.splits <= 1) {
+        if (*repair) f32_repair<BN, kMode>(p, bx, by, bz);
+        return;
+    }
 
     // ---- slice sum (as in pf_tc_gemm_kernel.cuh): once all slices of the tile are in the workspace, each CTA adds its
     // share of them in slice order and stores the sums
@@ -588,6 +682,8 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
             }
             const int row = f32_row<kMode>(p, org, bx, rr), col = n0 + cq * kCols + pc * 4;
             if (row < 0) continue;
+            if (fmaf(a.x, 0.f, fmaf(a.y, 0.f, fmaf(a.z, 0.f, a.w * 0.f))) != 0.f) *repair = 1u;
+            a = make_float4(a.x * kUnscale, a.y * kUnscale, a.z * kUnscale, a.w * kUnscale);
             const float v[4] = {a.x, a.y, a.z, a.w};
             float* dst = p.C + static_cast<size_t>(row) * p.ldc + col;
             if (vec && col + 3 < p.N) *reinterpret_cast<float4*>(dst) = a;
@@ -608,6 +704,7 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
             __threadfence();
         }
     }
+    if (*repair) f32_repair<BN, kMode>(p, bx, by, bz);
 }
 
 // Up to three independent products in one launch, blocks [end[i - 1], end[i]) working on product i; kConv compiles the
