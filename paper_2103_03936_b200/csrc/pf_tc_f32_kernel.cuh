@@ -12,8 +12,11 @@
 // Accumulation.  A tcgen05.mma truncates when it adds to its fp32 accumulator (measured: -0.5 ulp per MMA on
 // sums of one sign), so long sums must not stay in tensor memory: the main products a1 b1 accumulate over 64
 // elements of the contraction in one of two accumulators, which the worker warps then add, with
-// round-to-nearest, to fp32 sums in their registers; the five correction products, 2^-8 of the sum, have an
-// accumulator of their own, added once at the end.  The result is as accurate as an fp32 FMA kernel.
+// round-to-nearest, to fp32 sums in their registers.  The five correction products, at most 2^-7 of the sum, have an
+// accumulator of their own for 512 elements: then a chunk's main products go on top of it, so that it is drained as
+// that chunk's accumulator, and the buffer they would have used takes the corrections from there on.  160 truncated
+// additions lose at most 160 ulps of that 2^-7th, 1.5e-7 of the sum, whatever its length; left to pile up over 32768
+// elements of one sign they lost 6.9e-6.  The result is as accurate as an fp32 FMA kernel.
 //
 // One CTA computes a 128 x BN tile of C = A * B or one slice of its contraction.  Warps: 0 = TMA producer of
 // A, 1 = tensor memory + MMA issue, 2..17 = workers (split the operands, drain the accumulators, epilogue),
@@ -82,6 +85,8 @@ constexpr int kF32Threads = 608;
 constexpr int kF32MaxStages = 8;
 constexpr int kChunk = 2;                    // k-blocks per main accumulator: 64 elements of the contraction
 static_assert(kChunk == 2, "one k-block per worker group and chunk");
+constexpr int kCorrChunks = 8;               // chunks per correction accumulator
+static_assert(kCorrChunks % 2 == 0, "it changes places with the accumulator of the odd chunks");
 constexpr uint32_t kF32TileA = 16384;        // 128 x 32 floats
 constexpr uint32_t kColsA = 16;              // tensor-memory columns of one plane of A's k-block (32 bf16 per row)
 
@@ -466,32 +471,43 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
             const uint32_t b_half = p.b_mn ? 256u : 4u;      // 16-byte units to half 1
             const uint32_t b_step = p.b_mn ? 128u : 2u;      // ... to the next 16 elements
             constexpr uint32_t pb = kPlaneB >> 4;
-            const uint32_t corr = tmem + 2 * BN;
             bool ok = true;
             int in_chunk = 0;
+            uint32_t odd = tmem + BN, corr = tmem + 2 * BN;      // accumulators of the odd chunks (the even ones': tmem) and of the corrections
+            uint32_t main_acc = 0, corr_acc = 0;          // 0: the next product starts the accumulator
             uint32_t buf = 0, bufph = 1;                  // phase of main_empty[buf]: the first use of each finds it free
             for (int i = 0; i < nkb; ++i) {
                 const uint32_t h = static_cast<uint32_t>(i) & 1u;
                 if (in_chunk == 0) {
                     ok = mbar_wait(smem_u32(&ctl->main_empty[buf]), bufph, abort_flag, p.status);
                     if (!ok) break;
+                    main_acc = 0;
+                    if ((i / kChunk) % kCorrChunks == kCorrChunks - 1) {      // on top of the corrections so far
+                        const uint32_t c = odd;
+                        odd = corr;
+                        corr = c;
+                        main_acc = 1;
+                        corr_acc = 0;
+                    }
                 }
                 ok = mbar_wait(smem_u32(&ctl->split_full[h]), static_cast<uint32_t>(i >> 1) & 1u, abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t b0 = b_desc0 + h * b_half;
-                const uint32_t a0 = tmem + kTmemA + h * (3 * kColsA), d = tmem + buf * BN;
+                const uint32_t a0 = tmem + kTmemA + h * (3 * kColsA);
+                const uint32_t d = buf ? odd : tmem;
 #pragma unroll
                 for (int ks = 0; ks < 2; ++ks) {
                     const uint64_t b = b0 + ks * b_step;
                     const uint32_t a = a0 + ks * 8u;
-                    tc_mma_bf16_ta(corr, a + 2 * kColsA, b, idesc, (i > 0 || ks > 0) ? 1u : 0u);
+                    tc_mma_bf16_ta(corr, a + 2 * kColsA, b, idesc, ks > 0 ? 1u : corr_acc);
                     tc_mma_bf16_ta(corr, a, b + 2 * pb, idesc, 1u);
                     tc_mma_bf16_ta(corr, a + kColsA, b + pb, idesc, 1u);
                     tc_mma_bf16_ta(corr, a + kColsA, b, idesc, 1u);
                     tc_mma_bf16_ta(corr, a, b + pb, idesc, 1u);
-                    tc_mma_bf16_ta(d, a, b, idesc, (in_chunk > 0 || ks > 0) ? 1u : 0u);
+                    tc_mma_bf16_ta(d, a, b, idesc, ks > 0 ? 1u : main_acc);
                 }
+                main_acc = corr_acc = 1;
                 tc_commit(smem_u32(&ctl->split_empty[h]));
                 if (++in_chunk == kChunk || i + 1 == nkb) {
                     tc_commit(smem_u32(&ctl->main_full[buf]));
@@ -522,12 +538,14 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
             for (int e = 0; e < kCols; ++e) acc[e] += __uint_as_float(v[e]);
         };
         bool ok = true;
+        uint32_t odd = BN;         // columns of the odd chunks' accumulator; the corrections have the other of BN and 2 BN
         auto drain = [&](int c) {
             const uint32_t b = static_cast<uint32_t>(c) & 1u;
             ok = mbar_wait_warp(smem_u32(&ctl->main_full[b]), static_cast<uint32_t>(c >> 1) & 1u, abort_flag, p.status);
             tc_fence_after();
             if (!ok) return;
-            add_from(lane_base + b * BN);
+            if (c % kCorrChunks == kCorrChunks - 1) odd = 3 * BN - odd;
+            add_from(lane_base + (b ? odd : 0u));
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl->main_empty[b]));
@@ -564,7 +582,7 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
             tc_fence_after();
         }
         if (ok) {
-            add_from(lane_base + 2 * BN);
+            add_from(lane_base + (3 * BN - odd));
             constexpr uint32_t kPieces = kCols / 4, kRowBytes = kCols * 4;
             if (p.splits > 1) {
                 // slice: straight to the workspace, [column quarter][quadrant][4-column group][row][4], a run of 512 bytes
