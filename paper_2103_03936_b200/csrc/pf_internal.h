@@ -114,7 +114,7 @@ cudaError_t bias_act_inplace(void* y, int64_t ld, int64_t rows, int64_t cols, co
                              cudaStream_t stream);
 
 // Copies to 16-byte aligned rows whose pitch is a multiple of 8 elements (the tail of a row's last 8 elements
-// is zeroed), up to six in one launch.  A job covers `groups` matrices gs_src elements apart (0 is one matrix),
+// is zeroed), all in one launch (up to six jobs and 2^31 - 1 pieces of 16 bytes, else in several).  A job covers `groups` matrices gs_src elements apart (0 is one matrix),
 // which land one after the other.
 struct RepackJob {
     const void* src;

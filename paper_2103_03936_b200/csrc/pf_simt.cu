@@ -6,6 +6,8 @@
 // and dU), or the gather form of the transposed convolution (dX).  Products accumulate in
 // fp32; a reduction split over K writes fp32 partials that a second kernel sums in a fixed
 // order, so results are bit-reproducible run to run.
+#include <algorithm>
+
 #include "pf_internal.h"
 
 namespace pf {
@@ -590,38 +592,66 @@ cudaError_t repack_rows_bf16(const void* src, int64_t ld_src, void* dst, int64_t
     return cudaGetLastError();
 }
 
+// One launch holds kRepackJobs runs of rows and counts its pieces in 32 bits; what is more goes into further launches.
 cudaError_t repack_rows_bf16_multi(const RepackJob* jobs, int count, cudaStream_t stream) {
-    if (count > kRepackJobs) return cudaErrorInvalidValue;
+    constexpr long long kMostPieces = 0x7fffffffLL;
     RepackBatchArgs a = {};
     long long total = 0;
+    auto launch = [&]() -> cudaError_t {
+        if (a.count == 0) return cudaSuccess;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(static_cast<unsigned>(ceil_div(total, 256) < 16 * num_sms() ? ceil_div(total, 256) : 16 * num_sms()));
+        cfg.blockDim = dim3(256);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, repack_multi_kernel, a);
+        if (e == cudaSuccess) count_launch();
+        a.count = 0;
+        total = 0;
+        return e;
+    };
+    // rows of one matrix or of `groups` matrices gs elements apart (0: one run of rows), `first` rows into the destination
+    auto add = [&](const RepackJob& j, const unsigned short* src, int64_t first, int64_t rows, int64_t groups, int64_t gs) {
+        const int k = a.count++;
+        a.src[k] = src;
+        a.dst[k] = static_cast<unsigned short*>(j.dst) + first * j.ld_dst;
+        a.ld_src[k] = j.ld_src; a.ld_dst[k] = j.ld_dst;
+        a.gs_src[k] = gs;
+        a.cols[k] = static_cast<int>(j.cols);
+        a.rows[k] = static_cast<int>(rows);
+        a.pieces_per_row[k] = static_cast<int>((j.cols + 7) / 8);
+        total += rows * groups * a.pieces_per_row[k];
+        a.item_end[k] = static_cast<unsigned int>(total);
+    };
     for (int i = 0; i < count; ++i) {
         const RepackJob& j = jobs[i];
-        const long long rows = j.rows * j.groups, pieces = (j.cols + 7) / 8;
-        if (rows <= 0 || j.cols <= 0) continue;
-        if (total + rows * pieces > 0x7fffffffLL) return cudaErrorInvalidValue;
-        const int k = a.count++;
-        a.src[k] = static_cast<const unsigned short*>(j.src);
-        a.dst[k] = static_cast<unsigned short*>(j.dst);
-        a.ld_src[k] = j.ld_src; a.ld_dst[k] = j.ld_dst;
-        a.gs_src[k] = j.groups > 1 && j.gs_src != j.rows * j.ld_src ? j.gs_src : 0;   // 0: one run of rows
-        a.cols[k] = static_cast<int>(j.cols);
-        a.rows[k] = static_cast<int>(j.rows);
-        a.pieces_per_row[k] = static_cast<int>(pieces);
-        total += rows * pieces;
-        a.item_end[k] = static_cast<unsigned int>(total);
+        const int64_t pieces = (j.cols + 7) / 8;
+        if (j.rows <= 0 || j.groups <= 0 || j.cols <= 0) continue;
+        if (pieces > kMostPieces) return cudaErrorInvalidValue;
+        const unsigned short* src = static_cast<const unsigned short*>(j.src);
+        const bool apart = j.groups > 1 && j.gs_src != j.rows * j.ld_src;
+        if (apart && a.count < kRepackJobs && total + j.rows * j.groups * pieces <= kMostPieces) {
+            add(j, src, 0, j.rows, j.groups, j.gs_src);
+            continue;
+        }
+        const int64_t runs = apart ? j.groups : 1, rows = apart ? j.rows : j.rows * j.groups;
+        for (int64_t g = 0; g < runs; ++g) {
+            for (int64_t r = 0; r < rows;) {
+                const int64_t n = a.count < kRepackJobs ? std::min<int64_t>(rows - r, (kMostPieces - total) / pieces) : 0;
+                if (n == 0) {
+                    const cudaError_t e = launch();
+                    if (e != cudaSuccess) return e;
+                    continue;
+                }
+                add(j, src + g * j.gs_src + r * j.ld_src, g * rows + r, n, 1, 0);
+                r += n;
+            }
+        }
     }
-    if (a.count == 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(ceil_div(total, 256) < 16 * num_sms() ? ceil_div(total, 256) : 16 * num_sms()));
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, repack_multi_kernel, a);
-    if (e == cudaSuccess) count_launch();
-    return e;
+    return launch();
 }
 
 }  // namespace pf

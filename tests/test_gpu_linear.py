@@ -293,3 +293,26 @@ def test_row_tiles_of_96(m, k, n, r):
     tiles, both directions, padded pitches."""
     run_case(wl.LinearCase("rows", m, k, n, r, wl.BF16, 29))
     run_case(wl.LinearCase("rows", m, k, n, r, wl.BF16, 30), ld_pad=8)
+
+
+def test_re_pitch_copies_beyond_two_to_the_31_pieces():
+    """Ragged operands of more than 2^31 pieces of 16 bytes are copied in several launches: 34 GB of zeros with a few small
+    integers around the seams, so that every result is exact."""
+    m, k, n = 4100, 4194297, 8
+    if torch.cuda.mem_get_info()[0] < 80 << 30:
+        pytest.skip("needs 80 GB of device memory")
+    x = torch.zeros((m, k), dtype=torch.bfloat16, device="cuda")
+    U = torch.randint(-3, 4, (k, n), device="cuda").to(torch.bfloat16)
+    V = torch.eye(n, dtype=torch.bfloat16, device="cuda")
+    want = torch.zeros((m, n), dtype=torch.bfloat16, device="cuda")
+    cols = torch.tensor([0, 1, 7, 8, 63, 64, k // 2, k - 9, k - 2, k - 1], device="cuda")
+    for row in (0, 1, 2047, 2048, 4094, 4095, 4096, 4099):
+        x[row, cols] = torch.randint(-3, 4, (len(cols),), device="cuda").to(torch.bfloat16)
+        want[row] = (x[row, cols].float() @ U[cols].float()).to(torch.bfloat16)
+    launches = pf.pf_launch_count()
+    y = pf.pf_lowrank_linear_fwd(x, U, V)
+    assert pf.pf_launch_count() - launches == 3
+    assert torch.equal(y, want)
+    assert pf.pf_last_device_status() == 0
+    del x, y
+    torch.cuda.empty_cache()
