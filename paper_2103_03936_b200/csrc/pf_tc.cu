@@ -69,14 +69,8 @@ unsigned run_blocks(int64_t tiles, int64_t kblocks_per_tile, int stride) {
 template <int BN>
 cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p, dim3 grid,
                         cudaStream_t stream) {
-    cudaError_t e;
-    if (p.conv_mode != 0) {
-        e = launch_gemm_conv(BN, grid, gemm_smem(BN, p.num_stages, p.conv_mode == 1), stream, ta, tb, p);
-    } else {
-        e = allow_smem(tc_gemm_kernel<BN, 0>, std::min(gemm_smem(BN, kMaxStages), static_cast<size_t>(227 * 1024)));
-        if (e == cudaSuccess)
-            e = launch_overlapped(tc_gemm_kernel<BN, 0>, grid, dim3(kGemmThreads), gemm_smem(BN, p.num_stages), stream, ta, tb, p);
-    }
+    cudaError_t e = allow_smem(tc_gemm_kernel<BN, false>, std::min(gemm_smem(BN, kMaxStages), static_cast<size_t>(227 * 1024)));
+    if (e == cudaSuccess) e = launch_overlapped(tc_gemm_kernel<BN, false>, grid, dim3(kGemmThreads), gemm_smem(BN, p.num_stages), stream, ta, tb, p);
     if (e == cudaSuccess) count_launch();
     return e;
 }
@@ -292,10 +286,9 @@ int launch_prepared(const GemmLaunch& g, cudaStream_t stream) {
 // `copy2` (optional): asks for a second copy of C at pitch ldc2; *copy2_done tells whether the launch
 // wrote it (the CTA-pair kernel cannot), else the caller copies C itself.
 int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
-         int splits, float* partial, cudaStream_t stream, const ConvA* cv = nullptr, void* copy2 = nullptr,
-         int64_t ldc2 = 0, bool* copy2_done = nullptr, const void* bias = nullptr, int act = 0) {
+         int splits, float* partial, cudaStream_t stream, void* copy2 = nullptr, int64_t ldc2 = 0, bool* copy2_done = nullptr, const void* bias = nullptr, int act = 0) {
     // wide, many-tile (tensor-bound) products run on CTA pairs, which halve the operand traffic per SM
-    if (!cv && splits <= 1 && pair_worthwhile(M, N, K)) {
+    if (splits <= 1 && pair_worthwhile(M, N, K)) {
         PairJob j{A.p, A.ld, A.mn_major, 0, B.p, B.ld, B.mn_major, 0, M, N, K, C, ldc};
         j.bias = bias;
         j.act = act;
@@ -306,8 +299,8 @@ int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, vo
         }
     }
     GemmLaunch g;
-    int st = gemm_prepare(A, B, M, N, K, C, ldc, splits, partial, cv, &g);
-    if (st == PF_ERR_UNSUPPORTED && splits > 1) st = gemm_prepare(A, B, M, N, K, C, ldc, 1, nullptr, cv, &g);
+    int st = gemm_prepare(A, B, M, N, K, C, ldc, splits, partial, nullptr, &g);
+    if (st == PF_ERR_UNSUPPORTED && splits > 1) st = gemm_prepare(A, B, M, N, K, C, ldc, 1, nullptr, nullptr, &g);
     if (st != PF_OK) return st;
     if (copy2_done) *copy2_done = false;
     if (copy2) {
@@ -520,10 +513,10 @@ int linear_fwd(const LinearArgs& a, int* handled) {
     } else {
         float* p1 = reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * pad8(a.r) * 2, 256));
         st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, T, ldT,
-                  pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream, nullptr,
+                  pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream,
                   (a.T && !stash_direct) ? a.T : nullptr, a.ldt, &stash_written);
         if (st != PF_OK) return st;
-        st = gemm({T, ldT, false}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, a.stream, nullptr, nullptr, 0, nullptr,
+        st = gemm({T, ldT, false}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, a.stream, nullptr, 0, nullptr,
                   a.bias, a.act);
     }
     if (st != PF_OK) return st;
@@ -997,7 +990,7 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         if (st != PF_OK) return st;
     }
     *handled = 1;
-    {   // both reductions are launched exactly as prepared (together or one by one)
+    {   // both reductions are launched exactly as prepared
         const GemmLaunch* gs[2] = {&gu, &gv};
         LinearArgs::Slices* outs[2] = {a.du_slices, a.dv_slices};
         for (int i = 0; i < 2; ++i) {
@@ -1017,16 +1010,8 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     // start first and the many short dX tiles fill the second CTA slot of every SM beside them.
     const GemmLaunch* list[3] = {&gu, &gv, &gx};
     if (gu.p.splits <= 1 && gv.p.splits > 1) { list[0] = &gv; list[1] = &gu; }
-    st = gemm_multi(list, a.dX ? 3 : 2, a.stream);
-    if (st != PF_ERR_UNSUPPORTED) return st;
-    // separate launches (tile widths that cannot share one)
-    if (a.dX) {
-        st = launch_prepared(gx, a.stream);
-        if (st != PF_OK) return st;
-    }
-    st = launch_prepared(gu, a.stream);
-    if (st != PF_OK) return st;
-    return launch_prepared(gv, a.stream);
+    // (never declined: R <= 384 keeps the tiles at most 128 columns wide, and conv_splits fits the slices of both.)
+    return gemm_multi(list, a.dX ? 3 : 2, a.stream);
 }
 
 }  // namespace tc

@@ -1,5 +1,5 @@
-// The product kernels of pf_tc_gemm_kernel.cuh as the convolution's backward needs them (implicit-GEMM operands), in
-// a translation unit of their own so that the plain kernels keep a module without them.
+// The shared launch of pf_tc_gemm_kernel.cuh as the convolution's backward needs it (implicit-GEMM operands), in a
+// translation unit of its own so that the plain kernels keep a module without it.
 #include "pf_tc.h"
 
 #include "pf_tc_gemm_kernel.cuh"
@@ -7,21 +7,6 @@
 
 namespace pf {
 namespace tc {
-
-namespace {
-template <int BN, int kMode>
-cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p) {
-    const cudaError_t e = allow_smem(tc_gemm_kernel<BN, kMode>, 227 * 1024);
-    return e != cudaSuccess ? e : launch_overlapped(tc_gemm_kernel<BN, kMode>, grid, dim3(kGemmThreads), smem, stream, ta, tb, p);
-}
-}  // namespace
-
-cudaError_t launch_gemm_conv(int bn, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb,
-                             const GemmParams& p) {
-    if (bn > 128) return cudaErrorInvalidValue;
-    if (p.conv_mode == 1) return bn == 64 ? launch_one<64, 1>(grid, smem, stream, ta, tb, p) : launch_one<128, 1>(grid, smem, stream, ta, tb, p);
-    return bn == 64 ? launch_one<64, 2>(grid, smem, stream, ta, tb, p) : launch_one<128, 2>(grid, smem, stream, ta, tb, p);
-}
 
 cudaError_t launch_gemm3_conv(int blocks, size_t smem, cudaStream_t stream, const Gemm3Args& a) {
     const cudaError_t e = allow_smem(tc_gemm3_kernel<true>, 227 * 1024);

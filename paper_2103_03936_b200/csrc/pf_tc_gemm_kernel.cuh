@@ -6,7 +6,8 @@
 //   tc_gemm3_kernel     up to three such products in one launch.
 // Warp roles: warp 0 = TMA producer of operand A, warp 1 = TMEM allocation + MMA issue, warps 2..5 =
 // epilogue (each owns the 32 TMEM lanes of its warp-id quadrant), warp 6 = TMA producer of operand B.
-// The plain products are instantiated in pf_tc.cu, those of the convolution in pf_tc_conv.cu.
+// The plain products are instantiated in pf_tc.cu, several tiles per block in pf_tc_runs.cu, the convolution's in
+// pf_tc_conv.cu.
 #ifndef PF_TC_GEMM_KERNEL_CUH_
 #define PF_TC_GEMM_KERNEL_CUH_
 
@@ -61,10 +62,8 @@ struct GemmParams {
     long long c_gstride;
 };
 
-// Launches of the convolution instantiations (pf_tc_conv.cu); same arguments as the kernels.
+// Launches of the instantiations that have translation units of their own (pf_tc_runs.cu, pf_tc_conv.cu).
 cudaError_t launch_gemm_runs(int bn, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb,
-                             const GemmParams& p);
-cudaError_t launch_gemm_conv(int bn, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb,
                              const GemmParams& p);
 struct Gemm3Args {
     CUtensorMap ta[3], tb[3];
@@ -771,17 +770,15 @@ __device__ __forceinline__ void run_tiles(const CUtensorMap& tmA, const CUtensor
     if (warp == 1) tmem_dealloc(tmem_base, 2 * BN);
 }
 
-template <int BN, int kMode>
+template <int BN, bool kRuns>
 __global__ void __launch_bounds__(kGemmThreads, BN <= 128 ? 2 : 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const GemmParams p) {
-    if constexpr (kMode == 1) {
-        run_tiles<BN, 1>(tmA, tmB, p, blockIdx.x, gridDim.x);
-    } else if constexpr (kMode == 3) {
+    if constexpr (kRuns) {
         run_tiles<BN, 0>(tmA, tmB, p, blockIdx.x, gridDim.x);
     } else {
         const int sl = p.splits < 1 ? 1 : p.splits;
-        gemm_tile<BN, kMode>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
+        gemm_tile<BN, 0>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
     }
 }
 
