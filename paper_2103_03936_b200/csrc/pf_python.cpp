@@ -193,7 +193,11 @@ PyObject* tuple(std::initializer_list<at::Tensor> ts) {
     for (const at::Tensor& t : ts) PyTuple_SET_ITEM(out, i++, wrap(t));
     return out;
 }
-bool truth(PyObject* o) { return PyObject_IsTrue(o) == 1; }
+bool truth(PyObject* o) {
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw python_error();
+    return v == 1;
+}
 int64_t integer(PyObject* o) {
     const long long v = PyLong_AsLongLong(o);
     if (v == -1 && PyErr_Occurred()) throw python_error();

@@ -137,6 +137,17 @@ def test_pack_host_side_contract(L):
     assert L.pf_pack_factor_grads(ptrs, zeros, 3, 1, None, 0, offs, None, 0, None) == OK
 
 
+def test_an_argument_whose_truth_value_raises():
+    """The caller sees the error of a flag that has no truth value, not a call that took it as false."""
+    class Undecided:
+        def __bool__(self):
+            raise LookupError("undecided")
+
+    import torch
+    with pytest.raises(LookupError, match="undecided"):
+        pf.pf_pack_factor_grads([torch.zeros(4)], prepare=Undecided())
+
+
 def test_binding_raises_when_library_is_missing(monkeypatch, tmp_path):
     """No fallback: a missing library is an ImportError, not a silent slow path."""
     from paper_2103_03936_b200 import binding
