@@ -15,6 +15,7 @@ CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpf.so")
 NATIVE = os.path.join(PKG, "_pf_native.so")
+NATIVE_KEY = os.path.join(OBJ, "_pf_native.key")      # what _pf_native.so was built against
 SOURCES = ["pf_api.cu", "pf_simt.cu", "pf_small.cu", "pf_pack.cu", "pf_tc.cu", "pf_tc_conv.cu", "pf_tc_runs.cu", "pf_tc_conv_res.cu", "pf_tc_chain.cu", "pf_tc_chain_multi.cu", "pf_tc_chain_act.cu", "pf_tc_chain_conv.cu", "pf_tc_pair.cu", "pf_tc_f32.cu", "pf_tc_f32_conv.cu", "pf_static.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
 
@@ -55,9 +56,22 @@ def _build_lib(force: bool, verbose: bool) -> None:
     os.replace(tmp, LIB)
 
 
+def _torch_abi() -> int:
+    import torch
+    return int(torch.compiled_with_cxx11_abi())
+
+
+def _native_key() -> str:
+    """The torch, its C++ ABI and the Python that a built module fits."""
+    import torch
+    return f"torch {torch.__version__}, cxx11 abi {_torch_abi()}, {sys.implementation.cache_tag}"
+
+
 def _build_native(force: bool) -> None:
     src = os.path.join(CSRC, "pf_python.cpp")
-    if not force and _mtime(NATIVE) > _newest([src, os.path.join(ROOT, "include", "pf.h")]):
+    key = _native_key()
+    built_for = open(NATIVE_KEY).read() if os.path.exists(NATIVE_KEY) else ""
+    if not force and built_for == key and _mtime(NATIVE) > _newest([src, os.path.join(ROOT, "include", "pf.h")]):
         return
     torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
@@ -65,11 +79,14 @@ def _build_native(force: bool) -> None:
     includes = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
                 os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     subprocess.check_call(
-        [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=1", "-o", tmp, src] +
+        [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={_torch_abi()}", "-o", tmp, src] +
         [a for d in includes for a in ("-isystem", d)] +
         ["-I", os.path.join(ROOT, "include"), "-L", os.path.join(torch_dir, "lib"), "-L", PKG, "-l:libpf.so", "-ltorch_python", "-ltorch_cuda",
          "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN"])
     os.replace(tmp, NATIVE)
+    os.makedirs(OBJ, exist_ok=True)
+    with open(NATIVE_KEY, "w") as f:
+        f.write(key)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -137,6 +137,25 @@ def test_pack_host_side_contract(L):
     assert L.pf_pack_factor_grads(ptrs, zeros, 3, 1, None, 0, offs, None, 0, None) == OK
 
 
+@pytest.mark.parametrize("change,rebuilt", [(None, False), ("_native_key", True), ("_torch_abi", True)])
+def test_binding_is_rebuilt_for_another_torch(L, monkeypatch, tmp_path, change, rebuilt):
+    """A module built against another torch, Python or C++ ABI is not taken as current."""
+    (tmp_path / "key").write_text(pf_build._native_key())
+    monkeypatch.setattr(pf_build, "NATIVE_KEY", str(tmp_path / "key"))
+    if change == "_native_key":
+        monkeypatch.setattr(pf_build, "_native_key", lambda: "torch 0.0")
+    elif change == "_torch_abi":
+        other = 1 - pf_build._torch_abi()
+        monkeypatch.setattr(pf_build, "_torch_abi", lambda: other)
+    calls = []
+    monkeypatch.setattr(pf_build.subprocess, "check_call", calls.append)
+    monkeypatch.setattr(pf_build.os, "replace", lambda a, b: None)
+    pf_build._build_native(False)
+    assert bool(calls) == rebuilt
+    if calls:
+        assert f"-D_GLIBCXX_USE_CXX11_ABI={pf_build._torch_abi()}" in calls[0]
+
+
 def test_an_argument_whose_truth_value_raises():
     """The caller sees the error of a flag that has no truth value, not a call that took it as false."""
     class Undecided:
