@@ -91,8 +91,8 @@ def test_multi_tile(dtype, N, H, W, C, R, O):
                                            (2, 16, 16, 128, 256, 64, 3), (2, 16, 16, 128, 320, 128, 3),
                                            (2, 16, 16, 128, 384, 72, 3)])
 def test_tensor_core_envelope(N, H, W, C, R, O, k):
-    """Shapes inside the implicit-GEMM tensor-core envelope (stride 1, 'same' padding, C % 128 == 0,
-    R % 64 == 0, image rows packing into 128- and 64-pixel tiles), with and without stash / dX.  The
+    """Stride-1, 'same'-padded shapes whose channels fill the 64-channel blocks of the implicit GEMMs and whose image rows
+    pack into 128- and 64-pixel tiles (other tilings: below), with and without stash / dX.  The
     ranks 256, 320 and 384 reach the parts of the fused kernel that only ranks above 192 use (a
     second group of first-product MMAs, the short ring, store staging inside the ring stages)."""
     run_conv(wl.ConvCase("tc", N, H, W, C, R, O, wl.BF16, 63, kh=k, kw=k, pad=(k - 1) // 2))
@@ -158,11 +158,11 @@ def test_empty_batch():
 
 
 @pytest.mark.parametrize("dtype,N,H,W,C,R,O,stride", [(wl.BF16, 4, 16, 16, 128, 64, 128, 1), (wl.BF16, 2, 8, 8, 24, 8, 16, 2),
-                                                      (wl.F32, 2, 8, 8, 16, 8, 24, 1)])
+                                                      (wl.BF16, 2, 8, 8, 20, 6, 12, 2), (wl.F32, 2, 8, 8, 16, 8, 24, 1)])
 def test_conv_grads_fp32_and_accumulated(dtype, N, H, W, C, R, O, stride):
     """pf_lowrank_conv_bwd_ex: fp32 factor gradients reproduce the plain call when rounded (same sums),
     and accumulation over two halves of the batch gives the whole batch's gradient on top of the
-    previous contents; tensor-core envelope, FMA kernels (stride 2), fp32 storage."""
+    previous contents; tensor cores at both strides, FMA kernels (channels that are no multiples of 8), fp32 storage."""
     c = wl.ConvCase("cg", N, H, W, C, R, O, dtype, 71, stride=stride)
     d = c.generate()
     x, U, V, dY = (dev(d[k_], dtype) for k_ in ("x", "U", "V", "dY"))
@@ -190,7 +190,7 @@ def test_conv_grads_fp32_and_accumulated(dtype, N, H, W, C, R, O, stride):
 def test_stride2_forward_on_tensor_cores(N, H, W, C, R, O):
     """Stride-2 3 x 3 convolutions (the first convolution of a ResNet stage): the forward runs on the fused
     tensor-core kernel with image tiles fetched two pixels apart (one launch; even and odd image sizes,
-    output rows that do not fill a tile, more tiles than SMs); the backward runs on the FMA kernels."""
+    output rows that do not fill a tile, more tiles than SMs), and the backward on the tensor cores too."""
     c = wl.ConvCase("s2", N, H, W, C, R, O, wl.BF16, 81, stride=2)
     d = c.generate()
     x, U, V = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V"))
