@@ -303,7 +303,7 @@ int forward(const tc::LinearArgs& a, void* T, int64_t ldt) {
 
 bool linear_fwd_fits(int64_t m, int64_t k, int64_t n, int64_t r) {
     // beyond about 2^26 multiplications the 128-row tiles win (4096 x 4096, r 256: 11.2 against 13.0 us at 20 rows, 15.0
-    // against 13.1 at 32), beyond 2^27 where they need re-pitch copies; up to 8 rows never
+    // against 13.1 at 32; caches warm), beyond 2^27 where they need re-pitch copies; up to 8 rows never
     const int64_t most = (k % 8 || r % 8) ? 1LL << 27 : 1LL << 26;
     return m >= 1 && m <= 32 && k <= (1 << 24) && n <= (1 << 24) && r <= (1 << 16) && out_smem(m, r) <= 190 * 1024 &&
            (m <= 8 || m * (k + n) * r < most);
@@ -323,7 +323,7 @@ int linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt) {
 // The smallest fp32 layers (a few million multiplications per product) are all latency: the split-operand tensor-core
 // kernel needs 6 us a launch for them (set-up, ring fill, splitting, drains).  Here a CTA computes a 16 x 32 tile of
 // C with plain FMAs: all loads of 128 elements of the contraction are in flight at once, the next 128 while these
-// are multiplied.  64 x 256 -> 256 at r 32, forward + backward: 25.8 -> 17.1 us.
+// are multiplied.  64 x 256 -> 256 at r 32, forward + backward: 25.8 -> 17.1 us (back to back, caches warm).
 namespace {
 
 constexpr int kF32Chunk = 128;
@@ -419,7 +419,8 @@ int f32_run(const F32Product& a, const F32Product* b, cudaStream_t stream) {
 }  // namespace
 
 // Every product short (its contraction in two loads) and small.  Beyond, the tensor cores are as fast or faster
-// (128 x 512 -> 512, r 64: 13.7 + 15.2 against 13.4 + 15.4 us; 512 x 512 -> 512, r 32: 14.0 against 16.4).
+// (128 x 512 -> 512, r 64: 13.7 + 15.2 against 13.4 + 15.4 us; 512 x 512 -> 512, r 32: 14.0 against 16.4;
+// caches warm).
 bool f32_fits(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd) {
     const int64_t longest = std::max({k, r, bwd ? std::max(n, m) : int64_t{1}});
     return longest <= 256 && n <= 4096 && m <= 4096 && m * r * std::max(k, n) <= (1 << 21);

@@ -57,7 +57,8 @@ int pick_stages(int bn, int64_t ctas, bool dx = false) {
 
 // Blocks that share the tiles of a convolution's dX: runs of about 16 k-blocks hide the start of a block (2 tiles of a
 // stride-1 layer, 8 of a strided one, whose tiles are short), longer ones make the blocks of the launch unequal
-// (32 x 56 x 56, 64 -> 16 -> 64 with 6 tiles per block: 61 us instead of 56); every SM gets a block first.
+// (backward of 32 x 56 x 56, 64 -> 16 -> 64 with 6 tiles per block: 61 us instead of 56, cold L2); every SM gets a
+// block first.
 // The tiles of a block are that many blocks apart: no multiple of the stride's factors, so that it gets every class.
 unsigned run_blocks(int64_t tiles, int64_t kblocks_per_tile, int stride) {
     const int64_t want = std::min<int64_t>(8, std::max<int64_t>(2, ceil_div(16, std::max<int64_t>(1, kblocks_per_tile))));

@@ -87,7 +87,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     // path, so SMs that 128-row tiles leave idle take some of them (the idle MMA rows cost nothing).  Not where the output
     // columns are split (148 instead of 128 blocks of an FFN layer delay the next launch's start: training step 1-3 %
     // slower), and not where another launch counts on the idle SMs (max_split).  Forward, 12000 rows, 768 -> 96 -> 3072:
-    // 29.2 -> 25.1 us (125 blocks instead of 94).  112 rows would help 16384-row layers by 1-2 % (147 blocks instead of 128),
+    // 29.2 -> 25.1 us (125 blocks instead of 94; caches warm, 30.7 with a cold L2).  112 rows would help 16384-row layers by 1-2 % (147 blocks instead of 128),
     // but need output boxes of 16 rows, which slowed the 128-row tiles as much.
     if (!conv && out && max_split <= 0 && plan.nsplit == 1 && ceil_div(M, 96) <= num_sms()) rows_tile = 96;
     if (!conv) plan.row_tiles = static_cast<int>(ceil_div(M, rows_tile));

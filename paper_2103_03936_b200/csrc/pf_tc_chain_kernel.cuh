@@ -5,24 +5,25 @@
 //   backward  dX = (dY V) U^T      A = dY, B1 = V [n, r],  B2 = U [k, r]
 // of the factorized linear layer.
 //
-// One CTA owns one 128-row tile of A (and a contiguous range of 128-column output tiles when the
+// One CTA owns one tile of 128 (or 96) rows of A (and a contiguous range of 128-column output tiles when the
 // grid splits N2 to fill the machine; each split then recomputes the intermediate).
 //   phase 1  T = A * B1: TMA ring over K1 in 64-element blocks; A tile is a K-major operand,
 //            the B1 tile [64 x r] is an MN-major operand (r contiguous in memory); fp32
 //            accumulator of r columns in TMEM.
-//   switch   the four epilogue warps read T from TMEM, round to bf16 and lay it out in shared
+//   switch   the eight epilogue warps read T from TMEM, round to bf16 and lay it out in shared
 //            memory as the K-major (128-byte swizzled) A operand of phase 2; the same bytes are
 //            what TMA stores as the stash.
 //   phase 2  for each 128-column tile: out_tile = T * B2_tile^T with B2 tiles streamed through
-//            the same ring; accumulators double-buffered in TMEM so the MMAs of tile j+1 overlap
-//            the epilogue of tile j; the epilogue stages bf16 rows in swizzled shared memory and
+//            the same ring; four accumulators in TMEM so the MMAs of the next tiles overlap the
+//            epilogue of tile j; the epilogue stages bf16 rows in swizzled shared memory and
 //            writes them with TMA stores (coalesced, clipped at the matrix edge).
-// When there are more row tiles than SMs (and r <= 128) the kernel is persistent: a CTA walks over row
-// tiles blockIdx.x, blockIdx.x + gridDim.x, ...; the producers run ahead into the next tile's phase 1
-// while the epilogue warps still convert and store the outputs of the current one, and the phase-2
-// accumulators then live beside T's in tensor memory (128 + 3 x 128 columns) instead of on top of it.
+// When there are more row tiles than SMs (and r <= 128) the grid is persistent, in the form of pf_tc_chain_pipe.cuh
+// or, with the bias / activation epilogue, in this kernel's multi-tile form: a CTA walks over row tiles
+// blockIdx.x, blockIdx.x + gridDim.x, ...; the producers run ahead into the next tile's phase 1 while the
+// epilogue warps still convert and store the outputs of the current one, and the phase-2 accumulators
+// then live beside T's in tensor memory (128 + 3 x 128 columns) instead of on top of it.
 // Shared memory: control block | T (r_pad x 256 B) | ring of stages (16 KB A or B2 tile + r_pad x
-// 128 B B1 tile).  In phase 2 the B1 part of every stage is idle and serves as store staging.
+// 128 B B1 tile) | store staging (r <= 128; for larger ranks the B1 part of every stage, idle in phase 2, serves as that).
 // This header holds the kernel (a template, instantiated in several translation units: the single-tile
 // form in pf_tc_chain.cu, the forms with a bias / activation epilogue in pf_tc_chain_act.cu, the convolution in
 // pf_tc_chain_conv.cu, so that each lives in a module of its own) and the parameter block the host fills.

@@ -499,7 +499,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     // fences between the proxies and a bulk copy back, which together took 6.3 us from the last MMA to the stored sum
     // (7 slices of 128 x 128).  Backward of 8192 rows, 512 -> 128 -> 2048: 24.6 -> 22.6 us; 1070 rows, 888 -> 208 ->
     // 3552: 28.0 -> 26.3.  One version of short code: it runs once, from a cold instruction cache, and variants per slice
-    // count with deeper unrolling lost up to 5 us.  (Half the loads in flight: 24.2 and 28.8 us.)
+    // count with deeper unrolling lost up to 5 us.  (Half the loads in flight: 24.2 and 28.8 us.)  All of these back to
+    // back on one set of buffers, caches warm; with a cold L2 the two take 33.8 and 31.7 us.
     unsigned int* cnt = p.counters + 2 * tile;
     const int S = p.splits;
     if (threadIdx.x == 0) {
@@ -586,7 +587,8 @@ __device__ __forceinline__ int run_tile(const GemmParams& p, int t, int* by) {
 // start, the first loads and the epilogue cost as much as the products.  Here the producers run on into the next tiles
 // while the epilogue warps store the last one from the other of two accumulators.  What bounds it now is the SM's load
 // path.  Whole backward, one tile per block -> runs: 128 x 32 x 32, 128 -> 64 -> 256, stride 2: 42 -> 34 us; 128 x 16 x 16,
-// 512 -> 128 -> 512: 114 -> 91 (against 256-column tiles); 128 x 32 x 32, 256 -> 64 -> 256: 122 -> 117. 
+// 512 -> 128 -> 512: 114 -> 91 (against 256-column tiles); 128 x 32 x 32, 256 -> 64 -> 256: 122 -> 117 (back to back,
+// caches warm, dT still one tile per block; with its runs 30.7, 90.5 and 114.6, with a cold L2 39.9, 101 and 128).
 template <int BN, int kMode>
 __device__ __forceinline__ void run_tiles(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, const int first, const int step) {
     constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2, kStageBytes = kABytes + kBBytes;

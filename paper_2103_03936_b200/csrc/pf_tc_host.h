@@ -31,9 +31,10 @@ inline EncodeTiledFn encode_fn() {
 }
 
 // Encoding a tensor map costs a driver call of one to two microseconds, and a training step issues the
-// same maps over and over, so encoded maps are kept in a small cache keyed by everything the encoding depends
-// on (the map holds no data, only addresses and shapes).  Four ways per set: a step uses some dozens of maps,
-// and with a direct-mapped cache a colliding pair was encoded anew on every call.
+// same maps over and over, so encoded maps are kept in a small cache, one for each kind of map (the template is
+// instantiated once for each `make`), keyed by everything the encoding depends on (the map holds no data, only
+// addresses and shapes).  Four ways per set: a step uses some dozens of maps, and with a direct-mapped cache a
+// colliding pair was encoded anew on every call.
 struct MapKey {
     const void* p;
     int64_t v[8];
