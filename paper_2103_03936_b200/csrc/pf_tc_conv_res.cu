@@ -15,7 +15,8 @@
 //
 // Forward: T = taps(x, U), then per 128 output channels y = T V^T with T (bf16) in shared memory; software-pipelined:
 // the first product of tile t + 1 is issued before the second of tile t.  What bounds it now is shared-memory
-// bandwidth (a 128 x 64 x 16 MMA reads 6 KB in 48 clocks).  128 x 32 x 32, 256 -> 64 -> 256: 65.5 -> 55.3 us;
+// bandwidth (a 128 x 64 x 16 MMA reads 6 KB in 48 clocks; at 128 x 32 x 32 the MMAs' reads take 63 % of the data pipe's
+// cycles and the epilogue's accesses 25 %, the tensor pipe is busy 35 %).  128 x 32 x 32, 256 -> 64 -> 256: 65.5 -> 55.3 us;
 // 256 x 14 x 14: 37.8 -> 30.6; 32 x 56 x 56, 64 -> 16 -> 64: 32.3 -> 19.5 (back to back, caches warm, images after
 // max(0, .); with a cold L2 60.4, 35.8 and 25.6).
 //

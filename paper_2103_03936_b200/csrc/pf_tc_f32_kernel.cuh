@@ -26,12 +26,13 @@
 // of waits and shared-memory round trips of about 1 us for a warp whatever it computes.
 // Splitting on chip rather than in a pass of its own: no workspace, no extra launch, 32 KB of loads per
 // k-block instead of 48 KB.
-// What bounds it is shared-memory bandwidth: an MMA that takes both operands from shared memory reads 128
-// bytes per clock, all there is, while TMA writes and the workers read and write the tiles.  So the planes of
-// A go to TENSOR memory (a thread splits 16 contraction elements of its row, whatever the operand's
+// An MMA that takes both operands from shared memory reads 128 bytes per clock, all there is, while TMA writes and the
+// workers read and write the tiles.  So the planes of A go to TENSOR memory (a thread splits 16 contraction elements of its row, whatever the operand's
 // orientation) and only B's planes, shared by all rows, to shared memory: 136 KB instead of 208 KB through
 // shared memory per k-block of a 128 x 128 tile.  A k-block takes 0.95 us with all SMs at work (0.67 us of a 128 x 64
-// tile), of which the MMAs are 0.4; a contraction of 4096 against one of 2048, caches warm.
+// tile), of which the MMAs are 0.4; a contraction of 4096 against one of 2048, caches warm.  What bounds it is that
+// chain of waits: on 18944 x 4096 -> 128 the tensor pipe is busy 40 % of the time, the shared-memory data pipe 54 %
+// (21 MMAs, 33 workers), the issue slots 58 %; in a step of 2048 x 512 -> 128 -> 2048 all of them less.
 #ifndef PF_TC_F32_KERNEL_CUH_
 #define PF_TC_F32_KERNEL_CUH_
 
