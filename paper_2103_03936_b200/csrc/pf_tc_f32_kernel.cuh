@@ -13,10 +13,11 @@
 // sums of one sign), so long sums must not stay in tensor memory: the main products a1 b1 accumulate over 64
 // elements of the contraction in one of two accumulators, which the worker warps then add, with
 // round-to-nearest, to fp32 sums in their registers.  The five correction products, at most 2^-7 of the sum, have an
-// accumulator of their own for 512 elements: then a chunk's main products go on top of it, so that it is drained as
-// that chunk's accumulator, and the buffer they would have used takes the corrections from there on.  160 truncated
-// additions lose at most 160 ulps of that 2^-7th, 1.5e-7 of the sum, whatever its length; left to pile up over 32768
-// elements of one sign they lost 6.9e-6.  The result is as accurate as an fp32 FMA kernel.
+// accumulator of their own for 2048 elements: then a chunk's main products go on top of it, so that it is drained as
+// that chunk's accumulator, and the buffer they would have used takes the corrections from there on.  640 truncated
+// additions lose at most 640 ulps of that 2^-7th, 6e-7 of the sum, whatever its length; left to pile up over 32768
+// elements of one sign they lost 6.9e-6.  (Not more often: the chunk on top of the corrections is truncated once
+// more, 1 % of the error of random sums at every 512 elements.)  The result is as accurate as an fp32 FMA kernel.
 //
 // One CTA computes a 128 x BN tile of C = A * B or one slice of its contraction.  Warps: 0 = TMA producer of
 // A, 1 = tensor memory + MMA issue, 2..17 = workers (split the operands, drain the accumulators, epilogue),
@@ -87,7 +88,7 @@ constexpr int kF32Threads = 608;
 constexpr int kF32MaxStages = 8;
 constexpr int kChunk = 2;                    // k-blocks per main accumulator: 64 elements of the contraction
 static_assert(kChunk == 2, "one k-block per worker group and chunk");
-constexpr int kCorrChunks = 8;               // chunks per correction accumulator
+constexpr int kCorrChunks = 32;              // chunks per correction accumulator
 static_assert(kCorrChunks % 2 == 0, "it changes places with the accumulator of the odd chunks");
 constexpr uint32_t kF32TileA = 16384;        // 128 x 32 floats
 constexpr uint32_t kColsA = 16;              // tensor-memory columns of one plane of A's k-block (32 bf16 per row)
@@ -248,8 +249,8 @@ __device__ __forceinline__ void repair_run(const float* a, long long sa, const f
 }
 // The outputs of this CTA (its share of the tile's units of 8 rows x 16 columns) from the operands in global memory,
 // by the definition of the product.  Rare and therefore plain: a lane sums one row's four columns.  The test for it
-// and the factor cost 1-2 % (training step of 2048 rows, 512 -> 128 -> 2048, cold L2: 73.2 -> 74.3 us; convolutions up to
-// 4 %: 32 x 28 x 28, 128 -> 32 -> 128, 176 -> 180 us); with a NaN in every row that linear step takes 1.8 ms.
+// and the factor cost 0-2 % (training step of 2048 rows, 512 -> 128 -> 2048, cold L2: 73.2 -> 74.1 us; 32 x 28 x 28, 128 ->
+// 32 -> 256, stride 2: 86.0 -> 88.1, stride 1 176.1 before and after); with a NaN in every row that linear step takes 1.8 ms.
 // (A second pass over the ring by the same roles was slower where nothing is repaired: 83 us.)
 template <int BN, int kMode>
 __device__ __noinline__ void f32_repair(const F32Params& p, int bx, int by, int bz) {
