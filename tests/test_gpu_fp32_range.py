@@ -53,7 +53,8 @@ def check(got, want, tol=1e-5):
         assert err <= tol, f"{k}: rel err {err:.3e}"
 
 
-SHAPES = [(300, 520, 264, 72), (2500, 300, 1028, 40), (130, 1000, 36, 200)]      # sliced and whole contractions, both tile widths
+# sliced and whole contractions, both tile widths, operands that are copied to padded pitches (and a stash that is a second copy)
+SHAPES = [(300, 520, 264, 72), (2500, 300, 1028, 40), (130, 1000, 36, 200), (257, 301, 133, 71)]
 
 
 # exponents of the four operands: results stay normal fp32 numbers.  A bf16 part of an operand reaches down to 2^-133
@@ -97,11 +98,27 @@ def test_results_near_overflow():
     assert not torch.isfinite(T).any()                     # 2^130 does not exist, so neither does their sum
 
 
+def test_bias_after_a_result_that_is_computed_again():
+    d = wl.LinearCase("bias", 300, 520, 264, 72, wl.F32, 35).generate()
+    d["x"][17, 200] = np.inf
+    d["V"][100] = np.ldexp(d["V"][100], 121)               # a column whose results need the full exponent range
+    b = wl.round_to(wl.normal(36, 0, (264,), 0.5), wl.F32)
+    y, T = pf.pf_lowrank_linear_fwd_act(*(dev(d[k], wl.F32) for k in ("x", "U", "V")), bias=dev(b, wl.F32), want_stash=True)
+    with np.errstate(all="ignore"):
+        want = dict(zip(("y", "T"), oracle.linear_fwd_act(d["x"], d["U"], d["V"], b)))
+    got = {"y": host(y, wl.F32).astype(np.float64), "T": host(T, wl.F32).astype(np.float64)}
+    check(got, want)
+    for k in ("y", "T"):                                   # and column by column, so that the large one hides none
+        for c in range(0, want[k].shape[1], 25):
+            check({k: got[k][:, c]}, {k: want[k][:, c]})
+
+
 @pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad,at", [
     (2, 13, 6, 36, 20, 24, 3, 1, 0, (0, 11, 2, 5)),       # the last block of pixels reaches past the last output row
     (2, 9, 43, 36, 20, 24, 3, 1, 0, (1, 4, 41, 5)),       # ... past the last output column
     (3, 11, 13, 100, 12, 40, 3, 2, 1, (2, 4, 6, 99)),
-    (5, 5, 5, 64, 16, 64, 3, 1, 1, (4, 0, 0, 63))])
+    (5, 5, 5, 64, 16, 64, 3, 1, 1, (4, 0, 0, 63)),
+    (6, 56, 56, 132, 72, 40, 3, 1, 1, (5, 30, 31, 131))])      # tiles of 128 columns
 def test_convolution_range(N, H, W, C, R, O, k, stride, pad, at):
     """The convolution's products on the same kernel: an infinite input or gradient reaches its own window only, small and
     large operands keep fp32 accuracy."""
