@@ -134,8 +134,8 @@ int pf_lowrank_linear_fwd_act(const void* x, int64_t ldx, const void* U, int64_t
  *              rounded once to `dtype`)                    [n], NULL = not wanted
  * (Section 2.4: the feed-forward block max(0, x W1 + b1) W2 + b2; biases are trained unfactorized,
  * Section 2.1.)  y (ldy) is the forward's output and is read only for PF_ACT_RELU.  The workspace of
- * pf_bias_act_bwd_workspace(m, n) bytes is needed only when dbias is given.  Two launches with
- * dbias, one without; m = 0 zeroes dbias. */
+ * pf_bias_act_bwd_workspace(m, n) bytes is needed only when dbias is given.  One launch, two
+ * with dbias and more than 4096 rows; m = 0 zeroes dbias. */
 size_t pf_bias_act_bwd_workspace(int64_t m, int64_t n);
 int pf_bias_act_bwd(const void* y, int64_t ldy, void* dY, int64_t lddy, void* dbias,
                     int64_t m, int64_t n, int act, int dtype,

@@ -127,3 +127,23 @@ def test_bias_act_bwd(dtype, relu, m, n, ld_pad):
     assert pf.pf_bias_act_bwd(gy.t, gd.t, act=pf.PF_ACT_RELU if relu else pf.PF_ACT_NONE, want_dbias=False) is None
     assert pf.pf_launch_count() - l0 == 1
     assert pf.pf_last_device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", [wl.F32, wl.BF16])
+@pytest.mark.parametrize("relu", [True, False])
+@pytest.mark.parametrize("m,n,launches", [(1, 64, 1), (63, 65, 1), (64, 60, 1), (513, 130, 1), (4096, 2, 1), (4096, 264, 1), (4097, 64, 2)])
+def test_bias_act_bwd_one_launch(dtype, relu, m, n, launches):
+    """The blocks of a cluster sum their rows in one launch (any width, remainders of rows and columns, the most rows that
+    take it); beyond that two launches.  Sums of m values: fp32 error of order m * 2^-24, then one rounding."""
+    y_h = wl.round_to(np.maximum(wl.normal(62, 0, (m, n)), 0.0), dtype)
+    g_h = wl.round_to(wl.normal(62, 1, (m, n)), dtype)
+    y, gd, gb = dev(y_h, dtype), Guarded((m, n), dtype), Guarded((1, n), dtype)
+    gd.t.copy_(dev(g_h, dtype))
+    l0 = pf.pf_launch_count()
+    pf.pf_bias_act_bwd(y, gd.t, act=pf.PF_ACT_RELU if relu else pf.PF_ACT_NONE, dbias=gb.t.view(-1))
+    assert pf.pf_launch_count() - l0 == launches
+    dZ_ref, db_ref = oracle.bias_act_bwd(y_h, g_h, relu=relu)
+    np.testing.assert_array_equal(oracle.widen(wl.from_torch(gd.t.contiguous(), dtype)), dZ_ref)
+    assert_close(gb.t.view(-1), db_ref, dtype, f"dbias {m}x{n} {dtype} relu={relu}", tol=1e-2 if dtype == wl.BF16 else 1e-4)
+    gd.check()
+    gb.check()
