@@ -317,8 +317,8 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
     if (dtype == PF_BF16) {
         tc::LinearArgs::Slices su_info, sv_info;
         if (flags) {
-            // plain gradients go to the workspace; where a reduction was split, its fp32 slices are still
-            // there afterwards and are summed once more, unrounded, into the caller's matrix
+            // plain gradients go to the workspace; where a reduction left fp32 slices there, they are summed (once more
+            // if there are several), unrounded, into the caller's matrix
             indirect = true;
             dU = ws + w.off_gtmp; lddu = r;
             dV = ws + w.off_gtmp + align_up(static_cast<size_t>(k) * r * s, 256); lddv = r;
@@ -331,12 +331,12 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
         if (handled && flags) {
             SliceSums jobs[2];
             int nj = 0;
-            if (su_info.splits > 1)
+            if (su_info.partial)
                 jobs[nj++] = SliceSums{su_info.partial, user_dU, user_lddu, static_cast<int>(k), static_cast<int>(r), su_info.splits,
                                        su_info.bn, su_info.tiles_x, su_info.tiles_y, g_f32, g_acc};
             else
                 PF_CUDA(grad_combine(user_dU, user_lddu, gdtype, dU, lddu, dtype, k, r, g_acc, stream));
-            if (sv_info.splits > 1)
+            if (sv_info.partial)
                 jobs[nj++] = SliceSums{sv_info.partial, user_dV, user_lddv, static_cast<int>(n), static_cast<int>(r), sv_info.splits,
                                        sv_info.bn, sv_info.tiles_x, sv_info.tiles_y, g_f32, g_acc};
             else
@@ -667,12 +667,12 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         if (!flags) return PF_OK;
         SliceSums jobs[2];
         int nj = 0;
-        if (su_info.splits > 1)
+        if (su_info.partial)
             jobs[nj++] = SliceSums{su_info.partial, user_dU, R, static_cast<int>(Keff), R, su_info.splits, su_info.bn,
                                    su_info.tiles_x, su_info.tiles_y, g_f32, g_acc, su_info.conv_c};
         else
             PF_CUDA(grad_combine(user_dU, R, gdtype, dU, R, dtype, Keff, R, g_acc, stream));
-        if (sv_info.splits > 1)
+        if (sv_info.partial)
             jobs[nj++] = SliceSums{sv_info.partial, user_dV, R, O, R, sv_info.splits, sv_info.bn, sv_info.tiles_x,
                                    sv_info.tiles_y, g_f32, g_acc};
         else
@@ -689,7 +689,7 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         a.N = N; a.H = H; a.W = W; a.C = C; a.R = R; a.O = O; a.kh = kh; a.kw = kw;
         a.stride = stride; a.pad = pad; a.Ho = w.Ho; a.Wo = w.Wo;
         a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.ws_G = ws + w.off_dT; a.stream = stream;
-        a.du_slices = &su_info; a.dv_slices = &sv_info;
+        if (flags) { a.du_slices = &su_info; a.dv_slices = &sv_info; }
         int handled = 0;
         st = dtype == PF_BF16 ? tc::conv_bwd(a, &handled) : tc::f32_conv_bwd(a, &handled);
         if (st != PF_OK) return st;

@@ -76,48 +76,45 @@ cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const Gemm
     return e;
 }
 
-// Workspace floats of a split product: one 128 x bn block per (tile, slice).
-size_t partial_bytes(int64_t M, int64_t N, int splits) {
-    if (splits <= 1) return 0;
+// Workspace floats of a product's slices: one 128 x bn block per (tile, slice).
+size_t slice_bytes(int64_t M, int64_t N, int splits) {
     const int bn = N <= 64 ? 64 : 128;
-    return static_cast<size_t>(ceil_div(M, kBM) * ceil_div(N, bn)) * splits * kBM * bn * 4;
+    return static_cast<size_t>(ceil_div(M, kBM) * ceil_div(N, bn)) * std::max(1, splits) * kBM * bn * 4;
 }
+size_t partial_bytes(int64_t M, int64_t N, int splits) { return splits <= 1 ? 0 : slice_bytes(M, N, splits); }      // a split product
 
-int pick_splits(int64_t M, int64_t N, int bn, int64_t K) {
-    const int64_t tiles = ceil_div(M, kBM) * ceil_div(N, bn);
-    const int64_t nkb = ceil_div(K, kBK);
-    if (tiles < 1 || nkb < 1) return 1;
-    int64_t s = num_sms() / tiles;
-    if (s > nkb / 4) s = nkb / 4;     // at least 4 k-blocks per slice
-    if (s > 64) s = 64;
-    if (s < 1) s = 1;
-    return static_cast<int>(s);
+// What a block that is alone on its SM spends on kb k-blocks of a contraction cut into s slices, beyond its start and
+// end: 0.16 us per k-block on warm caches, 0.3 on cold ones, and for the sum of the slices 5 us at two slices, 4.2 at
+// four, 3.8 at eight (the fewer slices, the larger the share that a block sums).  So short contractions stay whole:
+// 1024 x 256 over 512: 9.3 us in two slices, 4.8 whole; over 1024: 8.4 in four, 6.0 whole; over 2048: 8.4 in eight, 8.4
+// whole; over 4096: 9.3 in eight, 13.0 whole.
+double slice_us(int64_t nkb, int64_t s) {
+    return 0.2 * static_cast<double>(ceil_div(nkb, s)) + (s > 1 ? 3.4 + 3.4 / static_cast<double>(s) : 0.0);
 }
+// Slices of a contraction that is alone in its launch.
+int slices_of(int64_t tiles, int64_t nkb) {
+    if (tiles < 1 || nkb < 1) return 1;
+    const int64_t s = std::min<int64_t>(64, std::min(num_sms() / tiles, nkb / 4));     // at least 4 k-blocks per slice
+    return s > 1 && slice_us(nkb, s) < slice_us(nkb, 1) ? static_cast<int>(s) : 1;
+}
+int pick_splits(int64_t M, int64_t N, int bn, int64_t K) { return slices_of(ceil_div(M, kBM) * ceil_div(N, bn), ceil_div(K, kBK)); }
 int pick_bn(int64_t N) { return N <= 64 ? 64 : 128; }
 
-// CTA pairs (256 x 256 tiles, persistent) pay off for wide outputs once every pair gets at least two
-// tiles, or fewer tiles with a long contraction each; short products with few tiles are better
-// off as many small single-CTA tiles.
-bool pair_worthwhile(int64_t M, int64_t N, int64_t K) {
-    const int64_t tiles = ceil_div(M, 256) * ceil_div(N, 256);
-    return N >= 256 && (tiles >= num_sms() || (tiles >= 48 && K >= 2048));
-}
-
 // Slice counts for two products that share one launch (dU: Mu x N over nkb_u k-blocks, dV: Mv x N over nkb_v):
-// all CTAs should fit one wave and finish together, so the longest CTA (in k-blocks) is
+// all CTAs should fit one wave and finish together, so the time of the longest CTA is
 // minimised subject to tiles_u * su + tiles_v * sv <= SM count.
 void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t nkb_u, int64_t nkb_v, int* su, int* sv) {
     const int bn = pick_bn(N);
     const int64_t tu = ceil_div(Mu, kBM) * ceil_div(N, bn), tv = ceil_div(Mv, kBM) * ceil_div(N, bn);
     *su = 1; *sv = 1;
     if (tu < 1 || tv < 1 || nkb_u < 1 || nkb_v < 1 || tu + tv > num_sms()) return;
-    int64_t best = std::max(nkb_u, nkb_v) + 1;
+    double best = std::max(slice_us(nkb_u, 1), slice_us(nkb_v, 1));
+    if (best < slice_us(1, 64)) return;      // shorter than any sum of slices
     for (int64_t a = 1; a <= 64 && a <= nkb_u && tu * a + tv <= num_sms(); ++a) {
-        int64_t b = (num_sms() - tu * a) / tv;
-        if (b > 64) b = 64;
-        if (b > nkb_v) b = nkb_v;
-        if (b < 1) continue;
-        const int64_t longest = std::max(ceil_div(nkb_u, a), ceil_div(nkb_v, b));
+        const double u = slice_us(nkb_u, a);
+        const int64_t most = std::min(std::min<int64_t>(64, nkb_v), (num_sms() - tu * a) / tv);
+        const int64_t b = slice_us(nkb_v, most) < slice_us(nkb_v, 1) ? most : 1;
+        const double longest = std::max(u, slice_us(nkb_v, b));
         if (longest < best) { best = longest; *su = static_cast<int>(a); *sv = static_cast<int>(b); }
     }
 }
@@ -132,9 +129,15 @@ void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t nkb_u, int64_t 
 // 20 SMs the split fused kernel leaves idle are free, loses more through the long dV blocks than the
 // overlap gains.)
 void bwd_split_plan(int64_t m, int64_t k, int64_t n, int64_t r, bool fused_dx, int* su, int* sv, bool* beside) {
+    if (!fused_dx) {        // each shares a launch with a product that waits for nothing (see linear_bwd)
+        *su = pick_splits(k, r, pick_bn(r), m);
+        *sv = pick_splits(n, r, pick_bn(r), m);
+        *beside = false;
+        return;
+    }
     pick_pair_splits(k, n, r, ceil_div(m, kBK), ceil_div(m, kBK), su, sv);
     *beside = false;
-    if (!fused_dx || n < 2 * k) return;
+    if (n < 2 * k) return;
     const int bn = pick_bn(r);
     const int64_t row_tiles = ceil_div(m, kBM), nkb = ceil_div(m, kBK);
     const int64_t tu = ceil_div(k, kBM) * ceil_div(r, bn), tv = ceil_div(n, kBM) * ceil_div(r, bn);
@@ -177,9 +180,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     const int groups = gr ? gr->groups : 1;
     const bool sum_groups = gr && gr->sum_groups;
     if (gr && (cv || groups < 1 || groups > 1024 || (sum_groups && (A.mn_major || B.mn_major)))) return PF_ERR_UNSUPPORTED;
-    // wide outputs that would need more than one wave of 128-column tiles (two CTAs per SM) take
-    // 256-column tiles
-    const int bn = (!(cv && cv->mode == 1) && splits <= 1 && N >= 512 && ceil_div(M, kBM) * ceil_div(N, 128) > 2 * num_sms()) ? 256 : pick_bn(N);
+    const int bn = pick_bn(N);
     CUtensorMap& ta = out->ta;
     CUtensorMap& tb = out->tb;
     bool oka, okb;
@@ -204,7 +205,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     GemmParams& p = out->p;
     p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
     p.a_mn = A.mn_major; p.b_mn = B.mn_major;
-    p.C = C; p.ldc = ldc; p.partial = partial;
+    p.C = C; p.ldc = ldc;
     p.C2 = nullptr; p.ldc2 = 0; p.c2_gstride = 0;
     p.bias = nullptr; p.act = 0;
     p.conv_mode = 0; p.cv_blks = 1; p.cv_kw = 1; p.cv_kh = 1; p.cv_pad = 0; p.cv_stride = 1; p.cv_C = 1; p.cv_bh = 1; p.cv_nb = 1;
@@ -257,11 +258,12 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     if (dx) grid = dim3(run_blocks(static_cast<int64_t>(p.tiles_x) * p.tiles_y, nkb / (cv->stride * cv->stride), cv->stride));
     p.num_stages = pick_stages(bn, static_cast<int64_t>(grid.x) * grid.y * grid.z, dx);
     p.counters = nullptr;
+    p.partial = p.splits > 1 ? partial : nullptr;
     p.independent = 0;
     if (p.splits > 1) {
         // the CTAs of a tile wait for one another, so all of them must be resident at once
         if (static_cast<int64_t>(grid.x) * grid.y * out_groups > kFixTiles || static_cast<int64_t>(grid.x) * grid.y * grid.z > num_sms() ||
-            bn == 256 || partial == nullptr)
+            partial == nullptr)
             return PF_ERR_UNSUPPORTED;
         p.counters = split_counters();
         if (!p.counters) return PF_ERR_CUDA;
@@ -278,41 +280,7 @@ int launch_prepared(const GemmLaunch& g, cudaStream_t stream) {
         count_launch();
         return PF_OK;
     }
-    const cudaError_t e = g.bn == 64    ? launch_gemm<64>(g.ta, g.tb, g.p, g.grid, stream)
-                          : g.bn == 128 ? launch_gemm<128>(g.ta, g.tb, g.p, g.grid, stream)
-                                        : launch_gemm<256>(g.ta, g.tb, g.p, g.grid, stream);
-    return e == cudaSuccess ? PF_OK : PF_ERR_CUDA;
-}
-
-// `copy2` (optional): asks for a second copy of C at pitch ldc2; *copy2_done tells whether the launch
-// wrote it (the CTA-pair kernel cannot), else the caller copies C itself.
-int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
-         int splits, float* partial, cudaStream_t stream, void* copy2 = nullptr, int64_t ldc2 = 0, bool* copy2_done = nullptr, const void* bias = nullptr, int act = 0) {
-    // wide, many-tile (tensor-bound) products run on CTA pairs, which halve the operand traffic per SM
-    if (splits <= 1 && pair_worthwhile(M, N, K)) {
-        PairJob j{A.p, A.ld, A.mn_major, 0, B.p, B.ld, B.mn_major, 0, M, N, K, C, ldc};
-        j.bias = bias;
-        j.act = act;
-        const int st2 = gemm_pairs(&j, 1, 1, stream);
-        if (st2 != PF_ERR_UNSUPPORTED) {
-            if (copy2_done) *copy2_done = false;
-            return st2;
-        }
-    }
-    GemmLaunch g;
-    int st = gemm_prepare(A, B, M, N, K, C, ldc, splits, partial, nullptr, &g);
-    if (st == PF_ERR_UNSUPPORTED && splits > 1) st = gemm_prepare(A, B, M, N, K, C, ldc, 1, nullptr, nullptr, &g);
-    if (st != PF_OK) return st;
-    if (copy2_done) *copy2_done = false;
-    if (copy2) {
-        g.p.C2 = copy2; g.p.ldc2 = ldc2;
-        if (copy2_done) *copy2_done = true;
-    }
-    g.p.bias = bias; g.p.act = act;               // (given for unsplit products only)
-    const GemmParams& p = g.p;
-    cudaError_t e = g.bn == 64    ? launch_gemm<64>(g.ta, g.tb, p, g.grid, stream)
-                    : g.bn == 128 ? launch_gemm<128>(g.ta, g.tb, p, g.grid, stream)
-                                  : launch_gemm<256>(g.ta, g.tb, p, g.grid, stream);
+    const cudaError_t e = g.bn == 64 ? launch_gemm<64>(g.ta, g.tb, g.p, g.grid, stream) : launch_gemm<128>(g.ta, g.tb, g.p, g.grid, stream);
     return e == cudaSuccess ? PF_OK : PF_ERR_CUDA;
 }
 
@@ -324,7 +292,6 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
     int total = 0, split_ctas = 0;
     bool seen_plain = false;
     for (int i = 0; i < count; ++i) {
-        if (g[i]->bn != 64 && g[i]->bn != 128) return PF_ERR_UNSUPPORTED;
         ctas[i] = static_cast<int>(g[i]->grid.x * g[i]->grid.y * g[i]->grid.z);
         total += ctas[i];
         if (g[i]->p.splits > 1) {
@@ -374,6 +341,116 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
     return PF_OK;
 }
 
+// Expected microseconds of one launch of prepared products on single CTAs, and of the same products on CTA pairs, fitted
+// to launches of one product between 512 and 16384 rows, 256 to 4096 columns and contractions of 256 to 16384 (within
+// 20 %, mostly 10 %).  A single CTA's 128 x 128 tile: 3.6 us of start and end and slice_us alone on its SM; 4.1 us and
+// 0.42 us per k-block beside another (its SM's load path is what it waits for).  A pair's 256 x 256 tile: 0.28 us per
+// k-block (the tensor cores), and 2 us of every tile but the first do not hide (the results' way to memory).  Output rows
+// that take no 16-byte stores: 2.4 us more per single tile, 3 per tile of a pair.
+bool vector_rows(const void* C, int64_t ldc, int64_t gs) { return ldc % 8 == 0 && gs % 8 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0; }
+double single_us(const GemmLaunch* const* g, int count) {
+    double ctas = 0, load = 0, alone = 0, beside = 0, shortest = 1e30;
+    for (int i = 0; i < count; ++i) shortest = std::min<double>(shortest, g[i]->p.kb_per_split);
+    for (int i = 0; i < count; ++i) {
+        const double n = static_cast<double>(g[i]->grid.x) * g[i]->grid.y * g[i]->grid.z, kb = g[i]->p.kb_per_split;
+        const double sum = slice_us(g[i]->p.nkb_total, g[i]->p.splits) - 0.2 * kb + (g[i]->p.splits > 1 || vector_rows(g[i]->p.C, g[i]->p.ldc, g[i]->p.c_gstride) ? 0.0 : 2.4);
+        ctas += n;
+        load += n * (0.42 * kb + 4.1 + sum);
+        alone = std::max(alone, 0.2 * kb + sum);
+        beside = std::max(beside, 0.42 * shortest + 0.2 * (kb - shortest) + sum);
+    }
+    if (ctas <= num_sms()) return 3.6 + alone;
+    return std::max(load / (2.0 * num_sms()), beside + 4.1);
+}
+double pairs_us(const PairJob* j, int count) {
+    double load = 0, longest = 0, tiles = 0;
+    for (int i = 0; i < count; ++i) {
+        const double n = static_cast<double>(ceil_div(j[i].M, 256) * ceil_div(j[i].N, 256)) * (j[i].sum_groups ? 1 : j[i].groups);
+        const double kb = static_cast<double>(ceil_div(j[i].K, 64)) * (j[i].sum_groups ? j[i].groups : 1);
+        const double us = 0.28 * kb + (vector_rows(j[i].C, j[i].ldc, j[i].c_gs) ? 2.0 : 5.0);
+        tiles += n;
+        load += n * us;
+        longest = std::max(longest, us);
+    }
+    const int pairs = num_sms() / 2;
+    double total = load / pairs;
+    if (count == 1) total = longest * static_cast<double>(ceil_div(static_cast<int64_t>(tiles), pairs));
+    return std::max(total, longest) + 3.4;
+}
+// One launch of up to three products on single CTAs (one launch each where they cannot share it).
+int launch_singles(const GemmLaunch* const* g, int count, cudaStream_t stream) {
+    if (count == 1) return launch_prepared(*g[0], stream);
+    const GemmLaunch* list[3];
+    int n = 0;
+    for (int i = 0; i < count; ++i) list[n++] = g[i];
+    // split products first, then the longest tiles (backward of 1000 x 512 -> 128 -> 512, dX of 2 k-blocks in
+    // front of dU of 16: 12.5 us, behind it 11.8)
+    std::stable_sort(list, list + n, [](const GemmLaunch* x, const GemmLaunch* y) {
+        return (x->p.splits > 1) != (y->p.splits > 1) ? x->p.splits > 1 : x->p.kb_per_split > y->p.kb_per_split;
+    });
+    int st = gemm_multi(list, count, stream);
+    for (int i = 0; st == PF_ERR_UNSUPPORTED && i < count; ++i) {
+        const int one = launch_prepared(*list[i], stream);
+        if (one != PF_OK) return one;
+        if (i + 1 == count) return PF_OK;
+    }
+    return st;
+}
+// One launch of one or two products, on whichever form is expected to be faster.  The products are independent of
+// each other; jobs[i] describes the same product as *g[i].  pair_extra: microseconds that the caller has to spend after
+// pairs only; *pairs tells which form it was.
+int launch_faster(const GemmLaunch* const* g, const PairJob* jobs, int count, cudaStream_t stream, double pair_extra = 0.0,
+                  bool* pairs = nullptr) {
+    if (pairs_us(jobs, count) + pair_extra < 0.9 * single_us(g, count)) {
+        PairJob order[2] = {jobs[0], jobs[count > 1 ? 1 : 0]};
+        auto kb = [](const PairJob& j) { return ceil_div(j.K, 64) * (j.sum_groups ? j.groups : 1); };
+        if (count > 1 && kb(order[1]) > kb(order[0])) std::swap(order[0], order[1]);     // long tiles first
+        const int st = gemm_pairs(order, count, 1, stream);
+        if (st != PF_ERR_UNSUPPORTED) {
+            if (pairs) *pairs = true;
+            return st;
+        }
+    }
+    return launch_singles(g, count, stream);
+}
+// One launch of up to three products on single CTAs, or the first of them on CTA pairs by itself and then the others.
+int launch_with(const GemmLaunch* const* g, const PairJob* first, int count, cudaStream_t stream) {
+    if (pairs_us(first, 1) + single_us(g + 1, count - 1) < 0.9 * single_us(g, count)) {
+        const int st = gemm_pairs(first, 1, 1, stream);
+        if (st == PF_OK) return launch_singles(g + 1, count - 1, stream);
+        if (st != PF_ERR_UNSUPPORTED) return st;
+    }
+    return launch_singles(g, count, stream);
+}
+
+// Prepares a product, unsplit where its slices do not fit the counters or the machine.
+int gemm_prepare_any(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc, int splits, float* partial,
+                     const ConvA* cv, GemmLaunch* out) {
+    const int st = gemm_prepare(A, B, M, N, K, C, ldc, splits, partial, cv, out);
+    return st == PF_ERR_UNSUPPORTED && splits > 1 ? gemm_prepare(A, B, M, N, K, C, ldc, 1, nullptr, cv, out) : st;
+}
+// One product in a launch of its own.  `copy2` (optional): asks for a second copy of C at pitch ldc2; *copy2_done tells
+// whether the launch wrote it (the CTA-pair kernel cannot), else the caller copies C itself.
+int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
+         int splits, float* partial, cudaStream_t stream, void* copy2 = nullptr, int64_t ldc2 = 0, bool* copy2_done = nullptr,
+         const void* bias = nullptr, int act = 0) {
+    GemmLaunch g;
+    const int st = gemm_prepare_any(A, B, M, N, K, C, ldc, splits, partial, nullptr, &g);
+    if (st != PF_OK) return st;
+    if (copy2) {
+        g.p.C2 = copy2; g.p.ldc2 = ldc2;
+    }
+    g.p.bias = bias; g.p.act = act;               // (given for unsplit products only)
+    PairJob j{A.p, A.ld, A.mn_major, 0, B.p, B.ld, B.mn_major, 0, M, N, K, C, ldc};
+    j.bias = bias;
+    j.act = act;
+    const GemmLaunch* const list[1] = {&g};
+    bool pairs = false;
+    const int rc = launch_faster(list, &j, 1, stream, copy2 ? 6.0 : 0.0, &pairs);
+    if (copy2_done) *copy2_done = copy2 != nullptr && !pairs;
+    return rc;
+}
+
 // A row-major bf16 matrix that TMA must read: used as is when 16-byte aligned with a pitch that is
 // a multiple of 8 elements, otherwise copied to `scratch` with the pitch rounded up.
 struct Staged {
@@ -412,15 +489,31 @@ size_t repack_room(int64_t rows, int64_t cols) {
     return cols % 8 == 0 ? 0 : align_up(static_cast<size_t>(rows) * pad8(cols) * 2, 256);
 }
 
+// Whether the tiles of dU (rows_u x r) and dV (rows_v x r) fit the machine together.  Such reductions run on single CTAs,
+// split or whole, and can leave their fp32 slices to a call that wants unrounded gradients.
+bool narrow_reductions(int64_t rows_u, int64_t rows_v, int64_t r) {
+    return (ceil_div(rows_u, kBM) + ceil_div(rows_v, kBM)) * ceil_div(r, pick_bn(r)) <= num_sms();
+}
 // Room for the fp32 slices of dU and dV under either backward structure (which one a call takes
 // depends on pointers the workspace query does not see): no block count exceeds one per SM per product.
 void bwd_partial_bytes(int64_t m, int64_t k, int64_t n, int64_t r, size_t* bytes_u, size_t* bytes_v) {
+    *bytes_u = *bytes_v = 0;
+    if (!narrow_reductions(k, n, r)) return;        // (never split)
     int su, sv, su2, sv2;
     bool beside;
     bwd_split_plan(m, k, n, r, false, &su, &sv, &beside);
     bwd_split_plan(m, k, n, r, true, &su2, &sv2, &beside);
-    *bytes_u = align_up(std::max(partial_bytes(k, r, su), partial_bytes(k, r, su2)), 256);
-    *bytes_v = align_up(std::max(partial_bytes(n, r, sv), partial_bytes(n, r, sv2)), 256);
+    *bytes_u = align_up(slice_bytes(k, r, std::max(su, su2)), 256);
+    *bytes_v = align_up(slice_bytes(n, r, std::max(sv, sv2)), 256);
+}
+// Where a prepared reduction leaves its fp32 slices; an unsplit one is told to leave its one slice.
+void keep_slices(LinearArgs::Slices* out, GemmLaunch* g, float* room, int conv_c = 0) {
+    if (!out) return;
+    *out = LinearArgs::Slices();
+    if (!room) return;
+    g->p.partial = room;
+    out->partial = room; out->splits = g->p.splits; out->bn = g->bn;
+    out->tiles_x = static_cast<int>(g->grid.x); out->tiles_y = static_cast<int>(g->grid.y); out->conv_c = conv_c;
 }
 
 }  // namespace
@@ -574,122 +667,76 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     float* pv = reinterpret_cast<float*>(scratch);
     scratch += pv_bytes;
     float* p1 = reinterpret_cast<float*>(scratch);
-    // the slices of the reductions as they will be launched (the last prepared product is the launched one)
-    auto note = [](LinearArgs::Slices* out, const GemmLaunch* g) {
-        if (!out) return;
-        *out = LinearArgs::Slices();
-        if (g && g->p.splits > 1) {
-            out->partial = g->p.partial; out->splits = g->p.splits; out->bn = g->bn;
-            out->tiles_x = static_cast<int>(g->grid.x); out->tiles_y = static_cast<int>(g->grid.y);
-        }
-    };
     // G = dY V ; dX = G U^T ; dU = x^T G ; dV = dY^T T
     if (need_T) {   // no stash: recompute T = x U
         st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, Tbuf, pad8(a.r),
                   pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream);
         if (st != PF_OK) return st;
     }
-    bool dx_pending = false;     // dX still to be computed as a plain product G U^T
     if (fused_dx) {
         st = chain(dY.p, dY.ld, a.m, a.n, V.p, V.ld, a.r, U.p, U.ld, a.k, a.dX, a.lddx, G, ldG, a.stream, nullptr,
                    dv_beside ? 1 : 0);
         if (st != PF_OK) return st;
-    } else if (!a.du_slices && pair_worthwhile(a.m, a.r, a.n) && pair_worthwhile(a.n, a.r, a.m) && pair_worthwhile(a.k, a.r, a.m) &&
-               (!a.dX || pair_worthwhile(a.m, a.k, a.r))) {
-        // Large ranks, tensor-bound: two launches of CTA pairs, G beside dV and dU beside dX, so that the tiles of the
-        // second product fill the pairs that the few long tiles of the first leave free (16384 x 4096 -> 4096 at
-        // r 1024: each product alone left 14 % of the pairs idle).  Calls that want the slices go product by product.
-        const PairJob jg{dY.p, dY.ld, false, 0, V.p, V.ld, true, 0, a.m, a.r, a.n, G, ldG};
-        const PairJob jv{dY.p, dY.ld, true, 0, T.p, T.ld, true, 0, a.n, a.r, a.m, a.dV, a.lddv};
-        const PairJob ju{x.p, x.ld, true, 0, G, ldG, true, 0, a.k, a.r, a.m, a.dU, a.lddu};
-        const PairJob jx{G, ldG, false, 0, U.p, U.ld, false, 0, a.m, a.k, a.r, a.dX, a.lddx};
-        const PairJob first[2] = {a.m >= a.n ? jv : jg, a.m >= a.n ? jg : jv};
-        const PairJob second[2] = {a.m >= a.r || !a.dX ? ju : jx, a.m >= a.r ? jx : ju};
-        st = gemm_pairs(first, 2, 1, a.stream);
-        if (st != PF_OK) return st;
-        return gemm_pairs(second, a.dX ? 2 : 1, 1, a.stream);
     } else {
-        // Few rows: G = dY V is a contraction split across blocks, and dV = dY^T T, which needs nothing
-        // of it, shares its launch (the second block slot of every SM); dU and dX follow in a second one.
-        const int sg = pick_splits(a.m, a.r, pick_bn(a.r), a.n);
+        // Two launches: G = dY V with dV = dY^T T, which needs nothing of it, then dU = x^T G with dX = G U^T.  Where the
+        // tiles of dU and dV fit the machine they run on single CTAs, split or whole, and G and dX share their launches
+        // or, where that is faster, run on CTA pairs by themselves; larger ones run on whichever form is faster.
         GemmLaunch gg, gv, gu, gx;
-        bool ok = !pair_worthwhile(a.m, a.r, a.n) && !pair_worthwhile(a.n, a.r, a.m) &&
-                  gemm_prepare({dY.p, dY.ld, false}, {V.p, V.ld, true}, a.m, a.r, a.n, G, ldG, sg, p1, nullptr, &gg) == PF_OK &&
-                  gemm_prepare({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv) == PF_OK &&
-                  gemm_prepare({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu) == PF_OK;
-        if (ok && a.dX)
-            ok = gemm_prepare({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gx) == PF_OK;
-        ok = ok && (gg.p.splits > 1 || gv.p.splits <= 1) && (gu.p.splits > 1 || !a.dX || gx.p.splits <= 1);
-        if (ok) {
-            note(a.du_slices, &gu);
-            note(a.dv_slices, &gv);
-            const GemmLaunch* first[2] = {&gg, &gv};
-            st = gemm_multi(first, 2, a.stream);
-            if (st == PF_OK) {
-                const GemmLaunch* second[2] = {&gu, &gx};
-                st = gemm_multi(second, a.dX ? 2 : 1, a.stream);
-                if (st != PF_ERR_UNSUPPORTED) return st;
-                // tile widths that cannot share a launch: one launch each
-                st = launch_prepared(gu, a.stream);
-                if (st == PF_OK && a.dX) st = launch_prepared(gx, a.stream);
-                return st;
-            }
-            if (st != PF_ERR_UNSUPPORTED) return st;
+        const int bn = pick_bn(a.r);
+        const int64_t tr = ceil_div(a.r, bn), tg = ceil_div(a.m, kBM) * tr, tv = ceil_div(a.n, kBM) * tr;
+        int sg = pick_splits(a.m, a.r, bn, a.n);
+        if (sg > 1 && sv > 1 && tg * sg + tv * sv > num_sms()) {        // both sums in one launch: their blocks must fit together
+            int sg2 = 1, sv2 = 1;
+            pick_pair_splits(a.m, a.n, a.r, ceil_div(a.n, kBK), ceil_div(a.m, kBK), &sg2, &sv2);
+            sg = std::min(sg, sg2);                                      // (no more slices than the workspace holds)
+            sv = std::min(sv, sv2);
         }
-        st = gemm({dY.p, dY.ld, false}, {V.p, V.ld, true}, a.m, a.r, a.n, G, ldG, sg, p1, a.stream);
+        st = gemm_prepare_any({dY.p, dY.ld, false}, {V.p, V.ld, true}, a.m, a.r, a.n, G, ldG, sg, p1, nullptr, &gg);
+        if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
+        if (st == PF_OK) st = gemm_prepare_any({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
+        if (st == PF_OK && a.dX) st = gemm_prepare({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gx);
         if (st != PF_OK) return st;
-        dx_pending = a.dX != nullptr;
-    }
-    {   // dU = x^T G, dV = dY^T T (and dX = G U^T when it is still due): one launch when their tiles allow
-        GemmLaunch gu, gv, gx;
-        bool ok = gemm_prepare({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu) == PF_OK &&
-                  gemm_prepare({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv) == PF_OK;
-        if (ok && dx_pending)
-            ok = gemm_prepare({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gx) == PF_OK;
-        if (ok) {
-            note(a.du_slices, &gu);
-            note(a.dv_slices, &gv);
-            const GemmLaunch* list[3] = {&gu, &gv, &gx};
-            // a split product has to come before the plain ones
-            if (gu.p.splits <= 1 && gv.p.splits > 1) { list[0] = &gv; list[1] = &gu; }
-            if (dv_beside && !dx_pending) {
-                // dV first (its blocks are dispatched first, onto the SMs the fused kernel left free) and
-                // without waiting for the fused kernel; dU follows as that kernel's blocks retire
-                gv.p.independent = 1;
-                list[0] = &gv; list[1] = &gu;
-            }
-            st = gemm_multi(list, dx_pending ? 3 : 2, a.stream);
-            if (st != PF_ERR_UNSUPPORTED) return st;
-            if (dx_pending) {
-                // dX has wide tiles of its own (CTA pairs): launch it alone, dU and dV still together
-                st = gemm({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, a.stream);
-                if (st != PF_OK) return st;
-                dx_pending = false;
-                if (!(pair_worthwhile(a.k, a.r, a.m) && pair_worthwhile(a.n, a.r, a.m))) {
-                    st = gemm_multi(list, 2, a.stream);
-                    if (st != PF_ERR_UNSUPPORTED) return st;
-                }
-            }
+        const PairJob j1[2] = {{dY.p, dY.ld, false, 0, V.p, V.ld, true, 0, a.m, a.r, a.n, G, ldG},
+                               {dY.p, dY.ld, true, 0, T.p, T.ld, true, 0, a.n, a.r, a.m, a.dV, a.lddv}};
+        const PairJob j2[2] = {{G, ldG, false, 0, U.p, U.ld, false, 0, a.m, a.k, a.r, a.dX, a.lddx},
+                               {x.p, x.ld, true, 0, G, ldG, true, 0, a.k, a.r, a.m, a.dU, a.lddu}};
+        const GemmLaunch* const l1[2] = {&gg, &gv};
+        const GemmLaunch* const l2[2] = {&gx, &gu};
+        if (!narrow_reductions(a.k, a.n, a.r)) {
+            st = launch_faster(l1, j1, 2, a.stream);
+            if (st != PF_OK) return st;
+            return a.dX ? launch_faster(l2, j2, 2, a.stream) : launch_faster(l2 + 1, j2 + 1, 1, a.stream);
         }
-    }
-    if (dx_pending) {
-        st = gemm({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, a.stream);
+        keep_slices(a.du_slices, &gu, pu);
+        keep_slices(a.dv_slices, &gv, pv);
+        st = launch_with(l1, j1, 2, a.stream);
         if (st != PF_OK) return st;
+        return a.dX ? launch_with(l2, j2, 2, a.stream) : launch_singles(l2 + 1, 1, a.stream);
     }
-    note(a.du_slices, nullptr);      // launched by gemm(), which may choose other kernels and slice counts
-    note(a.dv_slices, nullptr);
-    st = gemm({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, a.stream);
+    // dU = x^T G, dV = dY^T T: one launch when their tiles allow
+    GemmLaunch gu, gv;
+    st = gemm_prepare_any({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
+    if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
     if (st != PF_OK) return st;
-    return gemm({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, a.stream);
+    keep_slices(a.du_slices, &gu, pu_bytes ? pu : nullptr);
+    keep_slices(a.dv_slices, &gv, pv_bytes ? pv : nullptr);
+    const GemmLaunch* list[2] = {&gu, &gv};
+    if (gu.p.splits <= 1 && gv.p.splits > 1) std::swap(list[0], list[1]);       // a split product has to come before the plain ones
+    if (dv_beside) {
+        // dV first (its blocks are dispatched first, onto the SMs the fused kernel left free) and
+        // without waiting for the fused kernel; dU follows as that kernel's blocks retire
+        gv.p.independent = 1;
+        list[0] = &gv; list[1] = &gu;
+    }
+    st = gemm_multi(list, 2, a.stream);
+    if (st != PF_ERR_UNSUPPORTED) return st;
+    gv.p.independent = 0;
+    st = launch_prepared(gu, a.stream);      // tile widths that cannot share a launch: one launch each
+    return st == PF_OK ? launch_prepared(gv, a.stream) : st;
 }
 
 // ------------------------------------------------------------------------------ grouped linear layer
 namespace {
-int grouped_splits(int64_t tiles, int64_t nkb) {
-    int64_t s = num_sms() / std::max<int64_t>(tiles, 1);
-    s = std::min<int64_t>(s, std::min<int64_t>(64, nkb / 4));
-    return static_cast<int>(std::max<int64_t>(s, 1));
-}
 struct GroupedPlan {
     int bn;                       // tile width of the m x r and (k|n) x r products
     int s1, sg, su, sv;           // slices of x U, dY V, dU, dV
@@ -700,10 +747,10 @@ GroupedPlan grouped_plan(int groups, int64_t m, int64_t k, int64_t n, int64_t r)
     g.bn = pick_bn(r);
     const int64_t tr = ceil_div(r, g.bn);
     const int64_t tm = ceil_div(m, kBM) * tr * groups, tk = ceil_div(k, kBM) * tr * groups, tn = ceil_div(n, kBM) * tr * groups;
-    g.s1 = grouped_splits(tm, ceil_div(k, kBK));
-    g.sg = grouped_splits(tm, ceil_div(n, kBK));
-    g.su = grouped_splits(tk, ceil_div(m, kBK));
-    g.sv = grouped_splits(tn, ceil_div(m, kBK));
+    g.s1 = slices_of(tm, ceil_div(k, kBK));
+    g.sg = slices_of(tm, ceil_div(n, kBK));
+    g.su = slices_of(tk, ceil_div(m, kBK));
+    g.sv = slices_of(tn, ceil_div(m, kBK));
     if (tm > kFixTiles) g.s1 = g.sg = 1;
     if (tk > kFixTiles) g.su = 1;
     if (tn > kFixTiles) g.sv = 1;
@@ -714,60 +761,6 @@ GroupedPlan grouped_plan(int groups, int64_t m, int64_t k, int64_t n, int64_t r)
     return g;
 }
 bool grouped_ok(const void* p, int64_t ld, int64_t gs) { return tma_ok(p, ld) && gs % 8 == 0; }
-
-// Expected microseconds of one launch of prepared products on single CTAs, and of the same products on CTA pairs:
-// a single CTA's 128 x 128 tile takes 0.31 us per k-block alone on its SM and 0.55 us beside another (its SM's load
-// path is what it waits for), a pair's 256 x 256 tile 0.28 us (the tensor cores); 3 - 4.5 us of start-up and
-// epilogue, of which a persistent pair overlaps all but the first and last; an output pitch that TMA and 16-byte
-// stores cannot take makes a pair's epilogue 3 us.
-double single_us(const GemmLaunch* const* g, int count) {
-    double ctas = 0, load = 0, longest = 0;
-    bool split = false;
-    for (int i = 0; i < count; ++i) {
-        const double n = static_cast<double>(g[i]->grid.x) * g[i]->grid.y * g[i]->grid.z, kb = g[i]->p.kb_per_split;
-        ctas += n;
-        load += n * (0.55 * kb + 4.5);
-        longest = std::max(longest, kb);
-        split = split || g[i]->p.splits > 1;
-    }
-    if (ctas <= num_sms()) return 0.31 * longest + 3.0 + (split ? 6.5 : 0.0);
-    return std::max(load / (2.0 * num_sms()), 0.55 * longest + 4.5);
-}
-double pairs_us(const PairJob* j, int count) {
-    double load = 0, longest = 0;
-    for (int i = 0; i < count; ++i) {
-        const double tiles = static_cast<double>(ceil_div(j[i].M, 256) * ceil_div(j[i].N, 256)) * (j[i].sum_groups ? 1 : j[i].groups);
-        const double kb = static_cast<double>(ceil_div(j[i].K, 64)) * (j[i].sum_groups ? j[i].groups : 1);
-        const bool vec = j[i].ldc % 8 == 0 && j[i].c_gs % 8 == 0 && (reinterpret_cast<uintptr_t>(j[i].C) & 15) == 0;
-        const double us = std::max(0.28 * kb, vec ? 1.3 : 3.0);
-        load += tiles * us;
-        longest = std::max(longest, us);
-    }
-    const int pairs = num_sms() / 2;
-    double total = load / pairs;
-    if (count == 1) total = longest * static_cast<double>(ceil_div(static_cast<int64_t>(load / longest + 0.5), pairs));
-    return std::max(total, longest) + 4.0;
-}
-// One launch of one or two products, on whichever form is expected to be faster.  The products are independent of
-// each other; jobs[i] describes the same product as *g[i].
-int launch_faster(const GemmLaunch* const* g, const PairJob* jobs, int count, cudaStream_t stream) {
-    if (pairs_us(jobs, count) < 0.9 * single_us(g, count)) {
-        PairJob order[2] = {jobs[0], jobs[count > 1 ? 1 : 0]};
-        auto kb = [](const PairJob& j) { return ceil_div(j.K, 64) * (j.sum_groups ? j.groups : 1); };
-        if (count > 1 && kb(order[1]) > kb(order[0])) std::swap(order[0], order[1]);     // long tiles first
-        const int st = gemm_pairs(order, count, 1, stream);
-        if (st != PF_ERR_UNSUPPORTED) return st;
-    }
-    const GemmLaunch* list[2] = {g[0], g[count > 1 ? 1 : 0]};
-    if (count > 1 && list[0]->p.splits <= 1 && list[1]->p.splits > 1) std::swap(list[0], list[1]);   // split products first
-    int st = count > 1 ? gemm_multi(list, count, stream) : PF_ERR_UNSUPPORTED;
-    for (int i = 0; st == PF_ERR_UNSUPPORTED && i < count; ++i) {
-        const int one = launch_prepared(*g[i], stream);
-        if (one != PF_OK) return one;
-        if (i + 1 == count) return PF_OK;
-    }
-    return st;
-}
 
 // A grouped operand that TMA must read: as it is, or (ragged widths) all its groups copied to `scratch` at a
 // padded pitch.  A shared operand is one matrix.
@@ -915,18 +908,25 @@ void conv_splits(const ConvA& c, int O, int* su, int* sv) {
     pick_pair_splits(conv_du_tiles(c.kh, c.kw, c.C) * kBM, O, c.R, conv_k_tiling(c).blocks,
                      ceil_div(static_cast<int64_t>(c.N) * c.Ho * c.Wo, kBK), su, sv);
 }
-size_t conv_du_partials(const ConvA& c, int su) { return align_up(partial_bytes(conv_du_tiles(c.kh, c.kw, c.C) * kBM, c.R, su), 256); }
+// Room for the slices of dU and dV ((kh*kw*C) x R and O x R), as bwd_partial_bytes.
+void conv_partial_bytes(const ConvA& c, int O, int su, int sv, size_t* bytes_u, size_t* bytes_v) {
+    const int64_t rows = conv_du_tiles(c.kh, c.kw, c.C) * kBM;
+    const bool narrow = narrow_reductions(rows, O, c.R);
+    *bytes_u = narrow ? align_up(slice_bytes(rows, c.R, su), 256) : 0;
+    *bytes_v = narrow ? align_up(slice_bytes(O, c.R, sv), 256) : 0;
+}
 }  // namespace
 
 size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad,
                             bool bwd) {
     const int Ho = (H + 2 * pad - kh) / stride + 1, Wo = (W + 2 * pad - kw) / stride + 1;
     if (!bwd || N < 1 || Ho < 1 || Wo < 1) return 0;
-    // split partials of dU ((kh*kw*C) x R) and dV (O x R)
     const ConvA c{2, N, H, W, C, R, Ho, Wo, kh, kw, pad, stride};
     int su, sv;
+    size_t bu, bv;
     conv_splits(c, O, &su, &sv);
-    return conv_du_partials(c, su) + align_up(partial_bytes(O, R, sv), 256);
+    conv_partial_bytes(c, O, su, sv, &bu, &bv);
+    return bu + bv;
 }
 
 int conv_fwd(const ConvArgs& a, int* handled) {
@@ -960,20 +960,16 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     cx.mode = 1;
     int su, sv;
     conv_splits(cu, a.O, &su, &sv);
+    size_t bu, bv;
+    conv_partial_bytes(cu, a.O, su, sv, &bu, &bv);
     float* pu = reinterpret_cast<float*>(a.ws);
-    float* pv = reinterpret_cast<float*>(a.ws + conv_du_partials(cu, su));
+    float* pv = reinterpret_cast<float*>(a.ws + bu);
     GemmLaunch gt, gu, gv, gx;
-    auto prepare = [](const Operand& A, const Operand& B, int64_t Mm, int64_t Nn, int64_t Kk, void* C, int64_t ldc,
-                      int splits, float* partial, const ConvA* cv, GemmLaunch* out) {
-        int r = gemm_prepare(A, B, Mm, Nn, Kk, C, ldc, splits, partial, cv, out);
-        if (r == PF_ERR_UNSUPPORTED && splits > 1) r = gemm_prepare(A, B, Mm, Nn, Kk, C, ldc, 1, nullptr, cv, out);
-        return r;
-    };
-    st = prepare({a.dY, a.O, false}, {a.V, a.R, true}, P, a.R, a.O, dT, a.R, 1, nullptr, nullptr, &gt);
-    if (st == PF_OK) st = prepare({a.x, a.C, true}, {dT, a.R, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
-    if (st == PF_OK) st = prepare({a.dY, a.O, true}, {T, a.R, true}, a.O, a.R, P, a.dV, a.R, sv, pv, nullptr, &gv);
+    st = gemm_prepare_any({a.dY, a.O, false}, {a.V, a.R, true}, P, a.R, a.O, dT, a.R, 1, nullptr, nullptr, &gt);
+    if (st == PF_OK) st = gemm_prepare_any({a.x, a.C, true}, {dT, a.R, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
+    if (st == PF_OK) st = gemm_prepare_any({a.dY, a.O, true}, {T, a.R, true}, a.O, a.R, P, a.dV, a.R, sv, pv, nullptr, &gv);
     if (st == PF_OK && a.dX)
-        st = prepare({dT, a.R, false}, {a.U, a.R, false}, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
+        st = gemm_prepare_any({dT, a.R, false}, {a.U, a.R, false}, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
                      static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1, nullptr, &cx, &gx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     if (st != PF_OK) return st;
@@ -991,19 +987,9 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         if (st != PF_OK) return st;
     }
     *handled = 1;
-    {   // both reductions are launched exactly as prepared
-        const GemmLaunch* gs[2] = {&gu, &gv};
-        LinearArgs::Slices* outs[2] = {a.du_slices, a.dv_slices};
-        for (int i = 0; i < 2; ++i) {
-            if (!outs[i]) continue;
-            *outs[i] = LinearArgs::Slices();
-            if (gs[i]->p.splits > 1) {
-                outs[i]->partial = gs[i]->p.partial; outs[i]->splits = gs[i]->p.splits; outs[i]->bn = gs[i]->bn;
-                outs[i]->tiles_x = static_cast<int>(gs[i]->grid.x); outs[i]->tiles_y = static_cast<int>(gs[i]->grid.y);
-                outs[i]->conv_c = i == 0 ? a.C : 0;
-            }
-        }
-    }
+    const bool narrow = narrow_reductions(conv_du_tiles(a.kh, a.kw, a.C) * kBM, a.O, a.R);
+    keep_slices(a.du_slices, &gu, narrow ? pu : nullptr, a.C);
+    keep_slices(a.dv_slices, &gv, narrow ? pv : nullptr);
     // dT = dY V  (per pixel)
     st = launch_prepared(gt, a.stream);
     if (st != PF_OK) return st;

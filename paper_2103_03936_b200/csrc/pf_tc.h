@@ -21,9 +21,8 @@ struct LinearArgs {
     cudaStream_t stream = nullptr;
     const void* bias = nullptr;   // forward: y = act((x U) V^T + bias)
     int act = 0;
-    // backward: where the fp32 slices of dU / dV were left in the workspace (filled in when the reduction
-    // over the batch was split across thread blocks; splits <= 1 otherwise), for callers that want the
-    // unrounded sums
+    // backward: where the fp32 slices of dU / dV were left in the workspace (partial null: nowhere), for callers that want
+    // the unrounded sums; a product that is one slice leaves only that
     struct Slices {
         const float* partial = nullptr;
         int splits = 0, bn = 0, tiles_x = 0, tiles_y = 0;

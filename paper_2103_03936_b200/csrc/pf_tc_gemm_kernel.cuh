@@ -32,7 +32,7 @@ struct GemmParams {
     long long ldc2, c2_gstride;
     const void* bias;        // unsplit plain products: C = act(A B + bias), bias [N] in bf16 or null
     int act;
-    float* partial;          // splits > 1: fp32 slices, one 128 x BN block per (tile, slice)
+    float* partial;          // fp32 slices, one 128 x BN block per (tile, slice); an unsplit product that has it leaves its one slice there instead of writing C
     unsigned int* counters;  // splits > 1: two counters per tile
     unsigned int* status;
     // Implicit-GEMM convolution (conv_mode 0 = plain product); blocks of pixels are cv_bh full-width rows of cv_nb
@@ -357,7 +357,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
         tc_fence_after();
         if (ok) {
             const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-            if (p.splits > 1) {
+            if (p.partial) {
                 // fp32 slice: straight from registers, [quadrant][4-column group][row][4], so that every store
                 // instruction of a warp is one run of 512 bytes; then the warp reports
                 float* dst = p.partial + (static_cast<size_t>(tile) * p.splits + bz) * (kBM * BN) +
@@ -374,7 +374,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                             make_uint4(v[g >> 3][4 * (g & 7)], v[g >> 3][4 * (g & 7) + 1], v[g >> 3][4 * (g & 7) + 2], v[g >> 3][4 * (g & 7) + 3]);
                 }
                 __syncwarp();
-                if (lane == 0) red_release_gpu(p.counters + 2 * tile, 1u);
+                if (lane == 0 && p.splits > 1) red_release_gpu(p.counters + 2 * tile, 1u);
             } else {
                 // every MMA has completed, so the pipeline stages are free: 32 x 33-word panel per warp
                 uint32_t* stg = reinterpret_cast<uint32_t*>(tiles) + (warp - 2) * (32 * 33);
