@@ -346,14 +346,14 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
 // 20 %, mostly 10 %).  A single CTA's 128 x 128 tile: 3.6 us of start and end and slice_us alone on its SM; 4.1 us and
 // 0.42 us per k-block beside another (its SM's load path is what it waits for).  A pair's 256 x 256 tile: 0.28 us per
 // k-block (the tensor cores), and 2 us of every tile but the first do not hide (the results' way to memory).  Output rows
-// that take no 16-byte stores: 2.4 us more per single tile, 3 per tile of a pair.
+// that take no 16-byte stores: 1.2 us more per single tile, 2.1 per tile of a pair.
 bool vector_rows(const void* C, int64_t ldc, int64_t gs) { return ldc % 8 == 0 && gs % 8 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0; }
 double single_us(const GemmLaunch* const* g, int count) {
     double ctas = 0, load = 0, alone = 0, beside = 0, shortest = 1e30;
     for (int i = 0; i < count; ++i) shortest = std::min<double>(shortest, g[i]->p.kb_per_split);
     for (int i = 0; i < count; ++i) {
         const double n = static_cast<double>(g[i]->grid.x) * g[i]->grid.y * g[i]->grid.z, kb = g[i]->p.kb_per_split;
-        const double sum = slice_us(g[i]->p.nkb_total, g[i]->p.splits) - 0.2 * kb + (g[i]->p.splits > 1 || vector_rows(g[i]->p.C, g[i]->p.ldc, g[i]->p.c_gstride) ? 0.0 : 2.4);
+        const double sum = slice_us(g[i]->p.nkb_total, g[i]->p.splits) - 0.2 * kb + (g[i]->p.splits > 1 || vector_rows(g[i]->p.C, g[i]->p.ldc, g[i]->p.c_gstride) ? 0.0 : 1.2);
         ctas += n;
         load += n * (0.42 * kb + 4.1 + sum);
         alone = std::max(alone, 0.2 * kb + sum);
@@ -367,7 +367,7 @@ double pairs_us(const PairJob* j, int count) {
     for (int i = 0; i < count; ++i) {
         const double n = static_cast<double>(ceil_div(j[i].M, 256) * ceil_div(j[i].N, 256)) * (j[i].sum_groups ? 1 : j[i].groups);
         const double kb = static_cast<double>(ceil_div(j[i].K, 64)) * (j[i].sum_groups ? j[i].groups : 1);
-        const double us = 0.28 * kb + (vector_rows(j[i].C, j[i].ldc, j[i].c_gs) ? 2.0 : 5.0);
+        const double us = 0.28 * kb + (vector_rows(j[i].C, j[i].ldc, j[i].c_gs) ? 2.0 : 4.1);
         tiles += n;
         load += n * us;
         longest = std::max(longest, us);

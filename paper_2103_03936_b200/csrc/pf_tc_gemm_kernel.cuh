@@ -135,12 +135,26 @@ __device__ __forceinline__ int output_row(const GemmParams& p, const TileOrigin&
     }
 }
 
+// Four columns of a row, of which `left` exist, in the widest stores that the address takes.
 __device__ __forceinline__ void store_columns(__nv_bfloat16* dst, uint32_t lo, uint32_t hi, int left) {
     unsigned short* d = reinterpret_cast<unsigned short*>(dst);
+    const uint32_t off = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(dst)) & 7u;
+    if (left >= 4) {
+        if (off == 0) {
+            *reinterpret_cast<uint2*>(d) = make_uint2(lo, hi);
+        } else if ((off & 2u) == 0) {
+            *reinterpret_cast<uint32_t*>(d) = lo;
+            *reinterpret_cast<uint32_t*>(d + 2) = hi;
+        } else {
+            d[0] = static_cast<unsigned short>(lo);
+            *reinterpret_cast<uint32_t*>(d + 1) = __funnelshift_r(lo, hi, 16);
+            d[3] = static_cast<unsigned short>(hi >> 16);
+        }
+        return;
+    }
     if (left > 0) d[0] = static_cast<unsigned short>(lo);
     if (left > 1) d[1] = static_cast<unsigned short>(lo >> 16);
     if (left > 2) d[2] = static_cast<unsigned short>(hi);
-    if (left > 3) d[3] = static_cast<unsigned short>(hi >> 16);
 }
 
 // One output tile (128 rows x BN columns) of C = A * B, or one slice of its contraction.
@@ -376,10 +390,9 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                 __syncwarp();
                 if (lane == 0 && p.splits > 1) red_release_gpu(p.counters + 2 * tile, 1u);
             } else {
-                // every MMA has completed, so the pipeline stages are free: 32 x 33-word panel per warp
-                uint32_t* stg = reinterpret_cast<uint32_t*>(tiles) + (warp - 2) * (32 * 33);
+                // every MMA has completed, so the pipeline stages are free: 16 KB of vector panels, then word panels
+                uint32_t* stg = reinterpret_cast<uint32_t*>(tiles + 16384) + (warp - 2) * (32 * kRaggedWords);
                 __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
-                const bool pair_ok = (p.ldc % 2) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 3) == 0;
                 const bool vec_ok = (p.ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0;
                 if (vec_ok) {
                     // 16-byte aligned rows: stage 32 rows x 64 columns (128 bytes per row, 16-byte pieces
@@ -432,24 +445,11 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                                 }
                             }
                         }
-                        if (p.C2) {          // the second copy, at a pitch that takes element pairs at best
-                            __nv_bfloat16* C2b = reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride;
-                            const bool pair2 = (p.ldc2 % 2) == 0 && (reinterpret_cast<uintptr_t>(C2b) & 3) == 0;
-                            const int c2 = n0 + c * 64 + 2 * lane;
-                            for (int j = 0; j < 32; ++j) {
-                                const int rowj = m0 + q * 32 + j;          // plain products only
-                                if (rowj >= p.M) break;
-                                uint32_t w;
-                                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(panel + static_cast<uint32_t>(j) * 128u +
-                                             ((static_cast<uint32_t>(lane >> 2) ^ static_cast<uint32_t>(j & 7)) << 4) + static_cast<uint32_t>(lane & 3) * 4u));
-                                __nv_bfloat16* d2 = C2b + static_cast<size_t>(rowj) * p.ldc2 + c2;
-                                if (pair2 && c2 + 1 < p.N) {
-                                    *reinterpret_cast<uint32_t*>(d2) = w;
-                                } else {
-                                    if (c2 < p.N) d2[0] = __ushort_as_bfloat16(static_cast<unsigned short>(w & 0xffffu));
-                                    if (c2 + 1 < p.N) d2[1] = __ushort_as_bfloat16(static_cast<unsigned short>(w >> 16));
-                                }
-                            }
+                        if (p.C2) {          // the second copy, at a pitch that the first cannot have
+                            stage_ragged(stg, v0, v1, lane);
+                            __syncwarp();
+                            store_ragged(stg, reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride, p.ldc2, n0 + c * 64,
+                                         p.N, lane, [&](int r) { return output_row<kMode>(p, org, bx, q * 32 + r); });
                         }
                         __syncwarp();
                     }
@@ -461,27 +461,9 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                     tmem_ld32(lane_base + c * 64 + 32, v1);
                     tmem_ld_wait();
                     if (kMode == 0 && (p.bias || p.act)) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
-#pragma unroll
-                    for (int w = 0; w < 16; ++w) {
-                        stg[lane * 33 + w] = pack_bf16x2(__uint_as_float(v0[2 * w]), __uint_as_float(v0[2 * w + 1]));
-                        stg[lane * 33 + 16 + w] = pack_bf16x2(__uint_as_float(v1[2 * w]), __uint_as_float(v1[2 * w + 1]));
-                    }
+                    stage_ragged(stg, v0, v1, lane);
                     __syncwarp();
-                    const int col = n0 + c * 64 + 2 * lane;
-#pragma unroll 4
-                    for (int j = 0; j < 32; ++j) {
-                        const int rowj = output_row<kMode>(p, org, bx, q * 32 + j);
-                        if (rowj >= 0) {
-                            const uint32_t w = stg[j * 33 + lane];
-                            __nv_bfloat16* dst = Cb + static_cast<size_t>(rowj) * p.ldc + col;
-                            if (pair_ok && col + 1 < p.N) {
-                                *reinterpret_cast<uint32_t*>(dst) = w;
-                            } else {
-                                if (col < p.N) dst[0] = __ushort_as_bfloat16(static_cast<unsigned short>(w & 0xffffu));
-                                if (col + 1 < p.N) dst[1] = __ushort_as_bfloat16(static_cast<unsigned short>(w >> 16));
-                            }
-                        }
-                    }
+                    store_ragged(stg, Cb, p.ldc, n0 + c * 64, p.N, lane, [&](int r) { return output_row<kMode>(p, org, bx, q * 32 + r); });
                     __syncwarp();
                 }
             }
@@ -519,7 +501,6 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     if (ctl->fix_ok) {
         __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
         __nv_bfloat16* C2b = p.C2 ? reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride : nullptr;
-        const bool vec8 = (p.ldc % 4) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 7) == 0;
         // units of 8 rows x 32 columns: a lane holds two 4-column groups of a row, 16 columns apart
         constexpr int kUnits = kBM / 8 * (BN / 32);
         constexpr size_t kSlice = static_cast<size_t>(kBM) * BN / 4;       // float4s
@@ -554,8 +535,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                 const int col = n0 + pc * 4 + j * 16;
                 __nv_bfloat16* dst = Cb + static_cast<size_t>(row) * p.ldc + col;
                 const uint32_t lo = pack_bf16x2(acc[j].x, acc[j].y), hi = pack_bf16x2(acc[j].z, acc[j].w);
-                if (vec8 && col + 3 < p.N) *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
-                else store_columns(dst, lo, hi, p.N - col);
+                store_columns(dst, lo, hi, p.N - col);
                 // the same sums once more, for a destination whose pitch the first cannot have
                 if (C2b) store_columns(C2b + static_cast<size_t>(row) * p.ldc2 + col, lo, hi, p.N - col);
             }

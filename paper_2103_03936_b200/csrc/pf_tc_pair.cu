@@ -40,7 +40,7 @@ constexpr int kPairStages = 6;
 constexpr uint32_t kHalfBytes = 16384;          // 128 rows x 64 bf16
 constexpr uint32_t kPairStageBytes = 2 * kHalfBytes;
 constexpr uint32_t kPairCols = 256;             // fp32 accumulator columns per CTA and buffer
-constexpr uint32_t kPairStaging = 32768;        // 8 epilogue warps x 4 KB store panels
+constexpr uint32_t kPairStaging = 8 * 32 * kRaggedWords * 4;        // 8 epilogue warps: 4 KB panels, or 33 words a row
 
 struct PairCtl {
     uint64_t full[kPairStages];
@@ -199,7 +199,7 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
 }
 
 // kForm 0: one ungrouped product with 16-byte aligned output rows (its parameters stay at fixed places and its
-// epilogue, which paces short contractions, has one form); 1: several; 2: grouped products.
+// epilogue, which paces short contractions, has one form); 1: several, or any output rows; 2: grouped products.
 template <int kForm>
 __global__ void __launch_bounds__(kPairThreads, 1)
 tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
@@ -352,7 +352,8 @@ tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
         // 32 rows x 64 columns staged per warp (128 bytes per row, 16-byte pieces XOR-swizzled by
         // the row), then four whole 128-byte row segments per store instruction
-        const uint32_t panel = smem_u32(staging) + static_cast<uint32_t>(warp - 2) * 4096u;
+        const uint32_t panel = smem_u32(staging) + static_cast<uint32_t>(warp - 2) * (32 * kRaggedWords * 4);
+        uint32_t* words = reinterpret_cast<uint32_t*>(staging) + (warp - 2) * (32 * kRaggedWords);
         const uint32_t own = panel + static_cast<uint32_t>(lane) * 128u, sw = static_cast<uint32_t>(lane & 7);
         const int sub = lane >> 3, piece = lane & 7;
         const uint32_t acc_empty_leader0 = map_to_cta(smem_u32(&ctl->acc_empty[0]), 0);
@@ -371,7 +372,6 @@ tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
             const int m0 = tm * 256 + static_cast<int>(rank) * 128, n0 = tn * 256;
             const size_t row_step = static_cast<size_t>(4) * p.ldc;
             const bool vec = (p.ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0;
-            const bool even = (p.ldc % 2) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 3) == 0;
             if (!mbar_wait_warp(smem_u32(&ctl->acc_full[buf]), (j >> 1) & 1u, abort_flag, L.status)) break;
             tc_fence_after();
 #pragma unroll 1
@@ -387,6 +387,13 @@ tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
                     if (lane == 0) mbar_arrive_cluster(acc_empty_leader0 + 8 * buf);
                 }
                 if (p.bias || p.act) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
+                if (kForm != 0 && !vec) {        // other pitches and alignments
+                    stage_ragged(words, v0, v1, lane);
+                    __syncwarp();
+                    store_ragged(words, Cb, p.ldc, n0 + c * 64, p.N, lane, [&](int r) { const int row = m0 + q * 32 + r; return row < p.M ? row : -1; });
+                    __syncwarp();
+                    continue;
+                }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     uint4 o;
@@ -402,29 +409,6 @@ tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
                     st_shared_v4(own + ((static_cast<uint32_t>(4 + u) ^ sw) << 4), o);
                 }
                 __syncwarp();
-                if (kForm != 0 && !vec) {
-                    // other pitches and alignments: a lane takes one pair of columns of each row
-                    const int col = n0 + c * 64 + 2 * lane, rows = min(32, p.M - m0 - q * 32);
-                    const bool in0 = col < p.N, in1 = col + 1 < p.N;
-                    unsigned short* d = reinterpret_cast<unsigned short*>(Cb) + static_cast<long long>(m0 + q * 32) * p.ldc + col;
-#pragma unroll 8
-                    for (int r = 0; r < 32; ++r) {
-                        const uint32_t w = ld_shared_u32(panel + static_cast<uint32_t>(r) * 128u +
-                                                         ((static_cast<uint32_t>(lane >> 2) ^ static_cast<uint32_t>(r & 7)) << 4) +
-                                                         static_cast<uint32_t>(lane & 3) * 4u);
-                        if (r < rows) {
-                            if (even && in1) {
-                                *reinterpret_cast<uint32_t*>(d) = w;
-                            } else {
-                                if (in0) d[0] = static_cast<unsigned short>(w & 0xffffu);
-                                if (in1) d[1] = static_cast<unsigned short>(w >> 16);
-                            }
-                        }
-                        d += p.ldc;
-                    }
-                    __syncwarp();
-                    continue;
-                }
                 const int col = n0 + c * 64 + piece * 8;
                 const int rin0 = q * 32 + sub;
                 __nv_bfloat16* dst = Cb + static_cast<size_t>(m0 + rin0) * p.ldc + col;
@@ -504,8 +488,7 @@ int gemm_pairs(const PairJob* jobs, int count, int first, cudaStream_t stream) {
     L.delay = extra == 0 || first == count ? 0 : static_cast<int>((L.p[0].nkb + L.p[first].nkb / 2) / L.p[first].nkb);
     L.status = device_status_ptr();
     const bool aligned = (reinterpret_cast<uintptr_t>(jobs[0].C) & 15) == 0 && jobs[0].ldc % 8 == 0;
-    if (count == 1 && !grouped && !aligned) return PF_ERR_UNSUPPORTED;
-    auto* kernel = grouped ? tc_gemm_pair_kernel<2> : count > 1 ? tc_gemm_pair_kernel<1> : tc_gemm_pair_kernel<0>;
+    auto* kernel = grouped ? tc_gemm_pair_kernel<2> : count > 1 || !aligned ? tc_gemm_pair_kernel<1> : tc_gemm_pair_kernel<0>;
     const size_t smem = 1024 + 1024 + kPairStaging + static_cast<size_t>(kPairStages) * kPairStageBytes;
     if (allow_smem(kernel, smem) != cudaSuccess) return PF_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};

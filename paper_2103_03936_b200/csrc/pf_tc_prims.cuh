@@ -265,6 +265,45 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// Results whose rows TMA and 16-byte stores cannot take (any pitch, any alignment): a warp stages 32 rows x 64 columns as
+// words, 33 to a row (free of bank conflicts both ways), and stores each row's whole 16-byte pieces of the DESTINATION,
+// assembled from five words with a funnel shift, four rows to an instruction; what is left of a row in front and behind is
+// stored by elements.  (One pair of columns per lane, a row per instruction: 700 x 1504 over 376, rows of even pitch 8.0 us,
+// of odd pitch 8.7; this way 7.0 and 7.1, against 6.0 with 16-byte stores.)
+constexpr int kRaggedWords = 33;
+__device__ __forceinline__ void stage_ragged(uint32_t* stg, const uint32_t (&v0)[32], const uint32_t (&v1)[32], int lane) {
+#pragma unroll
+    for (int w = 0; w < 16; ++w) {
+        stg[lane * kRaggedWords + w] = pack_bf16x2(__uint_as_float(v0[2 * w]), __uint_as_float(v0[2 * w + 1]));
+        stg[lane * kRaggedWords + 16 + w] = pack_bf16x2(__uint_as_float(v1[2 * w]), __uint_as_float(v1[2 * w + 1]));
+    }
+}
+// `row_of(r)`: row of C that staged row r goes to, negative = none; columns col0 .. col0 + 63, clipped at n.
+template <typename RowOf>
+__device__ __forceinline__ void store_ragged(const uint32_t* stg, __nv_bfloat16* C, long long ldc, int col0, int n, int lane, RowOf row_of) {
+    const int p = lane & 7, count = min(64, n - col0);
+#pragma unroll 2
+    for (int i = 0; i < 8; ++i) {
+        const int r = i * 4 + (lane >> 3), row = row_of(r);
+        if (row < 0) continue;
+        unsigned short* d = reinterpret_cast<unsigned short*>(C) + static_cast<long long>(row) * ldc + col0;
+        const uint32_t* words = stg + r * kRaggedWords;
+        const unsigned short* elems = reinterpret_cast<const unsigned short*>(words);
+        const int head = static_cast<int>((0u - static_cast<uint32_t>(reinterpret_cast<uintptr_t>(d))) & 15u) >> 1;     // elements before the first whole piece
+        const int e = head + 8 * p;
+        if (e + 8 <= count) {
+            const uint32_t* w = words + (e >> 1);
+            const uint32_t bit = (e & 1) * 16;
+            const uint32_t w0 = w[0], w1 = w[1], w2 = w[2], w3 = w[3], w4 = w[4];       // (the last one may be the row's padding word)
+            *reinterpret_cast<uint4*>(d + e) = make_uint4(__funnelshift_r(w0, w1, bit), __funnelshift_r(w1, w2, bit), __funnelshift_r(w2, w3, bit),
+                                                          __funnelshift_r(w3, w4, bit));
+        }
+        if (p < min(head, count)) d[p] = elems[p];
+        const int t = count > head ? head + ((count - head) & ~7) + p : count;
+        if (t < count) d[t] = elems[t];
+    }
+}
+
 // Bias and activation (1 = max(0, .)) on 64 accumulator columns col .. col + 63 of a row, before the rounding: every
 // lane fetches two of the columns' values (bf16), the columns take them from the lanes.
 __device__ __forceinline__ void bias_act64(uint32_t (&v0)[32], uint32_t (&v1)[32], const void* bias, int act, int col, int n, int lane) {

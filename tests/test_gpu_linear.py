@@ -316,3 +316,38 @@ def test_re_pitch_copies_beyond_two_to_the_31_pieces():
     assert pf.pf_last_device_status() == 0
     del x, y
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("m,k,n,r", [(130, 64, 1, 16), (300, 64, 63, 16), (300, 72, 129, 40), (160, 64, 200, 392), (4200, 64, 2561, 256)])
+@pytest.mark.parametrize("base,pad", [(0, 1), (1, 0), (3, 5), (4, 4), (7, 2)])
+def test_output_rows_of_any_alignment(m, k, n, r, base, pad):
+    """Output rows that start anywhere and whose pitch is anything hold, bit for bit, what rows on 16-byte boundaries
+    hold, and nothing around them is touched (single tiles, CTA pairs, y and the stash)."""
+    d = wl.LinearCase("rows", m, k, n, r, wl.BF16, 71).generate()
+    x, U, V = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V"))
+
+    def rows(cols, start, ld):
+        buf = torch.full((start + m * ld + 64,), -7.0, dtype=torch.bfloat16, device="cuda")
+        return buf, buf[start:start + m * ld].view(m, ld)[:, :cols]
+
+    _, y0 = rows(n, 64, (n + 7) // 8 * 8)
+    _, T0 = rows(r, 64, (r + 7) // 8 * 8)
+    pf.pf_lowrank_linear_fwd(x, U, V, y=y0, T_stash=T0)
+    by, y1 = rows(n, 64 + base, n + pad)
+    bT, T1 = rows(r, 64 + base, r + pad + (r + pad + 1) % 2)        # an odd pitch: the second copy
+    pf.pf_lowrank_linear_fwd(x, U, V, y=y1, T_stash=T1)
+    torch.cuda.synchronize()
+    assert_close(y0, oracle.linear_fwd(d["x"], d["U"], d["V"])[0], wl.BF16, f"{m}x{k}->{n} r{r} y")
+    for want, got, buf in ((y0, y1, by), (T0, T1, bT)):
+        assert torch.equal(want, got)
+        got.fill_(-7.0)
+        assert bool((buf == -7.0).all()), "written outside the rows"
+    assert pf.pf_last_device_status() == 0
+
+
+@pytest.mark.parametrize("m,k,n,r", [(1100, 256, 264, 40), (1216, 264, 256, 40), (4096, 256, 256, 256), (2050, 520, 520, 200), (700, 2056, 1032, 264),
+                                     (2500, 1032, 4104, 520)])
+def test_whole_and_split_contractions_and_pairs(m, k, n, r):
+    """Either side of the lengths from which contractions are split, and of the sizes from which products run on CTA
+    pairs; dU and dV split by themselves beside a product that is whole."""
+    run_case(wl.LinearCase("forms", m, k, n, r, wl.BF16, 72), blocks=True)
