@@ -14,7 +14,7 @@ namespace pf {
 namespace tc {
 namespace {
 
-int64_t pad4(int64_t v) { return (v + 3) / 4 * 4; }
+int64_t f32_pitch(int64_t v) { return v > 16 ? (v + 31) / 32 * 32 : (v + 3) / 4 * 4; }      // whole 128-byte lines, as row_pitch
 bool f32_tma_ok(const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 4 == 0 && ld * 4 < (1LL << 40); }
 
 // fp32 tensor maps with boxes of 32 columns (128 bytes): rank 2 = [rows, cols], rank 3 = [planes][rows][cols]
@@ -238,14 +238,14 @@ bool f32_stage(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& scr
     *out = Staged32{p, ld};
     if (f32_tma_ok(p, ld)) return true;
     if (cols % 4 == 0) return false;      // the workspace query reserves repack room only for ragged widths
-    const int64_t ldp = pad4(cols);
+    const int64_t ldp = f32_pitch(cols);
     jobs[(*count)++] = RepackJob{p, 2 * ld, scratch, 2 * ldp, rows, 2 * cols};
     *out = Staged32{scratch, ldp};
     scratch += align_up(static_cast<size_t>(rows) * ldp * 4, 256);
     return true;
 }
-size_t f32_room(int64_t rows, int64_t cols) { return cols % 4 == 0 ? 0 : align_up(static_cast<size_t>(rows) * pad4(cols) * 4, 256); }
-size_t f32_mat(int64_t rows, int64_t cols) { return align_up(static_cast<size_t>(rows) * pad4(cols) * 4, 256); }
+size_t f32_room(int64_t rows, int64_t cols) { return cols % 4 == 0 ? 0 : align_up(static_cast<size_t>(rows) * f32_pitch(cols) * 4, 256); }
+size_t f32_mat(int64_t rows, int64_t cols) { return align_up(static_cast<size_t>(rows) * f32_pitch(cols) * 4, 256); }
 
 // The products of the two layers in the order they are launched, planned from the sizes alone.
 struct F32Fwd {
@@ -321,7 +321,7 @@ int f32_linear_fwd(const LinearArgs& a, int* handled, size_t room) {
     // T: the stash itself when TMA can read it back, else scratch; the first product then writes the stash beside it
     const bool direct = a.T && f32_tma_ok(a.T, a.ldt);
     float* T = direct ? static_cast<float*>(a.T) : reinterpret_cast<float*>(ws);
-    const int64_t ldT = direct ? a.ldt : pad4(a.r);
+    const int64_t ldT = direct ? a.ldt : f32_pitch(a.r);
     ws += f32_mat(a.m, a.r);
     F32Launch l1, l2;
     if (!f32_prepare(f.t, {x.p, x.ld, false}, {U.p, U.ld, true}, T, ldT, reinterpret_cast<float*>(ws), &l1.ta[0], &l1.tb[0], &l1.p[0]) ||
@@ -354,14 +354,14 @@ int f32_linear_bwd(const LinearArgs& a, int* handled) {
         if (f32_tma_ok(a.T, a.ldt)) {
             T = Staged32{a.T, a.ldt};
         } else {
-            jobs[nj++] = RepackJob{a.T, 2 * a.ldt, Tbuf, 2 * pad4(a.r), a.m, 2 * a.r};
-            T = Staged32{Tbuf, pad4(a.r)};
+            jobs[nj++] = RepackJob{a.T, 2 * a.ldt, Tbuf, 2 * f32_pitch(a.r), a.m, 2 * a.r};
+            T = Staged32{Tbuf, f32_pitch(a.r)};
         }
     } else {
-        T = Staged32{Tbuf, pad4(a.r)};
+        T = Staged32{Tbuf, f32_pitch(a.r)};
     }
     float* G = reinterpret_cast<float*>(ws);
-    const int64_t ldG = pad4(a.r);
+    const int64_t ldG = f32_pitch(a.r);
     ws += f32_mat(a.m, a.r);
     float* p1 = reinterpret_cast<float*>(ws);
     ws += std::max(b.t.partial_bytes(), b.g.partial_bytes());
@@ -371,7 +371,7 @@ int f32_linear_bwd(const LinearArgs& a, int* handled) {
     F32Launch lt, la, lb;
     bool ok = true;
     if (!a.T)
-        ok = f32_prepare(b.t, {x.p, x.ld, false}, {U.p, U.ld, true}, reinterpret_cast<float*>(Tbuf), pad4(a.r), p1, &lt.ta[0], &lt.tb[0], &lt.p[0]);
+        ok = f32_prepare(b.t, {x.p, x.ld, false}, {U.p, U.ld, true}, reinterpret_cast<float*>(Tbuf), f32_pitch(a.r), p1, &lt.ta[0], &lt.tb[0], &lt.p[0]);
     ok = ok && f32_prepare(b.g, {dY.p, dY.ld, false}, {V.p, V.ld, true}, G, ldG, p1, &la.ta[0], &la.tb[0], &la.p[0]) &&
          f32_prepare(b.dv, {dY.p, dY.ld, true}, {T.p, T.ld, true}, static_cast<float*>(a.dV), a.lddv, pv, &la.ta[1], &la.tb[1], &la.p[1]) &&
          f32_prepare(b.du, {x.p, x.ld, true}, {G, ldG, true}, static_cast<float*>(a.dU), a.lddu, pu, &lb.ta[0], &lb.tb[0], &lb.p[0]);
