@@ -110,13 +110,27 @@ void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t nkb_u, int64_t 
     if (tu < 1 || tv < 1 || nkb_u < 1 || nkb_v < 1 || tu + tv > num_sms()) return;
     double best = std::max(slice_us(nkb_u, 1), slice_us(nkb_v, 1));
     if (best < slice_us(1, 64)) return;      // shorter than any sum of slices
-    for (int64_t a = 1; a <= 64 && a <= nkb_u && tu * a + tv <= num_sms(); ++a) {
+    auto consider = [&](int64_t a) {         // a slices of dU, and what is left of the machine to dV; true: dU is not the longer one
         const double u = slice_us(nkb_u, a);
         const int64_t most = std::min(std::min<int64_t>(64, nkb_v), (num_sms() - tu * a) / tv);
-        const int64_t b = slice_us(nkb_v, most) < slice_us(nkb_v, 1) ? most : 1;
-        const double longest = std::max(u, slice_us(nkb_v, b));
-        if (longest < best) { best = longest; *su = static_cast<int>(a); *sv = static_cast<int>(b); }
+        const double whole = slice_us(nkb_v, 1), cut = slice_us(nkb_v, most), v = std::min(whole, cut);
+        if (std::max(u, v) < best) {
+            best = std::max(u, v);
+            *su = static_cast<int>(a);
+            *sv = static_cast<int>(cut < whole ? most : 1);
+        }
+        return u <= v;
+    };
+    consider(1);
+    // from two slices on, more slices shorten dU and lengthen dV: the best count is where the two meet
+    int64_t lo = 2, hi = std::min(std::min<int64_t>(64, nkb_u), (num_sms() - tv) / tu);
+    if (lo > hi) return;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) / 2;
+        if (consider(mid)) hi = mid; else lo = mid + 1;
     }
+    consider(lo);
+    if (lo > 2) consider(lo - 1);
 }
 
 // Slices of dU (k x r) and dV (n x r) in the backward of the linear layer, and whether dV runs BESIDE

@@ -126,3 +126,14 @@ def test_unpack_round_trip_at_model_scale():
     with pytest.raises(pf.PfError) as e:          # a list longer than the flat buffer is refused
         pf.pf_unpack_factor_grads(flat[:100], back)
     assert e.value.status == 3
+
+
+@pytest.mark.parametrize("count", [31, 32, 33, 512, 513])
+def test_lists_around_the_table_sizes(count):
+    """Either side of the lengths from which a list takes the long table, or two launches."""
+    check_unpack([(7 * i) % 41 for i in range(count)], wl.BF16)
+    tensors = [torch.randn(1 + (5 * i) % 37, device="cuda").to(torch.bfloat16) for i in range(count)]
+    before = pf.pf_launch_count()
+    flat, _ = pf.pf_pack_factor_grads(tensors)
+    assert pf.pf_launch_count() - before == (count + 511) // 512
+    assert torch.equal(flat, torch.cat(tensors))
