@@ -208,49 +208,49 @@ struct RepackBatchArgs {
     unsigned int item_end[kRepackJobs];   // running total of items up to and including job j
     int count;
 };
-__device__ __forceinline__ uint4 shifted_vector(const uint4 lo, const uint4 hi, unsigned q, unsigned bit) {
-    unsigned w0, w1, w2, w3, w4;
-    switch (q) {
-        case 0: w0 = lo.x; w1 = lo.y; w2 = lo.z; w3 = lo.w; w4 = hi.x; break;
-        case 1: w0 = lo.y; w1 = lo.z; w2 = lo.w; w3 = hi.x; w4 = hi.y; break;
-        case 2: w0 = lo.z; w1 = lo.w; w2 = hi.x; w3 = hi.y; w4 = hi.z; break;
-        default: w0 = lo.w; w1 = hi.x; w2 = hi.y; w3 = hi.z; w4 = hi.w; break;
-    }
-    return make_uint4(__funnelshift_r(w0, w1, bit), __funnelshift_r(w1, w2, bit), __funnelshift_r(w2, w3, bit),
-                      __funnelshift_r(w3, w4, bit));
+// Bytes [4 q + bit / 8, + 16) of the window lo:hi.
+__device__ __forceinline__ uint4 shifted_vector(const uint4 o, const uint4 h, unsigned q, unsigned bit) {
+    const bool q1 = q & 1, q2 = q & 2;
+    const unsigned x0 = q2 ? o.z : o.x, x1 = q2 ? o.w : o.y, x2 = q2 ? h.x : o.z, x3 = q2 ? h.y : o.w, x4 = q2 ? h.z : h.x, x5 = q2 ? h.w : h.y;
+    const unsigned w0 = q1 ? x1 : x0, w1 = q1 ? x2 : x1, w2 = q1 ? x3 : x2, w3 = q1 ? x4 : x3, w4 = q1 ? x5 : x4;
+    return make_uint4(__funnelshift_r(w0, w1, bit), __funnelshift_r(w1, w2, bit), __funnelshift_r(w2, w3, bit), __funnelshift_r(w3, w4, bit));
 }
 __global__ void __launch_bounds__(256)
 repack_multi_kernel(const __grid_constant__ RepackBatchArgs a) {
-    const unsigned int total = a.item_end[a.count - 1];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    for (unsigned int it = blockIdx.x * blockDim.x + threadIdx.x; it < total; it += gridDim.x * blockDim.x) {
+    const unsigned int total = a.item_end[a.count - 1], step = gridDim.x * blockDim.x;
+    const unsigned short* sp = nullptr;
+    unsigned short* to = nullptr;
+    int left = 0;
+    auto place = [&](unsigned int it) {
         int j = 0;
         while (j + 1 < a.count && it >= a.item_end[j]) ++j;
-        const unsigned int local = it - (j > 0 ? a.item_end[j - 1] : 0u);
-        const unsigned int ppr = static_cast<unsigned int>(a.pieces_per_row[j]);
+        const unsigned int local = it - (j > 0 ? a.item_end[j - 1] : 0u), ppr = static_cast<unsigned int>(a.pieces_per_row[j]);
         const unsigned int row = local / ppr;
         const int c0 = static_cast<int>(local - row * ppr) * 8;
         const unsigned int g = a.gs_src[j] ? row / static_cast<unsigned int>(a.rows[j]) : 0u;
-        const unsigned short* sp = a.src[j] + g * a.gs_src[j] + (row - g * static_cast<unsigned int>(a.rows[j])) * a.ld_src[j] + c0;
-        const int left = a.cols[j] - c0;
-        uint4 o;
-        if (left >= 8) {
-            const unsigned int sh = static_cast<unsigned int>(reinterpret_cast<uintptr_t>(sp)) & 15u;
-            const uint4* v = reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(sp) - sh);
-            const uint4 lo = __ldg(v);
-            o = lo;
-            if (sh) o = shifted_vector(lo, __ldg(v + 1), sh >> 2, (sh & 3u) * 8u);
-        } else {
-            unsigned short e[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) e[i] = i < left ? sp[i] : static_cast<unsigned short>(0);
-            o.x = e[0] | (static_cast<unsigned int>(e[1]) << 16);
-            o.y = e[2] | (static_cast<unsigned int>(e[3]) << 16);
-            o.z = e[4] | (static_cast<unsigned int>(e[5]) << 16);
-            o.w = e[6] | (static_cast<unsigned int>(e[7]) << 16);
+        sp = a.src[j] + g * a.gs_src[j] + (row - g * static_cast<unsigned int>(a.rows[j])) * a.ld_src[j] + c0;
+        to = a.dst[j] + row * a.ld_dst[j] + c0;
+        left = a.cols[j] - c0;
+    };
+    unsigned int it = blockIdx.x * blockDim.x + threadIdx.x;
+    if (it < total) place(it);            // (reads the kernel's parameters only: beside the previous kernel's tail)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    while (it < total) {
+        // the aligned vectors that hold at least one byte of the piece
+        const unsigned int sh = static_cast<unsigned int>(reinterpret_cast<uintptr_t>(sp)) & 15u;
+        const uint4* v = reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(sp) - sh);
+        const uint4 lo = __ldg(v);
+        uint4 hi = make_uint4(0u, 0u, 0u, 0u);
+        if (static_cast<int>(sh) + 2 * min(left, 8) > 16) hi = __ldg(v + 1);
+        uint4 o = shifted_vector(lo, hi, sh >> 2, (sh & 3u) * 8u);
+        if (left < 8) {                   // zeros behind the row's end
+            auto keep = [&](int e) { return (e < left ? 0xffffu : 0u) | (e + 1 < left ? 0xffff0000u : 0u); };
+            o.x &= keep(0); o.y &= keep(2); o.z &= keep(4); o.w &= keep(6);
         }
-        *reinterpret_cast<uint4*>(a.dst[j] + row * a.ld_dst[j] + c0) = o;
+        *reinterpret_cast<uint4*>(to) = o;
+        it += step;
+        if (it < total) place(it);
     }
 }
 
