@@ -182,7 +182,7 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.stream = stream;
     a.bias = bias; a.act = act;
     size_t need = w.total;
-    const bool is_small = dtype == PF_BF16 ? small::linear_fwd_fits(m, k, n, r) : small::f32_fits(m, k, n, r, false);
+    const bool is_small = dtype == PF_BF16 ? small::linear_fwd_fits(m, k, n, r) && !tc::few_rows_fused(a) : small::f32_fits(m, k, n, r, false);
     if (exact_need && is_small) {
         need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * dtype_size(dtype);
     } else if (exact_need) {

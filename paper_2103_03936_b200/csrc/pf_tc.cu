@@ -497,10 +497,20 @@ int stage_operand(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& 
     scratch += align_up(static_cast<size_t>(rows) * ldp * 2, 256);
     return 0;
 }
-// The fused chain pays off once there are enough 128-row tiles to fill the machine, and while the
+// The backward's fused chain pays off once there are enough 128-row tiles to fill the machine, and while the
 // rank is small enough for the layer to be bound by memory traffic: from r = 256 up the two
 // products are tensor-bound and run faster unfused on CTA pairs (the intermediate is only m x r).
 bool use_chain(int64_t m, int64_t r) { return m >= 2048 && r <= 192; }
+// The forward's fused kernel is one launch instead of two, so it takes smaller batches too, while its first product, which
+// one block contracts alone where the unfused one is split over the SMs, is short.  Fused against unfused, caches warm:
+// 300 x 512 -> 128 -> 2048: 6.4 against 8.7 us; 1000 x 1536 -> 128 -> 1536: 10.5 / 11.7; 500 x 2048 -> 128 -> 2048: 11.7 / 11.7;
+// 1024 x 4096 -> 128 -> 1024: 18.6 / 12.1; r 256, 1024 x 1024 -> 1024: 11.8 / 10.3.  Up to 32 rows against the kernels of
+// pf_small.cu: 20 x 512 -> 128 -> 2048: 5.9 / 6.8; 8 x 1024 -> 64 -> 1024: 6.5 / 5.4.  A stash that TMA cannot write would take
+// a launch of its own again.
+bool use_chain_fwd(const LinearArgs& a) {
+    if (a.r > 192 || !tma_ok(a.y, a.ldy)) return false;
+    return a.m >= 2048 || (a.k <= 1536 && (!a.T || tma_ok(a.T, a.ldt)));
+}
 
 size_t repack_room(int64_t rows, int64_t cols) {
     return cols % 8 == 0 ? 0 : align_up(static_cast<size_t>(rows) * row_pitch(cols) * 2, 256);
@@ -590,9 +600,14 @@ size_t linear_fwd_need(const LinearArgs& a, bool* handles) {
     const size_t t_bytes = align_up(static_cast<size_t>(a.m) * row_pitch(a.r) * 2, 256);
     const bool stash_direct = a.T && tma_ok(a.T, a.ldt);
     ChainPlan plan;
-    if (use_chain(a.m, a.r) && tma_ok(a.y, a.ldy) && chain_plan(a.m, a.k, a.n, a.r, true, &plan))
+    if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan))
         return room + ((a.T && !stash_direct) ? t_bytes : 0);
     return room + t_bytes + align_up(partial_bytes(a.m, a.r, pick_splits(a.m, a.r, pick_bn(a.r), a.k)), 256);
+}
+
+// Whether a forward of few rows runs on the fused kernel, which takes its operands as they are, instead of pf_small.cu.
+bool few_rows_fused(const LinearArgs& a) {
+    return encode_fn() != nullptr && a.k <= 512 && a.n <= (1 << 22) && use_chain_fwd(a) && tma_ok(a.x, a.ldx) && tma_ok(a.U, a.ldu) && tma_ok(a.V, a.ldv);
 }
 
 int linear_fwd(const LinearArgs& a, int* handled) {
@@ -617,7 +632,7 @@ int linear_fwd(const LinearArgs& a, int* handled) {
     if (stash_direct) { T = a.T; ldT = a.ldt; }
     ChainPlan plan;
     bool stash_written = false;   // the stash at its own (TMA-unreadable) pitch came out of the first product
-    if (use_chain(a.m, a.r) && tma_ok(a.y, a.ldy) && chain_plan(a.m, a.k, a.n, a.r, true, &plan)) {
+    if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan)) {
         // one fused kernel; the intermediate leaves the chip only if a stash was asked for
         st = chain(x.p, x.ld, a.m, a.k, U.p, U.ld, a.r, V.p, V.ld, a.n, a.y, a.ldy, a.T ? T : nullptr, ldT,
                    a.stream, nullptr, 0, a.bias, a.act);

@@ -114,6 +114,7 @@ size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, in
 void reset_fix_counters();  // clears the slice-sum counters (after PF_ERR_TIMEOUT)
 size_t linear_fwd_need(const LinearArgs& a, bool* handles);   // bytes of a.ws the forward really touches
 int linear_fwd(const LinearArgs& a, int* handled);
+bool few_rows_fused(const LinearArgs& a);     // a forward that small::linear_fwd fits, but the fused kernel takes
 int linear_bwd(const LinearArgs& a, int* handled);
 
 // fp32 storage (pf_tc_f32.cu).  `room`: bytes available at a.ws (a call that does not fit is declined).

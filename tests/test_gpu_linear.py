@@ -351,3 +351,29 @@ def test_whole_and_split_contractions_and_pairs(m, k, n, r):
     """Either side of the lengths from which contractions are split, and of the sizes from which products run on CTA
     pairs; dU and dV split by themselves beside a product that is whole."""
     run_case(wl.LinearCase("forms", m, k, n, r, wl.BF16, 72), blocks=True)
+
+
+@pytest.mark.parametrize("m,k,n,r", [(1, 8, 8, 8), (5, 512, 136, 24), (32, 512, 1032, 192), (33, 1536, 264, 64), (129, 72, 4104, 136), (2047, 1536, 128, 16)])
+def test_fused_forward_of_smaller_batches(m, k, n, r):
+    """Forward with k <= 1536 (512 up to 32 rows) and r <= 192: one launch; one column more, a rank more or a stash that TMA
+    cannot write take the unfused kernels."""
+    case = wl.LinearCase("fused small", m, k, n, r, wl.BF16, 73)
+    run_case(case, blocks=m > 100)
+    d = case.generate()
+    x, U, V = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V"))
+    before = pf.pf_launch_count()
+    pf.pf_lowrank_linear_fwd(x, U, V, want_stash=True)
+    assert pf.pf_launch_count() - before == 1
+    before = pf.pf_launch_count()
+    pf.pf_lowrank_linear_fwd(x, U, V, T_stash=Guarded((m, r), wl.BF16, ld=r + 4).t)
+    assert pf.pf_launch_count() - before == 2
+
+
+@pytest.mark.parametrize("m,k,n,r", [(32, 520, 136, 24), (40, 1544, 136, 24), (300, 512, 136, 200)])
+def test_forward_beyond_the_fused_sizes(m, k, n, r):
+    case = wl.LinearCase("unfused small", m, k, n, r, wl.BF16, 74)
+    run_case(case)
+    d = case.generate()
+    before = pf.pf_launch_count()
+    pf.pf_lowrank_linear_fwd(*(dev(d[k_], wl.BF16) for k_ in ("x", "U", "V")))
+    assert pf.pf_launch_count() - before == 2
