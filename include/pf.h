@@ -226,7 +226,7 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
  * matrices themselves are as in the ungrouped calls.  sx = 0 means ONE input x shared by all groups
  * (the gates of an LSTM all read the same x_t); factors and outputs are always per group.
  * With bf16 and 16-byte aligned pointers, pitches and strides the whole call is two launches
- * (all x_g U_g, then all T_g V_g^T), whatever `groups`; ragged widths (not a multiple of 8) add one launch
+ * (all x_g U_g, then all T_g V_g^T, or half of the groups each), whatever `groups`; ragged widths (not a multiple of 8) add one launch
  * that copies those operands to 16-byte pitches; other layouts, and fp32, run group by group through the
  * ungrouped kernels (same results, more launches).
  *

@@ -103,9 +103,9 @@ int pick_bn(int64_t N) { return N <= 64 ? 64 : 128; }
 // Slice counts for two products that share one launch (dU: Mu x N over nkb_u k-blocks, dV: Mv x N over nkb_v):
 // all CTAs should fit one wave and finish together, so the time of the longest CTA is
 // minimised subject to tiles_u * su + tiles_v * sv <= SM count.
-void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t nkb_u, int64_t nkb_v, int* su, int* sv) {
+void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t nkb_u, int64_t nkb_v, int* su, int* sv, int groups = 1) {
     const int bn = pick_bn(N);
-    const int64_t tu = ceil_div(Mu, kBM) * ceil_div(N, bn), tv = ceil_div(Mv, kBM) * ceil_div(N, bn);
+    const int64_t tu = ceil_div(Mu, kBM) * ceil_div(N, bn) * groups, tv = ceil_div(Mv, kBM) * ceil_div(N, bn) * groups;
     *su = 1; *sv = 1;
     if (tu < 1 || tv < 1 || nkb_u < 1 || nkb_v < 1 || tu + tv > num_sms()) return;
     double best = std::max(slice_us(nkb_u, 1), slice_us(nkb_v, 1));
@@ -844,6 +844,25 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     const bool stash_direct = a.T && grouped_ok(a.T, a.ldt, a.st);
     void* T = stash_direct ? a.T : static_cast<void*>(Tbuf);
     const int64_t ldT = stash_direct ? a.ldt : row_pitch(a.r), sT = stash_direct ? a.st : a.m * row_pitch(a.r);
+    // The fused kernel where it pays for one group (see use_chain_fwd; k up to 1024, as the groups share the SMs), in two
+    // launches of half of the groups each (the call's launches are documented as two) that run side by side.  Not for more
+    // than two waves of the smallest tiles, whose starts the two products hide better.  Against two products one after the
+    // other: 4 x (1024 x 512 -> 128 -> 512): 13.0 -> 8.3 us, 4 x (8192 x 512 -> 128 -> 512): 26.7 -> 19.3, 2 x (7666 x 1976 ->
+    // 120 -> 1976): 51 -> 42; 4 x (185 x 1536 -> 192 -> 1536): 12.1 -> 12.8; 8 x (4789 x 72 -> 8 -> 72): 18.3 -> 18.8.
+    ChainPlan plan;
+    if (a.r <= 192 && (a.m >= 2048 || a.k <= 1024) && (a.k + a.n >= 512 || ceil_div(a.m, kBM) * a.groups <= 2 * num_sms()) && grouped_ok(a.y, a.ldy, a.sy) && (!a.T || stash_direct) &&
+        chain_plan(a.m, a.k, a.n, a.r, true, &plan, 128, 0, a.groups)) {
+        *handled = 1;
+        int st = repacks.flush(a.stream);
+        const int half[3] = {0, a.groups / 2, a.groups};
+        auto at = [](const void* p, int64_t gs, int g) { return const_cast<char*>(static_cast<const char*>(p)) + static_cast<size_t>(g) * gs * 2; };
+        for (int h = 0; h < 2 && st == PF_OK; ++h) {
+            const int g = half[h];
+            st = chain_groups(half[h + 1] - g, a.groups, at(x.p, x.gs, g), x.ld, x.gs, a.m, a.k, at(U.p, U.gs, g), U.ld, U.gs, a.r, at(V.p, V.gs, g), V.ld, V.gs, a.n,
+                              at(a.y, a.sy, g), a.ldy, a.sy, a.T ? at(a.T, a.st, g) : nullptr, a.ldt, a.st, h == 1, a.stream);
+        }
+        return st;
+    }
     GemmLaunch g1, g2;
     const Grouping gt{a.groups, sT, false}, gy{a.groups, a.sy, false};
     int st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, T, ldT, gp.s1, p1, nullptr, &g1, &gt);
@@ -884,6 +903,19 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
         stage_groups(a.dY, a.lddy, a.sdy, a.groups, false, a.m, a.n, ws, &dY, &repacks) ||
         (a.T && stage_groups(a.T, a.ldt, a.st, a.groups, false, a.m, a.r, ws, &T, &repacks)))
         return PF_OK;
+    // The fused kernel for G and dX as in linear_bwd, then dU and dV, whose slices have to fit the machine together:
+    // 2 x (8000 x 1024 -> 64 -> 256): 44.6 -> 23.4 us, 4 x (8192 x 512 -> 128 -> 512): 48.8 -> 42.1, 2 x (7666 x 1976 -> 120 -> 1976):
+    // 104 -> 78.
+    ChainPlan plan;
+    const bool fused = !shared_x && a.dX && use_chain(a.m, a.r) && grouped_ok(a.dX, a.lddx, a.sdx) && chain_plan(a.m, a.n, a.k, a.r, true, &plan, 128, 0, a.groups);
+    int su = gp.su, sv = gp.sv;
+    if (fused) {
+        const int64_t nkb = ceil_div(a.m, kBK);
+        int su2, sv2;
+        pick_pair_splits(a.k, a.n, a.r, nkb, nkb, &su2, &sv2, a.groups);
+        su = std::min(su, su2);
+        sv = std::min(sv, sv2);
+    }
     GemmLaunch gT, gG, gV, gU, gX;
     const Grouping gw{a.groups, sW, false}, gdv{a.groups, a.sdv, false}, gdu{a.groups, a.sdu, false};
     const Grouping gdx{a.groups, shared_x ? 0 : a.sdx, shared_x};
@@ -891,8 +923,8 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     if (!a.T) st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, Tbuf, ldW, gp.s1, p1, nullptr, &gT, &gw);
     // the recomputed T and G share the slice buffer p1: they are separate launches, one after the other
     if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, false, dY.gs}, {V.p, V.ld, true, V.gs}, a.m, a.r, a.n, Gbuf, ldW, gp.sg, p1, nullptr, &gG, &gw);
-    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, true, dY.gs}, {T.p, T.ld, true, T.gs}, a.n, a.r, a.m, a.dV, a.lddv, gp.sv, pv, nullptr, &gV, &gdv);
-    if (st == PF_OK) st = gemm_prepare({x.p, x.ld, true, x.gs}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, gp.su, pu, nullptr, &gU, &gdu);
+    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, true, dY.gs}, {T.p, T.ld, true, T.gs}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gV, &gdv);
+    if (st == PF_OK) st = gemm_prepare({x.p, x.ld, true, x.gs}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gU, &gdu);
     if (st == PF_OK && a.dX)
         st = gemm_prepare({Gbuf, ldW, false, sW}, {U.p, U.ld, false, U.gs}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gX, &gdx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
@@ -903,6 +935,15 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     if (!a.T) {
         st = launch_prepared(gT, a.stream);
         if (st != PF_OK) return st;
+    }
+    if (fused) {
+        st = chain_groups(a.groups, a.groups, dY.p, dY.ld, dY.gs, a.m, a.n, V.p, V.ld, V.gs, a.r, U.p, U.ld, U.gs, a.k, a.dX, a.lddx, a.sdx, Gbuf, ldW, sW,
+                          false, a.stream);
+        if (st != PF_OK) return st;
+        const PairJob jf[2] = {{x.p, x.ld, true, x.gs, Gbuf, ldW, true, sW, a.k, a.r, a.m, a.dU, a.lddu, a.sdu, a.groups},
+                               {dY.p, dY.ld, true, dY.gs, T.p, T.ld, true, T.gs, a.n, a.r, a.m, a.dV, a.lddv, a.sdv, a.groups}};
+        const GemmLaunch* const lf[2] = {&gU, &gV};
+        return launch_faster(lf, jf, 2, a.stream);
     }
     // launch A: G = dY V and dV = dY^T T (independent of each other); launch B: dU = x^T G and dX = G U^T
     const PairJob ja[2] = {{dY.p, dY.ld, false, dY.gs, V.p, V.ld, true, V.gs, a.m, a.r, a.n, Gbuf, ldW, sW, a.groups},

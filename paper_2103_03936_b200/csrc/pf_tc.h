@@ -47,9 +47,9 @@ struct ChainPlan {
     int r_pad, num_stages, stage_bytes, nsplit, tiles_per_split, row_tiles, boxes_per_stage, staging_off;
     size_t smem;
 };
-// `max_split` caps the number of column ranges the output is split into (0 = no cap).
+// `max_split` caps the number of column ranges the output is split into (0 = no cap); `groups` problems share the launch.
 bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, ChainPlan* plan, int rows_tile = 128,
-                int max_split = 0);
+                int max_split = 0, int groups = 1);
 // Blocks of output pixels of a convolution (see conv_tiling): bh full-width rows of nb images, tpi blocks per
 // image (nb > 1 only with whole images).
 struct ConvTiling {
@@ -67,6 +67,10 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
           const void* B2, int64_t ldb2, int64_t N2, void* out, int64_t ldo, void* T, int64_t ldt,
           cudaStream_t stream, const ChainConv* conv = nullptr, int max_split = 0, const void* bias = nullptr,
           int act = 0);   // bias [N2] (bf16) and act (0 identity, 1 max(0, .)) apply to `out`
+
+int chain_groups(int groups, int all, const void* A, int64_t lda, int64_t sA, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t sB1, int64_t r,
+                 const void* B2, int64_t ldb2, int64_t sB2, int64_t N2, void* out, int64_t ldo, int64_t sO, void* T, int64_t ldt, int64_t sT,
+                 bool late_wait, cudaStream_t stream);
 
 // Products on CTA pairs (pf_tc_pair.cu): C[M,N] = act(A * B + bias) for `groups` problems of one shape, matrices *_gs
 // elements apart (0 = one operand shared by all groups); sum_groups: the groups are summed into one C.

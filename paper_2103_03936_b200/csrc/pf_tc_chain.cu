@@ -29,7 +29,7 @@ ConvTiling conv_tiling(int N, int Ho, int Wo, int limit) {
 }
 
 // Shape envelope of the fused kernel and its launch geometry.
-bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, ChainPlan* plan, int rows_tile, int max_split) {
+bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, ChainPlan* plan, int rows_tile, int max_split, int groups) {
     const int64_t r_pad = (r + 63) / 64 * 64;
     if (r_pad > 384 || M > 0x7fffffff || K1 > 0x7fffffff || N2 > 0x7fffffff) return false;
     const int64_t stage = kTileBytes + r_pad * 128;
@@ -40,14 +40,14 @@ bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, Chai
     int64_t ns = budget / stage;
     if (ns > kMaxStages) ns = kMaxStages;
     if (ns < 2 || (!dedicated && ns * (r_pad / 32) < 8)) return false;
-    const int64_t row_tiles = ceil_div(M, rows_tile), nt = ceil_div(N2, 128);
+    const int64_t row_tiles = ceil_div(M, rows_tile), all_tiles = row_tiles * groups, nt = ceil_div(N2, 128);
     // Split N2 over blockIdx.y while that shortens the critical path of a CTA (each split repeats
     // phase 1, cost ~ K1; phase 2 costs ~ N2 / split) and the grid still fits one wave.
     int64_t best = 1;
     if (has_out) {
         double best_cost = 1e30;
-        for (int64_t s = 1; s <= nt && (s == 1 || row_tiles * s <= num_sms()) && (max_split <= 0 || s <= max_split); ++s) {
-            const double waves = static_cast<double>(ceil_div(row_tiles * s, num_sms()));
+        for (int64_t s = 1; s <= nt && (s == 1 || all_tiles * s <= num_sms()) && (max_split <= 0 || s <= max_split); ++s) {
+            const double waves = static_cast<double>(ceil_div(all_tiles * s, num_sms()));
             const double cost = waves * (static_cast<double>(K1) + 128.0 * ceil_div(nt, s));
             if (cost < best_cost * 0.97) { best_cost = cost; best = s; }
         }
@@ -131,6 +131,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     }
     p.bias = bias; p.act = act;
     p.status = device_status_ptr();
+    p.a_shared = 0; p.late_wait = 0;
     dim3 grid(static_cast<unsigned>(grid_x), static_cast<unsigned>(plan.nsplit), 1);
     if (out && (bias || act)) return chain_launch_act(persistent, grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
     if (persistent) {
@@ -155,6 +156,37 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
         return PF_ERR_CUDA;
     count_launch();
     return PF_OK;
+}
+
+// The chain for several groups of one shape, sA (0: one A read by all) ... sT elements apart; out or T may be null.
+// The launch shares the machine with those of the other groups of `all`; late_wait: the launch before in the stream is one of them.
+int chain_groups(int groups, int all, const void* A, int64_t lda, int64_t sA, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t sB1, int64_t r,
+                 const void* B2, int64_t ldb2, int64_t sB2, int64_t N2, void* out, int64_t ldo, int64_t sO, void* T, int64_t ldt, int64_t sT,
+                 bool late_wait, cudaStream_t stream) {
+    ChainPlan plan;
+    if (groups > 65535 || !chain_plan(M, K1, N2, r, out != nullptr, &plan, 128, 0, all)) return PF_ERR_UNSUPPORTED;
+    // (row tiles of 96 rows: see chain)
+    const int rows_tile = out && plan.nsplit == 1 && ceil_div(M, 96) * all <= num_sms() ? 96 : 128;
+    CUtensorMap ta, tb1, tb2, to, tt;
+    const bool ok = cached_map_3d(&ta, A, sA == 0 ? 1 : groups, M, K1, lda, sA, rows_tile) && cached_map_3d(&tb1, B1, groups, K1, r, ldb1, sB1, 64) &&
+                    cached_map_3d(&tb2, B2, groups, N2, r, ldb2, sB2, 128) &&
+                    (out ? cached_map_3d(&to, out, groups, M, N2, ldo, sO, 32) : cached_map_3d(&to, B2, groups, N2, r, ldb2, sB2, 32)) &&
+                    (T ? cached_map_3d(&tt, T, groups, M, r, ldt, sT, rows_tile) : cached_map_3d(&tt, B2, groups, N2, r, ldb2, sB2, 128));
+    if (!ok) return PF_ERR_CUDA;
+    ChainParams p = {};
+    p.M = static_cast<int>(M); p.K1 = static_cast<int>(K1); p.N2 = static_cast<int>(N2);
+    p.r_pad = plan.r_pad; p.num_stages = plan.num_stages; p.stage_bytes = plan.stage_bytes;
+    p.tiles_per_split = plan.tiles_per_split; p.store_T = T != nullptr;
+    p.boxes_per_stage = plan.boxes_per_stage; p.staging_off = plan.staging_off;
+    p.conv_kw = p.conv_stride = p.conv_bh = p.conv_nb = p.conv_tpi = p.conv_Ho = p.conv_N = 1;
+    p.rows_tile = rows_tile;
+    p.row_tiles = static_cast<int>(ceil_div(M, rows_tile));
+    p.acc_bufs = kAccBufs;
+    p.status = device_status_ptr();
+    p.a_shared = sA == 0;
+    p.late_wait = late_wait;
+    const dim3 grid(static_cast<unsigned>(p.row_tiles), static_cast<unsigned>(plan.nsplit), static_cast<unsigned>(groups));
+    return chain_launch_groups(grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
 }
 
 }  // namespace tc

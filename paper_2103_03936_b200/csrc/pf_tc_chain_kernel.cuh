@@ -60,6 +60,8 @@ struct ChainParams {
     const void* bias;
     int act;
     unsigned int* status;
+    int a_shared;           // grouped (kConv 3): all groups read one A
+    int late_wait;          // grouped: the kernel before is the other half of the groups, whose results nothing here reads
 };
 
 namespace {
@@ -131,7 +133,8 @@ struct RingPos {
 // the loops over tiles below fold away at compile time.
 // kEpi: the output epilogue adds a bias row and applies the activation (see ChainParams).
 // kConv: 0 = plain, 1 = convolution, 2 = convolution whose C is not a multiple of 64: tmB1 is then 3-D, [taps][C][r],
-// zero-filled past a tap's channels (the 3-D map costs 10 % of the pace, so the others stay 2-D).
+// zero-filled past a tap's channels (the 3-D map costs 10 % of the pace, so the others stay 2-D); 3 = plain products of
+// several groups, blockIdx.z = group = outermost coordinate of every map.
 template <bool kMulti, bool kEpi, int kConv>
 __global__ void __launch_bounds__(kChainThreads, 1)
 tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB1,
@@ -145,7 +148,9 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t ring = t_smem + static_cast<uint32_t>(p.r_pad) * 256u;
     volatile uint32_t* abort_flag = &ctl->abort;
 
+    constexpr bool kIm = kConv == 1 || kConv == 2, kGroups = kConv == 3;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int group = kGroups ? static_cast<int>(blockIdx.z) : 0, group_a = kGroups && !p.a_shared ? group : 0;
     const int tile0 = blockIdx.x, tile_step = gridDim.x;
     const int nt_total = (p.N2 + 127) / 128;
     const int t_beg = blockIdx.y * p.tiles_per_split;
@@ -184,15 +189,24 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     // While the previous kernel of the stream finishes, ask L2 for this block's first tiles.  A prefetch
     // only moves lines into L2, the point of coherence, so it is harmless even if that kernel is
     // still writing the tensor; the loads that consume the data are issued after the wait below.
-    if (kConv == 0) {
+    if constexpr (!kIm) {
         if (warp == 0 && elect_one()) {
-            for (int kb = 0; kb < kEarlyTiles && kb < nkb1; ++kb) tma_prefetch_l2_2d(&tmA, kb * 64, tile0 * p.rows_tile);
+            for (int kb = 0; kb < kEarlyTiles && kb < nkb1; ++kb) {
+                if constexpr (kGroups) tma_prefetch_l2_3d(&tmA, kb * 64, tile0 * p.rows_tile, group_a);
+                else tma_prefetch_l2_2d(&tmA, kb * 64, tile0 * p.rows_tile);
+            }
         } else if (warp == 10 && elect_one()) {
             for (int kb = 0; kb < 2 && kb < nkb1; ++kb)
-                for (int q = 0; q < nkb2; ++q) tma_prefetch_l2_2d(&tmB1, q * 64, kb * 64);
+                for (int q = 0; q < nkb2; ++q) {
+                    if constexpr (kGroups) tma_prefetch_l2_3d(&tmB1, q * 64, kb * 64, group);
+                    else tma_prefetch_l2_2d(&tmB1, q * 64, kb * 64);
+                }
         }
     }
-    pdl_wait();                 // everything above overlapped the previous kernel's tail
+    // (The second half of the groups runs beside the first: when it starts, everything older than that is complete, since
+    // every kernel of this library lets its successor start only after its own wait.  It waits before it ends, so that
+    // whoever waits for it has waited for both.)
+    if (!kGroups || !p.late_wait) pdl_wait();                 // everything above overlapped the previous kernel's tail
     pdl_launch_dependents();
     const uint32_t tmem = ctl->tmem_base;
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
@@ -213,9 +227,9 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int m0 = tile * p.rows_tile;
                 // convolution: (tap row, tap column, channel block) advance as counters; integer divisions
                 // in the loop over k-blocks would sit on the producer's critical path
-                const ConvOrigin cv = kConv ? conv_origin(p, tile) : ConvOrigin{0, 0};
+                const ConvOrigin cv = kIm ? conv_origin(p, tile) : ConvOrigin{0, 0};
                 const int cv_img = cv.img, cv_h0 = cv.row * p.conv_stride - p.conv_pad;
-                if constexpr (kConv != 0) {
+                if constexpr (kIm) {
                     const int cblks = p.conv_cblks, kw = p.conv_kw, x0 = -p.conv_pad, x1 = kw - p.conv_pad;
                     int cb = 0, x = x0, y = cv_h0;
                     for (int kb = 0; kb < nkb1; ++kb) {
@@ -236,7 +250,8 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         if (!ok) break;
                         const uint32_t full = full0 + 8 * rp.s;
                         mbar_expect_tx(full, txa);
-                        tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0);
+                        if constexpr (kGroups) tma_load_3d(ring + rp.off, &tmA, full, kb * 64, m0, group_a);
+                        else tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0);
                         rp.advance(NS, S);
                     }
                 }
@@ -264,7 +279,10 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             // runs.  The CTAs that share these tiles each ask for a different one.
             if (ntile > 0) {
                 const int n0 = (t_beg + static_cast<int>(blockIdx.x) % ntile) * 128;
-                for (int q = 0; q < nkb2; ++q) tma_prefetch_l2_2d(&tmB2, q * 64, n0);
+                for (int q = 0; q < nkb2; ++q) {
+                    if constexpr (kGroups) tma_prefetch_l2_3d(&tmB2, q * 64, n0, group);
+                    else tma_prefetch_l2_2d(&tmB2, q * 64, n0);
+                }
             }
             const uint32_t txb = static_cast<uint32_t>(p.r_pad) * 128u;
             int tile = tile0;
@@ -280,6 +298,8 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     if constexpr (kConv == 2) {
                         for (int q = 0; q < nkb2; ++q) tma_load_3d(dst + q * 8192, &tmB1, full, q * 64, cb * 64, tap);
                         if (++cb == cblks) { cb = 0; ++tap; }
+                    } else if constexpr (kGroups) {
+                        for (int q = 0; q < nkb2; ++q) tma_load_3d(dst + q * 8192, &tmB1, full, q * 64, kb * 64, group);
                     } else {
                         for (int q = 0; q < nkb2; ++q) tma_load_2d(dst + q * 8192, &tmB1, full, q * 64, kb * 64);
                     }
@@ -294,8 +314,10 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         const uint32_t full = full0 + 8 * rp.s;
                         mbar_arrive(full);                      // stands in for the A producer, idle in phase 2
                         mbar_expect_tx(full, kTileBytes * nb);
-                        for (int q = 0; q < nb; ++q)
-                            tma_load_2d(ring + rp.off + q * kTileBytes, &tmB2, full, (kb + q) * 64, n0);
+                        for (int q = 0; q < nb; ++q) {
+                            if constexpr (kGroups) tma_load_3d(ring + rp.off + q * kTileBytes, &tmB2, full, (kb + q) * 64, n0, group);
+                            else tma_load_2d(ring + rp.off + q * kTileBytes, &tmB2, full, (kb + q) * 64, n0);
+                        }
                         rp.advance(NS, S);
                     }
                 }
@@ -351,9 +373,10 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 if (!ok) break;
                 tc_fence_after();
                 if (p.store_T && blockIdx.y == 0) {
-                    const int crow = kConv ? conv_out_row(p, tile) : 0;
+                    const int crow = kIm ? conv_out_row(p, tile) : 0;
                     for (int q = 0; q < nkb2; ++q) {
-                        if constexpr (kConv != 0) tma_store_3d(&tmT, t_smem + q * kTileBytes, q * 64, 0, crow);
+                        if constexpr (kIm) tma_store_3d(&tmT, t_smem + q * kTileBytes, q * 64, 0, crow);
+                        else if constexpr (kGroups) tma_store_3d(&tmT, t_smem + q * kTileBytes, q * 64, tile * p.rows_tile, group);
                         else tma_store_2d(&tmT, t_smem + q * kTileBytes, q * 64, tile * p.rows_tile);
                     }
                     tma_store_commit();
@@ -433,7 +456,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (lane == 0) mbar_arrive(smem_u32(&ctl->t_ready));
 
             const int r0 = tile * p.rows_tile + q * 32;
-            const int crow = kConv ? conv_out_row(p, tile) : 0;
+            const int crow = kIm ? conv_out_row(p, tile) : 0;
             for (int j = 0; j < ntile; ++j) {
                 // kEpi: the bias of this warp's 64 columns, as 32 bf16 pairs per thread (every lane loads the
                 // same addresses: one broadcast transaction per load), fetched before the accumulator arrives
@@ -494,7 +517,8 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 if (lane == 0) {
                     const int n0 = (t_beg + j) * 128 + hcol * 64;
                     if (r0 < p.M && q * 32 < p.rows_tile && n0 < p.N2) {
-                        if constexpr (kConv != 0) tma_store_3d(&tmOut, stg, n0, q * 32, crow);
+                        if constexpr (kIm) tma_store_3d(&tmOut, stg, n0, q * 32, crow);
+                        else if constexpr (kGroups) tma_store_3d(&tmOut, stg, n0, r0, group);
                         else tma_store_2d(&tmOut, stg, n0, r0);
                         tma_store_commit();
                         stored = true;
@@ -513,6 +537,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         __syncwarp();
         tmem_dealloc(tmem, 512);
     }
+    if (kGroups && p.late_wait) pdl_wait();
 }
 
 }  // namespace
@@ -527,6 +552,10 @@ int chain_launch_pipe(dim3 grid, size_t smem, cudaStream_t stream, const CUtenso
 // Launch of the forms with a convolution as first product (pf_tc_chain_conv.cu); pipe = software-pipelined persistent.
 int chain_launch_conv(bool pipe, bool ragged, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1,
                       const CUtensorMap& tb2, const CUtensorMap& to, const CUtensorMap& tt, const ChainParams& p);
+
+// Launch of the grouped form (pf_tc_chain_group.cu).
+int chain_launch_groups(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1, const CUtensorMap& tb2,
+                        const CUtensorMap& to, const CUtensorMap& tt, const ChainParams& p);
 
 }  // namespace tc
 }  // namespace pf

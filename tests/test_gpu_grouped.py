@@ -158,3 +158,13 @@ def test_invalid_arguments_are_refused_on_the_host():
                                          None, 0, 0, 5, 8, 6, 4, pf.PF_BF16, ws.data_ptr(), ws.numel(), None)
     assert st == 1
     assert pf.pf_launch_count() == before
+
+
+@pytest.mark.parametrize("G,m,k,n,r,shared_x", [(2, 1, 64, 64, 8, True), (3, 97, 1024, 72, 192, False), (3, 97, 1032, 72, 192, True), (5, 300, 72, 520, 64, True),
+                                                (9, 2049, 64, 72, 16, False), (3, 2100, 520, 200, 160, False), (2, 2100, 200, 1032, 40, False)])
+def test_fused_kernel_over_groups(G, m, k, n, r, shared_x):
+    """Either side of the sizes from which groups run on the fused kernel, odd group counts (the halves differ), with and
+    without the stash; guard bands and every group by itself."""
+    lf, lb = run_grouped(G, m, k, n, r, wl.BF16, 250, shared_x, blocks=True)
+    assert (lf, lb) == (2, 2)
+    run_grouped(G, m, k, n, r, wl.BF16, 251, shared_x, stash=False, blocks=True)
