@@ -67,11 +67,21 @@ unsigned run_blocks(int64_t tiles, int64_t kblocks_per_tile, int stride) {
     return static_cast<unsigned>(blocks);
 }
 
+bool vector_rows(const void* C, int64_t ldc, int64_t gs) { return ldc % 8 == 0 && gs % 8 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0; }
+// A product that needs the kernels compiled for any form (see gemm_tile).
+bool any_form(const GemmParams& p) { return p.bias || p.act || p.C2 || (p.partial && p.splits <= 1) || !vector_rows(p.C, p.ldc, p.c_gstride); }
+
 template <int BN>
 cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p, dim3 grid,
                         cudaStream_t stream) {
-    cudaError_t e = allow_smem(tc_gemm_kernel<BN, false>, std::min(gemm_smem(BN, kMaxStages), static_cast<size_t>(227 * 1024)));
-    if (e == cudaSuccess) e = launch_overlapped(tc_gemm_kernel<BN, false>, grid, dim3(kGemmThreads), gemm_smem(BN, p.num_stages), stream, ta, tb, p);
+    cudaError_t e = cudaSuccess;
+    if (any_form(p)) {
+        e = launch_gemm_any(BN, grid, gemm_smem(BN, p.num_stages), stream, ta, tb, p);
+    } else {
+        e = allow_smem(tc_gemm_kernel<BN, false, false>, gemm_smem(BN, kMaxStages));
+        if (e == cudaSuccess)
+            e = launch_overlapped(tc_gemm_kernel<BN, false, false>, grid, dim3(kGemmThreads), gemm_smem(BN, p.num_stages), stream, ta, tb, p);
+    }
     if (e == cudaSuccess) count_launch();
     return e;
 }
@@ -87,9 +97,11 @@ size_t partial_bytes(int64_t M, int64_t N, int splits) { return splits <= 1 ? 0 
 // end: 0.16 us per k-block on warm caches, 0.3 on cold ones, and for the sum of the slices 5 us at two slices, 4.2 at
 // four, 3.8 at eight (the fewer slices, the larger the share that a block sums).  So short contractions stay whole:
 // 1024 x 256 over 512: 9.3 us in two slices, 4.8 whole; over 1024: 8.4 in four, 6.0 whole; over 2048: 8.4 in eight, 8.4
-// whole; over 4096: 9.3 in eight, 13.0 whole.
+// whole; over 4096: 9.3 in eight, 13.0 whole.  (dU of 26 x 7 x 7, 160 -> 40 -> 160 over 26 blocks of 49 pixels: backward 13.8 us
+// split, 16.0 whole; of 16 x 14 x 14, stride 2, over 16: 12.8 and 9.8.)
+constexpr double kBlockUs = 0.23;
 double slice_us(int64_t nkb, int64_t s) {
-    return 0.2 * static_cast<double>(ceil_div(nkb, s)) + (s > 1 ? 3.4 + 3.4 / static_cast<double>(s) : 0.0);
+    return kBlockUs * static_cast<double>(ceil_div(nkb, s)) + (s > 1 ? 3.4 + 3.4 / static_cast<double>(s) : 0.0);
 }
 // Slices of a contraction that is alone in its launch.
 int slices_of(int64_t tiles, int64_t nkb) {
@@ -333,21 +345,24 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
         if (i < count) smem = std::max(smem, gemm_smem(src->bn, stages, dx));
     }
     Gemm3Args k;
-    bool conv = false;
+    bool conv = false, any = false;
     for (int i = 0; i < 3; ++i) {
         const GemmLaunch* src = g[i < count ? i : 0];
+        any = any || any_form(src->p);
         k.ta[i] = src->ta; k.tb[i] = src->tb; k.p[i] = prm[i];
         k.tiles[i] = make_int2(src->grid.x, src->grid.y);
         conv = conv || src->p.conv_mode != 0;
     }
     k.end0 = ctas[0]; k.end1 = ctas[0] + ctas[1];
     cudaError_t e;
-    if (conv) {
+    if (any) {
+        e = launch_gemm3_any(conv, total, smem, stream, k);
+    } else if (conv) {
         e = launch_gemm3_conv(total, smem, stream, k);
     } else {
-        e = allow_smem(tc_gemm3_kernel<false>, gemm_smem(128, kMaxStages));
+        e = allow_smem(tc_gemm3_kernel<false, false>, gemm_smem(128, kMaxStages));
         if (e == cudaSuccess)
-            e = launch_overlapped(tc_gemm3_kernel<false>, dim3(static_cast<unsigned>(total)), dim3(kGemmThreads), smem, stream, k.ta[0], k.tb[0],
+            e = launch_overlapped(tc_gemm3_kernel<false, false>, dim3(static_cast<unsigned>(total)), dim3(kGemmThreads), smem, stream, k.ta[0], k.tb[0],
                                   k.ta[1], k.tb[1], k.ta[2], k.tb[2], k.p[0], k.p[1], k.p[2], k.end0, k.end1, k.tiles[0], k.tiles[1], k.tiles[2]);
     }
     if (e != cudaSuccess) return PF_ERR_CUDA;
@@ -361,13 +376,12 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
 // 0.42 us per k-block beside another (its SM's load path is what it waits for).  A pair's 256 x 256 tile: 0.28 us per
 // k-block (the tensor cores), and 2 us of every tile but the first do not hide (the results' way to memory).  Output rows
 // that take no 16-byte stores: 1.2 us more per single tile, 2.1 per tile of a pair.
-bool vector_rows(const void* C, int64_t ldc, int64_t gs) { return ldc % 8 == 0 && gs % 8 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0; }
 double single_us(const GemmLaunch* const* g, int count) {
     double ctas = 0, load = 0, alone = 0, beside = 0, shortest = 1e30;
     for (int i = 0; i < count; ++i) shortest = std::min<double>(shortest, g[i]->p.kb_per_split);
     for (int i = 0; i < count; ++i) {
         const double n = static_cast<double>(g[i]->grid.x) * g[i]->grid.y * g[i]->grid.z, kb = g[i]->p.kb_per_split;
-        const double sum = slice_us(g[i]->p.nkb_total, g[i]->p.splits) - 0.2 * kb + (g[i]->p.splits > 1 || vector_rows(g[i]->p.C, g[i]->p.ldc, g[i]->p.c_gstride) ? 0.0 : 1.2);
+        const double sum = slice_us(g[i]->p.nkb_total, g[i]->p.splits) - kBlockUs * kb + (g[i]->p.splits > 1 || vector_rows(g[i]->p.C, g[i]->p.ldc, g[i]->p.c_gstride) ? 0.0 : 1.2);
         ctas += n;
         load += n * (0.42 * kb + 4.1 + sum);
         alone = std::max(alone, 0.2 * kb + sum);

@@ -72,6 +72,9 @@ struct Gemm3Args {
     int2 tiles[3];
 };
 cudaError_t launch_gemm3_conv(int blocks, size_t smem, cudaStream_t stream, const Gemm3Args& a);
+// ... with products of any form (pf_tc_any.cu; see gemm_tile).
+cudaError_t launch_gemm_any(int bn, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p);
+cudaError_t launch_gemm3_any(bool conv, int blocks, size_t smem, cudaStream_t stream, const Gemm3Args& a);
 
 namespace {
 
@@ -167,7 +170,11 @@ __device__ __forceinline__ void store_columns(__nv_bfloat16* dst, uint32_t lo, u
 // order, its share over all slices and writes bf16 (bit-reproducible, no second launch).
 // kMode: 0 = plain (or grouped) product, 2 = dU of a convolution (dX: run_tiles), compiled apart so that the plain
 // kernels carry none of its code (with all of them in one kernel the FFN backward ran 12 % slower).
-template <int BN, int kMode>
+// kAny: any output rows, second copies, bias and activation, one fp32 slice instead of C.  Without it: rows of whole 16-byte
+// pieces and none of that; the code behind the main loop runs once, from a cold instruction cache, so what a product does
+// not need is not compiled into its kernel (all of it in one kernel: backward of 8192 x 2048 -> 128 -> 512 30.0 us, apart 28.5; 64 x 512 ->
+// 128 -> 512: 8.6 and 8.0).
+template <int BN, int kMode, bool kAny>
 __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p,
                                           const int bx, const int by, const int bz, const int bg) {
     constexpr uint32_t kABytes = kBM * kBK * 2;          // 16 KB
@@ -371,7 +378,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
         tc_fence_after();
         if (ok) {
             const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-            if (p.partial) {
+            if (kAny ? p.partial != nullptr : p.splits > 1) {
                 // fp32 slice: straight from registers, [quadrant][4-column group][row][4], so that every store
                 // instruction of a warp is one run of 512 bytes; then the warp reports
                 float* dst = p.partial + (static_cast<size_t>(tile) * p.splits + bz) * (kBM * BN) +
@@ -388,12 +395,12 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                             make_uint4(v[g >> 3][4 * (g & 7)], v[g >> 3][4 * (g & 7) + 1], v[g >> 3][4 * (g & 7) + 2], v[g >> 3][4 * (g & 7) + 3]);
                 }
                 __syncwarp();
-                if (lane == 0 && p.splits > 1) red_release_gpu(p.counters + 2 * tile, 1u);
+                if (lane == 0 && (!kAny || p.splits > 1)) red_release_gpu(p.counters + 2 * tile, 1u);
             } else {
                 // every MMA has completed, so the pipeline stages are free: 16 KB of vector panels, then word panels
                 uint32_t* stg = reinterpret_cast<uint32_t*>(tiles + 16384) + (warp - 2) * (32 * kRaggedWords);
                 __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
-                const bool vec_ok = (p.ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0;
+                const bool vec_ok = !kAny || ((p.ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(Cb) & 15) == 0);
                 if (vec_ok) {
                     // 16-byte aligned rows: stage 32 rows x 64 columns (128 bytes per row, 16-byte pieces
                     // XOR-swizzled by the row so that both passes are free of bank conflicts), then
@@ -410,7 +417,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                         tmem_ld32(lane_base + c * 64, v0);
                         tmem_ld32(lane_base + c * 64 + 32, v1);
                         tmem_ld_wait();
-                        if (kMode == 0 && (p.bias || p.act)) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
+                        if (kAny && kMode == 0 && (p.bias || p.act)) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
 #pragma unroll
                         for (int t = 0; t < 4; ++t) {
                             uint4 o;
@@ -445,7 +452,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                                 }
                             }
                         }
-                        if (p.C2) {          // the second copy, at a pitch that the first cannot have
+                        if (kAny && p.C2) {          // the second copy, at a pitch that the first cannot have
                             stage_ragged(stg, v0, v1, lane);
                             __syncwarp();
                             store_ragged(stg, reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride, p.ldc2, n0 + c * 64,
@@ -453,18 +460,19 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                         }
                         __syncwarp();
                     }
-                } else
+                } else if constexpr (kAny) {
 #pragma unroll 1
-                for (int c = 0; c < BN / 64; ++c) {
-                    uint32_t v0[32], v1[32];
-                    tmem_ld32(lane_base + c * 64, v0);
-                    tmem_ld32(lane_base + c * 64 + 32, v1);
-                    tmem_ld_wait();
-                    if (kMode == 0 && (p.bias || p.act)) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
-                    stage_ragged(stg, v0, v1, lane);
-                    __syncwarp();
-                    store_ragged(stg, Cb, p.ldc, n0 + c * 64, p.N, lane, [&](int r) { return output_row<kMode>(p, org, bx, q * 32 + r); });
-                    __syncwarp();
+                    for (int c = 0; c < BN / 64; ++c) {
+                        uint32_t v0[32], v1[32];
+                        tmem_ld32(lane_base + c * 64, v0);
+                        tmem_ld32(lane_base + c * 64 + 32, v1);
+                        tmem_ld_wait();
+                        if (kAny && kMode == 0 && (p.bias || p.act)) bias_act64(v0, v1, p.bias, p.act, n0 + c * 64, p.N, lane);
+                        stage_ragged(stg, v0, v1, lane);
+                        __syncwarp();
+                        store_ragged(stg, Cb, p.ldc, n0 + c * 64, p.N, lane, [&](int r) { return output_row<kMode>(p, org, bx, q * 32 + r); });
+                        __syncwarp();
+                    }
                 }
             }
         }
@@ -500,7 +508,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     __syncthreads();
     if (ctl->fix_ok) {
         __nv_bfloat16* Cb = reinterpret_cast<__nv_bfloat16*>(p.C) + static_cast<long long>(bg) * p.c_gstride;
-        __nv_bfloat16* C2b = p.C2 ? reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride : nullptr;
+        __nv_bfloat16* C2b = kAny && p.C2 ? reinterpret_cast<__nv_bfloat16*>(p.C2) + static_cast<long long>(bg) * p.c2_gstride : nullptr;
         // units of 8 rows x 32 columns: a lane holds two 4-column groups of a row, 16 columns apart
         constexpr int kUnits = kBM / 8 * (BN / 32);
         constexpr size_t kSlice = static_cast<size_t>(kBM) * BN / 4;       // float4s
@@ -535,9 +543,10 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                 const int col = n0 + pc * 4 + j * 16;
                 __nv_bfloat16* dst = Cb + static_cast<size_t>(row) * p.ldc + col;
                 const uint32_t lo = pack_bf16x2(acc[j].x, acc[j].y), hi = pack_bf16x2(acc[j].z, acc[j].w);
-                store_columns(dst, lo, hi, p.N - col);
+                if (!kAny && col + 3 < p.N) *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
+                else store_columns(dst, lo, hi, p.N - col);
                 // the same sums once more, for a destination whose pitch the first cannot have
-                if (C2b) store_columns(C2b + static_cast<size_t>(row) * p.ldc2 + col, lo, hi, p.N - col);
+                if (kAny && C2b) store_columns(C2b + static_cast<size_t>(row) * p.ldc2 + col, lo, hi, p.N - col);
             }
         }
     }
@@ -752,7 +761,7 @@ __device__ __forceinline__ void run_tiles(const CUtensorMap& tmA, const CUtensor
     if (warp == 1) tmem_dealloc(tmem_base, 2 * BN);
 }
 
-template <int BN, bool kRuns>
+template <int BN, bool kRuns, bool kAny>
 __global__ void __launch_bounds__(kGemmThreads, BN <= 128 ? 2 : 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const GemmParams p) {
@@ -760,7 +769,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         run_tiles<BN, 0>(tmA, tmB, p, blockIdx.x, gridDim.x);
     } else {
         const int sl = p.splits < 1 ? 1 : p.splits;
-        gemm_tile<BN, 0>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
+        gemm_tile<BN, 0, kAny>(tmA, tmB, p, blockIdx.x, blockIdx.y, static_cast<int>(blockIdx.z) % sl, static_cast<int>(blockIdx.z) / sl);
     }
 }
 
@@ -769,8 +778,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // product 2; each decodes (row tile, column tile, slice) from its linear index.  One launch pays the
 // start-up latency once and packs the short CTAs of one product beside the long ones of another.
 // Tiles may be 64 or 128 columns wide per product.
-template <bool kConv>
-__device__ __forceinline__ void gemm_any(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, int idx,
+template <bool kConv, bool kAny>
+__device__ __forceinline__ void gemm_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, int idx,
                                          const int2 t) {
     if constexpr (kConv) {
         if (p.conv_mode == 1) {             // t.x = the blocks that share the tiles
@@ -783,15 +792,15 @@ __device__ __forceinline__ void gemm_any(const CUtensorMap& tmA, const CUtensorM
     const int bx = idx % t.x, by = (idx / t.x) % t.y, zz = idx / (t.x * t.y);
     if constexpr (kConv) {
         if (p.conv_mode == 2) {
-            if (p.bn == 64) gemm_tile<64, 2>(tmA, tmB, p, bx, by, zz, 0);
-            else gemm_tile<128, 2>(tmA, tmB, p, bx, by, zz, 0);
+            if (p.bn == 64) gemm_tile<64, 2, kAny>(tmA, tmB, p, bx, by, zz, 0);
+            else gemm_tile<128, 2, kAny>(tmA, tmB, p, bx, by, zz, 0);
             return;
         }
     }
-    if (p.bn == 64) gemm_tile<64, 0>(tmA, tmB, p, bx, by, zz % sl, zz / sl);
-    else gemm_tile<128, 0>(tmA, tmB, p, bx, by, zz % sl, zz / sl);
+    if (p.bn == 64) gemm_tile<64, 0, kAny>(tmA, tmB, p, bx, by, zz % sl, zz / sl);
+    else gemm_tile<128, 0, kAny>(tmA, tmB, p, bx, by, zz % sl, zz / sl);
 }
-template <bool kConv>
+template <bool kConv, bool kAny>
 __global__ void __launch_bounds__(kGemmThreads, 2)
 tc_gemm3_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                 const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
@@ -799,9 +808,9 @@ tc_gemm3_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant_
                 const GemmParams p0, const GemmParams p1, const GemmParams p2, const int end0, const int end1,
                 const int2 tiles0, const int2 tiles1, const int2 tiles2) {
     const int idx = blockIdx.x;
-    if (idx < end0) gemm_any<kConv>(tmA0, tmB0, p0, idx, tiles0);
-    else if (idx < end1) gemm_any<kConv>(tmA1, tmB1, p1, idx - end0, tiles1);
-    else gemm_any<kConv>(tmA2, tmB2, p2, idx - end1, tiles2);
+    if (idx < end0) gemm_one<kConv, kAny>(tmA0, tmB0, p0, idx, tiles0);
+    else if (idx < end1) gemm_one<kConv, kAny>(tmA1, tmB1, p1, idx - end0, tiles1);
+    else gemm_one<kConv, kAny>(tmA2, tmB2, p2, idx - end1, tiles2);
 }
 
 }  // namespace

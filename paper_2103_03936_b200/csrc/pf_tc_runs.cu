@@ -11,8 +11,8 @@ namespace tc {
 namespace {
 template <int BN>
 cudaError_t launch_one(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p) {
-    const cudaError_t e = allow_smem(tc_gemm_kernel<BN, true>, 227 * 1024);
-    return e != cudaSuccess ? e : launch_overlapped(tc_gemm_kernel<BN, true>, grid, dim3(kGemmThreads), smem, stream, ta, tb, p);
+    const cudaError_t e = allow_smem(tc_gemm_kernel<BN, true, false>, 227 * 1024);
+    return e != cudaSuccess ? e : launch_overlapped(tc_gemm_kernel<BN, true, false>, grid, dim3(kGemmThreads), smem, stream, ta, tb, p);
 }
 }  // namespace
 
