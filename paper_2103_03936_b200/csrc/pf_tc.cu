@@ -520,10 +520,16 @@ bool use_chain(int64_t m, int64_t r) { return m >= 2048 && r <= 192; }
 // 300 x 512 -> 128 -> 2048: 6.4 against 8.7 us; 1000 x 1536 -> 128 -> 1536: 10.5 / 11.7; 500 x 2048 -> 128 -> 2048: 11.7 / 11.7;
 // 1024 x 4096 -> 128 -> 1024: 18.6 / 12.1; r 256, 1024 x 1024 -> 1024: 11.8 / 10.3.  Up to 32 rows against the kernels of
 // pf_small.cu: 20 x 512 -> 128 -> 2048: 5.9 / 6.8; 8 x 1024 -> 64 -> 1024: 6.5 / 5.4.  A stash that TMA cannot write would take
-// a launch of its own again.
+// a launch of its own again.  Rows that do not start on 128-byte lines cost two lines per row of a box: 500 x 1480 -> 120 ->
+// 1480: 14.5 / 12.4; 400 x 1096 -> 136 -> 4384: 16.9 / 14.5; 1000 x 1336 -> 80 -> 344: 11.4 / 14.1.
+bool short_first_product(int64_t k, int64_t r, int64_t ldx, int64_t ldu, int64_t most) {
+    const int64_t lines = 128 * (ldx % 64 ? 2 : 1) + ceil_div(r, 64) * 64 * (ldu % 64 ? 2 : 1);      // of a k-block
+    return k <= most && ceil_div(k, kBK) * lines <= 11000;
+}
 bool use_chain_fwd(const LinearArgs& a) {
     if (a.r > 192 || !tma_ok(a.y, a.ldy)) return false;
-    return a.m >= 2048 || (a.k <= 1536 && (!a.T || tma_ok(a.T, a.ldt)));
+    // (operands that are copied first arrive on whole lines)
+    return a.m >= 2048 || (short_first_product(a.k, a.r, tma_ok(a.x, a.ldx) ? a.ldx : 0, tma_ok(a.U, a.ldu) ? a.ldu : 0, 1536) && (!a.T || tma_ok(a.T, a.ldt)));
 }
 
 size_t repack_room(int64_t rows, int64_t cols) {
@@ -864,7 +870,7 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     // other: 4 x (1024 x 512 -> 128 -> 512): 13.0 -> 8.3 us, 4 x (8192 x 512 -> 128 -> 512): 26.7 -> 19.3, 2 x (7666 x 1976 ->
     // 120 -> 1976): 51 -> 42; 4 x (185 x 1536 -> 192 -> 1536): 12.1 -> 12.8; 8 x (4789 x 72 -> 8 -> 72): 18.3 -> 18.8.
     ChainPlan plan;
-    if (a.r <= 192 && (a.m >= 2048 || a.k <= 1024) && (a.k + a.n >= 512 || ceil_div(a.m, kBM) * a.groups <= 2 * num_sms()) && grouped_ok(a.y, a.ldy, a.sy) && (!a.T || stash_direct) &&
+    if (a.r <= 192 && (a.m >= 2048 || short_first_product(a.k, a.r, x.ld, U.ld, 1024)) && (a.k + a.n >= 512 || ceil_div(a.m, kBM) * a.groups <= 2 * num_sms()) && grouped_ok(a.y, a.ldy, a.sy) && (!a.T || stash_direct) &&
         chain_plan(a.m, a.k, a.n, a.r, true, &plan, 128, 0, a.groups)) {
         *handled = 1;
         int st = repacks.flush(a.stream);
