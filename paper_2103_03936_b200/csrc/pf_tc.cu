@@ -286,6 +286,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.counters = nullptr;
     p.partial = p.splits > 1 ? partial : nullptr;
     p.independent = 0;
+    p.keep_a = 0.f;
     if (p.splits > 1) {
         // the CTAs of a tile wait for one another, so all of them must be resident at once
         if (static_cast<int64_t>(grid.x) * grid.y * out_groups > kFixTiles || static_cast<int64_t>(grid.x) * grid.y * grid.z > num_sms() ||
@@ -526,6 +527,9 @@ bool short_first_product(int64_t k, int64_t r, int64_t ldx, int64_t ldu, int64_t
     const int64_t lines = 128 * (ldx % 64 ? 2 : 1) + ceil_div(r, 64) * 64 * (ldu % 64 ? 2 : 1);      // of a k-block
     return k <= most && ceil_div(k, kBK) * lines <= 11000;
 }
+// Whether a fused launch streams more than L2 holds: its output is then the first to leave L2, and so is an operand's row once
+// read.  (An output that fits stays, for whoever reads it next.)
+bool beyond_l2(int64_t m, int64_t k, int64_t n) { return static_cast<double>(m) * static_cast<double>(k + n) * 2.0 > kL2Bytes; }
 bool use_chain_fwd(const LinearArgs& a) {
     if (a.r > 192 || !tma_ok(a.y, a.ldy)) return false;
     // (operands that are copied first arrive on whole lines)
@@ -655,7 +659,7 @@ int linear_fwd(const LinearArgs& a, int* handled) {
     if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan)) {
         // one fused kernel; the intermediate leaves the chip only if a stash was asked for
         st = chain(x.p, x.ld, a.m, a.k, U.p, U.ld, a.r, V.p, V.ld, a.n, a.y, a.ldy, a.T ? T : nullptr, ldT,
-                   a.stream, nullptr, 0, a.bias, a.act);
+                   a.stream, nullptr, 0, a.bias, a.act, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f);
     } else {
         float* p1 = reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * row_pitch(a.r) * 2, 256));
         st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, T, ldT,
@@ -726,8 +730,9 @@ int linear_bwd(const LinearArgs& a, int* handled) {
         if (st != PF_OK) return st;
     }
     if (fused_dx) {
+        const bool big = beyond_l2(a.m, a.k, a.n);
         st = chain(dY.p, dY.ld, a.m, a.n, V.p, V.ld, a.r, U.p, U.ld, a.k, a.dX, a.lddx, G, ldG, a.stream, nullptr,
-                   dv_beside ? 1 : 0);
+                   dv_beside ? 1 : 0, nullptr, 0, big ? 0.2f : 0.f, big ? kL2Stream : 0.f);
         if (st != PF_OK) return st;
     } else {
         // Two launches: G = dY V with dV = dY^T T, which needs nothing of it, then dU = x^T G with dX = G U^T.  Where the
@@ -772,6 +777,11 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     if (st != PF_OK) return st;
     keep_slices(a.du_slices, &gu, pu_bytes ? pu : nullptr);
     keep_slices(a.dv_slices, &gv, pv_bytes ? pv : nullptr);
+    // dY and x are read for the last time: they make room.  In a step that streams more than L2 holds a fifth of dY is kept for
+    // this launch, and everything else passes through: 16384 x 4096 -> 64 -> 4096: 161 -> 149 us, 8192 x 4096 -> 64 -> 4096: 101 -> 88,
+    // 16384 x 2048 -> 64 -> 2048: 91 -> 81.  The last reads alone: 8192 x 512 -> 128 -> 2048: 42.3 -> 40.7, 12000 x 2048 -> 96 -> 2048:
+    // 84.5 -> 80.0.
+    gu.p.keep_a = gv.p.keep_a = kL2Stream;
     const GemmLaunch* list[2] = {&gu, &gv};
     if (gu.p.splits <= 1 && gv.p.splits > 1) std::swap(list[0], list[1]);       // a split product has to come before the plain ones
     if (dv_beside) {

@@ -66,7 +66,8 @@ struct ChainConv {
 int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t r,
           const void* B2, int64_t ldb2, int64_t N2, void* out, int64_t ldo, void* T, int64_t ldt,
           cudaStream_t stream, const ChainConv* conv = nullptr, int max_split = 0, const void* bias = nullptr,
-          int act = 0);   // bias [N2] (bf16) and act (0 identity, 1 max(0, .)) apply to `out`
+          int act = 0,    // bias [N2] (bf16) and act (0 identity, 1 max(0, .)) apply to `out`
+          float keep_a = 0.f, float keep_out = 0.f);      // how L2 treats A and `out` (l2_policy in pf_tc_prims.cuh)
 
 int chain_groups(int groups, int all, const void* A, int64_t lda, int64_t sA, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t sB1, int64_t r,
                  const void* B2, int64_t ldb2, int64_t sB2, int64_t N2, void* out, int64_t ldo, int64_t sO, void* T, int64_t ldt, int64_t sT,

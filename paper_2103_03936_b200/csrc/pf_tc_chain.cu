@@ -68,7 +68,7 @@ bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, Chai
 // out may be null (phase 1 only: T is written and nothing else).  All pointers must satisfy tma_ok.
 int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t r,
           const void* B2, int64_t ldb2, int64_t N2, void* out, int64_t ldo, void* T, int64_t ldt,
-          cudaStream_t stream, const ChainConv* conv, int max_split, const void* bias, int act) {
+          cudaStream_t stream, const ChainConv* conv, int max_split, const void* bias, int act, float keep_a, float keep_out) {
     ChainPlan plan;
     const int cs = conv ? conv->stride : 1;
     const int Ho = conv ? (conv->H + 2 * conv->pad - conv->kh) / cs + 1 : 1;
@@ -132,6 +132,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     p.bias = bias; p.act = act;
     p.status = device_status_ptr();
     p.a_shared = 0; p.late_wait = 0;
+    p.keep_a = keep_a; p.keep_out = keep_out;
     dim3 grid(static_cast<unsigned>(grid_x), static_cast<unsigned>(plan.nsplit), 1);
     if (out && (bias || act)) return chain_launch_act(persistent, grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
     if (persistent) {

@@ -60,6 +60,7 @@ struct ChainParams {
     const void* bias;
     int act;
     unsigned int* status;
+    float keep_a, keep_out; // plain products: how L2 treats A and the output (see l2_policy)
     int a_shared;           // grouped (kConv 3): all groups read one A
     int late_wait;          // grouped: the kernel before is the other half of the groups, whose results nothing here reads
 };
@@ -219,6 +220,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (elect_one()) {
             // -------------------------------------------------------------- TMA producer of A (phase 1)
             RingPos rp;
+            const uint64_t a_policy = kConv == 0 ? l2_policy(p.keep_a) : 0;
             const uint32_t txa = static_cast<uint32_t>(p.rows_tile) * 128u;
             const int skip = ntile * ((nkb2 + bps - 1) / bps);      // stages of a tile's phase 2 (B2 only)
             bool ok = true;
@@ -251,7 +253,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         const uint32_t full = full0 + 8 * rp.s;
                         mbar_expect_tx(full, txa);
                         if constexpr (kGroups) tma_load_3d(ring + rp.off, &tmA, full, kb * 64, m0, group_a);
-                        else tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0);
+                        else tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0, a_policy);
                         rp.advance(NS, S);
                     }
                 }
@@ -433,6 +435,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             stg = ring + (ew / per_stage) * S + kTileBytes + (ew % per_stage) * 4096;
         }
         const uint32_t prow = stg + lane * 128;
+        const uint64_t out_policy = kConv == 0 ? l2_policy(p.keep_out) : 0;
         bool stored = false, ok = true;
         AccPos ap;
         uint32_t it = 0;
@@ -519,7 +522,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     if (r0 < p.M && q * 32 < p.rows_tile && n0 < p.N2) {
                         if constexpr (kIm) tma_store_3d(&tmOut, stg, n0, q * 32, crow);
                         else if constexpr (kGroups) tma_store_3d(&tmOut, stg, n0, r0, group);
-                        else tma_store_2d(&tmOut, stg, n0, r0);
+                        else tma_store_2d(&tmOut, stg, n0, r0, out_policy);
                         tma_store_commit();
                         stored = true;
                     }

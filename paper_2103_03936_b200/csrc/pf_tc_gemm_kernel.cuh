@@ -52,6 +52,7 @@ struct GemmParams {
     int kpix;                // conv_mode 2: pixels per k-block (<= 64), else 64
     int ksteps;              // 16-element steps of a k-block that can be non-zero (1..4)
     int nkb_total;           // k-blocks of the whole contraction
+    float keep_a;            // plain products: how L2 treats A (see l2_policy)
     int independent;         // 1: reads nothing the preceding kernel of the stream writes (see gemm_tile)
     // Grouped products (several problems of one shape in a launch): tmA / tmB are 3-D maps whose outermost
     // coordinate is the group (a shared operand has one group only), outputs of group g start g * c_gstride
@@ -321,9 +322,10 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
                     });
                 }
             } else if (do_a && p.a_mn) {
+                const uint64_t policy = l2_policy(p.keep_a);
                 produce([&](uint32_t dst, uint32_t full) {
-                    tma_load_2d(dst, &tmA, full, m0, k0);
-                    tma_load_2d(dst + 8192, &tmA, full, m0 + 64, k0);
+                    tma_load_2d(dst, &tmA, full, m0, k0, policy);
+                    tma_load_2d(dst + 8192, &tmA, full, m0 + 64, k0, policy);
                     k0 += kBK;
                 });
             } else if (do_a) {
