@@ -85,6 +85,10 @@ void du_blocks(F32Work* w) {
         w->ct.blocks = static_cast<int64_t>(c.N) * c.Ho;
     }
 }
+void f32_tiles(F32Work* w, int bn) {
+    w->bn = bn;
+    w->tiles_y = ceil_div(w->N, bn);
+}
 F32Work f32_work(int64_t M, int64_t N, int64_t K, const F32Conv* cv = nullptr) {
     F32Work w;
     w.M = M; w.N = N; w.K = K;
@@ -108,15 +112,14 @@ F32Work f32_work(int64_t M, int64_t N, int64_t K, const F32Conv* cv = nullptr) {
             w.nkb = static_cast<int64_t>(taps) * ceil_div(cv->C, 32);
         }
     }
-    // narrow tiles where 128-column ones would leave half of the machine idle
-    w.bn = (N <= 64 || w.tiles_x * ceil_div(N, 128) * 2 <= num_sms()) ? 64 : 128;
-    w.tiles_y = ceil_div(N, w.bn);
+    // narrow tiles where 128-column ones would leave half of the machine idle (f32_split looks at both)
+    f32_tiles(&w, (N <= 64 || w.tiles_x * ceil_div(N, 128) * 2 <= num_sms()) ? 64 : 128);
     return w;
 }
 // Slice counts of the products of one launch (`can` = which may be split): every block should carry about the same
 // number of k-blocks and all of them fit the machine at once.  A slice sum costs about as much as 12 k-blocks
 // (5 us of L2 round trips), so contractions shorter than that stay whole.
-void f32_split(F32Work* const* w, const bool* can, int count) {
+void f32_slices(F32Work* const* w, const bool* can, int count) {
     int64_t work = 0, longest = 0;
     for (int i = 0; i < count; ++i) {
         work += w[i]->tiles() * w[i]->nkb;
@@ -135,6 +138,41 @@ void f32_split(F32Work* const* w, const bool* can, int count) {
         if (split_blocks <= num_sms()) return;
     }
     for (int i = 0; i < count; ++i) w[i]->splits = 1;
+}
+
+// Expected microseconds of the launch: 5 of start and end, a k-block of a 128-column tile 0.95 and of a 64-column one 0.67,
+// 5 for a sum of slices; one block per SM at a time.
+double f32_us(F32Work* const* w, int count) {
+    double blocks = 0, load = 0, longest = 0;
+    for (int i = 0; i < count; ++i) {
+        const double n = static_cast<double>(w[i]->tiles() * w[i]->splits);
+        const double us = 5.0 + (w[i]->bn == 64 ? 0.67 : 0.95) * static_cast<double>(ceil_div(w[i]->nkb, w[i]->splits)) + (w[i]->splits > 1 ? 5.0 : 0.0);
+        blocks += n;
+        load += n * us;
+        longest = std::max(longest, us);
+    }
+    return blocks <= num_sms() ? longest : count == 1 ? longest * static_cast<double>(ceil_div(static_cast<int64_t>(blocks), num_sms()))
+                                                      : std::max(longest, 1.1 * load / num_sms());
+}
+// Slices, and the widths of the tiles: 128 columns do in one k-block of 0.95 us what two 64-column tiles do in 1.34, so long
+// contractions are better cut into more slices of wide tiles: backward of 2048 x 512 -> 128 -> 2048: 45.7 -> 37.3 us, of 1000 x 1024 ->
+// 256 -> 1024: 43.1 -> 31.9; forward of 2048 x 2048 -> 128 -> 512: 26.1 -> 23.3.
+void f32_split(F32Work* const* w, const bool* can, int count) {
+    f32_slices(w, can, count);
+    F32Work wide[2];
+    F32Work* pw[2] = {&wide[0], &wide[1]};
+    bool other = false;
+    for (int i = 0; i < count; ++i) {
+        wide[i] = *w[i];
+        if (w[i]->bn == 64 && w[i]->N > 64) {
+            f32_tiles(&wide[i], 128);
+            other = true;
+        }
+    }
+    if (!other) return;
+    f32_slices(pw, can, count);
+    if (f32_us(pw, count) < f32_us(w, count))
+        for (int i = 0; i < count; ++i) *w[i] = wide[i];
 }
 
 size_t f32_smem(int bn, int stages) { return 2048 + 3 * static_cast<size_t>(bn) * 128 + static_cast<size_t>(stages) * (16384 + static_cast<size_t>(bn) * 128); }

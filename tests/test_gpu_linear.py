@@ -377,3 +377,10 @@ def test_forward_beyond_the_fused_sizes(m, k, n, r):
     before = pf.pf_launch_count()
     pf.pf_lowrank_linear_fwd(*(dev(d[k_], wl.BF16) for k_ in ("x", "U", "V")))
     assert pf.pf_launch_count() - before == 2
+
+
+@pytest.mark.parametrize("m,k,n,r", [(1030, 260, 260, 68), (516, 1540, 1030, 128), (2048, 128, 516, 132)])
+def test_fp32_wide_tiles_in_more_slices(m, k, n, r):
+    """fp32 reductions that take 128-column tiles in more slices instead of 64-column ones: ragged tiles, same accuracy."""
+    errs = run_case(wl.LinearCase("f32wide", m, k, n, r, wl.F32, 75))
+    assert max(errs.values()) <= 1e-5, errs
