@@ -166,7 +166,7 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
                     int64_t ldv, void* y, int64_t ldy, void* T_stash, int64_t ldt,
                     int64_t m, int64_t k, int64_t n, int64_t r, int dtype,
                     void* workspace, size_t workspace_bytes, void* cuda_stream, bool exact_need, const void* bias,
-                    int act) {
+                    int act, bool group_member) {
     int st = validate_linear_common(x, ldx, U, ldu, V, ldv, m, k, n, r, dtype);
     if (st != PF_OK) return st;
     if ((act != PF_ACT_NONE && act != PF_ACT_RELU) || (bias && !elem_aligned(bias, dtype))) return PF_ERR_INVALID_ARG;
@@ -180,7 +180,7 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
     a.y = y; a.ldy = ldy; a.T = T_stash; a.ldt = ldt;
     a.m = m; a.k = k; a.n = n; a.r = r;
     a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.stream = stream;
-    a.bias = bias; a.act = act;
+    a.bias = bias; a.act = act; a.group_member = group_member;
     size_t need = w.total;
     const bool is_small = dtype == PF_BF16 ? small::linear_fwd_fits(m, k, n, r) && !tc::few_rows_fused(a) : small::f32_fits(m, k, n, r, false);
     if (exact_need && is_small) {
@@ -314,6 +314,7 @@ int pf_lowrank_linear_bwd_ex(const void* x, int64_t ldx, const void* U, int64_t 
     a.dX = dX; a.lddx = lddx; a.dU = dU; a.lddu = lddu; a.dV = dV; a.lddv = lddv;
     a.m = m; a.k = k; a.n = n; a.r = r;
     a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.ws_G = ws + w.off_G; a.stream = stream;
+    if (T_stash && small::tiny_fits(m, k, n, r, dtype)) return small::tiny_bwd(a, dtype, gdtype == PF_F32, g_acc);
     if (dtype == PF_BF16) {
         tc::LinearArgs::Slices su_info, sv_info;
         if (flags) {
@@ -452,7 +453,7 @@ int pf_lowrank_linear_grouped_fwd(int groups, const void* x, int64_t ldx, int64_
     for (int g = 0; g < groups; ++g) {
         rc = linear_fwd_impl(at_c(x, sx, g, dtype), ldx, at_c(U, su, g, dtype), ldu, at_c(V, sv, g, dtype), ldv, at_m(y, sy, g, dtype),
                              ldy, at_m(T_stash, st, g, dtype), ldt, m, k, n, r, dtype, ws + w.off_single, single, cuda_stream,
-                             false);
+                             false, nullptr, 0, true);
         if (rc != PF_OK) return rc;
     }
     return PF_OK;

@@ -138,7 +138,7 @@ cudaError_t unpack_launch(const void* flat, void* const* grads, const int64_t* n
 int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, const void* V, int64_t ldv, void* y,
                     int64_t ldy, void* T_stash, int64_t ldt, int64_t m, int64_t k, int64_t n, int64_t r, int dtype,
                     void* workspace, size_t workspace_bytes, void* cuda_stream, bool exact_need,
-                    const void* bias = nullptr, int act = 0);
+                    const void* bias = nullptr, int act = 0, bool group_member = false);
 
 // host-side count of kernels launched by this library
 void count_launch(int n = 1);

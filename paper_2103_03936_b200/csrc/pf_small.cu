@@ -418,6 +418,229 @@ int f32_run(const F32Product& a, const F32Product* b, cudaStream_t stream) {
 }
 }  // namespace
 
+// ------------------------------------------------------------------------------ the smallest layers in one launch each way
+// Up to 128 rows, k and n up to 256, r up to 32: every launch is a start, a trip to memory and a few dozen FMAs per thread,
+// so the intermediate is computed where it is needed instead of by a launch of its own.
+//   forward (fp32)  a CTA computes T of its 16 rows, whole, and then its 16 x 32 tile of y.
+//   backward        a cluster of CTAs, 16 rows each, computes G = dY V, exchanges it through distributed shared memory and
+//                   computes 32 columns of dX and 32 rows of dU; other clusters compute tiles of dV.
+// 1024 threads, so that a whole contraction is one trip to memory and a quarter of it per thread.  bf16 operands are widened
+// as they are staged, T and G rounded to bf16 as everywhere.  What bounds them is latency.
+// 64 x 256 -> 32 -> 256, fp32: forward 8.6 -> 5.8 us, backward 8.8 -> 8.2, training step 17.1 -> 13.7 with two launches less;
+// 36 x 64 -> 16 -> 64, bf16: backward 6.3 -> 5.5.
+namespace {
+
+constexpr int kTinyThreads = 1024, kTinyRows = 128, kTinyWide = 256, kTinyRank = 32;
+
+__device__ __forceinline__ float widen(float v) { return v; }
+__device__ __forceinline__ float widen(unsigned short v) { return __uint_as_float(static_cast<uint32_t>(v) << 16); }
+__device__ __forceinline__ float rounded(float v, float) { return v; }
+__device__ __forceinline__ float rounded(float v, unsigned short) { return __bfloat162float(__float2bfloat16_rn(v)); }
+__device__ __forceinline__ void put(float* p, float v) { *p = v; }
+__device__ __forceinline__ void put(unsigned short* p, float v) { *p = __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
+
+// A matrix as a contraction reads it: element (i, l) at p[i * si + l * sl], zero outside rows x len.
+template <typename E>
+struct Side {
+    const E* p;
+    long long si, sl;
+    int rows, len;
+};
+
+struct TinyTiles {
+    float a[16][kTinyWide + 4];
+    float b[kTinyWide][34];
+    float part[4][16][34];
+};
+// Element (tid / 32, tid % 32) of a 16 x 32 tile of A B, in the first 512 threads.
+template <typename E>
+__device__ __forceinline__ float tiny_product(TinyTiles& s, const Side<E>& A, int i0, const Side<E>& B, int j0) {
+    const int tid = threadIdx.x;
+    // consecutive threads read consecutive addresses: along the contraction, or along the rows / columns
+    const bool al = A.sl == 1, bl = B.sl == 1;
+    const int ai = al ? tid >> 8 : tid & 15, ak = al ? tid & 255 : tid >> 4, ai_step = al ? 4 : 0, ak_step = al ? 0 : 64;
+    const int bj = bl ? tid >> 8 : tid & 31, bk = bl ? tid & 255 : tid >> 5, bj_step = bl ? 4 : 0, bk_step = bl ? 0 : 32;
+    E ra[4], rb[8];                                   // (widened afterwards: all loads come first)
+    const E *pa = A.p + (i0 + ai) * A.si + ak * A.sl, *pb = B.p + (j0 + bj) * B.si + bk * B.sl;
+    const long long sa = ai_step * A.si + ak_step * A.sl, sb = bj_step * B.si + bk_step * B.sl;
+#pragma unroll
+    for (int q = 0; q < 4; ++q, pa += sa) ra[q] = i0 + ai + q * ai_step < A.rows && ak + q * ak_step < A.len ? __ldg(pa) : E(0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q, pb += sb) rb[q] = j0 + bj + q * bj_step < B.rows && bk + q * bk_step < B.len ? __ldg(pb) : E(0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s.a[ai + q * ai_step][ak + q * ak_step] = widen(ra[q]);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s.b[bk + q * bk_step][bj + q * bj_step] = widen(rb[q]);
+    __syncthreads();
+    const int group = tid >> 8, ti = (tid & 255) >> 4, tj = (tid & 15) * 2, l0 = group * 64, left = min(64, A.len - l0);
+    float c0 = 0.f, c1 = 0.f;
+#pragma unroll 4
+    for (int l = l0; l < l0 + left; l += 4) {         // (zeros behind the end)
+        const float4 a = *reinterpret_cast<const float4*>(&s.a[ti][l]);
+        const float2 b0 = *reinterpret_cast<const float2*>(&s.b[l][tj]), b1 = *reinterpret_cast<const float2*>(&s.b[l + 1][tj]);
+        const float2 b2 = *reinterpret_cast<const float2*>(&s.b[l + 2][tj]), b3 = *reinterpret_cast<const float2*>(&s.b[l + 3][tj]);
+        c0 = fmaf(a.x, b0.x, c0); c1 = fmaf(a.x, b0.y, c1);
+        c0 = fmaf(a.y, b1.x, c0); c1 = fmaf(a.y, b1.y, c1);
+        c0 = fmaf(a.z, b2.x, c0); c1 = fmaf(a.z, b2.y, c1);
+        c0 = fmaf(a.w, b3.x, c0); c1 = fmaf(a.w, b3.y, c1);
+    }
+    s.part[group][ti][tj] = c0;
+    s.part[group][ti][tj + 1] = c1;
+    __syncthreads();
+    const int row = (tid >> 5) & 15, col = tid & 31;
+    return (s.part[0][row][col] + s.part[1][row][col]) + (s.part[2][row][col] + s.part[3][row][col]);
+}
+
+struct TinyFwd {
+    const float *x, *U, *V, *bias;
+    float *y, *T;                     // T: the stash or null
+    long long ldx, ldu, ldv, ldy, ldt;
+    int m, k, n, r, act;
+};
+struct TinyFwdSmem {
+    TinyTiles s;
+    float t[16][kTinyRank + 1], v[kTinyRank][33];
+};
+__global__ void __launch_bounds__(kTinyThreads) tiny_fwd_kernel(const __grid_constant__ TinyFwd p) {
+    extern __shared__ __align__(16) uint8_t tiny_smem[];
+    TinyFwdSmem& s = *reinterpret_cast<TinyFwdSmem*>(tiny_smem);
+    const int tid = threadIdx.x, row = tid >> 5, col = tid & 31, i0 = blockIdx.x * 16, j0 = blockIdx.y * 32, j = j0 + col;
+    pdl_wait();
+    pdl_launch_dependents();
+    const float v = j0 + row < p.n && col < p.r ? __ldg(p.V + (j0 + row) * p.ldv + col) : 0.f;      // in flight beside the first product
+    const float bias = p.bias && j < p.n ? __ldg(p.bias + j) : 0.f;
+    const float t = tiny_product(s.s, Side<float>{p.x, p.ldx, 1, p.m, p.k}, i0, Side<float>{p.U, 1, p.ldu, p.r, p.k}, 0);
+    s.v[col][row] = v;
+    if (tid < 512) {
+        s.t[row][col] = t;
+        if (p.T && blockIdx.y == 0 && i0 + row < p.m && col < p.r) p.T[(i0 + row) * p.ldt + col] = t;
+    }
+    __syncthreads();
+    if (tid >= 512 || i0 + row >= p.m || j >= p.n) return;
+    float c = 0.f;
+#pragma unroll 8
+    for (int l = 0; l < p.r; ++l) c = fmaf(s.t[row][l], s.v[l][col], c);
+    c += bias;
+    if (p.act == PF_ACT_RELU) c = fmaxf(c, 0.f);
+    p.y[(i0 + row) * p.ldy + j] = c;
+}
+
+struct TinyBwd {
+    const void *x, *U, *V, *dY, *T;
+    void *dX, *dU, *dV;               // dX may be null
+    long long ldx, ldu, ldv, lddy, ldt, lddx, lddu, lddv;
+    int m, k, n, r;
+    int ranks, k_clusters;            // CTAs of a cluster; clusters that compute dX and dU
+    int grads_f32, accumulate;
+};
+struct TinyBwdSmem {
+    TinyTiles s;
+    float g[kTinyRows][kTinyRank + 1];
+    float u[kTinyRank][33];           // rows j0 .. j0 + 31 of U, by rank
+    float x[2][kTinyRows][17];        // 16 columns of x per half of the threads
+};
+template <typename E>
+__device__ __forceinline__ void put_grad(const TinyBwd& p, void* grad, long long at, float v) {
+    if (p.grads_f32) {
+        float* d = static_cast<float*>(grad) + at;
+        *d = p.accumulate ? *d + v : v;
+    } else {
+        E* d = static_cast<E*>(grad) + at;
+        put(d, p.accumulate ? widen(*d) + v : v);
+    }
+}
+template <typename E>
+__global__ void __launch_bounds__(kTinyThreads) tiny_bwd_kernel(const __grid_constant__ TinyBwd p) {
+    extern __shared__ __align__(16) uint8_t tiny_smem[];
+    TinyBwdSmem& s = *reinterpret_cast<TinyBwdSmem*>(tiny_smem);
+    const int tid = threadIdx.x, half = tid >> 9, row = (tid >> 5) & 15, col = tid & 31;
+    const int cluster = blockIdx.x / p.ranks, rank = blockIdx.x - cluster * p.ranks;
+    const E *x = static_cast<const E*>(p.x), *U = static_cast<const E*>(p.U), *V = static_cast<const E*>(p.V), *dY = static_cast<const E*>(p.dY);
+    const bool with_k = cluster < p.k_clusters;
+    if (with_k) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");      // (waited for before G travels: every CTA runs by then)
+    pdl_wait();
+    pdl_launch_dependents();
+    if (!with_k) {                    // tiles of dV = dY^T T
+        const int i0 = ((cluster - p.k_clusters) * p.ranks + rank) * 16;
+        if (i0 >= p.n) return;
+        const float v = tiny_product(s.s, Side<E>{dY, 1, p.lddy, p.n, p.m}, i0, Side<E>{static_cast<const E*>(p.T), 1, p.ldt, p.r, p.m}, 0);
+        if (half == 0 && i0 + row < p.n && col < p.r) put_grad<E>(p, p.dV, (i0 + row) * p.lddv + col, v);
+        return;
+    }
+    const int i0 = rank * 16, j0 = cluster * 32;
+    // dU's two tiles of 16 rows: both on one CTA, a half of the threads each, or one on each of the first two ranks
+    const int tile = p.ranks == 1 ? half : half == 0 ? rank : 2, r0 = j0 + tile * 16;
+    const bool with_u = tile < 2 && r0 < p.k;
+    // in flight beside the first product: U's rows and x's columns
+    const E ru = p.dX && j0 + (tid >> 5) < p.k && col < p.r ? __ldg(U + (j0 + (tid >> 5)) * p.ldu + col) : E(0);
+    E rx[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = tid & 15, l = ((tid & 511) >> 4) + 32 * q;
+        rx[q] = with_u && l < p.m && r0 + i < p.k ? __ldg(x + l * p.ldx + r0 + i) : E(0);
+    }
+    const float g = rounded(tiny_product(s.s, Side<E>{dY, p.lddy, 1, p.m, p.n}, i0, Side<E>{V, 1, p.ldv, p.r, p.n}, 0), E());
+    s.u[col][tid >> 5] = widen(ru);
+    if (with_u)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s.x[half][((tid & 511) >> 4) + 32 * q][tid & 15] = widen(rx[q]);
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    const uint32_t local = static_cast<uint32_t>(__cvta_generic_to_shared(&s.g[i0 + row][col]));
+    for (int to = half; to < p.ranks; to += 2) {
+        uint32_t addr;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(local), "r"(to));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(g) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (p.dX && half == 1 && i0 + row < p.m && j0 + col < p.k) {       // dX = G U^T: this rank's rows, 32 columns
+        float c = 0.f;
+#pragma unroll 8
+        for (int l = 0; l < p.r; ++l) c = fmaf(s.g[i0 + row][l], s.u[l][col], c);
+        put(static_cast<E*>(p.dX) + (i0 + row) * p.lddx + j0 + col, c);
+    }
+    if (with_u && r0 + row < p.k && col < p.r) {      // dU = x^T G
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int l = 0; l < p.m; l += 4)              // (rows of G behind the batch are zero, and so is x)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c[e] = fmaf(s.x[half][l + e][row], s.g[l + e][col], c[e]);
+        put_grad<E>(p, p.dU, (r0 + row) * p.lddu + col, (c[0] + c[1]) + (c[2] + c[3]));
+    }
+}
+}  // namespace
+
+// bf16 only up to a width of 128: the backward of 128 x 256 -> 32 -> 256 takes 10.4 us here, 7.1 in two launches on the tensor
+// cores; of 100 x 250 -> 30 -> 130 8.0 and 10.6.
+bool tiny_fits(int64_t m, int64_t k, int64_t n, int64_t r, int dtype) {
+    const int wide = dtype == PF_BF16 ? kTinyWide / 2 : kTinyWide;
+    return m >= 1 && m <= kTinyRows && k <= wide && n <= wide && r <= kTinyRank;
+}
+// The whole backward in one launch, T given; gradients in fp32 and / or accumulated directly.
+int tiny_bwd(const tc::LinearArgs& a, int dtype, bool grads_f32, bool accumulate) {
+    TinyBwd p;
+    p.x = a.x; p.U = a.U; p.V = a.V; p.dY = a.dY; p.T = a.T; p.dX = a.dX; p.dU = a.dU; p.dV = a.dV;
+    p.ldx = a.ldx; p.ldu = a.ldu; p.ldv = a.ldv; p.lddy = a.lddy; p.ldt = a.ldt; p.lddx = a.lddx; p.lddu = a.lddu; p.lddv = a.lddv;
+    p.m = static_cast<int>(a.m); p.k = static_cast<int>(a.k); p.n = static_cast<int>(a.n); p.r = static_cast<int>(a.r);
+    p.ranks = (p.m + 15) / 16;                      // at most 8, the largest portable cluster
+    p.k_clusters = (p.k + 31) / 32;
+    p.grads_f32 = grads_f32; p.accumulate = accumulate;
+    const int v_tiles = (p.n + 15) / 16;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((p.k_clusters + (v_tiles + p.ranks - 1) / p.ranks) * p.ranks)); cfg.blockDim = dim3(kTinyThreads);
+    cfg.dynamicSmemBytes = sizeof(TinyBwdSmem); cfg.stream = a.stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(p.ranks); attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    auto* kernel = dtype == PF_BF16 ? tiny_bwd_kernel<unsigned short> : tiny_bwd_kernel<float>;
+    if (tc::allow_smem(kernel, sizeof(TinyBwdSmem)) != cudaSuccess || cudaLaunchKernelEx(&cfg, kernel, p) != cudaSuccess) return PF_ERR_CUDA;
+    count_launch();
+    return PF_OK;
+}
+
 // Every product short (its contraction in two loads) and small.  Beyond, the tensor cores are as fast or faster
 // (128 x 512 -> 512, r 64: 13.7 + 15.2 against 13.4 + 15.4 us; 512 x 512 -> 512, r 32: 14.0 against 16.4;
 // caches warm).
@@ -426,6 +649,20 @@ bool f32_fits(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd) {
     return longest <= 256 && n <= 4096 && m <= 4096 && m * r * std::max(k, n) <= (1 << 21);
 }
 int f32_linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt) {
+    if (!a.group_member && tiny_fits(a.m, a.k, a.n, a.r, PF_F32)) {
+        TinyFwd p;
+        p.x = static_cast<const float*>(a.x); p.U = static_cast<const float*>(a.U); p.V = static_cast<const float*>(a.V);
+        p.bias = static_cast<const float*>(a.bias);
+        p.y = static_cast<float*>(a.y); p.T = static_cast<float*>(a.T);
+        p.ldx = a.ldx; p.ldu = a.ldu; p.ldv = a.ldv; p.ldy = a.ldy; p.ldt = a.ldt;
+        p.m = static_cast<int>(a.m); p.k = static_cast<int>(a.k); p.n = static_cast<int>(a.n); p.r = static_cast<int>(a.r); p.act = a.act;
+        const dim3 grid(static_cast<unsigned>(ceil_div(a.m, 16)), static_cast<unsigned>(ceil_div(a.n, 32)));
+        if (tc::allow_smem(tiny_fwd_kernel, sizeof(TinyFwdSmem)) != cudaSuccess ||
+            tc::launch_overlapped(tiny_fwd_kernel, grid, dim3(kTinyThreads), sizeof(TinyFwdSmem), a.stream, p) != cudaSuccess)
+            return PF_ERR_CUDA;
+        count_launch();
+        return PF_OK;
+    }
     const int st = f32_run(f32_product(a.x, a.ldx, 1, a.U, a.ldu, 1, T, ldt, a.m, a.r, a.k), nullptr, a.stream);
     if (st != PF_OK) return st;
     F32Product y = f32_product(T, ldt, 1, a.V, 1, a.ldv, a.y, a.ldy, a.m, a.n, a.r);

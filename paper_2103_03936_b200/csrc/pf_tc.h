@@ -21,6 +21,7 @@ struct LinearArgs {
     cudaStream_t stream = nullptr;
     const void* bias = nullptr;   // forward: y = act((x U) V^T + bias)
     int act = 0;
+    bool group_member = false;    // one of several calls that make up a grouped one (two launches each, as documented)
     // backward: where the fp32 slices of dU / dV were left in the workspace (partial null: nowhere), for callers that want
     // the unrounded sums; a product that is one slice leaves only that
     struct Slices {
@@ -142,6 +143,9 @@ int conv_bwd(const ConvArgs& a, int* handled);
 namespace small {
 bool linear_fwd_fits(int64_t m, int64_t k, int64_t n, int64_t r);
 int linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt);
+// The smallest layers, any layout: the whole backward in one launch (needs T; a.dU and a.dV are the caller's).
+bool tiny_fits(int64_t m, int64_t k, int64_t n, int64_t r, int dtype);
+int tiny_bwd(const tc::LinearArgs& a, int dtype, bool grads_f32, bool accumulate);
 // fp32, small products, any layout.
 bool f32_fits(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd);
 int f32_linear_fwd(const tc::LinearArgs& a, void* T, int64_t ldt);

@@ -384,3 +384,46 @@ def test_fp32_wide_tiles_in_more_slices(m, k, n, r):
     """fp32 reductions that take 128-column tiles in more slices instead of 64-column ones: ragged tiles, same accuracy."""
     errs = run_case(wl.LinearCase("f32wide", m, k, n, r, wl.F32, 75))
     assert max(errs.values()) <= 1e-5, errs
+
+
+@pytest.mark.parametrize("dtype", [wl.F32, wl.BF16])
+@pytest.mark.parametrize("m,k,n,r", [(1, 1, 1, 1), (16, 32, 16, 32), (17, 33, 17, 31), (64, 256, 256, 32), (128, 128, 128, 32), (113, 100, 7, 31), (128, 5, 128, 2), (40, 24, 16, 8)])
+def test_smallest_layers_in_one_launch_each_way(dtype, m, k, n, r):
+    """Up to 128 rows, k and n up to 256 (bf16: 128), r up to 32: edges of the 16- and 32-wide tiles and of the cluster, any
+    pitch; the backward is one launch, and so is the fp32 forward."""
+    if dtype == wl.BF16:
+        k, n = min(k, 128), min(n, 128)
+    case = wl.LinearCase("tiny", m, k, n, r, dtype, 76)
+    run_case(case, ld_pad=0, tiny=True)
+    run_case(case, ld_pad=3, tiny=True, need_dX=False)
+    d = case.generate()
+    x, U, V, dY = (dev(d[k_], dtype) for k_ in ("x", "U", "V", "dY"))
+    before = pf.pf_launch_count()
+    _, T = pf.pf_lowrank_linear_fwd(x, U, V, want_stash=True)
+    assert dtype == wl.BF16 or pf.pf_launch_count() - before == 1
+    before = pf.pf_launch_count()
+    dX, dU, dV = pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T)
+    assert pf.pf_launch_count() - before == 1
+    # fp32 gradients are the same sums, unrounded; accumulating adds to them once
+    gU, gV = torch.ones_like(dU, dtype=torch.float32), torch.ones_like(dV, dtype=torch.float32)
+    pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T, dU=gU, dV=gV, grads_f32=True)
+    assert torch.equal(gU.to(dU.dtype), dU) and torch.equal(gV.to(dV.dtype), dV)
+    aU, aV = torch.ones_like(gU), torch.ones_like(gV)
+    pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T, dU=aU, dV=aV, grads_f32=True, accumulate=True)
+    assert torch.equal(aU, gU + 1) and torch.equal(aV, gV + 1)
+    bU, bV = torch.ones_like(dU), torch.ones_like(dV)
+    pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T, dU=bU, dV=bV, accumulate=True)
+    assert torch.equal(bU, (gU + 1).to(dU.dtype)) and torch.equal(bV, (gV + 1).to(dV.dtype))
+
+
+def test_smallest_layers_with_infinities_and_nan():
+    """What is not finite reaches the outputs it belongs to and no others."""
+    m, k, n, r = 40, 64, 48, 16
+    for dtype in (torch.float32, torch.bfloat16):
+        x, U = torch.ones(m, k, device="cuda", dtype=dtype), torch.ones(k, r, device="cuda", dtype=dtype)
+        V, dY, T = torch.ones(n, r, device="cuda", dtype=dtype), torch.ones(m, n, device="cuda", dtype=dtype), torch.ones(m, r, device="cuda", dtype=dtype)
+        dY[3, 5], T[7, 2], x[9, 11] = float("inf"), float("nan"), float("-inf")
+        dX, dU, dV = pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T)
+        assert torch.isinf(dX[3]).all() and torch.isfinite(dX[torch.arange(m, device="cuda") != 3]).all()
+        assert torch.isnan(dV[:, 2]).all() and torch.isinf(dV[5, 0]) and torch.isfinite(dV[6, 0])
+        assert (dU[11].isinf() | dU[11].isnan()).all() and torch.isinf(dU[0]).all()
