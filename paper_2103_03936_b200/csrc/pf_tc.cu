@@ -174,6 +174,10 @@ void bwd_split_plan(int64_t m, int64_t k, int64_t n, int64_t r, bool fused_dx, i
     // dU gets the SMs that dV does not hold: dV may still be running when the fused kernel retires
     const int64_t a = std::min((num_sms() - tv * b) / tu, smax);
     if (a < 1 || b < 1) return;
+    // ... unless too few SMs are left: dV has to be done with about when the fused kernel is (16384 rows, 512 -> 128 -> 2048, 16
+    // of the 20 free SMs: 84 us beside, 38.5 behind; 256 -> 32 -> 1024: 32.1 and 23.7)
+    const double chain_us = 3.8 + 0.31 * static_cast<double>(ceil_div(n, kBK)) + 0.65 * static_cast<double>(ceil_div(k, 128));
+    if (slice_us(nkb, b) > 1.5 * chain_us) return;
     *su = static_cast<int>(a);
     *sv = static_cast<int>(b);
     *beside = true;
@@ -516,6 +520,10 @@ int stage_operand(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& 
 // rank is small enough for the layer to be bound by memory traffic: from r = 256 up the two
 // products are tensor-bound and run faster unfused on CTA pairs (the intermediate is only m x r).
 bool use_chain(int64_t m, int64_t r) { return m >= 2048 && r <= 192; }
+// Batches that just fill a few SMs per row tile, with the longer contraction in the fused kernel's first product, which a block
+// contracts alone: 2048 x 512 -> 128 -> 2048: 22.0 us fused, 18.3 unfused; 3000: 22.3 and 19.8; 4096: 23.2 and 22.2; 2048 x 1024 ->
+// 64 -> 1024: 15.9 and 14.9; but 2048 x 2048 -> 128 -> 512: 17.6 and 19.4, 2048 x 768 -> 192 -> 768: 18.9 and 20.5.
+bool unfused_backward(int64_t m, int64_t k, int64_t n, int64_t r) { return m < 3500 && n >= k && n >= 1024 && r <= 128; }
 // The forward's fused kernel is one launch instead of two, so it takes smaller batches too, while its first product, which
 // one block contracts alone where the unfused one is split over the SMs, is short.  Fused against unfused, caches warm:
 // 300 x 512 -> 128 -> 2048: 6.4 against 8.7 us; 1000 x 1536 -> 128 -> 1536: 10.5 / 11.7; 500 x 2048 -> 128 -> 2048: 11.7 / 11.7;
@@ -712,7 +720,7 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     scratch += align_up(static_cast<size_t>(a.m) * ldG * 2, 256);
     size_t pu_bytes = 0, pv_bytes = 0;
     ChainPlan plan;
-    const bool fused_dx = use_chain(a.m, a.r) && (!a.dX || tma_ok(a.dX, a.lddx)) &&
+    const bool fused_dx = use_chain(a.m, a.r) && !unfused_backward(a.m, a.k, a.n, a.r) && (!a.dX || tma_ok(a.dX, a.lddx)) &&
                           chain_plan(a.m, a.n, a.k, a.r, a.dX != nullptr, &plan);
     int su, sv;
     bool dv_beside;

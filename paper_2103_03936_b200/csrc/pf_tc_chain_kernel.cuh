@@ -204,6 +204,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 }
         }
     }
+    const uint64_t a_policy = kConv == 0 ? l2_policy(p.keep_a) : 0, out_policy = kConv == 0 ? l2_policy(p.keep_out) : 0;
     // (The second half of the groups runs beside the first: when it starts, everything older than that is complete, since
     // every kernel of this library lets its successor start only after its own wait.  It waits before it ends, so that
     // whoever waits for it has waited for both.)
@@ -220,7 +221,6 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (elect_one()) {
             // -------------------------------------------------------------- TMA producer of A (phase 1)
             RingPos rp;
-            const uint64_t a_policy = kConv == 0 ? l2_policy(p.keep_a) : 0;
             const uint32_t txa = static_cast<uint32_t>(p.rows_tile) * 128u;
             const int skip = ntile * ((nkb2 + bps - 1) / bps);      // stages of a tile's phase 2 (B2 only)
             bool ok = true;
@@ -435,7 +435,6 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             stg = ring + (ew / per_stage) * S + kTileBytes + (ew % per_stage) * 4096;
         }
         const uint32_t prow = stg + lane * 128;
-        const uint64_t out_policy = kConv == 0 ? l2_policy(p.keep_out) : 0;
         bool stored = false, ok = true;
         AccPos ap;
         uint32_t it = 0;

@@ -427,3 +427,9 @@ def test_smallest_layers_with_infinities_and_nan():
         assert torch.isinf(dX[3]).all() and torch.isfinite(dX[torch.arange(m, device="cuda") != 3]).all()
         assert torch.isnan(dV[:, 2]).all() and torch.isinf(dV[5, 0]) and torch.isfinite(dV[6, 0])
         assert (dU[11].isinf() | dU[11].isnan()).all() and torch.isinf(dU[0]).all()
+
+
+@pytest.mark.parametrize("m,k,n,r", [(2049, 136, 1032, 64), (3499, 136, 1032, 72), (3500, 136, 1032, 72), (2100, 1032, 1024, 40), (16300, 72, 264, 16), (12000, 72, 1032, 16)])
+def test_backward_schedules(m, k, n, r):
+    """Either side of the sizes from which the backward's fused kernel is used, and from which dV runs beside it."""
+    run_case(wl.LinearCase("schedule", m, k, n, r, wl.BF16, 77), blocks=True)
