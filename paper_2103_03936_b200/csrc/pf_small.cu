@@ -579,7 +579,8 @@ __global__ void __launch_bounds__(kTinyThreads) tiny_bwd_kernel(const __grid_con
         const int i = tid & 15, l = ((tid & 511) >> 4) + 32 * q;
         rx[q] = with_u && l < p.m && r0 + i < p.k ? __ldg(x + l * p.ldx + r0 + i) : E(0);
     }
-    const float g = rounded(tiny_product(s.s, Side<E>{dY, p.lddy, 1, p.m, p.n}, i0, Side<E>{V, 1, p.ldv, p.r, p.n}, 0), E());
+    const float sum = tiny_product(s.s, Side<E>{dY, p.lddy, 1, p.m, p.n}, i0, Side<E>{V, 1, p.ldv, p.r, p.n}, 0);
+    const float g = i0 + row < p.m ? rounded(sum, E()) : 0.f;         // (zero times an infinity of V is no zero)
     s.u[col][tid >> 5] = widen(ru);
     if (with_u)
 #pragma unroll

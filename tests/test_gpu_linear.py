@@ -429,6 +429,17 @@ def test_smallest_layers_with_infinities_and_nan():
         assert (dU[11].isinf() | dU[11].isnan()).all() and torch.isinf(dU[0]).all()
 
 
+def test_smallest_layers_infinite_factor_and_a_ragged_batch():
+    """An infinity in V makes its column of dY V and of dU infinite; the rows that pad the batch to whole tiles add nothing."""
+    m, k, n, r = 41, 64, 48, 16
+    for dtype in (torch.float32, torch.bfloat16):
+        x, U, V, dY, T = (torch.ones(s, device="cuda", dtype=dtype) for s in ((m, k), (k, r), (n, r), (m, n), (m, r)))
+        V[5, 3] = float("inf")
+        dX, dU, dV = pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T)
+        assert torch.isposinf(dX).all() and torch.isposinf(dU[:, 3]).all()
+        assert (dU[:, 4] == m * n).all() and (dV == m).all()
+
+
 @pytest.mark.parametrize("m,k,n,r", [(2049, 136, 1032, 64), (3499, 136, 1032, 72), (3500, 136, 1032, 72), (2100, 1032, 1024, 40), (16300, 72, 264, 16), (12000, 72, 1032, 16)])
 def test_backward_schedules(m, k, n, r):
     """Either side of the sizes from which the backward's fused kernel is used, and from which dV runs beside it."""
