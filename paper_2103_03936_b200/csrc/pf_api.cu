@@ -187,11 +187,13 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
         need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * dtype_size(dtype);
     } else if (exact_need) {
         bool tc_handles = false;
-        size_t tc_need = dtype == PF_BF16 ? tc::linear_fwd_need(a, &tc_handles) : 0;
-        if (dtype == PF_F32) {        // (taken only when it fits; the FMA kernels need less)
-            tc_need = tc::f32_linear_workspace(m, k, n, r, false);
-            tc_handles = w.off_tc + tc_need <= workspace_bytes;
+        size_t tc_need = 0;
+        for (int lean = 0; lean < 2; ++lean) {
+            a.tight = lean;
+            tc_need = dtype == PF_BF16 ? tc::linear_fwd_need(a, &tc_handles) : tc::f32_linear_workspace(m, k, n, r, false, lean);
+            if (w.off_tc + tc_need <= workspace_bytes) break;
         }
+        if (dtype == PF_F32) tc_handles = tc_need > 0 && w.off_tc + tc_need <= workspace_bytes;        // (taken only when it fits; the FMA kernels need less)
         if (tc_handles) need = tc_need ? w.off_tc + tc_need : 0;
         else need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * dtype_size(dtype);   // FMA kernels: x U only
     }

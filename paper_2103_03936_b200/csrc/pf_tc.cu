@@ -493,7 +493,7 @@ struct Staged {
 // Pitch of a matrix in the workspace: whole 128-byte lines, so that no 128-byte row of a TMA box touches two of them (narrow
 // rows: whole 16-byte pieces).  8 x (700 x 1500 -> 1500), r 375: forward 43.7 -> 37.5 us, backward 81.0 -> 62.5, against
 // pitches of 376 and 1504 elements; 3000 x 2000 -> 500 -> 500: 28.7 -> 24.4 and 48.8 -> 39.7.
-int64_t row_pitch(int64_t v) { return v > 32 ? (v + 63) / 64 * 64 : (v + 7) / 8 * 8; }
+int64_t row_pitch(int64_t v, bool tight = false) { return v > 32 && !tight ? (v + 63) / 64 * 64 : (v + 7) / 8 * 8; }
 
 // The re-pitch copies of one call are collected and issued as one launch.
 struct RepackList {
@@ -507,10 +507,10 @@ struct RepackList {
 };
 
 // returns 0 = usable, 1 = needs repack but no room reserved (decline), <0 never
-int stage_operand(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& scratch, Staged* out, RepackList* list) {
+int stage_operand(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& scratch, Staged* out, RepackList* list, bool tight = false) {
     if (tma_ok(p, ld)) { out->p = p; out->ld = ld; return 0; }
     if (cols % 8 == 0) return 1;   // the workspace query reserves repack room only for ragged widths
-    const int64_t ldp = row_pitch(cols);
+    const int64_t ldp = row_pitch(cols, tight);
     list->jobs[list->count++] = RepackJob{p, ld, scratch, ldp, rows, cols};
     out->p = scratch; out->ld = ldp;
     scratch += align_up(static_cast<size_t>(rows) * ldp * 2, 256);
@@ -544,8 +544,8 @@ bool use_chain_fwd(const LinearArgs& a) {
     return a.m >= 2048 || (short_first_product(a.k, a.r, tma_ok(a.x, a.ldx) ? a.ldx : 0, tma_ok(a.U, a.ldu) ? a.ldu : 0, 1536) && (!a.T || tma_ok(a.T, a.ldt)));
 }
 
-size_t repack_room(int64_t rows, int64_t cols) {
-    return cols % 8 == 0 ? 0 : align_up(static_cast<size_t>(rows) * row_pitch(cols) * 2, 256);
+size_t repack_room(int64_t rows, int64_t cols, bool tight = false) {
+    return cols % 8 == 0 ? 0 : align_up(static_cast<size_t>(rows) * row_pitch(cols, tight) * 2, 256);
 }
 
 // Whether the tiles of dU (rows_u x r) and dV (rows_v x r) fit the machine together.  Such reductions run on single CTAs,
@@ -626,10 +626,10 @@ size_t linear_fwd_need(const LinearArgs& a, bool* handles) {
     for (const auto& o : ops) {
         if (tma_ok(o.p, o.ld)) continue;
         if (o.cols % 8 == 0) return 0;               // declined: FMA kernels
-        room += repack_room(o.rows, o.cols);
+        room += repack_room(o.rows, o.cols, a.tight);
     }
     *handles = true;
-    const size_t t_bytes = align_up(static_cast<size_t>(a.m) * row_pitch(a.r) * 2, 256);
+    const size_t t_bytes = align_up(static_cast<size_t>(a.m) * row_pitch(a.r, a.tight) * 2, 256);
     const bool stash_direct = a.T && tma_ok(a.T, a.ldt);
     ChainPlan plan;
     if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan))
@@ -651,15 +651,15 @@ int linear_fwd(const LinearArgs& a, int* handled) {
     char* scratch = a.ws;
     Staged x, U, V;
     RepackList repacks;
-    if (stage_operand(a.x, a.ldx, a.m, a.k, scratch, &x, &repacks)) return PF_OK;
-    if (stage_operand(a.U, a.ldu, a.k, a.r, scratch, &U, &repacks)) return PF_OK;
-    if (stage_operand(a.V, a.ldv, a.n, a.r, scratch, &V, &repacks)) return PF_OK;
+    if (stage_operand(a.x, a.ldx, a.m, a.k, scratch, &x, &repacks, a.tight)) return PF_OK;
+    if (stage_operand(a.U, a.ldu, a.k, a.r, scratch, &U, &repacks, a.tight)) return PF_OK;
+    if (stage_operand(a.V, a.ldv, a.n, a.r, scratch, &V, &repacks, a.tight)) return PF_OK;
     st = repacks.flush(a.stream);
     if (st != PF_OK) return st;
     *handled = 1;
     // T: written straight into the stash when TMA can read it back, else into padded scratch
     void* T = scratch;
-    int64_t ldT = row_pitch(a.r);
+    int64_t ldT = row_pitch(a.r, a.tight);
     const bool stash_direct = a.T && tma_ok(a.T, a.ldt);
     if (stash_direct) { T = a.T; ldT = a.ldt; }
     ChainPlan plan;
@@ -669,7 +669,7 @@ int linear_fwd(const LinearArgs& a, int* handled) {
         st = chain(x.p, x.ld, a.m, a.k, U.p, U.ld, a.r, V.p, V.ld, a.n, a.y, a.ldy, a.T ? T : nullptr, ldT,
                    a.stream, nullptr, 0, a.bias, a.act, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f);
     } else {
-        float* p1 = reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * row_pitch(a.r) * 2, 256));
+        float* p1 = reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * row_pitch(a.r, a.tight) * 2, 256));
         st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, T, ldT,
                   pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream,
                   (a.T && !stash_direct) ? a.T : nullptr, a.ldt, &stash_written);

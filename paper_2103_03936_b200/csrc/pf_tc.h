@@ -21,6 +21,7 @@ struct LinearArgs {
     cudaStream_t stream = nullptr;
     const void* bias = nullptr;   // forward: y = act((x U) V^T + bias)
     int act = 0;
+    bool tight = false;           // forward: the leaner plan, for a workspace of a given size that the faster one does not fit
     bool group_member = false;    // one of several calls that make up a grouped one (two launches each, as documented)
     // backward: where the fp32 slices of dU / dV were left in the workspace (partial null: nowhere), for callers that want
     // the unrounded sums; a product that is one slice leaves only that
@@ -124,7 +125,7 @@ bool few_rows_fused(const LinearArgs& a);     // a forward that small::linear_fw
 int linear_bwd(const LinearArgs& a, int* handled);
 
 // fp32 storage (pf_tc_f32.cu).  `room`: bytes available at a.ws (a call that does not fit is declined).
-size_t f32_linear_workspace(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd);
+size_t f32_linear_workspace(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd, bool tight = false);
 int f32_linear_fwd(const LinearArgs& a, int* handled, size_t room);
 int f32_linear_bwd(const LinearArgs& a, int* handled);
 size_t f32_conv_workspace(const ConvArgs& a, bool bwd);      // a: sizes only

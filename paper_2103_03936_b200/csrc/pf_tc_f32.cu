@@ -14,7 +14,7 @@ namespace pf {
 namespace tc {
 namespace {
 
-int64_t f32_pitch(int64_t v) { return v > 16 ? (v + 31) / 32 * 32 : (v + 3) / 4 * 4; }      // whole 128-byte lines, as row_pitch
+int64_t f32_pitch(int64_t v, bool tight = false) { return v > 16 && !tight ? (v + 31) / 32 * 32 : (v + 3) / 4 * 4; }      // whole 128-byte lines, as row_pitch
 bool f32_tma_ok(const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 4 == 0 && ld * 4 < (1LL << 40); }
 
 // fp32 tensor maps with boxes of 32 columns (128 bytes): rank 2 = [rows, cols], rank 3 = [planes][rows][cols]
@@ -157,8 +157,10 @@ double f32_us(F32Work* const* w, int count) {
 // Slices, and the widths of the tiles: 128 columns do in one k-block of 0.95 us what two 64-column tiles do in 1.34, so long
 // contractions are better cut into more slices of wide tiles: backward of 2048 x 512 -> 128 -> 2048: 45.7 -> 37.3 us, of 1000 x 1024 ->
 // 256 -> 1024: 43.1 -> 31.9; forward of 2048 x 2048 -> 128 -> 512: 26.1 -> 23.3.
-void f32_split(F32Work* const* w, const bool* can, int count) {
+// tight: less room, not less time (the slices of wide tiles take up to twice the bytes).
+void f32_split(F32Work* const* w, const bool* can, int count, bool tight = false) {
     f32_slices(w, can, count);
+    if (tight) return;
     F32Work wide[2];
     F32Work* pw[2] = {&wide[0], &wide[1]};
     bool other = false;
@@ -272,28 +274,28 @@ struct Staged32 {
     const void* p;
     int64_t ld;
 };
-bool f32_stage(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& scratch, Staged32* out, RepackJob* jobs, int* count) {
+bool f32_stage(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& scratch, Staged32* out, RepackJob* jobs, int* count, bool tight = false) {
     *out = Staged32{p, ld};
     if (f32_tma_ok(p, ld)) return true;
     if (cols % 4 == 0) return false;      // the workspace query reserves repack room only for ragged widths
-    const int64_t ldp = f32_pitch(cols);
+    const int64_t ldp = f32_pitch(cols, tight);
     jobs[(*count)++] = RepackJob{p, 2 * ld, scratch, 2 * ldp, rows, 2 * cols};
     *out = Staged32{scratch, ldp};
     scratch += align_up(static_cast<size_t>(rows) * ldp * 4, 256);
     return true;
 }
-size_t f32_room(int64_t rows, int64_t cols) { return cols % 4 == 0 ? 0 : align_up(static_cast<size_t>(rows) * f32_pitch(cols) * 4, 256); }
-size_t f32_mat(int64_t rows, int64_t cols) { return align_up(static_cast<size_t>(rows) * f32_pitch(cols) * 4, 256); }
+size_t f32_mat(int64_t rows, int64_t cols, bool tight = false) { return align_up(static_cast<size_t>(rows) * f32_pitch(cols, tight) * 4, 256); }
+size_t f32_room(int64_t rows, int64_t cols, bool tight = false) { return cols % 4 == 0 ? 0 : f32_mat(rows, cols, tight); }
 
 // The products of the two layers in the order they are launched, planned from the sizes alone.
 struct F32Fwd {
     F32Work t, y;
 };
-F32Fwd f32_plan_fwd(const F32Work& t, const F32Work& y) {
+F32Fwd f32_plan_fwd(const F32Work& t, const F32Work& y, bool tight = false) {
     F32Fwd f{t, y};
     F32Work* w = &f.t;
     const bool can = true;
-    f32_split(&w, &can, 1);
+    f32_split(&w, &can, 1, tight);
     return f;
 }
 struct F32Bwd {
@@ -308,7 +310,7 @@ F32Bwd f32_plan_bwd(const F32Work& t, const F32Work& g, const F32Work& dv, const
     f32_split(wb, first, 2);
     return b;
 }
-F32Fwd linear_plan_fwd(int64_t m, int64_t k, int64_t n, int64_t r) { return f32_plan_fwd(f32_work(m, r, k), f32_work(m, n, r)); }
+F32Fwd linear_plan_fwd(int64_t m, int64_t k, int64_t n, int64_t r, bool tight) { return f32_plan_fwd(f32_work(m, r, k), f32_work(m, n, r), tight); }
 F32Bwd linear_plan_bwd(int64_t m, int64_t k, int64_t n, int64_t r) {
     return f32_plan_bwd(f32_work(m, r, k), f32_work(m, r, n), f32_work(n, r, m), f32_work(k, r, m), f32_work(m, k, r));
 }
@@ -336,31 +338,31 @@ bool sizes_ok(int64_t m, int64_t k, int64_t n, int64_t r) {
 bool tiles_ok(const F32Work& w) { return w.tiles() * w.splits < (1LL << 30) && w.nkb < (1LL << 28); }
 }  // namespace
 
-size_t f32_linear_workspace(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd) {
+size_t f32_linear_workspace(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd, bool tight) {
     if (!sizes_ok(m, k, n, r) || m < 1) return 0;
-    size_t b = f32_room(m, k) + f32_room(k, r) + f32_room(n, r) + f32_mat(m, r);      // x, U, V, T
-    if (!bwd) return b + linear_plan_fwd(m, k, n, r).t.partial_bytes();
+    size_t b = f32_room(m, k, tight) + f32_room(k, r, tight) + f32_room(n, r, tight) + f32_mat(m, r, tight);      // x, U, V, T
+    if (!bwd) return b + linear_plan_fwd(m, k, n, r, tight).t.partial_bytes();
     const F32Bwd p = linear_plan_bwd(m, k, n, r);
     return b + f32_room(m, n) + f32_mat(m, r) + std::max(p.t.partial_bytes(), p.g.partial_bytes()) + p.dv.partial_bytes() + p.du.partial_bytes();
 }
 
 int f32_linear_fwd(const LinearArgs& a, int* handled, size_t room) {
     *handled = 0;
-    if (encode_fn() == nullptr || !sizes_ok(a.m, a.k, a.n, a.r) || f32_linear_workspace(a.m, a.k, a.n, a.r, false) > room) return PF_OK;
-    const F32Fwd f = linear_plan_fwd(a.m, a.k, a.n, a.r);
+    if (encode_fn() == nullptr || !sizes_ok(a.m, a.k, a.n, a.r) || f32_linear_workspace(a.m, a.k, a.n, a.r, false, a.tight) > room) return PF_OK;
+    const F32Fwd f = linear_plan_fwd(a.m, a.k, a.n, a.r, a.tight);
     if (!tiles_ok(f.t) || !tiles_ok(f.y)) return PF_OK;
     char* ws = a.ws;
     Staged32 x, U, V;
     RepackJob jobs[3];
     int nj = 0;
-    if (!f32_stage(a.x, a.ldx, a.m, a.k, ws, &x, jobs, &nj) || !f32_stage(a.U, a.ldu, a.k, a.r, ws, &U, jobs, &nj) ||
-        !f32_stage(a.V, a.ldv, a.n, a.r, ws, &V, jobs, &nj))
+    if (!f32_stage(a.x, a.ldx, a.m, a.k, ws, &x, jobs, &nj, a.tight) || !f32_stage(a.U, a.ldu, a.k, a.r, ws, &U, jobs, &nj, a.tight) ||
+        !f32_stage(a.V, a.ldv, a.n, a.r, ws, &V, jobs, &nj, a.tight))
         return PF_OK;
     // T: the stash itself when TMA can read it back, else scratch; the first product then writes the stash beside it
     const bool direct = a.T && f32_tma_ok(a.T, a.ldt);
     float* T = direct ? static_cast<float*>(a.T) : reinterpret_cast<float*>(ws);
-    const int64_t ldT = direct ? a.ldt : f32_pitch(a.r);
-    ws += f32_mat(a.m, a.r);
+    const int64_t ldT = direct ? a.ldt : f32_pitch(a.r, a.tight);
+    ws += f32_mat(a.m, a.r, a.tight);
     F32Launch l1, l2;
     if (!f32_prepare(f.t, {x.p, x.ld, false}, {U.p, U.ld, true}, T, ldT, reinterpret_cast<float*>(ws), &l1.ta[0], &l1.tb[0], &l1.p[0]) ||
         !f32_prepare(f.y, {T, ldT, false}, {V.p, V.ld, false}, static_cast<float*>(a.y), a.ldy, nullptr, &l2.ta[0], &l2.tb[0], &l2.p[0]))

@@ -111,6 +111,20 @@ def test_which_benchmark_shapes_fit_the_array():
     assert pf.pf_last_device_status() == 0
 
 
+@pytest.mark.parametrize("m,k,n,r,dtype", [(4300, 489, 203, 201, wl.BF16), (2048, 2048, 64, 128, wl.F32)])
+def test_calls_that_fit_only_the_leaner_plan(m, k, n, r, dtype):
+    """With pitches of whole 128-byte lines (bf16), or the slices of wide tiles (fp32), these need more than the array holds:
+    pitches of whole 16 bytes, or narrow tiles, fit it (8.1 and 6.3 MB)."""
+    c = wl.LinearCase("lean", m, k, n, r, dtype, 24)
+    d = c.generate()
+    x, U, V = (dev(d[k_], dtype) for k_ in ("x", "U", "V"))
+    y = torch.empty((m, n), dtype=x.dtype, device="cuda")
+    pf.pf_lowrank_linear_fwd_static(x, U, V, y=y)
+    y_ref, _ = oracle.linear_fwd(d["x"], d["U"], d["V"])
+    assert_close(y, y_ref, dtype, c.name, tol=None if dtype == wl.BF16 else 1e-5)
+    assert pf.pf_last_device_status() == 0
+
+
 def test_problem_larger_than_the_array_is_refused_before_any_launch():
     assert pf.pf_static_scratch_bytes() == 8 << 20
     m, k, n, r = 2000, 64, 64, 4096           # few rows: unfused products, and x U alone is 16 MB
