@@ -131,9 +131,9 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     }
     p.bias = bias; p.act = act;
     p.status = device_status_ptr();
-    p.a_shared = 0; p.late_wait = 0;
-    p.keep_a = keep_a; p.keep_out = keep_out;
+    p.keep[0] = keep_a; p.keep[1] = keep_out;
     dim3 grid(static_cast<unsigned>(grid_x), static_cast<unsigned>(plan.nsplit), 1);
+    if (!conv && !persistent && (keep_a != 0.f || keep_out != 0.f)) return chain_launch_hints(grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
     if (out && (bias || act)) return chain_launch_act(persistent, grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
     if (persistent) {
         // software-pipelined form: two T accumulators and two T buffers, the ring (four stages or more) behind them,
@@ -184,8 +184,8 @@ int chain_groups(int groups, int all, const void* A, int64_t lda, int64_t sA, in
     p.row_tiles = static_cast<int>(ceil_div(M, rows_tile));
     p.acc_bufs = kAccBufs;
     p.status = device_status_ptr();
-    p.a_shared = sA == 0;
-    p.late_wait = late_wait;
+    p.group_flags[0] = sA == 0;
+    p.group_flags[1] = late_wait;
     const dim3 grid(static_cast<unsigned>(p.row_tiles), static_cast<unsigned>(plan.nsplit), static_cast<unsigned>(groups));
     return chain_launch_groups(grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
 }

@@ -60,9 +60,12 @@ struct ChainParams {
     const void* bias;
     int act;
     unsigned int* status;
-    float keep_a, keep_out; // plain products: how L2 treats A and the output (see l2_policy)
-    int a_shared;           // grouped (kConv 3): all groups read one A
-    int late_wait;          // grouped: the kernel before is the other half of the groups, whose results nothing here reads
+    // Kept short: with two words more the compiler lays the epilogue of the bias form out differently (8192 x 512 -> 128 -> 2048
+    // 13.8 -> 14.3 us).  No form needs both:
+    union {
+        float keep[2];       // kConv 4: how L2 treats A and the output (see l2_policy)
+        int group_flags[2];  // kConv 3: all groups read one A; the kernel before is the other half of the groups, whose results nothing here reads
+    };
 };
 
 namespace {
@@ -135,7 +138,8 @@ struct RingPos {
 // kEpi: the output epilogue adds a bias row and applies the activation (see ChainParams).
 // kConv: 0 = plain, 1 = convolution, 2 = convolution whose C is not a multiple of 64: tmB1 is then 3-D, [taps][C][r],
 // zero-filled past a tap's channels (the 3-D map costs 10 % of the pace, so the others stay 2-D); 3 = plain products of
-// several groups, blockIdx.z = group = outermost coordinate of every map.
+// several groups, blockIdx.z = group = outermost coordinate of every map; 4 = plain with hints to L2 (compiled into
+// the kernels that need none: the same forward 14.6 us instead of 14.3; 5000 x 768 -> 96 -> 3072 16.3 instead of 16.1).
 template <bool kMulti, bool kEpi, int kConv>
 __global__ void __launch_bounds__(kChainThreads, 1)
 tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB1,
@@ -149,9 +153,9 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t ring = t_smem + static_cast<uint32_t>(p.r_pad) * 256u;
     volatile uint32_t* abort_flag = &ctl->abort;
 
-    constexpr bool kIm = kConv == 1 || kConv == 2, kGroups = kConv == 3;
+    constexpr bool kIm = kConv == 1 || kConv == 2, kGroups = kConv == 3, kHints = kConv == 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int group = kGroups ? static_cast<int>(blockIdx.z) : 0, group_a = kGroups && !p.a_shared ? group : 0;
+    const int group = kGroups ? static_cast<int>(blockIdx.z) : 0, group_a = kGroups && !p.group_flags[0] ? group : 0;
     const int tile0 = blockIdx.x, tile_step = gridDim.x;
     const int nt_total = (p.N2 + 127) / 128;
     const int t_beg = blockIdx.y * p.tiles_per_split;
@@ -204,11 +208,11 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 }
         }
     }
-    const uint64_t a_policy = kConv == 0 ? l2_policy(p.keep_a) : 0, out_policy = kConv == 0 ? l2_policy(p.keep_out) : 0;
+    const uint64_t a_policy = kHints ? l2_policy(p.keep[0]) : 0, out_policy = kHints ? l2_policy(p.keep[1]) : 0;
     // (The second half of the groups runs beside the first: when it starts, everything older than that is complete, since
     // every kernel of this library lets its successor start only after its own wait.  It waits before it ends, so that
     // whoever waits for it has waited for both.)
-    if (!kGroups || !p.late_wait) pdl_wait();                 // everything above overlapped the previous kernel's tail
+    if (!kGroups || !p.group_flags[1]) pdl_wait();                 // everything above overlapped the previous kernel's tail
     pdl_launch_dependents();
     const uint32_t tmem = ctl->tmem_base;
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
@@ -253,7 +257,8 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         const uint32_t full = full0 + 8 * rp.s;
                         mbar_expect_tx(full, txa);
                         if constexpr (kGroups) tma_load_3d(ring + rp.off, &tmA, full, kb * 64, m0, group_a);
-                        else tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0, a_policy);
+                        else if constexpr (kHints) tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0, a_policy);
+                        else tma_load_2d(ring + rp.off, &tmA, full, kb * 64, m0);
                         rp.advance(NS, S);
                     }
                 }
@@ -521,7 +526,8 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     if (r0 < p.M && q * 32 < p.rows_tile && n0 < p.N2) {
                         if constexpr (kIm) tma_store_3d(&tmOut, stg, n0, q * 32, crow);
                         else if constexpr (kGroups) tma_store_3d(&tmOut, stg, n0, r0, group);
-                        else tma_store_2d(&tmOut, stg, n0, r0, out_policy);
+                        else if constexpr (kHints) tma_store_2d(&tmOut, stg, n0, r0, out_policy);
+                        else tma_store_2d(&tmOut, stg, n0, r0);
                         tma_store_commit();
                         stored = true;
                     }
@@ -539,7 +545,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         __syncwarp();
         tmem_dealloc(tmem, 512);
     }
-    if (kGroups && p.late_wait) pdl_wait();
+    if (kGroups && p.group_flags[1]) pdl_wait();
 }
 
 }  // namespace
@@ -554,6 +560,10 @@ int chain_launch_pipe(dim3 grid, size_t smem, cudaStream_t stream, const CUtenso
 // Launch of the forms with a convolution as first product (pf_tc_chain_conv.cu); pipe = software-pipelined persistent.
 int chain_launch_conv(bool pipe, bool ragged, dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1,
                       const CUtensorMap& tb2, const CUtensorMap& to, const CUtensorMap& tt, const ChainParams& p);
+
+// Launch of the forms with hints to L2 (pf_tc_chain_l2.cu).
+int chain_launch_hints(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1, const CUtensorMap& tb2,
+                       const CUtensorMap& to, const CUtensorMap& tt, const ChainParams& p);
 
 // Launch of the grouped form (pf_tc_chain_group.cu).
 int chain_launch_groups(dim3 grid, size_t smem, cudaStream_t stream, const CUtensorMap& ta, const CUtensorMap& tb1, const CUtensorMap& tb2,
