@@ -108,7 +108,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     if (!ok) return PF_ERR_CUDA;
     ChainParams p;
     p.M = static_cast<int>(M); p.K1 = static_cast<int>(K1); p.N2 = static_cast<int>(N2);
-    p.r_pad = plan.r_pad; p.num_stages = plan.num_stages; p.stage_bytes = plan.stage_bytes;
+    p.r = static_cast<int>(r); p.r_pad = plan.r_pad; p.num_stages = plan.num_stages; p.stage_bytes = plan.stage_bytes;
     p.tiles_per_split = plan.tiles_per_split; p.store_T = T != nullptr;
     p.boxes_per_stage = plan.boxes_per_stage; p.staging_off = plan.staging_off;
     p.conv_cblks = 0; p.conv_kw = 1; p.conv_pad = 0; p.conv_stride = 1; p.conv_bh = 1; p.conv_nb = 1; p.conv_tpi = 1;
@@ -176,7 +176,7 @@ int chain_groups(int groups, int all, const void* A, int64_t lda, int64_t sA, in
     if (!ok) return PF_ERR_CUDA;
     ChainParams p = {};
     p.M = static_cast<int>(M); p.K1 = static_cast<int>(K1); p.N2 = static_cast<int>(N2);
-    p.r_pad = plan.r_pad; p.num_stages = plan.num_stages; p.stage_bytes = plan.stage_bytes;
+    p.r = static_cast<int>(r); p.r_pad = plan.r_pad; p.num_stages = plan.num_stages; p.stage_bytes = plan.stage_bytes;
     p.tiles_per_split = plan.tiles_per_split; p.store_T = T != nullptr;
     p.boxes_per_stage = plan.boxes_per_stage; p.staging_off = plan.staging_off;
     p.conv_kw = p.conv_stride = p.conv_bh = p.conv_nb = p.conv_tpi = p.conv_Ho = p.conv_N = 1;

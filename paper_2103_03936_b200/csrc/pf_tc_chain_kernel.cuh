@@ -39,7 +39,7 @@ namespace tc {
 
 struct ChainParams {
     int M, K1, N2;
-    int r_pad;              // r rounded up to a multiple of 64, <= 384
+    int r, r_pad;           // r_pad: r rounded up to a multiple of 64, <= 384
     int num_stages;
     int stage_bytes;        // 16384 + r_pad * 128
     int tiles_per_split;    // 128-column output tiles per blockIdx.y (0: phase 1 only)
@@ -452,6 +452,10 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 uint32_t v[32];
                 tmem_ld32(lane_base + c * 32, v);
                 tmem_ld_wait();
+                if (c * 32 + 32 > p.r) {          // no column of T: zero, also for a row of A that holds an infinity
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) v[e] = c * 32 + e < p.r ? v[e] : 0u;
+                }
                 const uint32_t panel = t_smem + (c >> 1) * kTileBytes + row * 128;
                 const uint32_t cb = (c & 1) * 4;
 #pragma unroll

@@ -440,6 +440,17 @@ def test_smallest_layers_infinite_factor_and_a_ragged_batch():
         assert (dU[:, 4] == m * n).all() and (dV == m).all()
 
 
+@pytest.mark.parametrize("m,r", [(300, 24), (300, 33), (20, 64)])
+def test_fused_forward_infinite_input_and_a_ragged_rank(m, r):
+    """An infinity in x makes its row of x U and of y infinite, whatever the rank is padded to."""
+    k, n = 512, 136
+    x, U, V = (torch.ones(s, device="cuda", dtype=torch.bfloat16) for s in ((m, k), (k, r), (n, r)))
+    x[7, 11] = float("inf")
+    y = pf.pf_lowrank_linear_fwd(x, U, V)
+    rest = torch.arange(m, device="cuda") != 7
+    assert torch.isposinf(y[7]).all() and (y[rest] == float(torch.tensor(k * r).bfloat16())).all()
+
+
 @pytest.mark.parametrize("m,k,n,r", [(2049, 136, 1032, 64), (3499, 136, 1032, 72), (3500, 136, 1032, 72), (2100, 1032, 1024, 40), (16300, 72, 264, 16), (12000, 72, 1032, 16)])
 def test_backward_schedules(m, k, n, r):
     """Either side of the sizes from which the backward's fused kernel is used, and from which dV runs beside it."""
