@@ -39,7 +39,7 @@ namespace tc {
 
 struct ChainParams {
     int M, K1, N2;
-    int r, r_pad;           // r_pad: r rounded up to a multiple of 64, <= 384
+    int r, r_pad;           // r_pad: r rounded up to a multiple of 64, <= 384; columns of T from r on are zeroed (r = r_pad: left as they come)
     int num_stages;
     int stage_bytes;        // 16384 + r_pad * 128
     int tiles_per_split;    // 128-column output tiles per blockIdx.y (0: phase 1 only)
@@ -452,14 +452,17 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 uint32_t v[32];
                 tmem_ld32(lane_base + c * 32, v);
                 tmem_ld_wait();
-                if (c * 32 + 32 > p.r) {          // no column of T: zero, also for a row of A that holds an infinity
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] = c * 32 + e < p.r ? v[e] : 0u;
-                }
                 const uint32_t panel = t_smem + (c >> 1) * kTileBytes + row * 128;
                 const uint32_t cb = (c & 1) * 4;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) st_shared_v4(panel + (((cb + t) ^ sw) << 4), pack8(v + 8 * t));
+                if (c * 32 + 32 > p.r) {          // what is no column of T: zero, also for a row of A that holds an infinity
+#pragma unroll 1
+                    for (int t = max(0, (p.r - c * 32 + 7) >> 3); t < 4; ++t) st_shared_v4(panel + (((cb + t) ^ sw) << 4), make_uint4(0u, 0u, 0u, 0u));
+#pragma unroll 1
+                    for (int e = p.r; (e & 7) != 0 && c * 32 < p.r; ++e)
+                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(panel + (((static_cast<uint32_t>(e >> 3) & 7u) ^ sw) << 4) + static_cast<uint32_t>(e & 7) * 2u), "h"(static_cast<unsigned short>(0)) : "memory");
+                }
             }
             tc_fence_before();
             fence_proxy_async_smem();
