@@ -32,11 +32,13 @@ def _headers():
     return [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))] + [os.path.join(ROOT, "include", "pf.h")]
 
 
-def _build_lib(force: bool, verbose: bool) -> None:
+def nvcc() -> str:
+    return os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+
+
+def objects(force: bool = False, verbose: bool = False) -> list:
+    """The library's objects, compiled where a source or header is newer."""
     sources = [os.path.join(CSRC, s) for s in SOURCES]
-    if not force and _mtime(LIB) > _newest(sources + _headers()):
-        return
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ, exist_ok=True)
     headers = _newest(_headers())
 
@@ -44,15 +46,20 @@ def _build_lib(force: bool, verbose: bool) -> None:
         obj = os.path.join(OBJ, os.path.basename(src)[:-3] + ".o")
         if force or _mtime(obj) <= max(headers, os.path.getmtime(src)):
             tmp = obj + f".tmp{os.getpid()}.o"
-            subprocess.check_call([nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
+            subprocess.check_call([nvcc()] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) +
                                   ["-I", os.path.join(ROOT, "include"), "-I", CSRC, "-c", "-o", tmp, src])
             os.replace(tmp, obj)
         return obj
 
     with ThreadPoolExecutor(max_workers=min(len(sources), os.cpu_count() or 1)) as pool:
-        objects = list(pool.map(compile_one, sources))
+        return list(pool.map(compile_one, sources))
+
+
+def _build_lib(force: bool, verbose: bool) -> None:
+    if not force and _mtime(LIB) > _newest([os.path.join(CSRC, s) for s in SOURCES] + _headers()):
+        return
     tmp = LIB + f".tmp{os.getpid()}"
-    subprocess.check_call([nvcc] + NVCC_FLAGS + ["-shared", "-o", tmp] + objects)
+    subprocess.check_call([nvcc()] + NVCC_FLAGS + ["-shared", "-o", tmp] + objects(force, verbose))
     os.replace(tmp, LIB)
 
 
@@ -74,7 +81,7 @@ def _build_native(force: bool) -> None:
     if not force and built_for == key and _mtime(NATIVE) > _newest([src, os.path.join(ROOT, "include", "pf.h")]):
         return
     torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
-    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    cuda = os.path.dirname(os.path.dirname(nvcc()))
     tmp = NATIVE + f".tmp{os.getpid()}"
     includes = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
                 os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]

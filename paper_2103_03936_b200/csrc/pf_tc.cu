@@ -92,6 +92,11 @@ size_t slice_bytes(int64_t M, int64_t N, int splits) {
     return static_cast<size_t>(ceil_div(M, kBM) * ceil_div(N, bn)) * std::max(1, splits) * kBM * bn * 4;
 }
 size_t partial_bytes(int64_t M, int64_t N, int splits) { return splits <= 1 ? 0 : slice_bytes(M, N, splits); }      // a split product
+// Where a product may leave its slices, and how many bytes it may use there.
+struct SliceRoom {
+    float* p = nullptr;
+    size_t bytes = 0;
+};
 
 // What a block that is alone on its SM spends on kb k-blocks of a contraction cut into s slices, beyond its start and
 // end: 0.16 us per k-block on warm caches, 0.3 on cold ones, and for the sum of the slices 5 us at two slices, 4.2 at
@@ -155,7 +160,11 @@ void pick_pair_splits(int64_t Mu, int64_t Mv, int64_t N, int64_t nkb_u, int64_t 
 // 20 SMs the split fused kernel leaves idle are free, loses more through the long dV blocks than the
 // overlap gains.)
 void bwd_split_plan(int64_t m, int64_t k, int64_t n, int64_t r, bool fused_dx, int* su, int* sv, bool* beside) {
-    if (!fused_dx) {        // each shares a launch with a product that waits for nothing (see linear_bwd)
+    // Unfused, each shares a launch with a product that waits for nothing (see linear_bwd), so each may fill the machine by
+    // itself, also where the tiles of both do not fit it together.  Backward with both whole there / split: 8192 x 1504 -> 376 ->
+    // 6016: 161 / 146 us, 8192 x 768 -> 768 -> 3072: 106 / 86, 11209 x 3072 -> 768 -> 768: 139 / 114, 4096 x 1024 -> 1024 -> 4096:
+    // 75.5 / 74.1.
+    if (!fused_dx) {
         *su = pick_splits(k, r, pick_bn(r), m);
         *sv = pick_splits(n, r, pick_bn(r), m);
         *beside = false;
@@ -203,9 +212,15 @@ struct GemmLaunch {
     bool runs = false;       // several tiles per block (plain product, K-major A and MN-major B)
 };
 
-// Encodes the tensor maps and launch geometry of C[M,N] = A * B without launching.
+// Bytes of the slices of a prepared product.
+size_t slices_of_launch(const GemmParams& p) {
+    return static_cast<size_t>(p.tiles_x) * p.tiles_y * std::max(1, p.groups) * std::max(1, p.splits) * kBM * p.bn * 4;
+}
+
+// Encodes the tensor maps and launch geometry of C[M,N] = A * B without launching.  A contraction whose slices do not fit `room`
+// is refused.
 int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
-                 int splits, float* partial, const ConvA* cv, GemmLaunch* out, const Grouping* gr = nullptr) {
+                 int splits, SliceRoom room, const ConvA* cv, GemmLaunch* out, const Grouping* gr = nullptr) {
     if (M > 0x7fffffff || N > 0x7fffffff || K > 0x7fffffff) return PF_ERR_UNSUPPORTED;
     const int groups = gr ? gr->groups : 1;
     const bool sum_groups = gr && gr->sum_groups;
@@ -288,13 +303,13 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     if (dx) grid = dim3(run_blocks(static_cast<int64_t>(p.tiles_x) * p.tiles_y, nkb / (cv->stride * cv->stride), cv->stride));
     p.num_stages = pick_stages(bn, static_cast<int64_t>(grid.x) * grid.y * grid.z, dx);
     p.counters = nullptr;
-    p.partial = p.splits > 1 ? partial : nullptr;
+    p.partial = p.splits > 1 ? room.p : nullptr;
     p.independent = 0;
     p.keep_a = 0.f;
     if (p.splits > 1) {
         // the CTAs of a tile wait for one another, so all of them must be resident at once
         if (static_cast<int64_t>(grid.x) * grid.y * out_groups > kFixTiles || static_cast<int64_t>(grid.x) * grid.y * grid.z > num_sms() ||
-            partial == nullptr)
+            room.p == nullptr || slices_of_launch(p) > room.bytes)
             return PF_ERR_UNSUPPORTED;
         p.counters = split_counters();
         if (!p.counters) return PF_ERR_CUDA;
@@ -456,19 +471,19 @@ int launch_with(const GemmLaunch* const* g, const PairJob* first, int count, cud
     return launch_singles(g, count, stream);
 }
 
-// Prepares a product, unsplit where its slices do not fit the counters or the machine.
-int gemm_prepare_any(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc, int splits, float* partial,
+// Prepares a product, unsplit where its slices do not fit their room, the counters or the machine.
+int gemm_prepare_any(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc, int splits, SliceRoom room,
                      const ConvA* cv, GemmLaunch* out) {
-    const int st = gemm_prepare(A, B, M, N, K, C, ldc, splits, partial, cv, out);
-    return st == PF_ERR_UNSUPPORTED && splits > 1 ? gemm_prepare(A, B, M, N, K, C, ldc, 1, nullptr, cv, out) : st;
+    const int st = gemm_prepare(A, B, M, N, K, C, ldc, splits, room, cv, out);
+    return st == PF_ERR_UNSUPPORTED && splits > 1 ? gemm_prepare(A, B, M, N, K, C, ldc, 1, {}, cv, out) : st;
 }
 // One product in a launch of its own.  `copy2` (optional): asks for a second copy of C at pitch ldc2; *copy2_done tells
 // whether the launch wrote it (the CTA-pair kernel cannot), else the caller copies C itself.
 int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
-         int splits, float* partial, cudaStream_t stream, void* copy2 = nullptr, int64_t ldc2 = 0, bool* copy2_done = nullptr,
+         int splits, SliceRoom room, cudaStream_t stream, void* copy2 = nullptr, int64_t ldc2 = 0, bool* copy2_done = nullptr,
          const void* bias = nullptr, int act = 0) {
     GemmLaunch g;
-    const int st = gemm_prepare_any(A, B, M, N, K, C, ldc, splits, partial, nullptr, &g);
+    const int st = gemm_prepare_any(A, B, M, N, K, C, ldc, splits, room, nullptr, &g);
     if (st != PF_OK) return st;
     if (copy2) {
         g.p.C2 = copy2; g.p.ldc2 = ldc2;
@@ -553,25 +568,30 @@ size_t repack_room(int64_t rows, int64_t cols, bool tight = false) {
 bool narrow_reductions(int64_t rows_u, int64_t rows_v, int64_t r) {
     return (ceil_div(rows_u, kBM) + ceil_div(rows_v, kBM)) * ceil_div(r, pick_bn(r)) <= num_sms();
 }
-// Room for the fp32 slices of dU and dV under either backward structure (which one a call takes
-// depends on pointers the workspace query does not see): no block count exceeds one per SM per product.
+// Room for the fp32 slices of dU and dV under either backward structure (which one a call takes depends on pointers the
+// workspace query does not see).  Reductions that do not fit the machine together may each be split by themselves (they
+// share their launches with other products); only narrow ones leave one slice.
 void bwd_partial_bytes(int64_t m, int64_t k, int64_t n, int64_t r, size_t* bytes_u, size_t* bytes_v) {
-    *bytes_u = *bytes_v = 0;
-    if (!narrow_reductions(k, n, r)) return;        // (never split)
     int su, sv, su2, sv2;
     bool beside;
     bwd_split_plan(m, k, n, r, false, &su, &sv, &beside);
     bwd_split_plan(m, k, n, r, true, &su2, &sv2, &beside);
-    *bytes_u = align_up(slice_bytes(k, r, std::max(su, su2)), 256);
-    *bytes_v = align_up(slice_bytes(n, r, std::max(sv, sv2)), 256);
+    const auto bytes = narrow_reductions(k, n, r) ? slice_bytes : partial_bytes;
+    *bytes_u = align_up(bytes(k, r, std::max(su, su2)), 256);
+    *bytes_v = align_up(bytes(n, r, std::max(sv, sv2)), 256);
+}
+// ... and for those of the m x r products (x U and, backward, dY V), one after the other.
+size_t first_partial_bytes(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd) {
+    const int s = std::max(pick_splits(m, r, pick_bn(r), k), bwd ? pick_splits(m, r, pick_bn(r), n) : 1);
+    return align_up(partial_bytes(m, r, s), 256);
 }
 // Where a prepared reduction leaves its fp32 slices; an unsplit one is told to leave its one slice.
-void keep_slices(LinearArgs::Slices* out, GemmLaunch* g, float* room, int conv_c = 0) {
+void keep_slices(LinearArgs::Slices* out, GemmLaunch* g, SliceRoom room, int conv_c = 0) {
     if (!out) return;
     *out = LinearArgs::Slices();
-    if (!room) return;
-    g->p.partial = room;
-    out->partial = room; out->splits = g->p.splits; out->bn = g->bn;
+    if (!room.p || slices_of_launch(g->p) > room.bytes) return;
+    g->p.partial = room.p;
+    out->partial = room.p; out->splits = g->p.splits; out->bn = g->bn;
     out->tiles_x = static_cast<int>(g->grid.x); out->tiles_y = static_cast<int>(g->grid.y); out->conv_c = conv_c;
 }
 
@@ -608,9 +628,7 @@ size_t linear_extra_workspace(int64_t m, int64_t k, int64_t n, int64_t r, bool b
         b += bu + bv;
     }
     // skinny batches: the m x r products (x U, dY V) are split over their contraction to fill the SMs
-    const int s1 = std::max(pick_splits(m, r, pick_bn(r), k), bwd ? pick_splits(m, r, pick_bn(r), n) : 1);
-    b += align_up(partial_bytes(m, r, s1), 256);
-    return b;
+    return b + first_partial_bytes(m, k, n, r, bwd);
 }
 
 // Bytes of `a.ws` that linear_fwd(a) will really touch for these pointers and sizes (it takes the
@@ -634,7 +652,7 @@ size_t linear_fwd_need(const LinearArgs& a, bool* handles) {
     ChainPlan plan;
     if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan))
         return room + ((a.T && !stash_direct) ? t_bytes : 0);
-    return room + t_bytes + align_up(partial_bytes(a.m, a.r, pick_splits(a.m, a.r, pick_bn(a.r), a.k)), 256);
+    return room + t_bytes + first_partial_bytes(a.m, a.k, a.n, a.r, false);
 }
 
 // Whether a forward of few rows runs on the fused kernel, which takes its operands as they are, instead of pf_small.cu.
@@ -669,12 +687,13 @@ int linear_fwd(const LinearArgs& a, int* handled) {
         st = chain(x.p, x.ld, a.m, a.k, U.p, U.ld, a.r, V.p, V.ld, a.n, a.y, a.ldy, a.T ? T : nullptr, ldT,
                    a.stream, nullptr, 0, a.bias, a.act, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f);
     } else {
-        float* p1 = reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * row_pitch(a.r, a.tight) * 2, 256));
+        const SliceRoom p1{reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * row_pitch(a.r, a.tight) * 2, 256)),
+                           first_partial_bytes(a.m, a.k, a.n, a.r, false)};
         st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, T, ldT,
                   pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream,
                   (a.T && !stash_direct) ? a.T : nullptr, a.ldt, &stash_written);
         if (st != PF_OK) return st;
-        st = gemm({T, ldT, false}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, a.stream, nullptr, 0, nullptr,
+        st = gemm({T, ldT, false}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, a.stream, nullptr, 0, nullptr,
                   a.bias, a.act);
     }
     if (st != PF_OK) return st;
@@ -726,11 +745,12 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     bool dv_beside;
     bwd_split_plan(a.m, a.k, a.n, a.r, fused_dx, &su, &sv, &dv_beside);
     bwd_partial_bytes(a.m, a.k, a.n, a.r, &pu_bytes, &pv_bytes);
-    float* pu = reinterpret_cast<float*>(scratch);
+    const SliceRoom pu{reinterpret_cast<float*>(scratch), pu_bytes};
     scratch += pu_bytes;
-    float* pv = reinterpret_cast<float*>(scratch);
+    const SliceRoom pv{reinterpret_cast<float*>(scratch), pv_bytes};
     scratch += pv_bytes;
-    float* p1 = reinterpret_cast<float*>(scratch);
+    const SliceRoom p1{reinterpret_cast<float*>(scratch), first_partial_bytes(a.m, a.k, a.n, a.r, true)};
+    const bool narrow = narrow_reductions(a.k, a.n, a.r);
     // G = dY V ; dX = G U^T ; dU = x^T G ; dV = dY^T T
     if (need_T) {   // no stash: recompute T = x U
         st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, Tbuf, row_pitch(a.r),
@@ -759,7 +779,7 @@ int linear_bwd(const LinearArgs& a, int* handled) {
         st = gemm_prepare_any({dY.p, dY.ld, false}, {V.p, V.ld, true}, a.m, a.r, a.n, G, ldG, sg, p1, nullptr, &gg);
         if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
         if (st == PF_OK) st = gemm_prepare_any({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
-        if (st == PF_OK && a.dX) st = gemm_prepare({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gx);
+        if (st == PF_OK && a.dX) st = gemm_prepare({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gx);
         if (st != PF_OK) return st;
         const PairJob j1[2] = {{dY.p, dY.ld, false, 0, V.p, V.ld, true, 0, a.m, a.r, a.n, G, ldG},
                                {dY.p, dY.ld, true, 0, T.p, T.ld, true, 0, a.n, a.r, a.m, a.dV, a.lddv}};
@@ -767,7 +787,7 @@ int linear_bwd(const LinearArgs& a, int* handled) {
                                {x.p, x.ld, true, 0, G, ldG, true, 0, a.k, a.r, a.m, a.dU, a.lddu}};
         const GemmLaunch* const l1[2] = {&gg, &gv};
         const GemmLaunch* const l2[2] = {&gx, &gu};
-        if (!narrow_reductions(a.k, a.n, a.r)) {
+        if (!narrow) {
             st = launch_faster(l1, j1, 2, a.stream);
             if (st != PF_OK) return st;
             return a.dX ? launch_faster(l2, j2, 2, a.stream) : launch_faster(l2 + 1, j2 + 1, 1, a.stream);
@@ -783,8 +803,8 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     st = gemm_prepare_any({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
     if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
     if (st != PF_OK) return st;
-    keep_slices(a.du_slices, &gu, pu_bytes ? pu : nullptr);
-    keep_slices(a.dv_slices, &gv, pv_bytes ? pv : nullptr);
+    keep_slices(a.du_slices, &gu, narrow ? pu : SliceRoom());
+    keep_slices(a.dv_slices, &gv, narrow ? pv : SliceRoom());
     // dY and x are read for the last time: they make room.  In a step that streams more than L2 holds a fifth of dY is kept for
     // this launch, and everything else passes through: 16384 x 4096 -> 64 -> 4096: 161 -> 149 us, 8192 x 4096 -> 64 -> 4096: 101 -> 88,
     // 16384 x 2048 -> 64 -> 2048: 91 -> 81.  The last reads alone: 8192 x 512 -> 128 -> 2048: 42.3 -> 40.7, 12000 x 2048 -> 96 -> 2048:
@@ -870,7 +890,7 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     const bool shared_x = a.sx == 0 && a.groups > 1;
     char* ws = a.ws;
     char* Tbuf = ws; ws += gp.t_bytes;
-    float* p1 = reinterpret_cast<float*>(ws); ws += gp.p1_bytes;
+    const SliceRoom p1{reinterpret_cast<float*>(ws), gp.p1_bytes}; ws += gp.p1_bytes;
     StagedGroups x, U, V;
     RepackList repacks;
     if (stage_groups(a.x, a.ldx, a.sx, a.groups, shared_x, a.m, a.k, ws, &x, &repacks) ||
@@ -905,7 +925,7 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     const Grouping gt{a.groups, sT, false}, gy{a.groups, a.sy, false};
     int st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, T, ldT, gp.s1, p1, nullptr, &g1, &gt);
     if (st == PF_OK)
-        st = gemm_prepare({T, ldT, false, sT}, {V.p, V.ld, false, V.gs}, a.m, a.n, a.r, a.y, a.ldy, 1, nullptr, nullptr, &g2, &gy);
+        st = gemm_prepare({T, ldT, false, sT}, {V.p, V.ld, false, V.gs}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, nullptr, &g2, &gy);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
     if (a.T && !stash_direct) {
@@ -928,10 +948,10 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     const bool shared_x = a.sx == 0 && a.groups > 1;
     char* ws = a.ws;
     void* Tbuf = ws; ws += gp.t_bytes;
-    float* p1 = reinterpret_cast<float*>(ws); ws += gp.p1_bytes;
+    const SliceRoom p1{reinterpret_cast<float*>(ws), gp.p1_bytes}; ws += gp.p1_bytes;
     void* Gbuf = ws; ws += gp.t_bytes;
-    float* pu = reinterpret_cast<float*>(ws); ws += gp.pu_bytes;
-    float* pv = reinterpret_cast<float*>(ws); ws += gp.pv_bytes;
+    const SliceRoom pu{reinterpret_cast<float*>(ws), gp.pu_bytes}; ws += gp.pu_bytes;
+    const SliceRoom pv{reinterpret_cast<float*>(ws), gp.pv_bytes}; ws += gp.pv_bytes;
     const int64_t ldW = row_pitch(a.r), sW = a.m * row_pitch(a.r);
     StagedGroups x, U, V, dY, T{Tbuf, ldW, sW};
     RepackList repacks;
@@ -964,7 +984,7 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, true, dY.gs}, {T.p, T.ld, true, T.gs}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gV, &gdv);
     if (st == PF_OK) st = gemm_prepare({x.p, x.ld, true, x.gs}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gU, &gdu);
     if (st == PF_OK && a.dX)
-        st = gemm_prepare({Gbuf, ldW, false, sW}, {U.p, U.ld, false, U.gs}, a.m, a.k, a.r, a.dX, a.lddx, 1, nullptr, nullptr, &gX, &gdx);
+        st = gemm_prepare({Gbuf, ldW, false, sW}, {U.p, U.ld, false, U.gs}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gX, &gdx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
     *handled = 1;
@@ -1073,15 +1093,14 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     conv_splits(cu, a.O, &su, &sv);
     size_t bu, bv;
     conv_partial_bytes(cu, a.O, su, sv, &bu, &bv);
-    float* pu = reinterpret_cast<float*>(a.ws);
-    float* pv = reinterpret_cast<float*>(a.ws + bu);
+    const SliceRoom pu{reinterpret_cast<float*>(a.ws), bu}, pv{reinterpret_cast<float*>(a.ws + bu), bv};
     GemmLaunch gt, gu, gv, gx;
-    st = gemm_prepare_any({a.dY, a.O, false}, {a.V, a.R, true}, P, a.R, a.O, dT, a.R, 1, nullptr, nullptr, &gt);
+    st = gemm_prepare_any({a.dY, a.O, false}, {a.V, a.R, true}, P, a.R, a.O, dT, a.R, 1, {}, nullptr, &gt);
     if (st == PF_OK) st = gemm_prepare_any({a.x, a.C, true}, {dT, a.R, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
     if (st == PF_OK) st = gemm_prepare_any({a.dY, a.O, true}, {T, a.R, true}, a.O, a.R, P, a.dV, a.R, sv, pv, nullptr, &gv);
     if (st == PF_OK && a.dX)
         st = gemm_prepare_any({dT, a.R, false}, {a.U, a.R, false}, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
-                     static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1, nullptr, &cx, &gx);
+                     static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1, {}, &cx, &gx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     if (st != PF_OK) return st;
     // dT: more tiles than two per SM, of few k-blocks each, go up to four to a block
@@ -1099,8 +1118,8 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     }
     *handled = 1;
     const bool narrow = narrow_reductions(conv_du_tiles(a.kh, a.kw, a.C) * kBM, a.O, a.R);
-    keep_slices(a.du_slices, &gu, narrow ? pu : nullptr, a.C);
-    keep_slices(a.dv_slices, &gv, narrow ? pv : nullptr);
+    keep_slices(a.du_slices, &gu, narrow ? pu : SliceRoom(), a.C);
+    keep_slices(a.dv_slices, &gv, narrow ? pv : SliceRoom());
     // dT = dY V  (per pixel)
     st = launch_prepared(gt, a.stream);
     if (st != PF_OK) return st;

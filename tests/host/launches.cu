@@ -1,0 +1,122 @@
+// What a call of the library launches, looked over on the host (see runtime.cpp): every tensor map that is encoded and every
+// matrix and slice buffer that a launched kernel is given has to lie inside one of the buffers of the call (host_regions)
+// or inside a device array of the library; what does not is reported by host_faults.
+#include <cuda.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <map>
+#include <string>
+#include <vector>
+
+#include "pf_tc.h"
+#include "pf_tc_f32_kernel.cuh"
+#include "pf_tc_gemm_kernel.cuh"
+
+namespace {
+struct Range {
+    uint64_t base, bytes;
+};
+std::vector<Range> regions, written;      // `written`: what the products of the launch in hand write
+std::map<const void*, std::string>& kernels() { static std::map<const void*, std::string> m; return m; }
+std::map<const void*, Range>& arrays() { static std::map<const void*, Range> m; return m; }      // by host symbol
+std::string faults, launches;
+
+uint64_t address(const void* p) { return reinterpret_cast<uint64_t>(p); }
+// [base, base + bytes) has to lie inside one buffer.
+void inside(const std::string& what, uint64_t base, uint64_t bytes) {
+    auto holds = [&](const Range& r) { return base >= r.base && base + bytes <= r.base + r.bytes; };
+    if (bytes == 0 || std::any_of(regions.begin(), regions.end(), holds)) return;
+    for (const auto& a : arrays())
+        if (holds(a.second)) return;
+    uint64_t past = 0;
+    for (const Range& r : regions)
+        if (base >= r.base && base <= r.base + r.bytes) past = base + bytes - (r.base + r.bytes);
+    faults += what + ": " + std::to_string(bytes) + " bytes, " + (past ? std::to_string(past) + " of them past the end of their buffer\n" : "in no buffer\n");
+}
+// ... and what the products of one launch write there may not overlap.
+void writes(const std::string& what, uint64_t base, uint64_t bytes) {
+    inside(what, base, bytes);
+    for (const Range& w : written)
+        if (base < w.base + w.bytes && w.base < base + bytes) faults += what + ": overlaps what another product of the launch writes\n";
+    written.push_back(Range{base, bytes});
+}
+uint64_t matrix(int64_t rows, int64_t cols, int64_t ld, int64_t size) { return rows > 0 ? static_cast<uint64_t>(((rows - 1) * ld + cols) * size) : 0; }
+
+void check(const pf::tc::GemmParams& p) {
+    const int splits = p.splits < 1 ? 1 : p.splits, groups = p.groups < 1 ? 1 : p.groups;
+    if (p.partial) writes("slices of a product", address(p.partial), static_cast<uint64_t>(p.tiles_x) * p.tiles_y * groups * splits * 128 * p.bn * 4);
+    if (splits > 1 && !p.partial) faults += "a split product without slices\n";
+    if (p.partial && splits == 1) return;
+    for (int g = 0; g < groups; ++g) {
+        if (p.conv_mode != 1) writes("result of a product", address(p.C) + static_cast<uint64_t>(g) * p.c_gstride * 2, matrix(p.M, p.N, p.ldc, 2));
+        if (p.C2) writes("second copy of a result", address(p.C2) + static_cast<uint64_t>(g) * p.c2_gstride * 2, matrix(p.M, p.N, p.ldc2, 2));
+    }
+}
+void check(const pf::tc::F32Params& p) {
+    if (p.splits > 1) writes("slices of an fp32 product", address(p.partial), static_cast<uint64_t>(p.tiles_x) * p.tiles_y * p.splits * 128 * p.bn * 4);
+    if (p.mode == 0 || p.mode == 2) writes("result of an fp32 product", address(p.C), matrix(p.M, p.N, p.ldc, 4));
+    if (p.C2) writes("second copy of an fp32 result", address(p.C2), matrix(p.M, p.N, p.ldc2, 4));
+}
+void check(const pf::SimtGemm& g) {
+    const int64_t size = g.dtype == PF_BF16 ? 2 : 4;
+    if (g.splits > 1) inside("slices of an FMA product", address(g.partial), static_cast<uint64_t>(g.splits) * g.M * g.N * 4);
+    inside("result of an FMA product", address(g.C), matrix(g.M, g.N, g.ldc, size));
+}
+
+template <typename T>
+const T& arg(void** args, int i) { return *static_cast<const T*>(args[i]); }
+void launched(const void* kernel, unsigned blocks, void** args) {
+    const std::string& name = kernels()[kernel];
+    auto is = [&](const char* n) { return name.find(n) != std::string::npos; };
+    launches += name + "\n";
+    written.clear();
+    if (is("tc_gemm3_kernel")) {
+        const int end0 = arg<int>(args, 9), end1 = arg<int>(args, 10);
+        check(arg<pf::tc::GemmParams>(args, 6));
+        if (end1 > end0) check(arg<pf::tc::GemmParams>(args, 7));
+        if (static_cast<int>(blocks) > end1) check(arg<pf::tc::GemmParams>(args, 8));
+    } else if (is("tc_gemm_kernel")) {
+        check(arg<pf::tc::GemmParams>(args, 2));
+    } else if (is("tc_f32_kernel")) {
+        const pf::tc::F32Launch& l = arg<pf::tc::F32Launch>(args, 0);
+        for (int i = 0; i < 3; ++i)
+            if (i == 0 || l.end[i] > l.end[i - 1]) check(l.p[i]);
+    } else if (is("simt_gemm_kernel")) {
+        check(arg<pf::SimtGemm>(args, 0));
+    }
+}
+
+CUresult encode(CUtensorMap* map, CUtensorMapDataType type, cuuint32_t rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
+    const uint64_t size = type == CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 ? 2 : 4;
+    uint64_t bytes = dims[0] * size;
+    for (cuuint32_t i = 1; i < rank; ++i) bytes += (dims[i] - 1) * strides[i - 1];
+    inside("tensor map", address(base), bytes);
+    *map = CUtensorMap();
+    return CUDA_SUCCESS;
+}
+}  // namespace
+
+extern "C" {
+// The buffers of the calls that follow.  Maps are cached by address, so a call whose maps are to be seen has to use new ones.
+void host_regions(int count, const uint64_t* base, const uint64_t* bytes) {
+    regions.clear();
+    for (int i = 0; i < count; ++i) regions.push_back(Range{base[i], bytes[i]});
+    faults.clear();
+    launches.clear();
+}
+const char* host_faults() { return faults.c_str(); }
+const char* host_launches() { return launches.c_str(); }
+
+// For runtime.cpp:
+void host_kernel(const void* host, const char* name) { kernels()[host] = name; }
+void host_array(const void* host, size_t bytes) {
+    static uint64_t next = 1ull << 60;
+    arrays()[host] = Range{next, bytes};
+    next += (bytes + (1 << 20)) & ~static_cast<uint64_t>((1 << 20) - 1);
+}
+void* host_array_address(const void* host) { return arrays().count(host) ? reinterpret_cast<void*>(arrays()[host].base) : nullptr; }
+void host_launch(const void* kernel, unsigned blocks, void** args) { launched(kernel, blocks, args); }
+void* host_encode() { return reinterpret_cast<void*>(encode); }
+}
