@@ -3,10 +3,12 @@ import numpy as np
 import torch
 
 import oracle
+import paper_2103_03936_b200 as pf
 import pf_workloads as wl
 
 TOL = {wl.BF16: 1e-2, wl.F32: 1e-4}   # Frobenius-relative, per output tensor
 TDT = {wl.BF16: torch.bfloat16, wl.F32: torch.float32}
+PFDT = {wl.BF16: pf.PF_BF16, wl.F32: pf.PF_F32}
 GUARD = 64
 
 
@@ -39,6 +41,25 @@ class Guarded:
         if self.ld != self.cols:
             pad = b[GUARD:GUARD + self.rows * self.ld].view(self.rows, self.ld)[:, self.cols:]
             assert torch.all(pad == -7.0), "row padding overwritten"
+
+
+class Scratch:
+    """A workspace of exactly `need` bytes in front of a sentinel-filled guard, so that a call which uses more than its query
+    reports is detected.  Pass `t`."""
+    GUARD = 16 << 20
+
+    def __init__(self, need):
+        self.buf = torch.full((need + self.GUARD,), 0x5A, dtype=torch.uint8, device="cuda")
+        self.need = need
+        self.t = self.buf[:need]
+
+    def check(self):
+        assert bool((self.buf[self.need:] == 0x5A).all()), "written behind the end of the workspace"
+
+
+def linear_scratch(x, U, V, bwd):
+    dtype = pf.PF_F32 if x.dtype == torch.float32 else pf.PF_BF16
+    return Scratch(pf.pf_lowrank_linear_workspace(x.shape[0], x.shape[1], V.shape[0], U.shape[1], dtype, bwd))
 
 
 # Every (case, tensor) that took the cancellation rule below, in the order met.

@@ -6,7 +6,7 @@ import torch
 import oracle
 import paper_2103_03936_b200 as pf
 import pf_workloads as wl
-from _gpu import ESCAPES, Guarded, assert_blocks_close, assert_close, dev
+from _gpu import ESCAPES, PFDT, Guarded, Scratch, assert_blocks_close, assert_close, dev
 
 pytestmark = pytest.mark.gpu
 
@@ -18,12 +18,14 @@ def run_conv(case, stash=True, need_dX=True, tiny=False):
     Ho, Wo = case.Ho, case.Wo
     gy = Guarded((case.N, Ho, Wo, case.O), dt)
     gT = Guarded((case.N, Ho, Wo, case.R), dt)
+    scratch = [Scratch(pf.pf_lowrank_conv_workspace(case.N, case.H, case.W, case.C, case.R, case.O, case.kh, case.kw, case.stride, case.pad, PFDT[dt], bwd))
+               for bwd in (False, True)]
     pf.pf_lowrank_conv_fwd(x, U, V, stride=case.stride, pad=case.pad, y=gy.t,
-                           T_stash=gT.t if stash else None)
+                           T_stash=gT.t if stash else None, workspace=scratch[0].t)
     gdX, gdU, gdV = Guarded(x.shape, dt), Guarded(U.shape, dt), Guarded(V.shape, dt)
     pf.pf_lowrank_conv_bwd(x, U, V, dY, stride=case.stride, pad=case.pad,
                            T_stash=gT.t if stash else None, need_dX=need_dX,
-                           dX=gdX.t if need_dX else None, dU=gdU.t, dV=gdV.t)
+                           dX=gdX.t if need_dX else None, dU=gdU.t, dV=gdV.t, workspace=scratch[1].t)
     torch.cuda.synchronize()
     y_ref, T_ref = oracle.conv_fwd(d["x"], d["U"], d["V"], case.stride, case.pad)
     dX_ref, dU_ref, dV_ref = oracle.conv_bwd(d["x"], d["U"], d["V"], d["dY"], case.stride, case.pad)
@@ -40,7 +42,7 @@ def run_conv(case, stash=True, need_dX=True, tiny=False):
         checks.append(("dX", gdX, dX_ref))
     checks += [("dU", gdU, dU_ref), ("dV", gdV, dV_ref)]
     errs = {nm: assert_close(g.t, ref, dt, tag + nm, abs_ref64=ab.get(nm)) for nm, g, ref in checks}
-    for g in (gy, gT, gdX, gdU, gdV):
+    for g in (gy, gT, gdX, gdU, gdV, *scratch):
         g.check()
     assert pf.pf_last_device_status() == 0
     return errs

@@ -7,7 +7,7 @@ import torch
 import oracle
 import paper_2103_03936_b200 as pf
 import pf_workloads as wl
-from _gpu import Guarded, TDT, assert_blocks_close, assert_close, dev
+from _gpu import PFDT, Guarded, Scratch, TDT, assert_blocks_close, assert_close, dev
 
 pytestmark = pytest.mark.gpu
 
@@ -44,14 +44,15 @@ def run_grouped(G, m, k, n, r, dtype, seed, shared_x, stash=True, need_dX=True, 
     else:
         gT = Guarded((G, m, r), dtype)
         T_t = gT.t
+    scratch = [Scratch(pf.pf_lowrank_linear_grouped_workspace(G, m, k, n, r, PFDT[dtype], bwd)) for bwd in (False, True)]
     before = pf.pf_launch_count()
-    pf.pf_lowrank_linear_grouped_fwd(x, U, V, y=gy.t, T_stash=T_t if stash else None)
+    pf.pf_lowrank_linear_grouped_fwd(x, U, V, y=gy.t, T_stash=T_t if stash else None, workspace=scratch[0].t)
     launches_fwd = pf.pf_launch_count() - before
     gdX = Guarded((m, k) if shared_x else (G, m, k), dtype)
     gdU, gdV = Guarded((G, k, r), dtype), Guarded((G, n, r), dtype)
     before = pf.pf_launch_count()
     pf.pf_lowrank_linear_grouped_bwd(x, U, V, dY, T_stash=T_t if stash else None, need_dX=need_dX,
-                                     dX=gdX.t if need_dX else None, dU=gdU.t, dV=gdV.t)
+                                     dX=gdX.t if need_dX else None, dU=gdU.t, dV=gdV.t, workspace=scratch[1].t)
     launches_bwd = pf.pf_launch_count() - before
     torch.cuda.synchronize()
     y_ref, T_ref = oracle.linear_grouped_fwd(x_h, U_h, V_h)
@@ -74,7 +75,7 @@ def run_grouped(G, m, k, n, r, dtype, seed, shared_x, stash=True, need_dX=True, 
             assert_close(got, ref, dtype, tag + nm)
             if blocks:
                 assert_blocks_close(got, ref, dtype, tag + nm)
-    for g in (gy, gT, gdX, gdU, gdV):
+    for g in (gy, gT, gdX, gdU, gdV, *scratch):
         g.check()
     assert pf.pf_last_device_status() == 0
     return launches_fwd, launches_bwd

@@ -8,7 +8,7 @@ import torch
 import oracle
 import paper_2103_03936_b200 as pf
 import pf_workloads as wl
-from _gpu import ESCAPES, Guarded, assert_blocks_close, assert_close, dev, host
+from _gpu import ESCAPES, Guarded, assert_blocks_close, assert_close, dev, host, linear_scratch
 
 pytestmark = pytest.mark.gpu
 
@@ -28,14 +28,15 @@ def run_case(case, ld_pad=0, stash=True, need_dX=True, tiny=False, blocks=False)
     x, U, V, dY = up(d["x"], k), up(d["U"], r), up(d["V"], r), up(d["dY"], n)
     gy = Guarded((m, n), dt, ld=n + ld_pad if ld_pad else None)
     gT = Guarded((m, r), dt, ld=r + ld_pad if ld_pad else None)
-    out = pf.pf_lowrank_linear_fwd(x, U, V, y=gy.t, T_stash=gT.t if stash else None)
+    scratch = [linear_scratch(x, U, V, bwd) for bwd in (False, True)]
+    out = pf.pf_lowrank_linear_fwd(x, U, V, y=gy.t, T_stash=gT.t if stash else None, workspace=scratch[0].t)
     y_ref, T_ref = oracle.linear_fwd(d["x"], d["U"], d["V"])
     dX_ref, dU_ref, dV_ref = oracle.linear_bwd(d["x"], d["U"], d["V"], d["dY"])
     gdX = Guarded((m, k), dt, ld=k + ld_pad if ld_pad else None)
     gdU = Guarded((k, r), dt, ld=r + ld_pad if ld_pad else None)
     gdV = Guarded((n, r), dt, ld=r + ld_pad if ld_pad else None)
     pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=gT.t if stash else None, need_dX=need_dX,
-                             dX=gdX.t if need_dX else None, dU=gdU.t, dV=gdV.t)
+                             dX=gdX.t if need_dX else None, dU=gdU.t, dV=gdV.t, workspace=scratch[1].t)
     torch.cuda.synchronize()
     ab = {}
     if tiny:   # magnitude of the summands, for outputs of a handful of elements
@@ -54,7 +55,7 @@ def run_case(case, ld_pad=0, stash=True, need_dX=True, tiny=False, blocks=False)
         errs[nm] = assert_close(g.t, ref, dt, tag + nm, abs_ref64=ab.get(nm))
         if blocks:   # and no 128 x 128 block of the tensor may miss the same bound
             errs[nm + " worst block"] = assert_blocks_close(g.t, ref, dt, tag + nm)
-    for g in (gy, gT, gdX, gdU, gdV):
+    for g in (gy, gT, gdX, gdU, gdV, *scratch):
         g.check()
     assert pf.pf_last_device_status() == 0
     return errs
@@ -351,6 +352,13 @@ def test_whole_and_split_contractions_and_pairs(m, k, n, r):
     """Either side of the lengths from which contractions are split, and of the sizes from which products run on CTA
     pairs; dU and dV split by themselves beside a product that is whole."""
     run_case(wl.LinearCase("forms", m, k, n, r, wl.BF16, 72), blocks=True)
+
+
+@pytest.mark.parametrize("m,k,n,r", [(2048, 516, 2052, 1028), (2048, 2052, 516, 1028), (2100, 520, 3080, 520)])
+def test_reductions_that_do_not_fit_the_machine_together(m, k, n, r):
+    """The tiles of dU and dV are more than the SMs; each is split by itself, within the workspace that is asked for."""
+    run_case(wl.LinearCase("wide", m, k, n, r, wl.BF16, 78), blocks=True)
+    run_case(wl.LinearCase("wide", m, k, n, r, wl.BF16, 79), stash=False, need_dX=False)
 
 
 @pytest.mark.parametrize("m,k,n,r", [(1, 8, 8, 8), (5, 512, 136, 24), (32, 512, 1032, 192), (33, 1536, 264, 64), (129, 72, 4104, 136), (2047, 1536, 128, 16)])

@@ -6,7 +6,7 @@ import torch
 import oracle
 import paper_2103_03936_b200 as pf
 import pf_workloads as wl
-from _gpu import Guarded, assert_blocks_close, assert_close, dev
+from _gpu import Guarded, assert_blocks_close, assert_close, dev, linear_scratch
 
 pytestmark = pytest.mark.gpu
 
@@ -28,9 +28,10 @@ def run_act(case, bias=True, relu=True, stash=True, ld_pad=0):
     b = dev(b_host, dt) if bias else None
     gy = Guarded((m, n), dt, ld=n + ld_pad if ld_pad else None)
     gT = Guarded((m, r), dt, ld=r + ld_pad if ld_pad else None)
+    scratch = linear_scratch(x, U, V, False)
     l0 = pf.pf_launch_count()
     pf.pf_lowrank_linear_fwd_act(x, U, V, bias=b, act=pf.PF_ACT_RELU if relu else pf.PF_ACT_NONE, y=gy.t,
-                                 T_stash=gT.t if stash else None)
+                                 T_stash=gT.t if stash else None, workspace=scratch.t)
     launches = pf.pf_launch_count() - l0
     torch.cuda.synchronize()
     y_ref, T_ref = oracle.linear_fwd_act(d["x"], d["U"], d["V"], b_host, relu=relu)
@@ -44,8 +45,8 @@ def run_act(case, bias=True, relu=True, stash=True, ld_pad=0):
         assert float(gy.t.float().min()) >= 0.0
         # the activation really cut something, and kept something
         assert (y_ref == 0).mean() > 0.1 and (y_ref > 0).mean() > 0.1
-    gy.check()
-    gT.check()
+    for g in (gy, gT, scratch):
+        g.check()
     assert pf.pf_last_device_status() == 0
     return launches
 

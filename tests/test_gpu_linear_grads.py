@@ -7,7 +7,7 @@ import torch
 import oracle
 import paper_2103_03936_b200 as pf
 import pf_workloads as wl
-from _gpu import Guarded, assert_close, dev
+from _gpu import Guarded, assert_close, dev, linear_scratch
 
 pytestmark = pytest.mark.gpu
 
@@ -28,7 +28,8 @@ def run_f32(case, expect_native=None):
     dX0, dU0, dV0 = pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T)
     l1 = pf.pf_launch_count()
     gU, gV = Guarded((k, r), wl.F32), Guarded((n, r), wl.F32)
-    dX1, _, _ = pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T, dU=gU.t, dV=gV.t, grads_f32=True)
+    scratch = linear_scratch(x, U, V, True)
+    dX1, _, _ = pf.pf_lowrank_linear_bwd(x, U, V, dY, T_stash=T, dU=gU.t, dV=gV.t, grads_f32=True, workspace=scratch.t)
     l2 = pf.pf_launch_count()
     torch.cuda.synchronize()
     dX_ref, dU_ref, dV_ref = oracle.linear_bwd(d["x"], d["U"], d["V"], d["dY"])
@@ -38,8 +39,8 @@ def run_f32(case, expect_native=None):
     assert_close(gV.t, dV_ref, wl.F32, tag + "dV", tol=1e-2 if dt == wl.BF16 else 1e-4)
     assert torch.equal(gU.t.to(dU0.dtype), dU0) and torch.equal(gV.t.to(dV0.dtype), dV0)
     assert torch.equal(dX0, dX1)
-    gU.check()
-    gV.check()
+    for g in (gU, gV, scratch):
+        g.check()
     # unrounded sums carry more bits than bf16 holds; gradients that went through a bf16 copy do not
     native = bool((gU.t != gU.t.to(torch.bfloat16).float()).any()) and bool((gV.t != gV.t.to(torch.bfloat16).float()).any())
     if expect_native is not None:
