@@ -788,9 +788,12 @@ int linear_bwd(const LinearArgs& a, int* handled) {
         const GemmLaunch* const l1[2] = {&gg, &gv};
         const GemmLaunch* const l2[2] = {&gx, &gu};
         if (!narrow) {
-            st = launch_faster(l1, j1, 2, a.stream);
-            if (st != PF_OK) return st;
-            return a.dX ? launch_faster(l2, j2, 2, a.stream) : launch_faster(l2 + 1, j2 + 1, 1, a.stream);
+            bool pairs_v = false, pairs_u = false;
+            st = launch_faster(l1, j1, 2, a.stream, 0.0, &pairs_v);
+            if (st == PF_OK) st = a.dX ? launch_faster(l2, j2, 2, a.stream, 0.0, &pairs_u) : launch_faster(l2 + 1, j2 + 1, 1, a.stream, 0.0, &pairs_u);
+            keep_slices(a.du_slices, &gu, gu.p.splits > 1 && !pairs_u ? pu : SliceRoom());      // (split ones leave them anyway)
+            keep_slices(a.dv_slices, &gv, gv.p.splits > 1 && !pairs_v ? pv : SliceRoom());
+            return st;
         }
         keep_slices(a.du_slices, &gu, pu);
         keep_slices(a.dv_slices, &gv, pv);

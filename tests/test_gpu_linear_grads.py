@@ -51,6 +51,17 @@ def run_f32(case, expect_native=None):
     return native
 
 
+@pytest.mark.parametrize("m,k,n,r,split", [(2048, 516, 2052, 1028, "U"), (2048, 2052, 516, 1028, "V")])
+def test_one_split_reduction_of_two_that_do_not_fit_the_machine_together(m, k, n, r, split):
+    """The gradient whose reduction is split keeps its unrounded sums, also where the other one is whole."""
+    case = wl.LinearCase("wide", m, k, n, r, wl.BF16, 45)
+    run_f32(case)
+    _, (x, U, V, dY) = _inputs(case)
+    _, dU, dV = pf.pf_lowrank_linear_bwd(x, U, V, dY, grads_f32=True)
+    g = dU if split == "U" else dV
+    assert bool((g != g.to(torch.bfloat16).float()).any())
+
+
 def run_accumulate(case, f32, parts=3):
     """The batch cut into micro-batches whose gradients are accumulated: the result is the gradient of
     the whole batch (plain sums over rows), on top of what the matrices held before."""
