@@ -108,9 +108,9 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     if (!ok) return PF_ERR_CUDA;
     ChainParams p;
     p.M = static_cast<int>(M); p.K1 = static_cast<int>(K1); p.N2 = static_cast<int>(N2);
-    // Zeroing what pads T costs ragged ranks 0.1 us (2641 x 768 -> 80 -> 768: 10.25 -> 10.35).  It keeps an infinity in A one, as the
-    // unfused products do, which the callers of fewer rows would otherwise run on.
-    p.r = conv || M >= 2048 ? plan.r_pad : static_cast<int>(r);
+    // Zeros behind the rank for any number of rows, as the unfused products have them: 0.1 us where the rank is no multiple of
+    // 64 (2641 x 768 -> 80 -> 768: 9.9 -> 10.0; 9000 x 512 -> 100 -> 512: 12.2 -> 12.4; 19500 x 512 -> 96 -> 512, pipelined: 15.4 both).
+    p.r = conv ? plan.r_pad : static_cast<int>(r);
     p.r_pad = plan.r_pad; p.num_stages = plan.num_stages; p.stage_bytes = plan.stage_bytes;
     p.tiles_per_split = plan.tiles_per_split; p.store_T = T != nullptr;
     p.boxes_per_stage = plan.boxes_per_stage; p.staging_off = plan.staging_off;

@@ -133,6 +133,25 @@ struct RingPos {
     }
 };
 
+// Columns c * 32 .. c * 32 + 31 of a row of T that pad the rank become zero, also for a row of A that holds an infinity, whose
+// product with the zero columns of B1 is NaN.  Behind the stores of the row: selecting registers before them cost more.
+__device__ __forceinline__ void zero_padding(uint32_t panel, uint32_t cb, uint32_t sw, int c, int r) {
+    const int left = r - c * 32;          // columns of T among the 32
+    if (left >= 32) return;
+    int t = max(0, left) >> 3;
+    if (left > 0 && (left & 7) != 0) {    // the piece that the rank ends in
+        const uint32_t at = panel + (((cb + t) ^ sw) << 4);
+        uint4 v = ld_shared_v4(at);
+        const int e = left & 7;
+        auto keep = [&](int i) { return (i < e ? 0xffffu : 0u) | (i + 1 < e ? 0xffff0000u : 0u); };
+        v.x &= keep(0); v.y &= keep(2); v.z &= keep(4); v.w &= keep(6);
+        st_shared_v4(at, v);
+        ++t;
+    }
+#pragma unroll 1
+    for (; t < 4; ++t) st_shared_v4(panel + (((cb + t) ^ sw) << 4), make_uint4(0u, 0u, 0u, 0u));
+}
+
 // kMulti: a CTA may own several row tiles (persistent grid); otherwise exactly the tile blockIdx.x, and
 // the loops over tiles below fold away at compile time.
 // kEpi: the output epilogue adds a bias row and applies the activation (see ChainParams).
@@ -456,13 +475,7 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const uint32_t cb = (c & 1) * 4;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) st_shared_v4(panel + (((cb + t) ^ sw) << 4), pack8(v + 8 * t));
-                if (c * 32 + 32 > p.r) {          // what is no column of T: zero, also for a row of A that holds an infinity
-#pragma unroll 1
-                    for (int t = max(0, (p.r - c * 32 + 7) >> 3); t < 4; ++t) st_shared_v4(panel + (((cb + t) ^ sw) << 4), make_uint4(0u, 0u, 0u, 0u));
-#pragma unroll 1
-                    for (int e = p.r; (e & 7) != 0 && c * 32 < p.r; ++e)
-                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(panel + (((static_cast<uint32_t>(e >> 3) & 7u) ^ sw) << 4) + static_cast<uint32_t>(e & 7) * 2u), "h"(static_cast<unsigned short>(0)) : "memory");
-                }
+                zero_padding(panel, cb, sw, c, p.r);
             }
             tc_fence_before();
             fence_proxy_async_smem();

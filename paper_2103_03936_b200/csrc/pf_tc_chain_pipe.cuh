@@ -275,6 +275,7 @@ tc_chain_pipe_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                     const uint32_t cb = (c & 1) * 4;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) st_shared_v4(panel + (((cb + i) ^ sw) << 4), pack8(v + 8 * i));
+                    if constexpr (kConv == 0) zero_padding(panel, cb, sw, c, p.r);
                 }
                 tc_fence_before();
                 fence_proxy_async_smem();

@@ -448,15 +448,27 @@ def test_smallest_layers_infinite_factor_and_a_ragged_batch():
         assert (dU[:, 4] == m * n).all() and (dV == m).all()
 
 
-@pytest.mark.parametrize("m,r", [(300, 24), (300, 33), (20, 64)])
-def test_fused_forward_infinite_input_and_a_ragged_rank(m, r):
-    """An infinity in x makes its row of x U and of y infinite, whatever the rank is padded to."""
-    k, n = 512, 136
+@pytest.mark.parametrize("m,k,r", [(300, 512, 24), (300, 512, 33), (20, 512, 64), (2047, 136, 40), (2048, 136, 40), (5000, 136, 129),
+                                   (19500, 72, 33), (18000, 3600, 72)])
+def test_fused_forward_infinite_input_and_a_ragged_rank(m, k, r):
+    """An infinity in x makes its row of x U and of y infinite, whatever the rank is padded to and however many rows there are:
+    the single-tile, the persistent and the pipelined form of the fused kernel, with and without a bias, and beyond L2."""
+    n = 136
     x, U, V = (torch.ones(s, device="cuda", dtype=torch.bfloat16) for s in ((m, k), (k, r), (n, r)))
     x[7, 11] = float("inf")
-    y = pf.pf_lowrank_linear_fwd(x, U, V)
     rest = torch.arange(m, device="cuda") != 7
-    assert torch.isposinf(y[7]).all() and (y[rest] == float(torch.tensor(k * r).bfloat16())).all()
+    for y in (pf.pf_lowrank_linear_fwd(x, U, V), pf.pf_lowrank_linear_fwd_act(x, U, V, bias=torch.zeros(n, device="cuda", dtype=torch.bfloat16))):
+        assert torch.isposinf(y[7]).all() and (y[rest] == float((torch.tensor(float(k)).bfloat16().float() * r).bfloat16())).all()
+
+
+def test_fused_backward_infinite_gradient_and_a_ragged_rank():
+    """The same for an infinity in dY: its row of dX is infinite, the other rows are what they are without it."""
+    m, k, n, r = 2100, 1032, 264, 40
+    x, U, V, dY = (torch.ones(s, device="cuda", dtype=torch.bfloat16) for s in ((m, k), (k, r), (n, r), (m, n)))
+    dY[7, 11] = float("inf")
+    dX, _, _ = pf.pf_lowrank_linear_bwd(x, U, V, dY)
+    rest = torch.arange(m, device="cuda") != 7
+    assert torch.isposinf(dX[7]).all() and (dX[rest] == float((torch.tensor(float(n)).bfloat16().float() * r).bfloat16())).all()
 
 
 @pytest.mark.parametrize("m,k,n,r", [(2049, 136, 1032, 64), (3499, 136, 1032, 72), (3500, 136, 1032, 72), (2100, 1032, 1024, 40), (16300, 72, 264, 16), (12000, 72, 1032, 16)])
