@@ -550,9 +550,10 @@ bool short_first_product(int64_t k, int64_t r, int64_t ldx, int64_t ldu, int64_t
     const int64_t lines = 128 * (ldx % 64 ? 2 : 1) + ceil_div(r, 64) * 64 * (ldu % 64 ? 2 : 1);      // of a k-block
     return k <= most && ceil_div(k, kBK) * lines <= 11000;
 }
+double streamed_bytes(int64_t m, int64_t k, int64_t n) { return static_cast<double>(m) * static_cast<double>(k + n) * 2.0; }
 // Whether a fused launch streams more than L2 holds: its output is then the first to leave L2, and so is an operand's row once
 // read.  (An output that fits stays, for whoever reads it next.)
-bool beyond_l2(int64_t m, int64_t k, int64_t n) { return static_cast<double>(m) * static_cast<double>(k + n) * 2.0 > kL2Bytes; }
+bool beyond_l2(int64_t m, int64_t k, int64_t n) { return streamed_bytes(m, k, n) > kL2Bytes; }
 bool use_chain_fwd(const LinearArgs& a) {
     if (a.r > 192 || !tma_ok(a.y, a.ldy)) return false;
     // (operands that are copied first arrive on whole lines)
@@ -808,11 +809,15 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     if (st != PF_OK) return st;
     keep_slices(a.du_slices, &gu, narrow ? pu : SliceRoom());
     keep_slices(a.dv_slices, &gv, narrow ? pv : SliceRoom());
-    // dY and x are read for the last time: they make room.  In a step that streams more than L2 holds a fifth of dY is kept for
-    // this launch, and everything else passes through: 16384 x 4096 -> 64 -> 4096: 161 -> 149 us, 8192 x 4096 -> 64 -> 4096: 101 -> 88,
-    // 16384 x 2048 -> 64 -> 2048: 91 -> 81.  The last reads alone: 8192 x 512 -> 128 -> 2048: 42.3 -> 40.7, 12000 x 2048 -> 96 -> 2048:
-    // 84.5 -> 80.0.
-    gu.p.keep_a = gv.p.keep_a = kL2Stream;
+    // dY is read for the last time and makes room.  So does x, but it is the output of the layer below, whose activation's backward
+    // reads it next: in a step that streams less than a quarter of L2 it stays.  Blocks of two layers with their activations, six in
+    // a row, x first to go / as ever: 4096 x 512 -> 128 -> 2048 and back (21 MB a layer): 89.7 / 87.2 us a block, 6000: 98.9 / 97.1, 8192:
+    // 108.8 / 108.3, 12000: 141.4 / 143.9, 16384: 176.0 / 179.7; backward of one layer of 8192 x 2048 -> 128 -> 512: 27.0 / 28.3, of 12000 x
+    // 2048 -> 96 -> 2048: 51.8 / 56.0.  In a step that streams more than L2 holds a fifth of dY is kept for this launch, and
+    // everything else passes through: 16384 x 4096 -> 64 -> 4096: 161 -> 149 us, 8192 x 4096 -> 64 -> 4096: 101 -> 88, 16384 x 2048 -> 64 ->
+    // 2048: 91 -> 81.
+    gu.p.keep_a = streamed_bytes(a.m, a.k, a.n) > kL2Bytes / 4 ? kL2Stream : 0.f;
+    gv.p.keep_a = kL2Stream;
     const GemmLaunch* list[2] = {&gu, &gv};
     if (gu.p.splits <= 1 && gv.p.splits > 1) std::swap(list[0], list[1]);       // a split product has to come before the plain ones
     if (dv_beside) {
