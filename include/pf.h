@@ -199,11 +199,13 @@ int pf_lowrank_linear_bwd(const void* x, int64_t ldx, const void* U, int64_t ldu
  *                       `dtype` is: with PF_BF16 the fp32 sums are stored unrounded.
  * dX is never accumulated and stays in `dtype`.  flags = 0 is pf_lowrank_linear_bwd.  The call runs
  * the same kernels as the plain backward, with the plain gradients directed into the workspace, and
- * one more small launch writes the caller's matrices: where a reduction over the batch was split across
- * thread blocks (every benchmark shape) from the fp32 slices that reduction left in the workspace,
- * summed again in the same order, so that the values are the unrounded fp32 sums (rounded once when
- * added into a PF_BF16 matrix); on the remaining paths from the plain gradient (PF_BF16: the
- * micro-batch's gradient has then been rounded to bf16 before it is widened or added).
+ * one more small launch writes the caller's matrices: where a reduction over the batch left its fp32 slices in the
+ * workspace (split ones, every benchmark shape among them, and whole ones unless the tiles of dU and dV are more than
+ * the SMs) from those, summed again in the same order, so that the values are the unrounded fp32 sums (rounded
+ * once when added into a PF_BF16 matrix); on the remaining paths from the plain gradient (PF_BF16: the
+ * micro-batch's gradient has then been rounded to bf16 before it is widened or added).  With PF_BF16 the sums are those of
+ * the tensor cores (relative error 1e-7 to 5e-6, growing with the rows of a slice) of operands T and G that were
+ * rounded to bf16, which weighs about 1.7e-3.
  * Same workspace query, pitches and errors as pf_lowrank_linear_bwd; unknown flag bits are
  * PF_ERR_INVALID_ARG.  With m = 0 and PF_GRAD_ACCUMULATE nothing is written. */
 #define PF_GRAD_ACCUMULATE 1u

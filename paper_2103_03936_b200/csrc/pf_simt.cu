@@ -195,7 +195,8 @@ repack_rows_kernel(const unsigned short* __restrict__ src, int64_t ld_src,
 // destination row: the destination is 16-byte aligned with a pitch that is a multiple of 8
 // elements, the source may start at any element.  Pure streaming (4 bytes per element), so both sides move
 // 16 bytes per access: a whole piece is assembled from the two aligned source vectors that cover it with a
-// funnel shift (each of them holds at least one byte of the piece), only a row's last piece reads elements.
+// funnel shift; a row's last piece takes the vectors that hold at least one of its bytes and masks what lies behind the
+// row.  (Bytes beside the source inside an aligned vector are read, never used.)
 // A job may cover several matrices (groups) a fixed stride apart, which land one after the other.
 // Launched with programmatic dependent launch: its start hides behind the previous kernel's tail, and the
 // product that reads the copies starts its own prologue meanwhile.

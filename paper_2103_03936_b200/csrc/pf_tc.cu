@@ -48,7 +48,7 @@ size_t gemm_smem(int bn, int stages, bool dx = false) {
 // one CTA overlap the main loop of the other.
 int pick_stages(int bn, int64_t ctas, bool dx = false) {
     const size_t stage = static_cast<size_t>(kBM * kBK * 2 + bn * kBK * 2);
-    const size_t room = ((ctas > num_sms() && bn <= 128) ? (113 * 1024 - 2048) : (200 * 1024 - 2048)) - (dx ? 4 * kDxPanel : 0);
+    const size_t room = (ctas > num_sms() ? (113 * 1024 - 2048) : (200 * 1024 - 2048)) - (dx ? 4 * kDxPanel : 0);
     int ns = static_cast<int>(room / stage);
     if (ns > kMaxStages) ns = kMaxStages;
     if (ns < 2) ns = 2;
@@ -104,6 +104,10 @@ struct SliceRoom {
 // 1024 x 256 over 512: 9.3 us in two slices, 4.8 whole; over 1024: 8.4 in four, 6.0 whole; over 2048: 8.4 in eight, 8.4
 // whole; over 4096: 9.3 in eight, 13.0 whole.  (dU of 26 x 7 x 7, 160 -> 40 -> 160 over 26 blocks of 49 pixels: backward 13.8 us
 // split, 16.0 whole; of 16 x 14 x 14, stride 2, over 16: 12.8 and 9.8.)
+// What a whole contraction costs is exactness of the sum, which tensor memory truncates: dV = dY^T T of 512 -> 128 -> 512 in fp32
+// against 64 bits, 1000 rows: relative error 9.7e-7 whole, 1.0e-7 in sixteen slices; 512 rows 4.7e-7 and 0.9e-7 (8192 rows of 1024 ->
+// 256 -> 4096, two slices: 4.4e-6).  It does not show in the gradients of the layer, whose T and G are rounded to bf16: 1000
+// rows, fp32 dU and dV are off by 1.6625e-3 and 1.6439e-3 whole, 1.6625e-3 and 1.6442e-3 in slices; stored in bf16 by 2.34e-3.
 constexpr double kBlockUs = 0.23;
 double slice_us(int64_t nkb, int64_t s) {
     return kBlockUs * static_cast<double>(ceil_div(nkb, s)) + (s > 1 ? 3.4 + 3.4 / static_cast<double>(s) : 0.0);
@@ -392,7 +396,8 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
 
 // Expected microseconds of one launch of prepared products on single CTAs, and of the same products on CTA pairs, fitted
 // to launches of one product between 512 and 16384 rows, 256 to 4096 columns and contractions of 256 to 16384 (within
-// 20 %, mostly 10 %).  A single CTA's 128 x 128 tile: 3.6 us of start and end and slice_us alone on its SM; 4.1 us and
+// 20 %, mostly 10 %).  A single CTA's 128 x 128 tile alone on its SM: 3.6 us of start and end, 0.2 us per k-block and what
+// slice_us counts for the sum of its slices (whose own 0.23 decides between slices and whole only); 4.1 us and
 // 0.42 us per k-block beside another (its SM's load path is what it waits for).  A pair's 256 x 256 tile: 0.28 us per
 // k-block (the tensor cores), and 2 us of every tile but the first do not hide (the results' way to memory).  Output rows
 // that take no 16-byte stores: 1.2 us more per single tile, 2.1 per tile of a pair.
@@ -1113,7 +1118,7 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     if (st != PF_OK) return st;
     // dT: more tiles than two per SM, of few k-blocks each, go up to four to a block
     const int64_t gt_tiles = static_cast<int64_t>(gt.grid.x) * gt.grid.y;
-    if (gt.bn <= 128 && gt.p.nkb_total <= 8 && gt_tiles > 2 * num_sms()) {
+    if (gt.p.nkb_total <= 8 && gt_tiles > 2 * num_sms()) {
         gt.runs = true;
         gt.grid = dim3(static_cast<unsigned>(ceil_div(gt_tiles, std::min<int64_t>(4, ceil_div(gt_tiles, 2 * num_sms())))));
         gt.p.num_stages = pick_stages(gt.bn, gt.grid.x, true);

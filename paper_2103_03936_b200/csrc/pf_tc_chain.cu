@@ -136,6 +136,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     p.status = device_status_ptr();
     p.keep[0] = keep_a; p.keep[1] = keep_out;
     dim3 grid(static_cast<unsigned>(grid_x), static_cast<unsigned>(plan.nsplit), 1);
+    // (The persistent forms, which take over from 148 row tiles on, have no hints; with them they have not been measured.)
     if (!conv && !persistent && (keep_a != 0.f || keep_out != 0.f)) return chain_launch_hints(grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
     if (out && (bias || act)) return chain_launch_act(persistent, grid, plan.smem, stream, ta, tb1, tb2, to, tt, p);
     if (persistent) {
@@ -162,19 +163,19 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     return PF_OK;
 }
 
-// The chain for several groups of one shape, sA (0: one A read by all) ... sT elements apart; out or T may be null.
+// The chain for several groups of one shape, sA (0: one A read by all) ... sT elements apart; T may be null.
 // The launch shares the machine with those of the other groups of `all`; late_wait: the launch before in the stream is one of them.
 int chain_groups(int groups, int all, const void* A, int64_t lda, int64_t sA, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t sB1, int64_t r,
                  const void* B2, int64_t ldb2, int64_t sB2, int64_t N2, void* out, int64_t ldo, int64_t sO, void* T, int64_t ldt, int64_t sT,
                  bool late_wait, cudaStream_t stream) {
     ChainPlan plan;
-    if (groups > 65535 || !chain_plan(M, K1, N2, r, out != nullptr, &plan, 128, 0, all)) return PF_ERR_UNSUPPORTED;
+    if (groups > 65535 || !chain_plan(M, K1, N2, r, true, &plan, 128, 0, all)) return PF_ERR_UNSUPPORTED;
     // (row tiles of 96 rows: see chain)
-    const int rows_tile = out && plan.nsplit == 1 && ceil_div(M, 96) * all <= num_sms() ? 96 : 128;
+    const int rows_tile = plan.nsplit == 1 && ceil_div(M, 96) * all <= num_sms() ? 96 : 128;
     CUtensorMap ta, tb1, tb2, to, tt;
     const bool ok = cached_map_3d(&ta, A, sA == 0 ? 1 : groups, M, K1, lda, sA, rows_tile) && cached_map_3d(&tb1, B1, groups, K1, r, ldb1, sB1, 64) &&
                     cached_map_3d(&tb2, B2, groups, N2, r, ldb2, sB2, 128) &&
-                    (out ? cached_map_3d(&to, out, groups, M, N2, ldo, sO, 32) : cached_map_3d(&to, B2, groups, N2, r, ldb2, sB2, 32)) &&
+                    cached_map_3d(&to, out, groups, M, N2, ldo, sO, 32) &&
                     (T ? cached_map_3d(&tt, T, groups, M, r, ldt, sT, rows_tile) : cached_map_3d(&tt, B2, groups, N2, r, ldb2, sB2, 128));
     if (!ok) return PF_ERR_CUDA;
     ChainParams p = {};

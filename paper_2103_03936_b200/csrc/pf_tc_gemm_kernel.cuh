@@ -764,7 +764,7 @@ __device__ __forceinline__ void run_tiles(const CUtensorMap& tmA, const CUtensor
 }
 
 template <int BN, bool kRuns, bool kAny>
-__global__ void __launch_bounds__(kGemmThreads, BN <= 128 ? 2 : 1)
+__global__ void __launch_bounds__(kGemmThreads, 2)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const GemmParams p) {
     if constexpr (kRuns) {
