@@ -560,9 +560,9 @@ double streamed_bytes(int64_t m, int64_t k, int64_t n) { return static_cast<doub
 // read.  (An output that fits stays, for whoever reads it next.)
 bool beyond_l2(int64_t m, int64_t k, int64_t n) { return streamed_bytes(m, k, n) > kL2Bytes; }
 bool use_chain_fwd(const LinearArgs& a) {
-    if (a.r > 192 || !tma_ok(a.y, a.ldy)) return false;
+    if (a.r > 192 || !tma_out(a.y, a.ldy, a.n)) return false;
     // (operands that are copied first arrive on whole lines)
-    return a.m >= 2048 || (short_first_product(a.k, a.r, tma_ok(a.x, a.ldx) ? a.ldx : 0, tma_ok(a.U, a.ldu) ? a.ldu : 0, 1536) && (!a.T || tma_ok(a.T, a.ldt)));
+    return a.m >= 2048 || (short_first_product(a.k, a.r, tma_ok(a.x, a.ldx) ? a.ldx : 0, tma_ok(a.U, a.ldu) ? a.ldu : 0, 1536) && (!a.T || tma_out(a.T, a.ldt, a.r)));
 }
 
 size_t repack_room(int64_t rows, int64_t cols, bool tight = false) {
@@ -654,10 +654,9 @@ size_t linear_fwd_need(const LinearArgs& a, bool* handles) {
     }
     *handles = true;
     const size_t t_bytes = align_up(static_cast<size_t>(a.m) * row_pitch(a.r, a.tight) * 2, 256);
-    const bool stash_direct = a.T && tma_ok(a.T, a.ldt);
     ChainPlan plan;
     if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan))
-        return room + ((a.T && !stash_direct) ? t_bytes : 0);
+        return room + (a.T && !tma_out(a.T, a.ldt, a.r) ? t_bytes : 0);
     return room + t_bytes + first_partial_bytes(a.m, a.k, a.n, a.r, false);
 }
 
@@ -681,14 +680,15 @@ int linear_fwd(const LinearArgs& a, int* handled) {
     st = repacks.flush(a.stream);
     if (st != PF_OK) return st;
     *handled = 1;
-    // T: written straight into the stash when TMA can read it back, else into padded scratch
+    // T: written straight into the stash when TMA can store it (fused) or read it back, else into padded scratch
     void* T = scratch;
     int64_t ldT = row_pitch(a.r, a.tight);
-    const bool stash_direct = a.T && tma_ok(a.T, a.ldt);
-    if (stash_direct) { T = a.T; ldT = a.ldt; }
     ChainPlan plan;
+    const bool fused = use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan);
+    const bool stash_direct = a.T && (fused ? tma_out(a.T, a.ldt, a.r) : tma_ok(a.T, a.ldt));
+    if (stash_direct) { T = a.T; ldT = a.ldt; }
     bool stash_written = false;   // the stash at its own (TMA-unreadable) pitch came out of the first product
-    if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan)) {
+    if (fused) {
         // one fused kernel; the intermediate leaves the chip only if a stash was asked for
         st = chain(x.p, x.ld, a.m, a.k, U.p, U.ld, a.r, V.p, V.ld, a.n, a.y, a.ldy, a.T ? T : nullptr, ldT,
                    a.stream, nullptr, 0, a.bias, a.act, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f, beyond_l2(a.m, a.k, a.n) ? kL2Stream : 0.f);
@@ -745,7 +745,7 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     scratch += align_up(static_cast<size_t>(a.m) * ldG * 2, 256);
     size_t pu_bytes = 0, pv_bytes = 0;
     ChainPlan plan;
-    const bool fused_dx = use_chain(a.m, a.r) && !unfused_backward(a.m, a.k, a.n, a.r) && (!a.dX || tma_ok(a.dX, a.lddx)) &&
+    const bool fused_dx = use_chain(a.m, a.r) && !unfused_backward(a.m, a.k, a.n, a.r) && (!a.dX || tma_out(a.dX, a.lddx, a.k)) &&
                           chain_plan(a.m, a.n, a.k, a.r, a.dX != nullptr, &plan);
     int su, sv;
     bool dv_beside;
@@ -921,7 +921,7 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     // other: 4 x (1024 x 512 -> 128 -> 512): 13.0 -> 8.3 us, 4 x (8192 x 512 -> 128 -> 512): 26.7 -> 19.3, 2 x (7666 x 1976 ->
     // 120 -> 1976): 51 -> 42; 4 x (185 x 1536 -> 192 -> 1536): 12.1 -> 12.8; 8 x (4789 x 72 -> 8 -> 72): 18.3 -> 18.8.
     ChainPlan plan;
-    if (a.r <= 192 && (a.m >= 2048 || short_first_product(a.k, a.r, x.ld, U.ld, 1024)) && (a.k + a.n >= 512 || ceil_div(a.m, kBM) * a.groups <= 2 * num_sms()) && grouped_ok(a.y, a.ldy, a.sy) && (!a.T || stash_direct) &&
+    if (a.r <= 192 && (a.m >= 2048 || short_first_product(a.k, a.r, x.ld, U.ld, 1024)) && (a.k + a.n >= 512 || ceil_div(a.m, kBM) * a.groups <= 2 * num_sms()) && grouped_ok(a.y, a.ldy, a.sy) && a.n % 8 == 0 && (!a.T || (stash_direct && a.r % 8 == 0)) &&
         chain_plan(a.m, a.k, a.n, a.r, true, &plan, 128, 0, a.groups)) {
         *handled = 1;
         int st = repacks.flush(a.stream);
@@ -978,7 +978,7 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     // 2 x (8000 x 1024 -> 64 -> 256): 44.6 -> 23.4 us, 4 x (8192 x 512 -> 128 -> 512): 48.8 -> 42.1, 2 x (7666 x 1976 -> 120 -> 1976):
     // 104 -> 78.
     ChainPlan plan;
-    const bool fused = !shared_x && a.dX && use_chain(a.m, a.r) && grouped_ok(a.dX, a.lddx, a.sdx) && chain_plan(a.m, a.n, a.k, a.r, true, &plan, 128, 0, a.groups);
+    const bool fused = !shared_x && a.dX && use_chain(a.m, a.r) && grouped_ok(a.dX, a.lddx, a.sdx) && a.k % 8 == 0 && chain_plan(a.m, a.n, a.k, a.r, true, &plan, 128, 0, a.groups);
     int su = gp.su, sv = gp.sv;
     if (fused) {
         const int64_t nkb = ceil_div(a.m, kBK);

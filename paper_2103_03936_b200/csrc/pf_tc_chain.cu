@@ -65,7 +65,8 @@ bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, Chai
     return true;
 }
 
-// out may be null (phase 1 only: T is written and nothing else).  All pointers must satisfy tma_ok.
+// out may be null (phase 1 only: T is written and nothing else).  All pointers must satisfy tma_ok, those of the caller's
+// matrices that are written tma_out.
 int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t r,
           const void* B2, int64_t ldb2, int64_t N2, void* out, int64_t ldo, void* T, int64_t ldt,
           cudaStream_t stream, const ChainConv* conv, int max_split, const void* bias, int act, float keep_a, float keep_out) {

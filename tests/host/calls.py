@@ -146,6 +146,9 @@ def draw(rng, kind):
 
 
 def fixed(kind):
+    if kind in ("linear", "linear_bwd"):          # ragged widths at pitches of whole 16-byte pieces
+        for m in (20, 300, 2100, 19500):
+            yield linear, (m, 60, 140, 28, BF16), dict(bwd=kind == "linear_bwd", pads=(4,) * 8)
     if kind == "linear_bwd":
         for shape in WIDE:
             for flags in (0, ACCUMULATE, GRADS_F32):

@@ -10,6 +10,9 @@
 #include <vector>
 
 #include "pf_tc.h"
+#define kMaxStages kChainMaxStages      // (each of the two headers has one of its own)
+#include "pf_tc_chain_kernel.cuh"
+#undef kMaxStages
 #include "pf_tc_f32_kernel.cuh"
 #include "pf_tc_gemm_kernel.cuh"
 
@@ -64,6 +67,18 @@ void check(const pf::SimtGemm& g) {
     inside("result of an FMA product", address(g.C), matrix(g.M, g.N, g.ldc, size));
 }
 
+// What the recorded maps hold: where the matrix lies and the bytes of its rows.
+struct MapNote {
+    uint64_t base, row_bytes;
+};
+// A matrix that TMA stores: it fills the last 16-byte piece of a row, so unless it lies in the workspace (the last buffer) its rows
+// end with one.
+void stored(const char* what, const CUtensorMap& map) {
+    const MapNote& n = reinterpret_cast<const MapNote&>(map);
+    const bool in_workspace = !regions.empty() && n.base >= regions.back().base && n.base < regions.back().base + regions.back().bytes;
+    if (n.row_bytes % 16 != 0 && !in_workspace && n.base < (1ull << 60)) faults += std::string(what) + ": the store fills pieces behind the ends of the rows\n";
+}
+
 template <typename T>
 const T& arg(void** args, int i) { return *static_cast<const T*>(args[i]); }
 void launched(const void* kernel, unsigned blocks, void** args) {
@@ -78,6 +93,10 @@ void launched(const void* kernel, unsigned blocks, void** args) {
         if (static_cast<int>(blocks) > end1) check(arg<pf::tc::GemmParams>(args, 8));
     } else if (is("tc_gemm_kernel")) {
         check(arg<pf::tc::GemmParams>(args, 2));
+    } else if (is("tc_chain_kernel") || is("tc_chain_pipe_kernel")) {
+        const pf::tc::ChainParams& p = arg<pf::tc::ChainParams>(args, 5);
+        if (p.tiles_per_split > 0) stored("output of the fused kernel", arg<CUtensorMap>(args, 3));
+        if (p.store_T) stored("intermediate of the fused kernel", arg<CUtensorMap>(args, 4));
     } else if (is("tc_f32_kernel")) {
         const pf::tc::F32Launch& l = arg<pf::tc::F32Launch>(args, 0);
         for (int i = 0; i < 3; ++i)
@@ -94,6 +113,7 @@ CUresult encode(CUtensorMap* map, CUtensorMapDataType type, cuuint32_t rank, voi
     for (cuuint32_t i = 1; i < rank; ++i) bytes += (dims[i] - 1) * strides[i - 1];
     inside("tensor map", address(base), bytes);
     *map = CUtensorMap();
+    reinterpret_cast<MapNote&>(*map) = MapNote{address(base), dims[0] * size};
     return CUDA_SUCCESS;
 }
 }  // namespace

@@ -81,6 +81,13 @@ def run_grouped(G, m, k, n, r, dtype, seed, shared_x, stash=True, need_dX=True, 
     return launches_fwd, launches_bwd
 
 
+@pytest.mark.parametrize("m", [300, 2100])
+def test_ragged_stash_at_a_pitch_of_whole_16_byte_pieces(m):
+    """The stash's rows end inside a piece: what lies behind its last column is the caller's."""
+    run_grouped(3, m, 64, 72, 28, wl.BF16, 46, False, pad_to=8)
+    run_grouped(3, m, 64, 72, 28, wl.BF16, 47, True, pad_to=8)
+
+
 @pytest.mark.parametrize("dtype", [wl.F32, wl.BF16])
 @pytest.mark.parametrize("shared_x", [False, True])
 def test_small_and_ragged_shapes_run_group_by_group(dtype, shared_x):

@@ -120,6 +120,13 @@ def test_leading_dimensions_and_padding_untouched(dtype):
     run_case(wl.LinearCase("ld", 77, 33, 50, 7, dtype, 9), ld_pad=3)
 
 
+@pytest.mark.parametrize("m", [20, 300, 2100, 19500])
+def test_ragged_widths_at_pitches_of_whole_16_byte_pieces(m):
+    """Rows that end inside a piece at pitches that TMA takes: what lies behind the last column is the caller's."""
+    run_case(wl.LinearCase("ld", m, 60, 140, 28, wl.BF16, 80), ld_pad=4)
+    run_case(wl.LinearCase("ld", m, 60, 144, 28, wl.BF16, 81), ld_pad=4, stash=False)
+
+
 @pytest.mark.parametrize("dtype", [wl.F32, wl.BF16])
 def test_recompute_without_stash_and_no_dX(dtype):
     run_case(wl.LinearCase("ns", 300, 136, 72, 24, dtype, 10), stash=False)
