@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 
 #include "pf_tc_gemm_kernel.cuh"
 #include "pf_tc_host.h"
@@ -29,6 +30,7 @@ struct Operand {
     int64_t ld;
     bool mn_major;
     int64_t gs = 0;     // grouped products: elements between the matrices of consecutive groups (0 = one matrix shared by all)
+    bool warm = false;  // written by the launch before: in L2 if it fits
 };
 
 // Several problems of one shape in one product.  sum_groups: the groups are summed into ONE output (the
@@ -214,6 +216,7 @@ struct GemmLaunch {
     dim3 grid;
     int bn;
     bool runs = false;       // several tiles per block (plain product, K-major A and MN-major B)
+    bool straddles = false, warm = false;     // A's rows do not start on 128-byte lines; see Operand
 };
 
 // Bytes of the slices of a prepared product.
@@ -320,6 +323,8 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     }
     out->grid = grid;
     out->bn = bn;
+    out->straddles = A.ld % 64 != 0;
+    out->warm = A.warm;
     return PF_OK;
 }
 
@@ -394,41 +399,85 @@ int gemm_multi(const GemmLaunch* const* g, int count, cudaStream_t stream) {
     return PF_OK;
 }
 
-// Expected microseconds of one launch of prepared products on single CTAs, and of the same products on CTA pairs, fitted
-// to launches of one product between 512 and 16384 rows, 256 to 4096 columns and contractions of 256 to 16384 (within
-// 20 %, mostly 10 %).  A single CTA's 128 x 128 tile alone on its SM: 3.6 us of start and end, 0.2 us per k-block and what
-// slice_us counts for the sum of its slices (whose own 0.23 decides between slices and whole only); 4.1 us and
-// 0.42 us per k-block beside another (its SM's load path is what it waits for).  A pair's 256 x 256 tile: 0.28 us per
-// k-block (the tensor cores), and 2 us of every tile but the first do not hide (the results' way to memory).  Output rows
-// that take no 16-byte stores: 1.2 us more per single tile, 2.1 per tile of a pair.
-double single_us(const GemmLaunch* const* g, int count) {
-    double ctas = 0, load = 0, alone = 0, beside = 0, shortest = 1e30;
-    for (int i = 0; i < count; ++i) shortest = std::min<double>(shortest, g[i]->p.kb_per_split);
-    for (int i = 0; i < count; ++i) {
-        const double n = static_cast<double>(g[i]->grid.x) * g[i]->grid.y * g[i]->grid.z, kb = g[i]->p.kb_per_split;
-        const double sum = slice_us(g[i]->p.nkb_total, g[i]->p.splits) - kBlockUs * kb + (g[i]->p.splits > 1 || vector_rows(g[i]->p.C, g[i]->p.ldc, g[i]->p.c_gstride) ? 0.0 : 1.2);
-        ctas += n;
-        load += n * (0.42 * kb + 4.1 + sum);
-        alone = std::max(alone, 0.2 * kb + sum);
-        beside = std::max(beside, 0.42 * shortest + 0.2 * (kb - shortest) + sum);
-    }
-    if (ctas <= num_sms()) return 3.6 + alone;
-    return std::max(load / (2.0 * num_sms()), beside + 4.1);
+// What the expected time of a product depends on.
+struct Work {
+    double M, N, kb, blocks;      // kb: k-blocks of a thread block, all of the contraction's where there are no slices
+    double alone, beside;         // microseconds per k-block by itself on its SM, and beside another block
+    double a_bytes, cold, end;    // end: the sum of slices, rows that take no 16-byte stores
+    bool vec;
+};
+// groups: problems of one shape that the product covers (1 where they are part of the contraction).
+Work work_of(int64_t M, int64_t N, int64_t nkb, int splits, int64_t groups, bool a_mn, bool straddles, bool warm, bool vec) {
+    Work w;
+    const int bn = pick_bn(N);
+    const int64_t per = ceil_div(nkb, std::max(1, splits)), s = ceil_div(nkb, std::max<int64_t>(1, per));
+    w.M = static_cast<double>(M); w.N = static_cast<double>(N); w.kb = static_cast<double>(per);
+    w.blocks = static_cast<double>(ceil_div(M, kBM) * ceil_div(N, bn) * s * groups);
+    w.a_bytes = static_cast<double>(M) * static_cast<double>(nkb) * 128.0 * static_cast<double>(groups);
+    w.cold = warm && w.a_bytes < 6e7 ? 0.0 : std::min(1.0, w.a_bytes / 16e6);
+    const double lines = !straddles ? 1.0 : a_mn ? 1.55 : 1.15;
+    w.alone = (0.15 + 0.12 * w.cold) * lines;
+    w.beside = (0.33 + 0.28 * w.cold) * lines;
+    w.vec = vec;
+    w.end = s > 1 ? 3.6 + 3.6 / static_cast<double>(s) : vec ? 0.0 : 3.3;
+    return w;
 }
-double pairs_us(const PairJob* j, int count) {
-    double load = 0, longest = 0, tiles = 0;
+// Expected microseconds of one launch of products on single CTAs, and of one product on CTA pairs, fitted to forwards of 559
+// shapes on three forms each and backwards of 774 in two or three orders of launches (64 to 32768 rows, widths of 64 to 6912, ranks
+// of 8 to 1024), most within 15 %.  A single CTA's 128 x 128 tile alone on its SM: 3.7 us of start and end, 0.15 us per k-block from
+// L2 and 0.27 from memory; beside another 4.5 and 0.33 to 0.61, and whole rounds of two blocks per SM where the launch
+// is one product.  Rows of A that straddle 128-byte lines are two requests each: 1.55 times that where the contraction runs
+// down the rows.  A pair's 256 x 256 tile: 0.27 to 0.32 us per k-block, and 2.3 us of every tile do not hide.  An A that does
+// not stay in L2 is read from memory once per column of tiles.
+double singles_us(const Work* w, int count) {
+    const double sms = num_sms();
+    double blocks = 0, load = 0, alone = 0, beside = 0, memory = 0, shortest = 1e30;
+    for (int i = 0; i < count; ++i) shortest = std::min(shortest, w[i].kb);
     for (int i = 0; i < count; ++i) {
-        const double n = static_cast<double>(ceil_div(j[i].M, 256) * ceil_div(j[i].N, 256)) * (j[i].sum_groups ? 1 : j[i].groups);
-        const double kb = static_cast<double>(ceil_div(j[i].K, 64)) * (j[i].sum_groups ? j[i].groups : 1);
-        const double us = 0.28 * kb + (vector_rows(j[i].C, j[i].ldc, j[i].c_gs) ? 2.0 : 4.1);
+        blocks += w[i].blocks;
+        load += w[i].blocks * (w[i].beside * w[i].kb + 4.5 + w[i].end);
+        alone = std::max(alone, w[i].alone * w[i].kb + w[i].end);
+        beside = std::max(beside, w[i].beside * shortest + w[i].alone * (w[i].kb - shortest) + w[i].end);
+        if (w[i].a_bytes > 6e7) memory += w[i].a_bytes * std::ceil(w[i].N / pick_bn(static_cast<int64_t>(w[i].N))) / 6.7e6;
+    }
+    double us = 3.7 + alone;
+    if (blocks > sms) {
+        us = load / (2.0 * sms);
+        const int rounds = static_cast<int>(std::ceil(blocks / sms));
+        us = std::max(us, count == 1 ? (rounds / 2) * (w[0].beside * w[0].kb + 4.5) + (rounds % 2) * (w[0].alone * w[0].kb + 3.7) : beside + 4.5);
+    }
+    return std::max(us, memory + 3.7);
+}
+double pairs_us(const Work* w, int count) {      // unsplit products
+    const int pairs = num_sms() / 2;
+    double load = 0, longest = 0, tiles = 0, memory = 0;
+    for (int i = 0; i < count; ++i) {
+        const double per_group = std::ceil(w[i].M / kBM) * std::ceil(w[i].N / pick_bn(static_cast<int64_t>(w[i].N)));
+        const double n = std::ceil(w[i].M / 256) * std::ceil(w[i].N / 256) * (w[i].blocks / per_group);
+        const double us = (0.265 + 0.055 * w[i].cold) * w[i].kb + (w[i].vec ? 2.25 : 4.9);
         tiles += n;
         load += n * us;
         longest = std::max(longest, us);
+        if (w[i].a_bytes > 6e7) memory += w[i].a_bytes * std::ceil(w[i].N / 256) / 6.7e6;
     }
-    const int pairs = num_sms() / 2;
-    double total = load / pairs;
-    if (count == 1) total = longest * static_cast<double>(ceil_div(static_cast<int64_t>(tiles), pairs));
-    return std::max(total, longest) + 3.4;
+    const double total = count == 1 ? longest * std::ceil(tiles / pairs) : std::max(longest, load / pairs);
+    return std::max(total, memory) + 3.85;
+}
+Work work_of(const GemmLaunch& g) {
+    return work_of(g.p.M, g.p.N, g.p.nkb_total, g.p.splits, std::max(1, g.p.groups), g.p.a_mn != 0, g.straddles, g.warm, vector_rows(g.p.C, g.p.ldc, g.p.c_gstride));
+}
+double single_us(const GemmLaunch* const* g, int count) {
+    Work w[3];
+    for (int i = 0; i < count; ++i) w[i] = work_of(*g[i]);
+    return singles_us(w, count);
+}
+// The same products on pairs: whole, whatever the slices of the launches on single CTAs.
+double pairs_us(const GemmLaunch* const* g, int count) {
+    Work w[3];
+    for (int i = 0; i < count; ++i)
+        w[i] = work_of(g[i]->p.M, g[i]->p.N, g[i]->p.nkb_total, 1, std::max(1, g[i]->p.groups), g[i]->p.a_mn != 0, g[i]->straddles, g[i]->warm,
+                       vector_rows(g[i]->p.C, g[i]->p.ldc, g[i]->p.c_gstride));
+    return pairs_us(w, count);
 }
 // One launch of up to three products on single CTAs (one launch each where they cannot share it).
 int launch_singles(const GemmLaunch* const* g, int count, cudaStream_t stream) {
@@ -449,12 +498,13 @@ int launch_singles(const GemmLaunch* const* g, int count, cudaStream_t stream) {
     }
     return st;
 }
+constexpr double kPairMargin = 0.9;      // pairs have to be expected so much faster (the expectation is off by up to 15 %)
 // One launch of one or two products, on whichever form is expected to be faster.  The products are independent of
 // each other; jobs[i] describes the same product as *g[i].  pair_extra: microseconds that the caller has to spend after
 // pairs only; *pairs tells which form it was.
 int launch_faster(const GemmLaunch* const* g, const PairJob* jobs, int count, cudaStream_t stream, double pair_extra = 0.0,
                   bool* pairs = nullptr) {
-    if (pairs_us(jobs, count) + pair_extra < 0.9 * single_us(g, count)) {
+    if (pairs_us(g, count) + pair_extra < kPairMargin * single_us(g, count)) {
         PairJob order[2] = {jobs[0], jobs[count > 1 ? 1 : 0]};
         auto kb = [](const PairJob& j) { return ceil_div(j.K, 64) * (j.sum_groups ? j.groups : 1); };
         if (count > 1 && kb(order[1]) > kb(order[0])) std::swap(order[0], order[1]);     // long tiles first
@@ -468,7 +518,7 @@ int launch_faster(const GemmLaunch* const* g, const PairJob* jobs, int count, cu
 }
 // One launch of up to three products on single CTAs, or the first of them on CTA pairs by itself and then the others.
 int launch_with(const GemmLaunch* const* g, const PairJob* first, int count, cudaStream_t stream) {
-    if (pairs_us(first, 1) + single_us(g + 1, count - 1) < 0.9 * single_us(g, count)) {
+    if (pairs_us(g, 1) + single_us(g + 1, count - 1) < kPairMargin * single_us(g, count)) {
         const int st = gemm_pairs(first, 1, 1, stream);
         if (st == PF_OK) return launch_singles(g + 1, count - 1, stream);
         if (st != PF_ERR_UNSUPPORTED) return st;
@@ -582,6 +632,9 @@ void bwd_partial_bytes(int64_t m, int64_t k, int64_t n, int64_t r, size_t* bytes
     bool beside;
     bwd_split_plan(m, k, n, r, false, &su, &sv, &beside);
     bwd_split_plan(m, k, n, r, true, &su2, &sv2, &beside);
+    su = std::max(su, su2);
+    sv = std::max(sv, sv2);
+    pick_pair_splits(k, n, r, ceil_div(m, kBK), ceil_div(m, kBK), &su2, &sv2);
     const auto bytes = narrow_reductions(k, n, r) ? slice_bytes : partial_bytes;
     *bytes_u = align_up(bytes(k, r, std::max(su, su2)), 256);
     *bytes_v = align_up(bytes(n, r, std::max(sv, sv2)), 256);
@@ -699,7 +752,7 @@ int linear_fwd(const LinearArgs& a, int* handled) {
                   pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream,
                   (a.T && !stash_direct) ? a.T : nullptr, a.ldt, &stash_written);
         if (st != PF_OK) return st;
-        st = gemm({T, ldT, false}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, a.stream, nullptr, 0, nullptr,
+        st = gemm({T, ldT, false, 0, true}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, a.stream, nullptr, 0, nullptr,
                   a.bias, a.act);
     }
     if (st != PF_OK) return st;
@@ -769,23 +822,50 @@ int linear_bwd(const LinearArgs& a, int* handled) {
                    dv_beside ? 1 : 0, nullptr, 0, big ? 0.2f : 0.f, big ? kL2Stream : 0.f);
         if (st != PF_OK) return st;
     } else {
-        // Two launches: G = dY V with dV = dY^T T, which needs nothing of it, then dU = x^T G with dX = G U^T.  Where the
-        // tiles of dU and dV fit the machine they run on single CTAs, split or whole, and G and dX share their launches
-        // or, where that is faster, run on CTA pairs by themselves; larger ones run on whichever form is faster.
+        // G = dY V, then dU = x^T G and dX = G U^T, which need it; dV = dY^T T needs nothing.  Where the tiles of dU and dV fit the machine
+        // they run on single CTAs, split or whole, and the launches are ordered as is expected to be fastest:
+        //   two      {G, dV}, {dU, dX}: each reduction fills the machine, two sums of slices; few rows, or many columns of y
+        //   three    {G}, {dU, dV, dX}: one sum, and the long contraction behind one start only; 512 -> 128 -> 512: 1000 rows 10.8 us
+        //            against 12.3, 4096 x 1500 -> 256 -> 1500: 40.1 against 47.3; 8192 x 1024 -> 256 -> 4096: 78 against 61
+        //   pairs    G and dX on CTA pairs by themselves, {dU, dV}: 16384 x 768 -> 512 -> 3072: 123 us, two 144, three 150
+        // (G and dX run on pairs by themselves in the first two where that is faster.)  Larger reductions run on whichever form is faster.
         GemmLaunch gg, gv, gu, gx;
         const int bn = pick_bn(a.r);
-        const int64_t tr = ceil_div(a.r, bn), tg = ceil_div(a.m, kBM) * tr, tv = ceil_div(a.n, kBM) * tr;
-        int sg = pick_splits(a.m, a.r, bn, a.n);
+        const int64_t tr = ceil_div(a.r, bn), tg = ceil_div(a.m, kBM) * tr, tv = ceil_div(a.n, kBM) * tr, kb_n = ceil_div(a.n, kBK), kb_m = ceil_div(a.m, kBK);
+        const int sg_alone = pick_splits(a.m, a.r, bn, a.n);
+        int sg = sg_alone;
         if (sg > 1 && sv > 1 && tg * sg + tv * sv > num_sms()) {        // both sums in one launch: their blocks must fit together
             int sg2 = 1, sv2 = 1;
-            pick_pair_splits(a.m, a.n, a.r, ceil_div(a.n, kBK), ceil_div(a.m, kBK), &sg2, &sv2);
+            pick_pair_splits(a.m, a.n, a.r, kb_n, kb_m, &sg2, &sv2);
             sg = std::min(sg, sg2);                                      // (no more slices than the workspace holds)
             sv = std::min(sv, sv2);
+        }
+        enum { kTwo, kThree, kPairs } order = kTwo;
+        if (narrow) {
+            int su3, sv3;
+            pick_pair_splits(a.k, a.n, a.r, kb_m, kb_m, &su3, &sv3);
+            const bool sx = x.ld % 64 != 0, sy = dY.ld % 64 != 0, vu = vector_rows(a.dU, a.lddu, 0), vv = vector_rows(a.dV, a.lddv, 0);
+            const Work x_work = work_of(a.m, a.k, ceil_div(a.r, kBK), 1, 1, false, false, true, vector_rows(a.dX, a.lddx, 0));
+            const Work g_work = work_of(a.m, a.r, kb_n, sg_alone, 1, false, sy, false, true), g_whole = work_of(a.m, a.r, kb_n, 1, 1, false, sy, false, true);
+            const Work two1[2] = {work_of(a.m, a.r, kb_n, sg, 1, false, sy, false, true), work_of(a.n, a.r, kb_m, sv, 1, true, sy, false, vv)};
+            const Work two2[2] = {x_work, work_of(a.k, a.r, kb_m, su, 1, true, sx, false, vu)};
+            const Work all[3] = {work_of(a.k, a.r, kb_m, su3, 1, true, sx, false, vu), work_of(a.n, a.r, kb_m, sv3, 1, true, sy, false, vv), x_work};
+            const double pair_g = pairs_us(&g_whole, 1), pair_x = pairs_us(&x_work, 1);
+            const double two = std::min(singles_us(two1, 2), (pair_g + singles_us(two1 + 1, 1)) / kPairMargin) +
+                               (a.dX ? std::min(singles_us(two2, 2), (pair_x + singles_us(two2 + 1, 1)) / kPairMargin) : singles_us(two2 + 1, 1));
+            const double three = std::min(singles_us(&g_work, 1), pair_g / kPairMargin) + singles_us(all, a.dX ? 3 : 2);
+            const double pairs = a.dX ? pair_g + pair_x + singles_us(all, 2) : 1e30;
+            // (The expectation is too good for long reductions beside many tiles of dX.  Of 774 shapes 6 take more than 3 % longer than
+            // in two launches, 1 more than 8 %; all of them together 5.6 % less, 0.9 % more than the best order of each.)
+            const bool short_ones = std::max(all[0].kb, all[1].kb) <= 64 && (a.n < 2 * a.k || a.m < 2048);
+            if (short_ones && 1.08 * three < std::min(two, 1.1 * pairs)) order = kThree;
+            else if (1.1 * pairs < two) order = kPairs;
+            if (order != kTwo) { sg = sg_alone; su = su3; sv = sv3; }
         }
         st = gemm_prepare_any({dY.p, dY.ld, false}, {V.p, V.ld, true}, a.m, a.r, a.n, G, ldG, sg, p1, nullptr, &gg);
         if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
         if (st == PF_OK) st = gemm_prepare_any({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
-        if (st == PF_OK && a.dX) st = gemm_prepare({G, ldG, false}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gx);
+        if (st == PF_OK && a.dX) st = gemm_prepare({G, ldG, false, 0, true}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gx);
         if (st != PF_OK) return st;
         const PairJob j1[2] = {{dY.p, dY.ld, false, 0, V.p, V.ld, true, 0, a.m, a.r, a.n, G, ldG},
                                {dY.p, dY.ld, true, 0, T.p, T.ld, true, 0, a.n, a.r, a.m, a.dV, a.lddv}};
@@ -803,9 +883,21 @@ int linear_bwd(const LinearArgs& a, int* handled) {
         }
         keep_slices(a.du_slices, &gu, pu);
         keep_slices(a.dv_slices, &gv, pv);
-        st = launch_with(l1, j1, 2, a.stream);
-        if (st != PF_OK) return st;
-        return a.dX ? launch_with(l2, j2, 2, a.stream) : launch_singles(l2 + 1, 1, a.stream);
+        if (order == kTwo) {
+            st = launch_with(l1, j1, 2, a.stream);
+            if (st != PF_OK) return st;
+            return a.dX ? launch_with(l2, j2, 2, a.stream) : launch_singles(l2 + 1, 1, a.stream);
+        }
+        const GemmLaunch* const l3[3] = {&gu, &gv, &gx};
+        if (order == kPairs) {
+            st = gemm_pairs(j1, 1, 1, a.stream);
+            if (st == PF_ERR_UNSUPPORTED) st = launch_prepared(gg, a.stream);
+            if (st == PF_OK) st = gemm_pairs(j2, 1, 1, a.stream);
+            if (st == PF_ERR_UNSUPPORTED) st = launch_prepared(gx, a.stream);
+            return st == PF_OK ? launch_singles(l3, 2, a.stream) : st;
+        }
+        st = launch_faster(l1, j1, 1, a.stream);
+        return st == PF_OK ? launch_singles(l3, a.dX ? 3 : 2, a.stream) : st;
     }
     // dU = x^T G, dV = dY^T T: one launch when their tiles allow
     GemmLaunch gu, gv;
@@ -938,7 +1030,7 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     const Grouping gt{a.groups, sT, false}, gy{a.groups, a.sy, false};
     int st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, T, ldT, gp.s1, p1, nullptr, &g1, &gt);
     if (st == PF_OK)
-        st = gemm_prepare({T, ldT, false, sT}, {V.p, V.ld, false, V.gs}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, nullptr, &g2, &gy);
+        st = gemm_prepare({T, ldT, false, sT, true}, {V.p, V.ld, false, V.gs}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, nullptr, &g2, &gy);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
     if (a.T && !stash_direct) {
@@ -997,7 +1089,7 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, true, dY.gs}, {T.p, T.ld, true, T.gs}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gV, &gdv);
     if (st == PF_OK) st = gemm_prepare({x.p, x.ld, true, x.gs}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gU, &gdu);
     if (st == PF_OK && a.dX)
-        st = gemm_prepare({Gbuf, ldW, false, sW}, {U.p, U.ld, false, U.gs}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gX, &gdx);
+        st = gemm_prepare({Gbuf, ldW, false, sW, true}, {U.p, U.ld, false, U.gs}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gX, &gdx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
     *handled = 1;
