@@ -713,9 +713,14 @@ size_t linear_fwd_need(const LinearArgs& a, bool* handles) {
     return room + t_bytes + first_partial_bytes(a.m, a.k, a.n, a.r, false);
 }
 
-// Whether a forward of few rows runs on the fused kernel, which takes its operands as they are, instead of pf_small.cu.
+// Whether a forward of few rows runs on the fused kernel, which takes its operands as they are, instead of pf_small.cu.  Those kernels
+// take as long for 1 row as for 8 and more from there on, the fused one the same for all 32: 570 shapes, fused against pf_small.cu
+// in the mean 1.04 times up to 8 rows, 0.94 for 12 and 16, 0.92 for 20 and 24, 0.77 beyond.  Up to 8 rows the fused kernel is
+// faster where its first product is one k-block or pf_small.cu's would be cut finely, at small ranks (8 x 384 -> 32 -> 1536: 0.91; 8 x
+// 256 -> 192 -> 256: 1.21); a wide output of a small rank is many rows of V in few lines (20 x 512 -> 8 -> 6000: 1.18).
 bool few_rows_fused(const LinearArgs& a) {
-    return encode_fn() != nullptr && a.k <= 512 && a.n <= (1 << 22) && use_chain_fwd(a) && tma_ok(a.x, a.ldx) && tma_ok(a.U, a.ldu) && tma_ok(a.V, a.ldv);
+    const bool faster = a.m <= 8 ? a.r <= 64 && a.n <= 2048 && (a.k <= 64 || a.k > 256) : !(a.n > 4096 && a.m <= 24 && a.r < 64);
+    return faster && encode_fn() != nullptr && a.k <= 512 && a.n <= (1 << 22) && use_chain_fwd(a) && tma_ok(a.x, a.ldx) && tma_ok(a.U, a.ldu) && tma_ok(a.V, a.ldv);
 }
 
 int linear_fwd(const LinearArgs& a, int* handled) {
