@@ -1013,12 +1013,13 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     void* T = stash_direct ? a.T : static_cast<void*>(Tbuf);
     const int64_t ldT = stash_direct ? a.ldt : row_pitch(a.r), sT = stash_direct ? a.st : a.m * row_pitch(a.r);
     // The fused kernel where it pays for one group (see use_chain_fwd; k up to 1024, as the groups share the SMs), in two
-    // launches of half of the groups each (the call's launches are documented as two) that run side by side.  Not for more
-    // than two waves of the smallest tiles, whose starts the two products hide better.  Against two products one after the
+    // launches of half of the groups each (the call's launches are documented as two) that run side by side.  Not where the
+    // tiles are small and more than a wave or two, whose starts the two products hide better: 4 x (8000 x 256 -> 32 -> 64): 10.7 us
+    // unfused, 13.8 fused; 4 x (8000 x 64 -> 32 -> 256): 12.5 and 11.3.  Against two products one after the
     // other: 4 x (1024 x 512 -> 128 -> 512): 13.0 -> 8.3 us, 4 x (8192 x 512 -> 128 -> 512): 26.7 -> 19.3, 2 x (7666 x 1976 ->
     // 120 -> 1976): 51 -> 42; 4 x (185 x 1536 -> 192 -> 1536): 12.1 -> 12.8; 8 x (4789 x 72 -> 8 -> 72): 18.3 -> 18.8.
     ChainPlan plan;
-    if (a.r <= 192 && (a.m >= 2048 || short_first_product(a.k, a.r, x.ld, U.ld, 1024)) && (a.k + a.n >= 512 || ceil_div(a.m, kBM) * a.groups <= 2 * num_sms()) && grouped_ok(a.y, a.ldy, a.sy) && a.n % 8 == 0 && (!a.T || (stash_direct && a.r % 8 == 0)) &&
+    if (a.r <= 192 && (a.m >= 2048 || short_first_product(a.k, a.r, x.ld, U.ld, 1024)) && (a.k + a.n >= 512 || ceil_div(a.m, kBM) * a.groups <= (a.n >= 256 ? 2 : 1) * num_sms()) && grouped_ok(a.y, a.ldy, a.sy) && a.n % 8 == 0 && (!a.T || (stash_direct && a.r % 8 == 0)) &&
         chain_plan(a.m, a.k, a.n, a.r, true, &plan, 128, 0, a.groups)) {
         *handled = 1;
         int st = repacks.flush(a.stream);
@@ -1073,9 +1074,10 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
         return PF_OK;
     // The fused kernel for G and dX as in linear_bwd, then dU and dV, whose slices have to fit the machine together:
     // 2 x (8000 x 1024 -> 64 -> 256): 44.6 -> 23.4 us, 4 x (8192 x 512 -> 128 -> 512): 48.8 -> 42.1, 2 x (7666 x 1976 -> 120 -> 1976):
-    // 104 -> 78.
+    // 104 -> 78.  Narrow dX only while its tiles are one wave: 8 x (8000 x 64 -> 32 -> 256): 30.5 us unfused, 35.3 fused; 8 x (4000 x 256 ->
+    // 64 -> 64): 0.84 times.
     ChainPlan plan;
-    const bool fused = !shared_x && a.dX && use_chain(a.m, a.r) && grouped_ok(a.dX, a.lddx, a.sdx) && a.k % 8 == 0 && chain_plan(a.m, a.n, a.k, a.r, true, &plan, 128, 0, a.groups);
+    const bool fused = !shared_x && a.dX && use_chain(a.m, a.r) && grouped_ok(a.dX, a.lddx, a.sdx) && a.k % 8 == 0 && (a.k >= 256 || ceil_div(a.m, kBM) * a.groups <= num_sms()) && chain_plan(a.m, a.n, a.k, a.r, true, &plan, 128, 0, a.groups);
     int su = gp.su, sv = gp.sv;
     if (fused) {
         const int64_t nkb = ceil_div(a.m, kBK);
