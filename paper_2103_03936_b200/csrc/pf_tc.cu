@@ -611,6 +611,9 @@ double streamed_bytes(int64_t m, int64_t k, int64_t n) { return static_cast<doub
 bool beyond_l2(int64_t m, int64_t k, int64_t n) { return streamed_bytes(m, k, n) > kL2Bytes; }
 bool use_chain_fwd(const LinearArgs& a) {
     if (a.r > 192 || !tma_out(a.y, a.ldy, a.n)) return false;
+    // (rows of 16 bytes, eight to a line that every block asks for: 2000 x 1024 -> 8 -> 1024: 17.9 us, unfused 13.5; of 32 bytes: 12.0 and 12.3;
+    // 2000 x 512 -> 8 -> 512: 9.0 and 12.7; 1400 x 512 -> 8 -> 2048: 12.3 and 13.6)
+    if (a.r <= 8 && a.n >= 1024 && a.n < 2048 && a.m > 1024 && a.m < 2048) return false;
     // (operands that are copied first arrive on whole lines)
     return a.m >= 2048 || (short_first_product(a.k, a.r, tma_ok(a.x, a.ldx) ? a.ldx : 0, tma_ok(a.U, a.ldu) ? a.ldu : 0, 1536) && (!a.T || tma_out(a.T, a.ldt, a.r)));
 }
