@@ -81,6 +81,12 @@ def run_grouped(G, m, k, n, r, dtype, seed, shared_x, stash=True, need_dX=True, 
     return launches_fwd, launches_bwd
 
 
+@pytest.mark.parametrize("G,m,k,n,r", [(2, 9500, 64, 72, 16), (3, 6400, 72, 256, 16), (3, 6400, 256, 72, 24)])
+def test_narrow_groups_of_more_than_a_wave_of_tiles(G, m, k, n, r):
+    """Either side of the widths from which more than one wave of the fused kernel's tiles is taken, forward and backward."""
+    run_grouped(G, m, k, n, r, wl.BF16, 48, False)
+
+
 @pytest.mark.parametrize("m", [300, 2100])
 def test_ragged_stash_at_a_pitch_of_whole_16_byte_pieces(m):
     """The stash's rows end inside a piece: what lies behind its last column is the caller's."""

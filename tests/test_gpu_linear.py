@@ -361,6 +361,14 @@ def test_whole_and_split_contractions_and_pairs(m, k, n, r):
     run_case(wl.LinearCase("forms", m, k, n, r, wl.BF16, 72), blocks=True)
 
 
+@pytest.mark.parametrize("m,k,n,r", [(300, 136, 264, 40), (1100, 72, 1032, 200), (1000, 520, 520, 72), (1300, 104, 136, 24), (2320, 984, 2872, 440)])
+def test_orders_of_the_unfused_backward(m, k, n, r):
+    """Two launches (dV beside G, dU beside dX), three (dU, dV and dX behind G, whole and split) and G and dX on CTA pairs; with and
+    without dX and the stash."""
+    run_case(wl.LinearCase("order", m, k, n, r, wl.BF16, 82), blocks=m > 128)
+    run_case(wl.LinearCase("order", m, k, n, r, wl.BF16, 83), stash=False, need_dX=False)
+
+
 @pytest.mark.parametrize("m,k,n,r", [(2048, 516, 2052, 1028), (2048, 2052, 516, 1028), (2100, 520, 3080, 520)])
 def test_reductions_that_do_not_fit_the_machine_together(m, k, n, r):
     """The tiles of dU and dV are more than the SMs; each is split by itself, within the workspace that is asked for."""

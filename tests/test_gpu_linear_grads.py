@@ -96,7 +96,7 @@ def test_fp32_grads_fused_shapes_are_unrounded_sums(m, k, n, r):
     run_f32(wl.LinearCase("g32", m, k, n, r, wl.BF16, 51), expect_native=True)
 
 
-@pytest.mark.parametrize("m,k,n,r", [(700, 1504, 520, 376), (300, 136, 72, 24), (1000, 328, 520, 96)])
+@pytest.mark.parametrize("m,k,n,r", [(700, 1504, 520, 376), (300, 136, 72, 24), (1000, 328, 520, 96), (1300, 104, 136, 24), (2320, 984, 2872, 440)])
 def test_fp32_grads_few_rows(m, k, n, r):
     run_f32(wl.LinearCase("g32", m, k, n, r, wl.BF16, 52), expect_native=True)
 
