@@ -156,6 +156,8 @@ int pf_bias_act_bwd(const void* y, int64_t ldy, void* dY, int64_t lddy, void* db
  *     rows) take the fused kernel, which keeps x U on chip and needs nothing when the stash
  *     is written directly; otherwise one m x r copy of x U, the fp32 slices of a split first
  *     product, and re-pitched copies of operands whose row pitch is not a multiple of 16 bytes.
+ *     Only where the fused kernel would need nothing but cannot store rows of y or of the stash
+ *     (a width that is no multiple of 8 at a 16-byte pitch), as many rows at a time as fit.
  *     A call that needs more than PF_STATIC_SCRATCH_BYTES is rejected with PF_ERR_WORKSPACE
  *     before anything is launched.  Of the benchmark shapes both Transformer-FFN layers fit,
  *     the LSTM gate layer (700 x 1500 -> 6000, r = 375) fits with 16-byte row pitches and is

@@ -1,6 +1,7 @@
 // C-ABI entry points of libpf: argument validation, workspace layout, path selection
 // (tensor-core kernels for bf16 inside their envelope, FMA kernels otherwise) and launches.
 // Nothing here allocates or synchronises; see include/pf.h for the contract.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 
@@ -196,6 +197,20 @@ int linear_fwd_impl(const void* x, int64_t ldx, const void* U, int64_t ldu, cons
         if (dtype == PF_F32) tc_handles = tc_need > 0 && w.off_tc + tc_need <= workspace_bytes;        // (taken only when it fits; the FMA kernels need less)
         if (tc_handles) need = tc_need ? w.off_tc + tc_need : 0;
         else need = T_stash ? 0 : w.off_T + static_cast<size_t>(m) * r * dtype_size(dtype);   // FMA kernels: x U only
+        tc::LinearArgs b;
+        const int64_t rows = dtype == PF_BF16 && tc_handles && need > workspace_bytes ? tc::linear_fwd_rows(a, workspace_bytes, &b) : 0;
+        for (int64_t m0 = 0; rows > 0; m0 += rows) {
+            if (m0 >= m) return PF_OK;
+            int handled = 0;
+            b.m = std::min(rows, m - m0);
+            b.x = static_cast<const char*>(x) + m0 * ldx * 2;
+            b.y = static_cast<char*>(y) + m0 * ldy * 2;
+            if (T_stash) b.T = static_cast<char*>(T_stash) + m0 * ldt * 2;
+            b.ws = ws;
+            st = tc::linear_fwd(b, &handled);
+            if (st != PF_OK) return st;
+            if (!handled) return PF_ERR_UNSUPPORTED;
+        }
     }
     st = check_ws(workspace, workspace_bytes, need);
     if (st != PF_OK) return st;

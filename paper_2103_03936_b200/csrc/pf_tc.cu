@@ -613,7 +613,7 @@ bool use_chain_fwd(const LinearArgs& a) {
     if (a.r > 192 || !tma_out(a.y, a.ldy, a.n)) return false;
     // (rows of 16 bytes, eight to a line that every block asks for: 2000 x 1024 -> 8 -> 1024: 17.9 us, unfused 13.5; of 32 bytes: 12.0 and 12.3;
     // 2000 x 512 -> 8 -> 512: 9.0 and 12.7; 1400 x 512 -> 8 -> 2048: 12.3 and 13.6)
-    if (a.r <= 8 && a.n >= 1024 && a.n < 2048 && a.m > 1024 && a.m < 2048) return false;
+    if (!a.tight && a.r <= 8 && a.n >= 1024 && a.n < 2048 && a.m > 1024 && a.m < 2048) return false;
     // (operands that are copied first arrive on whole lines)
     return a.m >= 2048 || (short_first_product(a.k, a.r, tma_ok(a.x, a.ldx) ? a.ldx : 0, tma_ok(a.U, a.ldu) ? a.ldu : 0, 1536) && (!a.T || tma_out(a.T, a.ldt, a.r)));
 }
@@ -713,7 +713,27 @@ size_t linear_fwd_need(const LinearArgs& a, bool* handles) {
     ChainPlan plan;
     if (use_chain_fwd(a) && chain_plan(a.m, a.k, a.n, a.r, true, &plan))
         return room + (a.T && !tma_out(a.T, a.ldt, a.r) ? t_bytes : 0);
-    return room + t_bytes + first_partial_bytes(a.m, a.k, a.n, a.r, false);
+    return room + t_bytes + (a.whole ? 0 : first_partial_bytes(a.m, a.k, a.n, a.r, false));
+}
+
+// The fused kernel needs no room for x U, however many rows there are, and only its stores keep rows that end inside a 16-byte piece
+// from it.  In a workspace of a given size such a call runs on the products that take them, so many rows at a time as fit:
+// how many (0: it is no such call), where *b is how each of these calls is made.
+int64_t linear_fwd_rows(const LinearArgs& a, size_t room, LinearArgs* b) {
+    ChainPlan plan;
+    if (a.r > 192 || !tma_ok(a.y, a.ldy) || (a.n % 8 == 0 && (!a.T || !tma_ok(a.T, a.ldt) || a.r % 8 == 0))) return 0;
+    if (a.m < 2048 && !(short_first_product(a.k, a.r, tma_ok(a.x, a.ldx) ? a.ldx : 0, tma_ok(a.U, a.ldu) ? a.ldu : 0, 1536) && (!a.T || tma_ok(a.T, a.ldt)))) return 0;
+    if (!chain_plan(a.m, a.k, a.n, a.r, true, &plan)) return 0;
+    *b = a;
+    b->tight = b->whole = true;
+    for (int64_t rows = a.m;; rows = ceil_div(ceil_div(rows, 2), kBM) * kBM) {      // (whole tiles: blocks start where TMA takes them)
+        bool handles = false;
+        b->m = rows;
+        const size_t need = linear_fwd_need(*b, &handles);
+        if (!handles) return 0;
+        if (need <= room) return rows;
+        if (rows <= kBM) return 0;
+    }
 }
 
 // Whether a forward of few rows runs on the fused kernel, which takes its operands as they are, instead of pf_small.cu.  Those kernels
@@ -757,7 +777,7 @@ int linear_fwd(const LinearArgs& a, int* handled) {
         const SliceRoom p1{reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * row_pitch(a.r, a.tight) * 2, 256)),
                            first_partial_bytes(a.m, a.k, a.n, a.r, false)};
         st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, T, ldT,
-                  pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream,
+                  a.whole ? 1 : pick_splits(a.m, a.r, pick_bn(a.r), a.k), a.whole ? SliceRoom() : p1, a.stream,
                   (a.T && !stash_direct) ? a.T : nullptr, a.ldt, &stash_written);
         if (st != PF_OK) return st;
         st = gemm({T, ldT, false, 0, true}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, a.stream, nullptr, 0, nullptr,

@@ -22,6 +22,7 @@ struct LinearArgs {
     const void* bias = nullptr;   // forward: y = act((x U) V^T + bias)
     int act = 0;
     bool tight = false;           // forward: the leaner plan, for a workspace of a given size that the faster one does not fit
+    bool whole = false;           // forward: no slices of the first product, which take room
     bool group_member = false;    // one of several calls that make up a grouped one (two launches each, as documented)
     // backward: where the fp32 slices of dU / dV were left in the workspace (partial null: nowhere), for callers that want
     // the unrounded sums; a product that is one slice leaves only that
@@ -120,6 +121,7 @@ size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, in
                             int pad, bool bwd);
 void reset_fix_counters();  // clears the slice-sum counters (after PF_ERR_TIMEOUT)
 size_t linear_fwd_need(const LinearArgs& a, bool* handles);   // bytes of a.ws the forward really touches
+int64_t linear_fwd_rows(const LinearArgs& a, size_t room, LinearArgs* b);   // rows at a time in so much room, 0: not by rows
 int linear_fwd(const LinearArgs& a, int* handled);
 bool few_rows_fused(const LinearArgs& a);     // a forward that small::linear_fwd fits, but the fused kernel takes
 int linear_bwd(const LinearArgs& a, int* handled);

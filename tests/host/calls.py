@@ -52,8 +52,9 @@ def c(v):
     return ctypes.c_int(v)
 
 
-def linear(lib, m, k, n, r, dtype, *, bwd, stash=True, dX=True, flags=0, act=False, pads=(0,) * 8, offset=0, static=False):
-    """One linear call; pads: elements added to the pitches of x, U, V, y or dY, T, dX, dU, dV."""
+def linear(lib, m, k, n, r, dtype, *, bwd, stash=True, dX=True, flags=0, act=False, pads=(0,) * 8, offset=0, static=False, must=False):
+    """One linear call; pads: elements added to the pitches of x, U, V, y or dY, T, dX, dU, dV; must: the array without
+    allocation holds it."""
     size = 2 if dtype == BF16 else 4
     gsize = 4 if flags & GRADS_F32 else size
 
@@ -149,6 +150,10 @@ def fixed(kind):
     if kind in ("linear", "linear_bwd"):          # ragged widths at pitches of whole 16-byte pieces
         for m in (20, 300, 2100, 19500):
             yield linear, (m, 60, 140, 28, BF16), dict(bwd=kind == "linear_bwd", pads=(4,) * 8)
+    if kind == "linear":                          # ... which the array without allocation takes too, however many rows
+        for shape, pads in (((40000, 512, 2044, 128), (0, 0, 0, 4, 0)), ((200000, 64, 60, 32), (0, 0, 0, 4, 0)), ((600000, 64, 64, 28), (0, 4, 4, 0, 4)),
+                            ((1900, 512, 2044, 192), (0, 0, 0, 4, 0)), ((2047, 1500, 1504, 8), (0,) * 8), ((30001, 100, 100, 60), (4,) * 8)):
+            yield linear, shape + (BF16,), dict(bwd=False, static=True, must=True, pads=pads, stash=pads[4] != 0)
     if kind == "linear_bwd":
         for shape in WIDE:
             for flags in (0, ACCUMULATE, GRADS_F32):
@@ -161,7 +166,7 @@ def main(path, kind, count, seed):
     bad = 0
     for fn, args, kw in list(fixed(kind)) + [draw(rng, kind) for _ in range(count)]:
         status, faults, launches = fn(lib, *args, **kw)
-        if status == 3 and kw.get("static"):
+        if status == 3 and kw.get("static") and not kw.get("must"):
             continue                              # a problem that the fixed array does not hold is refused
         if status != 0 or faults or not launches:
             bad += 1

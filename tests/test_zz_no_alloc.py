@@ -125,6 +125,22 @@ def test_calls_that_fit_only_the_leaner_plan(m, k, n, r, dtype):
     assert pf.pf_last_device_status() == 0
 
 
+@pytest.mark.parametrize("m,k,n,r", [(43000, 64, 60, 100), (43000, 64, 64, 100)])
+def test_rows_that_end_inside_a_piece_go_through_the_array_in_blocks(m, k, n, r):
+    """y, or the stash, at a pitch of whole 16-byte pieces with a width that is none: x U is 8.9 MB, more than the array holds.
+    Nothing is written behind the last column."""
+    c = wl.LinearCase("blocks", m, k, n, r, wl.BF16, 25)
+    d = c.generate()
+    x, U, V = (dev(d[k_], c.dtype) for k_ in ("x", "U", "V"))
+    ybuf, Tbuf = (torch.full((m, w), -7.0, dtype=torch.bfloat16, device="cuda") for w in (64, 104))
+    pf.pf_lowrank_linear_fwd_static(x, U, V, y=ybuf[:, :n], T_stash=Tbuf[:, :r])
+    y_ref, T_ref = oracle.linear_fwd(d["x"], d["U"], d["V"])
+    assert_close(ybuf[:, :n], y_ref, c.dtype, "y", tol=TOL[c.dtype])
+    assert_close(Tbuf[:, :r], T_ref, c.dtype, "T", tol=TOL[c.dtype])
+    assert bool((ybuf[:, n:] == -7).all()) and bool((Tbuf[:, r:] == -7).all())
+    assert pf.pf_last_device_status() == 0
+
+
 def test_problem_larger_than_the_array_is_refused_before_any_launch():
     assert pf.pf_static_scratch_bytes() == 8 << 20
     m, k, n, r = 2000, 64, 64, 4096           # few rows: unfused products, and x U alone is 16 MB
