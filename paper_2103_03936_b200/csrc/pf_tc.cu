@@ -731,7 +731,7 @@ int64_t linear_fwd_rows(const LinearArgs& a, size_t room, LinearArgs* b) {
         b->m = rows;
         const size_t need = linear_fwd_need(*b, &handles);
         if (!handles) return 0;
-        if (rows == a.m) {      // what the fused kernel would need, the copies of all rows, has to fit behind x U
+        if (rows == a.m && !tma_ok(a.x, a.ldx)) {      // what the fused kernel would need, the copies of all rows, has to fit behind x U
             const size_t t_bytes = align_up(static_cast<size_t>(a.m) * row_pitch(a.r, true) * 2, 256), fused = need - (a.T && !tma_ok(a.T, a.ldt) ? 0 : t_bytes);
             if (fused > 0 && align_up(static_cast<size_t>(a.m) * a.r * 2, 256) + fused > room) return 0;
         }

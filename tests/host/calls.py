@@ -152,7 +152,7 @@ def fixed(kind):
             yield linear, (m, 60, 140, 28, BF16), dict(bwd=kind == "linear_bwd", pads=(4,) * 8)
     if kind == "linear":                          # ... which the array without allocation takes too, however many rows
         for shape, pads in (((40000, 512, 2044, 128), (0, 0, 0, 4, 0)), ((200000, 64, 60, 32), (0, 0, 0, 4, 0)), ((600000, 64, 64, 28), (0, 4, 4, 0, 4)),
-                            ((1900, 512, 2044, 192), (0, 0, 0, 4, 0)), ((2047, 1500, 1504, 8), (0,) * 8), ((30001, 100, 100, 60), (4,) * 8)):
+                            ((1900, 512, 2044, 192), (0, 0, 0, 4, 0)), ((43000, 64, 60, 100), (0, 0, 0, 4, 4)), ((43000, 64, 64, 100), (0, 0, 0, 0, 4)), ((2047, 1500, 1504, 8), (0,) * 8), ((30001, 100, 100, 60), (4,) * 8)):
             yield linear, shape + (BF16,), dict(bwd=False, static=True, must=True, pads=pads, stash=pads[4] != 0)
     if kind == "linear_bwd":
         for shape in WIDE:
