@@ -31,6 +31,7 @@ struct Operand {
     bool mn_major;
     int64_t gs = 0;     // grouped products: elements between the matrices of consecutive groups (0 = one matrix shared by all)
     bool warm = false;  // written by the launch before: in L2 if it fits
+    bool early = false; // neither written by the launch before nor by anything that may still run when that one has started (kEarlyA)
 };
 
 // Several problems of one shape in one product.  sum_groups: the groups are summed into ONE output (the
@@ -312,6 +313,7 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     p.counters = nullptr;
     p.partial = p.splits > 1 ? room.p : nullptr;
     p.independent = 0;
+    p.early = (A.early ? kEarlyA : 0) | (B.early ? kEarlyB : 0);
     p.keep_a = 0.f;
     if (p.splits > 1) {
         // the CTAs of a tile wait for one another, so all of them must be resident at once
@@ -547,6 +549,8 @@ int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, vo
     PairJob j{A.p, A.ld, A.mn_major, 0, B.p, B.ld, B.mn_major, 0, M, N, K, C, ldc};
     j.bias = bias;
     j.act = act;
+    j.a_early = A.early;
+    j.b_early = B.early;
     const GemmLaunch* const list[1] = {&g};
     bool pairs = false;
     const int rc = launch_faster(list, &j, 1, stream, copy2 ? 6.0 : 0.0, &pairs);
@@ -559,6 +563,7 @@ int gemm(const Operand& A, const Operand& B, int64_t M, int64_t N, int64_t K, vo
 struct Staged {
     const void* p;
     int64_t ld;
+    bool copied = false;
 };
 // Pitch of a matrix in the workspace: whole 128-byte lines, so that no 128-byte row of a TMA box touches two of them (narrow
 // rows: whole 16-byte pieces).  8 x (700 x 1500 -> 1500), r 375: forward 43.7 -> 37.5 us, backward 81.0 -> 62.5, against
@@ -582,7 +587,7 @@ int stage_operand(const void* p, int64_t ld, int64_t rows, int64_t cols, char*& 
     if (cols % 8 == 0) return 1;   // the workspace query reserves repack room only for ragged widths
     const int64_t ldp = row_pitch(cols, tight);
     list->jobs[list->count++] = RepackJob{p, ld, scratch, ldp, rows, cols};
-    out->p = scratch; out->ld = ldp;
+    out->p = scratch; out->ld = ldp; out->copied = true;
     scratch += align_up(static_cast<size_t>(rows) * ldp * 2, 256);
     return 0;
 }
@@ -762,6 +767,7 @@ int linear_fwd(const LinearArgs& a, int* handled) {
     if (stage_operand(a.x, a.ldx, a.m, a.k, scratch, &x, &repacks, a.tight)) return PF_OK;
     if (stage_operand(a.U, a.ldu, a.k, a.r, scratch, &U, &repacks, a.tight)) return PF_OK;
     if (stage_operand(a.V, a.ldv, a.n, a.r, scratch, &V, &repacks, a.tight)) return PF_OK;
+    const bool copies = repacks.count > 0;
     st = repacks.flush(a.stream);
     if (st != PF_OK) return st;
     *handled = 1;
@@ -780,11 +786,12 @@ int linear_fwd(const LinearArgs& a, int* handled) {
     } else {
         const SliceRoom p1{reinterpret_cast<float*>(scratch + align_up(static_cast<size_t>(a.m) * row_pitch(a.r, a.tight) * 2, 256)),
                            first_partial_bytes(a.m, a.k, a.n, a.r, false)};
-        st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, T, ldT,
+        // (V, and beside copies what was not copied, need not wait for the launch before)
+        st = gemm({x.p, x.ld, false, 0, false, copies && !x.copied}, {U.p, U.ld, true, 0, false, copies && !U.copied}, a.m, a.r, a.k, T, ldT,
                   a.whole ? 1 : pick_splits(a.m, a.r, pick_bn(a.r), a.k), a.whole ? SliceRoom() : p1, a.stream,
                   (a.T && !stash_direct) ? a.T : nullptr, a.ldt, &stash_written);
         if (st != PF_OK) return st;
-        st = gemm({T, ldT, false, 0, true}, {V.p, V.ld, false}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, a.stream, nullptr, 0, nullptr,
+        st = gemm({T, ldT, false, 0, true}, {V.p, V.ld, false, 0, false, true}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, a.stream, nullptr, 0, nullptr,
                   a.bias, a.act);
     }
     if (st != PF_OK) return st;
@@ -814,9 +821,10 @@ int linear_bwd(const LinearArgs& a, int* handled) {
         else if (a.r % 8 == 0) return PF_OK;   // odd pitch on an even width: FMA path
         else {
             repacks.jobs[repacks.count++] = RepackJob{a.T, a.ldt, Tbuf, row_pitch(a.r), a.m, a.r};
-            T.p = Tbuf; T.ld = row_pitch(a.r);
+            T.p = Tbuf; T.ld = row_pitch(a.r); T.copied = true;
         }
     }
+    const bool copies = repacks.count > 0;
     st = repacks.flush(a.stream);
     if (st != PF_OK) return st;
     *handled = 1;
@@ -844,7 +852,7 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     const bool narrow = narrow_reductions(a.k, a.n, a.r);
     // G = dY V ; dX = G U^T ; dU = x^T G ; dV = dY^T T
     if (need_T) {   // no stash: recompute T = x U
-        st = gemm({x.p, x.ld, false}, {U.p, U.ld, true}, a.m, a.r, a.k, Tbuf, row_pitch(a.r),
+        st = gemm({x.p, x.ld, false, 0, false, copies && !x.copied}, {U.p, U.ld, true, 0, false, copies && !U.copied}, a.m, a.r, a.k, Tbuf, row_pitch(a.r),
                   pick_splits(a.m, a.r, pick_bn(a.r), a.k), p1, a.stream);
         if (st != PF_OK) return st;
     }
@@ -894,15 +902,23 @@ int linear_bwd(const LinearArgs& a, int* handled) {
             else if (1.1 * pairs < two) order = kPairs;
             if (order != kTwo) { sg = sg_alone; su = su3; sv = sv3; }
         }
-        st = gemm_prepare_any({dY.p, dY.ld, false}, {V.p, V.ld, true}, a.m, a.r, a.n, G, ldG, sg, p1, nullptr, &gg);
-        if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
-        if (st == PF_OK) st = gemm_prepare_any({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
-        if (st == PF_OK && a.dX) st = gemm_prepare({G, ldG, false, 0, true}, {U.p, U.ld, false}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gx);
+        // What need not wait for the launch before: behind copies what was not copied, behind the recomputed T all but T, and behind
+        // G all but G.
+        const bool e_dy = need_T || (copies && !dY.copied), e_v = need_T || (copies && !V.copied);
+        const bool e_t = order == kThree || order == kPairs || (!need_T && copies && !T.copied);
+        const Operand op_dy{dY.p, dY.ld, false, 0, false, e_dy}, op_v{V.p, V.ld, true, 0, false, e_v};
+        const Operand op_dyt{dY.p, dY.ld, true, 0, false, order == kTwo ? e_dy : true}, op_t{T.p, T.ld, true, 0, false, e_t};
+        st = gemm_prepare_any(op_dy, op_v, a.m, a.r, a.n, G, ldG, sg, p1, nullptr, &gg);
+        if (st == PF_OK) st = gemm_prepare_any(op_dyt, op_t, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
+        if (st == PF_OK) st = gemm_prepare_any({x.p, x.ld, true, 0, false, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
+        if (st == PF_OK && a.dX) st = gemm_prepare({G, ldG, false, 0, true}, {U.p, U.ld, false, 0, false, true}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gx);
         if (st != PF_OK) return st;
-        const PairJob j1[2] = {{dY.p, dY.ld, false, 0, V.p, V.ld, true, 0, a.m, a.r, a.n, G, ldG},
-                               {dY.p, dY.ld, true, 0, T.p, T.ld, true, 0, a.n, a.r, a.m, a.dV, a.lddv}};
-        const PairJob j2[2] = {{G, ldG, false, 0, U.p, U.ld, false, 0, a.m, a.k, a.r, a.dX, a.lddx},
-                               {x.p, x.ld, true, 0, G, ldG, true, 0, a.k, a.r, a.m, a.dU, a.lddu}};
+        PairJob j1[2] = {{dY.p, dY.ld, false, 0, V.p, V.ld, true, 0, a.m, a.r, a.n, G, ldG},
+                         {dY.p, dY.ld, true, 0, T.p, T.ld, true, 0, a.n, a.r, a.m, a.dV, a.lddv}};
+        PairJob j2[2] = {{G, ldG, false, 0, U.p, U.ld, false, 0, a.m, a.k, a.r, a.dX, a.lddx},
+                         {x.p, x.ld, true, 0, G, ldG, true, 0, a.k, a.r, a.m, a.dU, a.lddu}};
+        j1[0].a_early = j1[1].a_early = e_dy; j1[0].b_early = e_v; j1[1].b_early = op_t.early;
+        j2[0].b_early = j2[1].a_early = true;
         const GemmLaunch* const l1[2] = {&gg, &gv};
         const GemmLaunch* const l2[2] = {&gx, &gu};
         if (!narrow) {
@@ -933,8 +949,8 @@ int linear_bwd(const LinearArgs& a, int* handled) {
     }
     // dU = x^T G, dV = dY^T T: one launch when their tiles allow
     GemmLaunch gu, gv;
-    st = gemm_prepare_any({x.p, x.ld, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
-    if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true}, {T.p, T.ld, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
+    st = gemm_prepare_any({x.p, x.ld, true, 0, false, true}, {G, ldG, true}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gu);
+    if (st == PF_OK) st = gemm_prepare_any({dY.p, dY.ld, true, 0, false, true}, {T.p, T.ld, true, 0, false, true}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gv);
     if (st != PF_OK) return st;
     keep_slices(a.du_slices, &gu, narrow ? pu : SliceRoom());
     keep_slices(a.dv_slices, &gv, narrow ? pv : SliceRoom());
@@ -994,6 +1010,7 @@ bool grouped_ok(const void* p, int64_t ld, int64_t gs) { return tma_ok(p, ld) &&
 struct StagedGroups {
     const void* p;
     int64_t ld, gs;
+    bool copied = false;
 };
 int stage_groups(const void* p, int64_t ld, int64_t gs, int groups, bool shared, int64_t rows, int64_t cols, char*& scratch,
                  StagedGroups* out, RepackList* list) {
@@ -1002,7 +1019,7 @@ int stage_groups(const void* p, int64_t ld, int64_t gs, int groups, bool shared,
     if (cols % 8 == 0) return 1;          // the workspace query reserves repack room only for ragged widths
     const int64_t ldp = row_pitch(cols), n = shared ? 1 : groups;
     list->jobs[list->count++] = RepackJob{p, ld, scratch, ldp, rows, cols, n, gs};
-    *out = StagedGroups{scratch, ldp, shared ? 0 : rows * ldp};
+    *out = StagedGroups{scratch, ldp, shared ? 0 : rows * ldp, true};
     scratch += align_up(static_cast<size_t>(n) * rows * ldp * 2, 256);
     return 0;
 }
@@ -1061,9 +1078,11 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     }
     GemmLaunch g1, g2;
     const Grouping gt{a.groups, sT, false}, gy{a.groups, a.sy, false};
-    int st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, T, ldT, gp.s1, p1, nullptr, &g1, &gt);
+    const bool copies = repacks.count > 0;      // (what need not wait for the launch before: as in linear_fwd)
+    int st = gemm_prepare({x.p, x.ld, false, x.gs, false, copies && !x.copied}, {U.p, U.ld, true, U.gs, false, copies && !U.copied}, a.m, a.r, a.k, T, ldT, gp.s1,
+                          p1, nullptr, &g1, &gt);
     if (st == PF_OK)
-        st = gemm_prepare({T, ldT, false, sT, true}, {V.p, V.ld, false, V.gs}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, nullptr, &g2, &gy);
+        st = gemm_prepare({T, ldT, false, sT, true}, {V.p, V.ld, false, V.gs, false, true}, a.m, a.n, a.r, a.y, a.ldy, 1, {}, nullptr, &g2, &gy);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
     if (a.T && !stash_direct) {
@@ -1074,6 +1093,7 @@ int linear_grouped_fwd(const GroupedArgs& a, int* handled) {
     if (st == PF_OK) st = launch_prepared(g1, a.stream);
     if (st != PF_OK) return st;
     PairJob jy{T, ldT, false, sT, V.p, V.ld, false, V.gs, a.m, a.n, a.r, a.y, a.ldy, a.sy, a.groups};
+    jy.b_early = true;
     const GemmLaunch* const ly[1] = {&g2};
     return launch_faster(ly, &jy, 1, a.stream);
 }
@@ -1117,13 +1137,16 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
     const Grouping gw{a.groups, sW, false}, gdv{a.groups, a.sdv, false}, gdu{a.groups, a.sdu, false};
     const Grouping gdx{a.groups, shared_x ? 0 : a.sdx, shared_x};
     int st = PF_OK;
-    if (!a.T) st = gemm_prepare({x.p, x.ld, false, x.gs}, {U.p, U.ld, true, U.gs}, a.m, a.r, a.k, Tbuf, ldW, gp.s1, p1, nullptr, &gT, &gw);
+    // What need not wait for the launch before: as in linear_bwd (behind the fused kernel everything but G).
+    const bool copies = repacks.count > 0, e_dy = !a.T || (copies && !dY.copied), e_v = !a.T || (copies && !V.copied), e_t = a.T && copies && !T.copied;
+    if (!a.T) st = gemm_prepare({x.p, x.ld, false, x.gs, false, copies && !x.copied}, {U.p, U.ld, true, U.gs, false, copies && !U.copied}, a.m, a.r, a.k, Tbuf, ldW,
+                                gp.s1, p1, nullptr, &gT, &gw);
     // the recomputed T and G share the slice buffer p1: they are separate launches, one after the other
-    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, false, dY.gs}, {V.p, V.ld, true, V.gs}, a.m, a.r, a.n, Gbuf, ldW, gp.sg, p1, nullptr, &gG, &gw);
-    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, true, dY.gs}, {T.p, T.ld, true, T.gs}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gV, &gdv);
-    if (st == PF_OK) st = gemm_prepare({x.p, x.ld, true, x.gs}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gU, &gdu);
+    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, false, dY.gs, false, e_dy}, {V.p, V.ld, true, V.gs, false, e_v}, a.m, a.r, a.n, Gbuf, ldW, gp.sg, p1, nullptr, &gG, &gw);
+    if (st == PF_OK) st = gemm_prepare({dY.p, dY.ld, true, dY.gs, false, fused || e_dy}, {T.p, T.ld, true, T.gs, false, fused || e_t}, a.n, a.r, a.m, a.dV, a.lddv, sv, pv, nullptr, &gV, &gdv);
+    if (st == PF_OK) st = gemm_prepare({x.p, x.ld, true, x.gs, false, true}, {Gbuf, ldW, true, sW}, a.k, a.r, a.m, a.dU, a.lddu, su, pu, nullptr, &gU, &gdu);
     if (st == PF_OK && a.dX)
-        st = gemm_prepare({Gbuf, ldW, false, sW, true}, {U.p, U.ld, false, U.gs}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gX, &gdx);
+        st = gemm_prepare({Gbuf, ldW, false, sW, true}, {U.p, U.ld, false, U.gs, false, true}, a.m, a.k, a.r, a.dX, a.lddx, 1, {}, nullptr, &gX, &gdx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     if (st != PF_OK) return st;
     *handled = 1;
@@ -1137,16 +1160,19 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled) {
         st = chain_groups(a.groups, a.groups, dY.p, dY.ld, dY.gs, a.m, a.n, V.p, V.ld, V.gs, a.r, U.p, U.ld, U.gs, a.k, a.dX, a.lddx, a.sdx, Gbuf, ldW, sW,
                           false, a.stream);
         if (st != PF_OK) return st;
-        const PairJob jf[2] = {{x.p, x.ld, true, x.gs, Gbuf, ldW, true, sW, a.k, a.r, a.m, a.dU, a.lddu, a.sdu, a.groups},
+        PairJob jf[2] = {{x.p, x.ld, true, x.gs, Gbuf, ldW, true, sW, a.k, a.r, a.m, a.dU, a.lddu, a.sdu, a.groups},
                                {dY.p, dY.ld, true, dY.gs, T.p, T.ld, true, T.gs, a.n, a.r, a.m, a.dV, a.lddv, a.sdv, a.groups}};
+        jf[0].a_early = jf[1].a_early = jf[1].b_early = true;
         const GemmLaunch* const lf[2] = {&gU, &gV};
         return launch_faster(lf, jf, 2, a.stream);
     }
     // launch A: G = dY V and dV = dY^T T (independent of each other); launch B: dU = x^T G and dX = G U^T
-    const PairJob ja[2] = {{dY.p, dY.ld, false, dY.gs, V.p, V.ld, true, V.gs, a.m, a.r, a.n, Gbuf, ldW, sW, a.groups},
+    PairJob ja[2] = {{dY.p, dY.ld, false, dY.gs, V.p, V.ld, true, V.gs, a.m, a.r, a.n, Gbuf, ldW, sW, a.groups},
                            {dY.p, dY.ld, true, dY.gs, T.p, T.ld, true, T.gs, a.n, a.r, a.m, a.dV, a.lddv, a.sdv, a.groups}};
-    const PairJob jb[2] = {{x.p, x.ld, true, x.gs, Gbuf, ldW, true, sW, a.k, a.r, a.m, a.dU, a.lddu, a.sdu, a.groups},
+    PairJob jb[2] = {{x.p, x.ld, true, x.gs, Gbuf, ldW, true, sW, a.k, a.r, a.m, a.dU, a.lddu, a.sdu, a.groups},
                            {Gbuf, ldW, false, sW, U.p, U.ld, false, U.gs, a.m, a.k, a.r, a.dX, a.lddx, shared_x ? 0 : a.sdx, a.groups, shared_x}};
+    ja[0].a_early = ja[1].a_early = e_dy; ja[0].b_early = e_v; ja[1].b_early = e_t;
+    jb[0].a_early = jb[1].b_early = true;
     const GemmLaunch* const la[2] = {&gG, &gV};
     const GemmLaunch* const lb[2] = {&gU, &gX};
     st = launch_faster(la, ja, 2, a.stream);
@@ -1235,10 +1261,11 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     const SliceRoom pu{reinterpret_cast<float*>(a.ws), bu}, pv{reinterpret_cast<float*>(a.ws + bu), bv};
     GemmLaunch gt, gu, gv, gx;
     st = gemm_prepare_any({a.dY, a.O, false}, {a.V, a.R, true}, P, a.R, a.O, dT, a.R, 1, {}, nullptr, &gt);
-    if (st == PF_OK) st = gemm_prepare_any({a.x, a.C, true}, {dT, a.R, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
-    if (st == PF_OK) st = gemm_prepare_any({a.dY, a.O, true}, {T, a.R, true}, a.O, a.R, P, a.dV, a.R, sv, pv, nullptr, &gv);
+    // (the launch before these three writes dT only)
+    if (st == PF_OK) st = gemm_prepare_any({a.x, a.C, true, 0, false, true}, {dT, a.R, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
+    if (st == PF_OK) st = gemm_prepare_any({a.dY, a.O, true, 0, false, true}, {T, a.R, true, 0, false, true}, a.O, a.R, P, a.dV, a.R, sv, pv, nullptr, &gv);
     if (st == PF_OK && a.dX)
-        st = gemm_prepare_any({dT, a.R, false}, {a.U, a.R, false}, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
+        st = gemm_prepare_any({dT, a.R, false}, {a.U, a.R, false, 0, false, true}, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
                      static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1, {}, &cx, &gx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     if (st != PF_OK) return st;

@@ -95,6 +95,7 @@ struct PairJob {
     bool sum_groups = false;
     const void* bias = nullptr;
     int act = 0;
+    bool a_early = false, b_early = false;      // see kEarlyA in pf_tc_prims.cuh
 };
 int gemm_pairs(const PairJob* jobs, int count, int first, cudaStream_t stream);
 

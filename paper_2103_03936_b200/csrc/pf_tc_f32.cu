@@ -56,6 +56,7 @@ struct F32Op {
     const void* p;
     int64_t ld;
     bool mn;                 // stored [K, MN] (the M / N index contiguous)
+    bool early = false;      // see kEarlyA in pf_tc_prims.cuh
 };
 struct F32Conv {
     int mode = 0;            // as F32Params::mode
@@ -233,6 +234,7 @@ bool f32_prepare(const F32Work& w, const F32Op& A, const F32Op& B, float* C, int
     p->rows_tile = w.ct.pixels;
     p->kpix = w.ct.pixels;
     p->ragged = c.C % 32 != 0;
+    p->early = (A.early ? kEarlyA : 0) | (B.early ? kEarlyB : 0);
     return true;
 }
 
@@ -365,7 +367,7 @@ int f32_linear_fwd(const LinearArgs& a, int* handled, size_t room) {
     ws += f32_mat(a.m, a.r, a.tight);
     F32Launch l1, l2;
     if (!f32_prepare(f.t, {x.p, x.ld, false}, {U.p, U.ld, true}, T, ldT, reinterpret_cast<float*>(ws), &l1.ta[0], &l1.tb[0], &l1.p[0]) ||
-        !f32_prepare(f.y, {T, ldT, false}, {V.p, V.ld, false}, static_cast<float*>(a.y), a.ldy, nullptr, &l2.ta[0], &l2.tb[0], &l2.p[0]))
+        !f32_prepare(f.y, {T, ldT, false}, {V.p, V.ld, false, true}, static_cast<float*>(a.y), a.ldy, nullptr, &l2.ta[0], &l2.tb[0], &l2.p[0]))
         return PF_ERR_CUDA;
     if (a.T && !direct) { l1.p[0].C2 = static_cast<float*>(a.T); l1.p[0].ldc2 = a.ldt; }
     l2.p[0].bias = static_cast<const float*>(a.bias);
@@ -412,11 +414,13 @@ int f32_linear_bwd(const LinearArgs& a, int* handled) {
     bool ok = true;
     if (!a.T)
         ok = f32_prepare(b.t, {x.p, x.ld, false}, {U.p, U.ld, true}, reinterpret_cast<float*>(Tbuf), f32_pitch(a.r), p1, &lt.ta[0], &lt.tb[0], &lt.p[0]);
-    ok = ok && f32_prepare(b.g, {dY.p, dY.ld, false}, {V.p, V.ld, true}, G, ldG, p1, &la.ta[0], &la.tb[0], &la.p[0]) &&
-         f32_prepare(b.dv, {dY.p, dY.ld, true}, {T.p, T.ld, true}, static_cast<float*>(a.dV), a.lddv, pv, &la.ta[1], &la.tb[1], &la.p[1]) &&
-         f32_prepare(b.du, {x.p, x.ld, true}, {G, ldG, true}, static_cast<float*>(a.dU), a.lddu, pu, &lb.ta[0], &lb.tb[0], &lb.p[0]);
+    // (the launch before is the recomputed T, or one of an earlier call)
+    const bool early = !a.T;
+    ok = ok && f32_prepare(b.g, {dY.p, dY.ld, false, early}, {V.p, V.ld, true, early}, G, ldG, p1, &la.ta[0], &la.tb[0], &la.p[0]) &&
+         f32_prepare(b.dv, {dY.p, dY.ld, true, early}, {T.p, T.ld, true}, static_cast<float*>(a.dV), a.lddv, pv, &la.ta[1], &la.tb[1], &la.p[1]) &&
+         f32_prepare(b.du, {x.p, x.ld, true, true}, {G, ldG, true}, static_cast<float*>(a.dU), a.lddu, pu, &lb.ta[0], &lb.tb[0], &lb.p[0]);
     if (ok && a.dX)
-        ok = f32_prepare(b.dx, {G, ldG, false}, {U.p, U.ld, false}, static_cast<float*>(a.dX), a.lddx, nullptr, &lb.ta[1], &lb.tb[1], &lb.p[1]);
+        ok = f32_prepare(b.dx, {G, ldG, false}, {U.p, U.ld, false, true}, static_cast<float*>(a.dX), a.lddx, nullptr, &lb.ta[1], &lb.tb[1], &lb.p[1]);
     if (!ok) return PF_ERR_CUDA;
     *handled = 1;
     if (nj > 0 && repack_rows_bf16_multi(jobs, nj, a.stream) != cudaSuccess) return PF_ERR_CUDA;
@@ -455,7 +459,7 @@ int f32_conv_fwd(const ConvArgs& a, int* handled) {
     float* T = static_cast<float*>(a.T ? a.T : a.ws_T);
     F32Launch l1, l2;
     if (!f32_prepare(f.t, {a.x, 0, false}, {a.U, a.R, true}, T, a.R, reinterpret_cast<float*>(a.ws), &l1.ta[0], &l1.tb[0], &l1.p[0]) ||
-        !f32_prepare(f.y, {T, a.R, false}, {a.V, a.R, false}, static_cast<float*>(a.y), a.O, nullptr, &l2.ta[0], &l2.tb[0], &l2.p[0]))
+        !f32_prepare(f.y, {T, a.R, false}, {a.V, a.R, false, true}, static_cast<float*>(a.y), a.O, nullptr, &l2.ta[0], &l2.tb[0], &l2.p[0]))
         return PF_ERR_CUDA;
     *handled = 1;
     const int st = f32_launch(&l1, 1, a.stream);
@@ -480,8 +484,8 @@ int f32_conv_bwd(const ConvArgs& a, int* handled) {
     if (!a.T) ok = f32_prepare(b.t, {a.x, 0, false}, {a.U, a.R, true}, reinterpret_cast<float*>(a.ws_T), a.R, p1, &lt.ta[0], &lt.tb[0], &lt.p[0]);
     ok = ok && f32_prepare(b.g, {a.dY, a.O, false}, {a.V, a.R, true}, dT, a.R, p1, &la.ta[0], &la.tb[0], &la.p[0]) &&
          f32_prepare(b.dv, {a.dY, a.O, true}, {T, a.R, true}, static_cast<float*>(a.dV), a.R, pv, &la.ta[1], &la.tb[1], &la.p[1]) &&
-         f32_prepare(b.du, {a.x, 0, true}, {dT, 0, true}, static_cast<float*>(a.dU), a.R, pu, &lb.ta[0], &lb.tb[0], &lb.p[0]);
-    if (ok && a.dX) ok = f32_prepare(b.dx, {dT, 0, false}, {a.U, a.R, false}, static_cast<float*>(a.dX), a.C, nullptr, &lb.ta[1], &lb.tb[1], &lb.p[1]);
+         f32_prepare(b.du, {a.x, 0, true, true}, {dT, 0, true}, static_cast<float*>(a.dU), a.R, pu, &lb.ta[0], &lb.tb[0], &lb.p[0]);
+    if (ok && a.dX) ok = f32_prepare(b.dx, {dT, 0, false}, {a.U, a.R, false, true}, static_cast<float*>(a.dX), a.C, nullptr, &lb.ta[1], &lb.tb[1], &lb.p[1]);
     if (!ok) return PF_ERR_CUDA;
     *handled = 1;
     int st = PF_OK;

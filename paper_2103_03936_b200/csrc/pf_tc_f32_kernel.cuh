@@ -72,6 +72,7 @@ struct F32Params {
     int cv_wblk;             // dU: blocks of cv_bw pixels per image row
     int rows_tile, kpix;
     int ragged;              // mode 3: C is not a multiple of 32, tmB is [taps][C][R]
+    int early;               // kEarlyA | kEarlyB
 };
 
 struct F32Launch {
@@ -361,8 +362,11 @@ __device__ __forceinline__ void f32_tile(const CUtensorMap& tmA, const CUtensorM
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();                 // everything above overlapped the previous kernel's tail
-    pdl_launch_dependents();
+    const bool ahead = (warp == 0 && (p.early & kEarlyA)) || (warp == 18 && (p.early & kEarlyB));
+    if (!ahead) {               // everything above overlapped the previous kernel's tail, as do the loads of an early operand
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     const uint32_t tmem = ctl->tmem_base;
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
 

@@ -54,6 +54,7 @@ struct GemmParams {
     int nkb_total;           // k-blocks of the whole contraction
     float keep_a;            // plain products: how L2 treats A (see l2_policy)
     int independent;         // 1: reads nothing the preceding kernel of the stream writes (see gemm_tile)
+    int early;               // kEarlyA | kEarlyB: the operands of which that is true
     // Grouped products (several problems of one shape in a launch): tmA / tmB are 3-D maps whose outermost
     // coordinate is the group (a shared operand has one group only), outputs of group g start g * c_gstride
     // elements after C.  kb_per_group > 0 instead makes the group part of the CONTRACTION: k-block kb reads
@@ -230,8 +231,10 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     // it does not wait for that kernel: its blocks run beside it on SMs that kernel leaves free.  (Every
     // kernel of this library lets its successor start only after its own wait has returned, i.e. once
     // everything older in the stream is complete, so older results are safe to read.)
-    if (!p.independent) pdl_wait();     // everything above overlapped the previous kernel's tail
-    pdl_launch_dependents();
+    // The same holds for a single operand (p.early): its producer fills the ring beside the previous kernel's tail.
+    const bool ahead = p.independent || (warp == 0 && (p.early & kEarlyA)) || (warp == 6 && (p.early & kEarlyB));
+    if (!ahead) pdl_wait();             // everything above overlapped the previous kernel's tail
+    if (!ahead || p.independent) pdl_launch_dependents();
     const uint32_t tmem_base = ctl->tmem_base;
 
     // Producers and MMA issuer are each one thread chosen with elect.sync that runs its whole role
@@ -612,8 +615,11 @@ __device__ __forceinline__ void run_tiles(const CUtensorMap& tmA, const CUtensor
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
-    pdl_launch_dependents();
+    const bool ahead = (warp == 0 && (p.early & kEarlyA)) || (warp == 6 && (p.early & kEarlyB));      // (see gemm_tile)
+    if (!ahead) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     const uint32_t tmem_base = ctl->tmem_base;
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
 

@@ -63,6 +63,7 @@ struct PairProduct {
     long long ldc, c_gstride;
     const void* bias;        // C = act(A B + bias), bias [N] in bf16 or null
     int act;
+    int early;               // kEarlyA | kEarlyB
 };
 // Up to three products.  Their tiles form two lists, the long ones first: list 0 (products 0 .. first - 1) is dealt
 // to the pairs in turn; list 1 (the rest) is dealt so that the pairs which got one tile of list 0 less start `delay`
@@ -236,8 +237,10 @@ tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
     __syncthreads();
     tc_fence_after();
     cluster_sync_all();
-    pdl_wait();
-    pdl_launch_dependents();
+    if (warp != 0 && warp != 10) {       // (the producers wait before the first operand that the previous kernel may have written)
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     const uint32_t tmem_base = ctl->tmem_base;
 
     if (warp == 0 || warp == 10) {
@@ -248,11 +251,15 @@ tc_gemm_pair_kernel(const __grid_constant__ PairLaunch L) {
             const uint32_t empty0 = smem_u32(&ctl->empty[0]), full0 = smem_u32(&ctl->full[0]);
             const uint32_t dst0 = smem_u32(tiles) + (do_a ? 0u : kHalfBytes);
             uint32_t s = 0, ph = 1, dst = dst0;
-            bool ok = true;
+            bool ok = true, waited = false;
             PairWalk walk(pair, npairs);
             int q, t;
             while (ok && walk.next<kForm == 0>(L, q, t)) {
                 const PairProduct& p = kForm == 0 ? L.p[0] : L.p[q];
+                if (!waited && !(p.early & (do_a ? kEarlyA : kEarlyB))) {
+                    pdl_wait();
+                    waited = true;
+                }
                 const CUtensorMap* map = kForm == 0 ? (do_a ? &L.ta[0] : &L.tb[0]) : (do_a ? &L.ta[q] : &L.tb[q]);
                 const int nkb = p.nkb;
                 int g = 0;
@@ -468,6 +475,7 @@ int gemm_pairs(const PairJob* jobs, int count, int first, cudaStream_t stream) {
         p.tiles_m = static_cast<int>(tiles_m); p.tiles_mn = static_cast<int>(tiles_mn); p.tiles = static_cast<int>(tiles);
         p.C = j.C; p.ldc = j.ldc; p.c_gstride = j.c_gs;
         p.bias = j.bias; p.act = j.act;
+        p.early = (j.a_early ? kEarlyA : 0) | (j.b_early ? kEarlyB : 0);
         if (i < count) totals[i < first ? 0 : 1] += tiles;
         bool ok;
         if (grouped) {

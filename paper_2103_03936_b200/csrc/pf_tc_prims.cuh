@@ -32,6 +32,9 @@ __device__ __forceinline__ bool elect_one() {
 // its own prologue early.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Operands of a product that were complete before the preceding kernel of the stream got past its own wait, i.e. that
+// neither that kernel writes nor a caller's kernel before it can still be writing: their producers do not wait for it.
+constexpr int kEarlyA = 1, kEarlyB = 2;
 
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
