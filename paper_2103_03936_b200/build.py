@@ -16,7 +16,7 @@ OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpf.so")
 NATIVE = os.path.join(PKG, "_pf_native.so")
 NATIVE_KEY = os.path.join(OBJ, "_pf_native.key")      # what _pf_native.so was built against
-SOURCES = ["pf_api.cu", "pf_simt.cu", "pf_small.cu", "pf_pack.cu", "pf_tc.cu", "pf_tc_conv.cu", "pf_tc_runs.cu", "pf_tc_any.cu", "pf_tc_conv_res.cu", "pf_tc_chain.cu", "pf_tc_chain_multi.cu", "pf_tc_chain_act.cu", "pf_tc_chain_conv.cu", "pf_tc_chain_group.cu", "pf_tc_chain_l2.cu", "pf_tc_pair.cu", "pf_tc_f32.cu", "pf_tc_f32_conv.cu", "pf_static.cu"]
+SOURCES = ["pf_api.cu", "pf_simt.cu", "pf_small.cu", "pf_pack.cu", "pf_tc.cu", "pf_tc_conv.cu", "pf_tc_runs.cu", "pf_tc_any.cu", "pf_tc_conv_res.cu", "pf_tc_conv_bwd.cu", "pf_tc_chain.cu", "pf_tc_chain_multi.cu", "pf_tc_chain_act.cu", "pf_tc_chain_conv.cu", "pf_tc_chain_group.cu", "pf_tc_chain_l2.cu", "pf_tc_pair.cu", "pf_tc_f32.cu", "pf_tc_f32_conv.cu", "pf_static.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
 
 

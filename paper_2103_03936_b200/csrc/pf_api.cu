@@ -687,7 +687,7 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         int nj = 0;
         if (su_info.partial)
             jobs[nj++] = SliceSums{su_info.partial, user_dU, R, static_cast<int>(Keff), R, su_info.splits, su_info.bn,
-                                   su_info.tiles_x, su_info.tiles_y, g_f32, g_acc, su_info.conv_c};
+                                   su_info.tiles_x, su_info.tiles_y, g_f32, g_acc, su_info.conv_c, su_info.conv_blks, su_info.tail, su_info.tail_splits};
         else
             PF_CUDA(grad_combine(user_dU, R, gdtype, dU, R, dtype, Keff, R, g_acc, stream));
         if (sv_info.partial)

@@ -1222,7 +1222,7 @@ size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, in
     size_t bu, bv;
     conv_splits(c, O, &su, &sv);
     conv_partial_bytes(c, O, su, sv, &bu, &bv);
-    return bu + bv;
+    return std::max(bu + bv, conv_flat_bwd_workspace(N, H, W, C, R, O, kh, kw, stride, pad));
 }
 
 int conv_fwd(const ConvArgs& a, int* handled) {
@@ -1247,6 +1247,16 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     int st;
     const void* T = a.T ? a.T : a.ws_T;
     void* dT = a.ws_G;
+    auto recompute = [&] {   // the thin convolution (phase 1 of the forward only)
+        const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
+        return chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
+    };
+    if (conv_flat_bwd_pays(a) && aligned16(a.dU) && aligned16(a.dV)) {
+        st = a.T ? PF_OK : recompute();
+        if (st == PF_ERR_UNSUPPORTED) return PF_OK;
+        *handled = 1;
+        return st == PF_OK ? conv_flat_bwd(a, T) : st;
+    }
     // Every product is prepared (tensor maps, geometry; nothing launched) before the call is
     // accepted, so a shape that one of them cannot take still reaches the FMA kernels.
     // dU[tap] = shifted x^T dT ; dV = dY^T T   (reductions over all output pixels, split across CTAs)
@@ -1276,9 +1286,8 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         gt.grid = dim3(static_cast<unsigned>(ceil_div(gt_tiles, std::min<int64_t>(4, ceil_div(gt_tiles, 2 * num_sms())))));
         gt.p.num_stages = pick_stages(gt.bn, gt.grid.x, true);
     }
-    if (!a.T) {   // recompute the thin convolution (phase 1 of the forward only)
-        const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
-        st = chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
+    if (!a.T) {
+        st = recompute();
         if (st == PF_ERR_UNSUPPORTED) return PF_OK;
         if (st != PF_OK) return st;
     }

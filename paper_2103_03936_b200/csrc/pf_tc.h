@@ -30,6 +30,8 @@ struct LinearArgs {
         const float* partial = nullptr;
         int splits = 0, bn = 0, tiles_x = 0, tiles_y = 0;
         int conv_c = 0;     // > 0: tiles are pairs of 64-channel blocks of a [taps][conv_c] row index
+        int conv_blks = 0;  // > 0: that many 64-channel blocks per tap (else the ones that exist)
+        int tail = 0, tail_splits = 0;     // tail > 0: from this tile on there are tail_splits slices
     };
     Slices* du_slices = nullptr;
     Slices* dv_slices = nullptr;
@@ -138,6 +140,10 @@ int f32_conv_bwd(const ConvArgs& a, int* handled);
 unsigned int* split_counters();
 // 3 x 3, stride-1 convolutions on resident image windows (pf_tc_conv_res.cu); PF_ERR_UNSUPPORTED outside their envelope.
 int conv_res_fwd(const ConvArgs& a);
+// Their backward (pf_tc_conv_bwd.cu), where `conv_flat_bwd_pays`; T is x U, a.ws_G takes dT.
+bool conv_flat_bwd_pays(const ConvArgs& a);
+size_t conv_flat_bwd_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad);
+int conv_flat_bwd(const ConvArgs& a, const void* T);
 int conv_fwd(const ConvArgs& a, int* handled);
 int conv_bwd(const ConvArgs& a, int* handled);
 

@@ -13,6 +13,7 @@
 #define kMaxStages kChainMaxStages      // (each of the two headers has one of its own)
 #include "pf_tc_chain_kernel.cuh"
 #undef kMaxStages
+#include "pf_tc_conv_flat.cuh"
 #include "pf_tc_f32_kernel.cuh"
 #include "pf_tc_gemm_kernel.cuh"
 
@@ -61,6 +62,19 @@ void check(const pf::tc::F32Params& p) {
     if (p.mode == 0 || p.mode == 2) writes("result of an fp32 product", address(p.C), matrix(p.M, p.N, p.ldc, 4));
     if (p.C2) writes("second copy of an fp32 result", address(p.C2), matrix(p.M, p.N, p.ldc2, 4));
 }
+constexpr uint64_t kSlice = 128 * 64 * 4;
+void check(const pf::tc::DtDvParams& p, unsigned blocks) {
+    writes("dT of a convolution", address(p.dT), matrix(p.rows, p.R, p.R, 2));
+    writes("slices of dV of a convolution", address(p.partial), p.pairs * blocks * kSlice);
+}
+void check(const pf::tc::DuParams& p) {
+    writes("slices of dU of a convolution", address(p.partial), static_cast<uint64_t>(6 * p.split[0] + 3 * p.split[1]) * p.tb * kSlice);
+    writes("dV of a convolution", address(p.sum.out), matrix(p.sum.rows, p.sum.R, p.sum.R, 2));
+}
+void check(const pf::tc::DxParams& p) {
+    if (p.tiles > 0) writes("dX of a convolution", address(p.out), matrix(static_cast<int64_t>(p.f.N) * p.f.H * p.f.W, p.C, p.C, 2));
+    writes("dU of a convolution", address(p.sum.out), matrix(static_cast<int64_t>(9) * p.sum.rows, p.sum.R, p.sum.R, 2));
+}
 void check(const pf::SimtGemm& g) {
     const int64_t size = g.dtype == PF_BF16 ? 2 : 4;
     if (g.splits > 1) inside("slices of an FMA product", address(g.partial), static_cast<uint64_t>(g.splits) * g.M * g.N * 4);
@@ -101,6 +115,12 @@ void launched(const void* kernel, unsigned blocks, void** args) {
         const pf::tc::F32Launch& l = arg<pf::tc::F32Launch>(args, 0);
         for (int i = 0; i < 3; ++i)
             if (i == 0 || l.end[i] > l.end[i - 1]) check(l.p[i]);
+    } else if (is("tc_conv_dt_dv_kernel")) {
+        check(arg<pf::tc::DtDvParams>(args, 3), blocks);
+    } else if (is("tc_conv_du_kernel")) {
+        check(arg<pf::tc::DuParams>(args, 2));
+    } else if (is("tc_conv_dx_kernel")) {
+        check(arg<pf::tc::DxParams>(args, 2));
     } else if (is("simt_gemm_kernel")) {
         check(arg<pf::SimtGemm>(args, 0));
     }

@@ -256,6 +256,33 @@ def test_resident_image_windows(N, H, W, C, R, O):
     run_conv(wl.ConvCase("res", N, H, W, C, R, O, wl.BF16, 95))
 
 
+@pytest.mark.parametrize("N,H,W,C,R,O", [
+    (30, 16, 16, 320, 40, 72),       # 16 divides the width: dU's blocks take the image's columns; an odd number of channel blocks; half a tile of dY
+    (8, 32, 48, 264, 56, 136),       # blocks of one row of 48; a ragged channel block
+    (300, 7, 7, 256, 40, 64),        # blocks of whole images
+    (120, 9, 13, 136, 24, 136),      # rows that do not divide into blocks
+    (8, 33, 63, 72, 24, 72),         # the widest image; one block of channels, ragged
+    (900, 3, 4, 512, 40, 24),        # windows of dX in boxes of whole images
+    (16, 32, 32, 512, 40, 512),      # the widest y
+    (60, 31, 15, 192, 48, 96),
+    (60, 28, 28, 128, 8, 128),       # one block of channels, the smallest rank
+])
+def test_flat_backward(N, H, W, C, R, O):
+    """3 x 3, stride-1 backwards in three launches that read their images once: edges of their blocks, with and without
+    stash and dX; gradients in fp32 are the sums that the plain ones are rounded from."""
+    c = wl.ConvCase("flat", N, H, W, C, R, O, wl.BF16, 97)
+    run_conv(c)
+    run_conv(c, stash=False, need_dX=False)
+    d = c.generate()
+    x, U, V, dY = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V", "dY"))
+    before = pf.pf_launch_count()
+    _, dU0, dV0 = pf.pf_lowrank_conv_bwd(x, U, V, dY)
+    assert pf.pf_launch_count() - before == 4         # (x U once more)
+    _, dU1, dV1 = pf.pf_lowrank_conv_bwd(x, U, V, dY, grads_f32=True)
+    torch.cuda.synchronize()
+    assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
+
+
 @pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad", [
     (163, 16, 16, 64, 16, 64, 3, 1, 1),      # two dX tiles per block, a last block with one
     (41, 30, 30, 136, 24, 40, 3, 2, 1),      # eight per block, two column tiles (one ragged), all classes in a block
