@@ -549,7 +549,7 @@ ConvWs conv_ws(int N, int H, int W, int C, int R, int O, int kh, int kw, int str
     size_t off = 0;
     w.off_T = off; off += align_up(static_cast<size_t>(w.P) * R * s, 256);
     if (bwd) {
-        w.off_dT = off; off += align_up(static_cast<size_t>(w.P) * R * s, 256);
+        w.off_dT = off; off += align_up(static_cast<size_t>(w.P) * (dtype == PF_BF16 ? tc::conv_dt_pitch(R) : R) * s, 256);
         const int64_t Keff = static_cast<int64_t>(kh) * kw * C;
         w.splits_dU = simt_pick_splits(Keff, R, w.P);
         w.splits_dV = simt_pick_splits(O, R, w.P);

@@ -240,12 +240,12 @@ int gemm_prepare(const Operand& A, const Operand& B, int64_t M, int64_t N, int64
     ConvTiling ct;
     if (cv && cv->mode == 1) {
         ct = conv_dx_tiling(*cv);
-        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->Ho, cv->Wo, cv->R, static_cast<int>(ceil_div(cv->W, cv->stride)), ct.bh, ct.nb, 1);
+        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->Ho, cv->Wo, cv->R, static_cast<int>(ceil_div(cv->W, cv->stride)), ct.bh, ct.nb, 1, A.ld);
         okb = cached_map_2d(&tb, B.p, static_cast<int64_t>(cv->kh) * cv->kw * cv->C, cv->R, B.ld, bn);   // rows past a tap's C: columns past N
     } else if (cv && cv->mode == 2) {
         ct = conv_k_tiling(*cv);
-        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->H, cv->W, cv->C, cv->Wo, ct.bh, ct.nb, cv->stride);
-        okb = cached_map_nhwc(&tb, B.p, cv->N, cv->Ho, cv->Wo, cv->R, cv->Wo, ct.bh, ct.nb, 1);
+        oka = cached_map_nhwc(&ta, A.p, cv->N, cv->H, cv->W, cv->C, cv->Wo, ct.bh, ct.nb, cv->stride, A.ld);
+        okb = cached_map_nhwc(&tb, B.p, cv->N, cv->Ho, cv->Wo, cv->R, cv->Wo, ct.bh, ct.nb, 1, B.ld);
     } else if (gr) {
         const int64_t ga = A.gs == 0 ? 1 : groups, gb = B.gs == 0 ? 1 : groups;
         oka = A.mn_major ? cached_map_3d(&ta, A.p, ga, K, M, A.ld, A.gs, 64) : cached_map_3d(&ta, A.p, ga, M, K, A.ld, A.gs, kBM);
@@ -1213,6 +1213,17 @@ void conv_partial_bytes(const ConvA& c, int O, int su, int sv, size_t* bytes_u, 
 }
 }  // namespace
 
+// Elements from one pixel of dT to the next: rows of 24, 40, 48, 56 or 80 ranks would straddle 128-byte lines, and the products that
+// read them once per tap take two requests for most.  (Ranks whose rows divide a line, or are made of lines, lie as they are.)  Backward of
+// 16 x 14 x 14, 160 -> 40 -> 160 18.9 -> 16.6 us, of 8 x 28 x 28, 192 -> 48 -> 192 18.9 -> 16.6, stride 2 of 64 x 14 x 14, 256 -> 72 -> 256 22.0 -> 19.9.
+int64_t conv_dt_pitch(int64_t R) { return R % 64 == 0 || 64 % R == 0 ? R : (R + 63) / 64 * 64; }
+// dX reads U once per tile, so for many pixels it too is copied to that pitch, beside the launch that makes dT (64 x 28 x 28: 320 -> 80 ->
+// 320 110.1 -> 99.8 us, 320 -> 40 -> 320 90.6 -> 79.4; 8 x 28 x 28 of it 33.2 -> 34.2; rows of 96 bytes take no harm: 192 -> 48 -> 192 46.9 -> 48.3).
+static size_t conv_factor_copy(int64_t pixels, int64_t Keff, int64_t R) {
+    if (pixels < 20000 || conv_dt_pitch(R) == R || R % 8 || (R < 64 && R % 16 == 0)) return 0;
+    return align_up(static_cast<size_t>(Keff) * conv_dt_pitch(R) * 2, 256);
+}
+
 size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad,
                             bool bwd) {
     const int Ho = (H + 2 * pad - kh) / stride + 1, Wo = (W + 2 * pad - kw) / stride + 1;
@@ -1222,7 +1233,7 @@ size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, in
     size_t bu, bv;
     conv_splits(c, O, &su, &sv);
     conv_partial_bytes(c, O, su, sv, &bu, &bv);
-    return std::max(bu + bv, conv_flat_bwd_workspace(N, H, W, C, R, O, kh, kw, stride, pad));
+    return conv_factor_copy(static_cast<int64_t>(N) * Ho * Wo, static_cast<int64_t>(kh) * kw * C, R) + std::max(bu + bv, conv_flat_bwd_workspace(N, H, W, C, R, O, kh, kw, stride, pad));
 }
 
 int conv_fwd(const ConvArgs& a, int* handled) {
@@ -1251,11 +1262,21 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
         return chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
     };
+    const int64_t ldt = conv_dt_pitch(a.R);
+    const size_t copy_bytes = conv_factor_copy(P, Keff, a.R);
+    const bool copy = a.dX && copy_bytes > 0;      // of U for dX; the launch that makes dT runs beside it
+    char* const ws = a.ws + copy_bytes;
+    const Operand U{copy ? a.ws : a.U, copy ? ldt : a.R, false, 0, false, true};
+    auto copy_factor = [&] {
+        const RepackJob job{a.U, a.R, a.ws, ldt, Keff, a.R};
+        return !copy || repack_rows_bf16_multi(&job, 1, a.stream) == cudaSuccess ? PF_OK : PF_ERR_CUDA;
+    };
     if (conv_flat_bwd_pays(a) && aligned16(a.dU) && aligned16(a.dV)) {
         st = a.T ? PF_OK : recompute();
         if (st == PF_ERR_UNSUPPORTED) return PF_OK;
         *handled = 1;
-        return st == PF_OK ? conv_flat_bwd(a, T) : st;
+        if (st == PF_OK) st = copy_factor();
+        return st == PF_OK ? conv_flat_bwd(a, T, U.p, U.ld, ws, copy) : st;
     }
     // Every product is prepared (tensor maps, geometry; nothing launched) before the call is
     // accepted, so a shape that one of them cannot take still reaches the FMA kernels.
@@ -1268,14 +1289,14 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     conv_splits(cu, a.O, &su, &sv);
     size_t bu, bv;
     conv_partial_bytes(cu, a.O, su, sv, &bu, &bv);
-    const SliceRoom pu{reinterpret_cast<float*>(a.ws), bu}, pv{reinterpret_cast<float*>(a.ws + bu), bv};
+    const SliceRoom pu{reinterpret_cast<float*>(ws), bu}, pv{reinterpret_cast<float*>(ws + bu), bv};
     GemmLaunch gt, gu, gv, gx;
-    st = gemm_prepare_any({a.dY, a.O, false}, {a.V, a.R, true}, P, a.R, a.O, dT, a.R, 1, {}, nullptr, &gt);
+    st = gemm_prepare_any({a.dY, a.O, false, 0, false, copy}, {a.V, a.R, true, 0, false, copy}, P, a.R, a.O, dT, ldt, 1, {}, nullptr, &gt);
     // (the launch before these three writes dT only)
-    if (st == PF_OK) st = gemm_prepare_any({a.x, a.C, true, 0, false, true}, {dT, a.R, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
+    if (st == PF_OK) st = gemm_prepare_any({a.x, a.C, true, 0, false, true}, {dT, ldt, true}, Keff, a.R, P, a.dU, a.R, su, pu, &cu, &gu);
     if (st == PF_OK) st = gemm_prepare_any({a.dY, a.O, true, 0, false, true}, {T, a.R, true, 0, false, true}, a.O, a.R, P, a.dV, a.R, sv, pv, nullptr, &gv);
     if (st == PF_OK && a.dX)
-        st = gemm_prepare_any({dT, a.R, false}, {a.U, a.R, false, 0, false, true}, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
+        st = gemm_prepare_any({dT, ldt, false}, U, static_cast<int64_t>(a.N) * a.H * a.W, a.C,
                      static_cast<int64_t>(a.kh) * a.kw * a.R, a.dX, a.C, 1, {}, &cx, &gx);
     if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     if (st != PF_OK) return st;
@@ -1292,6 +1313,8 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         if (st != PF_OK) return st;
     }
     *handled = 1;
+    st = copy_factor();
+    if (st != PF_OK) return st;
     const bool narrow = narrow_reductions(conv_du_tiles(a.kh, a.kw, a.C) * kBM, a.O, a.R);
     keep_slices(a.du_slices, &gu, narrow ? pu : SliceRoom(), a.C);
     keep_slices(a.dv_slices, &gv, narrow ? pv : SliceRoom());

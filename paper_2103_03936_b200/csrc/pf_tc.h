@@ -143,9 +143,10 @@ int conv_res_fwd(const ConvArgs& a);
 // Their backward (pf_tc_conv_bwd.cu), where `conv_flat_bwd_pays`; T is x U, a.ws_G takes dT.
 bool conv_flat_bwd_pays(const ConvArgs& a);
 size_t conv_flat_bwd_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad);
-int conv_flat_bwd(const ConvArgs& a, const void* T);
+int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early);     // early: the launch before copies U, nothing else
 int conv_fwd(const ConvArgs& a, int* handled);
-int conv_bwd(const ConvArgs& a, int* handled);
+int conv_bwd(const ConvArgs& a, int* handled);      // a.ws_G: conv_dt_pitch(R) elements per pixel
+int64_t conv_dt_pitch(int64_t R);
 
 }  // namespace tc
 

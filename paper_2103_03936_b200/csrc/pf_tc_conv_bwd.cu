@@ -69,8 +69,10 @@ tc_conv_dt_dv_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_wait();
-    pdl_launch_dependents();
+    if (warp != 0 || !p.early) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     const uint32_t tmem = ctl->tmem_base;
 
     if (warp == 0) {
@@ -166,7 +168,7 @@ tc_conv_dt_dv_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_const
             for (int e = 0; e < 8; ++e) {
                 const int rr = e * 4 + sub;
                 const uint4 w = ld_shared_v4(panel + static_cast<uint32_t>(rr) * 128u + ((static_cast<uint32_t>(piece) ^ static_cast<uint32_t>(rr & 7)) << 4));
-                if (row0 + rr < p.rows && piece * 8 < p.R) *reinterpret_cast<uint4*>(p.dT + static_cast<size_t>(row0 + rr) * p.R + piece * 8) = w;
+                if (row0 + rr < p.rows && piece * 8 < p.R) *reinterpret_cast<uint4*>(p.dT + static_cast<size_t>(row0 + rr) * p.ldt + piece * 8) = w;
             }
             __syncwarp();
         }
@@ -574,34 +576,34 @@ size_t conv_flat_bwd_workspace(int N, int H, int W, int C, int R, int O, int kh,
     return flat_bwd_plan(N, H, W, C, R, O, kh, kw, stride, pad, &b) ? b.bytes_u + b.bytes_v : 0;
 }
 
-// Expected microseconds of the launches here and of those that fetch pixels per tap, over the pixels and channels, fitted to 120
-// backwards of 1960 to 131072 pixels, 64 to 512 channels and ranks of 16 to 64 (cold L2; most within 7 and 10 %).  Rows of dT that straddle
-// 128-byte lines, of 24, 40, 48 or 56 ranks, are what those suffer from: 64 x 28 x 28, 160 -> 40 -> 160 100.7 us there, 63.3 here; 192 -> 48 -> 192
-// 62.5 and 46.3; 192 -> 64 -> 192 46.2 and 48.3; 128 x 32 x 32, 256 -> 64 -> 256 111.6 and 89.4; 64 x 14 x 14 of it 22.1 and 29.7: the sums of the slices
-// and three launches' starts cost 10 to 20 us.  The rule picks a form more than 3 % slower than the other for three of the 120.
+// Against the launches that fetch pixels per tap (old / here, cold L2).  Rows of dT and U that straddle lines are what those suffer from, so
+// at ranks of 24, 40 or 56 these pay early: 160 -> 40 -> 160 of 6272 pixels 23.2 / 25.9 us, 12544 36.4 / 31.3, 50176 96.5 / 59.8; 128 -> 40 -> 128
+// of 12544 24.0 / 24.9, 25088 37.5 / 29.7; 64 -> 24 -> 64 of 12544 20.1 / 24.6, 25088 30.9 / 30.2.  At 48: 192 -> 48 -> 192 of 12544 23.2 / 28.1, 25088
+// 36.0 / 32.4; 128 -> 48 -> 256 of 25088 26.7 / 30.4, 50176 41.2 / 40.7.  Elsewhere the starts of three launches and the sums of the slices (10 to 20
+// us) want more: 256 -> 64 -> 256 of 25088 31.5 / 34.4, 65536 60.2 / 55.3, 131072 111.6 / 89.4; 128 -> 32 -> 128 of 25088 23.7 / 26.5, 100352 63.4 / 50.9; an
+// expected time decides, fitted to 77 such backwards (most within 7 and 9 %; three of them more than 3 % slower than the better form).
 bool conv_flat_bwd_pays(const ConvArgs& a) {
     FlatBwd b;
     if (!flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b)) return false;
     const double c = a.C / 100.0, p = static_cast<double>(a.N) * a.H * a.W / 1000.0, pc = p * c, po = p * a.O / 100.0;
-    if (p < 2.0) return false;
-    if (a.R % 16 != 0 && 64 % a.R != 0) return 15.1 + 3.4 * c + 0.39 * p + 0.07 * pc + 0.11 * po < 0.95 * (12.4 + 0.19 * c + 0.75 * p + 0.67 * pc - 0.19 * po);
-    if (64 % a.R != 0) return 15.8 + 3.23 * c + 0.06 * p + 0.15 * pc + 0.07 * po < 0.95 * (13.9 - 0.92 * c + 0.12 * p + 0.51 * pc - 0.05 * po);
-    return 14.6 + 3.58 * c + 0.23 * p + 0.07 * pc + 0.05 * po < (a.R > 32 ? 0.9 : 1.05) * (12.35 + 0.07 * c + 0.16 * p + 0.19 * pc + 0.07 * po);
+    if (64 % a.R != 0) return a.R % 16 != 0 ? p >= (a.C >= 160 ? 11.0 : a.C >= 96 ? 16.0 : 25.0) : p >= (a.C >= 160 ? 20.0 : 50.0);
+    return p >= 2.0 && 14.6 + 3.58 * c + 0.23 * p + 0.07 * pc + 0.05 * po < (a.R > 32 ? 0.9 : 1.05) * (12.35 + 0.07 * c + 0.16 * p + 0.19 * pc + 0.07 * po);
 }
 
 // T: the stash, or x * U as a launch before left it.
-int conv_flat_bwd(const ConvArgs& a, const void* T) {
+int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early) {
     FlatBwd b;
     if (encode_fn() == nullptr || !flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b)) return PF_ERR_UNSUPPORTED;
     const int64_t P = static_cast<int64_t>(a.N) * a.H * a.W;
-    float* pu = reinterpret_cast<float*>(a.ws);
-    float* pv = reinterpret_cast<float*>(a.ws + b.bytes_u);
+    const int64_t ldt = conv_dt_pitch(a.R);
+    float* pu = reinterpret_cast<float*>(ws);
+    float* pv = reinterpret_cast<float*>(ws + b.bytes_u);
     unsigned int* status = device_status_ptr();
     CUtensorMap y, t, v, ux, ut, xa, xb;
     const bool ok = cached_map_2d(&y, a.dY, P, a.O, a.O, 128) && cached_map_2d(&t, T, P, a.R, a.R, 128) && cached_map_2d(&v, a.V, a.O, a.R, a.R, 64) &&
                     cached_map_nhwc(&ux, a.x, a.N, a.H, a.W, a.C, b.wx, b.ct.bh, b.ct.nb, 1) &&
-                    cached_map_nhwc(&ut, a.ws_G, a.N, a.H, a.W, a.R, a.W + 1, b.ct.bh, b.ct.nb, 1) && window_map(&xa, b.f, a.ws_G, a.R) &&
-                    cached_map_2d(&xb, a.U, static_cast<int64_t>(9) * a.C, a.R, a.R, 128);
+                    cached_map_nhwc(&ut, a.ws_G, a.N, a.H, a.W, a.R, a.W + 1, b.ct.bh, b.ct.nb, 1, ldt) && window_map(&xa, b.f, a.ws_G, a.R, ldt) &&
+                    cached_map_2d(&xb, U, static_cast<int64_t>(9) * a.C, a.R, ldu, 128);
     if (!ok) return PF_ERR_CUDA;
     DtDvParams sp = {};
     sp.rows = static_cast<int>(P); sp.O = a.O; sp.R = a.R;
@@ -609,6 +611,8 @@ int conv_flat_bwd(const ConvArgs& a, const void* T) {
     sp.panels = static_cast<int>(ceil_div(a.O, 64)); sp.pairs = b.pairs;
     sp.num_stages = b.v_stages;
     sp.dT = reinterpret_cast<__nv_bfloat16*>(a.ws_G);
+    sp.ldt = static_cast<int>(ldt);
+    sp.early = early;
     sp.partial = pv; sp.status = status;
     DuParams up = {};
     up.C = a.C; up.tb = b.tb;

@@ -87,6 +87,8 @@ struct DtDvParams {
     int panels, pairs;           // of 64 and 128 columns of dY
     int num_stages;
     __nv_bfloat16* dT;
+    int ldt;                     // elements of a row of dT
+    int early;                   // the launch before writes none of the operands
     float* partial;              // slices of dV: [tile][block][quadrant][4-column group][row][4]
     unsigned int* status;
 };
@@ -125,8 +127,8 @@ inline FlatImage flat_image(const ConvArgs& a) {
 }
 // Positions of a window that covers `span` consecutive positions wherever they start.
 inline int window_rows(const FlatImage& f, int span) { return ((span + f.unit_rows - 2) / f.unit_rows + 1) * f.unit_rows; }
-inline bool window_map(CUtensorMap* map, const FlatImage& f, const void* p, int channels) {
-    return cached_map_nhwc(map, p, f.N, f.H, f.W, channels, f.Wp, f.per_image ? f.Hp : 1, 1, 1);
+inline bool window_map(CUtensorMap* map, const FlatImage& f, const void* p, int channels, int64_t ld = 0) {
+    return cached_map_nhwc(map, p, f.N, f.H, f.W, channels, f.Wp, f.per_image ? f.Hp : 1, 1, 1, ld);
 }
 // A persistent grid of equally loaded CTAs.
 inline int even_grid(int tiles) { return static_cast<int>(ceil_div(tiles, ceil_div(tiles, num_sms()))); }

@@ -99,15 +99,16 @@ inline bool cached_map_3d(CUtensorMap* map, const void* p, int64_t groups, int64
 
 // 4-D bf16 tensor map over an NHWC image [N, H, W, C]: boxes are 64 channels x box_w x box_h pixels of box_n
 // images (box_w * box_h * box_n rows of 128 bytes in shared memory, pixel-major), taking every stride-th
-// pixel along W and H; coordinates may start outside the image (zero padding of the convolution),
+// pixel along W and H; ld: elements from one pixel to the next (0: C); coordinates may start outside the image (zero padding of the convolution),
 // out-of-range pixels, channels and images read as zero.
 inline bool cached_map_nhwc(CUtensorMap* map, const void* p, int64_t N, int64_t H, int64_t W, int64_t C, int box_w, int box_h,
-                            int box_n, int stride) {
-    return cached_map(map, MapKey{p, {N, H, W, C, box_w, box_h, box_n, stride}}, [&](EncodeTiledFn fn) {
+                            int box_n, int stride, int64_t ld = 0) {
+    if (ld == 0) ld = C;
+    return cached_map(map, MapKey{p, {N, H, W, C, ld, box_w, box_h * 4096LL + box_n, stride}}, [&](EncodeTiledFn fn) {
         const cuuint64_t dims[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W), static_cast<cuuint64_t>(H),
                                     static_cast<cuuint64_t>(N)};
-        const cuuint64_t strides[3] = {static_cast<cuuint64_t>(C) * 2, static_cast<cuuint64_t>(W) * C * 2,
-                                       static_cast<cuuint64_t>(H) * W * C * 2};
+        const cuuint64_t strides[3] = {static_cast<cuuint64_t>(ld) * 2, static_cast<cuuint64_t>(W) * ld * 2,
+                                       static_cast<cuuint64_t>(H) * W * ld * 2};
         // box extents are given in traversed elements, i.e. times the stride
         const cuuint32_t box[4] = {64u, static_cast<cuuint32_t>(box_w * stride), static_cast<cuuint32_t>(box_h * stride),
                                    static_cast<cuuint32_t>(box_n)};

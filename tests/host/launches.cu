@@ -64,7 +64,7 @@ void check(const pf::tc::F32Params& p) {
 }
 constexpr uint64_t kSlice = 128 * 64 * 4;
 void check(const pf::tc::DtDvParams& p, unsigned blocks) {
-    writes("dT of a convolution", address(p.dT), matrix(p.rows, p.R, p.R, 2));
+    writes("dT of a convolution", address(p.dT), matrix(p.rows, p.R, p.ldt, 2));
     writes("slices of dV of a convolution", address(p.partial), p.pairs * blocks * kSlice);
 }
 void check(const pf::tc::DuParams& p) {

@@ -257,12 +257,12 @@ def test_resident_image_windows(N, H, W, C, R, O):
 
 
 @pytest.mark.parametrize("N,H,W,C,R,O", [
-    (30, 16, 16, 320, 40, 72),       # 16 divides the width: dU's blocks take the image's columns; an odd number of channel blocks; half a tile of dY
+    (45, 16, 16, 320, 40, 72),       # 16 divides the width: dU's blocks take the image's columns; an odd number of channel blocks; half a tile of dY
     (8, 32, 48, 264, 56, 136),       # blocks of one row of 48; a ragged channel block
     (300, 7, 7, 256, 40, 64),        # blocks of whole images
-    (120, 9, 13, 136, 24, 136),      # rows that do not divide into blocks
-    (8, 33, 63, 72, 24, 72),         # the widest image; one block of channels, ragged
-    (900, 3, 4, 512, 40, 24),        # windows of dX in boxes of whole images
+    (140, 9, 13, 136, 24, 136),      # rows that do not divide into blocks
+    (13, 33, 63, 72, 24, 72),        # the widest image; one block of channels, ragged
+    (950, 3, 4, 512, 40, 24),        # windows of dX in boxes of whole images
     (16, 32, 32, 512, 40, 512),      # the widest y
     (60, 31, 15, 192, 48, 96),
     (60, 28, 28, 128, 8, 128),       # one block of channels, the smallest rank
@@ -277,7 +277,7 @@ def test_flat_backward(N, H, W, C, R, O):
     x, U, V, dY = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V", "dY"))
     before = pf.pf_launch_count()
     _, dU0, dV0 = pf.pf_lowrank_conv_bwd(x, U, V, dY)
-    assert pf.pf_launch_count() - before == 4         # (x U once more)
+    assert pf.pf_launch_count() - before == (5 if N * H * W >= 20000 and R % 16 and 64 % R else 4)         # (x U once more; many pixels: U copied where its rows straddle lines)
     _, dU1, dV1 = pf.pf_lowrank_conv_bwd(x, U, V, dY, grads_f32=True)
     torch.cuda.synchronize()
     assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
