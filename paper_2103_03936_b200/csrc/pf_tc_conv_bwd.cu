@@ -9,10 +9,10 @@
 // The two reductions leave slices in the workspace, which warps of the launch behind add up beside its products: nothing waits
 // for the sums.
 // The form before (dT; then dU, dV and dX in one launch of 128 x 128 and 128 x 64 tiles) moves 1.6 GB through the SMs' load paths at
-// 128 x 32 x 32, 256 -> 64 -> 256 (x once per tap for dU, dT once per tap for dX), 0.45 here: backward 111.6 -> 89.4 us, training step
-// 196.2 -> 164.9.  By ncu, one launch at a time, they take 26, 34 and 45 us: the first is bound by memory (120 MB, of which 10 are slices),
-// the second by the tensor cores (busy 57 %; a 128 x 192 x 16 MMA takes 101 clocks) and its 29 MB of slices, the third by shared
-// memory (a 128 x 128 x 16 MMA reads 8 KB in its 64 clocks, all there is, beside the factor's tiles and the epilogue; tensor cores 45 %).
+// 128 x 32 x 32, 256 -> 64 -> 256 (x once per tap for dU, dT once per tap for dX), 0.45 here: backward 111.6 -> 85.2 us, training step
+// 195.5 -> 160.  By ncu, one launch at a time, they take 24, 32 and 36 us: the first is bound by memory (104 MB and 7 of slices), the second
+// by the tensor cores (busy 58 %; a 128 x 192 x 16 MMA takes 101 clocks) and its 29 MB of slices, the third by the pace at which one
+// thread issues MMAs and by shared memory (a 128 x 128 x 16 MMA reads 8 KB in its 64 clocks, all there is).
 #include <cmath>
 
 #include "pf_tc_conv_flat.cuh"
@@ -315,26 +315,38 @@ tc_conv_du_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             const uint32_t idesc = make_idesc_bf16(128, 192, 1, 1);
             const uint32_t to_t = static_cast<uint32_t>(rows01 ? 2 : 4) * kDuX + (kDuLead - 1) * 128u;
             // second unit: the other copy of dT, or the other channels
-            const uint64_t da = rows01 ? 0u : (2 * kDuX) >> 4, db = rows01 ? kDuT >> 4 : 0u;
+            const uint32_t da = rows01 ? 0u : (2 * kDuX) >> 4, db = rows01 ? kDuT >> 4 : 0u;
+            const uint64_t a_desc = make_smem_desc(ring, kDuX, 1024), b_desc = make_smem_desc(ring + to_t, 128, 1024);
+            const uint32_t ah = desc_hi(a_desc), bh = desc_hi(b_desc), full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+            uint32_t a = desc_lo(a_desc), b = desc_lo(b_desc);
+            // a step of 16 positions: 16 rows, and over dT's zero column at the end of an image row
+            uint32_t to[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) to[k] = 128u * k + 8u * static_cast<uint32_t>(k / p.steps_row);
+            const int ksteps = p.ksteps;
             uint32_t s = 0, ph = 0;
             bool ok = true;
             for (int i = 0; i < n; ++i) {
-                ok = mbar_wait(smem_u32(&ctl->full[s]), ph, abort_flag, p.status);
+                ok = mbar_wait(full0 + 8 * s, ph, abort_flag, p.status);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t at = ring + s * kDuStage;
-                uint64_t a = make_smem_desc(at, kDuX, 1024), b = make_smem_desc(at + to_t, 128, 1024);
-                int left = p.steps_row;
-                for (int k = 0; k < p.ksteps; ++k) {
-                    const uint32_t acc = i + k > 0 ? 1u : 0u;
-                    tc_mma_bf16(tmem, a, b, idesc, acc);
-                    if (units == 2) tc_mma_bf16(tmem + 192, a + da, b + db, idesc, acc);
-                    a += 128;
-                    b += 128;
-                    if (--left == 0) { left = p.steps_row; b += 8; }       // over dT's zero column
+                auto step = [&](uint32_t k, uint32_t more) {
+                    tc_mma_bf16_words(tmem, a + 128 * k, ah, b + to[k], bh, idesc, more);
+                    if (units == 2) tc_mma_bf16_words(tmem + 192, a + da + 128 * k, ah, b + db + to[k], bh, idesc, more);
+                };
+                step(0, i > 0 ? 1u : 0u);
+                if (ksteps == 4) {
+                    step(1, 1u);
+                    step(2, 1u);
+                    step(3, 1u);
+                } else {
+                    if (ksteps > 1) step(1, 1u);
+                    if (ksteps > 2) step(2, 1u);
                 }
-                tc_commit(smem_u32(&ctl->empty[s]));
-                if (++s == kDuStages) { s = 0; ph ^= 1u; }
+                tc_commit(empty0 + 8 * s);
+                a += kDuStage >> 4;
+                b += kDuStage >> 4;
+                if (++s == kDuStages) { s = 0; a -= kDuStages * (kDuStage >> 4); b -= kDuStages * (kDuStage >> 4); ph ^= 1u; }
             }
             if (ok) tc_commit(smem_u32(&ctl->acc_full));
         }
@@ -381,6 +393,9 @@ struct DxCtl {
     uint64_t a_full[2], a_empty[2], full[kDxMaxStages], empty[kDxMaxStages], acc_full[2], acc_empty[2];
     uint32_t tmem_base, abort;
 };
+// kFull: more than 48 ranks, i.e. four steps of 16 (a loop of p.ksteps steps issues the MMAs at half the pace of the tensor cores: 42.7 us
+// by ncu at 128 x 32 x 32, 256 -> 64 -> 256, 36.2 unrolled).
+template <bool kFull>
 __global__ void __launch_bounds__(kDxThreads, 1)
 tc_conv_dx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ DxParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -453,31 +468,37 @@ tc_conv_dx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            const uint32_t idesc = make_idesc_bf16(128, 128, 0, 0);
-            uint32_t s = 0, ph = 0, b = 0, bph = 0, use = 0;
+            const uint32_t idesc = make_idesc_bf16(128, 128, 0, 0), full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+            const uint64_t u_desc = make_smem_desc(ring, 16, 1024);
+            const uint32_t hi = desc_hi(u_desc), u0 = desc_lo(u_desc);       // (A's tiles have the same strides)
+            const int ksteps = p.ksteps;
+            uint32_t u = u0, s = 0, ph = 0, b = 0, bph = 0, use = 0;
             bool ok = true;
             for (int t = first; t < p.tiles && ok; t += step) {
                 const int q0 = t * kDxRows, row0 = q0 - first_unit(q0) * f.unit_rows;
                 ok = mbar_wait(smem_u32(&ctl->a_full[b]), bph, abort_flag, p.status);
                 if (!ok) break;
-                const uint64_t a0 = make_smem_desc(abuf + b * p.a_bytes, 16, 1024) + static_cast<uint64_t>(row0) * 8u;
+                const uint32_t a0 = desc_lo(make_smem_desc(abuf + b * p.a_bytes, 16, 1024)) + static_cast<uint32_t>(row0) * 8u;
                 for (int j = 0; j < p.nblk && ok; ++j, ++use) {
                     ok = mbar_wait(smem_u32(&ctl->acc_empty[use & 1u]), ((use >> 1) & 1u) ^ 1u, abort_flag, p.status);
                     if (!ok) break;
                     const uint32_t d = tmem + (use & 1u) * 256u;
                     int o = f.Wp + 1;                        // tap (0, 0) takes dT from one row and one column further
                     for (int tap = 0; tap < 9; ++tap) {
-                        ok = mbar_wait(smem_u32(&ctl->full[s]), ph, abort_flag, p.status);
+                        ok = mbar_wait(full0 + 8 * s, ph, abort_flag, p.status);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint64_t a = a0 + static_cast<uint64_t>(static_cast<int64_t>(o) * 8), u = make_smem_desc(ring + s * kDxStage, 16, 1024);
-                        for (int k = 0; k < p.ksteps; ++k) {
+                        const uint32_t a = a0 + static_cast<uint32_t>(o * 8);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (!kFull && k >= ksteps) break;
                             const uint32_t acc = tap + k > 0 ? 1u : 0u;
-                            tc_mma_bf16(d, a + 2 * k, u + 2 * k, idesc, acc);
-                            tc_mma_bf16(d + 128, a + 1024 + 2 * k, u + 2 * k, idesc, acc);
+                            tc_mma_bf16_words(d, a + 2 * k, hi, u + 2 * k, hi, idesc, acc);
+                            tc_mma_bf16_words(d + 128, a + 1024 + 2 * k, hi, u + 2 * k, hi, idesc, acc);
                         }
-                        tc_commit(smem_u32(&ctl->empty[s]));
-                        if (++s == NS) { s = 0; ph ^= 1u; }
+                        tc_commit(empty0 + 8 * s);
+                        u += kDxStage >> 4;
+                        if (++s == NS) { s = 0; u = u0; ph ^= 1u; }
                         o -= tap == 2 || tap == 5 ? f.Wp - 2 : 1;
                     }
                     if (ok) tc_commit(smem_u32(&ctl->acc_full[use & 1u]));
@@ -643,9 +664,10 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
         *a.dv_slices = LinearArgs::Slices();
         a.dv_slices->partial = pv; a.dv_slices->splits = b.grid_v; a.dv_slices->bn = 64; a.dv_slices->tiles_x = b.pairs; a.dv_slices->tiles_y = 1;
     }
+    auto* dx_kernel = a.R > 48 ? tc_conv_dx_kernel<true> : tc_conv_dx_kernel<false>;
     const size_t smem_u = 1024 + 1024 + kDuStages * kDuStage;
     if (allow_smem(tc_conv_dt_dv_kernel, 227 * 1024) != cudaSuccess || allow_smem(tc_conv_du_kernel, smem_u) != cudaSuccess ||
-        allow_smem(tc_conv_dx_kernel, 227 * 1024) != cudaSuccess)
+        allow_smem(dx_kernel, 227 * 1024) != cudaSuccess)
         return PF_ERR_CUDA;
     if (launch_overlapped(tc_conv_dt_dv_kernel, dim3(static_cast<unsigned>(b.grid_v)), dim3(kStreamThreads), b.smem_v, a.stream, y, t, v, sp) != cudaSuccess) return PF_ERR_CUDA;
     count_launch();
@@ -654,7 +676,7 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
     count_launch();
     // (every SM has a block for the sums; tiles go round by an even number of blocks)
     xp.step = xp.tiles > 0 ? even_grid(xp.tiles) : 1;
-    if (launch_overlapped(tc_conv_dx_kernel, dim3(static_cast<unsigned>(num_sms())), dim3(kDxThreads), b.smem_x, a.stream, xa, xb, xp) != cudaSuccess) return PF_ERR_CUDA;
+    if (launch_overlapped(dx_kernel, dim3(static_cast<unsigned>(num_sms())), dim3(kDxThreads), b.smem_x, a.stream, xa, xb, xp) != cudaSuccess) return PF_ERR_CUDA;
     count_launch();
     return PF_OK;
 }

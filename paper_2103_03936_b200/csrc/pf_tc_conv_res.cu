@@ -155,26 +155,28 @@ tc_conv_res_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             uint32_t use = 0;                       // accumulator uses so far
             bool ok = true;
             // the nine taps of one window buffer, into d0 (first row tile) and d1
-            auto taps = [&](uint32_t buf, int row0, uint32_t d0, uint32_t d1, uint32_t idesc, uint32_t b_step, bool fresh) {
-                const uint64_t a0 = make_smem_desc(abuf + buf * p.a_bytes, 16, 1024) + static_cast<uint64_t>(row0) * 8u;
+            const uint64_t b_desc = make_smem_desc(ring, 8192, 1024);
+            const uint32_t a_hi = desc_hi(make_smem_desc(abuf, 16, 1024)), b_hi = desc_hi(b_desc), b_lo = desc_lo(b_desc);
+            const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+            auto taps = [&](uint32_t buf, int row0, uint32_t d0, uint32_t d1, uint32_t idesc, bool fresh) {
+                const uint32_t a0 = desc_lo(make_smem_desc(abuf + buf * p.a_bytes, 16, 1024)) + static_cast<uint32_t>(row0) * 8u;
                 int o = -f.Wp - 1;                       // tap (0, 0)
                 for (int tap = 0; tap < 9; ++tap) {
-                    ok = mbar_wait(smem_u32(&ctl->full[s]), ph, abort_flag, p.status);
+                    ok = mbar_wait(full0 + 8 * s, ph, abort_flag, p.status);
                     if (!ok) return;
                     tc_fence_after();
-                    const uint64_t a = a0 + static_cast<uint64_t>(static_cast<int64_t>(o) * 8);
-                    const uint64_t bd = make_smem_desc(ring + s * kStage, 8192, 1024);
+                    const uint32_t a = a0 + static_cast<uint32_t>(o * 8), bd = b_lo + s * (kStage >> 4);
                     const uint32_t acc = (fresh && tap == 0) ? 0u : 1u;
 #pragma unroll
                     for (int m = 0; m < 2; ++m) {
                         const uint32_t d = m ? d1 : d0;
-                        const uint64_t am = a + m * 128u * 8u;
-                        tc_mma_bf16(d, am, bd, idesc, acc);
-                        tc_mma_bf16(d, am + 2, bd + b_step, idesc, 1u);
-                        tc_mma_bf16(d, am + 4, bd + 2 * b_step, idesc, 1u);
-                        tc_mma_bf16(d, am + 6, bd + 3 * b_step, idesc, 1u);
+                        const uint32_t am = a + m * 128u * 8u;
+                        tc_mma_bf16_words(d, am, a_hi, bd, b_hi, idesc, acc);
+                        tc_mma_bf16_words(d, am + 2, a_hi, bd + 128, b_hi, idesc, 1u);
+                        tc_mma_bf16_words(d, am + 4, a_hi, bd + 256, b_hi, idesc, 1u);
+                        tc_mma_bf16_words(d, am + 6, a_hi, bd + 384, b_hi, idesc, 1u);
                     }
-                    tc_commit(smem_u32(&ctl->empty[s]));
+                    tc_commit(empty0 + 8 * s);
                     if (++s == NS) { s = 0; ph ^= 1u; }
                     o += tap == 2 || tap == 5 ? f.Wp - 2 : 1;
                 }
@@ -189,7 +191,7 @@ tc_conv_res_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     for (int cb = 0; cb < p.cblks && ok; ++cb) {
                         ok = mbar_wait(smem_u32(&ctl->a_full[b]), bph, abort_flag, p.status);
                         if (!ok) break;
-                        taps(b, row0, d, d + 64, idesc1, 128u, cb == 0);
+                        taps(b, row0, d, d + 64, idesc1, cb == 0);
                         if (!ok) break;
                         tc_commit(smem_u32(&ctl->a_empty[b]));
                         b ^= 1u;
