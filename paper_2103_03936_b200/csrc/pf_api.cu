@@ -608,7 +608,7 @@ int pf_lowrank_conv_fwd(const void* x, const void* U, const void* V, void* y, vo
     if ((!y && N > 0) || !elem_aligned(y, dtype) || (T_stash && !elem_aligned(T_stash, dtype)))
         return PF_ERR_INVALID_ARG;
     const ConvWs w = conv_ws(N, H, W, C, R, O, kh, kw, stride, pad, dtype, false);
-    st = check_ws(workspace, workspace_bytes, w.total);
+    st = check_ws(workspace, workspace_bytes, dtype == PF_BF16 ? w.off_tc : w.total);
     if (st != PF_OK) return st;
     if (w.P == 0) return PF_OK;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -620,7 +620,8 @@ int pf_lowrank_conv_fwd(const void* x, const void* U, const void* V, void* y, vo
         a.x = x; a.U = U; a.V = V; a.y = y; a.T = T_stash;
         a.N = N; a.H = H; a.W = W; a.C = C; a.R = R; a.O = O; a.kh = kh; a.kw = kw;
         a.stride = stride; a.pad = pad; a.Ho = w.Ho; a.Wo = w.Wo;
-        a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.stream = stream;
+        a.ws = workspace_bytes >= w.total ? ws + w.off_tc : nullptr;      // bf16: copies of the factors, left out where they do not fit
+        a.ws_T = ws + w.off_T; a.stream = stream;
         int handled = 0;
         st = dtype == PF_BF16 ? tc::conv_fwd(a, &handled) : tc::f32_conv_fwd(a, &handled);
         if (st != PF_OK || handled) return st;

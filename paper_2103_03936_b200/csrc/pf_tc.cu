@@ -1219,21 +1219,26 @@ void conv_partial_bytes(const ConvA& c, int O, int su, int sv, size_t* bytes_u, 
 int64_t conv_dt_pitch(int64_t R) { return R % 64 == 0 || 64 % R == 0 ? R : (R + 63) / 64 * 64; }
 // dX reads U once per tile, so for many pixels it too is copied to that pitch, beside the launch that makes dT (64 x 28 x 28: 320 -> 80 ->
 // 320 110.1 -> 99.8 us, 320 -> 40 -> 320 90.6 -> 79.4; 8 x 28 x 28 of it 33.2 -> 34.2; rows of 96 bytes take no harm: 192 -> 48 -> 192 46.9 -> 48.3).
-static size_t conv_factor_copy(int64_t pixels, int64_t Keff, int64_t R) {
-    if (pixels < 20000 || conv_dt_pitch(R) == R || R % 8 || (R < 64 && R % 16 == 0)) return 0;
+// The forward copies both factors, and from fewer pixels on: every block reads all of U, a box of 64 ranks' rows in up to twice
+// the requests.  28 x 28 images, 160 -> 40 -> 160: N = 64 30.9 -> 26.4 us, 16 17.9 -> 14.8, 4 11.8 -> 13.2; 96 -> 24 -> 96: N = 16 15.4 ->
+// 12.8, 8 9.4 -> 12.8; 256 -> 72 -> 256, N = 64 69.7 -> 47.6; 768 -> 200 -> 768, N = 64 260 -> 229; 192 -> 48 -> 192, N = 128 34.9 -> 35.9.
+static size_t conv_factor_copy(int64_t pixels, int64_t Keff, int64_t R, bool fwd) {
+    if (pixels < (fwd ? 12000 : 20000) || conv_dt_pitch(R) == R || R % 8 || (R < 64 && R % 16 == 0)) return 0;
     return align_up(static_cast<size_t>(Keff) * conv_dt_pitch(R) * 2, 256);
 }
 
 size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad,
                             bool bwd) {
     const int Ho = (H + 2 * pad - kh) / stride + 1, Wo = (W + 2 * pad - kw) / stride + 1;
-    if (!bwd || N < 1 || Ho < 1 || Wo < 1) return 0;
+    if (N < 1 || Ho < 1 || Wo < 1) return 0;
+    const size_t copy = conv_factor_copy(static_cast<int64_t>(N) * Ho * Wo, static_cast<int64_t>(kh) * kw * C, R, !bwd);
+    if (!bwd) return copy > 0 ? copy + align_up(static_cast<size_t>(O) * conv_dt_pitch(R) * 2, 256) : 0;
     const ConvA c{2, N, H, W, C, R, Ho, Wo, kh, kw, pad, stride};
     int su, sv;
     size_t bu, bv;
     conv_splits(c, O, &su, &sv);
     conv_partial_bytes(c, O, su, sv, &bu, &bv);
-    return conv_factor_copy(static_cast<int64_t>(N) * Ho * Wo, static_cast<int64_t>(kh) * kw * C, R) + std::max(bu + bv, conv_flat_bwd_workspace(N, H, W, C, R, O, kh, kw, stride, pad));
+    return copy + std::max(bu + bv, conv_flat_bwd_workspace(N, H, W, C, R, O, kh, kw, stride, pad));
 }
 
 int conv_fwd(const ConvArgs& a, int* handled) {
@@ -1242,9 +1247,21 @@ int conv_fwd(const ConvArgs& a, int* handled) {
         (a.T && !aligned16(a.T)))
         return PF_OK;
     const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
-    int st = conv_res_fwd(a);
-    if (st == PF_ERR_UNSUPPORTED) st = chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, a.y, a.O, a.T, a.R, a.stream, &cv);
-    if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
+    // the factors at a pitch of whole lines, where the caller's scratch holds the copies
+    const int64_t Keff = static_cast<int64_t>(a.kh) * a.kw * a.C;
+    const size_t copy = a.ws ? conv_factor_copy(static_cast<int64_t>(a.N) * a.Ho * a.Wo, Keff, a.R, true) : 0;
+    ConvArgs b = a;
+    int64_t ldf = a.R;
+    if (copy > 0) {
+        ldf = conv_dt_pitch(a.R);
+        const RepackJob jobs[2] = {RepackJob{a.U, a.R, a.ws, ldf, Keff, a.R}, RepackJob{a.V, a.R, a.ws + copy, ldf, a.O, a.R}};
+        if (repack_rows_bf16_multi(jobs, 2, a.stream) != cudaSuccess) return PF_ERR_CUDA;
+        b.U = a.ws;
+        b.V = a.ws + copy;
+    }
+    int st = conv_res_fwd(b, ldf);
+    if (st == PF_ERR_UNSUPPORTED) st = chain(b.x, b.C, 0, 0, b.U, ldf, b.R, b.V, ldf, b.O, b.y, b.O, b.T, b.R, b.stream, &cv);
+    if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing but the copies has been launched
     *handled = 1;
     return st;
 }
@@ -1263,7 +1280,7 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         return chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
     };
     const int64_t ldt = conv_dt_pitch(a.R);
-    const size_t copy_bytes = conv_factor_copy(P, Keff, a.R);
+    const size_t copy_bytes = conv_factor_copy(P, Keff, a.R, false);
     const bool copy = a.dX && copy_bytes > 0;      // of U for dX; the launch that makes dT runs beside it
     char* const ws = a.ws + copy_bytes;
     const Operand U{copy ? a.ws : a.U, copy ? ldt : a.R, false, 0, false, true};

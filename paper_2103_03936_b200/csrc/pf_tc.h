@@ -139,7 +139,7 @@ int f32_conv_bwd(const ConvArgs& a, int* handled);
 // Device counters for one product whose contraction is split (null on error).
 unsigned int* split_counters();
 // 3 x 3, stride-1 convolutions on resident image windows (pf_tc_conv_res.cu); PF_ERR_UNSUPPORTED outside their envelope.
-int conv_res_fwd(const ConvArgs& a);
+int conv_res_fwd(const ConvArgs& a, int64_t ldf);      // ldf: pitch of the factors
 // Their backward (pf_tc_conv_bwd.cu), where `conv_flat_bwd_pays`; T is x U, a.ws_G takes dT.
 bool conv_flat_bwd_pays(const ConvArgs& a);
 size_t conv_flat_bwd_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad);

@@ -95,7 +95,7 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
     CUtensorMap ta, tb1, tb2, to, tt;
     const bool ragged = conv && conv->C % 64 != 0;
     bool ok = conv ? cached_map_nhwc(&ta, A, conv->N, conv->H, conv->W, conv->C, Wo, ct.bh, ct.nb, cs) : cached_map_2d(&ta, A, M, K1, lda, rows_tile);
-    ok = ok && (ragged ? cached_map_planes(&tb1, B1, static_cast<int64_t>(conv->kh) * conv->kw, conv->C, r, conv->C, 64)
+    ok = ok && (ragged ? cached_map_planes(&tb1, B1, static_cast<int64_t>(conv->kh) * conv->kw, conv->C, r, conv->C, 64, ldb1)
                        : cached_map_2d(&tb1, B1, K1, r, ldb1, 64));
     ok = ok && cached_map_2d(&tb2, B2, N2, r, ldb2, 128);
     if (conv) {   // outputs as windows of one tile's rows that start at any image row and end with the tile

@@ -123,10 +123,11 @@ inline bool cached_map_nhwc(CUtensorMap* map, const void* p, int64_t N, int64_t 
 // (planes = taps), less for overlapping windows (the output tiles of a convolution, one window per
 // image row, so that a tile may start at any row and is clipped at its own end).
 inline bool cached_map_planes(CUtensorMap* map, const void* p, int64_t planes, int64_t rows, int64_t cols, int64_t plane_step,
-                              int box_rows) {
-    return cached_map(map, MapKey{p, {planes, rows, cols, plane_step, box_rows, -1, -1, -1}}, [&](EncodeTiledFn fn) {
+                              int box_rows, int64_t ld = 0) {
+    if (ld == 0) ld = cols;
+    return cached_map(map, MapKey{p, {planes, rows, cols, plane_step, box_rows, ld, -1, -1}}, [&](EncodeTiledFn fn) {
         const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(planes)};
-        const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 2, static_cast<cuuint64_t>(plane_step) * cols * 2};
+        const cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * 2, static_cast<cuuint64_t>(plane_step) * ld * 2};
         const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 1u};
         const cuuint32_t estr[3] = {1u, 1u, 1u};
         return encode_bf16(fn, map, p, 3, dims, strides, box, estr);

@@ -283,6 +283,31 @@ def test_flat_backward(N, H, W, C, R, O):
     assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
 
 
+@pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad,copied", [
+    (60, 15, 14, 40, 24, 40, 3, 1, 1, True),        # per tap, ragged channels, a rank within one line
+    (60, 14, 15, 64, 72, 72, 3, 2, 1, False),       # too few pixels once the stride is taken
+    (47, 16, 16, 64, 72, 200, 3, 1, 1, True),       # just enough pixels, two rank blocks
+    (46, 16, 16, 64, 72, 200, 3, 1, 1, False),
+    (200, 28, 28, 72, 40, 136, 3, 1, 1, True),      # resident windows, ragged channels: one plane of U per tap
+    (200, 28, 28, 128, 40, 64, 3, 1, 1, True),
+    (60, 16, 16, 64, 136, 64, 1, 1, 0, True),
+])
+def test_forward_copies_of_the_factors(N, H, W, C, R, O, k, stride, pad, copied):
+    """Rows of U and V that straddle lines are copied to a pitch of whole ones; scratch without room for that runs on the
+    rows as they lie, to the same sums in the same order."""
+    c = wl.ConvCase("copies", N, H, W, C, R, O, wl.BF16, 98, kh=k, kw=k, stride=stride, pad=pad)
+    run_conv(c)
+    d = c.generate()
+    x, U, V = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V"))
+    before = pf.pf_launch_count()
+    y, T = pf.pf_lowrank_conv_fwd(x, U, V, stride=stride, pad=pad, want_stash=True)
+    assert pf.pf_launch_count() - before == 1 + copied
+    room = (T.numel() * 2 + 255) // 256 * 256
+    y1, T1 = pf.pf_lowrank_conv_fwd(x, U, V, stride=stride, pad=pad, want_stash=True, workspace=torch.empty(room, dtype=torch.uint8, device="cuda"))
+    torch.cuda.synchronize()
+    assert torch.equal(y, y1) and torch.equal(T, T1)
+
+
 @pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad", [
     (163, 16, 16, 64, 16, 64, 3, 1, 1),      # two dX tiles per block, a last block with one
     (41, 30, 30, 136, 24, 40, 3, 2, 1),      # eight per block, two column tiles (one ragged), all classes in a block
