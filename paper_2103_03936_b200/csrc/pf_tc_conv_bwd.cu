@@ -195,36 +195,128 @@ tc_conv_dt_dv_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_const
 }
 
 // ------------------------------------------------------------------------------ sums of slices
-// Units of 8 rows x 16 columns, one per warp and step: a lane sums four columns of a row over all slices, in slice order,
-// sixteen slices in flight.
-__device__ __forceinline__ void sum_slices(const SumPart& s, int first, int step, int lane) {
+// Units of 8 rows x 16 columns: a lane sums four columns of a row over all slices, in slice order, sixteen slices in flight.
+struct SumAt {
+    int row, col;                // of the result; row -1: none
+    const float4* slices;        // S of them, 2048 apart
+    int S;
+    float4 v;
+};
+__device__ __forceinline__ SumAt sum_unit(const SumPart& s, int u, int lane) {
+    const int tile = u >> 6, in = u & 63, rr = (in >> 2) * 8 + (lane & 7), pc = (in & 3) * 4 + (lane >> 3);
+    const bool tail = tile >= s.tail;
+    const int S = tail ? s.split[1] : s.split[0];
+    const size_t base = tail ? static_cast<size_t>(s.tail) * s.split[0] + static_cast<size_t>(tile - s.tail) * S : static_cast<size_t>(tile) * S;
+    const float4* src = reinterpret_cast<const float4*>(s.partial) + base * 2048u + ((rr >> 5) * 16 + pc) * 32 + (rr & 31);
+    float4 a = make_float4(-0.f, -0.f, -0.f, -0.f);
+#pragma unroll 1
+    for (int s0 = 0; s0 < S; s0 += 16) {
+        float4 w[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (s0 + i < S) w[i] = __ldcg(src + static_cast<size_t>(s0 + i) * 2048u);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (s0 + i < S) { a.x += w[i].x; a.y += w[i].y; a.z += w[i].z; a.w += w[i].w; }
+    }
+    int row = tile * 128 + rr;
+    if (s.per_tap > 0) {
+        const int tap = tile / s.per_tap, c = (tile - tap * s.per_tap) * 128 + rr;
+        row = c < s.rows ? tap * s.rows + c : -1;
+    } else if (row >= s.rows) {
+        row = -1;
+    }
+    return SumAt{pc * 4 < s.R ? row : -1, pc * 4, src, S, a};
+}
+__device__ __forceinline__ void put_sum(const SumPart& s, const SumAt& a) {
+    *reinterpret_cast<uint2*>(s.out + static_cast<size_t>(a.row) * s.R + a.col) = make_uint2(pack_bf16x2(a.v.x, a.v.y), pack_bf16x2(a.v.z, a.v.w));
+}
+__device__ __forceinline__ bool has_nan(const float4& v) { return v.x != v.x || v.y != v.y || v.z != v.z || v.w != v.w; }
+// One unit per warp and step; returns whether this lane has left out sums that are NaN (kLeave).
+template <bool kLeave>
+__device__ __forceinline__ bool sum_slices(const SumPart& s, int first, int step, int lane) {
+    bool left = false;
 #pragma unroll 1
     for (int u = first; u < s.tiles * 64; u += step) {
-        const int tile = u >> 6, in = u & 63, rr = (in >> 2) * 8 + (lane & 7), pc = (in & 3) * 4 + (lane >> 3);
-        const bool tail = tile >= s.tail;
-        const int S = tail ? s.split[1] : s.split[0];
-        const size_t base = tail ? static_cast<size_t>(s.tail) * s.split[0] + static_cast<size_t>(tile - s.tail) * S : static_cast<size_t>(tile) * S;
-        const float4* src = reinterpret_cast<const float4*>(s.partial) + base * 2048u + ((rr >> 5) * 16 + pc) * 32 + (rr & 31);
-        float4 a = make_float4(-0.f, -0.f, -0.f, -0.f);
+        const SumAt a = sum_unit(s, u, lane);
+        if (a.row < 0) continue;
+        if (kLeave && has_nan(a.v)) left = true;
+        else put_sum(s, a);
+    }
+    return left;
+}
+
+// The sums of dU that sum_slices has left out.  The MMAs of tc_conv_du_kernel take the three taps of a row from one tile of x, so they
+// multiply border pixels by the zeros around dT for the taps that pair them with nothing: an infinity or NaN there makes those taps' sums
+// NaN.  So each NaN is computed once more, over the pairs that exist, in fp32: a warp for 16 columns of a row, lanes along the
+// pixels, up to where all 16 are NaN.  Finite data pay nothing (backward of 128 x 32 x 32, 256 -> 64 -> 256: 84.7 us with and without);
+// one infinity at a border makes it 2.0 ms, a column of them 14, one pixel in 10000 26.
+__device__ __noinline__ void mend_sums(const DxParams& p, int first, int step, int lane) {
+    const FlatImage& f = p.f;
+    const SumPart& s = p.sum;
 #pragma unroll 1
-        for (int s0 = 0; s0 < S; s0 += 16) {
-            float4 w[16];
+    for (int u = first; u < s.tiles * 64; u += step) {
+        SumAt a = sum_unit(s, u, lane);
+        const bool bad = a.row >= 0 && has_nan(a.v);
+        uint32_t rows = __ballot_sync(0xffffffffu, bad);
+        rows = (rows | rows >> 8 | rows >> 16 | rows >> 24) & 0xffu;
+        const int col0 = (u & 3) * 16;
+        const bool wide = col0 + 8 < s.R;
+#pragma unroll 1
+        for (; rows != 0; rows &= rows - 1) {
+            const int r = __ffs(rows) - 1, row = __shfl_sync(0xffffffffu, a.row, r), tap = row / s.rows, c = row - tap * s.rows;
+            const int dy = tap / 3 - 1, dx = tap - tap / 3 * 3 - 1, y0 = max(0, -dy), x0 = max(0, -dx);
+            const int cols = f.W - abs(dx), per_image = (f.H - abs(dy)) * cols, count = f.N * per_image;
+            float sum[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (s0 + i < S) w[i] = __ldcg(src + static_cast<size_t>(s0 + i) * 2048u);
+            for (int j = 0; j < 16; ++j) sum[j] = 0.f;
+#pragma unroll 1
+            for (int i0 = 0; i0 < count; i0 += 1024) {
+                float part[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (s0 + i < S) { a.x += w[i].x; a.y += w[i].y; a.z += w[i].z; a.w += w[i].w; }
+                for (int j = 0; j < 16; ++j) part[j] = 0.f;
+#pragma unroll 4
+                for (int i = i0 + lane; i < min(count, i0 + 1024); i += 32) {
+                    const int n = i / per_image, in = i - n * per_image, y = in / cols;
+                    const int64_t pix = (static_cast<int64_t>(n) * f.H + y0 + y) * f.W + x0 + in - y * cols;
+                    const float v = __bfloat162float(p.x[(pix + dy * f.W + dx) * p.C + c]);
+                    const uint4* src = reinterpret_cast<const uint4*>(p.dT + pix * p.ldt + col0);
+                    const uint4 lo = src[0], hi = wide ? src[1] : make_uint4(0u, 0u, 0u, 0u);
+                    const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        part[2 * j] = fmaf(v, __uint_as_float(w[j] << 16), part[2 * j]);
+                        part[2 * j + 1] = fmaf(v, __uint_as_float(w[j] & 0xffff0000u), part[2 * j + 1]);
+                    }
+                }
+                uint32_t nan = wide ? 0u : 0xff00u;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    sum[j] += part[j];
+                    if (sum[j] != sum[j]) nan |= 1u << j;
+                }
+                if (__reduce_or_sync(0xffffffffu, nan) == 0xffffu) break;
+            }
+            float t[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
+                if (lane >> 3 == j >> 2) t[j & 3] = sum[j];
+            }
+            if ((lane & 7) == r) {
+                if (a.v.x != a.v.x) a.v.x = t[0];
+                if (a.v.y != a.v.y) a.v.y = t[1];
+                if (a.v.z != a.v.z) a.v.z = t[2];
+                if (a.v.w != a.v.w) a.v.w = t[3];
+            }
         }
-        int row = tile * 128 + rr;
-        if (s.per_tap > 0) {
-            const int tap = tile / s.per_tap, c = (tile - tap * s.per_tap) * 128 + rr;
-            row = c < s.rows ? tap * s.rows + c : -1;
-        } else if (row >= s.rows) {
-            row = -1;
+        if (bad) {
+            put_sum(s, a);
+            float4* const to = const_cast<float4*>(a.slices);          // (a caller that wants fp32 adds the slices up again)
+            *to = a.v;
+            for (int i = 1; i < a.S; ++i) to[static_cast<size_t>(i) * 2048u] = make_float4(-0.f, -0.f, -0.f, -0.f);
         }
-        if (row >= 0 && pc * 4 < s.R)
-            *reinterpret_cast<uint2*>(s.out + static_cast<size_t>(row) * s.R + pc * 4) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
     }
 }
 
@@ -354,7 +446,7 @@ tc_conv_du_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         const int q = warp & 3;
         const uint32_t lanes = tmem + (static_cast<uint32_t>(q * 32) << 16);
         // while the products run: the slices of dV, which the launch before has left
-        sum_slices(p.sum, static_cast<int>(blockIdx.x) * 4 + warp - 2, static_cast<int>(gridDim.x) * 4, lane);
+        sum_slices<false>(p.sum, static_cast<int>(blockIdx.x) * 4 + warp - 2, static_cast<int>(gridDim.x) * 4, lane);
         const bool ok = mbar_wait_warp(smem_u32(&ctl->acc_full), 0, abort_flag, p.status);
         tc_fence_after();
         if (ok) {
@@ -526,7 +618,8 @@ tc_conv_dx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
     } else {
         // (blocks without a tile are not kept waiting: they take their share of the sums first)
-        sum_slices(p.sum, static_cast<int>(gridDim.x - 1 - blockIdx.x) * 4 + warp - 11, static_cast<int>(gridDim.x) * 4, lane);
+        const int unit = static_cast<int>(gridDim.x - 1 - blockIdx.x) * 4 + warp - 11, units = static_cast<int>(gridDim.x) * 4;
+        if (__any_sync(0xffffffffu, sum_slices<true>(p.sum, unit, units, lane))) mend_sums(p, unit, units, lane);
     }
     tc_fence_before();
     __syncthreads();
@@ -650,6 +743,7 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
     xp.tiles = a.dX ? static_cast<int>(ceil_div(static_cast<int64_t>(b.f.N) * b.f.Hp * b.f.Wp, kDxRows)) : 0;
     xp.C = a.C; xp.nblk = static_cast<int>(ceil_div(a.C, 128)); xp.ksteps = static_cast<int>(ceil_div(a.R, 16));
     xp.out = static_cast<__nv_bfloat16*>(a.dX);
+    xp.x = static_cast<const __nv_bfloat16*>(a.x); xp.dT = sp.dT; xp.ldt = sp.ldt;
     xp.a_bytes = b.a_bytes; xp.a_off = 1024; xp.stg_off = 1024 + 2 * b.a_bytes; xp.ring_off = xp.stg_off + 32768;
     xp.num_stages = b.x_stages;
     xp.sum = SumPart{pu, static_cast<__nv_bfloat16*>(a.dU), 9 * b.tb, b.tb, a.C, a.R, {b.split[0], b.split[1]}, 6 * b.tb};

@@ -111,6 +111,8 @@ struct DxParams {
     FlatImage f;
     int tiles, step, C, nblk, ksteps;
     __nv_bfloat16* out;
+    const __nv_bfloat16 *x, *dT;     // (for sums of dU that are NaN)
+    int ldt;
     uint32_t a_bytes, a_off, stg_off, ring_off;
     int num_stages;
     SumPart sum;                 // dU

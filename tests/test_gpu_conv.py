@@ -283,6 +283,49 @@ def test_flat_backward(N, H, W, C, R, O):
     assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
 
 
+@pytest.mark.parametrize("N,H,W,C,R,O", [(45, 16, 16, 320, 40, 72), (140, 9, 13, 136, 24, 136), (300, 7, 7, 256, 40, 64), (60, 28, 28, 128, 8, 128)])
+@pytest.mark.parametrize("how", ["plain", "grads_f32", "accumulate"])
+def test_flat_backward_infinities_at_the_border(N, H, W, C, R, O, how):
+    """A border pixel that is no number reaches only the taps that pair it with a pixel of y: the others of its channel are what
+    they are with a zero there, the other channels are untouched.  An infinity in dY likewise reaches the pixels of x that it is paired with."""
+    g = torch.Generator(device="cuda").manual_seed(99)
+    rand = lambda *s: torch.rand(s, generator=g, device="cuda").add_(0.25).bfloat16()       # (no zeros, no signs: infinities stay infinities)
+    x, U, V, dY = rand(N, H, W, C), rand(3, 3, C, R), rand(O, R), rand(N, H, W, O)
+    kw = dict(grads_f32=how == "grads_f32")
+
+    def grads(x, dY):
+        if how == "accumulate":
+            kw.update(accumulate=True, dU=torch.ones_like(U), dV=torch.ones_like(V))
+        return pf.pf_lowrank_conv_bwd(x, U, V, dY, **kw)[1:]
+
+    borders = [((3, 0, 2, 1), float("inf")), ((N - 1, H - 1, 4, 7), float("inf")), ((0, 3, 0, C - 1), float("nan")), ((5, 2, W - 1, 64), float("-inf")),
+               ((1, 0, 0, 2), float("inf")), ((2, H - 1, W - 1, 3), float("nan"))]
+    bad, zeroed = x.clone(), x.clone()
+    reached = torch.zeros(3, 3, C, dtype=torch.bool, device="cuda")
+    for at, v in borders:
+        bad[at], zeroed[at] = v, 0
+        for ky in range(3):
+            for kx in range(3):
+                reached[ky, kx, at[3]] |= 0 <= at[1] - (ky - 1) < H and 0 <= at[2] - (kx - 1) < W
+    (dU, dV), (dU0, dV0) = grads(bad, dY), grads(zeroed, dY)
+    assert not dU[reached].isfinite().any() and torch.isinf(dU[1, 1, 1]).all()
+    # fp32 sums of positive products in another order: n units in the last place of half of one each; bf16 rounds twice
+    tol = N * H * W * 2.0 ** -24 + (0 if how == "grads_f32" else 2.0 ** -7)
+    rest = ~reached
+    assert dU[rest].isfinite().all() and ((dU[rest].double() - dU0[rest].double()).abs() <= tol * dU0[rest].double()).all()
+    clean = torch.ones(C, dtype=torch.bool, device="cuda")
+    clean[[at[3] for at, _ in borders]] = False
+    assert torch.equal(dU[:, :, clean], dU0[:, :, clean])
+    inf_dY = dY.clone()
+    inf_dY[4, H - 1, 0, 5] = float("inf")
+    dU, dV = grads(x, inf_dY)
+    for ky in range(3):
+        for kx in range(3):
+            assert (dU[ky, kx].isfinite() if H - 1 + ky - 1 >= H or kx - 1 < 0 else dU[ky, kx].isinf()).all(), (ky, kx)
+    assert dV[5].isinf().all() and dV[6].isfinite().all()
+    assert pf.pf_last_device_status() == 0
+
+
 @pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad,copied", [
     (60, 15, 14, 40, 24, 40, 3, 1, 1, True),        # per tap, ragged channels, a rank within one line
     (60, 14, 15, 64, 72, 72, 3, 2, 1, False),       # too few pixels once the stride is taken
