@@ -279,6 +279,8 @@ int pf_lowrank_linear_grouped_bwd(int groups,
  *   y [N, Ho, Wo, O] NHWC,  Ho = (H + 2 pad - kh) / stride + 1 (floor), Wo likewise
  *   T_stash [N, Ho, Wo, R]: optional output of the thin convolution; NULL = not written.
  * Returns PF_ERR_UNSUPPORTED for kh != kw or stride < 1.
+ * bf16: the query is what the fastest kernels use.  A smaller workspace is taken down to what the slower ones cannot do without
+ * (T; backwards also dT, both of R elements per pixel, and the sums of the reductions), and selects those.
  * ------------------------------------------------------------------------------- */
 size_t pf_lowrank_conv_workspace(int N, int H, int W, int C, int R, int O,
                                  int kh, int kw, int stride, int pad, int dtype, int is_bwd);

@@ -535,8 +535,9 @@ struct ConvWs {
     int Ho, Wo;
     int64_t P, Pin;
 };
+// lean: what a bf16 backward needs at least.
 ConvWs conv_ws(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad,
-               int dtype, bool bwd) {
+               int dtype, bool bwd, bool lean = false) {
     ConvWs w;
     std::memset(&w, 0, sizeof(w));
     w.Ho = (H + 2 * pad - kh) / stride + 1;
@@ -549,7 +550,7 @@ ConvWs conv_ws(int N, int H, int W, int C, int R, int O, int kh, int kw, int str
     size_t off = 0;
     w.off_T = off; off += align_up(static_cast<size_t>(w.P) * R * s, 256);
     if (bwd) {
-        w.off_dT = off; off += align_up(static_cast<size_t>(w.P) * (dtype == PF_BF16 ? tc::conv_dt_pitch(R) : R) * s, 256);
+        w.off_dT = off; off += align_up(static_cast<size_t>(w.P) * (dtype == PF_BF16 && !lean ? tc::conv_dt_pitch(R) : R) * s, 256);
         const int64_t Keff = static_cast<int64_t>(kh) * kw * C;
         w.splits_dU = simt_pick_splits(Keff, R, w.P);
         w.splits_dV = simt_pick_splits(O, R, w.P);
@@ -561,7 +562,7 @@ ConvWs conv_ws(int N, int H, int W, int C, int R, int O, int kh, int kw, int str
     }
     w.off_tc = off;
     if (dtype == PF_BF16) {
-        off += align_up(tc::conv_extra_workspace(N, H, W, C, R, O, kh, kw, stride, pad, bwd), 256);
+        off += align_up(tc::conv_extra_workspace(N, H, W, C, R, O, kh, kw, stride, pad, bwd, lean), 256);
     } else {
         tc::ConvArgs a;
         std::memset(&a, 0, sizeof(a));
@@ -659,7 +660,9 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
     if (!elem_aligned(dY, dtype) || !elem_aligned(dU, gdtype) || !elem_aligned(dV, gdtype) ||
         (dX && !elem_aligned(dX, dtype)) || (T_stash && !elem_aligned(T_stash, dtype)))
         return PF_ERR_INVALID_ARG;
-    const ConvWs w = conv_ws(N, H, W, C, R, O, kh, kw, stride, pad, dtype, true);
+    ConvWs w = conv_ws(N, H, W, C, R, O, kh, kw, stride, pad, dtype, true);
+    const bool lean = dtype == PF_BF16 && workspace_bytes < w.total;      // the products that need least, in the room that they need
+    if (lean) w = conv_ws(N, H, W, C, R, O, kh, kw, stride, pad, dtype, true, true);
     st = check_ws(workspace, workspace_bytes, w.total);
     if (st != PF_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -708,6 +711,7 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         a.N = N; a.H = H; a.W = W; a.C = C; a.R = R; a.O = O; a.kh = kh; a.kw = kw;
         a.stride = stride; a.pad = pad; a.Ho = w.Ho; a.Wo = w.Wo;
         a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.ws_G = ws + w.off_dT; a.stream = stream;
+        a.lean = lean;
         if (flags) { a.du_slices = &su_info; a.dv_slices = &sv_info; }
         int handled = 0;
         st = dtype == PF_BF16 ? tc::conv_bwd(a, &handled) : tc::f32_conv_bwd(a, &handled);

@@ -1189,8 +1189,9 @@ void reset_fix_counters() {
 // Tensor-core envelope of the factorized convolution: channel counts that are multiples of 8 (TMA pitches; a
 // ragged 64-channel block is zero-filled), output rows that fit the tiles (128 pixels forward and dX, 64 for
 // the contraction of dU), and for a strided backward at least one tap per pixel class (kernel >= stride).
+constexpr int kConvMaxRank = 384;
 static bool conv_tc_ok(const ConvArgs& a, bool fwd) {
-    if (a.kh != a.kw || a.C % 8 != 0 || a.R % 8 != 0 || a.O % 8 != 0 || a.R > 384) return false;
+    if (a.kh != a.kw || a.C % 8 != 0 || a.R % 8 != 0 || a.O % 8 != 0 || a.R > kConvMaxRank) return false;
     if (a.stride > 4 || a.Wo > (fwd ? 128 : 64) || a.stride * a.Wo > 256) return false;
     if (!fwd && (a.kh < a.stride || ceil_div(a.W, a.stride) > 128)) return false;
     if (static_cast<int64_t>(a.N) * a.H * a.W > 0x7fffffff || static_cast<int64_t>(a.kh) * a.kw * a.C > 0x7fffffff) return false;
@@ -1216,7 +1217,8 @@ void conv_partial_bytes(const ConvA& c, int O, int su, int sv, size_t* bytes_u, 
 // Elements from one pixel of dT to the next: rows of 24, 40, 48, 56 or 80 ranks would straddle 128-byte lines, and the products that
 // read them once per tap take two requests for most.  (Ranks whose rows divide a line, or are made of lines, lie as they are.)  Backward of
 // 16 x 14 x 14, 160 -> 40 -> 160 18.9 -> 16.6 us, of 8 x 28 x 28, 192 -> 48 -> 192 18.9 -> 16.6, stride 2 of 64 x 14 x 14, 256 -> 72 -> 256 22.0 -> 19.9.
-int64_t conv_dt_pitch(int64_t R) { return R % 64 == 0 || 64 % R == 0 ? R : (R + 63) / 64 * 64; }
+// (Ranks that only the FMA kernels take have no such rows.)
+int64_t conv_dt_pitch(int64_t R) { return R % 64 == 0 || 64 % R == 0 || R % 8 != 0 || R > kConvMaxRank ? R : (R + 63) / 64 * 64; }
 // dX reads U once per tile, so for many pixels it too is copied to that pitch, beside the launch that makes dT (64 x 28 x 28: 320 -> 80 ->
 // 320 110.1 -> 99.8 us, 320 -> 40 -> 320 90.6 -> 79.4; 8 x 28 x 28 of it 33.2 -> 34.2; rows of 96 bytes take no harm: 192 -> 48 -> 192 46.9 -> 48.3).
 // The forward copies both factors, and from fewer pixels on: every block reads all of U, a box of 64 ranks' rows in up to twice
@@ -1228,17 +1230,19 @@ static size_t conv_factor_copy(int64_t pixels, int64_t Keff, int64_t R, bool fwd
 }
 
 size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad,
-                            bool bwd) {
+                            bool bwd, bool lean) {
     const int Ho = (H + 2 * pad - kh) / stride + 1, Wo = (W + 2 * pad - kw) / stride + 1;
     if (N < 1 || Ho < 1 || Wo < 1) return 0;
-    const size_t copy = conv_factor_copy(static_cast<int64_t>(N) * Ho * Wo, static_cast<int64_t>(kh) * kw * C, R, !bwd);
+    const size_t copy = lean ? 0 : conv_factor_copy(static_cast<int64_t>(N) * Ho * Wo, static_cast<int64_t>(kh) * kw * C, R, !bwd);
     if (!bwd) return copy > 0 ? copy + align_up(static_cast<size_t>(O) * conv_dt_pitch(R) * 2, 256) : 0;
     const ConvA c{2, N, H, W, C, R, Ho, Wo, kh, kw, pad, stride};
     int su, sv;
     size_t bu, bv;
     conv_splits(c, O, &su, &sv);
     conv_partial_bytes(c, O, su, sv, &bu, &bv);
-    return copy + std::max(bu + bv, conv_flat_bwd_workspace(N, H, W, C, R, O, kh, kw, stride, pad));
+    ConvArgs a = {};
+    a.N = N; a.H = H; a.W = W; a.C = C; a.R = R; a.O = O; a.kh = kh; a.kw = kw; a.stride = stride; a.pad = pad; a.Ho = Ho; a.Wo = Wo;
+    return lean ? bu + bv : copy + std::max(bu + bv, conv_flat_bwd_workspace(a));
 }
 
 int conv_fwd(const ConvArgs& a, int* handled) {
@@ -1279,8 +1283,8 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
         return chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
     };
-    const int64_t ldt = conv_dt_pitch(a.R);
-    const size_t copy_bytes = conv_factor_copy(P, Keff, a.R, false);
+    const int64_t ldt = a.lean ? a.R : conv_dt_pitch(a.R);
+    const size_t copy_bytes = a.lean ? 0 : conv_factor_copy(P, Keff, a.R, false);
     const bool copy = a.dX && copy_bytes > 0;      // of U for dX; the launch that makes dT runs beside it
     char* const ws = a.ws + copy_bytes;
     const Operand U{copy ? a.ws : a.U, copy ? ldt : a.R, false, 0, false, true};
@@ -1288,7 +1292,7 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         const RepackJob job{a.U, a.R, a.ws, ldt, Keff, a.R};
         return !copy || repack_rows_bf16_multi(&job, 1, a.stream) == cudaSuccess ? PF_OK : PF_ERR_CUDA;
     };
-    if (conv_flat_bwd_pays(a) && aligned16(a.dU) && aligned16(a.dV)) {
+    if (!a.lean && conv_flat_bwd_pays(a) && aligned16(a.dU) && aligned16(a.dV)) {
         st = a.T ? PF_OK : recompute();
         if (st == PF_ERR_UNSUPPORTED) return PF_OK;
         *handled = 1;

@@ -45,6 +45,7 @@ struct ConvArgs {
     cudaStream_t stream;
     // backward: where the fp32 slices of dU / dV were left (see LinearArgs::Slices); may be null
     LinearArgs::Slices *du_slices, *dv_slices;
+    bool lean;      // backward, bf16: ws and ws_G have room for the products that fetch pixels per tap only, ws_G with R elements per pixel
 };
 
 // Fused chain kernel (pf_tc_chain.cu): out = (A * B1) * B2^T with the intermediate on chip.
@@ -121,7 +122,7 @@ int linear_grouped_bwd(const GroupedArgs& a, int* handled);
 
 size_t linear_extra_workspace(int64_t m, int64_t k, int64_t n, int64_t r, bool bwd);
 size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride,
-                            int pad, bool bwd);
+                            int pad, bool bwd, bool lean = false);
 void reset_fix_counters();  // clears the slice-sum counters (after PF_ERR_TIMEOUT)
 size_t linear_fwd_need(const LinearArgs& a, bool* handles);   // bytes of a.ws the forward really touches
 int64_t linear_fwd_rows(const LinearArgs& a, size_t room, LinearArgs* b);   // rows at a time in so much room, 0: not by rows
@@ -142,10 +143,10 @@ unsigned int* split_counters();
 int conv_res_fwd(const ConvArgs& a, int64_t ldf);      // ldf: pitch of the factors
 // Their backward (pf_tc_conv_bwd.cu), where `conv_flat_bwd_pays`; T is x U, a.ws_G takes dT.
 bool conv_flat_bwd_pays(const ConvArgs& a);
-size_t conv_flat_bwd_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad);
+size_t conv_flat_bwd_workspace(const ConvArgs& a);      // a: sizes only; 0 where it does not pay
 int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early);     // early: the launch before copies U, nothing else
 int conv_fwd(const ConvArgs& a, int* handled);
-int conv_bwd(const ConvArgs& a, int* handled);      // a.ws_G: conv_dt_pitch(R) elements per pixel
+int conv_bwd(const ConvArgs& a, int* handled);      // a.ws_G: conv_dt_pitch(R) elements per pixel, unless lean
 int64_t conv_dt_pitch(int64_t R);
 
 }  // namespace tc

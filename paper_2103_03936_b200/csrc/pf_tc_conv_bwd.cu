@@ -685,11 +685,6 @@ bool flat_bwd_plan(int N, int H, int W, int C, int R, int O, int kh, int kw, int
 }
 }  // namespace
 
-size_t conv_flat_bwd_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad) {
-    FlatBwd b;
-    return flat_bwd_plan(N, H, W, C, R, O, kh, kw, stride, pad, &b) ? b.bytes_u + b.bytes_v : 0;
-}
-
 // Against the launches that fetch pixels per tap (old / here, cold L2).  Rows of dT and U that straddle lines are what those suffer from, so
 // at ranks of 24, 40 or 56 these pay early: 160 -> 40 -> 160 of 6272 pixels 23.2 / 25.9 us, 12544 36.4 / 31.3, 50176 96.5 / 59.8; 128 -> 40 -> 128
 // of 12544 24.0 / 24.9, 25088 37.5 / 29.7; 64 -> 24 -> 64 of 12544 20.1 / 24.6, 25088 30.9 / 30.2.  At 48: 192 -> 48 -> 192 of 12544 23.2 / 28.1, 25088
@@ -702,6 +697,11 @@ bool conv_flat_bwd_pays(const ConvArgs& a) {
     const double c = a.C / 100.0, p = static_cast<double>(a.N) * a.H * a.W / 1000.0, pc = p * c, po = p * a.O / 100.0;
     if (64 % a.R != 0) return a.R % 16 != 0 ? p >= (a.C >= 160 ? 11.0 : a.C >= 96 ? 16.0 : 25.0) : p >= (a.C >= 160 ? 20.0 : 50.0);
     return p >= 2.0 && 14.6 + 3.58 * c + 0.23 * p + 0.07 * pc + 0.05 * po < (a.R > 32 ? 0.9 : 1.05) * (12.35 + 0.07 * c + 0.16 * p + 0.19 * pc + 0.07 * po);
+}
+
+size_t conv_flat_bwd_workspace(const ConvArgs& a) {
+    FlatBwd b;
+    return conv_flat_bwd_pays(a) && flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b) ? b.bytes_u + b.bytes_v : 0;
 }
 
 // T: the stash, or x * U as a launch before left it.

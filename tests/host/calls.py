@@ -16,6 +16,11 @@ WIDE = [(8192, 1500, 6000, 375), (8192, 1504, 6016, 376), (4096, 1024, 4096, 102
         (4096, 6000, 1500, 375), (4944, 2048, 3768, 512), (2500, 1032, 4104, 520), (8192, 1024, 4096, 512), (8192, 4096, 1024, 512),
         (11209, 3072, 768, 768), (4756, 1728, 6912, 432)]
 
+# Convolution backwards and the bytes that they can do with: N, H, W, C, R, O, kernel, stride, pad
+LEAST = [((128, 32, 32, 256, 64, 256, 3, 1, 1), 44040192), ((64, 28, 28, 160, 40, 160, 3, 1, 1), 16001024), ((64, 28, 28, 160, 40, 160, 3, 2, 1), 9979904),
+         ((64, 28, 28, 320, 80, 320, 3, 1, 1), 29954048), ((64, 28, 28, 320, 80, 320, 1, 1, 0), 28864512), ((60, 28, 28, 128, 8, 128, 3, 1, 1), 7002112),
+         ((30, 16, 16, 96, 48, 64, 3, 1, 1), 10062848), ((8, 9, 11, 72, 24, 40, 3, 2, 1), 508416), ((16, 14, 14, 64, 33, 64, 3, 1, 1), 7207168)]
+
 
 class Library:
     def __init__(self, path):
@@ -93,13 +98,13 @@ def grouped(lib, g, m, k, n, r, dtype, *, bwd, stash=True, dX=True, shared=False
                     (mats(m, k, 1 if shared else g) if dX else none) + mats(k, r) + mats(n, r) + sizes, room)
 
 
-def conv(lib, N, H, W, C, R, O, kernel, stride, pad, dtype, *, bwd, stash=True, dX=True, flags=0):
+def conv(lib, N, H, W, C, R, O, kernel, stride, pad, dtype, *, bwd, stash=True, dX=True, flags=0, room=None):
     size = 2 if dtype == BF16 else 4
     gsize = 4 if flags & GRADS_F32 else size
     Ho, Wo = (H + 2 * pad - kernel) // stride + 1, (W + 2 * pad - kernel) // stride + 1
     x, U, V, y, T = ((v * size, 0) for v in (N * H * W * C, kernel * kernel * C * R, O * R, N * Ho * Wo * O, N * Ho * Wo * R))
     sizes = [c(v) for v in (N, H, W, C, R, O, kernel, kernel, stride, pad, dtype)]
-    room = lib.query("pf_lowrank_conv_workspace", *sizes, c(int(bwd)))
+    room = room or lib.query("pf_lowrank_conv_workspace", *sizes, c(int(bwd)))
     T = T if stash else None
     if not bwd:
         return lib.call("pf_lowrank_conv_fwd", [x, U, V, y, T] + sizes, room)
@@ -159,6 +164,13 @@ def fixed(kind):
             for flags in (0, ACCUMULATE, GRADS_F32):
                 yield linear, shape + (BF16,), dict(bwd=True, flags=flags)
             yield linear, shape + (BF16,), dict(bwd=True, stash=False, dX=False)
+
+
+    if kind == "conv_bwd":                        # workspaces from before some of these calls had a use for more
+        for shape, room in LEAST:
+            for flags in (0, ACCUMULATE, GRADS_F32):
+                yield conv, shape + (BF16,), dict(bwd=True, flags=flags, room=room)
+                yield conv, shape + (BF16,), dict(bwd=True, stash=False, dX=False, flags=flags, room=room)
 
 
 def main(path, kind, count, seed):

@@ -174,3 +174,18 @@ def test_binding_raises_when_library_is_missing(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "_LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(ImportError):
         binding.lib()
+
+
+def test_conv_backward_asks_for_what_it_uses(L):
+    """Ranks that only the FMA kernels take have no rows at a pitch of whole lines, small batches no slices of the form that
+    reads images once."""
+    least = lambda *a: pf.pf_lowrank_conv_workspace(*a, pf.PF_BF16, True)
+    assert least(256, 56, 56, 64, 5, 64, 3, 3, 1, 1) == 21292800 and least(256, 56, 56, 64, 5, 64, 1, 1, 1, 0) == 20334080
+    assert least(16, 14, 14, 64, 33, 64, 3, 3, 1, 1) == 7207168
+    assert least(8, 14, 14, 512, 64, 512, 3, 3, 1, 1) == 11804672 and least(32, 14, 14, 1024, 64, 512, 3, 3, 1, 1) == 14778368
+
+
+def test_conv_backward_refuses_less_than_the_least_workspace(L):
+    def bwd(room):
+        return L.pf_lowrank_conv_bwd(P, P, P, P, P, P, P, P, 128, 32, 32, 256, 64, 256, 3, 3, 1, 1, 1, P, room, 0)
+    assert bwd(44040191) == WORKSPACE and bwd(0) == WORKSPACE

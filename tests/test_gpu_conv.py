@@ -11,15 +11,15 @@ from _gpu import ESCAPES, PFDT, Guarded, Scratch, assert_blocks_close, assert_cl
 pytestmark = pytest.mark.gpu
 
 
-def run_conv(case, stash=True, need_dX=True, tiny=False):
+def run_conv(case, stash=True, need_dX=True, tiny=False, bwd_room=None):
     d = case.generate()
     dt = case.dtype
     x, U, V, dY = (dev(d[k_], dt) for k_ in ("x", "U", "V", "dY"))
     Ho, Wo = case.Ho, case.Wo
     gy = Guarded((case.N, Ho, Wo, case.O), dt)
     gT = Guarded((case.N, Ho, Wo, case.R), dt)
-    scratch = [Scratch(pf.pf_lowrank_conv_workspace(case.N, case.H, case.W, case.C, case.R, case.O, case.kh, case.kw, case.stride, case.pad, PFDT[dt], bwd))
-               for bwd in (False, True)]
+    scratch = [Scratch(pf.pf_lowrank_conv_workspace(case.N, case.H, case.W, case.C, case.R, case.O, case.kh, case.kw, case.stride, case.pad, PFDT[dt], bwd)
+                       if not (bwd and bwd_room) else bwd_room) for bwd in (False, True)]
     pf.pf_lowrank_conv_fwd(x, U, V, stride=case.stride, pad=case.pad, y=gy.t,
                            T_stash=gT.t if stash else None, workspace=scratch[0].t)
     gdX, gdU, gdV = Guarded(x.shape, dt), Guarded(U.shape, dt), Guarded(V.shape, dt)
@@ -281,6 +281,16 @@ def test_flat_backward(N, H, W, C, R, O):
     _, dU1, dV1 = pf.pf_lowrank_conv_bwd(x, U, V, dY, grads_f32=True)
     torch.cuda.synchronize()
     assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
+
+
+@pytest.mark.parametrize("N,H,W,C,R,O,stride,room", [(45, 16, 16, 320, 40, 72, 1, 10154752), (140, 9, 13, 136, 24, 136, 1, 8250624),
+                                                     (60, 15, 14, 40, 24, 40, 2, 6124800)])
+def test_backward_in_the_least_workspace(N, H, W, C, R, O, stride, room):
+    """Scratch without room for what reads less: the products that fetch pixels per tap, on rows as they lie."""
+    c = wl.ConvCase("least", N, H, W, C, R, O, wl.BF16, 96, stride=stride)
+    assert pf.pf_lowrank_conv_workspace(N, H, W, C, R, O, 3, 3, stride, 1, pf.PF_BF16, True) > room
+    run_conv(c, bwd_room=room)
+    run_conv(c, stash=False, need_dX=False, bwd_room=room)
 
 
 @pytest.mark.parametrize("N,H,W,C,R,O", [(45, 16, 16, 320, 40, 72), (140, 9, 13, 136, 24, 136), (300, 7, 7, 256, 40, 64), (60, 28, 28, 128, 8, 128)])
