@@ -685,13 +685,14 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         dV = ws + w.off_gtmp + align_up(static_cast<size_t>(Keff) * R * s, 256);
     }
     tc::LinearArgs::Slices su_info, sv_info;
+    tc::ConvArgs::Gradients user{user_dU, user_dV, g_f32, g_acc, false};
     auto finish = [&]() -> int {
-        if (!flags) return PF_OK;
+        if (!flags || user.written) return PF_OK;
         SliceSums jobs[2];
         int nj = 0;
         if (su_info.partial)
             jobs[nj++] = SliceSums{su_info.partial, user_dU, R, static_cast<int>(Keff), R, su_info.splits, su_info.bn,
-                                   su_info.tiles_x, su_info.tiles_y, g_f32, g_acc, su_info.conv_c, su_info.conv_blks, su_info.tail, su_info.tail_splits};
+                                   su_info.tiles_x, su_info.tiles_y, g_f32, g_acc, su_info.conv_c};
         else
             PF_CUDA(grad_combine(user_dU, R, gdtype, dU, R, dtype, Keff, R, g_acc, stream));
         if (sv_info.partial)
@@ -712,7 +713,7 @@ int pf_lowrank_conv_bwd_ex(const void* x, const void* U, const void* V, const vo
         a.stride = stride; a.pad = pad; a.Ho = w.Ho; a.Wo = w.Wo;
         a.ws = ws + w.off_tc; a.ws_T = ws + w.off_T; a.ws_G = ws + w.off_dT; a.stream = stream;
         a.lean = lean;
-        if (flags) { a.du_slices = &su_info; a.dv_slices = &sv_info; }
+        if (flags) { a.du_slices = &su_info; a.dv_slices = &sv_info; a.gradients = &user; }
         int handled = 0;
         st = dtype == PF_BF16 ? tc::conv_bwd(a, &handled) : tc::f32_conv_bwd(a, &handled);
         if (st != PF_OK) return st;

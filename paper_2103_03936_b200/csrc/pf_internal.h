@@ -102,8 +102,6 @@ struct SliceSums {
     int M, N, splits, bn, tiles_x, tiles_y;
     bool out_f32, accumulate;
     int conv_c = 0;     // > 0: rows are pairs of 64-channel blocks of a [taps][conv_c] index
-    int conv_blks = 0;  // > 0: that many blocks per tap
-    int tail = 0, tail_splits = 0;      // tail > 0: slices of the tiles from there on
 };
 cudaError_t slices_to_gradients(const SliceSums* jobs, int count, cudaStream_t stream);
 // Backward of y = act(z + bias): dY becomes dZ in place, db (optional) its column sums.  `part` holds

@@ -362,7 +362,7 @@ struct SliceSumJob {
     const float* partial;
     void* out;
     long long ld;
-    int M, N, S, bn, tiles_x, tiles_y, out_f32, accumulate, conv_c, conv_blks, tail, tail_S;
+    int M, N, S, bn, tiles_x, tiles_y, out_f32, accumulate, conv_c;
 };
 __global__ void __launch_bounds__(256) slices_to_gradients_kernel(const SliceSumJob j0, const SliceSumJob j1, int blocks0) {
     const bool first = static_cast<int>(blockIdx.x) < blocks0;
@@ -378,15 +378,13 @@ __global__ void __launch_bounds__(256) slices_to_gradients_kernel(const SliceSum
         const int col = by * j.bn + pc * 4;
         int row = bx * 128 + rin;
         if (j.conv_c > 0) {      // pairs of 64-channel blocks, ceil(C / 64) blocks per tap
-            const int blks = j.conv_blks, blk = row >> 6, tap = blk / blks, c = (blk - tap * blks) * 64 + (row & 63);
+            const int blks = (j.conv_c + 63) / 64, blk = row >> 6, tap = blk / blks, c = (blk - tap * blks) * 64 + (row & 63);
             row = c < j.conv_c ? tap * j.conv_c + c : j.M;
         }
         if (row >= j.M || col >= j.N) continue;
-        const int S = tile < j.tail ? j.S : j.tail_S;
-        const size_t slice = tile < j.tail ? static_cast<size_t>(tile) * j.S : static_cast<size_t>(j.tail) * j.S + static_cast<size_t>(tile - j.tail) * S;
-        const float* src = j.partial + slice * 128 * j.bn + static_cast<size_t>(in) * 4;
+        const float* src = j.partial + static_cast<size_t>(tile) * j.S * 128 * j.bn + static_cast<size_t>(in) * 4;
         float4 acc = *reinterpret_cast<const float4*>(src);
-        for (int s = 1; s < S; ++s) {
+        for (int s = 1; s < j.S; ++s) {
             const float4 w = *reinterpret_cast<const float4*>(src + static_cast<size_t>(s) * 128 * j.bn);
             acc.x += w.x; acc.y += w.y; acc.z += w.z; acc.w += w.w;
         }
@@ -409,8 +407,7 @@ cudaError_t slices_to_gradients(const SliceSums* jobs, int count, cudaStream_t s
     int blocks[2] = {0, 0};
     for (int i = 0; i < 2; ++i) {
         const SliceSums& s = jobs[i < count ? i : 0];
-        j[i] = SliceSumJob{s.partial, s.out, s.ld, s.M, s.N, s.splits, s.bn, s.tiles_x, s.tiles_y, s.out_f32 ? 1 : 0, s.accumulate ? 1 : 0, s.conv_c,
-                           s.conv_blks > 0 ? s.conv_blks : (s.conv_c + 63) / 64, s.tail > 0 ? s.tail : 0x7fffffff, s.tail_splits};
+        j[i] = SliceSumJob{s.partial, s.out, s.ld, s.M, s.N, s.splits, s.bn, s.tiles_x, s.tiles_y, s.out_f32 ? 1 : 0, s.accumulate ? 1 : 0, s.conv_c};
         if (i < count) {
             const long long total = static_cast<long long>(s.tiles_x) * s.tiles_y * 128 * (s.bn / 4);
             blocks[i] = static_cast<int>(std::min<long long>(ceil_div(total, 256), 4LL * num_sms()));

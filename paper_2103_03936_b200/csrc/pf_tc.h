@@ -30,8 +30,6 @@ struct LinearArgs {
         const float* partial = nullptr;
         int splits = 0, bn = 0, tiles_x = 0, tiles_y = 0;
         int conv_c = 0;     // > 0: tiles are pairs of 64-channel blocks of a [taps][conv_c] row index
-        int conv_blks = 0;  // > 0: that many 64-channel blocks per tap (else the ones that exist)
-        int tail = 0, tail_splits = 0;     // tail > 0: from this tile on there are tail_splits slices
     };
     Slices* du_slices = nullptr;
     Slices* dv_slices = nullptr;
@@ -45,6 +43,10 @@ struct ConvArgs {
     cudaStream_t stream;
     // backward: where the fp32 slices of dU / dV were left (see LinearArgs::Slices); may be null
     LinearArgs::Slices *du_slices, *dv_slices;
+    struct Gradients {            // the caller's matrices, of a call that wants them in fp32 or accumulated
+        void *dU, *dV;
+        bool f32, accumulate, written;      // written: by the launches themselves
+    } * gradients;                // null: dU and dV are the caller's
     bool lean;      // backward, bf16: ws and ws_G have room for the products that fetch pixels per tap only, ws_G with R elements per pixel
 };
 

@@ -198,8 +198,6 @@ tc_conv_dt_dv_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_const
 // Units of 8 rows x 16 columns: a lane sums four columns of a row over all slices, in slice order, sixteen slices in flight.
 struct SumAt {
     int row, col;                // of the result; row -1: none
-    const float4* slices;        // S of them, 2048 apart
-    int S;
     float4 v;
 };
 __device__ __forceinline__ SumAt sum_unit(const SumPart& s, int u, int lane) {
@@ -226,24 +224,45 @@ __device__ __forceinline__ SumAt sum_unit(const SumPart& s, int u, int lane) {
     } else if (row >= s.rows) {
         row = -1;
     }
-    return SumAt{pc * 4 < s.R ? row : -1, pc * 4, src, S, a};
+    return SumAt{pc * 4 < s.R ? row : -1, pc * 4, a};
 }
+// kPlain: bf16, not added to anything, on a 16-byte boundary.
+template <bool kPlain>
 __device__ __forceinline__ void put_sum(const SumPart& s, const SumAt& a) {
-    *reinterpret_cast<uint2*>(s.out + static_cast<size_t>(a.row) * s.R + a.col) = make_uint2(pack_bf16x2(a.v.x, a.v.y), pack_bf16x2(a.v.z, a.v.w));
+    const size_t at = static_cast<size_t>(a.row) * s.R + a.col;
+    if (kPlain) {
+        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(s.out) + at) = make_uint2(pack_bf16x2(a.v.x, a.v.y), pack_bf16x2(a.v.z, a.v.w));
+        return;
+    }
+    const float v[4] = {a.v.x, a.v.y, a.v.z, a.v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (s.f32) {
+            float* o = static_cast<float*>(s.out) + at + e;
+            *o = s.accumulate ? *o + v[e] : v[e];
+        } else {
+            __nv_bfloat16* o = static_cast<__nv_bfloat16*>(s.out) + at + e;
+            *o = __float2bfloat16_rn(s.accumulate ? __bfloat162float(*o) + v[e] : v[e]);
+        }
+    }
 }
 __device__ __forceinline__ bool has_nan(const float4& v) { return v.x != v.x || v.y != v.y || v.z != v.z || v.w != v.w; }
 // One unit per warp and step; returns whether this lane has left out sums that are NaN (kLeave).
-template <bool kLeave>
-__device__ __forceinline__ bool sum_slices(const SumPart& s, int first, int step, int lane) {
+template <bool kLeave, bool kPlain>
+__device__ __forceinline__ bool sum_units(const SumPart& s, int first, int step, int lane) {
     bool left = false;
 #pragma unroll 1
     for (int u = first; u < s.tiles * 64; u += step) {
         const SumAt a = sum_unit(s, u, lane);
         if (a.row < 0) continue;
         if (kLeave && has_nan(a.v)) left = true;
-        else put_sum(s, a);
+        else put_sum<kPlain>(s, a);
     }
     return left;
+}
+template <bool kLeave>
+__device__ __forceinline__ bool sum_slices(const SumPart& s, int first, int step, int lane) {
+    return s.plain ? sum_units<kLeave, true>(s, first, step, lane) : sum_units<kLeave, false>(s, first, step, lane);
 }
 
 // The sums of dU that sum_slices has left out.  The MMAs of tc_conv_du_kernel take the three taps of a row from one tile of x, so they
@@ -311,12 +330,7 @@ __device__ __noinline__ void mend_sums(const DxParams& p, int first, int step, i
                 if (a.v.w != a.v.w) a.v.w = t[3];
             }
         }
-        if (bad) {
-            put_sum(s, a);
-            float4* const to = const_cast<float4*>(a.slices);          // (a caller that wants fp32 adds the slices up again)
-            *to = a.v;
-            for (int i = 1; i < a.S; ++i) to[static_cast<size_t>(i) * 2048u] = make_float4(-0.f, -0.f, -0.f, -0.f);
-        }
+        if (bad) put_sum<false>(s, a);
     }
 }
 
@@ -746,18 +760,24 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
     xp.x = static_cast<const __nv_bfloat16*>(a.x); xp.dT = sp.dT; xp.ldt = sp.ldt;
     xp.a_bytes = b.a_bytes; xp.a_off = 1024; xp.stg_off = 1024 + 2 * b.a_bytes; xp.ring_off = xp.stg_off + 32768;
     xp.num_stages = b.x_stages;
-    xp.sum = SumPart{pu, static_cast<__nv_bfloat16*>(a.dU), 9 * b.tb, b.tb, a.C, a.R, {b.split[0], b.split[1]}, 6 * b.tb};
-    up.sum = SumPart{pv, static_cast<__nv_bfloat16*>(a.dV), b.pairs, 0, a.O, a.R, {b.grid_v, b.grid_v}, b.pairs};
+    // (straight into the caller's matrices, whatever they hold: one more launch would read every slice again)
+    const ConvArgs::Gradients* g = a.gradients;
+    auto part = [&](const float* slices, void* plain, void* user) {
+        SumPart s = {};
+        s.partial = slices;
+        s.out = g ? user : plain;
+        s.f32 = g && g->f32; s.accumulate = g && g->accumulate;
+        s.plain = !s.f32 && !s.accumulate && (reinterpret_cast<uintptr_t>(s.out) & 15) == 0;
+        s.R = a.R;
+        return s;
+    };
+    xp.sum = part(pu, a.dU, g ? g->dU : nullptr);
+    xp.sum.tiles = 9 * b.tb; xp.sum.per_tap = b.tb; xp.sum.rows = a.C;
+    xp.sum.split[0] = b.split[0]; xp.sum.split[1] = b.split[1]; xp.sum.tail = 6 * b.tb;
+    up.sum = part(pv, a.dV, g ? g->dV : nullptr);
+    up.sum.tiles = up.sum.tail = b.pairs; up.sum.rows = a.O;
+    up.sum.split[0] = up.sum.split[1] = b.grid_v;
     xp.status = status;
-    if (a.du_slices) {
-        *a.du_slices = LinearArgs::Slices();
-        a.du_slices->partial = pu; a.du_slices->splits = b.split[0]; a.du_slices->tail_splits = b.split[1]; a.du_slices->tail = 6 * b.tb;
-        a.du_slices->bn = 64; a.du_slices->tiles_x = 9 * b.tb; a.du_slices->tiles_y = 1; a.du_slices->conv_c = a.C; a.du_slices->conv_blks = 2 * b.tb;
-    }
-    if (a.dv_slices) {
-        *a.dv_slices = LinearArgs::Slices();
-        a.dv_slices->partial = pv; a.dv_slices->splits = b.grid_v; a.dv_slices->bn = 64; a.dv_slices->tiles_x = b.pairs; a.dv_slices->tiles_y = 1;
-    }
     auto* dx_kernel = a.R > 48 ? tc_conv_dx_kernel<true> : tc_conv_dx_kernel<false>;
     const size_t smem_u = 1024 + 1024 + kDuStages * kDuStage;
     if (allow_smem(tc_conv_dt_dv_kernel, 227 * 1024) != cudaSuccess || allow_smem(tc_conv_du_kernel, smem_u) != cudaSuccess ||
@@ -772,6 +792,7 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
     xp.step = xp.tiles > 0 ? even_grid(xp.tiles) : 1;
     if (launch_overlapped(dx_kernel, dim3(static_cast<unsigned>(num_sms())), dim3(kDxThreads), b.smem_x, a.stream, xa, xb, xp) != cudaSuccess) return PF_ERR_CUDA;
     count_launch();
+    if (a.gradients) a.gradients->written = true;
     return PF_OK;
 }
 

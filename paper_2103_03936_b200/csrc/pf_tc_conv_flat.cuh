@@ -94,7 +94,8 @@ struct DtDvParams {
 };
 struct SumPart {
     const float* partial;
-    __nv_bfloat16* out;
+    void* out;                   // fp32 or bf16, added to what it holds or not; plain: neither, on a 16-byte boundary
+    int f32, accumulate, plain;
     int tiles, per_tap, rows, R;             // tiles of 128 rows; per_tap > 0: tile = tap * per_tap + block of 128 of `rows` rows per tap
     int split[2], tail;                      // slices of the tiles before `tail`, and from there on
 };

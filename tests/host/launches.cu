@@ -69,11 +69,11 @@ void check(const pf::tc::DtDvParams& p, unsigned blocks) {
 }
 void check(const pf::tc::DuParams& p) {
     writes("slices of dU of a convolution", address(p.partial), static_cast<uint64_t>(6 * p.split[0] + 3 * p.split[1]) * p.tb * kSlice);
-    writes("dV of a convolution", address(p.sum.out), matrix(p.sum.rows, p.sum.R, p.sum.R, 2));
+    writes("dV of a convolution", address(p.sum.out), matrix(p.sum.rows, p.sum.R, p.sum.R, p.sum.f32 ? 4 : 2));
 }
 void check(const pf::tc::DxParams& p) {
     if (p.tiles > 0) writes("dX of a convolution", address(p.out), matrix(static_cast<int64_t>(p.f.N) * p.f.H * p.f.W, p.C, p.C, 2));
-    writes("dU of a convolution", address(p.sum.out), matrix(static_cast<int64_t>(9) * p.sum.rows, p.sum.R, p.sum.R, 2));
+    writes("dU of a convolution", address(p.sum.out), matrix(static_cast<int64_t>(9) * p.sum.rows, p.sum.R, p.sum.R, p.sum.f32 ? 4 : 2));
 }
 void check(const pf::SimtGemm& g) {
     const int64_t size = g.dtype == PF_BF16 ? 2 : 4;

@@ -283,6 +283,36 @@ def test_flat_backward(N, H, W, C, R, O):
     assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
 
 
+@pytest.mark.parametrize("N,H,W,C,R,O", [(45, 16, 16, 320, 40, 72), (13, 33, 63, 72, 24, 72), (60, 28, 28, 128, 8, 128)])
+def test_flat_backward_into_the_callers_sums(N, H, W, C, R, O):
+    """Gradients in fp32 or accumulated come from the launches of the plain ones, wherever the matrices lie: the fp32 sums that
+    the plain ones are rounded from, added once to what was there."""
+    c = wl.ConvCase("sums", N, H, W, C, R, O, wl.BF16, 94)
+    run_conv(c, need_dX=False)
+    d = c.generate()
+    x, U, V, dY = (dev(d[k_], wl.BF16) for k_ in ("x", "U", "V", "dY"))
+    T = pf.pf_lowrank_conv_fwd(x, U, V, want_stash=True)[1]
+    for dX in (True, False):
+        before = pf.pf_launch_count()
+        _, *plain = pf.pf_lowrank_conv_bwd(x, U, V, dY, T_stash=T, need_dX=dX)
+        launches = pf.pf_launch_count() - before
+        sums = None
+        for dtype in (torch.float32, torch.bfloat16):
+            for accumulate in (False, True):
+                for offset in (0, 1):
+                    out = [torch.full((g.numel() + 1,), 0.5, dtype=dtype, device="cuda")[offset:offset + g.numel()].view(g.shape) for g in plain]
+                    before = pf.pf_launch_count()
+                    pf.pf_lowrank_conv_bwd(x, U, V, dY, T_stash=T, need_dX=dX, dU=out[0], dV=out[1], accumulate=accumulate, grads_f32=dtype == torch.float32)
+                    if accumulate or dtype == torch.float32:
+                        assert pf.pf_launch_count() - before == launches
+                    torch.cuda.synchronize()
+                    if sums is None:
+                        sums = [o.clone() for o in out]
+                        assert all(torch.equal(s.bfloat16(), g) for s, g in zip(sums, plain))
+                    if dtype == torch.float32 or accumulate or offset == 0:      # (plain matrices off a 16-byte boundary take the other form)
+                        assert all(torch.equal(o, ((s + 0.5) if accumulate else s).to(dtype)) for o, s in zip(out, sums)), (dX, dtype, accumulate, offset)
+
+
 @pytest.mark.parametrize("N,H,W,C,R,O,stride,room", [(45, 16, 16, 320, 40, 72, 1, 10154752), (140, 9, 13, 136, 24, 136, 1, 8250624),
                                                      (60, 15, 14, 40, 24, 40, 2, 6124800)])
 def test_backward_in_the_least_workspace(N, H, W, C, R, O, stride, room):
