@@ -699,23 +699,29 @@ bool flat_bwd_plan(int N, int H, int W, int C, int R, int O, int kh, int kw, int
 }
 }  // namespace
 
-// Against the launches that fetch pixels per tap (old / here, cold L2).  Rows of dT and U that straddle lines are what those suffer from, so
-// at ranks of 24, 40 or 56 these pay early: 160 -> 40 -> 160 of 6272 pixels 23.2 / 25.9 us, 12544 36.4 / 31.3, 50176 96.5 / 59.8; 128 -> 40 -> 128
-// of 12544 24.0 / 24.9, 25088 37.5 / 29.7; 64 -> 24 -> 64 of 12544 20.1 / 24.6, 25088 30.9 / 30.2.  At 48: 192 -> 48 -> 192 of 12544 23.2 / 28.1, 25088
-// 36.0 / 32.4; 128 -> 48 -> 256 of 25088 26.7 / 30.4, 50176 41.2 / 40.7.  Elsewhere the starts of three launches and the sums of the slices (10 to 20
-// us) want more: 256 -> 64 -> 256 of 25088 31.5 / 34.4, 65536 60.2 / 55.3, 131072 111.6 / 89.4; 128 -> 32 -> 128 of 25088 23.7 / 26.5, 100352 63.4 / 50.9; an
-// expected time decides, fitted to 77 such backwards (most within 7 and 9 %; three of them more than 3 % slower than the better form).
-bool conv_flat_bwd_pays(const ConvArgs& a) {
+// Against the launches that fetch pixels per tap (those / here, passes over buffers that do not fit L2; both with dT at a pitch of whole
+// lines).  Rows of dT and U that straddle lines are what those suffer from, so at ranks of 24, 40 or 56 these pay early: 160 -> 40 -> 160 of 12544
+// pixels 37.8 / 31.9 us, 50176 107.0 / 56.1; 64 -> 24 -> 64 of 12544 21.4 / 26.2, 25088 32.3 / 29.9; 448 -> 56 -> 448 of 12544 48.9 / 45.9; wide
+// y later: 320 -> 56 -> 512 of 15680 42.0 / 46.6, 320 -> 24 -> 512 of 9200 39.3 / 40.5.  At 48: 192 -> 48 -> 192 of 12544 23.9 / 28.4, 25088
+// 37.3 / 33.5.  Elsewhere the starts of three launches and the sums of the slices (10 to 20 us) want more: 256 -> 64 -> 256 of 25088
+// 32.0 / 33.4, 50176 51.0 / 47.7, 131072 111.4 / 85.6; 128 -> 32 -> 128 of 25088 24.5 / 26.5, 100352 64.4 / 47.5; an expected time decides, fitted to an earlier
+// state of these kernels, so it keeps to the other form up to 12 % beyond the crossing (512 -> 64 -> 512 of 25088 56.2 / 51.3).
+// Without dX the other form has two launches and these still three, of which dX's share was the larger gain, so the line
+// is a work of reductions (pixels times channels) that grows with the channels' slices: 192 -> 48 -> 192 of 25088 23.2 / 30.3, 75264 45.1 / 43.2;
+// 256 -> 64 -> 256 of 50176 37.6 / 37.7, 75264 50.9 / 44.5; 64 -> 32 -> 64 of 131072 34.6 / 39.0; 160 -> 40 -> 160 of 12544 23.2 / 25.4, 37632 45.7 / 37.6;
+// 64 -> 24 -> 64 of 51200 31.6 / 33.1, 75264 36.5 / 35.7; 512 -> 24 -> 512 of 8000 31.6 / 35.2.
+bool conv_flat_bwd_pays(const ConvArgs& a, bool dX) {
     FlatBwd b;
     if (!flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b)) return false;
     const double c = a.C / 100.0, p = static_cast<double>(a.N) * a.H * a.W / 1000.0, pc = p * c, po = p * a.O / 100.0;
-    if (64 % a.R != 0) return a.R % 16 != 0 ? p >= (a.C >= 160 ? 11.0 : a.C >= 96 ? 16.0 : 25.0) : p >= (a.C >= 160 ? 20.0 : 50.0);
+    if (!dX) return pc >= (64 % a.R == 0 || a.R >= 48 ? (a.C > 64 ? 130.0 : 260.0) : a.R >= 40 ? 48.0 : 28.0 + 12.0 * c);
+    if (64 % a.R != 0) return a.R % 16 != 0 ? p >= (a.C >= 160 ? (a.O > a.C ? 18.0 : 11.0) : a.C >= 96 ? 16.0 : 25.0) : p >= (a.C >= 160 ? 20.0 : 50.0);
     return p >= 2.0 && 14.6 + 3.58 * c + 0.23 * p + 0.07 * pc + 0.05 * po < (a.R > 32 ? 0.9 : 1.05) * (12.35 + 0.07 * c + 0.16 * p + 0.19 * pc + 0.07 * po);
 }
 
 size_t conv_flat_bwd_workspace(const ConvArgs& a) {
     FlatBwd b;
-    return conv_flat_bwd_pays(a) && flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b) ? b.bytes_u + b.bytes_v : 0;
+    return (conv_flat_bwd_pays(a, true) || conv_flat_bwd_pays(a, false)) && flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b) ? b.bytes_u + b.bytes_v : 0;
 }
 
 // T: the stash, or x * U as a launch before left it.

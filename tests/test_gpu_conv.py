@@ -283,7 +283,7 @@ def test_flat_backward(N, H, W, C, R, O):
     assert torch.equal(dU1.to(dU0.dtype), dU0) and torch.equal(dV1.to(dV0.dtype), dV0)
 
 
-@pytest.mark.parametrize("N,H,W,C,R,O", [(45, 16, 16, 320, 40, 72), (13, 33, 63, 72, 24, 72), (60, 28, 28, 128, 8, 128)])
+@pytest.mark.parametrize("N,H,W,C,R,O", [(80, 16, 16, 320, 40, 72), (70, 28, 28, 72, 24, 72), (27, 33, 63, 264, 8, 72)])
 def test_flat_backward_into_the_callers_sums(N, H, W, C, R, O):
     """Gradients in fp32 or accumulated come from the launches of the plain ones, wherever the matrices lie: the fp32 sums that
     the plain ones are rounded from, added once to what was there."""
@@ -296,6 +296,7 @@ def test_flat_backward_into_the_callers_sums(N, H, W, C, R, O):
         before = pf.pf_launch_count()
         _, *plain = pf.pf_lowrank_conv_bwd(x, U, V, dY, T_stash=T, need_dX=dX)
         launches = pf.pf_launch_count() - before
+        assert launches == (4 if dX and R % 16 and 64 % R else 3)        # (dX reads a copy of U)
         sums = None
         for dtype in (torch.float32, torch.bfloat16):
             for accumulate in (False, True):
@@ -311,6 +312,20 @@ def test_flat_backward_into_the_callers_sums(N, H, W, C, R, O):
                         assert all(torch.equal(s.bfloat16(), g) for s, g in zip(sums, plain))
                     if dtype == torch.float32 or accumulate or offset == 0:      # (plain matrices off a 16-byte boundary take the other form)
                         assert all(torch.equal(o, ((s + 0.5) if accumulate else s).to(dtype)) for o, s in zip(out, sums)), (dX, dtype, accumulate, offset)
+
+
+@pytest.mark.parametrize("N,H,W,C,R,O,without", [
+    (32, 28, 28, 192, 48, 192, 2), (90, 28, 28, 192, 48, 192, 3), (28, 28, 28, 64, 24, 64, 2), (64, 28, 28, 64, 24, 64, 3), (20, 20, 20, 512, 24, 512, 2),
+    (20, 28, 28, 448, 56, 448, 2), (16, 28, 28, 160, 40, 160, 2), (48, 28, 28, 160, 40, 160, 3), (130, 32, 32, 64, 32, 64, 2)])
+def test_backward_without_dX_chooses_for_itself(N, H, W, C, R, O, without):
+    """What dX gains does not count for a call that does not want it."""
+    x, U, V, dY = (torch.zeros(*s, dtype=torch.bfloat16, device="cuda") for s in ((N, H, W, C), (3, 3, C, R), (O, R), (N, H, W, O)))
+    T = torch.zeros(N, H, W, R, dtype=torch.bfloat16, device="cuda")
+    before = pf.pf_launch_count()
+    pf.pf_lowrank_conv_bwd(x, U, V, dY, T_stash=T, need_dX=False)
+    assert pf.pf_launch_count() - before == without
+    if C * R <= 160 * 48 and N < 64:
+        run_conv(wl.ConvCase("no dX", N, H, W, C, R, O, wl.BF16, 93), need_dX=False)
 
 
 @pytest.mark.parametrize("N,H,W,C,R,O,stride,room", [(45, 16, 16, 320, 40, 72, 1, 10154752), (140, 9, 13, 136, 24, 136, 1, 8250624),
