@@ -1258,14 +1258,16 @@ int conv_fwd(const ConvArgs& a, int* handled) {
     int64_t ldf = a.R;
     if (copy > 0) {
         ldf = conv_dt_pitch(a.R);
-        const RepackJob jobs[2] = {RepackJob{a.U, a.R, a.ws, ldf, Keff, a.R}, RepackJob{a.V, a.R, a.ws + copy, ldf, a.O, a.R}};
-        if (repack_rows_bf16_multi(jobs, 2, a.stream) != cudaSuccess) return PF_ERR_CUDA;
         b.U = a.ws;
         b.V = a.ws + copy;
     }
-    int st = conv_res_fwd(b, ldf);
-    if (st == PF_ERR_UNSUPPORTED) st = chain(b.x, b.C, 0, 0, b.U, ldf, b.R, b.V, ldf, b.O, b.y, b.O, b.T, b.R, b.stream, &cv);
-    if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing but the copies has been launched
+    const Before copies = [&] {
+        const RepackJob jobs[2] = {RepackJob{a.U, a.R, a.ws, ldf, Keff, a.R}, RepackJob{a.V, a.R, a.ws + copy, ldf, a.O, a.R}};
+        return copy == 0 || repack_rows_bf16_multi(jobs, 2, a.stream) == cudaSuccess ? PF_OK : PF_ERR_CUDA;
+    };
+    int st = conv_res_fwd(b, ldf, copies);
+    if (st == PF_ERR_UNSUPPORTED) st = chain(b.x, b.C, 0, 0, b.U, ldf, b.R, b.V, ldf, b.O, b.y, b.O, b.T, b.R, b.stream, &cv, 0, nullptr, 0, 0.f, 0.f, copies);
+    if (st == PF_ERR_UNSUPPORTED) return PF_OK;      // declined: nothing has been launched
     *handled = 1;
     return st;
 }

@@ -4,6 +4,8 @@
 #ifndef PF_TC_H_
 #define PF_TC_H_
 
+#include <functional>
+
 #include "pf_internal.h"
 
 namespace pf {
@@ -50,6 +52,9 @@ struct ConvArgs {
     bool lean;      // backward, bf16: ws and ws_G have room for the products that fetch pixels per tap only, ws_G with R elements per pixel
 };
 
+// Launches that what follows reads: made once a call is accepted, i.e. when nothing can decline it any more.
+using Before = std::function<int()>;
+
 // Fused chain kernel (pf_tc_chain.cu): out = (A * B1) * B2^T with the intermediate on chip.
 struct ChainPlan {
     int r_pad, num_stages, stage_bytes, nsplit, tiles_per_split, row_tiles, boxes_per_stage, staging_off;
@@ -75,7 +80,8 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
           const void* B2, int64_t ldb2, int64_t N2, void* out, int64_t ldo, void* T, int64_t ldt,
           cudaStream_t stream, const ChainConv* conv = nullptr, int max_split = 0, const void* bias = nullptr,
           int act = 0,    // bias [N2] (bf16) and act (0 identity, 1 max(0, .)) apply to `out`
-          float keep_a = 0.f, float keep_out = 0.f);      // how L2 treats A and `out` (l2_policy in pf_tc_prims.cuh)
+          float keep_a = 0.f, float keep_out = 0.f,       // how L2 treats A and `out` (l2_policy in pf_tc_prims.cuh)
+          const Before& before = {});
 
 int chain_groups(int groups, int all, const void* A, int64_t lda, int64_t sA, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t sB1, int64_t r,
                  const void* B2, int64_t ldb2, int64_t sB2, int64_t N2, void* out, int64_t ldo, int64_t sO, void* T, int64_t ldt, int64_t sT,
@@ -142,7 +148,7 @@ int f32_conv_bwd(const ConvArgs& a, int* handled);
 // Device counters for one product whose contraction is split (null on error).
 unsigned int* split_counters();
 // 3 x 3, stride-1 convolutions on resident image windows (pf_tc_conv_res.cu); PF_ERR_UNSUPPORTED outside their envelope.
-int conv_res_fwd(const ConvArgs& a, int64_t ldf);      // ldf: pitch of the factors
+int conv_res_fwd(const ConvArgs& a, int64_t ldf, const Before& before);      // ldf: pitch of the factors
 // Their backward (pf_tc_conv_bwd.cu), where `conv_flat_bwd_pays`; T is x U, a.ws_G takes dT.
 bool conv_flat_bwd_pays(const ConvArgs& a, bool dX);      // a: sizes only
 size_t conv_flat_bwd_workspace(const ConvArgs& a);      // a: sizes only; 0 where it does not pay

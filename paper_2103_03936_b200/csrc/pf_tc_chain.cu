@@ -69,7 +69,7 @@ bool chain_plan(int64_t M, int64_t K1, int64_t N2, int64_t r, bool has_out, Chai
 // matrices that are written tma_out.
 int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int64_t ldb1, int64_t r,
           const void* B2, int64_t ldb2, int64_t N2, void* out, int64_t ldo, void* T, int64_t ldt,
-          cudaStream_t stream, const ChainConv* conv, int max_split, const void* bias, int act, float keep_a, float keep_out) {
+          cudaStream_t stream, const ChainConv* conv, int max_split, const void* bias, int act, float keep_a, float keep_out, const Before& before) {
     ChainPlan plan;
     const int cs = conv ? conv->stride : 1;
     const int Ho = conv ? (conv->H + 2 * conv->pad - conv->kh) / cs + 1 : 1;
@@ -107,6 +107,8 @@ int chain(const void* A, int64_t lda, int64_t M, int64_t K1, const void* B1, int
         ok = ok && (T ? cached_map_2d(&tt, T, M, r, ldt, rows_tile) : cached_map_2d(&tt, B2, N2, r, ldb2, 128));
     }
     if (!ok) return PF_ERR_CUDA;
+    const int st = before ? before() : PF_OK;
+    if (st != PF_OK) return st;
     ChainParams p;
     p.M = static_cast<int>(M); p.K1 = static_cast<int>(K1); p.N2 = static_cast<int>(N2);
     // Zeros behind the rank for any number of rows, as the unfused products have them: 0.1 us where the rank is no multiple of

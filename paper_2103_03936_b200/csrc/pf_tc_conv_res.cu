@@ -330,7 +330,7 @@ void fill(ResParams* p, const FlatImage& f, const ResLayout& l, const ConvArgs& 
 }
 }  // namespace
 
-int conv_res_fwd(const ConvArgs& a, int64_t ldf) {
+int conv_res_fwd(const ConvArgs& a, int64_t ldf, const Before& before) {
     if (!res_shape(a)) return PF_ERR_UNSUPPORTED;
     const FlatImage f = flat_image(a);
     ResLayout l;
@@ -351,9 +351,10 @@ int conv_res_fwd(const ConvArgs& a, int64_t ldf) {
     const bool ok = window_map(&ta, f, a.x, a.C) &&
                     (p.ragged ? cached_map_planes(&tb1, a.U, 9, a.C, a.R, a.C, 64, ldf) : cached_map_2d(&tb1, a.U, static_cast<int64_t>(9) * a.C, a.R, ldf, 64)) &&
                     cached_map_2d(&tb2, a.V, a.O, a.R, ldf, 64);
-    if (!ok) return PF_ERR_CUDA;
-    if (allow_smem(tc_conv_res_kernel, 227 * 1024) != cudaSuccess ||
-        launch_overlapped(tc_conv_res_kernel, dim3(static_cast<unsigned>(even_grid(p.tiles))), dim3(kResThreads), l.smem, a.stream, ta, tb1, tb2, p) != cudaSuccess)
+    if (!ok || allow_smem(tc_conv_res_kernel, 227 * 1024) != cudaSuccess) return PF_ERR_CUDA;
+    const int st = before();
+    if (st != PF_OK) return st;
+    if (launch_overlapped(tc_conv_res_kernel, dim3(static_cast<unsigned>(even_grid(p.tiles))), dim3(kResThreads), l.smem, a.stream, ta, tb1, tb2, p) != cudaSuccess)
         return PF_ERR_CUDA;
     count_launch();
     return PF_OK;
