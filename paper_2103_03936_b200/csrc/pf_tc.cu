@@ -1292,16 +1292,15 @@ int conv_bwd(const ConvArgs& a, int* handled) {
     const bool copy = a.dX && copy_bytes > 0;      // of U for dX; the launch that makes dT runs beside it
     char* const ws = a.ws + copy_bytes;
     const Operand U{copy ? a.ws : a.U, copy ? ldt : a.R, false, 0, false, true};
-    auto copy_factor = [&] {
+    const Before first = [&] {          // x U where there is no stash, and the copy of U
+        const int rc = a.T ? PF_OK : recompute();
         const RepackJob job{a.U, a.R, a.ws, ldt, Keff, a.R};
-        return !copy || repack_rows_bf16_multi(&job, 1, a.stream) == cudaSuccess ? PF_OK : PF_ERR_CUDA;
+        return rc != PF_OK || !copy || repack_rows_bf16_multi(&job, 1, a.stream) == cudaSuccess ? rc : PF_ERR_CUDA;
     };
     if (flat) {
-        st = a.T ? PF_OK : recompute();
-        if (st == PF_ERR_UNSUPPORTED) return PF_OK;
-        *handled = 1;
-        if (st == PF_OK) st = copy_factor();
-        return st == PF_OK ? conv_flat_bwd(a, T, U.p, U.ld, ws, copy) : st;
+        st = conv_flat_bwd(a, T, U.p, U.ld, ws, copy, first);
+        *handled = st != PF_ERR_UNSUPPORTED;
+        if (*handled) return st;
     }
     // Every product is prepared (tensor maps, geometry; nothing launched) before the call is
     // accepted, so a shape that one of them cannot take still reaches the FMA kernels.
@@ -1332,13 +1331,9 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         gt.grid = dim3(static_cast<unsigned>(ceil_div(gt_tiles, std::min<int64_t>(4, ceil_div(gt_tiles, 2 * num_sms())))));
         gt.p.num_stages = pick_stages(gt.bn, gt.grid.x, true);
     }
-    if (!a.T) {
-        st = recompute();
-        if (st == PF_ERR_UNSUPPORTED) return PF_OK;
-        if (st != PF_OK) return st;
-    }
+    st = first();
+    if (st == PF_ERR_UNSUPPORTED) return PF_OK;
     *handled = 1;
-    st = copy_factor();
     if (st != PF_OK) return st;
     const bool narrow = narrow_reductions(conv_du_tiles(a.kh, a.kw, a.C) * kBM, a.O, a.R);
     keep_slices(a.du_slices, &gu, narrow ? pu : SliceRoom(), a.C);

@@ -149,10 +149,11 @@ int f32_conv_bwd(const ConvArgs& a, int* handled);
 unsigned int* split_counters();
 // 3 x 3, stride-1 convolutions on resident image windows (pf_tc_conv_res.cu); PF_ERR_UNSUPPORTED outside their envelope.
 int conv_res_fwd(const ConvArgs& a, int64_t ldf, const Before& before);      // ldf: pitch of the factors
-// Their backward (pf_tc_conv_bwd.cu), where `conv_flat_bwd_pays`; T is x U, a.ws_G takes dT.
+// Their backward (pf_tc_conv_bwd.cu), where `conv_flat_bwd_pays`; T is x U, a.ws_G takes dT.  PF_ERR_UNSUPPORTED: nothing has been launched.
 bool conv_flat_bwd_pays(const ConvArgs& a, bool dX);      // a: sizes only
 size_t conv_flat_bwd_workspace(const ConvArgs& a);      // a: sizes only; 0 where it does not pay
-int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early);     // early: the launch before copies U, nothing else
+int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early,     // early: the launch before copies U, nothing else
+                  const Before& before);
 int conv_fwd(const ConvArgs& a, int* handled);
 int conv_bwd(const ConvArgs& a, int* handled);      // a.ws_G: conv_dt_pitch(R) elements per pixel, unless lean
 int64_t conv_dt_pitch(int64_t R);

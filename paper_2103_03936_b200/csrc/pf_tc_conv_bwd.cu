@@ -725,7 +725,7 @@ size_t conv_flat_bwd_workspace(const ConvArgs& a) {
 }
 
 // T: the stash, or x * U as a launch before left it.
-int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early) {
+int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early, const Before& before) {
     FlatBwd b;
     if (encode_fn() == nullptr || !flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b)) return PF_ERR_UNSUPPORTED;
     const int64_t P = static_cast<int64_t>(a.N) * a.H * a.W;
@@ -738,7 +738,7 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
                     cached_map_nhwc(&ux, a.x, a.N, a.H, a.W, a.C, b.wx, b.ct.bh, b.ct.nb, 1) &&
                     cached_map_nhwc(&ut, a.ws_G, a.N, a.H, a.W, a.R, a.W + 1, b.ct.bh, b.ct.nb, 1, ldt) && window_map(&xa, b.f, a.ws_G, a.R, ldt) &&
                     cached_map_2d(&xb, U, static_cast<int64_t>(9) * a.C, a.R, ldu, 128);
-    if (!ok) return PF_ERR_CUDA;
+    if (!ok) return PF_ERR_UNSUPPORTED;
     DtDvParams sp = {};
     sp.rows = static_cast<int>(P); sp.O = a.O; sp.R = a.R;
     sp.tiles = static_cast<int>(ceil_div(P, 128));
@@ -788,7 +788,9 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
     const size_t smem_u = 1024 + 1024 + kDuStages * kDuStage;
     if (allow_smem(tc_conv_dt_dv_kernel, 227 * 1024) != cudaSuccess || allow_smem(tc_conv_du_kernel, smem_u) != cudaSuccess ||
         allow_smem(dx_kernel, 227 * 1024) != cudaSuccess)
-        return PF_ERR_CUDA;
+        return PF_ERR_UNSUPPORTED;
+    const int st = before();
+    if (st != PF_OK) return st;
     if (launch_overlapped(tc_conv_dt_dv_kernel, dim3(static_cast<unsigned>(b.grid_v)), dim3(kStreamThreads), b.smem_v, a.stream, y, t, v, sp) != cudaSuccess) return PF_ERR_CUDA;
     count_launch();
     const int du_blocks = b.tb * b.split[0] + static_cast<int>(ceil_div(b.tb, 2)) * b.split[1];

@@ -149,7 +149,12 @@ void host_regions(int count, const uint64_t* base, const uint64_t* bytes) {
 const char* host_faults() { return faults.c_str(); }
 const char* host_launches() { return launches.c_str(); }
 
+// Kernels whose name holds `part` (null: none) get no shared memory beyond the default.
+static std::string refused;
+void host_refuse(const char* part) { refused = part ? part : ""; }
+
 // For runtime.cpp:
+bool host_refuses(const void* kernel) { return !refused.empty() && kernels()[kernel].find(refused) != std::string::npos; }
 void host_kernel(const void* host, const char* name) { kernels()[host] = name; }
 void host_array(const void* host, size_t bytes) {
     static uint64_t next = 1ull << 60;

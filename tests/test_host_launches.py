@@ -32,3 +32,24 @@ def test_nothing_reaches_outside_the_buffers_of_a_call(host_library, kind):
                           timeout=300)
     assert done.returncode == 0, done.stderr
     assert done.stdout == "calls reaching outside their buffers: 0\n", done.stdout[:4000]
+
+
+@pytest.mark.parametrize("kernel", ["tc_conv_dt_dv_kernel", "tc_conv_du_kernel", "tc_conv_dx_kernel"])
+def test_a_backward_that_cannot_be_prepared_launches_nothing_of_itself(host_library, kernel):
+    """Convolution backward in three launches: what cannot be prepared leaves the call to the products that fetch pixels per
+    tap, before x U has been recomputed or U copied for it."""
+    code = f"""
+import sys
+sys.path.insert(0, {HOST!r})
+import calls
+lib = calls.Library({host_library!r})
+lib.L.host_refuse({kernel.encode()!r})
+status, faults, launches = calls.conv(lib, 64, 28, 28, 160, 40, 160, 3, 1, 1, calls.BF16, bwd=True, stash=False)
+assert status == 0 and not faults, (status, faults)
+kernels = launches.split()
+named = lambda part: sum(part in k for k in kernels)
+assert not named("tc_conv_d") and named("tc_gemm") == 2, launches
+assert named("tc_conv_res_kernel") + named("tc_chain") == 1 and named("repack") == 1, launches
+"""
+    done = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stderr
