@@ -1219,21 +1219,46 @@ void conv_partial_bytes(const ConvA& c, int O, int su, int sv, size_t* bytes_u, 
 // 16 x 14 x 14, 160 -> 40 -> 160 18.9 -> 16.6 us, of 8 x 28 x 28, 192 -> 48 -> 192 18.9 -> 16.6, stride 2 of 64 x 14 x 14, 256 -> 72 -> 256 22.0 -> 19.9.
 // (Ranks that only the FMA kernels take have no such rows.)
 int64_t conv_dt_pitch(int64_t R) { return R % 64 == 0 || 64 % R == 0 || R % 8 != 0 || R > kConvMaxRank ? R : (R + 63) / 64 * 64; }
-// dX reads U once per tile, so for many pixels it too is copied to that pitch, beside the launch that makes dT (64 x 28 x 28: 320 -> 80 ->
-// 320 110.1 -> 99.8 us, 320 -> 40 -> 320 90.6 -> 79.4; 8 x 28 x 28 of it 33.2 -> 34.2; rows of 96 bytes take no harm: 192 -> 48 -> 192 46.9 -> 48.3).
-// The forward copies both factors, and from fewer pixels on: every block reads all of U, a box of 64 ranks' rows in up to twice
-// the requests.  28 x 28 images, 160 -> 40 -> 160: N = 64 30.9 -> 26.4 us, 16 17.9 -> 14.8, 4 11.8 -> 13.2; 96 -> 24 -> 96: N = 16 15.4 ->
-// 12.8, 8 9.4 -> 12.8; 256 -> 72 -> 256, N = 64 69.7 -> 47.6; 768 -> 200 -> 768, N = 64 260 -> 229; 192 -> 48 -> 192, N = 128 34.9 -> 35.9.
-static size_t conv_factor_copy(int64_t pixels, int64_t Keff, int64_t R, bool fwd) {
-    if (pixels < (fwd ? 12000 : 20000) || conv_dt_pitch(R) == R || R % 8 || (R < 64 && R % 16 == 0)) return 0;
-    return align_up(static_cast<size_t>(Keff) * conv_dt_pitch(R) * 2, 256);
+// dX reads U once per tile, so for many pixels it too is copied to that pitch, beside the launch that makes dT; the forward copies both
+// factors, and from fewer pixels on: every block reads all of U, a box of 64 ranks' rows in up to twice the requests.  What that
+// saves depends on how the rows lie, what it costs is a launch, so the lines are measured (passes over buffers that do not fit L2, without
+// and with copies; C is 2 or 4 ranks wide, square y):
+//   rows at an odd multiple of 16 bytes.  Above 64 ranks they gain most: forward 3 x 3, 12544 pixels: 72 26 -> 22 us, 120 35 -> 28, 136 45 -> 34, 184
+//     56 -> 46; one tap gains later (72: 12544 pixels 9.0 -> 9.4, 25088 13 -> 11; 136: 12544 16.2 -> 15.6).  24 and 40 ranks: 3 x 3 of 12544 15.0 -> 13.7 and 17.5
+//     -> 16.9, of 25088 21 -> 18 and 19.2 -> 18.2; one tap of 12544 8.7 -> 8.8 and 8.6 -> 9.5, of 25088 13 -> 11 and 13 -> 12; 5 x 5 of
+//     40 12544 31.7 -> 32.4, 25088 60 -> 57, but 96 -> 24 -> 96 of 100352 129 -> 136 (3 x 3: 32.7 -> 29.3).  56 ranks are
+//     nearly a line: 5 x 5 of 25088 43 -> 41, else 3 x 3 of 12544 13.8 -> 14.5, of 25088 17.0 -> 17.6, one tap 11.1 -> 11.6.
+//   rows at an odd multiple of 32 bytes, above 64 ranks: 3 x 3 of 25088: 80 37 -> 34, 112 47 -> 45, 144 62 -> 61, 176 84 -> 79; of 12544 within 2 %, one tap
+//     slower (80: 9.5 -> 10.7).  (48 ranks: 3 x 3 of 100352 34.9 -> 35.9.)
+//   rows at a multiple of 64 bytes: 96 13.9 -> 15.5 (12544), 39.0 -> 39.4 (25088); 160 73.0 -> 72.8.
+// Backward, stride 1 and more taps than one: 80 of 25088 51 -> 44, 120 70 -> 59, 184 222 -> 207, 24 45 -> 41, 40 43 -> 41, 96 46 -> 44; 56 36 -> 37, of 50176
+// 53 -> 52.  Stride 2 gains above 64 ranks with rows at odd multiples of 16 bytes (72 101 -> 94; 24 44 -> 44, 80 57 -> 58, 96 58 -> 60); one tap
+// does not (40 26 -> 28, 56 36 -> 39, 120 30 -> 30, 144 46 -> 48), nor 5 x 5 of many pixels (80 -> 40 -> 80 of 100352 262 -> 279).
+static size_t conv_factor_copy(int64_t pixels, int kernel, int64_t C, int64_t R, int stride, bool fwd) {
+    if (conv_dt_pitch(R) == R || (R < 64 && R % 16 == 0)) return 0;
+    const bool odd16 = R % 16 != 0, wide = R > 64;
+    int64_t least;
+    if (!fwd) {
+        if (kernel == 1 || (stride > 1 && !(odd16 && wide)) || (kernel > 3 && !wide && pixels > 80000)) return 0;
+        least = R == 56 ? 40000 : 20000;
+    } else if (!odd16) {
+        if (R % 32 == 0 || kernel == 1) return 0;
+        least = 20000;
+    } else if (wide) {
+        least = kernel == 1 && R < 128 ? 20000 : 12000;
+    } else {
+        if (R == 56 && kernel < 5) return 0;
+        if (kernel > 3 && C < 128 && pixels > 80000) return 0;
+        least = R == 24 && kernel > 1 ? 12000 : 20000;
+    }
+    return pixels < least ? 0 : align_up(static_cast<size_t>(kernel) * kernel * C * conv_dt_pitch(R) * 2, 256);
 }
 
 size_t conv_extra_workspace(int N, int H, int W, int C, int R, int O, int kh, int kw, int stride, int pad,
                             bool bwd, bool lean) {
     const int Ho = (H + 2 * pad - kh) / stride + 1, Wo = (W + 2 * pad - kw) / stride + 1;
     if (N < 1 || Ho < 1 || Wo < 1) return 0;
-    const size_t copy = lean ? 0 : conv_factor_copy(static_cast<int64_t>(N) * Ho * Wo, static_cast<int64_t>(kh) * kw * C, R, !bwd);
+    const size_t copy = lean ? 0 : conv_factor_copy(static_cast<int64_t>(N) * Ho * Wo, kh, C, R, stride, !bwd);
     if (!bwd) return copy > 0 ? copy + align_up(static_cast<size_t>(O) * conv_dt_pitch(R) * 2, 256) : 0;
     const ConvA c{2, N, H, W, C, R, Ho, Wo, kh, kw, pad, stride};
     int su, sv;
@@ -1253,7 +1278,7 @@ int conv_fwd(const ConvArgs& a, int* handled) {
     const ChainConv cv{a.N, a.H, a.W, a.C, a.kh, a.kw, a.pad, a.stride};
     // the factors at a pitch of whole lines, where the caller's scratch holds the copies
     const int64_t Keff = static_cast<int64_t>(a.kh) * a.kw * a.C;
-    const size_t copy = a.ws ? conv_factor_copy(static_cast<int64_t>(a.N) * a.Ho * a.Wo, Keff, a.R, true) : 0;
+    const size_t copy = a.ws ? conv_factor_copy(static_cast<int64_t>(a.N) * a.Ho * a.Wo, a.kh, a.C, a.R, a.stride, true) : 0;
     ConvArgs b = a;
     int64_t ldf = a.R;
     if (copy > 0) {
@@ -1286,9 +1311,10 @@ int conv_bwd(const ConvArgs& a, int* handled) {
         return chain(a.x, a.C, 0, 0, a.U, a.R, a.R, a.V, a.R, a.O, nullptr, a.O, a.ws_T, a.R, a.stream, &cv);
     };
     const bool flat = !a.lean && conv_flat_bwd_pays(a, a.dX != nullptr) && aligned16(a.dU) && aligned16(a.dV);
-    // (dU alone reads so narrow rows too seldom: without dX 64 -> 24 -> 64 of 25088 pixels 20.4 us, 20.9 at the pitch)
-    const int64_t ldt = a.lean || (!a.dX && !flat && a.R < 32) ? a.R : conv_dt_pitch(a.R);
-    const size_t copy_bytes = a.lean ? 0 : conv_factor_copy(P, Keff, a.R, false);
+    // (Narrow rows that are read once or by dU alone lie as they are: without dX 64 -> 24 -> 64 of 25088 pixels 20.4 us, 20.9 at the pitch; one
+    // tap, 160 -> 40 -> 160 of 50176 37.5 / 38.5, 64 -> 24 -> 64 of 100352 45.0 / 46.1.)
+    const int64_t ldt = a.lean || (a.R < 64 && a.kh == 1) || (!a.dX && !flat && a.R < 32) ? a.R : conv_dt_pitch(a.R);
+    const size_t copy_bytes = a.lean ? 0 : conv_factor_copy(P, a.kh, a.C, a.R, a.stride, false);
     const bool copy = a.dX && copy_bytes > 0;      // of U for dX; the launch that makes dT runs beside it
     char* const ws = a.ws + copy_bytes;
     const Operand U{copy ? a.ws : a.U, copy ? ldt : a.R, false, 0, false, true};

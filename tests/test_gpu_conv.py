@@ -406,6 +406,37 @@ def test_forward_copies_of_the_factors(N, H, W, C, R, O, k, stride, pad, copied)
     assert torch.equal(y, y1) and torch.equal(T, T1)
 
 
+@pytest.mark.parametrize("N,H,R,k,stride,forward,backward", [
+    (16, 28, 40, 1, 1, 0, 0), (32, 28, 40, 1, 1, 1, 0), (32, 28, 40, 3, 2, 0, 0), (16, 28, 56, 3, 1, 0, 0), (32, 28, 56, 3, 1, 0, 0), (32, 28, 56, 5, 1, 1, 0),
+    (32, 28, 72, 1, 1, 1, 0), (108, 28, 72, 3, 2, 1, 1), (16, 28, 80, 3, 1, 0, 0), (32, 28, 80, 3, 1, 1, 1), (32, 28, 80, 1, 1, 0, 0), (32, 28, 96, 3, 1, 0, 1),
+    (103, 28, 24, 5, 1, 0, 0)])
+def test_copies_where_they_are_worth_a_launch(N, H, R, k, stride, forward, backward):
+    """One launch more where the factors, or U for dX, are copied to a pitch of whole lines, none elsewhere; the results are
+    those of the rows as they lie."""
+    C, O, pad = 64, 64, k // 2
+    g = torch.Generator(device="cuda").manual_seed(92)
+    rand = lambda *s, scale=1.0: torch.randn(s, generator=g, device="cuda").mul_(scale).bfloat16()
+    x, U, V = rand(N, H, H, C), rand(k, k, C, R, scale=(k * k * C) ** -0.5), rand(O, R, scale=R ** -0.5)
+    before = pf.pf_launch_count()
+    y, T = pf.pf_lowrank_conv_fwd(x, U, V, stride=stride, pad=pad, want_stash=True)
+    assert pf.pf_launch_count() - before == 1 + forward
+    dY = rand(*y.shape)
+    before = pf.pf_launch_count()
+    out = pf.pf_lowrank_conv_bwd(x, U, V, dY, stride=stride, pad=pad, T_stash=T)
+    launches = pf.pf_launch_count() - before
+    before = pf.pf_launch_count()
+    pf.pf_lowrank_conv_bwd(x, U, V, dY, stride=stride, pad=pad, T_stash=T, need_dX=False)
+    without = pf.pf_launch_count() - before
+    assert launches == 2 + backward + (1 if without == 3 or (k == 3 and stride == 1 and R < 64 and N * H * H >= 25000) else 0)
+    room = (T.numel() * 2 + 255) // 256 * 256
+    y1, T1 = pf.pf_lowrank_conv_fwd(x, U, V, stride=stride, pad=pad, want_stash=True, workspace=torch.empty(room, dtype=torch.uint8, device="cuda"))
+    assert torch.equal(y, y1) and torch.equal(T, T1)
+    d64 = lambda t: t.double().permute(0, 3, 1, 2)
+    dT = (dY.double() @ V.double()).bfloat16()
+    dX = torch.nn.grad.conv2d_input((N, C, H, H), U.double().permute(3, 2, 0, 1), d64(dT), stride=stride, padding=pad).permute(0, 2, 3, 1)
+    assert (out[0].double() - dX).norm() <= 1e-2 * dX.norm()
+
+
 @pytest.mark.parametrize("N,H,W,C,R,O,k,stride,pad", [
     (163, 16, 16, 64, 16, 64, 3, 1, 1),      # two dX tiles per block, a last block with one
     (41, 30, 30, 136, 24, 40, 3, 2, 1),      # eight per block, two column tiles (one ragged), all classes in a block
