@@ -125,6 +125,16 @@ struct RepackJob {
     int64_t groups = 1, gs_src = 0;
 };
 cudaError_t repack_rows_bf16_multi(const RepackJob* jobs, int count, cudaStream_t stream);
+// Parameters of one such launch.
+constexpr int kRepackJobs = 6;
+struct RepackBatchArgs {
+    const unsigned short* src[kRepackJobs];
+    unsigned short* dst[kRepackJobs];
+    long long ld_src[kRepackJobs], ld_dst[kRepackJobs], gs_src[kRepackJobs];
+    int cols[kRepackJobs], pieces_per_row[kRepackJobs], rows[kRepackJobs];   // rows of one group
+    unsigned int item_end[kRepackJobs];   // running total of items up to and including job j
+    int count;
+};
 
 // pack
 cudaError_t pack_launch(const void* const* grads, const int64_t* numels, const int64_t* offsets,

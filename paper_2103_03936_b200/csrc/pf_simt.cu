@@ -200,15 +200,6 @@ repack_rows_kernel(const unsigned short* __restrict__ src, int64_t ld_src,
 // A job may cover several matrices (groups) a fixed stride apart, which land one after the other.
 // Launched with programmatic dependent launch: its start hides behind the previous kernel's tail, and the
 // product that reads the copies starts its own prologue meanwhile.
-constexpr int kRepackJobs = 6;
-struct RepackBatchArgs {
-    const unsigned short* src[kRepackJobs];
-    unsigned short* dst[kRepackJobs];
-    long long ld_src[kRepackJobs], ld_dst[kRepackJobs], gs_src[kRepackJobs];
-    int cols[kRepackJobs], pieces_per_row[kRepackJobs], rows[kRepackJobs];   // rows of one group
-    unsigned int item_end[kRepackJobs];   // running total of items up to and including job j
-    int count;
-};
 // Bytes [4 q + bit / 8, + 16) of the window lo:hi.
 __device__ __forceinline__ uint4 shifted_vector(const uint4 o, const uint4 h, unsigned q, unsigned bit) {
     const bool q1 = q & 1, q2 = q & 2;

@@ -233,8 +233,8 @@ tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
     const uint64_t a_policy = kHints ? l2_policy(p.keep[0]) : 0, out_policy = kHints ? l2_policy(p.keep[1]) : 0;
     // (The second half of the groups runs beside the first: when it starts, everything older than that is complete, since
-    // every kernel of this library lets its successor start only after its own wait.  It waits before it ends, so that
-    // whoever waits for it has waited for both.)
+    // the kernels of this library let their successors start only after their own wait.  It waits before it ends, so that
+    // whoever waits for it has waited for both.  It is the exception itself: see kEarlyA.)
     if (!kGroups || !p.group_flags[1]) pdl_wait();                 // everything above overlapped the previous kernel's tail
     pdl_launch_dependents();
     const uint32_t tmem = ctl->tmem_base;

@@ -414,7 +414,7 @@ int f32_linear_bwd(const LinearArgs& a, int* handled) {
     bool ok = true;
     if (!a.T)
         ok = f32_prepare(b.t, {x.p, x.ld, false}, {U.p, U.ld, true}, reinterpret_cast<float*>(Tbuf), f32_pitch(a.r), p1, &lt.ta[0], &lt.tb[0], &lt.p[0]);
-    // (the launch before is the recomputed T, or one of an earlier call)
+    // (the launch before is the recomputed T, this call's re-pitch copies, or one of an earlier call)
     const bool early = !a.T;
     ok = ok && f32_prepare(b.g, {dY.p, dY.ld, false, early}, {V.p, V.ld, true, early}, G, ldG, p1, &la.ta[0], &la.tb[0], &la.p[0]) &&
          f32_prepare(b.dv, {dY.p, dY.ld, true, early}, {T.p, T.ld, true}, static_cast<float*>(a.dV), a.lddv, pv, &la.ta[1], &la.tb[1], &la.p[1]) &&

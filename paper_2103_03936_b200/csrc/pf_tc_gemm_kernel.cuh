@@ -228,9 +228,9 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     __syncthreads();
     tc_fence_after();
     // A product marked independent reads nothing that the kernel launched just before it writes, so
-    // it does not wait for that kernel: its blocks run beside it on SMs that kernel leaves free.  (Every
-    // kernel of this library lets its successor start only after its own wait has returned, i.e. once
-    // everything older in the stream is complete, so older results are safe to read.)
+    // it does not wait for that kernel: its blocks run beside it on SMs that kernel leaves free.  (The kernels
+    // of this library let their successors start only after their own wait has returned, i.e. once
+    // everything older in the stream is complete, so older results are safe to read; the exceptions are named at kEarlyA.)
     // The same holds for a single operand (p.early): its producer fills the ring beside the previous kernel's tail.
     const bool ahead = p.independent || (warp == 0 && (p.early & kEarlyA)) || (warp == 6 && (p.early & kEarlyB));
     if (!ahead) pdl_wait();             // everything above overlapped the previous kernel's tail

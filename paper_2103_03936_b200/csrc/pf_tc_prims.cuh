@@ -33,7 +33,11 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Operands of a product that were complete before the preceding kernel of the stream got past its own wait, i.e. that
-// neither that kernel writes nor a caller's kernel before it can still be writing: their producers do not wait for it.
+// neither that kernel writes nor a caller's kernel before it can still be writing: their producers do not wait for it.  Never in a
+// call's first launch, which knows nothing of the kernel before.  Two kinds of blocks let their successor start without having waited: those
+// of a product marked `independent` (others of its launch do wait, so the launch as a whole is like any) and the second half of the
+// groups of a grouped forward (ChainParams::group_flags[1]).  Behind that half an operand is early only if it was complete before
+// the first half got past its wait; today nothing in a call follows it.  (tests/host/launches.cu checks all this over drawn calls.)
 constexpr int kEarlyA = 1, kEarlyB = 2;
 
 // ---------------------------------------------------------------- mbarrier

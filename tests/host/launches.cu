@@ -1,6 +1,7 @@
 // What a call of the library launches, looked over on the host (see runtime.cpp): every tensor map that is encoded and every
 // matrix and slice buffer that a launched kernel is given has to lie inside one of the buffers of the call (host_regions)
-// or inside a device array of the library; what does not is reported by host_faults.
+// or inside a device array of the library, and an operand that is read ahead of the launch before (kEarlyA) outside what that one writes;
+// what does not is reported by host_faults.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -16,12 +17,17 @@
 #include "pf_tc_conv_flat.cuh"
 #include "pf_tc_f32_kernel.cuh"
 #include "pf_tc_gemm_kernel.cuh"
+#include "pf_tc_pair_launch.h"
 
 namespace {
 struct Range {
     uint64_t base, bytes;
 };
 std::vector<Range> regions, written;      // `written`: what the products of the launch in hand write
+// What may still be being written when that launch starts: by the launch before, and, behind one that lets its successor start
+// without having waited itself, by what that one ran beside.
+std::vector<Range> before;
+bool before_known = false;                // (not behind the launches of another call, nor behind a kernel that is not looked over)
 std::map<const void*, std::string>& kernels() { static std::map<const void*, std::string> m; return m; }
 std::map<const void*, Range>& arrays() { static std::map<const void*, Range> m; return m; }      // by host symbol
 std::string faults, launches;
@@ -59,7 +65,8 @@ void check(const pf::tc::GemmParams& p) {
 }
 void check(const pf::tc::F32Params& p) {
     if (p.splits > 1) writes("slices of an fp32 product", address(p.partial), static_cast<uint64_t>(p.tiles_x) * p.tiles_y * p.splits * 128 * p.bn * 4);
-    if (p.mode == 0 || p.mode == 2) writes("result of an fp32 product", address(p.C), matrix(p.M, p.N, p.ldc, 4));
+    const bool whole = p.mode == 0 || p.mode == 2;      // (else the pixels of the images)
+    if (whole || p.splits <= 1) writes("result of an fp32 product", address(p.C), matrix(whole ? p.M : static_cast<int64_t>(p.cv_N) * p.out_h * p.out_w, p.N, p.ldc, 4));
     if (p.C2) writes("second copy of an fp32 result", address(p.C2), matrix(p.M, p.N, p.ldc2, 4));
 }
 constexpr uint64_t kSlice = 128 * 64 * 4;
@@ -81,15 +88,27 @@ void check(const pf::SimtGemm& g) {
     inside("result of an FMA product", address(g.C), matrix(g.M, g.N, g.ldc, size));
 }
 
-// What the recorded maps hold: where the matrix lies and the bytes of its rows.
+// What the recorded maps hold: where the matrix lies, the bytes of its rows and of all of it.
 struct MapNote {
-    uint64_t base, row_bytes;
+    uint64_t base, row_bytes, bytes;
 };
+void early(const char* what, const CUtensorMap& map) {
+    const MapNote& n = reinterpret_cast<const MapNote&>(map);
+    if (!before_known) faults += std::string(what) + ": read ahead of a launch that may write it\n";
+    for (const Range& w : before)
+        if (n.base < w.base + w.bytes && w.base < n.base + n.bytes) faults += std::string(what) + ": read ahead of the launch that writes it\n";
+}
+void early(int which, const CUtensorMap& a, const CUtensorMap& b) {
+    if (which & pf::tc::kEarlyA) early("first operand", a);
+    if (which & pf::tc::kEarlyB) early("second operand", b);
+}
+int early_of(const pf::tc::GemmParams& p) { return p.independent ? pf::tc::kEarlyA | pf::tc::kEarlyB : p.early; }
 // A matrix that TMA stores: it fills the last 16-byte piece of a row, so unless it lies in the workspace (the last buffer) its rows
 // end with one.
 void stored(const char* what, const CUtensorMap& map) {
     const MapNote& n = reinterpret_cast<const MapNote&>(map);
     const bool in_workspace = !regions.empty() && n.base >= regions.back().base && n.base < regions.back().base + regions.back().bytes;
+    writes(what, n.base, n.bytes);
     if (n.row_bytes % 16 != 0 && !in_workspace && n.base < (1ull << 60)) faults += std::string(what) + ": the store fills pieces behind the ends of the rows\n";
 }
 
@@ -100,30 +119,63 @@ void launched(const void* kernel, unsigned blocks, void** args) {
     auto is = [&](const char* n) { return name.find(n) != std::string::npos; };
     launches += name + "\n";
     written.clear();
+    bool known = true, late = false;
     if (is("tc_gemm3_kernel")) {
         const int end0 = arg<int>(args, 9), end1 = arg<int>(args, 10);
         check(arg<pf::tc::GemmParams>(args, 6));
         if (end1 > end0) check(arg<pf::tc::GemmParams>(args, 7));
         if (static_cast<int>(blocks) > end1) check(arg<pf::tc::GemmParams>(args, 8));
+        const int ends[4] = {0, end0, end1, static_cast<int>(blocks)};
+        for (int i = 0; i < 3; ++i)
+            if (ends[i + 1] > ends[i]) early(early_of(arg<pf::tc::GemmParams>(args, 6 + i)), arg<CUtensorMap>(args, 2 * i), arg<CUtensorMap>(args, 2 * i + 1));
     } else if (is("tc_gemm_kernel")) {
-        check(arg<pf::tc::GemmParams>(args, 2));
+        const pf::tc::GemmParams& p = arg<pf::tc::GemmParams>(args, 2);
+        check(p);
+        early(early_of(p), arg<CUtensorMap>(args, 0), arg<CUtensorMap>(args, 1));
+        late = p.independent;
+    } else if (is("tc_gemm_pair_kernel")) {
+        const pf::tc::PairLaunch& l = arg<pf::tc::PairLaunch>(args, 0);
+        for (int i = 0; i < l.count; ++i) {
+            const pf::tc::PairProduct& p = l.p[i];
+            const int outputs = p.kb_per_group > 0 ? 1 : p.tiles_mn > 0 ? p.tiles / p.tiles_mn : 1;
+            for (int g = 0; g < outputs; ++g) writes("result of a product on pairs", address(p.C) + static_cast<uint64_t>(g) * p.c_gstride * 2, matrix(p.M, p.N, p.ldc, 2));
+            early(p.early, l.ta[i], l.tb[i]);
+        }
+    } else if (is("repack_multi_kernel")) {
+        const pf::RepackBatchArgs& a = arg<pf::RepackBatchArgs>(args, 0);
+        for (int j = 0; j < a.count; ++j)
+            writes("copy", address(a.dst[j]), matrix((a.item_end[j] - (j > 0 ? a.item_end[j - 1] : 0u)) / a.pieces_per_row[j], a.pieces_per_row[j] * 8, a.ld_dst[j], 2));
     } else if (is("tc_chain_kernel") || is("tc_chain_pipe_kernel")) {
         const pf::tc::ChainParams& p = arg<pf::tc::ChainParams>(args, 5);
         if (p.tiles_per_split > 0) stored("output of the fused kernel", arg<CUtensorMap>(args, 3));
         if (p.store_T) stored("intermediate of the fused kernel", arg<CUtensorMap>(args, 4));
+        late = is("Li3E") && p.group_flags[1];
     } else if (is("tc_f32_kernel")) {
         const pf::tc::F32Launch& l = arg<pf::tc::F32Launch>(args, 0);
         for (int i = 0; i < 3; ++i)
-            if (i == 0 || l.end[i] > l.end[i - 1]) check(l.p[i]);
+            if (i == 0 || l.end[i] > l.end[i - 1]) {
+                check(l.p[i]);
+                early(l.p[i].early, l.ta[i], l.tb[i]);
+            }
     } else if (is("tc_conv_dt_dv_kernel")) {
-        check(arg<pf::tc::DtDvParams>(args, 3), blocks);
+        const pf::tc::DtDvParams& p = arg<pf::tc::DtDvParams>(args, 3);
+        check(p, blocks);
+        for (int i = 0; i < 3 && p.early; ++i) early("operand of dT and dV", arg<CUtensorMap>(args, i));
     } else if (is("tc_conv_du_kernel")) {
         check(arg<pf::tc::DuParams>(args, 2));
+        early("x of dU", arg<CUtensorMap>(args, 0));
     } else if (is("tc_conv_dx_kernel")) {
         check(arg<pf::tc::DxParams>(args, 2));
+        early("U of dX", arg<CUtensorMap>(args, 1));
     } else if (is("simt_gemm_kernel")) {
         check(arg<pf::SimtGemm>(args, 0));
+        known = false;
+    } else {
+        known = false;
     }
+    if (!late) before.clear();
+    before.insert(before.end(), written.begin(), written.end());
+    before_known = known && (before_known || !late);
 }
 
 CUresult encode(CUtensorMap* map, CUtensorMapDataType type, cuuint32_t rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides,
@@ -133,7 +185,7 @@ CUresult encode(CUtensorMap* map, CUtensorMapDataType type, cuuint32_t rank, voi
     for (cuuint32_t i = 1; i < rank; ++i) bytes += (dims[i] - 1) * strides[i - 1];
     inside("tensor map", address(base), bytes);
     *map = CUtensorMap();
-    reinterpret_cast<MapNote&>(*map) = MapNote{address(base), dims[0] * size};
+    reinterpret_cast<MapNote&>(*map) = MapNote{address(base), dims[0] * size, bytes};
     return CUDA_SUCCESS;
 }
 }  // namespace
@@ -145,6 +197,8 @@ void host_regions(int count, const uint64_t* base, const uint64_t* bytes) {
     for (int i = 0; i < count; ++i) regions.push_back(Range{base[i], bytes[i]});
     faults.clear();
     launches.clear();
+    before.clear();
+    before_known = false;
 }
 const char* host_faults() { return faults.c_str(); }
 const char* host_launches() { return launches.c_str(); }
