@@ -669,7 +669,6 @@ bool flat_bwd_plan(int N, int H, int W, int C, int R, int O, int kh, int kw, int
     b->smem_v = 1024 + fixed + b->v_stages * kStreamStage;
     b->bytes_v = align_up(static_cast<size_t>(b->pairs) * b->grid_v * 32768, 256);
     // dU
-    b->f = FlatImage{N, H, W, W + 1, H + 1, 0, 0};
     b->wx = W % 16 == 0 ? W : W + 1;
     b->ct = conv_tiling(N, H, b->wx, 64);
     b->tb = static_cast<int>(ceil_div(C, 128));
@@ -688,8 +687,7 @@ bool flat_bwd_plan(int N, int H, int W, int C, int R, int O, int kh, int kw, int
     }
     b->bytes_u = align_up((static_cast<size_t>(6) * b->split[0] + static_cast<size_t>(3) * b->split[1]) * b->tb * 32768, 256);
     // dX
-    b->f.per_image = b->f.Wp * b->f.Hp <= 64;
-    b->f.unit_rows = b->f.per_image ? b->f.Wp * b->f.Hp : b->f.Wp;
+    b->f = flat_image(N, H, W);
     b->a_bytes = static_cast<uint32_t>(align_up(static_cast<size_t>(window_rows(b->f, kDxRows + 2 * b->f.Wp + 2)) * 128, 1024));
     const size_t before = 1024 + 2 * static_cast<size_t>(b->a_bytes) + 32768;
     if (before + 3 * kDxStage > limit) return false;
@@ -740,7 +738,7 @@ int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, 
                     cached_map_2d(&xb, U, static_cast<int64_t>(9) * a.C, a.R, ldu, 128);
     if (!ok) return PF_ERR_UNSUPPORTED;
     DtDvParams sp = {};
-    sp.rows = static_cast<int>(P); sp.O = a.O; sp.R = a.R;
+    sp.rows = static_cast<int>(P); sp.R = a.R;
     sp.tiles = static_cast<int>(ceil_div(P, 128));
     sp.panels = static_cast<int>(ceil_div(a.O, 64)); sp.pairs = b.pairs;
     sp.num_stages = b.v_stages;

@@ -82,7 +82,7 @@ __device__ __forceinline__ void store_block(uint32_t acc, uint32_t panel, int la
 
 // Parameters of the backward's kernels (pf_tc_conv_bwd.cu).
 struct DtDvParams {
-    int rows, O, R;
+    int rows, R;
     int tiles;                   // of 128 rows
     int panels, pairs;           // of 64 and 128 columns of dY
     int num_stages;
@@ -121,9 +121,9 @@ struct DxParams {
 };
 
 // ------------------------------------------------------------------------------ host
-inline FlatImage flat_image(const ConvArgs& a) {
+inline FlatImage flat_image(int N, int H, int W) {
     FlatImage f;
-    f.N = a.N; f.H = a.H; f.W = a.W; f.Wp = a.W + 1; f.Hp = a.H + 1;
+    f.N = N; f.H = H; f.W = W; f.Wp = W + 1; f.Hp = H + 1;
     f.per_image = f.Wp * f.Hp <= 64;                 // boxes of a few KB at least: a TMA instruction costs 40 ns
     f.unit_rows = f.per_image ? f.Wp * f.Hp : f.Wp;
     return f;

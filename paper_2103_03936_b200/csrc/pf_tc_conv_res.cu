@@ -332,7 +332,7 @@ void fill(ResParams* p, const FlatImage& f, const ResLayout& l, const ConvArgs& 
 
 int conv_res_fwd(const ConvArgs& a, int64_t ldf, const Before& before) {
     if (!res_shape(a)) return PF_ERR_UNSUPPORTED;
-    const FlatImage f = flat_image(a);
+    const FlatImage f = flat_image(a.N, a.H, a.W);
     ResLayout l;
     if (!res_layout(f, &l)) return PF_ERR_UNSUPPORTED;
     // Per 64 channels a tile of 256 positions takes 3.05 us here, a tile of up to 128 pixels in the kernel that fetches
