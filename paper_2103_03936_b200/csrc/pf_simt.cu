@@ -207,42 +207,60 @@ __device__ __forceinline__ uint4 shifted_vector(const uint4 o, const uint4 h, un
     const unsigned w0 = q1 ? x1 : x0, w1 = q1 ? x2 : x1, w2 = q1 ? x3 : x2, w3 = q1 ? x4 : x3, w4 = q1 ? x5 : x4;
     return make_uint4(__funnelshift_r(w0, w1, bit), __funnelshift_r(w1, w2, bit), __funnelshift_r(w2, w3, bit), __funnelshift_r(w3, w4, bit));
 }
+// kDeep: pieces of a thread in flight together.
+template <int kDeep>
 __global__ void __launch_bounds__(256)
 repack_multi_kernel(const __grid_constant__ RepackBatchArgs a) {
     const unsigned int total = a.item_end[a.count - 1], step = gridDim.x * blockDim.x;
-    const unsigned short* sp = nullptr;
-    unsigned short* to = nullptr;
-    int left = 0;
-    auto place = [&](unsigned int it) {
-        int j = 0;
-        while (j + 1 < a.count && it >= a.item_end[j]) ++j;
-        const unsigned int local = it - (j > 0 ? a.item_end[j - 1] : 0u), ppr = static_cast<unsigned int>(a.pieces_per_row[j]);
-        const unsigned int row = local / ppr;
-        const int c0 = static_cast<int>(local - row * ppr) * 8;
-        const unsigned int g = a.gs_src[j] ? row / static_cast<unsigned int>(a.rows[j]) : 0u;
-        sp = a.src[j] + g * a.gs_src[j] + (row - g * static_cast<unsigned int>(a.rows[j])) * a.ld_src[j] + c0;
-        to = a.dst[j] + row * a.ld_dst[j] + c0;
-        left = a.cols[j] - c0;
+    const unsigned short* sp[kDeep];
+    unsigned short* to[kDeep];
+    int left[kDeep];                      // elements of the row from the piece on, 0: no piece
+    auto place = [&](unsigned int first) {
+#pragma unroll
+        for (int u = 0; u < kDeep; ++u) {
+            const unsigned int it = first + u * step;
+            left[u] = 0;
+            if (it >= total) continue;
+            int j = 0;
+            while (j + 1 < a.count && it >= a.item_end[j]) ++j;
+            const unsigned int local = it - (j > 0 ? a.item_end[j - 1] : 0u), ppr = static_cast<unsigned int>(a.pieces_per_row[j]);
+            const unsigned int row = local / ppr;
+            const int c0 = static_cast<int>(local - row * ppr) * 8;
+            const unsigned int g = a.gs_src[j] ? row / static_cast<unsigned int>(a.rows[j]) : 0u;
+            sp[u] = a.src[j] + g * a.gs_src[j] + (row - g * static_cast<unsigned int>(a.rows[j])) * a.ld_src[j] + c0;
+            to[u] = a.dst[j] + row * a.ld_dst[j] + c0;
+            left[u] = a.cols[j] - c0;
+        }
     };
-    unsigned int it = blockIdx.x * blockDim.x + threadIdx.x;
-    if (it < total) place(it);            // (reads the kernel's parameters only: beside the previous kernel's tail)
+    unsigned int first = blockIdx.x * blockDim.x + threadIdx.x;
+    place(first);                         // (reads the kernel's parameters only: beside the previous kernel's tail)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    while (it < total) {
-        // the aligned vectors that hold at least one byte of the piece
-        const unsigned int sh = static_cast<unsigned int>(reinterpret_cast<uintptr_t>(sp)) & 15u;
-        const uint4* v = reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(sp) - sh);
-        const uint4 lo = __ldg(v);
-        uint4 hi = make_uint4(0u, 0u, 0u, 0u);
-        if (static_cast<int>(sh) + 2 * min(left, 8) > 16) hi = __ldg(v + 1);
-        uint4 o = shifted_vector(lo, hi, sh >> 2, (sh & 3u) * 8u);
-        if (left < 8) {                   // zeros behind the row's end
-            auto keep = [&](int e) { return (e < left ? 0xffffu : 0u) | (e + 1 < left ? 0xffff0000u : 0u); };
-            o.x &= keep(0); o.y &= keep(2); o.z &= keep(4); o.w &= keep(6);
+    while (first < total) {
+        // the aligned vectors that hold at least one byte of each piece, all of them in flight together
+        uint4 lo[kDeep], hi[kDeep];
+        unsigned int sh[kDeep];
+#pragma unroll
+        for (int u = 0; u < kDeep; ++u) {
+            sh[u] = static_cast<unsigned int>(reinterpret_cast<uintptr_t>(sp[u])) & 15u;
+            const uint4* v = reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(sp[u]) - sh[u]);
+            lo[u] = hi[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (left[u] > 0) lo[u] = __ldg(v);
+            if (left[u] > 0 && static_cast<int>(sh[u]) + 2 * min(left[u], 8) > 16) hi[u] = __ldg(v + 1);
         }
-        *reinterpret_cast<uint4*>(to) = o;
-        it += step;
-        if (it < total) place(it);
+#pragma unroll
+        for (int u = 0; u < kDeep; ++u) {
+            if (left[u] <= 0) continue;
+            uint4 o = shifted_vector(lo[u], hi[u], sh[u] >> 2, (sh[u] & 3u) * 8u);
+            if (left[u] < 8) {            // zeros behind the row's end
+                auto keep = [&](int e) { return (e < left[u] ? 0xffffu : 0u) | (e + 1 < left[u] ? 0xffff0000u : 0u); };
+                o.x &= keep(0); o.y &= keep(2); o.z &= keep(4); o.w &= keep(6);
+            }
+            *reinterpret_cast<uint4*>(to[u]) = o;
+        }
+        if (total - first <= kDeep * step) break;
+        first += kDeep * step;
+        place(first);
     }
 }
 
@@ -702,17 +720,21 @@ cudaError_t repack_rows_bf16_multi(const RepackJob* jobs, int count, cudaStream_
     auto launch = [&]() -> cudaError_t {
         if (a.count == 0) return cudaSuccess;
         cudaLaunchConfig_t cfg = {};
-        // One piece of a thread in flight.  With four, in one wave of blocks, the copies of 8 MB in front of 700 x 1500 -> 375 -> 6000 take 0.5 us less
-        // where passes follow one another and 0.7 more where one runs by itself; smaller ones are slower either way (backward of 2048 x 500 -> 125 ->
-        // 2000 22.1 -> 22.6 us, of 1024 x 2044 -> 128 -> 512 14.8 -> 15.6), larger ones too.
-        cfg.gridDim = dim3(static_cast<unsigned>(ceil_div(total, 256) < 16 * num_sms() ? ceil_div(total, 256) : 16 * num_sms()));
+        // Copies of 7.3 to 9.7 MB are a trip and a half to memory with one piece of a thread in flight (twelve to sixteen blocks for an SM that
+        // holds eight): four pieces, in one wave of blocks (four to an SM).  Training steps, one piece / four: 700 x 1500 -> 375 -> 6000 49.4 / 47.8 us, 900 of them
+        // 58.2 / 56.4, 600 x 1996 -> 375 -> 6000 49.9 / 48.1, 1200 x 1500 -> 375 -> 3000 53.1 / 52.2; a forward or backward by itself 1 to 2 % longer.  Smaller
+        // ones fit a wave either way and pay for the longer start (3000 x 1004 -> 252 -> 1004, 7.1 MB, forward 19.8 / 20.1; backward of 2048 x 500 -> 125 -> 2000 22.1
+        // / 22.6, of 1024 x 2044 -> 128 -> 512 14.8 / 15.6); larger ones stream, for which twice the threads do better (8 x (700 x 1500 -> 375 ->
+        // 1500), 20 and 41 MB, 102.5 / 104.6).
+        const bool deep = total > 12 * 256 * num_sms() && total <= 16 * 256 * num_sms();
+        cfg.gridDim = dim3(static_cast<unsigned>(deep ? std::min<int64_t>(ceil_div(total, 256), 4 * num_sms()) : std::min<int64_t>(ceil_div(total, 256), 16 * num_sms())));
         cfg.blockDim = dim3(256);
         cfg.stream = stream;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, repack_multi_kernel, a);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, deep ? repack_multi_kernel<4> : repack_multi_kernel<1>, a);
         if (e == cudaSuccess) count_launch();
         a.count = 0;
         total = 0;

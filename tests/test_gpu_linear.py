@@ -490,3 +490,20 @@ def test_fused_backward_infinite_gradient_and_a_ragged_rank():
 def test_backward_schedules(m, k, n, r):
     """Either side of the sizes from which the backward's fused kernel is used, and from which dV runs beside it."""
     run_case(wl.LinearCase("schedule", m, k, n, r, wl.BF16, 77), blocks=True)
+
+
+@pytest.mark.parametrize("m", [2417, 2419, 3224, 3225])
+def test_copies_of_x_around_the_lines_of_their_two_forms(m):
+    """188 pieces of 16 bytes a row: 454 396 and 454 772 pieces, 606 112 and 606 300, either side of 12 and 16 blocks for each of
+    148 SMs.  Every row arrives whole: rows that are one power of two each make x U exact."""
+    k, r, n = 1500, 64, 64
+    g = torch.Generator(device="cuda").manual_seed(m)
+    scale = torch.randint(-3, 4, (m, 1), generator=g, device="cuda").float().exp2()
+    x = (scale * torch.ones(m, k, device="cuda")).bfloat16()
+    x[:, ::3] *= -1
+    U = torch.zeros(k, r, device="cuda")
+    U[torch.arange(k, device="cuda"), torch.arange(k, device="cuda") % r] = 1.0
+    V = torch.eye(n, r, device="cuda").bfloat16()
+    y, T = pf.pf_lowrank_linear_fwd(x, U.bfloat16(), V, want_stash=True)
+    want = x.double() @ U.double()          # at most 24 summands of one magnitude: exact in fp32 and in bf16
+    assert torch.equal(T.double(), want) and torch.equal(y.double(), want)
