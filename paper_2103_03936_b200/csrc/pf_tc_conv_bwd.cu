@@ -491,7 +491,7 @@ tc_conv_du_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 }
 
 // ------------------------------------------------------------------------------ dX, and the sums of the slices
-constexpr int kDxThreads = 480;              // 0 loads windows, 1 MMAs, 2..9 epilogue, 10 loads U, 11..14 sums
+constexpr int kDxThreads = 480;              // 0 loads windows, 1 MMAs, 2..9 epilogue, 10 loads U, 11..14 sums (without dX 2..9 too)
 constexpr int kDxRows = 256;                 // positions of a tile: two row tiles
 constexpr int kDxMaxStages = 8;
 constexpr uint32_t kDxStage = 16384;         // one tap of U^T: 128 channels x 64 ranks
@@ -542,6 +542,10 @@ tc_conv_dx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     }
     const uint32_t tmem = ctl->tmem_base;
     const FlatImage& f = p.f;
+    // Warps of a block that add up slices: without dX the epilogue's join where four have more than a unit each (backward of 128 x 32 x 32, 256 -> 64 -> 256
+    // 57.7 -> 54.9 us, of 64 x 28 x 28, 320 -> 40 -> 320 58.2 -> 50.0; with fewer units they would leave the blocks that end early nothing to end early
+    // with, and the next call's first launch starts on those: 60 x 28 x 28, 80 -> 40 -> 80 33.0, 35.8 with twelve).
+    const int own_sums = p.tiles == 0 && p.sum.tiles * 64 > 4 * static_cast<int>(gridDim.x) ? 12 : 4;
     auto first_unit = [&](int q0) { return floor_div(q0 - f.Wp - 1, f.unit_rows); };
 
     if (warp == 0) {
@@ -615,7 +619,7 @@ tc_conv_dx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 if (b == 0) bph ^= 1u;
             }
         }
-    } else if (warp < 10) {
+    } else if (warp < 10 && own_sums == 4) {
         const int m = (warp - 2) >> 2, q4 = warp & 3;
         const uint32_t lanes = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + static_cast<uint32_t>(m) * 128u;
         const uint32_t panel = base + p.stg_off + static_cast<uint32_t>(warp - 2) * 4096u;
@@ -632,7 +636,7 @@ tc_conv_dx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
     } else {
         // (blocks without a tile are not kept waiting: they take their share of the sums first)
-        const int unit = static_cast<int>(gridDim.x - 1 - blockIdx.x) * 4 + warp - 11, units = static_cast<int>(gridDim.x) * 4;
+        const int unit = static_cast<int>(gridDim.x - 1 - blockIdx.x) * own_sums + (warp > 10 ? warp - 11 : warp + 2), units = static_cast<int>(gridDim.x) * own_sums;
         if (__any_sync(0xffffffffu, sum_slices<true>(p.sum, unit, units, lane))) mend_sums(p, unit, units, lane);
     }
     tc_fence_before();
@@ -704,28 +708,40 @@ bool flat_bwd_plan(int N, int H, int W, int C, int R, int O, int kh, int kw, int
 // 37.3 / 33.5.  Elsewhere the starts of three launches and the sums of the slices (10 to 20 us) want more: 256 -> 64 -> 256 of 25088
 // 32.0 / 33.4, 50176 51.0 / 47.7, 131072 111.4 / 85.6; 128 -> 32 -> 128 of 25088 24.5 / 26.5, 100352 64.4 / 47.5; an expected time decides, fitted to an earlier
 // state of these kernels, so it keeps to the other form up to 12 % beyond the crossing (512 -> 64 -> 512 of 25088 56.2 / 51.3).
-// Without dX the other form has two launches and these still three, of which dX's share was the larger gain, so the line
-// is a work of reductions (pixels times channels) that grows with the channels' slices: 192 -> 48 -> 192 of 25088 23.2 / 30.3, 75264 45.1 / 43.2;
-// 256 -> 64 -> 256 of 50176 37.6 / 37.7, 75264 50.9 / 44.5; 64 -> 32 -> 64 of 131072 34.6 / 39.0; 160 -> 40 -> 160 of 12544 23.2 / 25.4, 37632 45.7 / 37.6;
-// 64 -> 24 -> 64 of 51200 31.6 / 33.1, 75264 36.5 / 35.7; 512 -> 24 -> 512 of 8000 31.6 / 35.2.
-bool conv_flat_bwd_pays(const ConvArgs& a, bool dX) {
-    FlatBwd b;
-    if (!flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b)) return false;
+// Without dX the other form has two launches and these still three, of which dX's share was the larger gain, so the line is a work of
+// reductions (pixels times channels), less where rows straddle lines or the other form works most for padding, more where a block of 128
+// channels is half empty: 192 -> 48 -> 192 of 25088 23.3 / 27.6, 50176 34.5 / 34.7, 75264 45.4 / 40.8; 256 -> 64 -> 256 of 25088 25.0 / 28.0, 50176 37.6 / 34.8; 128 ->
+// 32 -> 128 of 75264 32.5 / 34.2, 100352 39.2 / 38.4; 64 -> 32 -> 64 of 131072 34.4 / 39.4; 128 -> 16 -> 256 of 50176 31.2 / 33.5, 72128 38.9 / 37.9; 64 -> 24 ->
+// 64 of 75264 35.8 / 36.7, 100352 46.3 / 41.5; 160 -> 24 -> 160 of 26656 36.9 / 32.8; 160 -> 40 -> 160 of 12544 23.0 / 23.0, 25088 35.2 / 31.5; 320 ->
+// 40 -> 320 of 12544 31.4 / 27.9; 256 -> 8 -> 256 of 15680 29.3 / 27.5.
+namespace {
+bool flat_bwd_wanted(const ConvArgs& a, bool dX) {
+    if (a.kh != 3 || a.stride != 1 || a.R > 64) return false;       // (most calls of other kinds: no plan is made for them)
     const double c = a.C / 100.0, p = static_cast<double>(a.N) * a.H * a.W / 1000.0, pc = p * c, po = p * a.O / 100.0;
-    if (!dX) return pc >= (64 % a.R == 0 || a.R >= 48 ? (a.C > 64 ? 130.0 : 260.0) : a.R >= 40 ? 48.0 : 28.0 + 12.0 * c);
+    if (!dX) {
+        if (a.R == 8 || a.R == 16 || a.R == 40) return pc >= (a.R == 8 ? 36.0 : a.R == 16 ? 88.0 : 16.0 + 5.0 * c);
+        if (a.R == 24) return pc >= (a.C > 64 ? 33.0 + 2.0 * c : 56.0);
+        return pc >= (a.C <= 64 ? 260.0 : a.R == 32 ? std::max(100.0, 135.0 - 14.0 * c) : 114.0);
+    }
     if (64 % a.R != 0) return a.R % 16 != 0 ? p >= (a.C >= 160 ? (a.O > a.C ? 18.0 : 11.0) : a.C >= 96 ? 16.0 : 25.0) : p >= (a.C >= 160 ? 20.0 : 50.0);
     return p >= 2.0 && 14.6 + 3.58 * c + 0.23 * p + 0.07 * pc + 0.05 * po < (a.R > 32 ? 0.9 : 1.05) * (12.35 + 0.07 * c + 0.16 * p + 0.19 * pc + 0.07 * po);
 }
+bool flat_bwd_plan(const ConvArgs& a, FlatBwd* b) { return flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, b); }
+}  // namespace
 
+bool conv_flat_bwd_pays(const ConvArgs& a, bool dX) {
+    FlatBwd b;
+    return flat_bwd_wanted(a, dX) && flat_bwd_plan(a, &b);
+}
 size_t conv_flat_bwd_workspace(const ConvArgs& a) {
     FlatBwd b;
-    return (conv_flat_bwd_pays(a, true) || conv_flat_bwd_pays(a, false)) && flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b) ? b.bytes_u + b.bytes_v : 0;
+    return (flat_bwd_wanted(a, true) || flat_bwd_wanted(a, false)) && flat_bwd_plan(a, &b) ? b.bytes_u + b.bytes_v : 0;
 }
 
 // T: the stash, or x * U as a launch before left it.
 int conv_flat_bwd(const ConvArgs& a, const void* T, const void* U, int64_t ldu, char* ws, bool early, const Before& before) {
     FlatBwd b;
-    if (encode_fn() == nullptr || !flat_bwd_plan(a.N, a.H, a.W, a.C, a.R, a.O, a.kh, a.kw, a.stride, a.pad, &b)) return PF_ERR_UNSUPPORTED;
+    if (encode_fn() == nullptr || !flat_bwd_plan(a, &b)) return PF_ERR_UNSUPPORTED;
     const int64_t P = static_cast<int64_t>(a.N) * a.H * a.W;
     const int64_t ldt = conv_dt_pitch(a.R);
     float* pu = reinterpret_cast<float*>(ws);

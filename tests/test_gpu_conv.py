@@ -315,7 +315,7 @@ def test_flat_backward_into_the_callers_sums(N, H, W, C, R, O):
 
 
 @pytest.mark.parametrize("N,H,W,C,R,O,without", [
-    (32, 28, 28, 192, 48, 192, 2), (90, 28, 28, 192, 48, 192, 3), (28, 28, 28, 64, 24, 64, 2), (80, 28, 28, 64, 24, 64, 3), (20, 20, 20, 512, 24, 512, 2),
+    (32, 28, 28, 192, 48, 192, 2), (90, 28, 28, 192, 48, 192, 3), (28, 28, 28, 64, 24, 64, 2), (120, 28, 28, 64, 24, 64, 3), (20, 20, 20, 512, 24, 512, 2),
     (20, 28, 28, 448, 56, 448, 2), (16, 28, 28, 160, 40, 160, 2), (48, 28, 28, 160, 40, 160, 3), (130, 32, 32, 64, 32, 64, 2)])
 def test_backward_without_dX_chooses_for_itself(N, H, W, C, R, O, without):
     """What dX gains does not count for a call that does not want it."""
