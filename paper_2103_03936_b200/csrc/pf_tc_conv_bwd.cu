@@ -711,17 +711,18 @@ bool flat_bwd_plan(int N, int H, int W, int C, int R, int O, int kh, int kw, int
 // Without dX the other form has two launches and these still three, of which dX's share was the larger gain, so the line is a work of
 // reductions (pixels times channels), less where rows straddle lines or the other form works most for padding, more where a block of 128
 // channels is half empty: 192 -> 48 -> 192 of 25088 23.3 / 27.6, 50176 34.5 / 34.7, 75264 45.4 / 40.8; 256 -> 64 -> 256 of 25088 25.0 / 28.0, 50176 37.6 / 34.8; 128 ->
-// 32 -> 128 of 75264 32.5 / 34.2, 100352 39.2 / 38.4; 64 -> 32 -> 64 of 131072 34.4 / 39.4; 128 -> 16 -> 256 of 50176 31.2 / 33.5, 72128 38.9 / 37.9; 64 -> 24 ->
-// 64 of 75264 35.8 / 36.7, 100352 46.3 / 41.5; 160 -> 24 -> 160 of 26656 36.9 / 32.8; 160 -> 40 -> 160 of 12544 23.0 / 23.0, 25088 35.2 / 31.5; 320 ->
-// 40 -> 320 of 12544 31.4 / 27.9; 256 -> 8 -> 256 of 15680 29.3 / 27.5.
+// 32 -> 128 of 50176 25.8 / 28.8, 100352 40.1 / 37.9; 64 -> 32 -> 64 of 131072 34.6 / 39.0; 128 -> 16 -> 128 of 62720 32.3 / 31.6, 128 -> 16 -> 256 of 86016 43.2 / 38.5; 64 ->
+// 24 -> 64 of 50176 30.2 / 30.1, 75264 36.6 / 35.1; 160 -> 24 -> 160 of 26656 36.9 / 32.8; 160 -> 40 -> 160 of 12544 23.0 / 23.0, 25088 35.2 / 31.5; 320 ->
+// 40 -> 320 of 12544 31.4 / 27.9; 256 -> 8 -> 256 of 15680 29.3 / 27.5.  Channels that leave a block of 64 ragged cost the other form more: 96 -> 48 -> 96 of
+// 79968 40.2 / 35.0, 352 -> 56 -> 352 of 21952 37.9 / 31.3, 160 -> 64 -> 160 of 48608 32.2 / 33.9, 61152 37.4 / 37.0.
 namespace {
 bool flat_bwd_wanted(const ConvArgs& a, bool dX) {
     if (a.kh != 3 || a.stride != 1 || a.R > 64) return false;       // (most calls of other kinds: no plan is made for them)
     const double c = a.C / 100.0, p = static_cast<double>(a.N) * a.H * a.W / 1000.0, pc = p * c, po = p * a.O / 100.0;
     if (!dX) {
-        if (a.R == 8 || a.R == 16 || a.R == 40) return pc >= (a.R == 8 ? 36.0 : a.R == 16 ? 88.0 : 16.0 + 5.0 * c);
-        if (a.R == 24) return pc >= (a.C > 64 ? 33.0 + 2.0 * c : 56.0);
-        return pc >= (a.C <= 64 ? 260.0 : a.R == 32 ? std::max(100.0, 135.0 - 14.0 * c) : 114.0);
+        if (a.R == 8 || a.R == 16 || a.R == 40) return pc >= (a.R == 8 ? 36.0 : a.R == 16 ? 76.0 : 16.0 + 5.0 * c);
+        if (a.R == 24) return pc >= (a.C > 64 ? 33.0 + 2.0 * c : 44.0);
+        return pc >= (a.C <= 64 ? 260.0 : a.R == 32 ? std::max(100.0, 125.0 - 13.0 * c) : 114.0) * (a.C % 64 == 0 ? 1.0 : 64 % a.R == 0 ? 0.8 : 0.66);
     }
     if (64 % a.R != 0) return a.R % 16 != 0 ? p >= (a.C >= 160 ? (a.O > a.C ? 18.0 : 11.0) : a.C >= 96 ? 16.0 : 25.0) : p >= (a.C >= 160 ? 20.0 : 50.0);
     return p >= 2.0 && 14.6 + 3.58 * c + 0.23 * p + 0.07 * pc + 0.05 * po < (a.R > 32 ? 0.9 : 1.05) * (12.35 + 0.07 * c + 0.16 * p + 0.19 * pc + 0.07 * po);
