@@ -195,11 +195,12 @@ tc_conv_dt_dv_kernel(const __grid_constant__ CUtensorMap tmY, const __grid_const
 }
 
 // ------------------------------------------------------------------------------ sums of slices
-// Units of 8 rows x 16 columns: a lane sums four columns of a row over all slices, in slice order, sixteen slices in flight.
+// Units of 8 rows x 16 columns: a lane sums four columns of a row over all slices, in slice order, kDeep slices in flight.
 struct SumAt {
     int row, col;                // of the result; row -1: none
     float4 v;
 };
+template <int kDeep>
 __device__ __forceinline__ SumAt sum_unit(const SumPart& s, int u, int lane) {
     const int tile = u >> 6, in = u & 63, rr = (in >> 2) * 8 + (lane & 7), pc = (in & 3) * 4 + (lane >> 3);
     const bool tail = tile >= s.tail;
@@ -208,13 +209,13 @@ __device__ __forceinline__ SumAt sum_unit(const SumPart& s, int u, int lane) {
     const float4* src = reinterpret_cast<const float4*>(s.partial) + base * 2048u + ((rr >> 5) * 16 + pc) * 32 + (rr & 31);
     float4 a = make_float4(-0.f, -0.f, -0.f, -0.f);
 #pragma unroll 1
-    for (int s0 = 0; s0 < S; s0 += 16) {
-        float4 w[16];
+    for (int s0 = 0; s0 < S; s0 += kDeep) {
+        float4 w[kDeep];
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
+        for (int i = 0; i < kDeep; ++i)
             if (s0 + i < S) w[i] = __ldcg(src + static_cast<size_t>(s0 + i) * 2048u);
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
+        for (int i = 0; i < kDeep; ++i)
             if (s0 + i < S) { a.x += w[i].x; a.y += w[i].y; a.z += w[i].z; a.w += w[i].w; }
     }
     int row = tile * 128 + rr;
@@ -253,7 +254,7 @@ __device__ __forceinline__ bool sum_units(const SumPart& s, int first, int step,
     bool left = false;
 #pragma unroll 1
     for (int u = first; u < s.tiles * 64; u += step) {
-        const SumAt a = sum_unit(s, u, lane);
+        const SumAt a = sum_unit<16>(s, u, lane);
         if (a.row < 0) continue;
         if (kLeave && has_nan(a.v)) left = true;
         else put_sum<kPlain>(s, a);
@@ -267,67 +268,69 @@ __device__ __forceinline__ bool sum_slices(const SumPart& s, int first, int step
 
 // The sums of dU that sum_slices has left out.  The MMAs of tc_conv_du_kernel take the three taps of a row from one tile of x, so they
 // multiply border pixels by the zeros around dT for the taps that pair them with nothing: an infinity or NaN there makes those taps' sums
-// NaN.  So each NaN is computed once more, over the pairs that exist, in fp32: a warp for 16 columns of a row, lanes along the
-// pixels, up to where all 16 are NaN.  Finite data pay nothing (backward of 128 x 32 x 32, 256 -> 64 -> 256: 84.7 us with and without);
-// one infinity at a border makes it 2.0 ms, a column of them 14, one pixel in 10000 26.
+// NaN.  So each NaN is computed once more, over the pairs that exist, in fp32: a warp for 8 columns of a row, lanes along the
+// pixels, up to where all 8 are NaN.  Finite data pay nothing (backward of 128 x 32 x 32, 256 -> 64 -> 256: 84.7 us with and without);
+// one infinity at a border makes it 2.4 ms, a column of them 19, one pixel in 10000 42.  (In few registers, for they are the kernel's: with 128, 8 columns in
+// flight more, no block of the next kernel fits beside and the training step of that size took 164 us, 162 with 108.)
 __device__ __noinline__ void mend_sums(const DxParams& p, int first, int step, int lane) {
     const FlatImage& f = p.f;
     const SumPart& s = p.sum;
 #pragma unroll 1
     for (int u = first; u < s.tiles * 64; u += step) {
-        SumAt a = sum_unit(s, u, lane);
+        SumAt a = sum_unit<4>(s, u, lane);
         const bool bad = a.row >= 0 && has_nan(a.v);
         uint32_t rows = __ballot_sync(0xffffffffu, bad);
         rows = (rows | rows >> 8 | rows >> 16 | rows >> 24) & 0xffu;
         const int col0 = (u & 3) * 16;
-        const bool wide = col0 + 8 < s.R;
 #pragma unroll 1
         for (; rows != 0; rows &= rows - 1) {
             const int r = __ffs(rows) - 1, row = __shfl_sync(0xffffffffu, a.row, r), tap = row / s.rows, c = row - tap * s.rows;
             const int dy = tap / 3 - 1, dx = tap - tap / 3 * 3 - 1, y0 = max(0, -dy), x0 = max(0, -dx);
             const int cols = f.W - abs(dx), per_image = (f.H - abs(dy)) * cols, count = f.N * per_image;
-            float sum[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) sum[j] = 0.f;
 #pragma unroll 1
-            for (int i0 = 0; i0 < count; i0 += 1024) {
-                float part[16];
+            for (int half = 0; half < 2 && col0 + 8 * half < s.R; ++half) {
+                float sum[8];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) part[j] = 0.f;
+                for (int j = 0; j < 8; ++j) sum[j] = 0.f;
+#pragma unroll 1
+                for (int i0 = 0; i0 < count; i0 += 1024) {
+                    float part[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) part[j] = 0.f;
 #pragma unroll 4
-                for (int i = i0 + lane; i < min(count, i0 + 1024); i += 32) {
-                    const int n = i / per_image, in = i - n * per_image, y = in / cols;
-                    const int64_t pix = (static_cast<int64_t>(n) * f.H + y0 + y) * f.W + x0 + in - y * cols;
-                    const float v = __bfloat162float(p.x[(pix + dy * f.W + dx) * p.C + c]);
-                    const uint4* src = reinterpret_cast<const uint4*>(p.dT + pix * p.ldt + col0);
-                    const uint4 lo = src[0], hi = wide ? src[1] : make_uint4(0u, 0u, 0u, 0u);
-                    const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+                    for (int i = i0 + lane; i < min(count, i0 + 1024); i += 32) {
+                        const int n = i / per_image, in = i - n * per_image, y = in / cols;
+                        const int64_t pix = (static_cast<int64_t>(n) * f.H + y0 + y) * f.W + x0 + in - y * cols;
+                        const float v = __bfloat162float(p.x[(pix + dy * f.W + dx) * p.C + c]);
+                        const uint4 d = *reinterpret_cast<const uint4*>(p.dT + pix * p.ldt + col0 + 8 * half);
+                        const uint32_t w[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            part[2 * j] = fmaf(v, __uint_as_float(w[j] << 16), part[2 * j]);
+                            part[2 * j + 1] = fmaf(v, __uint_as_float(w[j] & 0xffff0000u), part[2 * j + 1]);
+                        }
+                    }
+                    uint32_t nan = 0;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        part[2 * j] = fmaf(v, __uint_as_float(w[j] << 16), part[2 * j]);
-                        part[2 * j + 1] = fmaf(v, __uint_as_float(w[j] & 0xffff0000u), part[2 * j + 1]);
+                        sum[j] += part[j];
+                        if (sum[j] != sum[j]) nan |= 1u << j;
                     }
+                    if (__reduce_or_sync(0xffffffffu, nan) == 0xffu) break;
                 }
-                uint32_t nan = wide ? 0u : 0xff00u;
+                float t[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    sum[j] += part[j];
-                    if (sum[j] != sum[j]) nan |= 1u << j;
+                for (int j = 0; j < 8; ++j) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
+                    if ((lane >> 3 & 1) == j >> 2) t[j & 3] = sum[j];
                 }
-                if (__reduce_or_sync(0xffffffffu, nan) == 0xffffu) break;
-            }
-            float t[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
-                if (lane >> 3 == j >> 2) t[j & 3] = sum[j];
-            }
-            if ((lane & 7) == r) {
-                if (a.v.x != a.v.x) a.v.x = t[0];
-                if (a.v.y != a.v.y) a.v.y = t[1];
-                if (a.v.z != a.v.z) a.v.z = t[2];
-                if (a.v.w != a.v.w) a.v.w = t[3];
+                if ((lane & 7) == r && lane >> 4 == half) {
+                    if (a.v.x != a.v.x) a.v.x = t[0];
+                    if (a.v.y != a.v.y) a.v.y = t[1];
+                    if (a.v.z != a.v.z) a.v.z = t[2];
+                    if (a.v.w != a.v.w) a.v.w = t[3];
+                }
             }
         }
         if (bad) put_sum<false>(s, a);
