@@ -10,7 +10,7 @@
 // for the sums.
 // The form before (dT; then dU, dV and dX in one launch of 128 x 128 and 128 x 64 tiles) moves 1.6 GB through the SMs' load paths at
 // 128 x 32 x 32, 256 -> 64 -> 256 (x once per tap for dU, dT once per tap for dX), 0.45 here: backward 111.6 -> 85.2 us, training step
-// 195.5 -> 160.  By ncu, one launch at a time, they take 24, 32 and 36 us: the first is bound by memory (104 MB and 7 of slices), the second
+// 196.4 -> 162.  By ncu, one launch at a time, they take 24, 32 and 36 us: the first is bound by memory (104 MB and 7 of slices), the second
 // by the tensor cores (busy 58 %; a 128 x 192 x 16 MMA takes 101 clocks) and its 29 MB of slices, the third by the pace at which one
 // thread issues MMAs and by shared memory (a 128 x 128 x 16 MMA reads 8 KB in its 64 clocks, all there is).
 #include <cmath>
